@@ -91,6 +91,10 @@ int pcr_num_groups(const pcr_record* rec);
 /* Sample metadata and output placement of image i (Section 3: labels are metadata). */
 int pcr_get_image(const pcr_record* rec, int i, pcr_image_info* info);
 
+/* The same for images first .. first + count - 1 in one call (a loader that needs the table of every
+ * record it opens).  Errors: PCR_E_ARG. */
+int pcr_get_images(const pcr_record* rec, int first, int count, pcr_image_info* info);
+
 /* Size the output buffer of pcr_decode must have.  Images are packed RGB, row-major,
  * 3*width bytes per row, image i at out_offset (a multiple of 128).  The size includes 16 spare
  * bytes behind the last image (never written; pcr_decode_tensor reads pixels as aligned words). */

@@ -18,7 +18,7 @@ EXPORTS = ("pcr_open", "pcr_num_images", "pcr_num_groups", "pcr_get_image", "pcr
            "pcr_decode", "pcr_evict", "pcr_status", "pcr_coeffs", "pcr_image_blocks", "pcr_launch_count",
            "pcr_strerror", "pcr_close", "pcr_get_scan", "pcr_set_profiling", "pcr_get_profile",
            "pcr_pixels_noalloc", "pcr_decode_more", "pcr_release_cached_memory", "pcr_decode_tensor", "pcr_msssim", "pcr_msssim_scratch_bytes", "pcr_set_upsampling",
-           "pcr_selftest_bounded_wait", "pcr_get_sampling", "pcr_set_record_cache")
+           "pcr_selftest_bounded_wait", "pcr_get_sampling", "pcr_set_record_cache", "pcr_get_images")
 
 
 class ImageInfo(C.Structure):
@@ -56,6 +56,7 @@ def lib():
         L.pcr_num_images.argtypes = [vp]
         L.pcr_num_groups.argtypes = [vp]
         L.pcr_get_image.argtypes = [vp, C.c_int, C.POINTER(ImageInfo)]
+        L.pcr_get_images.argtypes = [vp, C.c_int, C.c_int, C.POINTER(ImageInfo)]
         L.pcr_out_bytes.restype = C.c_size_t
         L.pcr_out_bytes.argtypes = [vp]
         L.pcr_prefix_bytes.restype = C.c_size_t
@@ -120,6 +121,13 @@ def pcr_num_groups(handle: int) -> int:
 def pcr_get_image(handle: int, i: int) -> ImageInfo:
     info = ImageInfo()
     _chk(lib().pcr_get_image(handle, i, C.byref(info)), "pcr_get_image")
+    return info
+
+
+def pcr_get_images(handle: int, first: int, count: int):
+    """ctypes array of the metadata of images first .. first + count - 1."""
+    info = (ImageInfo * count)()
+    _chk(lib().pcr_get_images(handle, first, count, info), "pcr_get_images")
     return info
 
 

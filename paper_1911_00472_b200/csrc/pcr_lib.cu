@@ -942,6 +942,12 @@ int pcr_get_image(const pcr_record* rec, int i, pcr_image_info* info) {
     return PCR_OK;
 }
 
+int pcr_get_images(const pcr_record* rec, int first, int count, pcr_image_info* info) {
+    if (!rec || !info || first < 0 || count < 0 || first > rec->N || count > rec->N - first) return PCR_E_ARG;
+    memcpy(info, rec->info.data() + first, (size_t)count * sizeof *info);
+    return PCR_OK;
+}
+
 size_t pcr_out_bytes(const pcr_record* rec) { return rec ? rec->out_bytes : 0; }
 
 size_t pcr_prefix_bytes(const pcr_record* rec, int k) {

