@@ -17,6 +17,7 @@
 // memory end up holding the final coefficients.
 #pragma once
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include "pcr_types.h"
@@ -163,6 +164,104 @@ __device__ __forceinline__ int extend_bits(uint32_t v, int s) {
 // the top n bits of x (n in 0..32)
 __device__ __forceinline__ uint32_t top_bits(uint32_t x, int n) { return n ? x >> (32 - n) : 0u; }
 
+struct ScanList { int32_t n; int32_t s[64]; };      // the scans one launch covers
+
+// ---------------------------------------------------------------------------------------
+// Tables of the interval kernels: one ScanTab per (scan, image, table), built once per decode beside the
+// restart-interval index (the entropy warps then only copy 2.3 KB; building the table in every entropy
+// warp took about 1000 instructions in front of a few hundred symbols).  An entry already holds what the
+// scan's decode loop needs of a symbol:
+//   bits 0..4   bits to skip: the code plus its extra bits (magnitude, sign, or run length)
+//   AC refinement: bit 5 a new coefficient, bits 8..14 run of zeros, or 64 + run-length exponent for an end
+//               of band (as a run it passes over every position there can be)
+//   otherwise:  bits 5..8 magnitude size, bits 9..12 run of zeros (an end of band: its run-length exponent),
+//               bit 13 end of band
+// 0 = a code longer than kTabBits bits, or no valid symbol of this kind of scan.
+// ---------------------------------------------------------------------------------------
+constexpr int kTabBits = 10;
+struct __align__(16) ScanTab {
+    uint16_t lut[1 << kTabBits];
+    uint16_t first[8], cnt[8], idx[8];      // codes of kTabBits + 1 + j bits: first code, how many, index of the first value
+    uint8_t vals[256];
+};
+static_assert(sizeof(ScanTab) % 16 == 0, "tables are copied as 16-byte vectors");
+enum { kTabDc = 0, kTabAcFirst = 1, kTabAcRefine = 2, kTabAcSeq = 3 };
+constexpr uint32_t kEntEob = 0x2000u;         // first passes and sequential scans
+constexpr uint32_t kEntEobRefine = 0x4000u;   // end of band of one block in a refinement
+
+__device__ __forceinline__ uint32_t sym_entry(int kind, uint32_t len, uint32_t sym) {
+    const uint32_t r = (sym >> 4) & 15u, sz = sym & 15u;
+    if (kind == kTabDc) return sym > 15u ? 0u : ((len + sz) | (sz << 5));
+    if (kind == kTabAcRefine) {
+        if (sz > 1u) return 0u;
+        if (sz || r == 15u) return (len + sz) | (sz << 5) | (r << 8);
+        return (len + r) | ((64u + r) << 8);
+    }
+    if (sz) return (len + sz) | (sz << 5) | (r << 9);
+    if (r == 15u) return len | (15u << 9);
+    if (kind == kTabAcSeq && r) return 0u;
+    return (len + r) | (r << 9) | kEntEob;
+}
+
+// One warp builds one table in device memory from a DHT body (16 length counts, then the values in code order).
+__device__ __forceinline__ void build_scan_tab(ScanTab* __restrict__ t, const uint8_t* __restrict__ dht, int kind, int lane,
+                                               uint32_t* s_code, uint8_t* s_vals) {
+    // s_code: [3][17] words of the warp: first code, first index, one past the last code left-aligned to kTabBits
+    const uint32_t my = lane < 16 ? dht[lane] : 0u;
+    uint32_t code = 0, p = 0;
+    for (int l = 1; l <= 16; ++l) {
+        const uint32_t c = __shfl_sync(0xffffffffu, my, l - 1);
+        if (lane == 0) {
+            s_code[l] = code; s_code[17 + l] = p;
+            s_code[34 + l] = l <= kTabBits ? (code + c) << (kTabBits - l) : 0u;
+            if (l > kTabBits) { const int j = l - kTabBits - 1; t->first[j] = (uint16_t)code; t->cnt[j] = (uint16_t)c; t->idx[j] = (uint16_t)p; }
+        }
+        code = (code + c) << 1;
+        p += c;
+    }
+    const uint32_t nvals = min(p, 256u);
+    for (uint32_t j = lane; j < 256u; j += 32) { const uint8_t v = j < nvals ? dht[16 + j] : 0; s_vals[j] = v; t->vals[j] = v; }
+    __syncwarp();
+    // every lane fills 32 consecutive entries; the code length only grows along them
+    int l = 1;
+    for (int g = 0; g < 4; ++g) {
+        uint32_t w[4];
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            uint32_t pair = 0;
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                const uint32_t x = 32u * (uint32_t)lane + 8u * (uint32_t)g + 2u * (uint32_t)h + (uint32_t)b;
+                while (l <= kTabBits && x >= s_code[34 + l]) ++l;
+                uint32_t e = 0;
+                if (l <= kTabBits) e = sym_entry(kind, (uint32_t)l, s_vals[(s_code[17 + l] + (x >> (kTabBits - l)) - s_code[l]) & 255u]);
+                pair |= e << (16 * b);
+            }
+            w[h] = pair;
+        }
+        reinterpret_cast<uint4*>(t->lut)[4 * lane + g] = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+}
+
+// One table per warp: the tables of the listed scans of images img0 .. img0 + nimg - 1 of the processing order,
+// slot by slot.  Follows the index warps of the same launch (see unstuff_index_kernel).
+__device__ __forceinline__ void tables_warp(const Params& P, const ScanList& sl, int img0, int nimg, uint32_t w, int lane,
+                                            uint32_t* s_code, uint8_t* s_vals) {
+    const int slot = (int)(w & 3u);
+    const uint32_t pair = w >> 2;
+    const int s = sl.s[pair / (uint32_t)nimg];
+    const ScanAux ax = P.saux[s];
+    if (slot >= ax.ntab) return;
+    const int img = (int)P.order[img0 + pair % (uint32_t)nimg];
+    const ScanDesc& sd = P.scans[(size_t)s * P.N + img];
+    const ScanScript sc = P.script[s];
+    const bool seq = sc.Ss == 0 && sc.Se == 63;
+    const uint32_t off = seq && slot >= 2 ? sd.tab_ac[slot - 2] : sd.tab_off[slot];
+    if (!off) return;
+    const int kind = seq ? (slot < 2 ? kTabDc : kTabAcSeq) : (sc.Ss == 0 ? kTabDc : (sc.Ah == 0 ? kTabAcFirst : kTabAcRefine));
+    build_scan_tab(P.tabs + ax.tab0 + (uint32_t)img * (uint32_t)ax.ntab + (uint32_t)slot, P.rec + off, kind, lane, s_code, s_vals);
+}
+
 // ---------------------------------------------------------------------------------------
 // Restart-interval index and unstuffing, one warp per (listed scan, image).
 // Copies the pair's entropy-coded bytes into P.ubuf with the zero byte after every 0xFF
@@ -172,11 +271,17 @@ __device__ __forceinline__ uint32_t top_bits(uint32_t x, int n) { return n ? x >
 // interval j spans [seg[j], seg[j+1] - 2).  Lanes take 16-byte slices; positions come from a
 // warp prefix sum of the bytes each slice keeps.
 // ---------------------------------------------------------------------------------------
-struct ScanList { int32_t n; int32_t s[64]; };      // the scans one launch covers
-
-__global__ void __launch_bounds__(256) unstuff_index_kernel(Params P, ScanList sl, int img0, int nimg) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+// Blocks from index_blocks on build the lookup tables of the same scans and images (one warp per table).
+__global__ void __launch_bounds__(256) unstuff_index_kernel(Params P, ScanList sl, int img0, int nimg, uint32_t index_blocks) {
     const int lane = threadIdx.x & 31;
+    if (blockIdx.x >= index_blocks) {
+        __shared__ uint32_t s_code[8][51];
+        __shared__ uint8_t s_vals[8][256];
+        const uint32_t w = ((blockIdx.x - index_blocks) * blockDim.x + threadIdx.x) >> 5;
+        if (w < 4u * (uint32_t)(sl.n * nimg)) tables_warp(P, sl, img0, nimg, w, lane, s_code[threadIdx.x >> 5], s_vals[threadIdx.x >> 5]);
+        return;
+    }
+    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (warp >= sl.n * nimg) return;
     const int img = (int)P.order[img0 + warp % nimg];      // img0, nimg: a run of the processing order
     const ScanDesc sd = P.scans[sl.s[warp / nimg] * P.N + img];
@@ -317,38 +422,149 @@ __device__ __forceinline__ uint64_t mcu_block(const Geometry& g, const Params& P
 
 __device__ __forceinline__ uint64_t low_mask(int p) { return p >= 64 ? ~0ull : ((1ull << p) - 1ull); }
 
-// position of the (r+1)-th set bit of z, or 64 if z has fewer: a fixed five-step search on
-// population counts, so lanes with different r stay converged
-__device__ __forceinline__ int select_bit(uint64_t z, int r) {
-    const uint32_t lo = (uint32_t)z, hi = (uint32_t)(z >> 32);
-    int c = __popc(lo), base = 0;
-    uint32_t x = lo;
-    if (r >= c) { r -= c; x = hi; base = 32; }
-    const bool none = r >= __popc(x);
-    c = __popc(x & 0xFFFFu); if (r >= c) { r -= c; x >>= 16; base += 16; }
-    c = __popc(x & 0xFFu);   if (r >= c) { r -= c; x >>= 8;  base += 8; }
-    c = __popc(x & 0xFu);    if (r >= c) { r -= c; x >>= 4;  base += 4; }
-    c = __popc(x & 0x3u);    if (r >= c) { r -= c; x >>= 2;  base += 2; }
-    if (r >= (int)(x & 1u)) base += 1;
-    return none ? 64 : base;
+// ---------------------------------------------------------------------------------------
+// Bit reader of the interval kernels.  The position is one number: bits counted from the first bit of a
+// 16-byte group of the unstuffed copy.  The words around it lie in the lane's column of a ring in shared
+// memory (one row more than the ring: it repeats row 0), so the window of the next 32 bits is two shared
+// loads and a funnel shift, and skipping is an addition: no buffer, no refill branch.  All lanes top their
+// columns up together.  `stop` is the first position at which a step may not begin (the ring runs out, the
+// interval has ended, the lane has nothing to do): one comparison per step.
+// Shared memory is addressed by 32-bit addresses (a generic pointer's window base was recomputed per access).
+// ---------------------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t lds32(uint32_t a) { uint32_t v; asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory"); return v; }
+__device__ __forceinline__ uint32_t lds16(uint32_t a) { uint32_t v; asm volatile("ld.shared.u16 %0, [%1];" : "=r"(v) : "r"(a) : "memory"); return v; }
+__device__ __forceinline__ uint32_t lds8(uint32_t a) { uint32_t v; asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a) : "memory"); return v; }
+__device__ __forceinline__ uint4 lds128(uint32_t a) { uint4 v; asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory"); return v; }
+__device__ __forceinline__ void sts32(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" : : "r"(a), "r"(v) : "memory"); }
+__device__ __forceinline__ void sts128(uint32_t a, const uint4& v) { asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" : : "r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory"); }
+// shifts that give 0 for counts of 32 and more
+__device__ __forceinline__ uint32_t shl0(uint32_t x, uint32_t n) { uint32_t y; asm("shl.b32 %0, %1, %2;" : "=r"(y) : "r"(x), "r"(n)); return y; }
+__device__ __forceinline__ uint32_t shr0(uint32_t x, uint32_t n) { uint32_t y; asm("shr.u32 %0, %1, %2;" : "=r"(y) : "r"(x), "r"(n)); return y; }
+// byte permutation with the selector's sign form (__byte_perm masks it out)
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t s) { uint32_t y; asm("prmt.b32 %0, %1, %2, %3;" : "=r"(y) : "r"(a), "r"(b), "r"(s)); return y; }
+
+struct LaneBits {
+    uint32_t col;          // shared address of this lane's column: row r at col + 128 r
+    const uint4* g4;       // the 16-byte group that position 0 lies in
+    uint32_t pos, wr;      // next bit; next word to fetch (a multiple of 4)
+    uint32_t limit;        // first bit behind the interval
+
+    __device__ __forceinline__ void init(uint32_t column, const uint8_t* ubuf, uint32_t bstart, uint32_t bend) {
+        col = column;
+        g4 = reinterpret_cast<const uint4*>(ubuf) + (bstart >> 4);
+        pos = 8u * (bstart & 15u);
+        limit = pos + 8u * (bend - bstart);
+        wr = 0;
+    }
+    __device__ __forceinline__ void put(uint32_t w, const uint4& v) {
+        const uint32_t p = col + (w & (kRingWords - 1)) * 128u;
+        sts32(p, v.x); sts32(p + 128u, v.y); sts32(p + 256u, v.z); sts32(p + 384u, v.w);
+        if ((w & (kRingWords - 1)) == 0) sts32(p + kRingWords * 128u, v.x);
+    }
+    // top-up in two halves (all lanes of the warp together), so that other loads can be requested between them
+    __device__ __forceinline__ int request(bool on, uint4 (&v)[4]) {
+        const int room = on ? (int)(kRingWords - (wr - (pos >> 5))) >> 2 : 0;
+        const uint4* g = g4 + (wr >> 2);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (room > q) v[q] = __ldg(g + q);
+        return room;
+    }
+    __device__ __forceinline__ void store(int room, const uint4 (&v)[4]) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (room > q) put(wr + 4 * q, v[q]);
+        wr += 4u * (uint32_t)min(max(room, 0), 4);
+    }
+    __device__ __forceinline__ void topup(bool on) {
+        uint4 v[4];
+        const int room = request(on, v);
+        store(room, v);
+    }
+    // steps may begin below this position: `words` words from the one the position lies in are in the ring
+    __device__ __forceinline__ uint32_t ring_stop(uint32_t words) const { return 32u * (wr - min(wr, words - 1u)); }
+    __device__ __forceinline__ uint32_t window(uint32_t at) const {
+        const uint32_t p = col + ((at << 2) & ((kRingWords - 1) * 128u));
+        return __funnelshift_l(lds32(p + 128u), lds32(p), at);    // (shift taken mod 32)
+    }
+};
+
+// The signed value of the sz-bit magnitude field that ends bit `skip` of the window.
+__device__ __forceinline__ int magnitude(uint32_t win, uint32_t skip, uint32_t sz) {
+    const uint32_t x = shl0(win, skip - sz);
+    const int v = (int)shr0(x, 32u - sz);
+    return (int)x < 0 ? v : v + 1 - (int)shl0(1u, sz);        // (sz = 0: 0)
+}
+
+// A code longer than kTabBits bits (or an undefined one) of the table at shared address t: entry as above, 0 if
+// there is no such symbol.
+__device__ __forceinline__ uint32_t long_code(uint32_t t, uint32_t win, int kind) {
+    const uint32_t w16 = win >> 16;
+#pragma unroll 1
+    for (uint32_t j = 0; j < 16 - kTabBits; ++j) {
+        const uint32_t l = kTabBits + 1u + j, d = (w16 >> (16u - l)) - lds16(t + (uint32_t)offsetof(ScanTab, first) + 2u * j);
+        if (d < lds16(t + (uint32_t)offsetof(ScanTab, cnt) + 2u * j))    // (index masked: damaged tables stay in bounds)
+            return sym_entry(kind, l, lds8(t + (uint32_t)offsetof(ScanTab, vals) + ((lds16(t + (uint32_t)offsetof(ScanTab, idx) + 2u * j) + d) & 255u)));
+    }
+    return 0;
+}
+
+// select_in_byte.at[8 * b + r] = position of the (r+1)-th set bit of byte b
+struct SelectTable {
+    uint8_t at[2048 + 16];
+    constexpr SelectTable() : at() {
+        for (int b = 0; b < 256; ++b) {
+            int r = 0;
+            for (int i = 0; i < 8; ++i)
+                if ((b >> i) & 1) at[8 * b + r++] = (uint8_t)i;
+        }
+    }
+};
+__device__ const __align__(16) SelectTable kSelect{};
+
+// Still-zero positions of a refinement's band in a block, prepared for rank queries: the mask and, byte by
+// byte, how many set bits lie in this byte and those below (at most 63, so that bytes can be compared with a
+// rank by one subtraction per word; the last one is the number of set bits).
+__device__ __forceinline__ uint4 rank_index(uint64_t z) {
+    const uint32_t z0 = (uint32_t)z, z1 = (uint32_t)(z >> 32);
+    auto bytes = [](uint32_t x) {
+        x = x - ((x >> 1) & 0x55555555u);
+        x = (x & 0x33333333u) + ((x >> 2) & 0x33333333u);
+        return (x + (x >> 4)) & 0x0F0F0F0Fu;
+    };
+    const uint32_t c0 = bytes(z0), c1 = bytes(z1);
+    const uint32_t low = (c0 * 0x01010101u) >> 24;
+    return make_uint4(z0, z1, c0 * 0x01010101u, (c1 + low) * 0x01010101u);
 }
 
 constexpr int kDecodeSteps = 16;     // decode steps between two top-ups of the rings
+constexpr int kMaskQueue = 8;        // blocks whose masks a refinement lane holds ahead
+
+// Shared memory of one warp (dynamic): two tables, the ring, and for waves with AC refinements the mask queue.
+constexpr uint32_t kWarpRing = 2 * sizeof(ScanTab), kWarpQueue = kWarpRing + (kRingWords + 1) * 128;
+template <bool kRefine> __host__ __device__ constexpr uint32_t warp_bytes() { return kWarpQueue + (kRefine ? kMaskQueue * 512 : 0); }
 
 // kRoi: restart intervals whose MCU rows lie wholly outside the MCU rows that the image's crop
 // rectangle (P.roi) touches are not decoded (their blocks are never transformed).
-template <bool kRoi>
+// kRefine: the wave holds AC refinements (its warps then need a mask queue; the other waves run with less
+// shared memory and fewer registers).
+template <bool kRoi, bool kRefine>
 __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, uint32_t item_begin, uint32_t item_count) {
-    __shared__ HuffTab tabs[kEntropyWarps][2];
-    __shared__ uint32_t s_ring[kEntropyWarps][kRingWords][32];
-    __shared__ uint64_t s_hq[kEntropyWarps][4][32];          // masks of the next blocks (AC refinement)
+    extern __shared__ __align__(16) uint8_t s_entropy[];
+    __shared__ __align__(16) uint8_t s_sel[kRefine ? sizeof(SelectTable) : 16];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t it = blockIdx.x * kEntropyWarps + wid;
+    if (kRefine) {
+        for (int i = threadIdx.x; i < (int)sizeof(SelectTable) / 16; i += 32 * kEntropyWarps)
+            reinterpret_cast<uint4*>(s_sel)[i] = __ldg(reinterpret_cast<const uint4*>(kSelect.at) + i);
+        __syncthreads();
+    }
     if (it >= item_count) return;                             // whole warp
     const Item item = P.items[item_begin + it];
     const ScanDesc sd0 = P.scans[item.si];
     const int s = item.si / P.N;
     const ScanScript sc = P.script[s];
+    const ScanAux ax = P.saux[s];
     const bool dc = sc.Ss == 0;              // a DC first pass (DC refinement scans go to dc_refine_kernel)
     // tables: a DC scan may use two tables of one image; an AC item may span two images
     const bool two_images = item.next != 0;
@@ -356,7 +572,7 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, u
     // From here on no lane leaves before the warp does: lanes without work just stay `done`.
     bool done = (uint32_t)lane >= item.count;
     const uint32_t rem0 = sd0.nseg - item.seg0;               // restart intervals left in the first image
-    const int which = (two_images && (uint32_t)lane >= rem0) ? 1 : 0;
+    const uint32_t which = (two_images && (uint32_t)lane >= rem0) ? 1u : 0u;
     uint32_t seg = which ? (uint32_t)lane - rem0 : item.seg0 + lane;
     const ScanDesc sd = which ? P.scans[si1] : sd0;
     const int img = (int)((which ? si1 : item.si) % (uint32_t)P.N);
@@ -383,9 +599,17 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, u
         }
         if (__all_sync(full, done)) return;                               // nothing of this item is wanted
     }
-    build_hufftab(tabs[wid][0], P.rec + sd0.tab_off[0], lane);
-    if (two_images) build_hufftab(tabs[wid][1], P.rec + P.scans[si1].tab_off[0], lane);
-    else if (sd0.tab_off[1]) build_hufftab(tabs[wid][1], P.rec + sd0.tab_off[1], lane);
+    const uint32_t mem = (uint32_t)__cvta_generic_to_shared(s_entropy) + (uint32_t)wid * warp_bytes<kRefine>();
+    {
+        const uint32_t t0 = ax.tab0 + (item.si % (uint32_t)P.N) * (uint32_t)ax.ntab;
+        const uint32_t t1 = two_images ? ax.tab0 + (si1 % (uint32_t)P.N) * (uint32_t)ax.ntab : t0 + 1u;
+        const bool second = two_images || (dc && sd0.tab_off[1]);
+        const uint4* a = reinterpret_cast<const uint4*>(P.tabs + t0);
+        const uint4* b = reinterpret_cast<const uint4*>(P.tabs + t1);
+        constexpr int n = (int)(sizeof(ScanTab) / 16);
+        for (int i = lane; i < n; i += 32) sts128(mem + 16 * i, __ldg(a + i));
+        if (second) for (int i = lane; i < n; i += 32) sts128(mem + 16 * (n + i), __ldg(b + i));
+    }
     const uint32_t* segtab = P.seg_start + sd.seg_base;
     uint32_t bstart = segtab[seg];
     uint32_t bend = segtab[seg + 1] - 2;
@@ -394,253 +618,256 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, u
         bad = true; done = true;
     }
     if (done) { bstart = sd.data_off; bend = sd.data_off; }
-    BitReader br;
-    br.init(&s_ring[wid][0][lane], P.ubuf, bstart, bend);
-    br.topup(!done);
-    br.prime();
-    const int Al = sc.Al, p1 = 1 << sc.Al;
+    LaneBits br;
+    br.init(mem + kWarpRing + 4u * lane, P.ubuf, bstart, bend);
+    const int Al = sc.Al;
+    if (m0 >= m1) done = true;
 
     if (dc) {
-        // ---- DC first pass: one block per step
-        const int bpm = inter ? P.hs * P.vs + 2 : 1;       // blocks per MCU
+        // ---- DC first pass: one MCU per step, its blocks unrolled
+        const int ny = P.hs * P.vs, bpm = inter ? ny + 2 : 1;       // blocks per MCU
         uint32_t m = m0, mrow = m0 / mcu_w, mcol = m0 % mcu_w;
-        int j = 0;                                         // block inside the MCU: the luminance blocks, Cb, Cr
         int pred0 = 0, pred1 = 0, pred2 = 0;
-        if (m >= m1) done = true;
+        // block numbers inside the image: the MCU's first luminance block (or the scan's own component) and its chroma blocks
+        const uint32_t hs = inter ? (uint32_t)P.hs : 1u, vs = inter ? (uint32_t)P.vs : 1u, bw0 = g.bw[inter ? 0 : c0];
+        const uint32_t y_off = inter ? 0u : (uint32_t)(g.coff[c0] - im.blk_base), c_off = (uint32_t)(g.coff[1] - im.blk_base), c_step = g.mx * g.my;
+        int16_t* const head = P.head + im.blk_base * 8;
         for (;;) {
             br.topup(!done);
             __syncwarp(full);
             if (__all_sync(full, done)) break;
+            // an MCU's symbols need at most 6 * 31 bits: seven words and the window's second one
+            const uint32_t stop = done ? 0u : min(br.ring_stop(8), br.limit + 1u);
 #pragma unroll 1
-            for (int t = 0; t < kDecodeSteps; ++t) {
-                if (done || !br.ready()) continue;
-                br.refill();
-                const uint32_t win = br.top32();
-                int ci = 0;
-                uint64_t blk;
-                if (inter) blk = mcu_block(g, P, mrow, mcol, j, &ci);
-                else blk = g.coff[c0] + (uint64_t)mrow * g.bw[c0] + mcol;
-                const int c = inter ? ci : c0;
-                int16_t* dcv = P.head + blk * 8;
-                {
-                    const HuffTab& tab = tabs[wid][(sd.slots >> (2 * ci)) & 1u];
-                    const uint32_t e = huff_lookup(tab, win);
-                    const int len = (int)(e >> 8), sz = (int)(e & 255u);
-                    if (e == 0 || sz > 15) { bad = true; done = true; continue; }
-                    const int d = extend_bits(top_bits(win << len, sz), sz);
-                    br.skip(len + sz);
-                    const int pv = (c == 0 ? pred0 : (c == 1 ? pred1 : pred2)) + d;
-                    if (c == 0) pred0 = pv; else if (c == 1) pred1 = pv; else pred2 = pv;
-                    *dcv = (int16_t)(pv << Al);
+            for (int t = 0; t < kDecodeSteps / 4; ++t) {
+                if (br.pos >= stop || m >= m1 || bad) continue;
+                const uint32_t yb = y_off + (vs * mrow) * bw0 + hs * mcol, cb = c_off + mrow * g.mx + mcol;
+                uint32_t e = 1;
+#pragma unroll
+                for (int j = 0; j < 6; ++j) {
+                    if (j >= bpm) break;
+                    if (br.pos > br.limit) break;
+                    const int ci = j < ny ? 0 : j - ny + 1;
+                    const uint32_t tab = mem + ((sd.slots >> (2 * ci)) & 1u) * (uint32_t)sizeof(ScanTab);
+                    const uint32_t win = br.window(br.pos);
+                    e = lds16(tab + ((win >> (32 - kTabBits)) << 1));
+                    if (e == 0) { e = long_code(tab, win, kTabDc); if (e == 0) break; }
+                    const uint32_t skip = e & 31u;
+                    const int d = magnitude(win, skip, e >> 5);
+                    br.pos += skip;
+                    int pv;
+                    uint32_t blk;
+                    if (j < ny || !inter) { pv = (pred0 += d); blk = yb + ((uint32_t)j & (hs - 1u)) + ((uint32_t)j >> (hs - 1u)) * bw0; }
+                    else if (j == ny) { pv = (pred1 += d); blk = cb; }
+                    else { pv = (pred2 += d); blk = cb + c_step; }
+                    head[(uint64_t)blk * 8] = (int16_t)(pv << Al);
                 }
-                if (++j == bpm) {
-                    j = 0; ++m;
-                    if (++mcol == mcu_w) { mcol = 0; ++mrow; }
-                }
-                if (br.overran()) { bad = true; done = true; }
-                if (m >= m1) done = true;
+                ++m;
+                if (++mcol == mcu_w) { mcol = 0; ++mrow; }
+                bad = e == 0;
             }
             __syncwarp(full);
+            bad = bad || br.pos > br.limit;
+            done = done || bad || m >= m1;
         }
     } else {
-        const HuffTab& tab = tabs[wid][which];
-        const int c = c0, Ss = sc.Ss, Se = sc.Se;
-        const ScanAux ax = P.saux[s];
+        const uint32_t tab = mem + which * (uint32_t)sizeof(ScanTab);
+        const uint32_t c = (uint32_t)c0, Ss = (uint32_t)sc.Ss, Se = (uint32_t)sc.Se;
         const uint32_t bw = g.bw[c];
         const uint32_t wrap = bw - mcu_w + 1;              // step of the block index at the end of a block row
         uint32_t m = m0, bcol = m0 % mcu_w;
         uint32_t bi = (m0 / mcu_w) * bw + bcol;            // block index inside the image's component
-        uint32_t eobrun = 0;
-        if (m >= m1) done = true;
-        if (sc.Ah == 0) {
+        if (!kRefine || sc.Ah == 0) {
             // ---- AC first pass: one Huffman symbol per step
             uint64_t* maskp = P.aux + ax.base + g.loff[c];
             int16_t* plane = P.planes + g.coff[c] * 64;
             int16_t* headp = P.head + g.coff[c] * 8;
-            uint64_t M = 0;
-            int k = Ss;
+            uint32_t M0 = 0, M1 = 0, k = Ss;
             for (;;) {
                 br.topup(!done);
                 __syncwarp(full);
                 if (__all_sync(full, done)) break;
+                uint32_t stop = done ? 0u : min(br.ring_stop(2), br.limit + 1u);
 #pragma unroll 1
                 for (int t = 0; t < kDecodeSteps; ++t) {
-                    if (done || !br.ready()) continue;
-                    br.refill();
-                    const uint32_t win = br.top32();
-                    uint32_t e = tab.lut[win >> (32 - kLutBits)];
-                    if (e == 0) e = huff_lookup(tab, win);
-                    const int len = (int)(e >> 8), r = (int)(e >> 4) & 15, sz = (int)(e & 15u);
-                    const bool is_coef = sz != 0, is_eob = sz == 0 && r < 15;
-                    const int kk = k + r;                                  // position of the coefficient
-                    const bool fail = e == 0 || (is_coef && kk > Se);
-                    const int extra = is_coef ? sz : (is_eob ? r : 0);
-                    const uint32_t xb = top_bits(win << len, extra);       // magnitude bits / run length bits
-                    br.skip(len + extra);
-                    if (is_coef && !fail) {
-                        const int16_t val = (int16_t)(extend_bits(xb, sz) * p1);
-                        if (kk < 8) headp[(uint64_t)bi * 8 + kk] = val;
-                        else plane[(uint64_t)bi * 64 + kk] = val;
-                        M |= 1ull << kk;
+                    if (br.pos >= stop) continue;
+                    const uint32_t win = br.window(br.pos);
+                    uint32_t e = lds16(tab + ((win >> (32 - kTabBits)) << 1));
+                    if (e == 0) e = long_code(tab, win, kTabAcFirst);
+                    const uint32_t skip = e & 31u, sz = (e >> 5) & 15u, r = (e >> 9) & 15u;
+                    br.pos += skip;
+                    k += r;                                                // position of the coefficient
+                    if (e == 0 || (sz && k > Se)) { bad = true; stop = 0; continue; }
+                    if (sz) {
+                        const int16_t val = (int16_t)(magnitude(win, skip, sz) << Al);
+                        int16_t* dst = k < 8u ? headp + ((uint64_t)bi * 8 + k) : plane + ((uint64_t)bi * 64 + k);
+                        *dst = val;
+                        M0 |= shl0(1u, k); M1 |= shl0(1u, k - 32u);
                     }
-                    k = is_coef ? kk + 1 : (is_eob ? k : k + 16);
-                    if (is_eob) eobrun = (1u << r) + xb - 1u;
-                    const bool fin = is_eob || k > Se;
-                    if (fail) { bad = true; done = true; continue; }
-                    if (fin) {
-                        if (M) maskp[bi] = M;
-                        uint32_t adv = 1;
-                        if (eobrun) {                      // the following blocks of the run are empty
-                            const uint32_t more = min(eobrun, m1 - (m + 1));
-                            eobrun -= more;
-                            adv += more;
+                    ++k;                                                   // (sixteen zeros: run 15 plus one)
+                    const bool is_eob = (e & kEntEob) != 0;
+                    if (is_eob || k > Se) {
+                        if (M0 | M1) *reinterpret_cast<uint2*>(maskp + bi) = make_uint2(M0, M1);
+                        k = Ss; M0 = 0; M1 = 0;
+                        ++m; ++bi;
+                        if (++bcol == mcu_w) { bcol = 0; bi += wrap - 1u; }
+                        if (is_eob && r) {                                 // the following blocks of the run are empty
+                            m = min(m - 1u + (1u << r) + shr0(shl0(win, skip - r), 32u - r), m1);
+                            bcol = m % mcu_w; bi = (m / mcu_w) * bw + bcol;
                         }
-                        m += adv;
-                        if (adv == 1) { if (++bcol == mcu_w) { bcol = 0; bi += wrap; } else ++bi; }
-                        else { bcol = m % mcu_w; bi = (m / mcu_w) * bw + bcol; }
-                        k = Ss; M = 0;
+                        if (m >= m1) stop = 0;
                     }
-                    if (br.overran()) { bad = true; done = true; }
-                    if (m >= m1) done = true;
                 }
                 __syncwarp(full);
+                bad = bad || br.pos > br.limit;
+                done = done || bad || m >= m1;
             }
         } else {
             // ---- AC refinement: one Huffman symbol, or one block of an end-of-band run, per step.
-            // Hs holds the already-non-zero positions of the band from the current position k on
-            // (bit 0 = position k), rem the positions left.  Skipping r zero positions: the target
-            // sits at distance t = r + (non-zero positions up to t), found by iterating from t = r;
-            // the count reached is also the number of correction bits that follow the symbol.
-            const uint64_t band = low_mask(Se + 1) & ~low_mask(Ss);
-            const uint64_t* src0 = nullptr; const uint64_t* src1 = nullptr; const uint64_t* src2 = nullptr; const uint64_t* src3 = nullptr;
-            uint32_t st0 = 0, st1 = 0, st2 = 0, st3 = 0;
-            {
-                const ScanAux x0 = P.saux[ax.src[0]];
-                src0 = P.aux + x0.base + g.loff[c] * x0.stride; st0 = x0.stride;
-                if (ax.nsrc > 1) { const ScanAux x = P.saux[ax.src[1]]; src1 = P.aux + x.base + g.loff[c] * x.stride; st1 = x.stride; }
-                if (ax.nsrc > 2) { const ScanAux x = P.saux[ax.src[2]]; src2 = P.aux + x.base + g.loff[c] * x.stride; st2 = x.stride; }
-                if (ax.nsrc > 3) { const ScanAux x = P.saux[ax.src[3]]; src3 = P.aux + x.base + g.loff[c] * x.stride; st3 = x.stride; }
-            }
-            uint64_t* outp = P.aux + ax.base + g.loff[c] * 4ull;
-            uint64_t* hq = &s_hq[wid][0][lane];                       // slot j at hq[j * 32]
-            uint32_t hm = m, hcol = bcol, hbi = bi;                    // fetch cursor of the mask queue
-            uint64_t H = 0, Hs = 0, cstr = 0, Nw = 0, NS = 0;
-            int k = Ss, cn = 0;
-            uint32_t rem = 0;
-            bool newblk = true;
-            for (;;) {
-                br.topup(!done);
-                // masks of the next blocks, up to four ahead
-                {
-                    uint64_t h[4];
-                    const int want = done ? 0 : (int)min(4u - (hm - m), m1 - hm);
+            // A run of r zeros ends at the (r+1)-th still-zero position not yet passed.  Positions are
+            // therefore counted by rank: T = rank of the target among the block's still-zero positions; its
+            // position comes from the byte counts (how many are at most T tells the byte, a table the bit
+            // inside it), with no search whose length depends on the data.  Position minus rank counts the
+            // non-zero positions below, so the number of correction bits that follow a symbol is the
+            // difference of two such values.
+            const uint64_t band = low_mask((int)Se + 1) & ~low_mask((int)Ss);
+            const uint32_t band0 = (uint32_t)band, band1 = (uint32_t)(band >> 32);
+            // history masks: the union of up to four earlier scans' (one or two in most scripts)
+            const uint64_t* src[4];
+            uint32_t st[4];
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        if (q < want) {
-                            uint64_t v = src0[(uint64_t)hbi * st0];
-                            if (src1) v |= src1[(uint64_t)hbi * st1];
-                            if (src2) v |= src2[(uint64_t)hbi * st2];
-                            if (src3) v |= src3[(uint64_t)hbi * st3];
-                            h[q] = v & band;
-                            hq[((hm + q) & 3u) * 32] = h[q];
-                            if (++hcol == mcu_w) { hcol = 0; hbi += wrap; } else ++hbi;
-                        }
+            for (int q = 0; q < 4; ++q) {
+                const ScanAux x = P.saux[ax.src[q < ax.nsrc ? q : 0]];
+                src[q] = P.aux + x.base + g.loff[c] * x.stride; st[q] = x.stride;
+            }
+            const bool two = ax.nsrc > 1, more = ax.nsrc > 2;
+            uint64_t* outp = P.aux + ax.base + g.loff[c] * 4ull;
+            const uint32_t queue = mem + kWarpQueue + 16u * lane;       // block m at queue + 512 (m % kMaskQueue)
+            uint32_t sel = (uint32_t)__cvta_generic_to_shared(s_sel);
+            asm volatile("" : "+r"(sel));                              // (kept in a register)
+            uint32_t hm = m, hbi = bi;                                 // fetch cursor of the queue
+            uint32_t wrap_m = m + mcu_w - bcol, hwrap_m = wrap_m;      // the first block of the next block row
+            uint32_t eobrun = 0;
+            uint4 Z = make_uint4(0, 0, 0, 0);                          // the block's still-zero positions (see rank_index)
+            uint32_t zi = 0, ep = Ss;                                  // zero positions passed; position minus rank of the last
+            uint32_t s0 = 0, s1 = 0, N0 = 0, N1 = 0, G0 = 0, G1 = 0;   // correction bits, new positions, positive ones
+            bool fresh = true;                                         // the block's entry has not been taken from the queue yet
+            auto take = [&]() { Z = lds128(queue + ((m & (kMaskQueue - 1)) << 9)); };
+            // what the next top-up will store is requested right after the previous one, so that its latency
+            // passes beside the decode steps
+            uint4 va = make_uint4(0, 0, 0, 0), vb = va;
+            uint64_t ha[4], hb[4];
+            auto request = [&]() {
+                const uint4* g = br.g4 + (br.wr >> 2);
+                va = __ldg(g); vb = __ldg(g + 1);
+                uint32_t b = hbi, mm = hm, wm = hwrap_m;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    ha[q] = hb[q] = 0;
+                    if (mm < m1) {
+                        ha[q] = src[0][(uint64_t)b * st[0]];
+                        if (two) hb[q] = src[1][(uint64_t)b * st[1]];
                     }
-                    hm += (uint32_t)max(want, 0);
+                    ++b; ++mm;
+                    if (mm == wm) { b += wrap - 1u; wm += mcu_w; }
+                }
+            };
+            if (!done) request();
+            for (;;) {
+                const uint32_t room = done ? 0u : (kRingWords - (br.wr - (br.pos >> 5))) >> 2;
+                if (room > 0) br.put(br.wr, va);
+                if (room > 1) br.put(br.wr + 4, vb);
+                if (room > 2) br.put(br.wr + 8, __ldg(br.g4 + (br.wr >> 2) + 2));
+                if (room > 3) br.put(br.wr + 12, __ldg(br.g4 + (br.wr >> 2) + 3));
+                br.wr += 4u * room;
+                const uint32_t want = done ? 0u : min((uint32_t)kMaskQueue - (hm - m), m1 - hm);
+#pragma unroll
+                for (int q = 0; q < kMaskQueue; ++q) {
+                    if (q == 4 && !__any_sync(full, want > 4u)) break;
+                    if (q < (int)want) {
+                        uint64_t x;
+                        if (q < 4) x = ha[q] | hb[q];
+                        else { x = src[0][(uint64_t)hbi * st[0]]; if (two) x |= src[1][(uint64_t)hbi * st[1]]; }
+                        if (more) x |= src[2][(uint64_t)hbi * st[2]] | src[3][(uint64_t)hbi * st[3]];
+                        sts128(queue + ((hm & (kMaskQueue - 1)) << 9), rank_index(~x & band));
+                        ++hm; ++hbi;
+                        if (hm == hwrap_m) { hbi += wrap - 1u; hwrap_m += mcu_w; }
+                    }
                 }
                 __syncwarp(full);
                 if (__all_sync(full, done)) break;
+                if (!done) {
+                    request();
+                    if (fresh) take();
+                }
+                // a step reads the window at its start and, at most 31 bits on, two words (three for more than
+                // 32 correction bits)
+                uint32_t stop = done ? 0u : min(br.ring_stop(4), br.limit + 1u);
 #pragma unroll 1
                 for (int t = 0; t < kDecodeSteps; ++t) {
-                    if (done || !br.ready() || m >= hm) continue;
-                    if (newblk) {
-                        H = hq[(m & 3u) * 32];
-                        Hs = H >> Ss;
-                        k = Ss; rem = (uint32_t)(Se - Ss + 1);
-                        cstr = 0; Nw = 0; NS = 0; cn = 0;
-                        newblk = false;
-                    }
-                    br.refill();
-                    const uint32_t win = br.top32();
-                    const bool run = eobrun > 0;                       // this block lies inside an end-of-band run
-                    uint32_t e = tab.lut[win >> (32 - kLutBits)];
-                    if (e == 0 && !run) e = huff_lookup(tab, win);
-                    const int len = (int)(e >> 8), r = (int)(e >> 4) & 15, sz = (int)(e & 15u);
-                    const bool is_new = !run && sz != 0;
-                    const bool is_eob = !run && sz == 0 && r < 15;
-                    bool fail = !run && (e == 0 || sz > 1);
-                    const int extra = is_new ? 1 : (is_eob ? r : 0);
-                    const uint32_t xbits = top_bits(win << len, extra);    // sign of a new coefficient / run length bits
-                    br.skip(run ? 0 : len + extra);
-                    if (is_eob) eobrun = (1u << r) + xbits;
-                    bool beyond = run || is_eob;                       // the rest of the band is passed over
-                    // three rounds of dist = r + (non-zero positions up to dist) settle all but rare
-                    // cases; those (and targets past bit 31) take the general search
-                    const uint32_t lo = (uint32_t)Hs;
-                    const uint32_t ur = (uint32_t)r;
-                    uint32_t dist, cnt;
-                    {
-                        const uint32_t c1 = __popc(lo & ((2u << ur) - 1u));                  // ur <= 15
-                        const uint32_t t1 = ur + c1;                                          // <= 31
-                        const uint32_t c2 = __popc(lo & ((2u << t1) - 1u));
-                        const uint32_t t2 = min(ur + c2, 31u);
-                        const uint32_t c3 = __popc(lo & ((2u << t2) - 1u));
-                        dist = ur + c3; cnt = c3;
-                        if (!beyond && (dist != ur + c2 || dist >= 32u) && dist < rem) {     // not settled
-                            const int sel = select_bit(~Hs & low_mask((int)rem), r);
-                            if (sel >= 64) dist = rem;
-                            else { dist = (uint32_t)sel; cnt = (uint32_t)__popcll(Hs & low_mask(sel)); }
+                    if (br.pos < stop) {
+                        const uint32_t win = br.window(br.pos), nz = Z.w >> 24;
+                        uint32_t e = lds16(tab + ((win >> (32 - kTabBits)) << 1));
+                        e = eobrun ? kEntEobRefine : e;                // this block lies inside an end-of-band run
+                        uint32_t T, k, n;
+                        auto target = [&]() {                          // -> T, k, n; ep moves on
+                            T = min(zi + (e >> 8), nz);                // the rank of the target; nz = behind the band
+                            const uint32_t tt = T * 0x01010101u + 0x80808080u;
+                            const uint32_t j = (uint32_t)(__popc((tt - Z.z) & 0x80808080u) + __popc((tt - Z.w) & 0x80808080u));
+                            const uint32_t zb = __byte_perm(Z.x, Z.y, j) & 255u, cj = prmt(Z.z, Z.w, j - 1u) & 255u;   // (j = 0: no byte below, the selector's sign form gives 0)
+                            k = 8u * j + lds8(sel + 8u * zb + T - cj);
+                            k = T < nz ? k : Se + 1u;
+                            n = k - T - ep;                            // correction bits behind the symbol
+                            ep += n;
+                        };
+                        target();
+                        uint32_t skip = e & 31u;
+                        s1 = __funnelshift_lc(s0, s1, n);
+                        s0 = shl0(s0, n) | shr0(shl0(win, skip), 32u - n);
+                        if (e == 0 || skip + n > 32u) {                // rare: a long code, or bits beyond the window
+                            s0 = __funnelshift_rc(s0, s1, n);          // (taken back: n > 32 left the low word in s1)
+                            s1 = shr0(s1, n);
+                            if (e == 0) {
+                                ep -= n;
+                                e = long_code(tab, win, kTabAcRefine);
+                                target();
+                                skip = e & 31u;
+                            }
+                            const uint32_t at = br.pos + skip, cw = br.window(at);
+                            if (n > 32u) {
+                                s1 = (cw >> (64u - n)) | (s0 << (n - 32u));
+                                s0 = __funnelshift_l(br.window(at + 32u), cw, n - 32u);
+                            } else {
+                                s1 = __funnelshift_lc(s0, s1, n);
+                                s0 = shl0(s0, n) | shr0(cw, 32u - n);
+                            }
+                            if (e == 0) { bad = true; stop = 0; k = 0; }   // no such symbol: the lane ends here
+                        }
+                        br.pos += skip + n;
+                        zi = T + 1u;
+                        const uint32_t x = (e >> 8) & 15u;
+                        const uint32_t run = shl0(1u, x) + shr0(shl0(win, skip - x), 32u - x) - 1u;   // of an end of band: blocks behind this one
+                        eobrun = e > kEntEobRefine + 0xFFu ? run : eobrun - (eobrun ? 1u : 0u);
+                        const uint32_t isnew = T < nz ? (e >> 5) & 1u : 0u, plus = isnew & shr0(win, 32u - skip);
+                        N0 |= shl0(isnew, k); N1 |= shl0(isnew, k - 32u);
+                        G0 |= shl0(plus, k); G1 |= shl0(plus, k - 32u);
+                        if (k >= Se) {                                 // block finished
+                            uint4* o = reinterpret_cast<uint4*>(outp + (uint64_t)bi * 4);
+                            o[0] = make_uint4((~Z.x & band0) | N0, (~Z.y & band1) | N1, s0, s1);
+                            o[1] = make_uint4(N0, N1, G0, G1);
+                            ++m; ++bi;
+                            if (m == wrap_m) { bi += wrap - 1u; wrap_m += mcu_w; }
+                            zi = 0; ep = Ss; s0 = s1 = N0 = N1 = G0 = G1 = 0;
+                            take();                                    // (not read when the queue is empty)
+                            stop = m < hm ? stop : 0u;                 // also at the interval's end: hm is at most m1
                         }
                     }
-                    beyond = beyond || dist >= rem;
-                    const int n = beyond ? __popcll(Hs) : (int)cnt;    // correction bits that follow
-                    const uint32_t adv = beyond ? rem : dist + 1u;
-                    fail = fail || cn + n > 64;
-                    if (n > 32) {                                      // rare: more than a word of correction bits
-                        br.refill();
-                        uint64_t bits = br.top32();
-                        br.skip(32);
-                        br.refill();
-                        bits = (bits << (n - 32)) | top_bits(br.top32(), n - 32);
-                        br.skip(n - 32);
-                        if (!fail) cstr |= bits << (64 - cn - n);
-                    } else {
-                        if (br.nbits < n) br.refill();
-                        const uint64_t bits = top_bits(br.top32(), n);
-                        br.skip(n);
-                        if (!fail && n) cstr |= bits << (64 - cn - n);
-                    }
-                    cn += n;
-                    if (fail) { bad = true; done = true; continue; }
-                    {
-                        const uint64_t bit = (uint64_t)(is_new && !beyond) << ((k + (int)dist) & 63);
-                        Nw |= bit;
-                        NS |= xbits ? bit : 0ull;
-                    }
-                    k += (int)adv;
-                    rem -= adv;
-                    Hs = adv >= 64u ? 0ull : Hs >> adv;
-                    eobrun -= (run || is_eob) ? 1u : 0u;
-                    fail = br.overran();
-                    if (rem == 0) {                                    // block finished
-                        uint64_t* o = outp + (uint64_t)bi * 4;
-                        *reinterpret_cast<ulonglong2*>(o) = make_ulonglong2(H | Nw, cstr);
-                        *reinterpret_cast<ulonglong2*>(o + 2) = make_ulonglong2(Nw, NS);
-                        ++m;
-                        if (++bcol == mcu_w) { bcol = 0; bi += wrap; } else ++bi;
-                        // the next block's mask is usually queued already
-                        newblk = m >= hm;
-                        H = hq[(m & 3u) * 32];
-                        Hs = H >> Ss;
-                        k = Ss; rem = (uint32_t)(Se - Ss + 1);
-                        cstr = 0; Nw = 0; NS = 0; cn = 0;
-                    }
-                    bad = bad || fail;
-                    done = fail || m >= m1;
                 }
                 __syncwarp(full);
+                fresh = m >= hm;
+                bad = bad || br.pos > br.limit;
+                done = done || bad || m >= m1;
             }
-
         }
     }
     if (bad) atomicMin(&P.status[img], kErrCorrupt);

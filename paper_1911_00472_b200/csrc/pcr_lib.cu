@@ -181,6 +181,7 @@ struct pcr_record {
     int decoded_k = 0;            // fidelity of the state the planes and side data hold (0: none)
     bool dc_merged = true;        // the planes hold the DC coefficients of the last decode
     bool planes_cleared = true;   // ... and zeros wherever the last decode left no coefficient
+    ScanTab* d_tabs = nullptr;
     ScanScript* d_script = nullptr;
     ScanAux* d_saux = nullptr;
     uint64_t* d_aux = nullptr;
@@ -718,9 +719,13 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     int n_refine[3] = {0, 0, 0};
     for (uint32_t s = 0; s < G; ++s)
         if (r->script[s].Ss > 0 && r->script[s].Ah > 0 && ++n_refine[r->script[s].comp[0]] > 4) return PCR_E_FORMAT;
+    uint64_t n_tabs = 0;
     for (uint32_t s = 0; s < G; ++s) {
         const ScanScript& sc = r->script[s];
         ScanAux& ax = r->saux[s];
+        ax.ntab = sc.Ss > 0 ? 1 : (sc.Se == 63 ? 4 : (sc.Ah == 0 ? 2 : 0));
+        ax.tab0 = (uint32_t)n_tabs;
+        n_tabs += (uint64_t)N * (uint64_t)ax.ntab;
         if (sc.Ss == 0) continue;
         ax.stride = sc.Ah ? 4u : 1u;
         ax.base = aux_words;
@@ -759,6 +764,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     if (int rc = take(r, &r->d_rec, (size_t)(len + 64))) return rc;
     if (int rc = take(r, &r->d_ubuf, (size_t)(len + 256))) return rc;
     zero.push_back({r->d_ubuf, len + 256});
+    if (int rc = take(r, &r->d_tabs, (size_t)(std::max<uint64_t>(n_tabs, 1) * sizeof(ScanTab)))) return rc;
     if (int rc = take(r, &r->d_planes, (size_t)(std::max<uint64_t>(blocks, 1) * 128))) return rc;
     if (int rc = take(r, &r->d_head, (size_t)(std::max<uint64_t>(blocks, 1) * 16))) return rc;
     zero.push_back({r->d_head, (size_t)(std::max<uint64_t>(blocks, 1) * 16)});
@@ -999,6 +1005,7 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
     P.rec = rec->d_rec; P.ubuf = rec->d_ubuf; P.planes = rec->d_planes; P.head = rec->d_head; P.script = rec->d_script; P.scans = rec->d_scans;
     P.saux = rec->d_saux; P.aux = rec->d_aux;
     P.imgs = rec->d_imgs; P.seg_start = rec->d_seg; P.items = rec->d_items; P.units = rec->d_units;
+    P.tabs = rec->d_tabs;
     P.qtab = rec->d_qtab; P.order = rec->d_order; P.status = rec->d_status; P.N = rec->N;
     P.hs = rec->hs; P.vs = rec->vs; P.nc = rec->nc;
     P.roi = targs ? targs->crops : nullptr;          // (only read by the crop-restricted kernels)
@@ -1046,17 +1053,23 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
     // (the pixel kernel also folds the refinement side data into the planes)
     const int W = rec->n_waves;
     std::vector<char> indexed(rec->n_waves, 0);     // wave w of the current slice has an index launch to wait for
+    // index (and lookup tables, where the interval kernels will want them) of the listed scans, all images
+    auto launch_index_kernel = [&](const ScanList& sl, cudaStream_t q) {
+        const uint32_t pairs = (uint32_t)sl.n * (uint32_t)rec->N, nb = (pairs + 7) / 8;
+        bool tables = false;
+        for (int i = 0; i < sl.n; ++i)
+            for (int g = 0; g < rec->n_slices; ++g) tables = tables || rec->item_count[(size_t)g * rec->G + sl.s[i]] > 0;
+        unstuff_index_kernel<<<nb + (tables ? (pairs + 1) / 2 : 0), 256, 0, q>>>(P, sl, 0, rec->N, nb);
+        ++g_launches;
+    };
     // restart-interval index of wave w of slice g on stream q: 1 launched, 0 nothing to do, -1 error
     auto launch_index = [&](int w, cudaStream_t q) -> int {
         ScanList sl;
         sl.n = 0;
         for (int s : rec->wave_scans[w]) if (s >= k0 && s < k) sl.s[sl.n++] = s;
         if (!sl.n) return 0;
-        const uint32_t i0 = 0, i1 = (uint32_t)rec->N;      // one launch covers every slice
         if (copied[w] && cudaStreamWaitEvent(q, rec->ev_copy[w], 0) != cudaSuccess) return -1;
-        const uint32_t warps = (uint32_t)sl.n * (i1 - i0);
-        unstuff_index_kernel<<<(warps + 7) / 8, 256, 0, q>>>(P, sl, (int)i0, (int)(i1 - i0));
-        ++g_launches;
+        launch_index_kernel(sl, q);
         return 1;
     };
     auto run_stage = [&](int stage, int g, cudaStream_t q) -> bool {
@@ -1070,13 +1083,11 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
             return cudaMemsetAsync(rec->d_planes, 0, rec->total_blocks * 128, q) == cudaSuccess;
         }
         if (stage == 1) {
-            if (pipelined) return true;          // done wave by wave, as the bytes arrive
+            if (pipelined || g != 0) return true;   // done wave by wave, as the bytes arrive; one launch covers every slice
             ScanList sl;
             sl.n = 0;
             for (int s = k0; s < k; ++s) sl.s[sl.n++] = s;
-            const uint32_t warps = (uint32_t)sl.n * (i1 - i0);
-            unstuff_index_kernel<<<(warps + 7) / 8, 256, 0, q>>>(P, sl, (int)i0, (int)(i1 - i0));
-            ++g_launches;
+            launch_index_kernel(sl, q);
             return true;
         }
         if (stage < 2 + W) {
@@ -1115,8 +1126,13 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
             }
             if (count) {
                 const unsigned nb = (count + kEntropyWarps - 1) / kEntropyWarps;
-                if (roi) entropy_kernel<true><<<nb, 32 * kEntropyWarps, 0, q>>>(P, begin, count);
-                else entropy_kernel<false><<<nb, 32 * kEntropyWarps, 0, q>>>(P, begin, count);
+                bool refine = false;                       // waves without AC refinements need no mask queues
+                for (int s : rec->wave_scans[w]) refine = refine || (rec->script[s].Ss > 0 && rec->script[s].Ah != 0);
+                const uint32_t smem = kEntropyWarps * (refine ? warp_bytes<true>() : warp_bytes<false>());
+                if (roi && refine) entropy_kernel<true, true><<<nb, 32 * kEntropyWarps, smem, q>>>(P, begin, count);
+                else if (roi) entropy_kernel<true, false><<<nb, 32 * kEntropyWarps, smem, q>>>(P, begin, count);
+                else if (refine) entropy_kernel<false, true><<<nb, 32 * kEntropyWarps, smem, q>>>(P, begin, count);
+                else entropy_kernel<false, false><<<nb, 32 * kEntropyWarps, smem, q>>>(P, begin, count);
                 ++g_launches;
             }
             // scans that are one long restart interval: the first passes of the wave (a contiguous run

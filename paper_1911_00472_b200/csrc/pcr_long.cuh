@@ -665,7 +665,7 @@ __global__ void __launch_bounds__(32 * kSeqLongWarps) sequential_long_kernel(Par
 // AC refinements of scans that are one restart interval.  The unit of work is a chain: one
 // refinement scan of one (image, component) group; a group has at most four (its "levels", in
 // scan order).  Side data written per block is that of entropy_kernel's refinement branch:
-// {non-zero mask of the band after the scan, correction bits in reading order from bit 63 down,
+// {non-zero mask of the band after the scan, correction bits in reading order, the last one in bit 0,
 // newly non-zero positions, the positive ones among them}.
 //
 // The time of a chain is the number of instructions one thread executes per symbol (every
@@ -1048,7 +1048,6 @@ __device__ __forceinline__ void chain_helper(const Params& P, const FinalizeList
                         bp += nn; n -= nn;
                     }
                 }
-                if (cn) cstr <<= 64u - cn;                     // first correction bit at bit 63
                 ulonglong2* o = reinterpret_cast<ulonglong2*>(outp + (uint64_t)block_index(m0 + lane) * 4);
                 o[0] = make_ulonglong2((L.h[lane] | Nw), cstr);
                 o[1] = make_ulonglong2(Nw, NS);

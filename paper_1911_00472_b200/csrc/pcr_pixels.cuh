@@ -225,10 +225,11 @@ __global__ void __launch_bounds__(kPixThreads, PCR_PIX_MIN_CTAS) pixel_kernel(Pa
                         a = __ldg(o); b = __ldg(o + 1);
                     }
                     // corrections: the coefficients that were non-zero before the scan, in zigzag order, take the
-                    // correction bits in reading order (from bit 63 down); the walk ends with the last set bit.
+                    // correction bits in reading order (as many as there are such positions, the last one in bit 0);
+                    // the walk ends with the last set bit.
                     // Positions 0..31 and 32..63 are walked as 32-bit masks.
                     const uint64_t hist = a.x & ~b.x;
-                    uint64_t cc = a.y;
+                    uint64_t cc = a.y ? a.y << (64 - __popcll(hist)) : 0ull;
 #pragma unroll
                     for (int half = 0; half < 2; ++half) {
                         uint32_t h32 = half ? (uint32_t)(hist >> 32) : (uint32_t)hist;

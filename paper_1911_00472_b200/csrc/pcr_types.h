@@ -15,7 +15,7 @@ struct ScanScript {
 // indexed by the block's number inside its component across the whole record):
 //  - a first-pass AC scan writes one word per block: the mask of zigzag positions it made non-zero;
 //  - an AC refinement scan writes four words per block: {mask of non-zero positions of its band
-//    after the scan, correction bits in reading order (first bit at bit 63), mask of newly
+//    after the scan, correction bits in reading order (last bit at bit 0), mask of newly
 //    non-zero positions, mask of those that are positive}.  The coefficient planes are updated
 //    from these by the pixel kernel.
 // A refinement scan finds the positions that were non-zero before it by OR-ing the masks of up
@@ -25,6 +25,8 @@ struct ScanAux {
     uint32_t stride;      // words per block: 1 or 4
     int32_t nsrc;
     int32_t src[4];       // scan indices
+    uint32_t tab0;        // first of the scan's lookup tables (see ScanTab): image i has ntab of them from tab0 + i * ntab on
+    int32_t ntab;         // 2 for a DC first pass, 1 for an AC scan, 4 for a sequential scan, 0 for a DC refinement
 };
 
 // Refinement scans to apply per component, in scan order (built per decode for the chosen k).
@@ -82,6 +84,8 @@ struct Unit {
     uint16_t mrow, mcol0;
 };
 
+struct ScanTab;             // lookup table of one Huffman table (pcr_entropy.cuh)
+
 struct Params {
     const uint8_t* rec;         // record bytes on the device
     uint8_t* ubuf;              // entropy-coded bytes without stuffing, big-endian words
@@ -102,6 +106,7 @@ struct Params {
     const uint16_t* qtab;       // [N][3][64] quantisers, zigzag order
     uint8_t* chroma;            // chroma sample planes (triangle upsampling only): per image, at 128 bytes
                                 // per MCU in front of it, a Cb plane then a Cr plane of 8*my rows x 8*mx bytes
+    ScanTab* tabs;              // lookup tables of the decoded scans, by ScanAux::tab0
     const uint32_t* order;      // [N] processing order of the images
     const CropRect* roi;        // [N] or null: only work units that touch the image's rectangle are transformed
     int* status;                // [N]
