@@ -76,73 +76,7 @@ __device__ __forceinline__ void build_hufftab(HuffTabT<kBits>& t, const uint8_t*
     __syncwarp();
 }
 
-// MSB-first bit reader over the unstuffed copy of the entropy-coded bytes (see
-// unstuff_index_kernel), which holds big-endian 32-bit words.  Each lane owns one column of a
-// 16-word ring in shared memory.  All lanes of the warp top their rings up together
-// (16-byte global loads), then decode for a while reading single words from the ring: the
-// serial decode chain only ever waits on shared memory, and the latency of global memory is
-// paid once per top-up for the whole warp instead of once per lane and load.
-constexpr int kRingWords = 16;
-
-struct BitReader {
-    uint32_t* col;        // this lane's ring column: word j lives at col[(j & 15) * 32]
-    const uint4* g4;      // the unstuffed copy as 16-byte groups
-    uint32_t rd, wr;      // next word to consume / to fetch (absolute word indices, wr a multiple of 4)
-    uint32_t rd0;         // first word of the restart interval
-    uint64_t buf;         // left-aligned bit buffer
-    int nbits;            // bits held in buf
-    uint32_t lead;        // bits of the first word that precede the interval
-    uint32_t limit;       // bits in the restart interval
-
-    __device__ __forceinline__ void init(uint32_t* ring_col, const uint8_t* ubuf, uint32_t bstart, uint32_t bend) {
-        col = ring_col;
-        g4 = reinterpret_cast<const uint4*>(ubuf);
-        rd = rd0 = bstart >> 2;
-        wr = rd & ~3u;
-        buf = 0; nbits = 0;
-        lead = 8u * (bstart & 3u);
-        limit = (bend - bstart) * 8u;
-    }
-    // fetch as many 16-byte groups as the ring has room for (all lanes call this together)
-    __device__ __forceinline__ void topup(bool on) {
-        const int room = on ? (int)(kRingWords - (wr - rd)) >> 2 : 0;
-        uint4 v0, v1, v2, v3;
-        if (room > 0) v0 = __ldg(g4 + (wr >> 2));
-        if (room > 1) v1 = __ldg(g4 + (wr >> 2) + 1);
-        if (room > 2) v2 = __ldg(g4 + (wr >> 2) + 2);
-        if (room > 3) v3 = __ldg(g4 + (wr >> 2) + 3);
-        if (room > 0) put(wr, v0);
-        if (room > 1) put(wr + 4, v1);
-        if (room > 2) put(wr + 8, v2);
-        if (room > 3) put(wr + 12, v3);
-        wr += 4u * (uint32_t)max(room, 0);
-    }
-    __device__ __forceinline__ void put(uint32_t w, const uint4& v) {
-        uint32_t* p = col + (w & (kRingWords - 1)) * 32;
-        p[0] = v.x; p[32] = v.y; p[64] = v.z; p[96] = v.w;
-    }
-    // enough words in the ring for one whole decode step (a code, its extra bits, 63 raw bits)
-    __device__ __forceinline__ bool ready() const { return wr - rd >= 3u; }
-    // once, after the first top-up: take the first word without the bytes that precede the interval
-    __device__ __forceinline__ void prime() {
-        const uint32_t w = col[(rd & (kRingWords - 1)) * 32] << lead;
-        buf = (uint64_t)w << 32;
-        nbits = 32 - (int)lead;
-        ++rd;
-    }
-    // afterwards at least 33 bits are held
-    __device__ __forceinline__ void refill() {
-        if (nbits <= 32) {
-            const uint32_t w = col[(rd & (kRingWords - 1)) * 32];
-            buf |= (uint64_t)w << (32 - nbits);
-            nbits += 32;
-            ++rd;
-        }
-    }
-    __device__ __forceinline__ uint32_t top32() const { return (uint32_t)(buf >> 32); }
-    __device__ __forceinline__ void skip(int n) { buf <<= n; nbits -= n; }
-    __device__ __forceinline__ bool overran() const { return (int)((rd - rd0) * 32u - lead) - nbits > (int)limit; }
-};
+constexpr int kRingWords = 16;       // words of the bitstream a lane of the interval kernels holds in shared memory
 
 // Huffman symbol at the top of the 32-bit window; returns (length << 8) | symbol, 0 if undefined
 template <int kBits>
@@ -537,6 +471,13 @@ __device__ __forceinline__ uint4 rank_index(uint64_t z) {
     return make_uint4(z0, z1, c0 * 0x01010101u, (c1 + low) * 0x01010101u);
 }
 
+// side data of a block of a first pass that reaches beyond position 7: the mask of its positions and where its
+// values for positions 8..63 begin
+__device__ __forceinline__ uint4 value_record(uint32_t m0, uint32_t m1, const int16_t* first) {
+    const uint64_t a = reinterpret_cast<uint64_t>(first);
+    return make_uint4(m0, m1, (uint32_t)a, (uint32_t)(a >> 32));
+}
+
 constexpr int kDecodeSteps = 16;     // decode steps between two top-ups of the rings
 constexpr int kMaskQueue = 8;        // blocks whose masks a refinement lane holds ahead
 
@@ -631,7 +572,7 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, u
         // block numbers inside the image: the MCU's first luminance block (or the scan's own component) and its chroma blocks
         const uint32_t hs = inter ? (uint32_t)P.hs : 1u, vs = inter ? (uint32_t)P.vs : 1u, bw0 = g.bw[inter ? 0 : c0];
         const uint32_t y_off = inter ? 0u : (uint32_t)(g.coff[c0] - im.blk_base), c_off = (uint32_t)(g.coff[1] - im.blk_base), c_step = g.mx * g.my;
-        int16_t* const head = P.head + im.blk_base * 8;
+        int16_t* const dcp = P.dc + im.blk_base;
         for (;;) {
             br.topup(!done);
             __syncwarp(full);
@@ -660,7 +601,7 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, u
                     if (j < ny || !inter) { pv = (pred0 += d); blk = yb + ((uint32_t)j & (hs - 1u)) + ((uint32_t)j >> (hs - 1u)) * bw0; }
                     else if (j == ny) { pv = (pred1 += d); blk = cb; }
                     else { pv = (pred2 += d); blk = cb + c_step; }
-                    head[(uint64_t)blk * 8] = (int16_t)(pv << Al);
+                    dcp[blk] = (int16_t)(pv << Al);
                 }
                 ++m;
                 if (++mcol == mcu_w) { mcol = 0; ++mrow; }
@@ -679,9 +620,12 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, u
         uint32_t bi = (m0 / mcu_w) * bw + bcol;            // block index inside the image's component
         if (!kRefine || sc.Ah == 0) {
             // ---- AC first pass: one Huffman symbol per step
-            uint64_t* maskp = P.aux + ax.base + g.loff[c];
-            int16_t* plane = P.planes + g.coff[c] * 64;
+            uint64_t* auxp = P.aux + ax.base + g.loff[c] * ax.stride;
             int16_t* headp = P.head + g.coff[c] * 8;
+            const bool lists = ax.stride == 2u;            // the band reaches beyond position 7
+            int16_t* vp = P.vals + 4ull * bstart;           // next value
+            int16_t* vb = vp;                               // the block's first one
+            uint32_t wrap_m = m + mcu_w - bcol;             // the first block of the next block row
             uint32_t M0 = 0, M1 = 0, k = Ss;
             for (;;) {
                 br.topup(!done);
@@ -690,32 +634,36 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, u
                 uint32_t stop = done ? 0u : min(br.ring_stop(2), br.limit + 1u);
 #pragma unroll 1
                 for (int t = 0; t < kDecodeSteps; ++t) {
-                    if (br.pos >= stop) continue;
-                    const uint32_t win = br.window(br.pos);
-                    uint32_t e = lds16(tab + ((win >> (32 - kTabBits)) << 1));
-                    if (e == 0) e = long_code(tab, win, kTabAcFirst);
-                    const uint32_t skip = e & 31u, sz = (e >> 5) & 15u, r = (e >> 9) & 15u;
-                    br.pos += skip;
-                    k += r;                                                // position of the coefficient
-                    if (e == 0 || (sz && k > Se)) { bad = true; stop = 0; continue; }
-                    if (sz) {
-                        const int16_t val = (int16_t)(magnitude(win, skip, sz) << Al);
-                        int16_t* dst = k < 8u ? headp + ((uint64_t)bi * 8 + k) : plane + ((uint64_t)bi * 64 + k);
-                        *dst = val;
-                        M0 |= shl0(1u, k); M1 |= shl0(1u, k - 32u);
-                    }
-                    ++k;                                                   // (sixteen zeros: run 15 plus one)
-                    const bool is_eob = (e & kEntEob) != 0;
-                    if (is_eob || k > Se) {
-                        if (M0 | M1) *reinterpret_cast<uint2*>(maskp + bi) = make_uint2(M0, M1);
-                        k = Ss; M0 = 0; M1 = 0;
-                        ++m; ++bi;
-                        if (++bcol == mcu_w) { bcol = 0; bi += wrap - 1u; }
-                        if (is_eob && r) {                                 // the following blocks of the run are empty
-                            m = min(m - 1u + (1u << r) + shr0(shl0(win, skip - r), 32u - r), m1);
-                            bcol = m % mcu_w; bi = (m / mcu_w) * bw + bcol;
+                    if (br.pos < stop) {
+                        const uint32_t win = br.window(br.pos);
+                        uint32_t e = lds16(tab + ((win >> (32 - kTabBits)) << 1));
+                        if (e == 0) e = long_code(tab, win, kTabAcFirst);
+                        const uint32_t skip = e & 31u, sz = (e >> 5) & 15u, r = (e >> 9) & 15u;
+                        br.pos += skip;
+                        k += r;                                            // position of the coefficient
+                        if (sz && k <= Se) {
+                            const int16_t val = (int16_t)(magnitude(win, skip, sz) << Al);
+                            if (k < 8u) headp[(uint64_t)bi * 8 + k] = val;
+                            else *vp++ = val;
+                            M0 |= shl0(1u, k); M1 |= shl0(1u, k - 32u);
+                        } else if (e == 0 || sz) { bad = true; stop = 0; k = 0; }   // no such symbol, or a coefficient behind the band
+                        ++k;                                               // (sixteen zeros: run 15 plus one)
+                        const bool is_eob = (e & kEntEob) != 0;
+                        if (is_eob || k > Se) {
+                            if (M0 | M1) {
+                                if (lists) *reinterpret_cast<uint4*>(auxp + (uint64_t)bi * 2) = value_record(M0, M1, vb);
+                                else *reinterpret_cast<uint2*>(auxp + bi) = make_uint2(M0, M1);
+                            }
+                            k = Ss; M0 = 0; M1 = 0; vb = vp;
+                            // an end of band may leave the following blocks empty too
+                            const uint32_t adv = is_eob ? (1u << r) + shr0(shl0(win, skip - r), 32u - r) : 1u;
+                            m += adv; bi += adv;
+                            if (m >= wrap_m) {                             // (rows in between only where an interval holds several)
+                                if (m >= m1) stop = 0;
+                                else { const uint32_t row = m / mcu_w; bi = row * bw + (m - row * mcu_w); wrap_m = (row + 1u) * mcu_w; }
+                            }
+                            if (m >= m1) stop = 0;
                         }
-                        if (m >= m1) stop = 0;
                     }
                 }
                 __syncwarp(full);
@@ -877,21 +825,23 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, u
 // Sequential (baseline) scans: one interleaved scan carries, block after block, the DC difference
 // and then the AC coefficients up to an end-of-block symbol.  Same decomposition as above (one
 // lane per restart interval, one Huffman symbol per step), four tables per warp (DC and AC,
-// luminance and chrominance).  Coefficients go where the progressive first passes put them:
-// zigzag positions 0..7 into the dense head plane, the rest into the block's line.
+// luminance and chrominance).  A block's first symbol goes through the same instructions as the others (its entry
+// has no run, its value is the difference): lanes stand at different kinds of symbol in every step.
+// Coefficients go where the progressive first passes put them.
 // ---------------------------------------------------------------------------------------
 constexpr int kSeqWarps = 2;
+constexpr uint32_t kSeqWarpBytes = 4 * sizeof(ScanTab) + (kRingWords + 1) * 128;
 
 template <bool kRoi>
 __global__ void __launch_bounds__(32 * kSeqWarps) sequential_kernel(Params P, uint32_t item_begin, uint32_t item_count) {
-    __shared__ HuffTab tabs[kSeqWarps][4];                    // DC 0, DC 1, AC 0, AC 1
-    __shared__ uint32_t s_ring[kSeqWarps][kRingWords][32];
+    __shared__ __align__(16) uint8_t s_seq[kSeqWarps * kSeqWarpBytes];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t it = blockIdx.x * kSeqWarps + wid;
     if (it >= item_count) return;                             // whole warp
     const Item item = P.items[item_begin + it];
     const ScanDesc sd = P.scans[item.si];
     const int img = (int)(item.si % (uint32_t)P.N);
+    const ScanAux ax = P.saux[item.si / (uint32_t)P.N];
     bool done = (uint32_t)lane >= item.count;
     uint32_t seg = item.seg0 + lane;
     if (seg >= sd.nseg) { done = true; seg = 0; }
@@ -911,74 +861,84 @@ __global__ void __launch_bounds__(32 * kSeqWarps) sequential_kernel(Params P, ui
         }
         if (__all_sync(full, done)) return;
     }
-    build_hufftab(tabs[wid][0], P.rec + sd.tab_off[0], lane);
-    if (sd.tab_off[1]) build_hufftab(tabs[wid][1], P.rec + sd.tab_off[1], lane);
-    build_hufftab(tabs[wid][2], P.rec + sd.tab_ac[0], lane);
-    if (sd.tab_ac[1]) build_hufftab(tabs[wid][3], P.rec + sd.tab_ac[1], lane);
+    const uint32_t mem = (uint32_t)__cvta_generic_to_shared(s_seq) + (uint32_t)wid * kSeqWarpBytes;
+    {
+        const uint4* a = reinterpret_cast<const uint4*>(P.tabs + ax.tab0 + 4u * (uint32_t)img);
+        for (int i = lane; i < (int)(4 * sizeof(ScanTab) / 16); i += 32) sts128(mem + 16 * i, __ldg(a + i));
+    }
     const uint32_t* segtab = P.seg_start + sd.seg_base;
     uint32_t bstart = segtab[seg];
     uint32_t bend = segtab[seg + 1] - 2;
     bool bad = false;
     if (!done && (bstart < sd.data_off || bend > sd.data_end || bend < bstart)) { bad = true; done = true; }
     if (done) { bstart = sd.data_off; bend = sd.data_off; }
-    BitReader br;
-    br.init(&s_ring[wid][0][lane], P.ubuf, bstart, bend);
-    br.topup(!done);
-    br.prime();
+    LaneBits br;
+    br.init(mem + 4u * (uint32_t)sizeof(ScanTab) + 4u * lane, P.ubuf, bstart, bend);
+    if (m0 >= m1) done = true;
 
+    const uint32_t ny = (uint32_t)(P.hs * P.vs), bpm = P.nc == 3 ? ny + 2u : 1u;      // blocks per MCU (a lone component: one block, no padding)
+    const uint32_t hs = (uint32_t)P.hs, vs = (uint32_t)P.vs, bw0 = g.bw[0], c_off = ny * total;
     uint32_t m = m0, mrow = m0 / mcu_w, mcol = m0 % mcu_w;
-    const int bpm = P.nc == 3 ? P.hs * P.vs + 2 : 1;      // blocks per MCU (a lone component: one block, no padding)
-    int j = 0;                                            // block inside the MCU: the luminance blocks, Cb, Cr
-    int k = 0;                                            // 0: the block's DC symbol comes next
+    uint32_t j = 0, c = 0;                                // block inside the MCU (the luminance blocks, Cb, Cr), its component
+    uint32_t ci = vs * mrow * bw0 + hs * mcol;            // its number inside the image's component
+    uint32_t k = 0, M0 = 0, M1 = 0;                       // position (0: the block's DC symbol comes next), mask
+    int16_t* vp = P.vals + 4ull * bstart;
+    int16_t* vb = vp;
     int pred0 = 0, pred1 = 0, pred2 = 0;
-    if (m >= m1) done = true;
+    const uint32_t slots = sd.slots, slots_ac = sd.slots_ac;
+    constexpr uint32_t kTab = (uint32_t)sizeof(ScanTab);
+    uint32_t tdc = mem + (slots & 1u) * kTab, tac = mem + (2u + (slots_ac & 1u)) * kTab;
+    int16_t* const dcp = P.dc + im.blk_base;
+    int16_t* const headp = P.head + im.blk_base * 8;
     for (;;) {
         br.topup(!done);
         __syncwarp(full);
         if (__all_sync(full, done)) break;
+        uint32_t stop = done ? 0u : min(br.ring_stop(2), br.limit + 1u);
 #pragma unroll 1
         for (int t = 0; t < kDecodeSteps; ++t) {
-            if (done || !br.ready()) continue;
-            br.refill();
-            const uint32_t win = br.top32();
-            int c = 0;
-            const uint64_t blk = P.nc == 3 ? mcu_block(g, P, mrow, mcol, j, &c) : g.coff[0] + (uint64_t)mrow * g.bw[0] + mcol;
-            const bool is_dc = k == 0;
-            const int ti = is_dc ? (int)((sd.slots >> (2 * c)) & 1u) : 2 + (int)((sd.slots_ac >> (2 * c)) & 1u);
-            const HuffTab& tab = tabs[wid][ti];
-            uint32_t e = tab.lut[win >> (32 - kLutBits)];
-            if (e == 0) e = huff_lookup(tab, win);
-            const int len = (int)(e >> 8), r = is_dc ? 0 : (int)(e >> 4) & 15, sz = is_dc ? (int)(e & 255u) : (int)(e & 15u);
-            const bool is_coef = sz != 0, is_zrl = !is_dc && sz == 0 && r == 15, is_eob = !is_dc && sz == 0 && r == 0;
-            const int kk = k + r;
-            const bool fail = e == 0 || sz > 15 || (!is_dc && !is_coef && !is_zrl && !is_eob) || (is_coef && kk > 63);
-            if (fail) { bad = true; done = true; continue; }
-            const int extra = is_coef ? sz : 0;
-            const int v = extend_bits(top_bits(win << len, extra), extra);
-            br.skip(len + extra);
-            if (is_dc) {
-                const int pv = (c == 0 ? pred0 : (c == 1 ? pred1 : pred2)) + v;
-                if (c == 0) pred0 = pv; else if (c == 1) pred1 = pv; else pred2 = pv;
-                P.head[blk * 8] = (int16_t)pv;
-                k = 1;
-            } else if (is_coef) {
-                if (kk < 8) P.head[blk * 8 + kk] = (int16_t)v;
-                else P.planes[blk * 64 + kk] = (int16_t)v;
-                k = kk + 1;
-            } else if (is_zrl) {
-                k += 16;
-            }
-            if (is_eob || k > 63) {                       // block finished
-                k = 0;
-                if (++j == bpm) {
-                    j = 0; ++m;
-                    if (++mcol == mcu_w) { mcol = 0; ++mrow; }
+            if (br.pos < stop) {
+                const uint32_t win = br.window(br.pos);
+                const bool is_dc = k == 0;
+                const uint32_t tab = is_dc ? tdc : tac;
+                uint32_t e = lds16(tab + ((win >> (32 - kTabBits)) << 1));
+                if (e == 0) e = long_code(tab, win, is_dc ? kTabDc : kTabAcSeq);
+                const uint32_t skip = e & 31u, sz = (e >> 5) & 15u;
+                br.pos += skip;
+                k += (e >> 9) & 15u;
+                int v = magnitude(win, skip, sz);
+                if (is_dc) {
+                    v += c == 0 ? pred0 : (c == 1 ? pred1 : pred2);
+                    if (c == 0) pred0 = v; else if (c == 1) pred1 = v; else pred2 = v;
+                }
+                const bool fail = e == 0 || k > 63u;                       // (sixteen zeros may end behind position 63)
+                const uint32_t blk = (c ? c_off + (c - 1u) * total : 0u) + ci;      // block number inside the image
+                if (!fail && (sz || is_dc)) {
+                    if (k >= 8u) *vp++ = (int16_t)v;
+                    else if (k) headp[(uint64_t)blk * 8 + k] = (int16_t)v;
+                    else dcp[blk] = (int16_t)v;
+                    M0 |= shl0(1u, k); M1 |= shl0(1u, k - 32u);
+                }
+                if (e == 0 || (sz && k > 63u)) { bad = true; stop = 0; k = 0; }
+                ++k;
+                if ((e & kEntEob) || k > 63u) {                            // block finished
+                    if (M1 | (M0 >> 8)) *reinterpret_cast<uint4*>(P.aux + (c ? ax.base_c[c - 1u] : ax.base) + 2ull * ((c ? g.loff[1] : g.loff[0]) + ci)) = value_record(M0 & ~1u, M1, vb);
+                    k = 0; M0 = 0; M1 = 0; vb = vp;
+                    ++j;
+                    if (j == bpm) {
+                        j = 0; ++m;
+                        if (++mcol == mcu_w) { mcol = 0; ++mrow; }
+                        if (m >= m1) stop = 0;
+                    }
+                    c = j < ny ? 0u : j - ny + 1u;
+                    ci = c ? mrow * mcu_w + mcol : (vs * mrow + (j >> (hs - 1u))) * bw0 + hs * mcol + (j & (hs - 1u));
+                    tdc = mem + ((slots >> (2u * c)) & 1u) * kTab; tac = mem + (2u + ((slots_ac >> (2u * c)) & 1u)) * kTab;
                 }
             }
-            if (br.overran()) { bad = true; done = true; }
-            if (m >= m1) done = true;
         }
         __syncwarp(full);
+        bad = bad || br.pos > br.limit;
+        done = done || bad || m >= m1;
     }
     if (bad) atomicMin(&P.status[img], kErrCorrupt);
 }

@@ -136,7 +136,7 @@ struct pcr_record {
     std::vector<uint64_t> blk_base, nblk;
     uint64_t total_blocks = 0, total_segs = 0;
     int hs = 2, vs = 2, nc = 3;     // chroma sampling, the same for every image of the record
-    uint32_t unit_mcus = kPixMcus;  // MCUs of a pixel work unit
+    uint32_t unit_mcus = 8, unit_rows = 2;   // MCUs across and MCU rows of a pixel work unit
     unsigned dc_refine_chunks = 1;  // 256-MCU chunks of the largest image, at most 8 (dc_refine_kernel's grid)
     bool widths_mult16 = true;    // every image is a multiple of 16 pixels wide (the DC-only pixel kernel's condition)
     size_t out_bytes = 0;
@@ -176,11 +176,13 @@ struct pcr_record {
     uint8_t* d_rec = nullptr;
     uint8_t* d_ubuf = nullptr;
     size_t resident = 0;
-    int16_t* d_planes = nullptr;
+    int16_t* d_planes = nullptr;  // canonical planes (allocated when pcr_coeffs first asks for them)
+    int16_t* d_dc = nullptr;
     int16_t* d_head = nullptr;
+    int16_t* d_vals = nullptr;
     int decoded_k = 0;            // fidelity of the state the planes and side data hold (0: none)
-    bool dc_merged = true;        // the planes hold the DC coefficients of the last decode
-    bool planes_cleared = true;   // ... and zeros wherever the last decode left no coefficient
+    int lists_k = 0;              // fidelity of the last decode, whatever rows it decoded
+    bool planes_current = false;  // d_planes holds the coefficients of the last decode
     ScanTab* d_tabs = nullptr;
     ScanScript* d_script = nullptr;
     ScanAux* d_saux = nullptr;
@@ -226,13 +228,13 @@ static inline uint64_t rd64(const uint8_t* p) { return (uint64_t)rd32(p) | ((uin
 
 // Writes the list of pixel work units at set-up: block = position of the processing order.
 __global__ void __launch_bounds__(128) units_kernel(const ImgDesc* __restrict__ imgs, const uint32_t* __restrict__ order,
-                                                    const uint32_t* __restrict__ prefix, Unit* __restrict__ units, uint32_t unit_mcus) {
+                                                    const uint32_t* __restrict__ prefix, Unit* __restrict__ units, uint32_t unit_mcus, uint32_t unit_rows) {
     const uint32_t img = order[blockIdx.x];
-    const uint32_t per_row = (imgs[img].mx + unit_mcus - 1) / unit_mcus, n = per_row * imgs[img].my;
+    const uint32_t per_row = (imgs[img].mx + unit_mcus - 1) / unit_mcus, n = per_row * ((imgs[img].my + unit_rows - 1) / unit_rows);
     Unit* dst = units + prefix[blockIdx.x];
     for (uint32_t j = threadIdx.x; j < n; j += 128) {
         Unit un;
-        un.img = img; un.mrow = (uint16_t)(j / per_row); un.mcol0 = (uint16_t)((j % per_row) * unit_mcus);
+        un.img = img; un.mrow = (uint16_t)(j / per_row * unit_rows); un.mcol0 = (uint16_t)((j % per_row) * unit_mcus);
         dst[j] = un;
     }
 }
@@ -539,7 +541,8 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     uint64_t blocks = 0, out_off = 0, segs = 0;
     r->hs = samplings[0] & 3; r->vs = (samplings[0] >> 2) & 3; r->nc = samplings[0] >> 4;
     const uint32_t bpm = (uint32_t)(r->hs * r->vs + (r->nc == 3 ? 2 : 0));      // blocks per MCU
-    r->unit_mcus = r->nc == 3 && r->hs == 2 ? 8u : 16u;                         // a work unit is 128 pixels wide
+    r->unit_mcus = kUnitMcus[sampling_code(r->hs, r->vs, r->nc)];
+    r->unit_rows = kUnitRows[sampling_code(r->hs, r->vs, r->nc)];
     for (uint32_t g = 0; g < G; ++g) r->script[g] = scripts[g];
     for (uint32_t i = 0; i < N; ++i) {
         if (i && memcmp(&scripts[(size_t)i * G], &scripts[0], sizeof(ScanScript) * G) != 0) return PCR_E_FORMAT;   // one script per record
@@ -698,13 +701,13 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
                 if (!items.empty() && items.back().next == kItemOpen) items.back().next = 0;
                 r->item_count[(size_t)g * G + s] = (uint32_t)items.size() - r->item_begin[(size_t)g * G + s];
             }
-    // pixel work units (8 MCUs of one MCU row), image by image in processing order, inside an image
+    // pixel work units (see Sampling in pcr_pixels.cuh), image by image in processing order, inside an image
     // MCU row by MCU row.  The host only counts them; a small kernel writes the list at set-up.
     std::vector<uint32_t> unit_prefix(N + 1, 0);
     for (uint32_t pos = 0; pos < N; ++pos) {
         const ImgDesc& im = imgs[order[pos]];
         if (im.my > 65535 || im.mx > 65535) return PCR_E_FORMAT;
-        const uint64_t nu = (uint64_t)((im.mx + r->unit_mcus - 1) / r->unit_mcus) * im.my;
+        const uint64_t nu = (uint64_t)((im.mx + r->unit_mcus - 1) / r->unit_mcus) * ((im.my + r->unit_rows - 1) / r->unit_rows);
         if (unit_prefix[pos] + nu >= (1ull << 32)) return PCR_E_FORMAT;
         unit_prefix[pos + 1] = unit_prefix[pos] + (uint32_t)nu;
     }
@@ -726,10 +729,11 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
         ax.ntab = sc.Ss > 0 ? 1 : (sc.Se == 63 ? 4 : (sc.Ah == 0 ? 2 : 0));
         ax.tab0 = (uint32_t)n_tabs;
         n_tabs += (uint64_t)N * (uint64_t)ax.ntab;
-        if (sc.Ss == 0) continue;
-        ax.stride = sc.Ah ? 4u : 1u;
+        if (sc.Ss == 0 && sc.Se != 63) continue;
+        ax.stride = sc.Ah ? 4u : (sc.Se >= 8 ? 2u : 1u);
         ax.base = aux_words;
         aux_words += (sc.comp[0] == 0 ? (uint64_t)(r->hs * r->vs) : 1ull) * total_mcus * ax.stride;
+        for (int c = 1; sc.Ss == 0 && c < r->nc; ++c) { ax.base_c[c - 1] = aux_words; aux_words += 2 * total_mcus; }
         aux_words = (aux_words + 1) & ~1ull;      // 16-byte alignment of every scan's area
         if (sc.Ah) {
             // positions already non-zero = union of the masks of earlier scans on this band; an
@@ -765,7 +769,9 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     if (int rc = take(r, &r->d_ubuf, (size_t)(len + 256))) return rc;
     zero.push_back({r->d_ubuf, len + 256});
     if (int rc = take(r, &r->d_tabs, (size_t)(std::max<uint64_t>(n_tabs, 1) * sizeof(ScanTab)))) return rc;
-    if (int rc = take(r, &r->d_planes, (size_t)(std::max<uint64_t>(blocks, 1) * 128))) return rc;
+    if (int rc = take(r, &r->d_vals, (size_t)(8 * (len + 256)))) return rc;      // four values per byte, two bytes each
+    if (int rc = take(r, &r->d_dc, (size_t)(std::max<uint64_t>(blocks, 1) * 2))) return rc;
+    zero.push_back({r->d_dc, (size_t)(std::max<uint64_t>(blocks, 1) * 2)});
     if (int rc = take(r, &r->d_head, (size_t)(std::max<uint64_t>(blocks, 1) * 16))) return rc;
     zero.push_back({r->d_head, (size_t)(std::max<uint64_t>(blocks, 1) * 16)});
     if (int rc = take(r, &r->d_seg, (size_t)((segs + 1) * 4))) return rc;
@@ -789,7 +795,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     if ((rc = upload(r, &r->d_unit_prefix, unit_prefix))) return rc;
     if ((rc = take(r, &r->d_units, (size_t)std::max<uint32_t>(r->n_units, 1) * sizeof(Unit)))) return rc;
     if ((rc = upload(r, &r->d_order, order))) return rc;
-    units_kernel<<<N, 128, 0, r->up_stream>>>(r->d_imgs, r->d_order, r->d_unit_prefix, r->d_units, r->unit_mcus);
+    units_kernel<<<N, 128, 0, r->up_stream>>>(r->d_imgs, r->d_order, r->d_unit_prefix, r->d_units, r->unit_mcus, r->unit_rows);
     ++g_launches;
     for (auto& z : zero)
         if (cudaMemsetAsync(z.first, 0, z.second, r->up_stream) != cudaSuccess) return PCR_E_CUDA;
@@ -914,7 +920,7 @@ int pcr_open(const void* bytes, size_t len, pcr_record** rec) {
             g_rcache.lru.erase(g_rcache.lru.begin() + (long)i);
             g_rcache.bytes -= c->device_bytes;
             // a fresh handle: nothing resident, nothing decoded, default settings
-            c->resident = 0; c->decoded_k = 0; c->upsampling = PCR_UPSAMPLE_REPLICATE; c->profiling = false;
+            c->resident = 0; c->decoded_k = 0; c->lists_k = 0; c->planes_current = false; c->upsampling = PCR_UPSAMPLE_REPLICATE; c->profiling = false;
             c->decode_enqueued = false;
             *rec = c;
             return PCR_OK;
@@ -969,10 +975,86 @@ int pcr_evict(pcr_record* rec) {
 
 }  // extern "C"
 
+// The pixel kernels of one slice at one fidelity (see pcr_pixels.cuh for what the template arguments choose).
+struct PixelPlan { bool dc_only, head_only, refine, widths_mult16, triangle, roi; int samp; };
+
 template <int kSamp>
-static void launch_pixels_sampled(bool refine, unsigned grid, cudaStream_t q, const Params& Q, const FinalizeList& fl, uint8_t* o8) {
-    if (refine) pixel_kernel<true, 1, false, 0, kSamp><<<grid, kPixThreads, 0, q>>>(Q, fl, o8);
-    else pixel_kernel<false, 1, false, 0, kSamp><<<grid, kPixThreads, 0, q>>>(Q, fl, o8);
+static void launch_pixels_sampled(const PixelPlan& pl, unsigned grid, cudaStream_t q, const Params& Q, const CoefLists& cl, uint8_t* o8) {
+    constexpr int T = unit_threads<kSamp>();
+    if (pl.refine) pixel_kernel<true, 1, false, 0, kSamp><<<grid, T, 0, q>>>(Q, cl, o8);
+    else pixel_kernel<false, 1, false, 0, kSamp><<<grid, T, 0, q>>>(Q, cl, o8);
+}
+
+template <bool kRoi>
+static void launch_pixels_420(const PixelPlan& pl, unsigned grid, cudaStream_t q, const Params& Q, const CoefLists& cl, uint8_t* o8) {
+    constexpr int T = unit_threads<kSamp420>();
+    if (pl.dc_only && pl.widths_mult16) dc_pixel_kernel<kRoi><<<grid, 128, 0, q>>>(Q, o8);
+    else if (pl.dc_only) dc_pixel_kernel<kRoi, false><<<grid, 128, 0, q>>>(Q, o8);
+    else if (pl.head_only) pixel_kernel<false, 3, kRoi><<<grid, T, 0, q>>>(Q, cl, o8);
+    else if (pl.refine) pixel_kernel<true, 1, kRoi><<<grid, T, 0, q>>>(Q, cl, o8);
+    else pixel_kernel<false, 1, kRoi><<<grid, T, 0, q>>>(Q, cl, o8);
+}
+
+static void launch_pixels(const PixelPlan& pl, unsigned grid, cudaStream_t q, const Params& Q, const CoefLists& cl, uint8_t* o8) {
+    constexpr int T = unit_threads<kSamp420>();
+    if (pl.samp == kSamp422) launch_pixels_sampled<kSamp422>(pl, grid, q, Q, cl, o8);
+    else if (pl.samp == kSamp440) launch_pixels_sampled<kSamp440>(pl, grid, q, Q, cl, o8);
+    else if (pl.samp == kSamp444) launch_pixels_sampled<kSamp444>(pl, grid, q, Q, cl, o8);
+    else if (pl.samp == kSampGrey) launch_pixels_sampled<kSampGrey>(pl, grid, q, Q, cl, o8);
+    else if (pl.roi) launch_pixels_420<true>(pl, grid, q, Q, cl, o8);
+    else if (pl.triangle) {
+        // chroma pass (samples of every chroma block into the sample planes), then the pixel pass
+        pixel_kernel<true, 1, false, 1><<<grid, T, 0, q>>>(Q, cl, o8);
+        pixel_kernel<true, 1, false, 2><<<grid, T, 0, q>>>(Q, cl, o8);
+        ++g_launches;
+    } else launch_pixels_420<false>(pl, grid, q, Q, cl, o8);
+    ++g_launches;
+}
+
+// The expanded blocks of the whole record into the canonical planes.
+static void launch_planes(int samp, unsigned grid, const Params& Q, const CoefLists& cl) {
+    if (samp == kSamp422) pixel_kernel<true, 1, false, 3, kSamp422><<<grid, unit_threads<kSamp422>()>>>(Q, cl, nullptr);
+    else if (samp == kSamp440) pixel_kernel<true, 1, false, 3, kSamp440><<<grid, unit_threads<kSamp440>()>>>(Q, cl, nullptr);
+    else if (samp == kSamp444) pixel_kernel<true, 1, false, 3, kSamp444><<<grid, unit_threads<kSamp444>()>>>(Q, cl, nullptr);
+    else if (samp == kSampGrey) pixel_kernel<true, 1, false, 3, kSampGrey><<<grid, unit_threads<kSampGrey>()>>>(Q, cl, nullptr);
+    else pixel_kernel<true, 1, false, 3, kSamp420><<<grid, unit_threads<kSamp420>()>>>(Q, cl, nullptr);
+    ++g_launches;
+}
+
+static Params record_params(const pcr_record* rec) {
+    Params P;
+    memset(&P, 0, sizeof P);
+    P.rec = rec->d_rec; P.ubuf = rec->d_ubuf; P.planes = rec->d_planes; P.dc = rec->d_dc; P.head = rec->d_head; P.vals = rec->d_vals;
+    P.script = rec->d_script; P.scans = rec->d_scans;
+    P.saux = rec->d_saux; P.aux = rec->d_aux;
+    P.imgs = rec->d_imgs; P.seg_start = rec->d_seg; P.items = rec->d_items; P.units = rec->d_units;
+    P.tabs = rec->d_tabs;
+    P.qtab = rec->d_qtab; P.order = rec->d_order; P.status = rec->d_status; P.N = rec->N;
+    P.hs = rec->hs; P.vs = rec->vs; P.nc = rec->nc;
+    P.chroma = rec->d_chroma;
+    return P;
+}
+
+// Where the coefficients of scans 0 .. k-1 lie.
+static void coef_lists(const pcr_record* rec, int k, CoefLists* cl) {
+    memset(cl, 0, sizeof *cl);
+    uint16_t mask[3][8] = {};
+    for (int s = 0; s < k; ++s) {
+        const ScanScript& sc = rec->script[s];
+        const ScanAux& ax = rec->saux[s];
+        if (sc.Ss == 0 && sc.Se != 63) continue;                   // DC scans: the DC plane
+        for (int i = 0; i < sc.ncomp; ++i) {
+            const int c = sc.comp[i];
+            for (int p = std::max(1, sc.Ss); p <= std::min(7, sc.Se); ++p) mask[c][p] = 0xFFFFu;
+            if (sc.Ah) {
+                cl->p1[c][cl->n_refine[c]] = 1 << sc.Al;
+                cl->refine[c][cl->n_refine[c]++] = ax.base;
+            } else if (sc.Se >= 8) {
+                cl->first[c][cl->n_first[c]++] = (sc.Ss == 0 && c > 0) ? ax.base_c[c - 1] : ax.base;
+            }
+        }
+    }
+    for (int c = 0; c < 3; ++c) memcpy(&cl->head_mask[c], mask[c], 16);
 }
 
 // Decode scans k0 .. k-1 on top of the state scans 0 .. k0-1 left behind (k0 = 0: from scratch),
@@ -1001,52 +1083,41 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
     }
     mark("h2d", 0);
     if (k0 == 0 && cudaMemsetAsync(rec->d_status, 0, (size_t)rec->N * 4, st) != cudaSuccess) return PCR_E_CUDA;
-    Params P;
-    P.rec = rec->d_rec; P.ubuf = rec->d_ubuf; P.planes = rec->d_planes; P.head = rec->d_head; P.script = rec->d_script; P.scans = rec->d_scans;
-    P.saux = rec->d_saux; P.aux = rec->d_aux;
-    P.imgs = rec->d_imgs; P.seg_start = rec->d_seg; P.items = rec->d_items; P.units = rec->d_units;
-    P.tabs = rec->d_tabs;
-    P.qtab = rec->d_qtab; P.order = rec->d_order; P.status = rec->d_status; P.N = rec->N;
-    P.hs = rec->hs; P.vs = rec->vs; P.nc = rec->nc;
+    Params P = record_params(rec);
     P.roi = targs ? targs->crops : nullptr;          // (only read by the crop-restricted kernels)
-    P.chroma = rec->d_chroma;
-    FinalizeList fl;
+    RefineList fl;                                    // the AC refinements this call decodes
     memset(&fl, 0, sizeof fl);
-    bool any_refine = false;
     for (int s = k0; s < k; ++s) {
         const ScanScript& sc = rec->script[s];
         if (sc.Ss == 0 || sc.Ah == 0) continue;
         const int c = sc.comp[0];
-        if (fl.n[c] < 4) {
-            fl.scan[c][fl.n[c]] = s;
-            fl.p1[c][fl.n[c]] = 1 << sc.Al;
-            fl.base[c][fl.n[c]] = rec->saux[s].base;
-            ++fl.n[c];
-            any_refine = true;
-        }
+        if (fl.n[c] < 4) fl.scan[c][fl.n[c]++] = s;
     }
+    CoefLists cl;                                     // everything the pixel stage shows, earlier calls' scans included
+    coef_lists(rec, k, &cl);
     int first_refine_wave = -1;                 // wave of the first AC refinement this call decodes
     for (int s = k0; s < k; ++s)
         if (rec->script[s].Ss > 0 && rec->script[s].Ah > 0 && (first_refine_wave < 0 || rec->wave_of_scan[s] < first_refine_wave))
             first_refine_wave = rec->wave_of_scan[s];
     const bool chains = first_refine_wave >= 0 && rec->n_groups > 0;
     const int chain_depth = kChainPairs / 4;    // chains per scheduler of the chain launch
-    bool dc_only = true, head_only = true;      // no AC scan at all / no scan beyond zigzag position 7
+    PixelPlan plan;
+    plan.samp = sampling_code(rec->hs, rec->vs, rec->nc);
+    const bool s420 = plan.samp == kSamp420;
+    plan.dc_only = plan.head_only = s420;             // no AC scan at all / no scan beyond zigzag position 7, no refinement
+    plan.refine = false;
     for (int s = 0; s < k; ++s) {
-        if (rec->script[s].Ss > 0 || rec->script[s].Se > 0) dc_only = false;
-        if (rec->script[s].Se > 7) head_only = false;
+        const ScanScript& sc = rec->script[s];
+        if (sc.Ss > 0 || sc.Se > 0) plan.dc_only = false;
+        if (sc.Se > 7 || (sc.Ss > 0 && sc.Ah > 0)) plan.head_only = false;
+        if (sc.Ss > 0 && sc.Ah > 0) plan.refine = true;
     }
-    // the specialised pixel kernels (DC only, head plane only, crop-restricted) exist for 4:2:0
-    const bool s420 = rec->hs == 2 && rec->vs == 2 && rec->nc == 3;
-    if (!s420) { dc_only = false; head_only = false; }
-    const bool roi = targs && s420;                 // decode only the MCU rows the crops touch
-    rec->dc_merged = false;
-    // the planes must be zero before the first AC scan writes into them
-    const bool clear_planes = !head_only && (k0 == 0 || !rec->planes_cleared);
-    const bool clear_dc = k0 == 0;
-    if (k0 == 0) rec->planes_cleared = false;
-    if (clear_planes) rec->planes_cleared = true;
-    rec->decoded_k = k;
+    plan.widths_mult16 = rec->widths_mult16;
+    plan.triangle = !targs && rec->upsampling == PCR_UPSAMPLE_TRIANGLE;
+    const bool roi = targs && s420;                   // decode only the MCU rows the crops touch (built for 4:2:0)
+    plan.roi = roi;
+    rec->planes_current = false;
+    rec->decoded_k = rec->lists_k = k;
     const int G = rec->G;
     std::vector<char> copied(rec->n_waves, 0);      // wave w has to wait for its copy event
     // the stages of one slice; stage numbers: 0 clear, 1 index, 2+w entropy wave w, 2+W unused, 3+W pixels
@@ -1075,13 +1146,7 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
     auto run_stage = [&](int stage, int g, cudaStream_t q) -> bool {
         const uint32_t i0 = rec->slice_img[g], i1 = rec->slice_img[g + 1];
         const uint32_t u0 = rec->slice_unit[g], nu = rec->slice_unit[g + 1] - u0;
-        if (stage == 0) {
-            if (pipelined) return true;           // zeroed once for all slices on the clear stream
-            if (g != 0) return true;              // the first slice zeroes for all (a slice's blocks are not contiguous)
-            if (clear_dc && cudaMemsetAsync(rec->d_head, 0, rec->total_blocks * 16, q) != cudaSuccess) return false;
-            if (!clear_planes) return true;       // no AC scan yet, or already zeroed by the decode this one continues
-            return cudaMemsetAsync(rec->d_planes, 0, rec->total_blocks * 128, q) == cudaSuccess;
-        }
+        if (stage == 0) return true;             // (nothing to clear: every decode writes the same values to the same places)
         if (stage == 1) {
             if (pipelined || g != 0) return true;   // done wave by wave, as the bytes arrive; one launch covers every slice
             ScanList sl;
@@ -1093,9 +1158,7 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
         if (stage < 2 + W) {
             const int w = stage - 2;
             if (pipelined) {
-                if (w == 0) {
-                    if (cudaStreamWaitEvent(q, rec->ev_clear, 0) != cudaSuccess) return false;
-                } else if (indexed[w]) {
+                if (w > 0 && indexed[w]) {
                     // the later waves were indexed on the side stream, beside the first wave
                     if (cudaStreamWaitEvent(q, rec->ev_index[w], 0) != cudaSuccess) return false;
                 }
@@ -1180,48 +1243,7 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
             return true;
         }
         if (nu) {
-            const unsigned grid = nu;
-            uint8_t* o8 = static_cast<uint8_t*>(out);
-            if (!s420) {
-                // other samplings: one general kernel per sampling (positions 0..7 from the head plane, the
-                // rest from the lines, which are always cleared for these records)
-                const int code = rec->nc == 1 ? kSampGrey : (rec->hs == 2 ? kSamp422 : (rec->vs == 2 ? kSamp440 : kSamp444));
-                if (code == kSamp422) launch_pixels_sampled<kSamp422>(any_refine, grid, q, Q, fl, o8);
-                else if (code == kSamp440) launch_pixels_sampled<kSamp440>(any_refine, grid, q, Q, fl, o8);
-                else if (code == kSamp444) launch_pixels_sampled<kSamp444>(any_refine, grid, q, Q, fl, o8);
-                else launch_pixels_sampled<kSampGrey>(any_refine, grid, q, Q, fl, o8);
-            } else if (!targs && rec->upsampling == PCR_UPSAMPLE_TRIANGLE) {
-                // chroma pass (samples of every chroma block into the sample planes), then the pixel pass
-                if (head_only && any_refine) {
-                    pixel_kernel<true, 3, false, 1><<<grid, kPixThreads, 0, q>>>(Q, fl, o8);
-                    pixel_kernel<true, 3, false, 2><<<grid, kPixThreads, 0, q>>>(Q, fl, o8);
-                } else if (head_only) {
-                    pixel_kernel<false, 3, false, 1><<<grid, kPixThreads, 0, q>>>(Q, fl, o8);
-                    pixel_kernel<false, 3, false, 2><<<grid, kPixThreads, 0, q>>>(Q, fl, o8);
-                } else if (any_refine) {
-                    pixel_kernel<true, 1, false, 1><<<grid, kPixThreads, 0, q>>>(Q, fl, o8);
-                    pixel_kernel<true, 1, false, 2><<<grid, kPixThreads, 0, q>>>(Q, fl, o8);
-                } else {
-                    pixel_kernel<false, 1, false, 1><<<grid, kPixThreads, 0, q>>>(Q, fl, o8);
-                    pixel_kernel<false, 1, false, 2><<<grid, kPixThreads, 0, q>>>(Q, fl, o8);
-                }
-                ++g_launches;
-            } else if (!targs) {
-                if (dc_only && rec->widths_mult16) dc_pixel_kernel<false><<<grid, 128, 0, q>>>(Q, o8);
-                else if (dc_only) dc_pixel_kernel<false, false><<<grid, 128, 0, q>>>(Q, o8);
-                else if (head_only && any_refine) pixel_kernel<true, 3><<<grid, kPixThreads, 0, q>>>(Q, fl, o8);
-                else if (head_only) pixel_kernel<false, 3><<<grid, kPixThreads, 0, q>>>(Q, fl, o8);
-                else if (any_refine) pixel_kernel<true, 1><<<grid, kPixThreads, 0, q>>>(Q, fl, o8);
-                else pixel_kernel<false, 1><<<grid, kPixThreads, 0, q>>>(Q, fl, o8);
-            } else {
-                if (dc_only && rec->widths_mult16) dc_pixel_kernel<true><<<grid, 128, 0, q>>>(Q, o8);
-                else if (dc_only) dc_pixel_kernel<true, false><<<grid, 128, 0, q>>>(Q, o8);
-                else if (head_only && any_refine) pixel_kernel<true, 3, true><<<grid, kPixThreads, 0, q>>>(Q, fl, o8);
-                else if (head_only) pixel_kernel<false, 3, true><<<grid, kPixThreads, 0, q>>>(Q, fl, o8);
-                else if (any_refine) pixel_kernel<true, 1, true><<<grid, kPixThreads, 0, q>>>(Q, fl, o8);
-                else pixel_kernel<false, 1, true><<<grid, kPixThreads, 0, q>>>(Q, fl, o8);
-            }
-            ++g_launches;
+            launch_pixels(plan, nu, q, Q, cl, static_cast<uint8_t*>(out));
             // the grid's second dimension (one image each) holds at most 65535 entries
             for (uint32_t p0 = i0; targs && p0 < i1; p0 += 65535u) {
                 const dim3 tg((unsigned)((targs->size + kTensorRows - 1) / kTensorRows), std::min(i1 - p0, 65535u));
@@ -1274,9 +1296,6 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
         // missing record bytes arrive on a copy stream, the scan groups of each wave behind an event
         if (cudaEventRecord(rec->ev_fork, st) != cudaSuccess) return PCR_E_CUDA;
         if (cudaStreamWaitEvent(rec->clear_stream, rec->ev_fork, 0) != cudaSuccess) return PCR_E_CUDA;
-        if (clear_dc && cudaMemsetAsync(rec->d_head, 0, rec->total_blocks * 16, rec->clear_stream) != cudaSuccess) return PCR_E_CUDA;
-        if (clear_planes && cudaMemsetAsync(rec->d_planes, 0, rec->total_blocks * 128, rec->clear_stream) != cudaSuccess) return PCR_E_CUDA;
-        if (cudaEventRecord(rec->ev_clear, rec->clear_stream) != cudaSuccess) return PCR_E_CUDA;
         if (rec->resident < need) {
             if (cudaStreamWaitEvent(rec->copy_stream, rec->ev_fork, 0) != cudaSuccess) return PCR_E_CUDA;
             bool any = false;
@@ -1491,20 +1510,15 @@ int pcr_status(pcr_record* rec, int* first_bad_image, int* code) {
 
 int pcr_coeffs(pcr_record* rec, const int16_t** dev_planes, size_t* bytes) {
     if (!rec || !dev_planes || !bytes) return PCR_E_ARG;
-    // the decode keeps the DC coefficients in a dense plane of their own (and leaves the planes
-    // alone when no AC scan was decoded): complete the canonical layout now
-    if (!rec->planes_cleared) {
-        if (cudaMemset(rec->d_planes, 0, rec->total_blocks * 128) != cudaSuccess) return PCR_E_CUDA;
-        rec->planes_cleared = true;
-    }
-    if (!rec->dc_merged && rec->total_blocks) {
-        Params P;
-        memset(&P, 0, sizeof P);
-        P.planes = rec->d_planes; P.head = rec->d_head;
-        merge_head_kernel<<<(unsigned)((rec->total_blocks + 255) / 256), 256>>>(P, rec->total_blocks);
-        ++g_launches;
+    // the decode keeps coefficients as lists: expand them into the canonical layout now
+    if (!rec->d_planes)
+        if (int rc = take(rec, &rec->d_planes, (size_t)(std::max<uint64_t>(rec->total_blocks, 1) * 128))) return rc;
+    if (!rec->planes_current && rec->total_blocks) {
+        CoefLists cl;
+        coef_lists(rec, rec->lists_k, &cl);
+        launch_planes(sampling_code(rec->hs, rec->vs, rec->nc), rec->n_units, record_params(rec), cl);
         if (cudaDeviceSynchronize() != cudaSuccess) return PCR_E_CUDA;
-        rec->dc_merged = true;
+        rec->planes_current = true;
     }
     *dev_planes = rec->d_planes;
     *bytes = (size_t)rec->total_blocks * 128;
@@ -1601,7 +1615,8 @@ const char* pcr_strerror(int code) {
 namespace {
 
 constexpr uint32_t kNoAllocMaxDim = 4096;                                         // pixels per side
-constexpr uint32_t kNoAllocMaxUnits = (kNoAllocMaxDim / 16) * (kNoAllocMaxDim / 16 / kPixMcus);
+constexpr uint32_t kNoAllocMcus = kUnitMcus[kSamp420], kNoAllocRows = kUnitRows[kSamp420];
+constexpr uint32_t kNoAllocMaxUnits = (kNoAllocMaxDim / 16 / kNoAllocRows) * (kNoAllocMaxDim / 16 / kNoAllocMcus);
 struct NoAllocScratch {
     ImgDesc img;
     uint16_t qtab[192];
@@ -1614,16 +1629,16 @@ struct QuantArg { uint16_t q[192]; };
 __global__ void noalloc_fill_kernel(uint32_t W, uint32_t H, QuantArg qa) {
     NoAllocScratch* s = reinterpret_cast<NoAllocScratch*>(g_noalloc_scratch);   // device code may name the array
     const uint32_t mx = (W + 15) / 16, my = (H + 15) / 16;
-    const uint32_t per_row = (mx + kPixMcus - 1) / kPixMcus;
+    const uint32_t per_row = (mx + kNoAllocMcus - 1) / kNoAllocMcus;
     const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
     if (tid == 0) {
         s->img.W = W; s->img.H = H; s->img.mx = mx; s->img.my = my;
         s->img.blk_base = 0; s->img.out_off = 0;
     }
     if (tid < 192) s->qtab[tid] = qa.q[tid];
-    for (uint32_t u = tid; u < per_row * my; u += nth) {
+    for (uint32_t u = tid; u < per_row * ((my + kNoAllocRows - 1) / kNoAllocRows); u += nth) {
         Unit un;
-        un.img = 0; un.mrow = (uint16_t)(u / per_row); un.mcol0 = (uint16_t)((u % per_row) * kPixMcus);
+        un.img = 0; un.mrow = (uint16_t)(u / per_row * kNoAllocRows); un.mcol0 = (uint16_t)((u % per_row) * kNoAllocMcus);
         s->units[u] = un;
     }
 }
@@ -1654,7 +1669,7 @@ int pcr_pixels_noalloc(const int16_t* dev_coeffs, uint32_t width, uint32_t heigh
     NoAllocScratch* s = static_cast<NoAllocScratch*>(g_noalloc_ptr[dev]);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const uint32_t mx = (width + 15) / 16, my = (height + 15) / 16;
-    const uint32_t n_units = ((mx + kPixMcus - 1) / kPixMcus) * my;
+    const uint32_t n_units = ((mx + kNoAllocMcus - 1) / kNoAllocMcus) * ((my + kNoAllocRows - 1) / kNoAllocRows);
     QuantArg qa;
     memcpy(qa.q, host_qtab, sizeof qa.q);
     noalloc_fill_kernel<<<(n_units + 255) / 256, 256, 0, st>>>(width, height, qa);
@@ -1663,9 +1678,9 @@ int pcr_pixels_noalloc(const int16_t* dev_coeffs, uint32_t width, uint32_t heigh
     memset(&P, 0, sizeof P);
     P.planes = const_cast<int16_t*>(dev_coeffs);     // read only by the pixel kernel
     P.imgs = &s->img; P.units = s->units; P.qtab = s->qtab; P.N = 1;
-    FinalizeList none;
+    CoefLists none;
     memset(&none, 0, sizeof none);
-    pixel_kernel<false, 0><<<n_units, kPixThreads, 0, st>>>(P, none, dev_rgb);
+    pixel_kernel<false, 0><<<n_units, unit_threads<kSamp420>(), 0, st>>>(P, none, dev_rgb);
     ++g_launches;
     if (cudaGetLastError() != cudaSuccess) return PCR_E_CUDA;
     return PCR_OK;

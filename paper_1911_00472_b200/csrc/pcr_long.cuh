@@ -74,8 +74,7 @@ __global__ void __launch_bounds__(256) dc_refine_kernel(Params P, int s, uint32_
             int comp;
             if (!inter) blk = g.coff[c0] + (uint64_t)mrow * g.bw[c0] + mcol;
             else blk = mcu_block(g, P, mrow, mcol, (int)j, &comp);
-            // coefficient 0 is the first int16 of the block's head entry; no other scan of the wave writes it
-            int16_t* dcv = P.head + blk * 8;
+            int16_t* dcv = P.dc + blk;                        // (no other scan of the wave writes it)
             *dcv = (int16_t)(*dcv | p1);
         }
     }
@@ -221,78 +220,75 @@ __device__ __forceinline__ void dc_search_span(const HuffTab* tabs2, const uint8
 
 // What one lane needs to write the coefficients of an AC first pass.
 struct AcWrite {
-    int16_t* plane;        // the component's lines
     int16_t* headp;        // the component's head entries
-    unsigned long long* maskp;   // the scan's non-zero masks, by block number inside the component
+    int16_t* vals;         // the value array from position 0 of the stream words on
+    uint64_t* auxp;        // the scan's side data of the image's component
+    bool lists;            // the band reaches beyond position 7: side data of two words, values in the array
     uint32_t mcu_w, bw;    // blocks per row of the scan's (unpadded) grid / of the padded grid
-    uint32_t m, m1;        // next block of the scan, one past its last
-    int p1;
+    uint32_t m, m1;        // the block the entry position lies in, one past the scan's last
+    int Al;
 };
 
-// Decodes the symbols of an AC first pass that START in [pos, pos_end), from zigzag position k of the
-// current block.  Every step consumes at least one bit, so the loop ends.  Without kWrite (search
-// for the true entry state) an undefined code is skipped by one bit and a coefficient beyond the
-// band ends the block: the lane is then reading from a wrong entry point and only has to arrive
-// somewhere.  With kWrite the entry state is the true one, such events mean a corrupt stream.
-template <bool kWrite>
-__device__ __forceinline__ void ac_first_span(const HuffTab& tab, const uint32_t* base, uint32_t pos, int k, uint32_t pos_end,
-                                              int Ss, int Se, uint32_t& pos_out, int& k_out, uint32_t& nblk, AcWrite& W, bool& bad) {
+// Decodes and writes the blocks of an AC first pass that BEGIN in [pos, pos_end), the last one to its end; k =
+// the zigzag position at pos (a block that began before pos is passed over: the thread before writes it).  So
+// every block has one writer and its values one run in the value array.  The entry state is the true one:
+// an undefined code or a coefficient beyond the band means a corrupt stream.  Every step consumes at least
+// one bit, so the loop ends.
+__device__ __forceinline__ void ac_write_span(const HuffTab& tab, const uint32_t* base, uint32_t pos, int k, uint32_t pos_end,
+                                              uint32_t endbit, int Ss, int Se, AcWrite& W, bool& bad) {
     WordReader br;
     br.init(base, pos);
-    uint32_t nb = 0;
-    unsigned long long M = 0;
-    uint32_t bcol = 0, bi = 0;
-    if (kWrite) { bcol = W.m % W.mcu_w; bi = (W.m / W.mcu_w) * W.bw + bcol; }
-    bool stop = kWrite && W.m >= W.m1;
-    while (!stop && br.pos() < pos_end) {
+    bool own = k == Ss;                                        // this block is this thread's to write
+    uint32_t M0 = 0, M1 = 0;
+    int16_t* vp = W.vals + ((pos + 1u) >> 1);
+    int16_t* vb = vp;
+    uint32_t bcol = W.m % W.mcu_w, bi = (W.m / W.mcu_w) * W.bw + bcol;
+    while (W.m < W.m1) {
+        const uint32_t at = br.pos();
+        if (at >= endbit || (k == Ss && at >= pos_end)) break;
+        if (!own && at >= pos_end) break;                      // the whole span lies inside a block of an earlier thread
         br.refill();
         const uint32_t win = br.top32();
         uint32_t e = tab.lut[win >> (32 - kLutBits)];
         if (e == 0) e = huff_lookup(tab, win);
-        if (e == 0) {
-            if (kWrite) { bad = true; break; }
-            br.skip(1);
-            continue;
-        }
+        if (e == 0) { bad = true; break; }
         const int len = (int)(e >> 8), r = (int)(e >> 4) & 15, sz = (int)(e & 15u);
         const bool is_coef = sz != 0, is_eob = sz == 0 && r < 15;
         const int kk = k + r;
-        const bool over = is_coef && kk > Se;
-        if (kWrite && over) { bad = true; break; }
+        if (is_coef && kk > Se) { bad = true; break; }
         const int extra = is_coef ? sz : (is_eob ? r : 0);
         const uint32_t xb = top_bits(win << len, extra);
         br.skip(len + extra);
-        if (kWrite && is_coef) {
-            const int16_t val = (int16_t)(extend_bits(xb, sz) * W.p1);
+        if (is_coef && own) {
+            const int16_t val = (int16_t)(extend_bits(xb, sz) << W.Al);
             if (kk < 8) W.headp[(uint64_t)bi * 8 + kk] = val;
-            else W.plane[(uint64_t)bi * 64 + kk] = val;
-            M |= 1ull << kk;
+            else *vp++ = val;
+            if (kk < 32) M0 |= 1u << kk; else M1 |= 1u << (kk - 32);
         }
         k = is_coef ? kk + 1 : (is_eob ? k : k + 16);
-        if (is_eob || over || k > Se) {                        // the block ends, an end-of-band run skips more
-            const uint32_t adv = 1u + (is_eob ? (1u << r) + xb - 1u : 0u);
-            nb += adv;
-            k = Ss;
-            if (kWrite) {
-                if (M) atomicOr(W.maskp + bi, M);              // a block may be shared with the neighbouring lane
-                M = 0;
-                W.m += adv;
-                if (W.m >= W.m1) stop = true;
-                else if (adv == 1u) { if (++bcol == W.mcu_w) { bcol = 0; bi += W.bw - W.mcu_w + 1u; } else ++bi; }
-                else { bcol = W.m % W.mcu_w; bi = (W.m / W.mcu_w) * W.bw + bcol; }
+        if (is_eob || k > Se) {                                // the block ends, an end-of-band run skips more
+            if (M0 | M1) {
+                if (W.lists) *reinterpret_cast<uint4*>(W.auxp + (uint64_t)bi * 2) = value_record(M0, M1, vb);
+                else *reinterpret_cast<uint2*>(W.auxp + bi) = make_uint2(M0, M1);
             }
+            const uint32_t adv = is_eob ? (1u << r) + xb : 1u;
+            k = Ss;
+            M0 = 0; M1 = 0;
+            if (!own) vp = W.vals + ((br.pos() + 1u) >> 1);     // this thread's values begin where its first block does
+            vb = vp;
+            own = true;
+            if (adv >= W.m1 - W.m) break;
+            W.m += adv;
+            bcol += adv; bi += adv;
+            if (bcol >= W.mcu_w) { bcol = W.m % W.mcu_w; bi = (W.m / W.mcu_w) * W.bw + bcol; }
         }
     }
-    if (kWrite && M) atomicOr(W.maskp + bi, M);                // the part of a block that ends in the next lane's span
-    pos_out = br.pos();
-    k_out = k;
-    nblk = nb;
 }
 
 // The same for a DC first pass: one symbol (size category, then that many difference bits) per block;
 // j = the block's place in its MCU (Y00 Y01 Y10 Y11 Cb Cr, or always 0 in a one-component scan).
 struct DcWrite {
-    int16_t* head;
+    int16_t* dc;
     uint64_t coff[3];
     uint32_t bw[3];
     uint32_t mcu_w;
@@ -302,19 +298,14 @@ struct DcWrite {
     int Al;
 };
 
-template <bool kWrite>
-__device__ __forceinline__ void dc_first_span(const HuffTab* tabs2, uint32_t slots, bool inter, int c0, const uint32_t* base,
-                                              uint32_t pos, int j, uint32_t pos_end, uint32_t& pos_out, int& j_out, uint32_t& nblk,
-                                              int& sum0, int& sum1, int& sum2, DcWrite& W, bool& bad) {
+__device__ __forceinline__ void dc_write_span(const HuffTab* tabs2, uint32_t slots, bool inter, int c0, const uint32_t* base,
+                                              uint32_t pos, int j, uint32_t pos_end, DcWrite& W, bool& bad) {
     WordReader br;
     br.init(base, pos);
     const int ny = (int)(W.hs * W.vs), bpm = inter ? ny + 2 : 1;
-    uint32_t nb = 0;
-    int s0 = 0, s1 = 0, s2 = 0;
-    uint32_t mrow = 0, mcol = 0;
-    if (kWrite) { const uint32_t m = W.n / (uint32_t)bpm; mrow = m / W.mcu_w; mcol = m - mrow * W.mcu_w; }
-    bool stop = kWrite && W.n >= W.n1;
-    while (!stop && br.pos() < pos_end) {
+    const uint32_t m = W.n / (uint32_t)bpm;
+    uint32_t mrow = m / W.mcu_w, mcol = m - mrow * W.mcu_w;
+    while (W.n < W.n1 && br.pos() < pos_end) {
         br.refill();
         const uint32_t win = br.top32();
         const int ci = inter ? (j < ny ? 0 : j - ny + 1) : 0;
@@ -322,33 +313,21 @@ __device__ __forceinline__ void dc_first_span(const HuffTab* tabs2, uint32_t slo
         const HuffTab& tab = tabs2[(slots >> (2 * ci)) & 1u];
         const uint32_t e = huff_lookup(tab, win);
         const int len = (int)(e >> 8), sz = (int)(e & 255u);
-        if (e == 0 || sz > 15) {
-            if (kWrite) { bad = true; break; }
-            br.skip(1);
-            continue;
-        }
+        if (e == 0 || sz > 15) { bad = true; break; }
         const int d = extend_bits(top_bits(win << len, sz), sz);
         br.skip(len + sz);
-        if (c == 0) s0 += d; else if (c == 1) s1 += d; else s2 += d;
-        if (kWrite) {
-            const int pv = (c == 0 ? W.pred[0] : (c == 1 ? W.pred[1] : W.pred[2])) + d;
-            if (c == 0) W.pred[0] = pv; else if (c == 1) W.pred[1] = pv; else W.pred[2] = pv;
-            uint64_t blk;
-            if (inter && c == 0) blk = W.coff[0] + (uint64_t)(W.vs * mrow + ((uint32_t)j >> (W.hs - 1u))) * W.bw[0] + W.hs * mcol + ((uint32_t)j & (W.hs - 1u));
-            else blk = W.coff[c] + (uint64_t)mrow * W.bw[c] + mcol;
-            W.head[blk * 8] = (int16_t)(pv << W.Al);
-            if (++W.n >= W.n1) stop = true;
-        }
-        ++nb;
+        const int pv = (c == 0 ? W.pred[0] : (c == 1 ? W.pred[1] : W.pred[2])) + d;
+        if (c == 0) W.pred[0] = pv; else if (c == 1) W.pred[1] = pv; else W.pred[2] = pv;
+        uint64_t blk;
+        if (inter && c == 0) blk = W.coff[0] + (uint64_t)(W.vs * mrow + ((uint32_t)j >> (W.hs - 1u))) * W.bw[0] + W.hs * mcol + ((uint32_t)j & (W.hs - 1u));
+        else blk = W.coff[c] + (uint64_t)mrow * W.bw[c] + mcol;
+        W.dc[blk] = (int16_t)(pv << W.Al);
+        ++W.n;
         if (++j == bpm) {
             j = 0;
-            if (kWrite) { if (++mcol == W.mcu_w) { mcol = 0; ++mrow; } }
+            if (++mcol == W.mcu_w) { mcol = 0; ++mrow; }
         }
     }
-    pos_out = br.pos();
-    j_out = j;
-    nblk = nb;
-    sum0 = s0; sum1 = s1; sum2 = s2;
 }
 
 // Exclusive prefix sum over the CTA's threads in thread order (warp scans, then the warps' totals
@@ -433,7 +412,7 @@ __global__ void __launch_bounds__(32 * kLongWarps) first_pass_long_kernel(Params
     };
     if (dc) {
         DcWrite W;
-        W.head = P.head; W.mcu_w = mcu_w; W.Al = sc.Al; W.hs = (uint32_t)P.hs; W.vs = (uint32_t)P.vs;
+        W.dc = P.dc; W.mcu_w = mcu_w; W.Al = sc.Al; W.hs = (uint32_t)P.hs; W.vs = (uint32_t)P.vs;
         const uint32_t bpm = inter ? (uint32_t)(P.hs * P.vs + 2) : 1u;
 #pragma unroll
         for (int c = 0; c < 3; ++c) { W.coff[c] = g.coff[c]; W.bw[c] = g.bw[c]; W.pred[c] = 0; }
@@ -467,15 +446,15 @@ __global__ void __launch_bounds__(32 * kLongWarps) first_pass_long_kernel(Params
         // the stream is damaged; taking it from the block number keeps every store inside the image)
         if (nb && (uint32_t)j != W.n % bpm) bad = true;
         j = (int)(W.n % bpm);
-        dc_first_span<true>(tabs, sd.slots, inter, c0, base, pos, j, my_end, pos_x, j_x, nb, a0, a1, a2, W, bad);
+        dc_write_span(tabs, sd.slots, inter, c0, base, pos, j, my_end, W, bad);
         if (all < total * bpm) bad = true;                     // the stream ends before the last block
     } else {
         const int c = c0, Ss = sc.Ss, Se = sc.Se;
         const ScanAux ax = P.saux[s];
         AcWrite W;
-        W.plane = P.planes + g.coff[c] * 64; W.headp = P.head + g.coff[c] * 8;
-        W.maskp = reinterpret_cast<unsigned long long*>(P.aux + ax.base + g.loff[c]);
-        W.mcu_w = mcu_w; W.bw = g.bw[c]; W.m = 0; W.m1 = total; W.p1 = 1 << sc.Al;
+        W.headp = P.head + g.coff[c] * 8; W.vals = P.vals + 16ull * (bstart >> 2);
+        W.auxp = P.aux + ax.base + g.loff[c] * ax.stride; W.lists = ax.stride == 2u;
+        W.mcu_w = mcu_w; W.bw = g.bw[c]; W.m = 0; W.m1 = total; W.Al = sc.Al;
         const HuffTab& tab = tabs[0];
         uint32_t pos = my_begin, pos_x = my_begin, nb = 0;
         int k = Ss, k_x = Ss;
@@ -490,7 +469,7 @@ __global__ void __launch_bounds__(32 * kLongWarps) first_pass_long_kernel(Params
         }
         uint32_t all;
         W.m = min(cta_exclusive_sum(nb, s_u, wid, lane, kLongWarps, all), total);
-        ac_first_span<true>(tab, base, pos, k, my_end, Ss, Se, pos_x, k_x, nb, W, bad);
+        ac_write_span(tab, base, pos, k, my_end, endbit, Ss, Se, W, bad);
         if (all < total) bad = true;                                         // the stream ends before the last block
     }
     if (__syncthreads_or(bad) && tid == 0) atomicMin(&P.status[img], kErrCorrupt);
@@ -503,8 +482,10 @@ __global__ void __launch_bounds__(32 * kLongWarps) first_pass_long_kernel(Params
 // differences it reads per component.
 // ---------------------------------------------------------------------------------------
 struct SeqWrite {
+    int16_t* dc;
     int16_t* head;
-    int16_t* planes;
+    int16_t* vals;         // the value array from position 0 of the stream words on
+    uint64_t* auxp[3];     // the scan's side data of the image's components
     uint64_t coff[3];
     uint32_t bw[3];
     uint32_t mcu_w;
@@ -513,66 +494,44 @@ struct SeqWrite {
     int pred[3];
 };
 
-template <bool kWrite>
-__device__ __forceinline__ void seq_span(const HuffTab* tabs4, uint32_t slots, uint32_t slots_ac, int nc, const uint32_t* base,
-                                         uint32_t pos, int j, int k, uint32_t pos_end, uint32_t& pos_out, int& j_out, int& k_out,
-                                         uint32_t& nblk, int& sum0, int& sum1, int& sum2, SeqWrite& W, bool& bad) {
+// a symbol of a sequential scan: false if there is none such (k, j: where the reader stands)
+struct SeqSymbol { int len, r, sz; bool is_coef, is_zrl, is_eob; };
+__device__ __forceinline__ bool seq_symbol(const HuffTab* tabs4, uint32_t slots, uint32_t slots_ac, int c, int k, uint32_t win, SeqSymbol& y) {
+    const bool is_dc = k == 0;
+    const int ti = is_dc ? (int)((slots >> (2 * c)) & 1u) : 2 + (int)((slots_ac >> (2 * c)) & 1u);
+    const uint32_t e = huff_lookup(tabs4[ti], win);
+    y.len = (int)(e >> 8); y.r = is_dc ? 0 : (int)(e >> 4) & 15; y.sz = is_dc ? (int)(e & 255u) : (int)(e & 15u);
+    y.is_coef = y.sz != 0; y.is_zrl = !is_dc && y.sz == 0 && y.r == 15; y.is_eob = !is_dc && y.sz == 0 && y.r == 0;
+    return !(e == 0 || y.sz > 15 || (!is_dc && !y.is_coef && !y.is_zrl && !y.is_eob) || (y.is_coef && k + y.r > 63));
+}
+
+// Search pass: from state (pos, j, k) to the end of the span (see the header comment); counts the blocks it
+// finishes and sums the DC differences it reads.
+__device__ __forceinline__ void seq_search_span(const HuffTab* tabs4, uint32_t slots, uint32_t slots_ac, int nc, uint32_t ny_, const uint32_t* base,
+                                                uint32_t pos, int j, int k, uint32_t pos_end, uint32_t& pos_out, int& j_out, int& k_out,
+                                                uint32_t& nblk, int& sum0, int& sum1, int& sum2) {
     WordReader br;
     br.init(base, pos);
-    const int ny = (int)(W.hs * W.vs), bpm = nc == 3 ? ny + 2 : 1;
+    const int ny = (int)ny_, bpm = nc == 3 ? ny + 2 : 1;
     uint32_t nb = 0;
     int s0 = 0, s1 = 0, s2 = 0;
-    uint32_t mrow = 0, mcol = 0;
-    if (kWrite) { const uint32_t m = W.n / (uint32_t)bpm; mrow = m / W.mcu_w; mcol = m - mrow * W.mcu_w; }
-    bool stop = kWrite && W.n >= W.n1;
-    while (!stop && br.pos() < pos_end) {
+    while (br.pos() < pos_end) {
         br.refill();
         const uint32_t win = br.top32();
         const int c = nc == 3 ? (j < ny ? 0 : j - ny + 1) : 0;
-        const bool is_dc = k == 0;
-        const int ti = is_dc ? (int)((slots >> (2 * c)) & 1u) : 2 + (int)((slots_ac >> (2 * c)) & 1u);
-        const uint32_t e = huff_lookup(tabs4[ti], win);
-        const int len = (int)(e >> 8), r = is_dc ? 0 : (int)(e >> 4) & 15, sz = is_dc ? (int)(e & 255u) : (int)(e & 15u);
-        const bool is_coef = sz != 0, is_zrl = !is_dc && sz == 0 && r == 15, is_eob = !is_dc && sz == 0 && r == 0;
-        const int kk = k + r;
-        if (e == 0 || sz > 15 || (!is_dc && !is_coef && !is_zrl && !is_eob) || (is_coef && kk > 63)) {
-            if (kWrite) { bad = true; break; }
-            br.skip(1);
-            continue;
-        }
-        const int extra = is_coef ? sz : 0;
-        const int v = extend_bits(top_bits(win << len, extra), extra);
-        br.skip(len + extra);
-        uint64_t blk = 0;
-        if (kWrite) {
-            if (nc == 3 && c == 0) blk = W.coff[0] + (uint64_t)(W.vs * mrow + ((uint32_t)j >> (W.hs - 1u))) * W.bw[0] + W.hs * mcol + ((uint32_t)j & (W.hs - 1u));
-            else blk = W.coff[c] + (uint64_t)mrow * W.bw[c] + mcol;
-        }
-        if (is_dc) {
+        SeqSymbol y;
+        if (!seq_symbol(tabs4, slots, slots_ac, c, k, win, y)) { br.skip(1); continue; }
+        br.skip(y.len + y.sz);
+        if (k == 0) {
+            const int v = extend_bits(top_bits(win << y.len, y.sz), y.sz);
             if (c == 0) s0 += v; else if (c == 1) s1 += v; else s2 += v;
-            if (kWrite) {
-                const int pv = (c == 0 ? W.pred[0] : (c == 1 ? W.pred[1] : W.pred[2])) + v;
-                if (c == 0) W.pred[0] = pv; else if (c == 1) W.pred[1] = pv; else W.pred[2] = pv;
-                W.head[blk * 8] = (int16_t)pv;
-            }
             k = 1;
-        } else if (is_coef) {
-            if (kWrite) {
-                if (kk < 8) W.head[blk * 8 + kk] = (int16_t)v;
-                else W.planes[blk * 64 + kk] = (int16_t)v;
-            }
-            k = kk + 1;
-        } else if (is_zrl) {
-            k += 16;
-        }
-        if (is_eob || k > 63) {                               // block finished
+        } else if (y.is_coef) k += y.r + 1;
+        else if (y.is_zrl) k += 16;
+        if (y.is_eob || k > 63) {                             // block finished
             k = 0;
             ++nb;
-            if (kWrite && ++W.n >= W.n1) stop = true;
-            if (++j == bpm) {
-                j = 0;
-                if (kWrite) { if (++mcol == W.mcu_w) { mcol = 0; ++mrow; } }
-            }
+            if (++j == bpm) j = 0;
         }
     }
     pos_out = br.pos();
@@ -580,6 +539,63 @@ __device__ __forceinline__ void seq_span(const HuffTab* tabs4, uint32_t slots, u
     k_out = k;
     nblk = nb;
     sum0 = s0; sum1 = s1; sum2 = s2;
+}
+
+// Decodes and writes the blocks that BEGIN in [pos, pos_end), the last one to its end (see ac_write_span).
+__device__ __forceinline__ void seq_write_span(const HuffTab* tabs4, uint32_t slots, uint32_t slots_ac, int nc, const uint32_t* base,
+                                               uint32_t pos, int j, int k, uint32_t pos_end, uint32_t endbit, SeqWrite& W, bool& bad) {
+    WordReader br;
+    br.init(base, pos);
+    const int ny = (int)(W.hs * W.vs), bpm = nc == 3 ? ny + 2 : 1;
+    bool own = k == 0;
+    uint32_t M0 = 0, M1 = 0;
+    int16_t* vp = W.vals + ((pos + 1u) >> 1);
+    int16_t* vb = vp;
+    const uint32_t m = W.n / (uint32_t)bpm;
+    uint32_t mrow = m / W.mcu_w, mcol = m - mrow * W.mcu_w;
+    while (W.n < W.n1) {
+        const uint32_t at = br.pos();
+        if (at >= endbit || ((k == 0 || !own) && at >= pos_end)) break;
+        br.refill();
+        const uint32_t win = br.top32();
+        const int c = nc == 3 ? (j < ny ? 0 : j - ny + 1) : 0;
+        SeqSymbol y;
+        if (!seq_symbol(tabs4, slots, slots_ac, c, k, win, y)) { bad = true; break; }
+        const int v = extend_bits(top_bits(win << y.len, y.sz), y.sz), kk = k + y.r;
+        br.skip(y.len + y.sz);
+        const uint32_t local = (nc == 3 && c == 0) ? (W.vs * mrow + ((uint32_t)j >> (W.hs - 1u))) * W.bw[0] + W.hs * mcol + ((uint32_t)j & (W.hs - 1u))
+                                                   : mrow * W.bw[c] + mcol;
+        const uint64_t blk = W.coff[c] + local;
+        if (k == 0) {
+            const int pv = (c == 0 ? W.pred[0] : (c == 1 ? W.pred[1] : W.pred[2])) + v;
+            if (c == 0) W.pred[0] = pv; else if (c == 1) W.pred[1] = pv; else W.pred[2] = pv;
+            W.dc[blk] = (int16_t)pv;
+            k = 1;
+        } else if (y.is_coef) {
+            if (own) {
+                if (kk < 8) W.head[blk * 8 + kk] = (int16_t)v;
+                else {
+                    *vp++ = (int16_t)v;
+                    if (kk < 32) M0 |= 1u << kk; else M1 |= 1u << (kk - 32);
+                }
+            }
+            k = kk + 1;
+        } else if (y.is_zrl) {
+            k += 16;
+        }
+        if (y.is_eob || k > 63) {                             // block finished
+            if (M0 | M1) *reinterpret_cast<uint4*>(W.auxp[c] + 2ull * local) = value_record(M0, M1, vb);
+            k = 0; M0 = 0; M1 = 0;
+            if (!own) vp = W.vals + ((br.pos() + 1u) >> 1);
+            vb = vp;
+            own = true;
+            ++W.n;
+            if (++j == bpm) {
+                j = 0;
+                if (++mcol == W.mcu_w) { mcol = 0; ++mrow; }
+            }
+        }
+    }
 }
 
 #ifndef PCR_SEQ_LONG_WARPS
@@ -625,7 +641,9 @@ __global__ void __launch_bounds__(32 * kSeqLongWarps) sequential_long_kernel(Par
     const uint32_t my_begin = min(max((uint32_t)tid * S, lead), endbit), my_end = min(((uint32_t)tid + 1u) * S, endbit);
     bool bad = false;
     SeqWrite W;
-    W.head = P.head; W.planes = P.planes; W.mcu_w = mcu_w; W.hs = (uint32_t)P.hs; W.vs = (uint32_t)P.vs;
+    const ScanAux ax = P.saux[si / (uint32_t)P.N];
+    W.dc = P.dc; W.head = P.head; W.vals = P.vals + 16ull * (bstart >> 2); W.mcu_w = mcu_w; W.hs = (uint32_t)P.hs; W.vs = (uint32_t)P.vs;
+    W.auxp[0] = P.aux + ax.base + 2ull * g.loff[0]; W.auxp[1] = P.aux + ax.base_c[0] + 2ull * g.loff[1]; W.auxp[2] = P.aux + ax.base_c[1] + 2ull * g.loff[1];
 #pragma unroll
     for (int c = 0; c < 3; ++c) { W.coff[c] = g.coff[c]; W.bw[c] = g.bw[c]; W.pred[c] = 0; }
     W.n = 0; W.n1 = total * bpm;
@@ -633,7 +651,7 @@ __global__ void __launch_bounds__(32 * kSeqLongWarps) sequential_long_kernel(Par
     int j = 0, k = 0, j_x = 0, k_x = 0, a0 = 0, a1 = 0, a2 = 0;
     bool again = true;
     for (int round = 0; round <= (int)kSubs; ++round) {
-        if (again) seq_span<false>(tabs, sd.slots, sd.slots_ac, P.nc, base, pos, j, k, my_end, pos_x, j_x, k_x, nb, a0, a1, a2, W, bad);
+        if (again) seq_search_span(tabs, sd.slots, sd.slots_ac, P.nc, W.hs * W.vs, base, pos, j, k, my_end, pos_x, j_x, k_x, nb, a0, a1, a2);
         // the state the previous thread ended in (block of the MCU and zigzag position in one word)
         const int st_x = j_x * 64 + k_x;
         if (lane == 31) { s_pos[wid] = pos_x; s_state[wid] = st_x; }
@@ -656,7 +674,7 @@ __global__ void __launch_bounds__(32 * kSeqLongWarps) sequential_long_kernel(Par
     // stream is damaged; taking it from the block number keeps every store inside the image)
     if ((nb || k) && (uint32_t)j != W.n % bpm) bad = true;
     j = (int)(W.n % bpm);
-    seq_span<true>(tabs, sd.slots, sd.slots_ac, P.nc, base, pos, j, k, my_end, pos_x, j_x, k_x, nb, a0, a1, a2, W, bad);
+    seq_write_span(tabs, sd.slots, sd.slots_ac, P.nc, base, pos, j, k, my_end, endbit, W, bad);
     if (all < total * bpm) bad = true;                         // the stream ends before the last block
     if (__syncthreads_or(bad) && tid == 0) atomicMin(&P.status[img], kErrCorrupt);
 }
@@ -804,7 +822,7 @@ __device__ __forceinline__ bool meet_helper(ChainShared& sh, uint32_t k, int lan
 // The decoding side of a chain: one thread.  It takes the pair's jobs (first the statically assigned
 // one, then tickets of its scheduler's queue), and per job follows the bit stream batch by batch:
 // the lists of still-zero positions of a batch come from the helper, the symbol records go back to it.
-__device__ __forceinline__ void chain_decoder(const FinalizeList& fl, ChainShared& sh, const uint32_t* __restrict__ list, uint32_t n_groups,
+__device__ __forceinline__ void chain_decoder(const RefineList& fl, ChainShared& sh, const uint32_t* __restrict__ list, uint32_t n_groups,
                                               uint32_t* sync, uint32_t levels, uint32_t rounds, uint32_t q, uint32_t slot) {
     const uint32_t per_round = 4u * gridDim.x, statics = per_round * rounds;
     uint32_t mk = 0;                                           // meeting points so far
@@ -923,7 +941,7 @@ __device__ __forceinline__ void chain_decoder(const FinalizeList& fl, ChainShare
 // of the decoder with the masks and lists of still-zero positions (waiting, with bounded polls, for
 // an earlier refinement of the same blocks when this launch decodes that too), keeps the ring of
 // bitstream words filled, and one batch behind it turns the symbol records into side data.
-__device__ __forceinline__ void chain_helper(const Params& P, const FinalizeList& fl, ChainShared& sh, const uint32_t* __restrict__ list,
+__device__ __forceinline__ void chain_helper(const Params& P, const RefineList& fl, ChainShared& sh, const uint32_t* __restrict__ list,
                                              uint32_t* progress_all, int lane) {
     const unsigned full = 0xffffffffu;
     uint32_t mk = 0;
@@ -1112,7 +1130,7 @@ __device__ __forceinline__ void chain_helper(const Params& P, const FinalizeList
 // long luminance chain before any gets a second, and a group's levels start together in one CTA);
 // after that a decoder that has finished takes the next entry of its queue from a counter in global
 // memory.  sync: four queue counters, then four progress words per group, all zero before the launch.
-__global__ void __launch_bounds__(64 * kChainPairs, 1) ac_refine_group_kernel(Params P, FinalizeList fl, const uint32_t* __restrict__ list,
+__global__ void __launch_bounds__(64 * kChainPairs, 1) ac_refine_group_kernel(Params P, RefineList fl, const uint32_t* __restrict__ list,
                                                                               uint32_t n_groups, uint32_t* __restrict__ sync, int levels, int rounds) {
     extern __shared__ __align__(16) unsigned char s_dyn[];     // one ChainShared per chain
     ChainShared* s_sh = reinterpret_cast<ChainShared*>(s_dyn);

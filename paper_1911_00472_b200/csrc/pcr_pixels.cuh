@@ -21,24 +21,26 @@
 
 namespace pcr {
 
-#ifndef PCR_PIX_MIN_CTAS
-#define PCR_PIX_MIN_CTAS 10                   // CTAs per SM the compiler must leave registers for (1: 13 % slower, 14: 8 % slower)
-#endif
-constexpr int kPixMcus = 8;                   // MCUs per CTA (4:2:0)
-constexpr int kPixThreads = 64;               // one thread per block for the transform
 constexpr int kStagePitch = 3 * 128 + 16;     // bytes per staged RGB row (+ spare, keeps rows 16-byte aligned)
 
 // Chroma sampling of a record as a template code: luminance blocks per MCU (horizontal, vertical),
-// components, and the MCUs of one work unit, chosen so that a unit is 128 pixels wide and has at
-// most 64 blocks: 4:2:0 -> 8 MCUs (32 Y + 8 Cb + 8 Cr), 4:2:2 -> 8 (16 + 8 + 8), 4:4:0 -> 16
-// (32 + 16 + 16), 4:4:4 -> 16 (16 + 16 + 16), greyscale -> 16 (16 Y).
+// components, and the MCUs (across) and MCU rows of one work unit.  A unit is 128 pixels wide and its blocks
+// fill whole warps, each of one kind (4:2:0: two warps of luminance, one of chroma): one thread per block.
 enum { kSamp420 = 0, kSamp422 = 1, kSamp440 = 2, kSamp444 = 3, kSampGrey = 4 };
 template <int kSamp> struct Sampling;
-template <> struct Sampling<kSamp420> { static constexpr int HS = 2, VS = 2, NC = 3, U = 8; };
-template <> struct Sampling<kSamp422> { static constexpr int HS = 2, VS = 1, NC = 3, U = 8; };
-template <> struct Sampling<kSamp440> { static constexpr int HS = 1, VS = 2, NC = 3, U = 16; };
-template <> struct Sampling<kSamp444> { static constexpr int HS = 1, VS = 1, NC = 3, U = 16; };
-template <> struct Sampling<kSampGrey> { static constexpr int HS = 1, VS = 1, NC = 1, U = 16; };
+template <> struct Sampling<kSamp420> { static constexpr int HS = 2, VS = 2, NC = 3, U = 8, R = 2; };
+template <> struct Sampling<kSamp422> { static constexpr int HS = 2, VS = 1, NC = 3, U = 8, R = 2; };
+template <> struct Sampling<kSamp440> { static constexpr int HS = 1, VS = 2, NC = 3, U = 16, R = 1; };
+template <> struct Sampling<kSamp444> { static constexpr int HS = 1, VS = 1, NC = 3, U = 16, R = 2; };
+template <> struct Sampling<kSampGrey> { static constexpr int HS = 1, VS = 1, NC = 1, U = 16, R = 4; };
+template <int kSamp> __host__ __device__ constexpr int unit_threads() {
+    using S = Sampling<kSamp>;
+    return S::U * S::R * (S::HS * S::VS + (S::NC == 3 ? 2 : 0));
+}
+constexpr int sampling_code(int hs, int vs, int nc) {
+    return nc == 1 ? kSampGrey : (hs == 2 ? (vs == 2 ? kSamp420 : kSamp422) : (vs == 2 ? kSamp440 : kSamp444));
+}
+constexpr uint32_t kUnitMcus[5] = {8, 8, 16, 16, 16}, kUnitRows[5] = {2, 2, 1, 2, 4};
 
 // zigzag position -> natural index, by walking the anti-diagonals
 struct ZigzagTable {
@@ -57,9 +59,10 @@ struct ZigzagTable {
 };
 __device__ constexpr ZigzagTable kZigzag{};
 
-// One 8-point pass on the integer matrix M (see the header comment): out[n] = (sum_k M[n][k] x[k] + rnd) >> shift
+// One 8-point pass on the integer matrix M (see the header comment): out[n] = (sum_k M[n][k] x[k] + rnd) >> kShift
+template <int kShift>
 __device__ __forceinline__ void idct8(uint32_t& x0, uint32_t& x1, uint32_t& x2, uint32_t& x3, uint32_t& x4, uint32_t& x5,
-                                      uint32_t& x6, uint32_t& x7, uint32_t rnd, int shift) {
+                                      uint32_t& x6, uint32_t& x7, uint32_t rnd) {
     constexpr uint32_t K1 = 8035, K2 = 7568, K3 = 6811, K4 = 5793, K5 = 4551, K6 = 3135, K7 = 1598;
     const uint32_t a0 = K4 * (x0 + x4) + rnd, a1 = K4 * (x0 - x4) + rnd;
     const uint32_t b0 = K2 * x2 + K6 * x6, b1 = K6 * x2 - K2 * x6;
@@ -68,347 +71,352 @@ __device__ __forceinline__ void idct8(uint32_t& x0, uint32_t& x1, uint32_t& x2, 
     const uint32_t o1 = K3 * x1 - K7 * x3 - K1 * x5 - K5 * x7;
     const uint32_t o2 = K5 * x1 - K1 * x3 + K7 * x5 + K3 * x7;
     const uint32_t o3 = K7 * x1 - K5 * x3 + K3 * x5 - K1 * x7;
-    x0 = (uint32_t)((int)(e0 + o0) >> shift); x7 = (uint32_t)((int)(e0 - o0) >> shift);
-    x1 = (uint32_t)((int)(e1 + o1) >> shift); x6 = (uint32_t)((int)(e1 - o1) >> shift);
-    x2 = (uint32_t)((int)(e2 + o2) >> shift); x5 = (uint32_t)((int)(e2 - o2) >> shift);
-    x3 = (uint32_t)((int)(e3 + o3) >> shift); x4 = (uint32_t)((int)(e3 - o3) >> shift);
+    x0 = (uint32_t)((int)(e0 + o0) >> kShift); x7 = (uint32_t)((int)(e0 - o0) >> kShift);
+    x1 = (uint32_t)((int)(e1 + o1) >> kShift); x6 = (uint32_t)((int)(e1 - o1) >> kShift);
+    x2 = (uint32_t)((int)(e2 + o2) >> kShift); x5 = (uint32_t)((int)(e2 - o2) >> kShift);
+    x3 = (uint32_t)((int)(e3 + o3) >> kShift); x4 = (uint32_t)((int)(e3 - o3) >> kShift);
 }
 
-// bytes {clamp(v0), clamp(v1), clamp(v2), clamp(v3)} of a little-endian word, clamp to 0..255
-__device__ __forceinline__ uint32_t pack4_sat(int v0, int v1, int v2, int v3) {
-    uint32_t hi, w;
-    asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, %3;" : "=r"(hi) : "r"(v3), "r"(v2), "r"(0));
-    asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, %3;" : "=r"(w) : "r"(v1), "r"(v0), "r"(hi));
-    return w;
+// Two samples as a pair of 16-bit numbers, {clamp((a >> 16) + 128), clamp((b >> 16) + 128)} with clamp to 0..255: the
+// upper halves by one permutation, then two packed operations.  The upper end is cut before 128 is added, so
+// nothing wraps for sums near the ends of the 32-bit range.
+__device__ __forceinline__ uint32_t sample_pair(uint32_t a, uint32_t b) {
+    return __viaddmax_s16x2(__vmins2(__byte_perm(a, b, 0x7632), 0x007F007Fu), 0x00800080u, 0u);
 }
+// bytes {lo(a), hi(a), lo(b), hi(b)} of two pairs
+__device__ __forceinline__ uint32_t pair_bytes(uint32_t a, uint32_t b) { return __byte_perm(a, b, 0x6420); }
 
-// bytes {clamp(v0 + 128), ..., clamp(v3 + 128)}, clamp to 0..255, for any 32-bit v: clamping v to
-// -128..127 and flipping the byte's top bit is the same as adding 128 and clamping to 0..255, and it
-// needs no addition that could overflow for v near the ends of the 32-bit range
-__device__ __forceinline__ uint32_t pack4_sat_plus128(int v0, int v1, int v2, int v3) {
-    uint32_t hi, w;
-    asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, %3;" : "=r"(hi) : "r"(v3), "r"(v2), "r"(0));
-    asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, %3;" : "=r"(w) : "r"(v1), "r"(v0), "r"(hi));
-    return w ^ 0x80808080u;
-}
-
-// kRefine: first fold the side data of the AC refinement scans (see ScanAux) into the block, in
-// scan order, and write the updated 128-byte line back, so the planes in device memory hold the
-// final coefficients.  The thread parks its line in shared memory for that (word w of thread t
-// at [w][t]): the walk over the set bits of the masks addresses coefficients by position, which
-// registers cannot do.  A correction moves a non-zero coefficient away from zero by 2^Al if its
-// bit Al is still clear; a new coefficient is +-2^Al.
+// Where a decode's coefficients lie (built per call for the chosen k, see CoefLists in pcr_types.h): the
+// DC plane, the head plane (positions 1..7), and per first pass and component the masks and values of the rest.
+// The refinements' side data is folded in here, in scan order.  Nothing of this is written back: the
+// lists of all decoded scans stay as they are, and whoever needs blocks expands them again.
 //
-// kDcMode: 0 = all 64 coefficients sit in the block's line; 1 = positions 0..7 come from the dense
-// head plane (the line's first 16 bytes are ignored); 2 = the block has nothing but its DC
-// coefficient (no AC scan decoded): only the head plane is read and the transform collapses to
-// one value; 3 = no decoded scan reaches beyond position 7: the lines are not read at all.
-// kRoi: only work units that touch their image's crop rectangle (P.roi) are processed.
+// Expands block `blk` of the planes (number `local` inside its component) into this thread's line in shared
+// memory: position p is the int16 at line + (p >> 2) * 8 * kT + 2 * (p & 3) (kT threads' lines interleaved by
+// eight bytes: every thread keeps to its own banks, whatever position it addresses).
+// A correction moves a non-zero coefficient away from zero by 2^Al if its bit Al is still clear; a
+// new coefficient is +-2^Al.
+template <int kT, bool kRefine>
+__device__ __forceinline__ void expand_block(const Params& P, const CoefLists& cl, int comp, uint64_t blk, uint64_t local, uint8_t* line) {
+    constexpr int kPitch = 8 * kT;
+    auto at = [&](int pos) { return reinterpret_cast<int16_t*>(line + (pos >> 2) * kPitch + 2 * (pos & 3)); };
+    const int nfirst = cl.n_first[comp], nref = kRefine ? cl.n_refine[comp] : 0;
+    // all of the block's loads are requested before the first is used
+    const uint4 zero4 = make_uint4(0, 0, 0, 0);
+    uint4 head = __ldg(reinterpret_cast<const uint4*>(P.head + blk * 8));
+    const uint32_t dc = __ldg(reinterpret_cast<const uint16_t*>(P.dc) + blk);
+    uint4 rec = zero4;
+    if (nfirst > 0) rec = __ldg(reinterpret_cast<const uint4*>(P.aux + cl.first[comp][0]) + local);
+    uint4 a0 = zero4, b0 = zero4, a1 = zero4, b1 = zero4;
+    if (kRefine) {
+        if (nref > 0) { const uint4* o = reinterpret_cast<const uint4*>(P.aux + cl.refine[comp][0]) + 2 * local; a0 = __ldg(o); b0 = __ldg(o + 1); }
+        if (nref > 1) { const uint4* o = reinterpret_cast<const uint4*>(P.aux + cl.refine[comp][1]) + 2 * local; a1 = __ldg(o); b1 = __ldg(o + 1); }
+    }
+#pragma unroll
+    for (int w = 2; w < 16; ++w) *reinterpret_cast<uint2*>(line + w * kPitch) = make_uint2(0, 0);
+    const uint4 hm = cl.head_mask[comp];           // positions that no decoded scan covers may hold a later scan's values
+    *reinterpret_cast<uint2*>(line) = make_uint2((head.x & hm.x) | dc, head.y & hm.y);
+    *reinterpret_cast<uint2*>(line + kPitch) = make_uint2(head.z & hm.z, head.w & hm.w);
+    for (int i = 0; i < nfirst; ++i) {
+        if (i) rec = __ldg(reinterpret_cast<const uint4*>(P.aux + cl.first[comp][i]) + local);
+        const int16_t* v = reinterpret_cast<const int16_t*>(((uint64_t)rec.w << 32) | rec.z);
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            uint32_t m = half ? rec.y : rec.x & ~0xFFu;
+            while (m) {
+                const int pos = 32 * half + __ffs((int)m) - 1;
+                m &= m - 1u;
+                *at(pos) = __ldg(v++);
+            }
+        }
+    }
+    if (kRefine) {
+        for (int i = 0; i < nref; ++i) {
+            const int p1 = cl.p1[comp][i];
+            uint4 a = i == 0 ? a0 : a1, b = i == 0 ? b0 : b1;    // {mask, corrections}, {new, signs}
+            if (i > 1) { const uint4* o = reinterpret_cast<const uint4*>(P.aux + cl.refine[comp][i]) + 2 * local; a = __ldg(o); b = __ldg(o + 1); }
+            // corrections: the coefficients that were non-zero before the scan, in zigzag order, take the
+            // correction bits in reading order (as many as there are such positions, the last one in bit 0);
+            // the walk ends with the last set bit
+            const uint32_t h0 = a.x & ~b.x, h1 = a.y & ~b.y;
+            uint64_t cc = ((uint64_t)a.w << 32) | a.z;
+            if (cc) cc <<= 64 - __popc(h0) - __popc(h1);
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                uint32_t h = half ? h1 : h0;
+                while (h && cc) {
+                    const int pos = 32 * half + __ffs((int)h) - 1;
+                    h &= h - 1u;
+                    if ((long long)cc < 0) {
+                        int16_t* e = at(pos);
+                        const int v = *e;
+                        if ((v & p1) == 0) *e = (int16_t)(v >= 0 ? v + p1 : v - p1);
+                    }
+                    cc <<= 1;
+                }
+            }
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                uint32_t nw = half ? b.y : b.x;
+                const uint32_t sg = half ? b.w : b.z;
+                while (nw) {
+                    const int bit = __ffs((int)nw) - 1;
+                    nw &= nw - 1u;
+                    *at(32 * half + bit) = (int16_t)(((sg >> bit) & 1u) ? p1 : -p1);
+                }
+            }
+        }
+    }
+}
+
+// kMode: 0 = all 64 coefficients sit in the block's 128-byte line (pcr_pixels_noalloc); 1 = coefficient lists
+// (expand_block); 3 = no decoded scan reaches beyond position 7 and none is a refinement: the head plane and
+// the DC plane are all there is.
+// kRefine: AC refinements among the decoded scans (kMode 1).
+// kRoi: only work units, and in them MCU rows, that touch their image's crop rectangle (P.roi) are processed.
 //
 // kStage serves triangle chroma upsampling, which needs chroma samples of neighbouring work
 // units: 0 = everything in one launch (2x2 replication); 1 = chroma pass: the chroma blocks are
-// folded, written back, transformed and their samples stored in P.chroma, nothing else; 2 = pixel
-// pass: luminance blocks as in 0, chroma samples with a one-sample border read back from
-// P.chroma, every pixel's chroma = (9 own + 3 horizontally nearer + 3 vertically nearer +
-// 1 diagonal + 8) >> 4, neighbours clamped to the MCU-padded planes.
+// transformed and their samples stored in P.chroma, nothing else; 2 = pixel pass: luminance blocks
+// as in 0, chroma samples with a one-sample border read back from P.chroma, every pixel's chroma = (9 own +
+// 3 horizontally nearer + 3 vertically nearer + 1 diagonal + 8) >> 4, neighbours clamped to the MCU-padded
+// planes.  3 = no pixels: the expanded blocks are written to P.planes (pcr_coeffs).
 // kSamp: the record's chroma sampling (see Sampling); the triangle filter (kStage 1, 2) exists for
 // 4:2:0 only.  A greyscale record has no chroma: every pixel is (Y, Y, Y).
-template <bool kRefine, int kDcMode, bool kRoi = false, int kStage = 0, int kSamp = kSamp420>
-__global__ void __launch_bounds__(kPixThreads, PCR_PIX_MIN_CTAS) pixel_kernel(Params P, FinalizeList fl, uint8_t* __restrict__ out) {
+//
+// One thread per block through the whole transform; the chroma samples go through shared memory, the luminance
+// samples stay in the registers of the thread that made them and meet the chroma there, two pixels
+// per instruction (16-bit pairs).  Bound by instruction issue: see the table of kernels for the counts.
+template <bool kRefine, int kMode, bool kRoi = false, int kStage = 0, int kSamp = kSamp420>
+__global__ void __launch_bounds__(unit_threads<kSamp>(), 672 / unit_threads<kSamp>())
+pixel_kernel(Params P, CoefLists cl, uint8_t* __restrict__ out) {
     using S = Sampling<kSamp>;
-    constexpr int HS = S::HS, VS = S::VS, NC = S::NC, U = S::U;
+    constexpr int HS = S::HS, VS = S::VS, NC = S::NC, U = S::U, R = S::R, kT = unit_threads<kSamp>();
     constexpr int kYCols = HS * U;                            // luminance blocks per block row of a unit
-    constexpr int kYBlocks = VS * kYCols;                      // luminance blocks of a unit
-    constexpr int kBlocks = kYBlocks + (NC == 3 ? 2 * U : 0);
+    constexpr int kYBlocks = R * VS * kYCols;                  // luminance blocks of a unit
     constexpr int kBpm = HS * VS + (NC == 3 ? 2 : 0);          // blocks per MCU
-    constexpr int kPxW = 8 * HS, kPxH = 8 * VS;                // pixels per MCU
-    static_assert(kBlocks <= kPixThreads && kPxW * U == 128, "a unit is 128 pixels wide and has at most 64 blocks");
-    static_assert(kStage == 0 || kSamp == kSamp420, "triangle upsampling is built for 4:2:0");
-    __shared__ __align__(16) uint32_t s_line[kRefine ? 32 * kPixThreads : 1];
-    __shared__ __align__(16) uint8_t s_y[kPxH][128];
-    __shared__ __align__(16) uint8_t s_c[2][8][8 * U];
-    __shared__ __align__(16) uint8_t s_stage[kPxH * kStagePitch];
-    __shared__ __align__(16) uint16_t s_q[3][64];
-    __shared__ uint8_t s_ct[kStage == 2 ? 2 : 1][kStage == 2 ? 10 : 1][kStage == 2 ? 8 * kPixMcus + 2 : 1];   // chroma tile + border
+    constexpr int kPxW = 8 * HS, kPxH = 8 * VS, kRows = R * kPxH;   // pixels per MCU, pixel rows of a unit
+    static_assert(kPxW * U == 128 && kT % 32 == 0 && kYBlocks % 32 == 0, "a unit is 128 pixels wide, its warps are of one kind");
+    static_assert(kStage == 0 || kStage == 3 || kSamp == kSamp420, "triangle upsampling is built for 4:2:0");
+    constexpr int kLineBytes = kMode == 1 ? 128 * kT : 16, kStageBytes = kRows * kStagePitch;
+    // the lines are read before, the staged rows written after the barrier behind the transform
+    __shared__ __align__(16) uint8_t s_mem[kStage == 3 || kLineBytes > kStageBytes ? kLineBytes : kStageBytes];
+    __shared__ __align__(16) uint8_t s_c[2][8 * R][8 * U];
+    __shared__ __align__(16) int32_t s_q[3][64];
+    __shared__ uint8_t s_ct[kStage == 2 ? 2 : 1][kStage == 2 ? 8 * R + 2 : 1][kStage == 2 ? 8 * U + 2 : 1];   // chroma tile + border
+    uint8_t* const s_stage = s_mem;
 
     const int tid = threadIdx.x;
     const Unit un = P.units[blockIdx.x];
     const ImgDesc im = P.imgs[un.img];
-    const int nm = min(U, (int)im.mx - (int)un.mcol0);                // MCUs in this unit
-    if (kRoi) {                                                       // whole CTA: nothing of this unit is wanted
+    const int nm = min(U, (int)im.mx - (int)un.mcol0);                // MCUs across in this unit
+    int r_lo = 0, r_hi = min(R, (int)im.my - (int)un.mrow);           // its MCU rows that are wanted
+    if (kRoi) {
         const CropRect r = P.roi[un.img];
-        const uint32_t ux0 = (uint32_t)kPxW * un.mcol0, uy0 = (uint32_t)kPxH * un.mrow;
-        if (ux0 >= r.x0 + r.w || ux0 + (uint32_t)(kPxW * nm) <= r.x0 || uy0 >= r.y0 + r.h || uy0 + (uint32_t)kPxH <= r.y0) return;
+        const int ux0 = kPxW * un.mcol0, y0 = (int)(r.y0 / kPxH) - (int)un.mrow, y1 = (int)((r.y0 + r.h - 1u) / kPxH) + 1 - (int)un.mrow;
+        r_lo = max(r_lo, y0); r_hi = min(r_hi, y1);
+        if (r_lo >= r_hi || ux0 >= (int)(r.x0 + r.w) || ux0 + kPxW * nm <= (int)r.x0) return;      // whole CTA: nothing of this unit is wanted
     }
-    for (int i = tid; i < 96; i += kPixThreads)
-        reinterpret_cast<uint32_t*>(&s_q[0][0])[i] = __ldg(reinterpret_cast<const uint32_t*>(P.qtab + (size_t)un.img * 192) + i);
-    __syncthreads();
-
-    // ---- transform: thread j owns block j; block order: the unit's luminance block rows, then Cb, then Cr
-    {
-        const int j = tid;
-        int comp = 0;
-        bool valid = false;
-        uint64_t blk = 0, local = 0;      // block number in the planes / inside its component
-        int yr = 0, yc = 0;               // block row / column inside the unit
-        if (j < kYBlocks) {
-            yr = j / kYCols; yc = j % kYCols;
-            valid = yc < HS * nm;
-            local = (uint64_t)(VS * un.mrow + yr) * (HS * im.mx) + HS * un.mcol0 + yc;
-            blk = im.blk_base + local;
-            local += (uint64_t)(HS * VS) * (im.blk_base / kBpm);
-        } else if (j < kBlocks) {
-            yc = (j - kYBlocks) % U;
-            comp = 1 + (j - kYBlocks) / U;
-            valid = yc < nm;
-            local = (uint64_t)un.mrow * im.mx + un.mcol0 + yc;
-            blk = im.blk_base + (uint64_t)(HS * VS + comp - 1) * im.mx * im.my + local;
-            local += im.blk_base / kBpm;
+    if (kStage != 3) {
+        for (int i = tid; i < 96; i += kT) {
+            const uint32_t q2 = __ldg(reinterpret_cast<const uint32_t*>(P.qtab + (size_t)un.img * 192) + i);
+            *reinterpret_cast<int2*>(&s_q[0][0] + 2 * i) = make_int2((int)(q2 & 0xFFFFu), (int)(q2 >> 16));
         }
-        if (kStage == 1 && comp == 0) valid = false;          // chroma pass
-        if (kStage == 2 && comp != 0) valid = false;          // pixel pass: chroma comes from the sample planes
-        uint8_t* cplane = nullptr;                            // chroma pass: where this block's samples go
-        if (kStage == 1 && comp != 0)
-            cplane = P.chroma + (im.blk_base / 6) * 128 + (comp == 2 ? 64ull * im.mx * im.my : 0ull) +
-                     (size_t)(8 * un.mrow) * (8 * im.mx) + 8 * (un.mcol0 + yc);
-        if (valid && kDcMode == 2) {
-            // all AC zero: both passes keep only the k = 0 term, every sample of the block is equal
-            constexpr uint32_t K4 = 5793;
-            const int F = (int)P.head[blk * 8] * (int)s_q[comp][0];
-            const int T = (int)(K4 * (uint32_t)F + (1u << 11)) >> 12;
-            const int smp = (int)(K4 * (uint32_t)T + (1u << 15)) >> 16;
-            const uint32_t w = pack4_sat_plus128(smp, smp, smp, smp);
-            uint8_t* dst;
-            int pitch;
-            if (comp == 0) { dst = &s_y[yr * 8][yc * 8]; pitch = 128; }
-            else { dst = &s_c[comp - 1][0][yc * 8]; pitch = 8 * U; }
-#pragma unroll
-            for (int y = 0; y < 8; ++y) *reinterpret_cast<uint2*>(dst + y * pitch) = make_uint2(w, w);
-        } else if (valid) {
-            uint4* line = reinterpret_cast<uint4*>(P.planes + blk * 64);
-            uint4 raw[8];
-            const uint4* headv = reinterpret_cast<const uint4*>(P.head + blk * 8);
-            if (kRefine && fl.n[comp] > 0) {
-                // the side data of the first two refinement scans is requested before the lines: all of the
-                // block's loads are then in flight together
-                const int nref = fl.n[comp];
-                const ulonglong2 zero2 = make_ulonglong2(0ull, 0ull);
-                ulonglong2 a0 = zero2, b0 = zero2, a1 = zero2, b1 = zero2;
-                {
-                    const ulonglong2* o = reinterpret_cast<const ulonglong2*>(P.aux + fl.base[comp][0] + local * 4);
-                    a0 = __ldg(o); b0 = __ldg(o + 1);                        // {mask, corrections}, {new, signs}
-                    if (nref > 1) {
-                        const ulonglong2* o1 = reinterpret_cast<const ulonglong2*>(P.aux + fl.base[comp][1] + local * 4);
-                        a1 = __ldg(o1); b1 = __ldg(o1 + 1);
-                    }
-                }
-                if (kDcMode == 3) {
-#pragma unroll
-                    for (int q = 1; q < 8; ++q) raw[q] = make_uint4(0, 0, 0, 0);
-                } else {
-#pragma unroll
-                    for (int q = (kDcMode == 0 ? 0 : 1); q < 8; ++q) raw[q] = line[q];
-                }
-                if (kDcMode != 0) raw[0] = *headv;
-                uint32_t* col = s_line + tid;
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    col[(4 * q) * kPixThreads] = raw[q].x; col[(4 * q + 1) * kPixThreads] = raw[q].y;
-                    col[(4 * q + 2) * kPixThreads] = raw[q].z; col[(4 * q + 3) * kPixThreads] = raw[q].w;
-                }
-                uint32_t dirty = 0;                                         // 16-byte chunks of the line that changed
-                for (int i = 0; i < nref; ++i) {
-                    const int p1 = fl.p1[comp][i];
-                    ulonglong2 a = i == 0 ? a0 : a1, b = i == 0 ? b0 : b1;
-                    if (i > 1) {
-                        const ulonglong2* o = reinterpret_cast<const ulonglong2*>(P.aux + fl.base[comp][i] + local * 4);
-                        a = __ldg(o); b = __ldg(o + 1);
-                    }
-                    // corrections: the coefficients that were non-zero before the scan, in zigzag order, take the
-                    // correction bits in reading order (as many as there are such positions, the last one in bit 0);
-                    // the walk ends with the last set bit.
-                    // Positions 0..31 and 32..63 are walked as 32-bit masks.
-                    const uint64_t hist = a.x & ~b.x;
-                    uint64_t cc = a.y ? a.y << (64 - __popcll(hist)) : 0ull;
-#pragma unroll
-                    for (int half = 0; half < 2; ++half) {
-                        uint32_t h32 = half ? (uint32_t)(hist >> 32) : (uint32_t)hist;
-                        uint32_t* hb = col + half * 16 * kPixThreads;
-                        while (h32 && cc) {
-                            const int pos = __ffs((int)h32) - 1;
-                            h32 &= h32 - 1u;
-                            if ((long long)cc < 0) {
-                                int16_t* e = reinterpret_cast<int16_t*>(hb + (pos >> 1) * kPixThreads) + (pos & 1);
-                                const int v = *e;
-                                if ((v & p1) == 0) { *e = (int16_t)(v >= 0 ? v + p1 : v - p1); dirty |= 1u << ((pos >> 3) + 4 * half); }
-                            }
-                            cc <<= 1;
-                        }
-                    }
-                    // new coefficients: +-2^Al at positions that were zero
-#pragma unroll
-                    for (int half = 0; half < 2; ++half) {
-                        uint32_t nw = half ? (uint32_t)(b.x >> 32) : (uint32_t)b.x;
-                        const uint32_t sg = half ? (uint32_t)(b.y >> 32) : (uint32_t)b.y;
-                        uint32_t* hb = col + half * 16 * kPixThreads;
-                        while (nw) {
-                            const int pos = __ffs((int)nw) - 1;
-                            nw &= nw - 1u;
-                            *(reinterpret_cast<int16_t*>(hb + (pos >> 1) * kPixThreads) + (pos & 1)) = (int16_t)(((sg >> pos) & 1u) ? p1 : -p1);
-                            dirty |= 1u << ((pos >> 3) + 4 * half);
-                        }
-                    }
-                }
-                // only the chunks that changed are read back and written to the planes
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    if ((dirty >> q) & 1u) {
-                        raw[q] = make_uint4(col[(4 * q) * kPixThreads], col[(4 * q + 1) * kPixThreads],
-                                            col[(4 * q + 2) * kPixThreads], col[(4 * q + 3) * kPixThreads]);
-                        if (q == 0 && kDcMode != 0) *reinterpret_cast<uint4*>(P.head + blk * 8) = raw[0];
-                        else if (kDcMode != 3) line[q] = raw[q];
-                    }
-                }
-            } else {
-                if (kDcMode == 3) {
-#pragma unroll
-                    for (int q = 1; q < 8; ++q) raw[q] = make_uint4(0, 0, 0, 0);
-                } else {
-#pragma unroll
-                    for (int q = (kDcMode == 0 ? 0 : 1); q < 8; ++q) raw[q] = __ldg(line + q);
-                }
-                if (kDcMode != 0) raw[0] = __ldg(headv);
-            }
-            const uint32_t* qw = reinterpret_cast<const uint32_t*>(&s_q[comp][0]);
-            uint32_t v[64];
+    }
+    // ---- thread j owns block j: the unit's luminance block rows, then its Cb rows, then its Cr rows
+    int comp = 0, yr, yc;                 // component, block row / column inside the unit
+    uint64_t blk, local;                  // block number in the planes / inside its component
+    bool valid;
+    if (NC == 1 || tid < kYBlocks) {
+        yr = tid / kYCols; yc = tid % kYCols;
+        valid = yc < HS * nm && yr >= VS * r_lo && yr < VS * r_hi && kStage != 1;
+        local = (uint64_t)(VS * un.mrow + yr) * (HS * im.mx) + HS * un.mcol0 + yc;
+        blk = im.blk_base + local;
+        local += (uint64_t)(HS * VS) * (im.blk_base / kBpm);
+    } else {
+        const int i = tid - kYBlocks;
+        comp = 1 + i / (U * R);
+        yr = i % (U * R) / U; yc = i % U;
+        valid = yc < nm && yr >= r_lo && yr < r_hi && kStage != 2;
+        local = (uint64_t)(un.mrow + yr) * im.mx + un.mcol0 + yc;
+        blk = im.blk_base + (uint64_t)(HS * VS + comp - 1) * im.mx * im.my + local;
+        local += im.blk_base / kBpm;
+    }
+    uint8_t* const line = s_mem + 8 * tid;
+    if (kMode == 1 && valid) expand_block<kT, kRefine>(P, cl, comp, blk, local, line);
+    if (kStage == 3) {
+        if (valid) {
+            uint4* dst = reinterpret_cast<uint4*>(P.planes + blk * 64);
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
-                const uint32_t w4[4] = {raw[q].x, raw[q].y, raw[q].z, raw[q].w};
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int k = 8 * q + 2 * e;                 // zigzag positions k, k + 1
-                    const uint32_t qq = qw[k >> 1];
-                    const int c0 = (int)(short)(w4[e] & 0xFFFFu), c1 = (int)w4[e] >> 16;
-                    v[kZigzag.nat[k]] = (uint32_t)(c0 * (int)(qq & 0xFFFFu));
-                    v[kZigzag.nat[k + 1]] = (uint32_t)(c1 * (int)(qq >> 16));
-                }
-            }
-            // pass 1: columns (two fraction bits kept)
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-                idct8(v[u], v[8 + u], v[16 + u], v[24 + u], v[32 + u], v[40 + u], v[48 + u], v[56 + u], 1u << 11, 12);
-            // pass 2: rows; the +128 level shift is part of the packing
-            uint8_t* dst;
-            int pitch;
-            if (kStage == 1) { dst = cplane; pitch = 8 * (int)im.mx; }
-            else if (comp == 0) { dst = &s_y[yr * 8][yc * 8]; pitch = 128; }
-            else { dst = &s_c[comp - 1][0][yc * 8]; pitch = 8 * U; }
-#pragma unroll
-            for (int y = 0; y < 8; ++y) {
-                idct8(v[8 * y], v[8 * y + 1], v[8 * y + 2], v[8 * y + 3], v[8 * y + 4], v[8 * y + 5], v[8 * y + 6], v[8 * y + 7],
-                      1u << 15, 16);
-                const uint32_t lo = pack4_sat_plus128((int)v[8 * y], (int)v[8 * y + 1], (int)v[8 * y + 2], (int)v[8 * y + 3]);
-                const uint32_t hi = pack4_sat_plus128((int)v[8 * y + 4], (int)v[8 * y + 5], (int)v[8 * y + 6], (int)v[8 * y + 7]);
-                *reinterpret_cast<uint2*>(dst + y * pitch) = make_uint2(lo, hi);
+                const uint2 lo = *reinterpret_cast<const uint2*>(line + (2 * q) * 8 * kT), hi = *reinterpret_cast<const uint2*>(line + (2 * q + 1) * 8 * kT);
+                dst[q] = make_uint4(lo.x, lo.y, hi.x, hi.y);
             }
         }
+        return;
     }
-    if (kStage == 1) return;                                // chroma pass: no pixels
+    __syncthreads();                  // the quantisers are there
+    uint32_t yp[32];                      // a luminance block's samples, two per word (row y: words 4y .. 4y + 3)
+    if (valid) {
+        uint32_t v[64];
+        const int4* q4 = reinterpret_cast<const int4*>(&s_q[comp][0]);
+        uint4 head = make_uint4(0, 0, 0, 0);
+        if (kMode == 3) {
+            const uint4 hm = cl.head_mask[comp];
+            head = __ldg(reinterpret_cast<const uint4*>(P.head + blk * 8));
+            head = make_uint4((head.x & hm.x) | __ldg(reinterpret_cast<const uint16_t*>(P.dc) + blk), head.y & hm.y, head.z & hm.z, head.w & hm.w);
+        }
+        const uint4* dense = reinterpret_cast<const uint4*>(P.planes + blk * 64);
+#pragma unroll
+        for (int w = 0; w < 16; ++w) {                                // zigzag positions 4w .. 4w + 3
+            uint2 c2;
+            if (kMode == 3) c2 = w == 0 ? make_uint2(head.x, head.y) : (w == 1 ? make_uint2(head.z, head.w) : make_uint2(0, 0));
+            else if (kMode == 0) c2 = __ldg(reinterpret_cast<const uint2*>(dense) + w);
+            else c2 = *reinterpret_cast<const uint2*>(line + w * 8 * kT);
+            const int4 q = q4[w];
+            v[kZigzag.nat[4 * w]] = (uint32_t)((int)(short)(c2.x & 0xFFFFu) * q.x);
+            v[kZigzag.nat[4 * w + 1]] = (uint32_t)(((int)c2.x >> 16) * q.y);
+            v[kZigzag.nat[4 * w + 2]] = (uint32_t)((int)(short)(c2.y & 0xFFFFu) * q.z);
+            v[kZigzag.nat[4 * w + 3]] = (uint32_t)(((int)c2.y >> 16) * q.w);
+        }
+        // pass 1: columns (two fraction bits kept)
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            idct8<12>(v[u], v[8 + u], v[16 + u], v[24 + u], v[32 + u], v[40 + u], v[48 + u], v[56 + u], 1u << 11);
+        // pass 2: rows; the final shift by 16 takes the upper halves, the level shift is part of the clamping
+#pragma unroll
+        for (int y = 0; y < 8; ++y) {
+            uint32_t* r = v + 8 * y;
+            idct8<0>(r[0], r[1], r[2], r[3], r[4], r[5], r[6], r[7], 1u << 15);
+#pragma unroll
+            for (int p = 0; p < 4; ++p) yp[4 * y + p] = sample_pair(r[2 * p], r[2 * p + 1]);
+        }
+        if (NC == 3 && comp != 0) {
+            uint8_t* dst;
+            int pitch;
+            if (kStage == 1) {
+                pitch = 8 * (int)im.mx;
+                dst = P.chroma + (im.blk_base / 6) * 128 + (comp == 2 ? 64ull * im.mx * im.my : 0ull) +
+                      (size_t)(8 * (un.mrow + yr)) * pitch + 8 * (un.mcol0 + yc);
+            } else { dst = &s_c[comp - 1][8 * yr][8 * yc]; pitch = 8 * U; }
+#pragma unroll
+            for (int y = 0; y < 8; ++y)
+                *reinterpret_cast<uint2*>(dst + y * pitch) = make_uint2(pair_bytes(yp[4 * y], yp[4 * y + 1]), pair_bytes(yp[4 * y + 2], yp[4 * y + 3]));
+        }
+    }
+    if (kStage == 1) return;                                          // chroma pass: no pixels
     if (kStage == 2) {
         // chroma tile of the unit with a one-sample border, clamped to the padded planes
         const int cw = 8 * (int)im.mx, chh = 8 * (int)im.my, tw = 8 * nm + 2;
         const uint8_t* cbase = P.chroma + (im.blk_base / 6) * 128;
-        for (int i = tid; i < 2 * 10 * tw; i += kPixThreads) {
-            const int c = i / (10 * tw), rem2 = i - c * 10 * tw, r = rem2 / tw, x = rem2 - r * tw;
+        for (int i = tid; i < 2 * (8 * R + 2) * tw; i += kT) {
+            const int c = i / ((8 * R + 2) * tw), rem2 = i - c * (8 * R + 2) * tw, r = rem2 / tw, x = rem2 - r * tw;
             const int gy = min(max(8 * (int)un.mrow + r - 1, 0), chh - 1), gx2 = min(max(8 * (int)un.mcol0 + x - 1, 0), cw - 1);
             s_ct[c][r][x] = cbase[(size_t)c * cw * chh + (size_t)gy * cw + gx2];
         }
     }
     __syncthreads();
 
-    // ---- colour: 4 pixels per step, staged as the output's byte layout
-    for (int gi = tid; gi < kPxH * 32; gi += kPixThreads) {
-        const int row = gi / 32, gx = gi % 32;                  // 32 groups of four pixels per row
-        if (4 * gx >= kPxW * nm) continue;
-        const uint32_t yw = *reinterpret_cast<const uint32_t*>(&s_y[row][4 * gx]);
-        int px[12];
-        if (kStage == 2) {
-            const int ry = 1 + (row >> 1), rn = ry + ((row & 1) ? 1 : -1);       // own / vertically nearer tile row
+    // ---- colour, staged as the output's byte layout: 8 pixels of a row = 24 bytes
+    if (valid && (NC == 1 || comp == 0)) {
+        // chroma terms of a sample c (0..255): the upper halves of kR * c + rR and so on
+        constexpr int kRr = 91881, kGb = -22553, kGr = -46802, kBb = 116130, kRnd = 32768;
+        auto red = [&](int cr) { return (uint32_t)(kRr * cr + (kRnd - 128 * kRr)); };
+        auto green = [&](int cb, int cr) { return (uint32_t)(kGb * cb + kGr * cr + (kRnd - 128 * (kGb + kGr))); };
+        auto blue = [&](int cb) { return (uint32_t)(kBb * cb + (kRnd - 128 * kBb)); };
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int x = 4 * gx + e, cx = 1 + (x >> 1), cn = cx + ((x & 1) ? 1 : -1);
-                const int cb = ((9 * s_ct[0][ry][cx] + 3 * s_ct[0][ry][cn] + 3 * s_ct[0][rn][cx] + s_ct[0][rn][cn] + 8) >> 4) - 128;
-                const int cr = ((9 * s_ct[1][ry][cx] + 3 * s_ct[1][ry][cn] + 3 * s_ct[1][rn][cx] + s_ct[1][rn][cn] + 8) >> 4) - 128;
-                const int Y = (int)((yw >> (8 * e)) & 255u);
-                px[e * 3 + 0] = Y + ((91881 * cr + 32768) >> 16);
-                px[e * 3 + 1] = Y + ((-22553 * cb - 46802 * cr + 32768) >> 16);
-                px[e * 3 + 2] = Y + ((116130 * cb + 32768) >> 16);
+        for (int y = 0; y < 8; ++y) {
+            uint32_t dr[4], dg[4], db[4];                             // per pixel pair
+            if (kStage == 2) {
+                const int row = 8 * yr + y, ry = 1 + (row >> 1), rn = ry + ((row & 1) ? 1 : -1);   // own / vertically nearer tile row
+#pragma unroll
+                for (int p = 0; p < 4; ++p) {
+                    uint32_t x2[3][2];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int cx = 1 + 4 * yc + p, cn = cx + (e ? 1 : -1);
+                        int m[2];
+#pragma unroll
+                        for (int c = 0; c < 2; ++c)
+                            m[c] = (9 * s_ct[c][ry][cx] + 3 * s_ct[c][ry][cn] + 3 * s_ct[c][rn][cx] + s_ct[c][rn][cn] + 8) >> 4;
+                        x2[0][e] = red(m[1]); x2[1][e] = green(m[0], m[1]); x2[2][e] = blue(m[0]);
+                    }
+                    dr[p] = __byte_perm(x2[0][0], x2[0][1], 0x7632); dg[p] = __byte_perm(x2[1][0], x2[1][1], 0x7632); db[p] = __byte_perm(x2[2][0], x2[2][1], 0x7632);
+                }
+            } else if (NC == 3 && HS == 2) {
+                if (y % VS == 0) {
+                    const uint32_t cbw = *reinterpret_cast<const uint32_t*>(&s_c[0][(8 * yr + y) / VS][4 * yc]);
+                    const uint32_t crw = *reinterpret_cast<const uint32_t*>(&s_c[1][(8 * yr + y) / VS][4 * yc]);
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) {                     // two pixels share a sample
+                        const int cb = (int)((cbw >> (8 * p)) & 255u), cr = (int)((crw >> (8 * p)) & 255u);
+                        dr[p] = __byte_perm(red(cr), 0, 0x3232); dg[p] = __byte_perm(green(cb, cr), 0, 0x3232); db[p] = __byte_perm(blue(cb), 0, 0x3232);
+                    }
+                }
+            } else if (NC == 3) {
+                if (y % VS == 0) {
+                    const uint2 cb2 = *reinterpret_cast<const uint2*>(&s_c[0][(8 * yr + y) / VS][8 * yc]);
+                    const uint2 cr2 = *reinterpret_cast<const uint2*>(&s_c[1][(8 * yr + y) / VS][8 * yc]);
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) {
+                        const uint32_t cbw = (p < 2 ? cb2.x : cb2.y) >> (16 * (p & 1)), crw = (p < 2 ? cr2.x : cr2.y) >> (16 * (p & 1));
+                        const int cb0 = (int)(cbw & 255u), cb1 = (int)((cbw >> 8) & 255u), cr0 = (int)(crw & 255u), cr1 = (int)((crw >> 8) & 255u);
+                        dr[p] = __byte_perm(red(cr0), red(cr1), 0x7632); dg[p] = __byte_perm(green(cb0, cr0), green(cb1, cr1), 0x7632);
+                        db[p] = __byte_perm(blue(cb0), blue(cb1), 0x7632);
+                    }
+                }
             }
-        } else if (NC == 1) {
+            uint32_t w[6];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) px[3 * e] = px[3 * e + 1] = px[3 * e + 2] = (int)((yw >> (8 * e)) & 255u);
-        } else if (HS == 1) {
-            // every pixel its own chroma sample of row (row / VS)
-            const uint32_t cbw = *reinterpret_cast<const uint32_t*>(&s_c[0][row / VS][4 * gx]);
-            const uint32_t crw = *reinterpret_cast<const uint32_t*>(&s_c[1][row / VS][4 * gx]);
+            for (int h = 0; h < 2; ++h) {                             // four pixels: RGBR GBRG BRGB
+                uint32_t rg[2], b[2];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int cb = (int)((cbw >> (8 * e)) & 255u) - 128, cr = (int)((crw >> (8 * e)) & 255u) - 128;
-                const int Y = (int)((yw >> (8 * e)) & 255u);
-                px[e * 3 + 0] = Y + ((91881 * cr + 32768) >> 16);
-                px[e * 3 + 1] = Y + ((-22553 * cb - 46802 * cr + 32768) >> 16);
-                px[e * 3 + 2] = Y + ((116130 * cb + 32768) >> 16);
+                for (int e = 0; e < 2; ++e) {
+                    const uint32_t Y = yp[4 * y + 2 * h + e];
+                    if (NC == 1) { rg[e] = __byte_perm(Y, Y, 0x6240); b[e] = Y; }
+                    else {
+                        const uint32_t r2 = __viaddmin_s16x2_relu(Y, dr[2 * h + e], 0x00FF00FFu), g2 = __viaddmin_s16x2_relu(Y, dg[2 * h + e], 0x00FF00FFu);
+                        b[e] = __viaddmin_s16x2_relu(Y, db[2 * h + e], 0x00FF00FFu);
+                        rg[e] = __byte_perm(r2, g2, 0x6240);          // R0 G0 R1 G1
+                    }
+                }
+                w[3 * h] = __byte_perm(rg[0], b[0], 0x2410);          // R0 G0 B0 R1
+                w[3 * h + 1] = __byte_perm(__byte_perm(rg[0], b[0], 0x0063), rg[1], 0x5410);   // G1 B1 R2 G2
+                w[3 * h + 2] = __byte_perm(rg[1], b[1], 0x6324);      // B2 R3 G3 B3
             }
-        } else {
-        const uint32_t cbw = *reinterpret_cast<const uint16_t*>(&s_c[0][row / VS][2 * gx]);
-        const uint32_t crw = *reinterpret_cast<const uint16_t*>(&s_c[1][row / VS][2 * gx]);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int cb = (int)((cbw >> (8 * h)) & 255u) - 128, cr = (int)((crw >> (8 * h)) & 255u) - 128;
-            const int dr = (91881 * cr + 32768) >> 16;
-            const int dg = (-22553 * cb - 46802 * cr + 32768) >> 16;
-            const int db = (116130 * cb + 32768) >> 16;
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int Y = (int)((yw >> (8 * (2 * h + e))) & 255u);
-                px[(2 * h + e) * 3 + 0] = Y + dr;
-                px[(2 * h + e) * 3 + 1] = Y + dg;
-                px[(2 * h + e) * 3 + 2] = Y + db;
-            }
+            uint2* d = reinterpret_cast<uint2*>(s_stage + (8 * yr + y) * kStagePitch + 24 * yc);
+            d[0] = make_uint2(w[0], w[1]); d[1] = make_uint2(w[2], w[3]); d[2] = make_uint2(w[4], w[5]);
         }
-        }
-        uint32_t* d = reinterpret_cast<uint32_t*>(s_stage + row * kStagePitch + 12 * gx);
-        d[0] = pack4_sat(px[0], px[1], px[2], px[3]);
-        d[1] = pack4_sat(px[4], px[5], px[6], px[7]);
-        d[2] = pack4_sat(px[8], px[9], px[10], px[11]);
     }
     __syncthreads();
 
     // ---- store: each staged row is a contiguous byte run of the output
     const int x0 = kPxW * (int)un.mcol0;
     const int npx = min(kPxW * nm, (int)im.W - x0);
-    const int nrows = min(kPxH, (int)im.H - kPxH * (int)un.mrow);
+    const int row0 = kPxH * r_lo;                                     // first staged row that is wanted
+    const int nrows = min(kPxH * r_hi, (int)im.H - kPxH * (int)un.mrow) - row0;
     const int nbytes = 3 * npx;
-    uint8_t* gbase = out + im.out_off + ((uint64_t)(kPxH * un.mrow) * im.W + x0) * 3;
+    const uint8_t* const stage0 = s_stage + row0 * kStagePitch;
+    uint8_t* gbase = out + im.out_off + ((uint64_t)(kPxH * un.mrow + row0) * im.W + x0) * 3;
     const size_t gpitch = (size_t)im.W * 3;
     if (((reinterpret_cast<uintptr_t>(gbase) | gpitch | (uintptr_t)nbytes) & 15u) == 0) {
         // rows start and end on 16-byte boundaries: whole 16-byte vectors
         const int vec = nbytes >> 4;
-        for (int i = tid; i < nrows * vec; i += kPixThreads) {
-            const int row = i / vec, c = i % vec;
-            *reinterpret_cast<uint4*>(gbase + row * gpitch + 16 * c) = *reinterpret_cast<const uint4*>(s_stage + row * kStagePitch + 16 * c);
+        for (int i = tid; i < nrows * 24; i += kT) {                   // (24 vectors in a full row)
+            const int row = i / 24, c = i - 24 * row;
+            if (c < vec) *reinterpret_cast<uint4*>(gbase + row * gpitch + 16 * c) = *reinterpret_cast<const uint4*>(stage0 + row * kStagePitch + 16 * c);
         }
     } else {
         // rows at any byte address.  The 16-byte-aligned chunks of global memory that lie inside a row:
         // five staged words shifted into place, one 16-byte store
         constexpr int kInner = (3 * 128) / 16 - 1;
-        for (int i = tid; i < nrows * kInner; i += kPixThreads) {
+        for (int i = tid; i < nrows * kInner; i += kT) {
             const int row = i / kInner, slot = 1 + (i - row * kInner);
             uint8_t* gp = gbase + row * gpitch;
             const int lead = (int)(reinterpret_cast<uintptr_t>(gp) & 15u);
             if (16 * slot + 16 > lead + nbytes) continue;     // the row's last chunk, or behind it
             const int o0 = 16 * slot - lead;                  // the chunk's first byte, counted from the row's first
-            const uint32_t* q = reinterpret_cast<const uint32_t*>(s_stage + row * kStagePitch) + (o0 >> 2);
+            const uint32_t* q = reinterpret_cast<const uint32_t*>(stage0 + row * kStagePitch) + (o0 >> 2);
             const int sh = 8 * (o0 & 3);
             const uint32_t p0 = q[0], p1 = q[1], p2 = q[2], p3 = q[3], p4 = q[4];   // (the spare bytes keep p4 in bounds)
             *reinterpret_cast<uint4*>(gp + o0) = make_uint4(__funnelshift_r(p0, p1, sh), __funnelshift_r(p1, p2, sh),
@@ -422,7 +430,7 @@ __global__ void __launch_bounds__(kPixThreads, PCR_PIX_MIN_CTAS) pixel_kernel(Pa
             const int nch = (lead + nbytes + 15) >> 4;
             if (!(tid & 1) || nch > 1) {
                 const int o0 = 16 * ((tid & 1) ? nch - 1 : 0) - lead;
-                const uint8_t* srow = s_stage + row * kStagePitch;
+                const uint8_t* srow = stage0 + row * kStagePitch;
                 const uint32_t* sw = reinterpret_cast<const uint32_t*>(srow);
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -442,7 +450,7 @@ __global__ void __launch_bounds__(kPixThreads, PCR_PIX_MIN_CTAS) pixel_kernel(Pa
 // Pixel stage when nothing but DC coefficients has been decoded and every image is a multiple of
 // 16 pixels wide: each 8x8 luminance block is one constant sample, each MCU one chroma pair, so
 // an MCU row of the output is runs of eight equal pixels.  A CTA takes one work unit (8 MCUs of
-// one MCU row): 32 threads turn the unit's 32 luminance blocks into RGB triples (the same
+// two MCU rows): 64 threads turn the unit's luminance blocks into RGB triples (the same
 // arithmetic as the general kernel: the transform collapses to its k = 0 term, samples clamp to
 // 0..255), then every thread writes 16-byte vectors whose bytes are picked from the two triples
 // of the vector's MCU half-row.  48 bytes per MCU row = 3 vectors, so a vector never leaves its MCU.
@@ -452,39 +460,44 @@ __global__ void __launch_bounds__(kPixThreads, PCR_PIX_MIN_CTAS) pixel_kernel(Pa
 // when it lies inside the row, byte by byte at the row's two ends.
 template <bool kRoi, bool kAligned = true>
 __global__ void __launch_bounds__(128) dc_pixel_kernel(Params P, uint8_t* __restrict__ out) {
-    __shared__ uint32_t s_tri[2][2 * kPixMcus];        // [block row of the MCU row][block column]: R | G << 8 | B << 16
+    constexpr int U = Sampling<kSamp420>::U, R = Sampling<kSamp420>::R;
+    __shared__ uint32_t s_tri[2 * R][2 * U];           // [block row of the unit][block column]: R | G << 8 | B << 16
     const int tid = threadIdx.x;
     const Unit un = P.units[blockIdx.x];
     const ImgDesc im = P.imgs[un.img];
-    const int nm = min((int)kPixMcus, (int)im.mx - (int)un.mcol0);
+    const int nm = min(U, (int)im.mx - (int)un.mcol0);
+    int r_lo = 0, r_hi = min(R, (int)im.my - (int)un.mrow);
     if (kRoi) {
         const CropRect r = P.roi[un.img];
-        const uint32_t ux0 = 16u * un.mcol0, uy0 = 16u * un.mrow;
-        if (ux0 >= r.x0 + r.w || ux0 + 16u * (uint32_t)nm <= r.x0 || uy0 >= r.y0 + r.h || uy0 + 16u <= r.y0) return;
+        const int ux0 = 16 * un.mcol0;
+        r_lo = max(r_lo, (int)(r.y0 / 16u) - (int)un.mrow); r_hi = min(r_hi, (int)((r.y0 + r.h - 1u) / 16u) + 1 - (int)un.mrow);
+        if (r_lo >= r_hi || ux0 >= (int)(r.x0 + r.w) || ux0 + 16 * nm <= (int)r.x0) return;
     }
-    if (tid < 4 * nm) {
+    {
         constexpr uint32_t K4 = 5793;
-        const int brow = tid / (2 * nm), bcol = tid % (2 * nm);
-        const uint16_t* q = P.qtab + (size_t)un.img * 192;
-        auto sample = [&](uint64_t blk, int comp) {
-            const int F = (int)P.head[blk * 8] * (int)q[64 * comp];
-            const int T = (int)(K4 * (uint32_t)F + (1u << 11)) >> 12;
-            const int smp = ((int)(K4 * (uint32_t)T + (1u << 15)) >> 16) + 128;
-            return min(max(smp, 0), 255);
-        };
-        const uint64_t mcus = (uint64_t)im.mx * im.my;
-        const uint64_t yb = im.blk_base + (uint64_t)(2 * un.mrow + brow) * (2 * im.mx) + 2 * un.mcol0 + bcol;
-        const uint64_t cbk = im.blk_base + 4 * mcus + (uint64_t)un.mrow * im.mx + un.mcol0 + (bcol >> 1);
-        const int Y = sample(yb, 0), cb = sample(cbk, 1) - 128, cr = sample(cbk + mcus, 2) - 128;
-        const int R = Y + ((91881 * cr + 32768) >> 16);
-        const int G = Y + ((-22553 * cb - 46802 * cr + 32768) >> 16);
-        const int B = Y + ((116130 * cb + 32768) >> 16);
-        s_tri[brow][bcol] = (uint32_t)min(max(R, 0), 255) | ((uint32_t)min(max(G, 0), 255) << 8) | ((uint32_t)min(max(B, 0), 255) << 16);
+        const int brow = tid / (2 * U), bcol = tid % (2 * U);
+        if (brow >= 2 * r_lo && brow < 2 * r_hi && bcol < 2 * nm) {
+            const uint16_t* q = P.qtab + (size_t)un.img * 192;
+            auto sample = [&](uint64_t blk, int comp) {
+                const int F = (int)__ldg(P.dc + blk) * (int)q[64 * comp];
+                const int T = (int)(K4 * (uint32_t)F + (1u << 11)) >> 12;
+                const int smp = ((int)(K4 * (uint32_t)T + (1u << 15)) >> 16) + 128;
+                return min(max(smp, 0), 255);
+            };
+            const uint64_t mcus = (uint64_t)im.mx * im.my;
+            const uint64_t yb = im.blk_base + (uint64_t)(2 * un.mrow + brow) * (2 * im.mx) + 2 * un.mcol0 + bcol;
+            const uint64_t cbk = im.blk_base + 4 * mcus + (uint64_t)(un.mrow + (brow >> 1)) * im.mx + un.mcol0 + (bcol >> 1);
+            const int Y = sample(yb, 0), cb = sample(cbk, 1) - 128, cr = sample(cbk + mcus, 2) - 128;
+            const int Rv = Y + ((91881 * cr + 32768) >> 16);
+            const int G = Y + ((-22553 * cb - 46802 * cr + 32768) >> 16);
+            const int B = Y + ((116130 * cb + 32768) >> 16);
+            s_tri[brow][bcol] = (uint32_t)min(max(Rv, 0), 255) | ((uint32_t)min(max(G, 0), 255) << 8) | ((uint32_t)min(max(B, 0), 255) << 16);
+        }
     }
     __syncthreads();
-    const int nrows = min(16, (int)im.H - 16 * (int)un.mrow);
+    const int row0 = 16 * r_lo, nrows = min(16 * r_hi, (int)im.H - 16 * (int)un.mrow) - row0;
     const size_t gpitch = (size_t)im.W * 3;
-    uint8_t* gbase = out + im.out_off + ((uint64_t)(16 * un.mrow) * im.W + 16 * (uint64_t)un.mcol0) * 3;
+    uint8_t* gbase = out + im.out_off + ((uint64_t)(16 * un.mrow + row0) * im.W + 16 * (uint64_t)un.mcol0) * 3;
     if (!kAligned) {
         const int len = 3 * min(16 * nm, (int)im.W - 16 * (int)un.mcol0);      // bytes of the unit in one output row
         // the four bytes at offset o of a row (o may lie up to 15 bytes before the row or behind its end:
@@ -498,9 +511,9 @@ __global__ void __launch_bounds__(128) dc_pixel_kernel(Params P, uint8_t* __rest
         };
         // the bytes of one output row of the unit, once per block row (the eight pixel rows of a block row are
         // equal), with 16 bytes of margin on either side so that a chunk may begin before the row or end behind it
-        constexpr int kPatWords = (16 + 3 * 16 * kPixMcus + 16) / 4;
-        __shared__ __align__(16) uint32_t s_pat[2][kPatWords];
-        for (int i = tid; i < 2 * kPatWords; i += 128) {
+        constexpr int kPatWords = (16 + 3 * 16 * U + 16) / 4;
+        __shared__ __align__(16) uint32_t s_pat[2 * R][kPatWords];
+        for (int i = tid; i < 2 * R * kPatWords; i += 128) {
             const int br = i / kPatWords, wi = i - br * kPatWords;
             s_pat[br][wi] = word_at(s_tri[br], 4 * wi - 16);
         }
@@ -513,14 +526,14 @@ __global__ void __launch_bounds__(128) dc_pixel_kernel(Params P, uint8_t* __rest
             return make_uint4(__funnelshift_r(p0, p1, a), __funnelshift_r(p1, p2, a), __funnelshift_r(p2, p3, a), __funnelshift_r(p3, p4, a));
         };
         // chunks that lie inside the row: whole 16-byte stores
-        constexpr int kInner = (3 * 16 * kPixMcus) / 16 - 1;
+        constexpr int kInner = (3 * 16 * U) / 16 - 1;
         for (int i = tid; i < nrows * kInner; i += 128) {
             const int row = i / kInner, slot = 1 + (i - row * kInner);
             uint8_t* g = gbase + row * gpitch;                                  // first byte of the row
             const int lead = (int)(reinterpret_cast<uintptr_t>(g) & 15u);
             if (16 * slot + 16 > lead + len) continue;                          // the row's last chunk, or behind it
             const int o0 = 16 * slot - lead;                                    // the chunk's first byte, counted from g
-            *reinterpret_cast<uint4*>(g + o0) = chunk_at(s_pat[row >> 3], o0);
+            *reinterpret_cast<uint4*>(g + o0) = chunk_at(s_pat[(row0 + row) >> 3], o0);
         }
         // the first and the last chunk of every row: whole words where they lie inside, else bytes
         if (tid < 2 * nrows) {
@@ -531,7 +544,7 @@ __global__ void __launch_bounds__(128) dc_pixel_kernel(Params P, uint8_t* __rest
             const int slot = (tid & 1) ? nch - 1 : 0;
             if (!(tid & 1) || nch > 1) {
                 const int o0 = 16 * slot - lead;
-                const uint4 v = chunk_at(s_pat[row >> 3], o0);
+                const uint4 v = chunk_at(s_pat[(row0 + row) >> 3], o0);
                 const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -549,9 +562,10 @@ __global__ void __launch_bounds__(128) dc_pixel_kernel(Params P, uint8_t* __rest
         return;
     }
     const int vec = 3 * nm;                                 // 16-byte vectors per output row of this unit
-    for (int i = tid; i < nrows * vec; i += 128) {
-        const int row = i / vec, v = i - row * vec, mcu = v / 3, kk = v - 3 * mcu;
-        const uint32_t A = s_tri[row >> 3][2 * mcu], Bt = s_tri[row >> 3][2 * mcu + 1];
+    for (int i = tid; i < nrows * 3 * U; i += 128) {        // (as if the unit were full: the division is by a constant)
+        const int row = i / (3 * U), v = i - row * (3 * U), mcu = v / 3, kk = v - 3 * mcu, br = (row0 + row) >> 3;
+        if (v >= vec) continue;
+        const uint32_t A = s_tri[br][2 * mcu], Bt = s_tri[br][2 * mcu + 1];
         // four-byte words of a run of equal pixels repeat with period three: RGBR GBRG BRGB
         const uint32_t aw0 = __byte_perm(A, 0, 0x0210), aw1 = __byte_perm(A, 0, 0x1021), aw2 = __byte_perm(A, 0, 0x2102);
         const uint32_t bw0 = __byte_perm(Bt, 0, 0x0210), bw1 = __byte_perm(Bt, 0, 0x1021), bw2 = __byte_perm(Bt, 0, 0x2102);
@@ -653,12 +667,6 @@ __global__ void __launch_bounds__(256) tensor_kernel(Params P, TensorArgs T, con
             tensor_store(o + 2 * plane, ((by * tb + ay * hb) * k255 - m2) * i2);
         }
     }
-}
-
-// Copies the head plane into positions 0..7 of every block (for readers of the full planes).
-__global__ void __launch_bounds__(256) merge_head_kernel(Params P, uint64_t n_blocks) {
-    const uint64_t b = (uint64_t)blockIdx.x * 256 + threadIdx.x;
-    if (b < n_blocks) *reinterpret_cast<uint4*>(P.planes + b * 64) = *reinterpret_cast<const uint4*>(P.head + b * 8);
 }
 
 }  // namespace pcr

@@ -1,6 +1,7 @@
 // Structures shared by the host side and the kernels of the PCR decoder.
 #pragma once
 #include <stdint.h>
+#include <vector_types.h>
 
 namespace pcr {
 
@@ -13,28 +14,39 @@ struct ScanScript {
 
 // Where an AC scan keeps its per-block side data in the auxiliary array (units of uint64,
 // indexed by the block's number inside its component across the whole record):
-//  - a first-pass AC scan writes one word per block: the mask of zigzag positions it made non-zero;
+//  - a first-pass AC scan writes the mask of zigzag positions it made non-zero and, if its band reaches beyond
+//    position 7, a second word: where the block's values for those positions begin in the value array;
 //  - an AC refinement scan writes four words per block: {mask of non-zero positions of its band
 //    after the scan, correction bits in reading order (last bit at bit 0), mask of newly
-//    non-zero positions, mask of those that are positive}.  The coefficient planes are updated
-//    from these by the pixel kernel.
+//    non-zero positions, mask of those that are positive}.  The pixel kernel applies them to a block
+//    when it expands it.
+//  - a sequential scan writes what a first pass over 1..63 would (component c from base + base_c[c - 1] on).
 // A refinement scan finds the positions that were non-zero before it by OR-ing the masks of up
 // to four earlier scans (src), each read with its own stride.
 struct ScanAux {
     uint64_t base;        // first word of this scan's side data
-    uint32_t stride;      // words per block: 1 or 4
+    uint64_t base_c[2];   // sequential scans: the chroma components' first words
+    uint32_t stride;      // words per block: 1 or 2 (first passes), 4 (refinements)
     int32_t nsrc;
     int32_t src[4];       // scan indices
     uint32_t tab0;        // first of the scan's lookup tables (see ScanTab): image i has ntab of them from tab0 + i * ntab on
     int32_t ntab;         // 2 for a DC first pass, 1 for an AC scan, 4 for a sequential scan, 0 for a DC refinement
 };
 
-// Refinement scans to apply per component, in scan order (built per decode for the chosen k).
-struct FinalizeList {
+// Where the coefficients of the decoded scans lie, per component (built per call for the chosen k).
+constexpr int kMaxFirst = 56;      // first passes of a component that reach beyond position 7: at most one per position
+struct CoefLists {
+    uint4 head_mask[3];            // positions 1..7 that a decoded scan covers, as 16-bit lanes of the head plane's entries
+    int32_t n_first[3], n_refine[3];
+    uint64_t first[3][kMaxFirst];  // first word of the scan's side data (two words per block)
+    uint64_t refine[3][4];         // the refinement scans in scan order: first word of the side data (four words per block)
+    int32_t p1[3][4];              // 1 << Al of the scan
+};
+
+// The AC refinements one call decodes, per component in scan order (for the chain launch).
+struct RefineList {
     int32_t n[3];
     int32_t scan[3][4];
-    int32_t p1[3][4];      // 1 << Al of the scan
-    uint64_t base[3][4];   // first word of the scan's side data
 };
 
 // One (scan, image) pair: where its entropy-coded bytes and Huffman tables live.
@@ -89,12 +101,17 @@ struct ScanTab;             // lookup table of one Huffman table (pcr_entropy.cu
 struct Params {
     const uint8_t* rec;         // record bytes on the device
     uint8_t* ubuf;              // entropy-coded bytes without stuffing, big-endian words
-    int16_t* planes;            // coefficient planes, 64 int16 per block, zigzag order
-    int16_t* head;              // zigzag positions 0..7 of every block, dense (8 int16 = 16 bytes per
-                                // block, same block numbering).  First passes store these positions
-                                // here and only positions 8..63 in the 128-byte line: the dense
-                                // plane stays in L2 while it is written, instead of one cold
-                                // 128-byte line being read and written back per coefficient
+    int16_t* planes;            // coefficient planes, 64 int16 per block, zigzag order: only written when somebody asks
+                                // for them (pcr_coeffs); the decode itself keeps coefficients as
+    int16_t* dc;                //  - the DC coefficient of every block, dense (same block numbering),
+    int16_t* head;              //  - zigzag positions 1..7 of every block, dense (8 int16 = 16 bytes per block, the first
+                                //    one unused),
+    int16_t* vals;              //  - the non-zero values of positions 8..63, block after block in reading order; their
+                                //    positions are the masks of the scan's side data.  A coefficient takes at least two
+                                //    bits of the stream, so the values of whatever begins at byte b of the
+                                //    unstuffed copy begin at index 4 b and nothing overlaps.
+                                // Every decode of a record writes the same values to the same places, so none of this is
+                                // cleared between decodes
     const ScanScript* script;   // [G]
     const ScanAux* saux;        // [G]
     uint64_t* aux;              // side data of the AC scans
