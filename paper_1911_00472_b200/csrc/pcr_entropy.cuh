@@ -202,10 +202,32 @@ __device__ __forceinline__ void tables_warp(const Params& P, const ScanList& sl,
 // removed, bytes of each aligned group of four stored in reverse (big-endian words), at the
 // same start offset as in the record.  Records, in offsets of that copy, the first byte of every
 // restart interval (the byte after each RSTn marker) plus one final entry = end of data + 2, so
-// interval j spans [seg[j], seg[j+1] - 2).  Lanes take 16-byte slices; positions come from a
-// warp prefix sum of the bytes each slice keeps.
-// ---------------------------------------------------------------------------------------
+// interval j spans [seg[j], seg[j+1] - 2).
+// Tile by tile of 512 bytes, lanes take 16-byte slices.  Stuffed zeros and markers are found four bytes at
+// a time; one warp prefix sum places the slices; a lane writes the output words that begin in its slice,
+// taking up to three bytes of the last one from its neighbour, so nothing goes through shared memory.  (The
+// byte-by-byte form with a staging row took 680 warp instructions a tile, this one about 200; bound by the
+// latency of one warp's tiles, up to 50 for a baseline JPEG of 25 KB.)
 // Blocks from index_blocks on build the lookup tables of the same scans and images (one warp per table).
+// ---------------------------------------------------------------------------------------
+
+// bit 7 of every byte that is zero
+__device__ __forceinline__ uint32_t zero_bytes(uint32_t x) { return ~(((x & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | x) & 0x80808080u; }
+// the bit 7s of four words' bytes as a 16-bit mask
+__device__ __forceinline__ uint32_t byte_mask(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    constexpr uint32_t k = 0x00204081u;
+    return ((a * k) >> 28) | (((b * k) >> 28) << 4) | (((c * k) >> 28) << 8) | (((d * k) >> 28) << 12);
+}
+// removes byte i (0..15) of the sixteen in k[0..3] (later bytes move down)
+__device__ __forceinline__ void drop_byte(uint32_t (&k)[4], uint32_t i) {
+#pragma unroll
+    for (uint32_t w = 0; w < 4; ++w) {
+        const uint32_t moved = __funnelshift_r(k[w], w < 3 ? k[w + 1] : 0u, 8);
+        const uint32_t m = i < 4u * w ? 0u : (i >= 4u * w + 4u ? 0xFFFFFFFFu : (1u << (8u * (i & 3u))) - 1u);   // bytes that stay
+        k[w] = (k[w] & m) | (moved & ~m);
+    }
+}
+
 __global__ void __launch_bounds__(256) unstuff_index_kernel(Params P, ScanList sl, int img0, int nimg, uint32_t index_blocks) {
     const int lane = threadIdx.x & 31;
     if (blockIdx.x >= index_blocks) {
@@ -215,102 +237,116 @@ __global__ void __launch_bounds__(256) unstuff_index_kernel(Params P, ScanList s
         if (w < 4u * (uint32_t)(sl.n * nimg)) tables_warp(P, sl, img0, nimg, w, lane, s_code[threadIdx.x >> 5], s_vals[threadIdx.x >> 5]);
         return;
     }
+    const unsigned full = 0xffffffffu;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (warp >= sl.n * nimg) return;
     const int img = (int)P.order[img0 + warp % nimg];      // img0, nimg: a run of the processing order
-    const ScanDesc sd = P.scans[sl.s[warp / nimg] * P.N + img];
+    const ScanDesc& sd = P.scans[sl.s[warp / nimg] * P.N + img];
+    const uint32_t a = sd.data_off, b = sd.data_end, nseg = sd.nseg;
     uint32_t* seg = P.seg_start + sd.seg_base;
-    const uint32_t a = sd.data_off, b = sd.data_end;
+    uint32_t* out = reinterpret_cast<uint32_t*>(P.ubuf);
     if (lane == 0) seg[0] = a;
-    uint32_t found = 0;      // markers seen so far (warp uniform)
-    uint32_t kept = 0;       // bytes written so far (warp uniform)
-    // the next tile's 16 bytes are loaded while the current tile is processed; the byte before
-    // and the byte after a lane's slice come from its neighbours by shuffle
+    uint32_t found = 0, kept = 0;            // markers seen, bytes written so far (warp uniform)
+    uint32_t held = 0, nheld = a & 3u;       // the bytes of an output word that the previous tile left incomplete (at first: that precede the data)
+    uint32_t before = 0;                     // last byte of the previous tile, in the top byte
     const uint4 zero4 = make_uint4(0, 0, 0, 0);
-    uint4 ahead = zero4;
+    uint4 ahead = zero4;                     // the next tile is loaded while this one is worked on
     {
         const uint32_t p = (a & ~15u) + 16u * lane;
         if (p < b) ahead = __ldg(reinterpret_cast<const uint4*>(P.rec + p));   // chunks are padded to 16 bytes
     }
-    uint32_t carry = 0;      // last byte of the previous tile
-    __shared__ __align__(16) uint8_t s_stage[8][528];
-    uint8_t* stage = s_stage[threadIdx.x >> 5];
-    uint32_t* out32 = reinterpret_cast<uint32_t*>(P.ubuf);
-    uint32_t gpos = a & ~3u;                 // position in the copy of stage[0]
-    uint32_t pend = a & 3u;                  // bytes already staged in front of the next tile's
-    if (lane < 4) stage[lane] = 0;
-    __syncwarp();
     for (uint32_t p0 = a & ~15u; p0 < b; p0 += 512) {
         const uint32_t p = p0 + 16u * lane;
         const uint4 v = ahead;
         ahead = zero4;
         if (p + 512 < b) ahead = __ldg(reinterpret_cast<const uint4*>(P.rec + p + 512));
-        const uint32_t first_next_tile = __shfl_sync(0xffffffffu, ahead.x & 255u, 0);
-        uint32_t nxt = __shfl_down_sync(0xffffffffu, v.x & 255u, 1);
-        if (lane == 31) nxt = first_next_tile;
-        uint32_t prev = __shfl_up_sync(0xffffffffu, v.w >> 24, 1);
-        if (lane == 0) prev = carry;
-        carry = __shfl_sync(0xffffffffu, v.w >> 24, 31);
-        const uint32_t w[5] = {v.x, v.y, v.z, v.w, nxt};
-        uint32_t keep = 0, mark = 0;
+        const bool last_tile = p0 + 512 >= b;
+        uint32_t prev = __shfl_up_sync(full, v.w, 1), next = __shfl_down_sync(full, v.x, 1);
+        const uint32_t next_tile = __shfl_sync(full, ahead.x, 0);
+        if (lane == 0) prev = before;
+        if (lane == 31) next = next_tile;
+        before = __shfl_sync(full, v.w, 31);
+        // the bytes of [a, b) among the slice's sixteen
+        uint32_t range = 0xFFFFu;
+        if (p < a) { range &= 0xFFFFu << (a - p); if (lane == 0) prev = 0; }    // (only the first slice; nothing precedes the data)
+        if (p + 16u > b) range &= p < b ? (1u << (b - p)) - 1u : 0u;
+        uint32_t k[4] = {v.x, v.y, v.z, v.w};
+        uint32_t ff[4], rst[5];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            const uint32_t c0 = (w[j >> 2] >> (8 * (j & 3))) & 255u;
-            const uint32_t c1 = (w[(j + 1) >> 2] >> (8 * ((j + 1) & 3))) & 255u;
-            const uint32_t cp = j ? (w[(j - 1) >> 2] >> (8 * ((j - 1) & 3))) & 255u : prev;
-            const uint32_t q = p + j;
-            const bool in = q >= a && q < b;
-            if (in && !(c0 == 0u && cp == 0xFFu && q > a)) keep |= 1u << j;
-            if (in && q + 1 < b && c0 == 0xFFu && (c1 & 0xF8u) == 0xD0u) mark |= 1u << j;
+        for (int i = 0; i < 4; ++i) {
+            ff[i] = zero_bytes(~k[i]);
+            rst[i] = zero_bytes((k[i] ^ 0xD0D0D0D0u) & 0xF8F8F8F8u);
         }
-        // exclusive prefix sums over lanes of kept bytes and of markers
-        uint32_t kc = __popc(keep), mc = __popc(mark), kin = kc, min_ = mc;
+        rst[4] = zero_bytes((next ^ 0xD0D0D0D0u) & 0xF8F8F8F8u);
+        const uint32_t pff = zero_bytes(~prev);
+        uint32_t drop = byte_mask(zero_bytes(k[0]) & __funnelshift_l(pff, ff[0], 8), zero_bytes(k[1]) & __funnelshift_l(ff[0], ff[1], 8),
+                                  zero_bytes(k[2]) & __funnelshift_l(ff[1], ff[2], 8), zero_bytes(k[3]) & __funnelshift_l(ff[2], ff[3], 8));
+        uint32_t mark = byte_mask(ff[0] & __funnelshift_r(rst[0], rst[1], 8), ff[1] & __funnelshift_r(rst[1], rst[2], 8),
+                                  ff[2] & __funnelshift_r(rst[2], rst[3], 8), ff[3] & __funnelshift_r(rst[3], rst[4], 8));
+        // a zero in front of the data's first byte does not count; a marker's second byte has to lie inside the data
+        if (p < a) drop &= ~(1u << (a - p));
+        mark &= range & (p + 16u >= b ? range >> 1 : 0xFFFFu);
+        const uint32_t keep = range & ~drop, c = (uint32_t)__popc(keep);
+        uint32_t sum = c | ((uint32_t)__popc(mark) << 16);
+        const uint32_t own = sum;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
-            const uint32_t ok = __shfl_up_sync(0xffffffffu, kin, d), om = __shfl_up_sync(0xffffffffu, min_, d);
-            if (lane >= d) { kin += ok; min_ += om; }
+            const uint32_t o = __shfl_up_sync(full, sum, d);
+            if (lane >= d) sum += o;
         }
-        // kept bytes go to the warp's staging row (after the bytes left over from the last tile),
-        // from there to the copy as whole byte-reversed words
-        const uint32_t obase = a + kept + kin - kc;
-        const uint32_t sbase = pend + kin - kc;
-        uint32_t ord = found + min_ - mc;
+        const uint32_t tile = __shfl_sync(full, sum, 31);
+        const uint32_t o = a + kept + ((sum - own) & 0xFFFFu);       // where the slice's first kept byte goes
+        uint32_t ord = found + ((sum - own) >> 16);
+        while (mark) {
+            const uint32_t i = (uint32_t)__ffs((int)mark) - 1u;
+            mark &= mark - 1u;
+            ++ord;
+            if (ord < nseg) seg[ord] = o + (uint32_t)__popc(keep & ((1u << i) - 1u)) + 2u;
+        }
+        // the kept bytes to the front
+        if (p < a) {                                                 // bytes in front of the data
+            const uint32_t n = a - p;
+            if (n & 8u) { k[0] = k[2]; k[1] = k[3]; }
+            if (n & 4u) { k[0] = k[1]; k[1] = k[2]; k[2] = k[3]; }
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            if ((keep >> j) & 1u) {
-                const uint32_t off = __popc(keep & ((1u << j) - 1u));
-                stage[sbase + off] = (uint8_t)((w[j >> 2] >> (8 * (j & 3))) & 255u);
-                if ((mark >> j) & 1u) {
-                    ++ord;
-                    if (ord < sd.nseg) seg[ord] = obase + off + 2;
-                }
-            }
+            for (int i = 0; i < 4; ++i) k[i] = __funnelshift_r(k[i], i < 3 ? k[i + 1] : 0u, 8u * (n & 3u));
+            drop >>= n;
         }
-        const uint32_t tile_kept = __shfl_sync(0xffffffffu, kin, 31);
-        __syncwarp();
-        const uint32_t total = pend + tile_kept, nwords = total >> 2;
-        for (uint32_t i = lane; i < nwords; i += 32)
-            out32[(gpos >> 2) + i] = __byte_perm(reinterpret_cast<const uint32_t*>(stage)[i], 0, 0x0123);
-        __syncwarp();
-        const uint32_t left = total & 3u;
-        uint32_t lb = 0;
-        if (lane < left) lb = stage[4 * nwords + lane];
-        __syncwarp();
-        if (lane < left) stage[lane] = (uint8_t)lb;
-        __syncwarp();
-        gpos += 4 * nwords;
-        pend = left;
-        kept += tile_kept;
-        found += __shfl_sync(0xffffffffu, min_, 31);
-    }
-    if (pend && lane == 0) {                // the last, incomplete word (zero padded)
-        uint32_t wlast = 0;
-        for (uint32_t i = 0; i < pend; ++i) wlast |= (uint32_t)stage[i] << (8 * i);
-        out32[gpos >> 2] = __byte_perm(wlast, 0, 0x0123);
+        for (uint32_t m = drop & 0xFFFFu, n = 0; m; ++n) {
+            const uint32_t i = (uint32_t)__ffs((int)m) - 1u;
+            m &= m - 1u;
+            drop_byte(k, i - n);
+        }
+        // and the neighbour's first bytes behind them (a slice that ends the data has none; what lies there is never decoded)
+        const uint32_t follow = __shfl_down_sync(full, k[0], 1);
+        uint32_t k4 = follow;
+        if (c < 16u) {
+            const uint32_t sh = 8u * (c & 3u), lo = follow << sh, hi = sh ? follow >> (32u - sh) : 0u, m = (1u << sh) - 1u;
+#pragma unroll
+            for (uint32_t w = 0; w < 4; ++w) k[w] = (c >> 2) == w ? (k[w] & m) | lo : (c >> 2) + 1u == w ? hi : k[w];
+            k4 = hi;
+        }
+        // output words that begin in [o, o + c); one that the tile's end cuts off is held back for the next tile
+        const uint32_t s = (0u - o) & 3u, w0 = (o + 3u) >> 2, end = o + c;
+        const bool cut = lane == 31 && !last_tile && (end & 3u) != 0;
+        const uint32_t w1 = cut ? end >> 2 : (end + 3u) >> 2;
+        uint32_t word = 0;
+#pragma unroll
+        for (uint32_t j = 0; j < 4; ++j) {
+            const uint32_t x = __funnelshift_r(k[j], j < 3 ? k[j + 1] : k4, 8u * s);
+            if (w0 + j < w1) out[w0 + j] = __byte_perm(x, 0, 0x0123);
+            if (w0 + j == w1) word = x;
+        }
+        if (lane == 0 && nheld) out[(o - nheld) >> 2] = __byte_perm(held | (k[0] << (8u * nheld)), 0, 0x0123);
+        const uint32_t q = __shfl_sync(full, cut ? end & 3u : 0u, 31);
+        held = __shfl_sync(full, word, 31) & ((1u << (8u * q)) - 1u);
+        nheld = q;
+        kept += tile & 0xFFFFu;
+        found += tile >> 16;
     }
     if (lane == 0) {
-        seg[sd.nseg] = a + kept + 2;
-        if (found != sd.nseg - 1) atomicMin(&P.status[img], kErrCorrupt);
+        seg[nseg] = a + kept + 2;
+        if (found != nseg - 1) atomicMin(&P.status[img], kErrCorrupt);
     }
 }
 
@@ -377,6 +413,13 @@ __device__ __forceinline__ uint32_t shr0(uint32_t x, uint32_t n) { uint32_t y; a
 // byte permutation with the selector's sign form (__byte_perm masks it out)
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t s) { uint32_t y; asm("prmt.b32 %0, %1, %2, %3;" : "=r"(y) : "r"(a), "r"(b), "r"(s)); return y; }
 
+// keeps a pointer in registers (instead of being put together from the kernel's parameters at every use)
+template <class T> __device__ __forceinline__ void pin(T*& p) {
+    size_t a = __cvta_generic_to_global(p);
+    asm volatile("" : "+l"(a));
+    p = static_cast<T*>(__cvta_global_to_generic(a));
+}
+
 struct LaneBits {
     uint32_t col;          // shared address of this lane's column: row r at col + 128 r
     const uint4* g4;       // the 16-byte group that position 0 lies in
@@ -389,31 +432,28 @@ struct LaneBits {
         pos = 8u * (bstart & 15u);
         limit = pos + 8u * (bend - bstart);
         wr = 0;
+        request();
     }
     __device__ __forceinline__ void put(uint32_t w, const uint4& v) {
         const uint32_t p = col + (w & (kRingWords - 1)) * 128u;
         sts32(p, v.x); sts32(p + 128u, v.y); sts32(p + 256u, v.z); sts32(p + 384u, v.w);
         if ((w & (kRingWords - 1)) == 0) sts32(p + kRingWords * 128u, v.x);
     }
-    // top-up in two halves (all lanes of the warp together), so that other loads can be requested between them
-    __device__ __forceinline__ int request(bool on, uint4 (&v)[4]) {
-        const int room = on ? (int)(kRingWords - (wr - (pos >> 5))) >> 2 : 0;
+    // Top-up (all lanes of the warp together): what the next one will store first is requested right after
+    // the previous one, so that its latency passes beside the decode steps.
+    uint4 va, vb;
+    __device__ __forceinline__ void request() {
         const uint4* g = g4 + (wr >> 2);
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            if (room > q) v[q] = __ldg(g + q);
-        return room;
-    }
-    __device__ __forceinline__ void store(int room, const uint4 (&v)[4]) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            if (room > q) put(wr + 4 * q, v[q]);
-        wr += 4u * (uint32_t)min(max(room, 0), 4);
+        va = __ldg(g); vb = __ldg(g + 1);
     }
     __device__ __forceinline__ void topup(bool on) {
-        uint4 v[4];
-        const int room = request(on, v);
-        store(room, v);
+        const uint32_t room = on ? (kRingWords - (wr - (pos >> 5))) >> 2 : 0u;
+        if (room > 0) put(wr, va);
+        if (room > 1) put(wr + 4, vb);
+        if (room > 2) put(wr + 8, __ldg(g4 + (wr >> 2) + 2));
+        if (room > 3) put(wr + 12, __ldg(g4 + (wr >> 2) + 3));
+        wr += 4u * room;
+        if (on) request();
     }
     // steps may begin below this position: `words` words from the one the position lies in are in the ring
     __device__ __forceinline__ uint32_t ring_stop(uint32_t words) const { return 32u * (wr - min(wr, words - 1u)); }
@@ -572,7 +612,8 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, u
         // block numbers inside the image: the MCU's first luminance block (or the scan's own component) and its chroma blocks
         const uint32_t hs = inter ? (uint32_t)P.hs : 1u, vs = inter ? (uint32_t)P.vs : 1u, bw0 = g.bw[inter ? 0 : c0];
         const uint32_t y_off = inter ? 0u : (uint32_t)(g.coff[c0] - im.blk_base), c_off = (uint32_t)(g.coff[1] - im.blk_base), c_step = g.mx * g.my;
-        int16_t* const dcp = P.dc + im.blk_base;
+        int16_t* dcp = P.dc + im.blk_base;
+        pin(dcp);
         for (;;) {
             br.topup(!done);
             __syncwarp(full);
@@ -622,6 +663,7 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, u
             // ---- AC first pass: one Huffman symbol per step
             uint64_t* auxp = P.aux + ax.base + g.loff[c] * ax.stride;
             int16_t* headp = P.head + g.coff[c] * 8;
+            pin(auxp); pin(headp);
             const bool lists = ax.stride == 2u;            // the band reaches beyond position 7
             int16_t* vp = P.vals + 4ull * bstart;           // next value
             int16_t* vb = vp;                               // the block's first one
@@ -641,12 +683,13 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, u
                         const uint32_t skip = e & 31u, sz = (e >> 5) & 15u, r = (e >> 9) & 15u;
                         br.pos += skip;
                         k += r;                                            // position of the coefficient
-                        if (sz && k <= Se) {
-                            const int16_t val = (int16_t)(magnitude(win, skip, sz) << Al);
-                            if (k < 8u) headp[(uint64_t)bi * 8 + k] = val;
-                            else *vp++ = val;
-                            M0 |= shl0(1u, k); M1 |= shl0(1u, k - 32u);
-                        } else if (e == 0 || sz) { bad = true; stop = 0; k = 0; }   // no such symbol, or a coefficient behind the band
+                        const bool coef = sz && k <= Se, far = coef && k >= 8u;
+                        const int val = magnitude(win, skip, sz) << Al;
+                        if (coef && !far) headp[8u * (uint64_t)bi + k] = (int16_t)val;
+                        if (far) *vp = (int16_t)val;
+                        vp += far ? 1 : 0;
+                        M0 |= shl0(coef ? 1u : 0u, k); M1 |= shl0(coef ? 1u : 0u, k - 32u);
+                        if (e == 0 || (sz && k > Se)) { bad = true; stop = 0; k = 0; }   // no such symbol, or a coefficient behind the band
                         ++k;                                               // (sixteen zeros: run 15 plus one)
                         const bool is_eob = (e & kEntEob) != 0;
                         if (is_eob || k > Se) {
@@ -690,6 +733,7 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, u
             }
             const bool two = ax.nsrc > 1, more = ax.nsrc > 2;
             uint64_t* outp = P.aux + ax.base + g.loff[c] * 4ull;
+            pin(outp);
             const uint32_t queue = mem + kWarpQueue + 16u * lane;       // block m at queue + 512 (m % kMaskQueue)
             uint32_t sel = (uint32_t)__cvta_generic_to_shared(s_sel);
             asm volatile("" : "+r"(sel));                              // (kept in a register)
@@ -701,13 +745,9 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, u
             uint32_t s0 = 0, s1 = 0, N0 = 0, N1 = 0, G0 = 0, G1 = 0;   // correction bits, new positions, positive ones
             bool fresh = true;                                         // the block's entry has not been taken from the queue yet
             auto take = [&]() { Z = lds128(queue + ((m & (kMaskQueue - 1)) << 9)); };
-            // what the next top-up will store is requested right after the previous one, so that its latency
-            // passes beside the decode steps
-            uint4 va = make_uint4(0, 0, 0, 0), vb = va;
+            // (the masks are requested ahead like the words of the stream)
             uint64_t ha[4], hb[4];
             auto request = [&]() {
-                const uint4* g = br.g4 + (br.wr >> 2);
-                va = __ldg(g); vb = __ldg(g + 1);
                 uint32_t b = hbi, mm = hm, wm = hwrap_m;
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
@@ -722,12 +762,7 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, u
             };
             if (!done) request();
             for (;;) {
-                const uint32_t room = done ? 0u : (kRingWords - (br.wr - (br.pos >> 5))) >> 2;
-                if (room > 0) br.put(br.wr, va);
-                if (room > 1) br.put(br.wr + 4, vb);
-                if (room > 2) br.put(br.wr + 8, __ldg(br.g4 + (br.wr >> 2) + 2));
-                if (room > 3) br.put(br.wr + 12, __ldg(br.g4 + (br.wr >> 2) + 3));
-                br.wr += 4u * room;
+                br.topup(!done);
                 const uint32_t want = done ? 0u : min((uint32_t)kMaskQueue - (hm - m), m1 - hm);
 #pragma unroll
                 for (int q = 0; q < kMaskQueue; ++q) {
@@ -825,12 +860,15 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, u
 // Sequential (baseline) scans: one interleaved scan carries, block after block, the DC difference
 // and then the AC coefficients up to an end-of-block symbol.  Same decomposition as above (one
 // lane per restart interval, one Huffman symbol per step), four tables per warp (DC and AC,
-// luminance and chrominance).  A block's first symbol goes through the same instructions as the others (its entry
-// has no run, its value is the difference): lanes stand at different kinds of symbol in every step.
-// Coefficients go where the progressive first passes put them.
+// luminance and chrominance).  Lanes stand at different kinds of symbol in every step, so a block's first
+// symbol goes through the same instructions as the others (its entry has no run, its value is the
+// difference), stores are predicated, and what changes from block to block comes from a small table
+// in shared memory.  Coefficients go where the progressive first passes put them.
+// Bound by the length of a lane's chain (a row of 31 MCUs has about 2200 symbols).
 // ---------------------------------------------------------------------------------------
 constexpr int kSeqWarps = 2;
-constexpr uint32_t kSeqWarpBytes = 4 * sizeof(ScanTab) + (kRingWords + 1) * 128;
+constexpr uint32_t kSeqRing = 4 * sizeof(ScanTab), kSeqPlaces = kSeqRing + (kRingWords + 1) * 128, kSeqPreds = kSeqPlaces + 8 * 16;
+constexpr uint32_t kSeqWarpBytes = kSeqPreds + 3 * 128;
 
 template <bool kRoi>
 __global__ void __launch_bounds__(32 * kSeqWarps) sequential_kernel(Params P, uint32_t item_begin, uint32_t item_count) {
@@ -846,8 +884,7 @@ __global__ void __launch_bounds__(32 * kSeqWarps) sequential_kernel(Params P, ui
     uint32_t seg = item.seg0 + lane;
     if (seg >= sd.nseg) { done = true; seg = 0; }
     const ImgDesc im = P.imgs[img];
-    const Geometry g = make_geometry(im, P);
-    const uint32_t mcu_w = g.mx, total = g.mx * g.my;
+    const uint32_t mcu_w = im.mx, total = im.mx * im.my;
     const uint32_t m0 = sd.ri ? seg * sd.ri : 0;
     const uint32_t m1 = sd.ri ? min(m0 + sd.ri, total) : total;
     const unsigned full = 0xffffffffu;
@@ -862,9 +899,22 @@ __global__ void __launch_bounds__(32 * kSeqWarps) sequential_kernel(Params P, ui
         if (__all_sync(full, done)) return;
     }
     const uint32_t mem = (uint32_t)__cvta_generic_to_shared(s_seq) + (uint32_t)wid * kSeqWarpBytes;
+    const uint32_t hs = (uint32_t)P.hs, vs = (uint32_t)P.vs, bw0 = hs * mcu_w;
+    const uint32_t ny = hs * vs, bpm = P.nc == 3 ? ny + 2u : 1u;      // blocks per MCU (a lone component: one block, no padding)
     {
         const uint4* a = reinterpret_cast<const uint4*>(P.tabs + ax.tab0 + 4u * (uint32_t)img);
         for (int i = lane; i < (int)(4 * sizeof(ScanTab) / 16); i += 32) sts128(mem + 16 * i, __ldg(a + i));
+        // per block of the MCU: its two tables (shared addresses), where its predictor lies, its block number
+        // relative to the MCU's first luminance block or to the MCU's chroma place (bit 31)
+        if ((uint32_t)lane < bpm) {
+            const uint32_t j = (uint32_t)lane, c = j < ny ? 0u : j - ny + 1u;
+            const uint32_t tdc = mem + ((sd.slots >> (2u * c)) & 1u) * (uint32_t)sizeof(ScanTab);
+            const uint32_t tac = mem + (2u + ((sd.slots_ac >> (2u * c)) & 1u)) * (uint32_t)sizeof(ScanTab);
+            const uint32_t off = c ? (ny * total + (c - 1u) * total) | 0x80000000u : (j >> (hs - 1u)) * bw0 + (j & (hs - 1u));
+            sts128(mem + kSeqPlaces + 16u * j, make_uint4(tdc, tac, mem + kSeqPreds + 128u * c, off));
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) sts32(mem + kSeqPreds + 128u * c + 4u * lane, 0u);
     }
     const uint32_t* segtab = P.seg_start + sd.seg_base;
     uint32_t bstart = segtab[seg];
@@ -873,27 +923,33 @@ __global__ void __launch_bounds__(32 * kSeqWarps) sequential_kernel(Params P, ui
     if (!done && (bstart < sd.data_off || bend > sd.data_end || bend < bstart)) { bad = true; done = true; }
     if (done) { bstart = sd.data_off; bend = sd.data_off; }
     LaneBits br;
-    br.init(mem + 4u * (uint32_t)sizeof(ScanTab) + 4u * lane, P.ubuf, bstart, bend);
+    br.init(mem + kSeqRing + 4u * lane, P.ubuf, bstart, bend);
     if (m0 >= m1) done = true;
 
-    const uint32_t ny = (uint32_t)(P.hs * P.vs), bpm = P.nc == 3 ? ny + 2u : 1u;      // blocks per MCU (a lone component: one block, no padding)
-    const uint32_t hs = (uint32_t)P.hs, vs = (uint32_t)P.vs, bw0 = g.bw[0], c_off = ny * total;
-    uint32_t m = m0, mrow = m0 / mcu_w, mcol = m0 % mcu_w;
-    uint32_t j = 0, c = 0;                                // block inside the MCU (the luminance blocks, Cb, Cr), its component
-    uint32_t ci = vs * mrow * bw0 + hs * mcol;            // its number inside the image's component
-    uint32_t k = 0, M0 = 0, M1 = 0;                       // position (0: the block's DC symbol comes next), mask
-    int16_t* vp = P.vals + 4ull * bstart;
-    int16_t* vb = vp;
-    int pred0 = 0, pred1 = 0, pred2 = 0;
-    const uint32_t slots = sd.slots, slots_ac = sd.slots_ac;
-    constexpr uint32_t kTab = (uint32_t)sizeof(ScanTab);
-    uint32_t tdc = mem + (slots & 1u) * kTab, tac = mem + (2u + (slots_ac & 1u)) * kTab;
-    int16_t* const dcp = P.dc + im.blk_base;
-    int16_t* const headp = P.head + im.blk_base * 8;
+    uint32_t m = m0, wrap_m = (m0 / mcu_w + 1u) * mcu_w;       // MCU, the first one of the next row
+    uint32_t my = (m0 / mcu_w) * vs * bw0 + hs * (m0 % mcu_w); // block number of the MCU's first luminance block (its chroma place is m)
+    const uint32_t my_wrap = (vs - 1u) * bw0;                  // what a new row adds beside hs per MCU
+    uint32_t place = mem + kSeqPlaces;                         // of the current block in the table
+    const uint32_t place_end = place + 16u * bpm;
+    uint32_t k = 0, M0 = 0, M1 = 0;                            // position (0: the block's DC symbol comes next), mask
+    int16_t* vp = P.vals + 4ull * bstart;                      // next value
+    int16_t* vb = vp;                                          // the block's first one
+    int16_t* dcp = P.dc + im.blk_base;
+    int16_t* headp = P.head + im.blk_base * 8;
+    uint64_t* auxp = P.aux + ax.base + im.blk_base * 2;
+    pin(dcp); pin(headp); pin(auxp);
+    uint32_t tdc = 0, tac = 0, pred = 0, blk = 0;
+    auto take = [&]() {
+        const uint4 v = lds128(place);
+        tdc = v.x; tac = v.y; pred = v.z + 4u * lane;
+        blk = (v.w & 0x7FFFFFFFu) + ((v.w >> 31) ? m : my);
+    };
+    bool fresh = true;
     for (;;) {
         br.topup(!done);
         __syncwarp(full);
         if (__all_sync(full, done)) break;
+        if (fresh) { take(); fresh = false; }
         uint32_t stop = done ? 0u : min(br.ring_stop(2), br.limit + 1u);
 #pragma unroll 1
         for (int t = 0; t < kDecodeSteps; ++t) {
@@ -902,37 +958,34 @@ __global__ void __launch_bounds__(32 * kSeqWarps) sequential_kernel(Params P, ui
                 const bool is_dc = k == 0;
                 const uint32_t tab = is_dc ? tdc : tac;
                 uint32_t e = lds16(tab + ((win >> (32 - kTabBits)) << 1));
-                if (e == 0) e = long_code(tab, win, is_dc ? kTabDc : kTabAcSeq);
+                if (e == 0) {
+                    e = long_code(tab, win, is_dc ? kTabDc : kTabAcSeq);
+                    if (e == 0) { bad = true; stop = 0; }
+                }
                 const uint32_t skip = e & 31u, sz = (e >> 5) & 15u;
                 br.pos += skip;
                 k += (e >> 9) & 15u;
                 int v = magnitude(win, skip, sz);
-                if (is_dc) {
-                    v += c == 0 ? pred0 : (c == 1 ? pred1 : pred2);
-                    if (c == 0) pred0 = v; else if (c == 1) pred1 = v; else pred2 = v;
-                }
-                const bool fail = e == 0 || k > 63u;                       // (sixteen zeros may end behind position 63)
-                const uint32_t blk = (c ? c_off + (c - 1u) * total : 0u) + ci;      // block number inside the image
-                if (!fail && (sz || is_dc)) {
-                    if (k >= 8u) *vp++ = (int16_t)v;
-                    else if (k) headp[(uint64_t)blk * 8 + k] = (int16_t)v;
-                    else dcp[blk] = (int16_t)v;
-                    M0 |= shl0(1u, k); M1 |= shl0(1u, k - 32u);
-                }
-                if (e == 0 || (sz && k > 63u)) { bad = true; stop = 0; k = 0; }
+                if (is_dc) { v += (int)lds32(pred); sts32(pred, (uint32_t)v); }
+                const bool coef = sz && k <= 63u, far = coef && k >= 8u;
+                if (is_dc) dcp[blk] = (int16_t)v;                          // (stored even if there was no such symbol: the image is corrupt then)
+                if (coef && !far && !is_dc) headp[8u * (uint64_t)blk + k] = (int16_t)v;
+                if (far) *vp = (int16_t)v;
+                vp += far ? 1 : 0;
+                M0 |= shl0(far ? 1u : 0u, k); M1 |= shl0(far ? 1u : 0u, k - 32u);
+                if (sz && k > 63u) { bad = true; stop = 0; }
                 ++k;
                 if ((e & kEntEob) || k > 63u) {                            // block finished
-                    if (M1 | (M0 >> 8)) *reinterpret_cast<uint4*>(P.aux + (c ? ax.base_c[c - 1u] : ax.base) + 2ull * ((c ? g.loff[1] : g.loff[0]) + ci)) = value_record(M0 & ~1u, M1, vb);
+                    if (M0 | M1) *reinterpret_cast<uint4*>(auxp + 2ull * blk) = value_record(M0, M1, vb);
                     k = 0; M0 = 0; M1 = 0; vb = vp;
-                    ++j;
-                    if (j == bpm) {
-                        j = 0; ++m;
-                        if (++mcol == mcu_w) { mcol = 0; ++mrow; }
+                    place += 16u;
+                    if (place == place_end) {
+                        place = mem + kSeqPlaces;
+                        ++m; my += hs;
+                        if (m == wrap_m) { wrap_m += mcu_w; my += my_wrap; }
                         if (m >= m1) stop = 0;
                     }
-                    c = j < ny ? 0u : j - ny + 1u;
-                    ci = c ? mrow * mcu_w + mcol : (vs * mrow + (j >> (hs - 1u))) * bw0 + hs * mcol + (j & (hs - 1u));
-                    tdc = mem + ((slots >> (2u * c)) & 1u) * kTab; tac = mem + (2u + ((slots_ac >> (2u * c)) & 1u)) * kTab;
+                    take();
                 }
             }
         }

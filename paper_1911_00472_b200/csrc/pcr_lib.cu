@@ -732,8 +732,8 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
         if (sc.Ss == 0 && sc.Se != 63) continue;
         ax.stride = sc.Ah ? 4u : (sc.Se >= 8 ? 2u : 1u);
         ax.base = aux_words;
+        if (sc.Ss == 0) { aux_words += 2 * blocks; continue; }
         aux_words += (sc.comp[0] == 0 ? (uint64_t)(r->hs * r->vs) : 1ull) * total_mcus * ax.stride;
-        for (int c = 1; sc.Ss == 0 && c < r->nc; ++c) { ax.base_c[c - 1] = aux_words; aux_words += 2 * total_mcus; }
         aux_words = (aux_words + 1) & ~1ull;      // 16-byte alignment of every scan's area
         if (sc.Ah) {
             // positions already non-zero = union of the masks of earlier scans on this band; an
@@ -1050,7 +1050,8 @@ static void coef_lists(const pcr_record* rec, int k, CoefLists* cl) {
                 cl->p1[c][cl->n_refine[c]] = 1 << sc.Al;
                 cl->refine[c][cl->n_refine[c]++] = ax.base;
             } else if (sc.Se >= 8) {
-                cl->first[c][cl->n_first[c]++] = (sc.Ss == 0 && c > 0) ? ax.base_c[c - 1] : ax.base;
+                cl->first[c][cl->n_first[c]++] = ax.base;
+                cl->sequential = sc.Ss == 0;
             }
         }
     }

@@ -485,7 +485,7 @@ struct SeqWrite {
     int16_t* dc;
     int16_t* head;
     int16_t* vals;         // the value array from position 0 of the stream words on
-    uint64_t* auxp[3];     // the scan's side data of the image's components
+    uint64_t* auxp;        // the scan's side data
     uint64_t coff[3];
     uint32_t bw[3];
     uint32_t mcu_w;
@@ -584,7 +584,7 @@ __device__ __forceinline__ void seq_write_span(const HuffTab* tabs4, uint32_t sl
             k += 16;
         }
         if (y.is_eob || k > 63) {                             // block finished
-            if (M0 | M1) *reinterpret_cast<uint4*>(W.auxp[c] + 2ull * local) = value_record(M0, M1, vb);
+            if (M0 | M1) *reinterpret_cast<uint4*>(W.auxp + 2ull * blk) = value_record(M0, M1, vb);
             k = 0; M0 = 0; M1 = 0;
             if (!own) vp = W.vals + ((br.pos() + 1u) >> 1);
             vb = vp;
@@ -643,7 +643,7 @@ __global__ void __launch_bounds__(32 * kSeqLongWarps) sequential_long_kernel(Par
     SeqWrite W;
     const ScanAux ax = P.saux[si / (uint32_t)P.N];
     W.dc = P.dc; W.head = P.head; W.vals = P.vals + 16ull * (bstart >> 2); W.mcu_w = mcu_w; W.hs = (uint32_t)P.hs; W.vs = (uint32_t)P.vs;
-    W.auxp[0] = P.aux + ax.base + 2ull * g.loff[0]; W.auxp[1] = P.aux + ax.base_c[0] + 2ull * g.loff[1]; W.auxp[2] = P.aux + ax.base_c[1] + 2ull * g.loff[1];
+    W.auxp = P.aux + ax.base;
 #pragma unroll
     for (int c = 0; c < 3; ++c) { W.coff[c] = g.coff[c]; W.bw[c] = g.bw[c]; W.pred[c] = 0; }
     W.n = 0; W.n1 = total * bpm;

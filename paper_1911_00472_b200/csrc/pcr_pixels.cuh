@@ -106,7 +106,8 @@ __device__ __forceinline__ void expand_block(const Params& P, const CoefLists& c
     uint4 head = __ldg(reinterpret_cast<const uint4*>(P.head + blk * 8));
     const uint32_t dc = __ldg(reinterpret_cast<const uint16_t*>(P.dc) + blk);
     uint4 rec = zero4;
-    if (nfirst > 0) rec = __ldg(reinterpret_cast<const uint4*>(P.aux + cl.first[comp][0]) + local);
+    const uint64_t at_rec = cl.sequential ? blk : local;
+    if (nfirst > 0) rec = __ldg(reinterpret_cast<const uint4*>(P.aux + cl.first[comp][0]) + at_rec);
     uint4 a0 = zero4, b0 = zero4, a1 = zero4, b1 = zero4;
     if (kRefine) {
         if (nref > 0) { const uint4* o = reinterpret_cast<const uint4*>(P.aux + cl.refine[comp][0]) + 2 * local; a0 = __ldg(o); b0 = __ldg(o + 1); }
@@ -118,7 +119,7 @@ __device__ __forceinline__ void expand_block(const Params& P, const CoefLists& c
     *reinterpret_cast<uint2*>(line) = make_uint2((head.x & hm.x) | dc, head.y & hm.y);
     *reinterpret_cast<uint2*>(line + kPitch) = make_uint2(head.z & hm.z, head.w & hm.w);
     for (int i = 0; i < nfirst; ++i) {
-        if (i) rec = __ldg(reinterpret_cast<const uint4*>(P.aux + cl.first[comp][i]) + local);
+        if (i) rec = __ldg(reinterpret_cast<const uint4*>(P.aux + cl.first[comp][i]) + at_rec);
         const int16_t* v = reinterpret_cast<const int16_t*>(((uint64_t)rec.w << 32) | rec.z);
 #pragma unroll
         for (int half = 0; half < 2; ++half) {

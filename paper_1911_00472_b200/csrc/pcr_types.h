@@ -20,12 +20,12 @@ struct ScanScript {
 //    after the scan, correction bits in reading order (last bit at bit 0), mask of newly
 //    non-zero positions, mask of those that are positive}.  The pixel kernel applies them to a block
 //    when it expands it.
-//  - a sequential scan writes what a first pass over 1..63 would (component c from base + base_c[c - 1] on).
+//  - a sequential scan writes the same for positions 8..63 of the blocks of all components, indexed by the
+//    block's number in the planes.
 // A refinement scan finds the positions that were non-zero before it by OR-ing the masks of up
 // to four earlier scans (src), each read with its own stride.
 struct ScanAux {
     uint64_t base;        // first word of this scan's side data
-    uint64_t base_c[2];   // sequential scans: the chroma components' first words
     uint32_t stride;      // words per block: 1 or 2 (first passes), 4 (refinements)
     int32_t nsrc;
     int32_t src[4];       // scan indices
@@ -38,6 +38,7 @@ constexpr int kMaxFirst = 56;      // first passes of a component that reach bey
 struct CoefLists {
     uint4 head_mask[3];            // positions 1..7 that a decoded scan covers, as 16-bit lanes of the head plane's entries
     int32_t n_first[3], n_refine[3];
+    int32_t sequential;            // side data indexed by the block's number in the planes, not inside its component
     uint64_t first[3][kMaxFirst];  // first word of the scan's side data (two words per block)
     uint64_t refine[3][4];         // the refinement scans in scan order: first word of the side data (four words per block)
     int32_t p1[3][4];              // 1 << Al of the scan
