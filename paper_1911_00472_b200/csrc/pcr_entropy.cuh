@@ -529,8 +529,14 @@ template <bool kRefine> __host__ __device__ constexpr uint32_t warp_bytes() { re
 // rectangle (P.roi) touches are not decoded (their blocks are never transformed).
 // kRefine: the wave holds AC refinements (its warps then need a mask queue; the other waves run with less
 // shared memory and fewer registers).
+//
+// Pairs: a refinement that needs nothing but the masks of the refinement before it (same component, same band, same
+// restart intervals) does not have to wait for that one's launch.  Lanes 0..15 of a warp decode sixteen intervals of the
+// earlier scan, lanes 16..31 the same intervals of the later one, never further than the blocks their partner
+// has finished; what is there is agreed upon at every top-up, where the warp meets anyway.  The chain of a
+// row is then as long as the longer of its two scans instead of their sum.
 template <bool kRoi, bool kRefine>
-__global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, uint32_t item_begin, uint32_t item_count) {
+__global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, ItemRuns runs) {
     extern __shared__ __align__(16) uint8_t s_entropy[];
     __shared__ __align__(16) uint8_t s_sel[kRefine ? sizeof(SelectTable) : 16];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -540,21 +546,25 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, u
             reinterpret_cast<uint4*>(s_sel)[i] = __ldg(reinterpret_cast<const uint4*>(kSelect.at) + i);
         __syncthreads();
     }
-    if (it >= item_count) return;                             // whole warp
-    const Item item = P.items[item_begin + it];
+    if (it >= runs.end[runs.n - 1]) return;                   // whole warp
+    int run_no = 0;
+    while (it >= runs.end[run_no]) ++run_no;
+    const Item item = P.items[runs.first[run_no] + it - (run_no ? runs.end[run_no - 1] : 0u)];
+    const bool half = kRefine && item.pair && lane >= 16;     // this lane decodes the later scan of the pair
+    const uint32_t li = kRefine && item.pair ? (uint32_t)lane & 15u : (uint32_t)lane;
     const ScanDesc sd0 = P.scans[item.si];
-    const int s = item.si / P.N;
+    const int s = (int)((item.si + (half ? item.pair : 0u)) / (uint32_t)P.N);
     const ScanScript sc = P.script[s];
     const ScanAux ax = P.saux[s];
     const bool dc = sc.Ss == 0;              // a DC first pass (DC refinement scans go to dc_refine_kernel)
     // tables: a DC scan may use two tables of one image; an AC item may span two images
     const bool two_images = item.next != 0;
-    const uint32_t si1 = two_images ? item.next - 1u : item.si;
+    const uint32_t si1 = two_images ? item.next - 1u : item.si + item.pair;
     // From here on no lane leaves before the warp does: lanes without work just stay `done`.
-    bool done = (uint32_t)lane >= item.count;
+    bool done = li >= item.count;
     const uint32_t rem0 = sd0.nseg - item.seg0;               // restart intervals left in the first image
-    const uint32_t which = (two_images && (uint32_t)lane >= rem0) ? 1u : 0u;
-    uint32_t seg = which ? (uint32_t)lane - rem0 : item.seg0 + lane;
+    const uint32_t which = half || (two_images && li >= rem0) ? 1u : 0u;
+    uint32_t seg = two_images && li >= rem0 ? li - rem0 : item.seg0 + li;
     const ScanDesc sd = which ? P.scans[si1] : sd0;
     const int img = (int)((which ? si1 : item.si) % (uint32_t)P.N);
     if (seg >= sd.nseg) { done = true; seg = 0; }
@@ -582,9 +592,11 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, u
     }
     const uint32_t mem = (uint32_t)__cvta_generic_to_shared(s_entropy) + (uint32_t)wid * warp_bytes<kRefine>();
     {
-        const uint32_t t0 = ax.tab0 + (item.si % (uint32_t)P.N) * (uint32_t)ax.ntab;
-        const uint32_t t1 = two_images ? ax.tab0 + (si1 % (uint32_t)P.N) * (uint32_t)ax.ntab : t0 + 1u;
-        const bool second = two_images || (dc && sd0.tab_off[1]);
+        const ScanAux ax0 = P.saux[item.si / (uint32_t)P.N];
+        const uint32_t t0 = ax0.tab0 + (item.si % (uint32_t)P.N) * (uint32_t)ax0.ntab;
+        const ScanAux ax1 = P.saux[si1 / (uint32_t)P.N];
+        const uint32_t t1 = dc ? t0 + 1u : ax1.tab0 + (si1 % (uint32_t)P.N) * (uint32_t)ax1.ntab;
+        const bool second = two_images || item.pair || (dc && sd0.tab_off[1]);
         const uint4* a = reinterpret_cast<const uint4*>(P.tabs + t0);
         const uint4* b = reinterpret_cast<const uint4*>(P.tabs + t1);
         constexpr int n = (int)(sizeof(ScanTab) / 16);
@@ -747,12 +759,15 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, u
             auto take = [&]() { Z = lds128(queue + ((m & (kMaskQueue - 1)) << 9)); };
             // (the masks are requested ahead like the words of the stream)
             uint64_t ha[4], hb[4];
+            uint32_t hlimit = half ? m : m1;                           // blocks whose masks are there
+            uint32_t asked = hm;                                       // one past the blocks whose masks have been requested
             auto request = [&]() {
                 uint32_t b = hbi, mm = hm, wm = hwrap_m;
+                asked = min(hm + 4u, hlimit);
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     ha[q] = hb[q] = 0;
-                    if (mm < m1) {
+                    if (mm < hlimit) {
                         ha[q] = src[0][(uint64_t)b * st[0]];
                         if (two) hb[q] = src[1][(uint64_t)b * st[1]];
                     }
@@ -763,7 +778,8 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, u
             if (!done) request();
             for (;;) {
                 br.topup(!done);
-                const uint32_t want = done ? 0u : min((uint32_t)kMaskQueue - (hm - m), m1 - hm);
+                uint32_t want = done ? 0u : min((uint32_t)kMaskQueue - (hm - m), hlimit - hm);
+                if (half) want = min(want, asked - hm);                // (what the partner finished since is requested below)
 #pragma unroll
                 for (int q = 0; q < kMaskQueue; ++q) {
                     if (q == 4 && !__any_sync(full, want > 4u)) break;
@@ -778,14 +794,22 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, u
                     }
                 }
                 __syncwarp(full);
+                if (item.pair) {                                       // how far the partner is (all lanes take part)
+                    const uint32_t pm = __shfl_sync(full, m, (int)li);
+                    const bool stuck = __shfl_sync(full, (int)(done && m < m1), (int)li) != 0;     // ... and that it will get no further
+                    if (half) {
+                        hlimit = min(pm, m1);
+                        if (stuck && m >= hlimit) done = true;
+                    }
+                }
                 if (__all_sync(full, done)) break;
                 if (!done) {
                     request();
-                    if (fresh) take();
+                    if (fresh && m < hm) take();
                 }
                 // a step reads the window at its start and, at most 31 bits on, two words (three for more than
                 // 32 correction bits)
-                uint32_t stop = done ? 0u : min(br.ring_stop(4), br.limit + 1u);
+                uint32_t stop = done || m >= hm ? 0u : min(br.ring_stop(4), br.limit + 1u);
 #pragma unroll 1
                 for (int t = 0; t < kDecodeSteps; ++t) {
                     if (br.pos < stop) {

@@ -170,6 +170,12 @@ struct pcr_record {
     std::vector<cudaEvent_t> ev_copy;                           // [n_waves] bytes of wave w have arrived
     std::vector<cudaEvent_t> ev_join;
     std::vector<std::vector<int>> wave_scans;
+    // The same with pairs of AC refinements in one wave (see entropy_kernel); pair_of[s] = the earlier refinement that
+    // scan s follows, or -1.  Empty when the script has no such pair.
+    std::vector<std::vector<int>> paired_waves;
+    std::vector<int> pair_of;
+    bool pairs_fit = true;                                      // the waves with pairs fit the machine at once
+    std::vector<uint32_t> pair_begin, pair_count;               // [n_slices][G] items of the pair, by its later scan
     uint32_t n_units = 0;
     // device state
     int device = 0;
@@ -584,6 +590,44 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     }
     r->wave_scans.assign(r->n_waves, {});
     for (uint32_t s = 0; s < G; ++s) r->wave_scans[r->wave_of_scan[s]].push_back((int)s);
+    // pairs of AC refinements
+    r->pair_of.assign(G, -1);
+    {
+        std::vector<int> wave(G, 0);
+        bool any = false;
+        for (uint32_t s = 0; s < G; ++s) {
+            const ScanScript& sc = r->script[s];
+            int w = 0, prev = -1, before = 0;     // the last earlier scan that touches the band; the wave all others allow
+            for (uint32_t t = 0; t < s; ++t) {
+                const ScanScript& st = r->script[t];
+                bool share = false;
+                for (int a = 0; a < sc.ncomp; ++a)
+                    for (int b = 0; b < st.ncomp; ++b)
+                        if (sc.comp[a] == st.comp[b]) share = true;
+                if (!share || sc.Ss > st.Se || st.Ss > sc.Se) continue;
+                if (prev >= 0) before = std::max(before, wave[prev] + 1);
+                prev = (int)t;
+                w = std::max(w, wave[t] + 1);
+            }
+            const ScanScript* sp = prev >= 0 ? &r->script[prev] : nullptr;
+            bool pair = sp && sc.Ss > 0 && sc.Ah && sp->Ss == sc.Ss && sp->Se == sc.Se && sp->Ah && r->pair_of[prev] < 0 && before <= wave[prev];
+            for (uint32_t i = 0; pair && i < N; ++i) {
+                const ScanDesc &x = scans[(size_t)prev * N + i], &y = scans[(size_t)s * N + i];
+                pair = x.nseg == y.nseg && x.ri == y.ri;
+            }
+            if (pair) { r->pair_of[s] = prev; w = wave[prev]; any = true; }
+            wave[s] = w;
+        }
+        int n = 0;
+        for (uint32_t s = 0; s < G; ++s) {
+            n = std::max(n, wave[s] + 1);
+            if (r->script[s].Ah == 0 && wave[s] != r->wave_of_scan[s]) any = false;    // (first passes keep their place)
+        }
+        if (any) {
+            r->paired_waves.assign(n, {});
+            for (uint32_t s = 0; s < G; ++s) r->paired_waves[wave[s]].push_back((int)s);
+        } else r->pair_of.assign(G, -1);
+    }
     // slices: enough images each to fill the machine, few enough to keep launches cheap
     {
         // four at most: one record decodes as fast with four slices as with eight, and two records
@@ -695,12 +739,43 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
                     for (; j < sd.nseg; j += kSegsPerItem) {
                         const uint32_t cnt = std::min<uint32_t>(kSegsPerItem, sd.nseg - j);
                         // kItemOpen marks an unfilled last item that the next image may extend
-                        items.push_back(Item{(uint32_t)(s * N + i), j, cnt, (ac && cnt < (uint32_t)kSegsPerItem) ? kItemOpen : 0u});
+                        items.push_back(Item{(uint32_t)(s * N + i), j, cnt, (ac && cnt < (uint32_t)kSegsPerItem) ? kItemOpen : 0u, 0u});
                     }
                 }
                 if (!items.empty() && items.back().next == kItemOpen) items.back().next = 0;
                 r->item_count[(size_t)g * G + s] = (uint32_t)items.size() - r->item_begin[(size_t)g * G + s];
             }
+    // the pairs' items: sixteen intervals of one image
+    r->pair_begin.assign((size_t)r->n_slices * G, 0); r->pair_count.assign((size_t)r->n_slices * G, 0);
+    for (int g = 0; g < r->n_slices; ++g)
+        for (uint32_t s = 0; s < G; ++s) {
+            r->pair_begin[(size_t)g * G + s] = (uint32_t)items.size();
+            for (uint32_t pos = r->slice_img[g]; r->pair_of[s] >= 0 && pos < r->slice_img[g + 1]; ++pos) {
+                const uint32_t i = order[pos], a = (uint32_t)r->pair_of[s];
+                if (takes_long_kernel((int)s, i)) continue;
+                const uint32_t nseg = scans[(size_t)s * N + i].nseg;
+                for (uint32_t j = 0; j < nseg; j += kSegsPerItem / 2)
+                    items.push_back(Item{a * N + i, j, std::min<uint32_t>(kSegsPerItem / 2, nseg - j), 0u, (s - a) * N});
+            }
+            r->pair_count[(size_t)g * G + s] = (uint32_t)items.size() - r->pair_begin[(size_t)g * G + s];
+        }
+    // Pairs shorten the chain but leave the lanes of the shorter scan idle (about 1.4 times the warp instructions for the
+    // ten-scan script), so they are for records whose waves fit the machine at once (18 warps an SM): 96 images of
+    // 4:4:4 552 -> 434 us, 512 ImageNet-shaped images raised 2 -> 10 797 -> 768, 1024 of them at k = 10 991 -> 1022.
+    if (cudaGetDevice(&r->device) != cudaSuccess) return PCR_E_CUDA;
+    if (cudaDeviceGetAttribute(&r->n_sms, cudaDevAttrMultiProcessorCount, r->device) != cudaSuccess) return PCR_E_CUDA;
+    for (const std::vector<int>& scans_of_wave : r->paired_waves) {
+        std::vector<char> in_pair(G, 0);
+        for (int s : scans_of_wave) if (r->pair_of[s] >= 0) in_pair[s] = in_pair[r->pair_of[s]] = 1;
+        uint64_t n = 0;
+        bool any = false;
+        for (int s : scans_of_wave)
+            for (int g = 0; g < r->n_slices; ++g) {
+                n += r->pair_count[(size_t)g * G + s] + (in_pair[s] ? 0u : r->item_count[(size_t)g * G + s]);
+                any = any || in_pair[s];
+            }
+        if (any && n > 20ull * (uint64_t)r->n_sms) r->pairs_fit = false;
+    }
     // pixel work units (see Sampling in pcr_pixels.cuh), image by image in processing order, inside an image
     // MCU row by MCU row.  The host only counts them; a small kernel writes the list at set-up.
     std::vector<uint32_t> unit_prefix(N + 1, 0);
@@ -758,7 +833,6 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     }
 
     // device state
-    if (cudaGetDevice(&r->device) != cudaSuccess) return PCR_E_CUDA;
     if (!(r->up_stream = pool_stream_get(r->device))) return PCR_E_CUDA;
     if (int rc = take(r, &r->d_aux, (size_t)(std::max<uint64_t>(aux_words, 2) * 8))) return rc;
     // zeroing is enqueued after the table uploads: a copy from pageable memory first waits for
@@ -788,7 +862,6 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     if ((rc = upload(r, &r->d_group, groups))) return rc;
     if (r->n_groups) {
         if ((rc = take(r, &r->d_chain_sync, (size_t)(4 + 4 * (size_t)r->n_groups) * 4))) return rc;
-        if (cudaDeviceGetAttribute(&r->n_sms, cudaDevAttrMultiProcessorCount, r->device) != cudaSuccess) return PCR_E_CUDA;
         if (cudaFuncSetAttribute(ac_refine_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kChainPairs * sizeof(ChainShared))) != cudaSuccess) return PCR_E_CUDA;
     }
     if ((rc = upload(r, &r->d_qtab, qtab))) return rc;
@@ -1096,6 +1169,10 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
     }
     CoefLists cl;                                     // everything the pixel stage shows, earlier calls' scans included
     coef_lists(rec, k, &cl);
+    // the waves of this call: with pairs of refinements when both scans of a pair are to be decoded
+    bool paired = false;
+    for (int s = 0; s < k && rec->pairs_fit; ++s) paired = paired || (rec->pair_of[s] >= k0);
+    const std::vector<std::vector<int>>& waves = paired ? rec->paired_waves : rec->wave_scans;
     int first_refine_wave = -1;                 // wave of the first AC refinement this call decodes
     for (int s = k0; s < k; ++s)
         if (rec->script[s].Ss > 0 && rec->script[s].Ah > 0 && (first_refine_wave < 0 || rec->wave_of_scan[s] < first_refine_wave))
@@ -1123,7 +1200,7 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
     std::vector<char> copied(rec->n_waves, 0);      // wave w has to wait for its copy event
     // the stages of one slice; stage numbers: 0 clear, 1 index, 2+w entropy wave w, 2+W unused, 3+W pixels
     // (the pixel kernel also folds the refinement side data into the planes)
-    const int W = rec->n_waves;
+    const int W = (int)waves.size();
     std::vector<char> indexed(rec->n_waves, 0);     // wave w of the current slice has an index launch to wait for
     // index (and lookup tables, where the interval kernels will want them) of the listed scans, all images
     auto launch_index_kernel = [&](const ScanList& sl, cudaStream_t q) {
@@ -1138,7 +1215,7 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
     auto launch_index = [&](int w, cudaStream_t q) -> int {
         ScanList sl;
         sl.n = 0;
-        for (int s : rec->wave_scans[w]) if (s >= k0 && s < k) sl.s[sl.n++] = s;
+        for (int s : waves[w]) if (s >= k0 && s < k) sl.s[sl.n++] = s;
         if (!sl.n) return 0;
         if (copied[w] && cudaStreamWaitEvent(q, rec->ev_copy[w], 0) != cudaSuccess) return -1;
         launch_index_kernel(sl, q);
@@ -1164,23 +1241,52 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
                     if (cudaStreamWaitEvent(q, rec->ev_index[w], 0) != cudaSuccess) return false;
                 }
             }
-            const ScanScript& first = rec->script[rec->wave_scans[w][0]];
+            const ScanScript& first = rec->script[waves[w][0]];
             const bool sequential = first.Ss == 0 && first.Se == 63;   // a baseline record: its one scan is sequential
-            // the items of the wave's scans lie one after the other
-            uint32_t begin = 0, count = 0;
-            for (int s : rec->wave_scans[w]) {
-                if (s >= k) break;   // scans of a wave are stored in ascending order
-                if (s < k0) continue;
-                if (!count) begin = rec->item_begin[(size_t)g * G + s];
-                count += rec->item_count[(size_t)g * G + s];
+            // the runs of items of the wave's scans, pairs (the longest chains) first
+            ItemRuns runs;
+            runs.n = 0;
+            uint32_t count = 0;
+            bool refine = false;                           // waves without AC refinements need no mask queues
+            auto launch_items = [&]() {
+                if (!count) return;
+                const unsigned nb = (count + kEntropyWarps - 1) / kEntropyWarps;
+                const uint32_t smem = kEntropyWarps * (refine ? warp_bytes<true>() : warp_bytes<false>());
+                if (roi && refine) entropy_kernel<true, true><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
+                else if (roi) entropy_kernel<true, false><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
+                else if (refine) entropy_kernel<false, true><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
+                else entropy_kernel<false, false><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
+                ++g_launches;
+                runs.n = 0; count = 0;
+            };
+            auto add_run = [&](uint32_t first, uint32_t n) {
+                if (!n) return;
+                count += n;
+                if (runs.n && runs.first[runs.n - 1] + (runs.end[runs.n - 1] - (runs.n > 1 ? runs.end[runs.n - 2] : 0u)) == first) { runs.end[runs.n - 1] = count; return; }
+                runs.first[runs.n] = first; runs.end[runs.n] = count;
+                ++runs.n;
+            };
+            std::vector<char> in_pair(rec->G, 0);
+            for (int s : waves[w]) {
+                if (s < k0 || s >= k) continue;
+                refine = refine || (rec->script[s].Ss > 0 && rec->script[s].Ah != 0);
+                if (!paired || rec->pair_of[s] < k0) continue;
+                in_pair[s] = in_pair[rec->pair_of[s]] = 1;
+                if (!sequential) add_run(rec->pair_begin[(size_t)g * G + s], rec->pair_count[(size_t)g * G + s]);
             }
+            for (int s : waves[w]) {
+                if (s < k0 || s >= k || in_pair[s]) continue;
+                if (runs.n == kMaxRuns && !sequential) launch_items();
+                add_run(rec->item_begin[(size_t)g * G + s], rec->item_count[(size_t)g * G + s]);
+            }
+            const uint32_t begin = runs.n ? runs.first[0] : 0u;
             if (sequential) {
                 if (count) {
                     if (roi) sequential_kernel<true><<<(count + kSeqWarps - 1) / kSeqWarps, 32 * kSeqWarps, 0, q>>>(P, begin, count);
                     else sequential_kernel<false><<<(count + kSeqWarps - 1) / kSeqWarps, 32 * kSeqWarps, 0, q>>>(P, begin, count);
                     ++g_launches;
                 }
-                const int s0 = rec->wave_scans[w][0];      // the record's one scan
+                const int s0 = waves[w][0];      // the record's one scan
                 const uint32_t lc = (s0 >= k0 && s0 < k) ? rec->long_count[(size_t)g * G + s0] : 0u;
                 if (lc) {                                  // images whose scan is one long restart interval
                     sequential_long_kernel<<<lc, 32 * kSeqLongWarps, 0, q>>>(P, rec->d_long + rec->long_begin[(size_t)g * G + s0], lc);
@@ -1188,23 +1294,13 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
                 }
                 return true;
             }
-            if (count) {
-                const unsigned nb = (count + kEntropyWarps - 1) / kEntropyWarps;
-                bool refine = false;                       // waves without AC refinements need no mask queues
-                for (int s : rec->wave_scans[w]) refine = refine || (rec->script[s].Ss > 0 && rec->script[s].Ah != 0);
-                const uint32_t smem = kEntropyWarps * (refine ? warp_bytes<true>() : warp_bytes<false>());
-                if (roi && refine) entropy_kernel<true, true><<<nb, 32 * kEntropyWarps, smem, q>>>(P, begin, count);
-                else if (roi) entropy_kernel<true, false><<<nb, 32 * kEntropyWarps, smem, q>>>(P, begin, count);
-                else if (refine) entropy_kernel<false, true><<<nb, 32 * kEntropyWarps, smem, q>>>(P, begin, count);
-                else entropy_kernel<false, false><<<nb, 32 * kEntropyWarps, smem, q>>>(P, begin, count);
-                ++g_launches;
-            }
+            launch_items();
             // scans that are one long restart interval: the first passes of the wave (a contiguous run
             // of the list) ...
             {
                 uint32_t lb = 0, lc = 0;
                 bool lany = false;
-                for (int s : rec->wave_scans[w]) {
+                for (int s : waves[w]) {
                     if (s >= k) break;
                     if (s < k0 || rec->script[s].Ah != 0) continue;
                     if (!lany) { lb = rec->long_begin[(size_t)g * G + s]; lany = true; }
@@ -1217,7 +1313,7 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
             }
             // ... (their AC refinements follow in one launch for the whole record, once every slice
             // has finished its waves) and the DC refinement scans of every record
-            for (int s : rec->wave_scans[w]) {
+            for (int s : waves[w]) {
                 if (s >= k) break;
                 const ScanScript& sc = rec->script[s];
                 if (s < k0 || sc.Ss != 0 || sc.Ah == 0) continue;
@@ -1261,7 +1357,7 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
         if (stage == 2 + W) return chains ? 1 : 0;
         if (stage >= 2 && stage < 2 + W) {
             bool any = false;
-            for (int s : rec->wave_scans[stage - 2]) if (s >= k0 && s < k) any = true;
+            for (int s : waves[stage - 2]) if (s >= k0 && s < k) any = true;
             if (!any) return 0;
         }
         return rec->n_slices;
@@ -1302,7 +1398,7 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
             bool any = false;
             for (int w = 0; w < W; ++w) {
                 size_t upto = 0;
-                for (int s : rec->wave_scans[w]) if (s < k) upto = std::max(upto, (size_t)rec->group_end[s + 1]);
+                for (int s : waves[w]) if (s < k) upto = std::max(upto, (size_t)rec->group_end[s + 1]);
                 if (upto > rec->resident) {
                     const size_t from = rec->resident & ~(size_t)15;
                     if (cudaMemcpyAsync(rec->d_rec + from, rec->host + from, upto - from, cudaMemcpyHostToDevice, rec->copy_stream) != cudaSuccess) return PCR_E_CUDA;

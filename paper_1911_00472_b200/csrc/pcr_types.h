@@ -76,12 +76,20 @@ struct ImgDesc {
 #endif
 constexpr int kSegsPerItem = PCR_SEGS_PER_ITEM;
 
-// Entropy work item: up to kSegsPerItem consecutive restart intervals of one (scan, image).
+// Entropy work item: up to kSegsPerItem consecutive restart intervals of one (scan, image); or up to half as many of
+// two AC refinements of the same band that follow one another (see entropy_kernel).
 struct Item {
     uint32_t si;          // scan * N + image
     uint32_t seg0;        // first restart interval of the item
     uint32_t count;       // restart intervals in the item (<= kSegsPerItem)
     uint32_t next;        // 0, or 1 + (scan * N + image) of the image whose first intervals the item runs on into
+    uint32_t pair;        // 0, or the distance to the later refinement of the pair (in scan * N + image)
+};
+// The runs of the item list that one launch covers.
+constexpr int kMaxRuns = 24;
+struct ItemRuns {
+    int32_t n;
+    uint32_t first[kMaxRuns], end[kMaxRuns];   // first item of the run; items in this run and those before it
 };
 constexpr uint32_t kItemOpen = 0xFFFFFFFFu;   // host only, while the list is built: the item may still be extended
 
