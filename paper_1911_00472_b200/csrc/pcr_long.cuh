@@ -686,13 +686,16 @@ __global__ void __launch_bounds__(32 * kSeqLongWarps) sequential_long_kernel(Par
 // {non-zero mask of the band after the scan, correction bits in reading order, the last one in bit 0,
 // newly non-zero positions, the positive ones among them}.
 //
-// The time of a chain is the number of instructions one thread executes per symbol (every
-// instruction waits for the one before), so the decoding thread only follows the chain: Huffman
-// symbol -> run r -> position of the (r+1)-th still-zero coefficient -> number of correction bits
-// passed -> next symbol.  For every symbol it leaves a record {bit position behind the sign, new
-// position, number of correction bits}; the chain's helper warp lists the still-zero positions
-// of the next 32 blocks meanwhile and afterwards turns the records of 32 blocks into the side
-// data (one lane per block, reading sign and correction bits back from the ring).
+// The time of a chain is the latency of what one thread does per symbol, so the decoding thread only follows
+// the chain, through two shared-memory tables that the chain's helper warp prepares:
+//   q[bit]       what the symbol that begins at this bit of the stream is (skip, run, flags): every bit position is
+//                decoded in advance, 32 at a time, so the thread neither assembles a window nor looks up a code;
+//   zpos[i][b]   position of the i-th still-zero coefficient of block b, minus i: the run's target, and by
+//                differences the number of correction bits passed.
+// A symbol is two dependent loads and a handful of additions (about 15 instructions; 35 with a bit reader and
+// symbol records).  Per block the thread leaves the bit position where it began; the helper warp decodes the
+// 32 blocks of a finished batch once more, one lane per block, to make the side data.
+// HAM-shaped record, 1024 images: the launch 3.4 -> @@ ms.
 //
 // A later refinement of the same component needs the masks the earlier one leaves, block by
 // block.  Both walk the same block grid in the same order, so the later chain runs behind the
@@ -702,44 +705,12 @@ __global__ void __launch_bounds__(32 * kSeqLongWarps) sequential_long_kernel(Par
 // started after the chains it depends on (queue order), so its producer is running or done.
 // ---------------------------------------------------------------------------------------
 constexpr int kChainPairs = 16;          // chains per CTA of the persistent refinement launch (four per scheduler), two warps each
-constexpr int kChainRing = 256;          // words of bitstream per chain in shared memory
-constexpr int kChainRecs = 512;          // symbol records per batch of blocks (four bytes each)
+constexpr uint32_t kChainRing = 128;     // words of bitstream per chain in shared memory
+constexpr uint32_t kChainBits = 32 * kChainRing;
 constexpr int kChainLutBits = 9;         // refinement alphabets are small (runs 0..15 with size 0 or 1): short codes
 constexpr uint32_t kChainBlockWords = 44;   // a block never needs more: 63 symbols of at most 17 bits, 3 sixteen-zero runs, one run length, 63 correction bits
 constexpr uint32_t kSpinLimit = 1u << 22;   // polls (of at least 64 ns) before a wait gives up
 constexpr int kErrTimeout = -4;
-
-struct ChainBits {
-    const uint32_t* ring;
-    uint32_t w0, w1, w2;   // the word the next bit lies in and the two after it
-    uint32_t bits;         // position of the next bit, counted from the first bit of ring word `org`
-    uint32_t org;          // absolute index of that word (moved up at the start of every batch)
-    __device__ __forceinline__ void init(const uint32_t* r, uint32_t first, uint32_t lead) {
-        ring = r;
-        w0 = r[first & (kChainRing - 1)]; w1 = r[(first + 1) & (kChainRing - 1)]; w2 = r[(first + 2) & (kChainRing - 1)];
-        org = first;
-        bits = lead;
-    }
-    __device__ __forceinline__ uint32_t win() const { return __funnelshift_l(w1, w0, bits); }   // the next 32 bits (shift taken mod 32)
-    __device__ __forceinline__ uint32_t word() const { return org + (bits >> 5); }               // absolute index of the word of the next bit
-    __device__ __forceinline__ void skip(uint32_t n) {
-        const uint32_t nb = bits + n, adv = (nb >> 5) - (bits >> 5);
-        bits = nb;
-        if (adv) {
-            const uint32_t wi = org + (nb >> 5);
-            if (adv == 1u) { w0 = w1; w1 = w2; }
-            else { w0 = ring[wi & (kChainRing - 1)]; w1 = ring[(wi + 1u) & (kChainRing - 1)]; }
-            w2 = ring[(wi + 2u) & (kChainRing - 1)];
-        }
-    }
-    __device__ __forceinline__ void rebase() { org += bits >> 5; bits &= 31u; }
-};
-
-// the n bits (1..32) at bit position p (counted from the first bit of word `base`) of the ring
-__device__ __forceinline__ uint32_t ring_bits(const uint32_t* ring, uint32_t base, uint32_t p, uint32_t n) {
-    const uint32_t a = ring[(base + (p >> 5)) & (kChainRing - 1)], b = ring[(base + (p >> 5) + 1u) & (kChainRing - 1)];
-    return __funnelshift_l(b, a, p & 31u) >> (32u - n);
-}
 
 // Polls *flag until it reaches `need`, sleeping `ns` nanoseconds between polls; false after `limit` polls.
 __device__ __forceinline__ bool wait_at_least(const volatile uint32_t* flag, uint32_t need, uint32_t limit, uint32_t ns = 64) {
@@ -751,39 +722,44 @@ __device__ __forceinline__ bool wait_at_least(const volatile uint32_t* flag, uin
     return false;
 }
 
-// Entry of the chain's own lookup table on the next kChainLutBits bits, made from the Huffman table:
-// bits 0..4 = bits to skip (code, plus the sign bit of a new coefficient), 5..11 = run r, 15 = a new
-// coefficient follows the run; the end of band of a single block is entered as a run of 64 without a
-// new coefficient (it passes over the rest of the band like a run that overshoots); 0 = everything
-// else (longer end-of-band runs, codes longer than the index, undefined codes): the general path.
-__device__ __noinline__ uint32_t chain_lookup(const HuffTabT<kChainLutBits>& tab, uint32_t win) { return huff_lookup(tab, win); }
+// Entry of q: twice the bits to skip (code, sign bit, run-length bits) in bits 0..5, 6 = a new coefficient, 7 = not a
+// plain step (an end-of-band run of more than this block: bits 9..12 its exponent; or no symbol: the rest is zero),
+// 9..15 = run of zeros (64: the rest of the band, the end of band of this block alone).
+constexpr uint32_t kQNew = 0x40u, kQSpecial = 0x80u;
+__device__ __forceinline__ uint32_t chain_entry(uint32_t len, uint32_t rs) {
+    const uint32_t r = rs >> 4, newc = rs & 1u;
+    if (len == 0 || (rs & 14u)) return kQSpecial;                       // a refinement symbol has size 0 or 1
+    if (newc || r == 15u) return (2u * (len + newc)) | (newc ? kQNew : 0u) | (r << 9);
+    if (r == 0u) return (2u * len) | (64u << 9);
+    return (2u * (len + r)) | kQSpecial | (r << 9);
+}
 
-struct ChainLists {
-    uint64_t h[32];                    // positions of the band that are already non-zero, per block of the batch
-    uint8_t zpos[64][32];              // [i][block]: position of the block's i-th still-zero coefficient of the band, minus i;
-                                       // entry nz: Se + 1 - nz (as if position Se + 1 followed)
-    uint8_t nz[32];                    // how many such positions there are (at most 63)
-};
-struct ChainRecs {
-    uint32_t rec[kChainRecs];          // corrections | position << 8 | new << 15 | (bit position behind the sign bit - base) << 16
-    uint32_t first[33];                // first record of each block of the batch
-    uint32_t base;                     // bit position at which the batch starts
-};
 struct ChainMail {                     // what the two warps of a chain tell each other at a meeting point
-    uint32_t nd, rd, err_c;            // decoder: blocks it decoded, oldest ring word it still needs, error
+    uint32_t nd, rd, err_c;            // decoder: blocks it decoded, the word it stands at, error
     uint32_t wr, err_h;                // helper: the ring is filled up to this word, error
 };
 struct ChainShared {
-    HuffTabT<kChainLutBits> tab;
-    uint32_t quick[1 << kChainLutBits];
+    uint16_t q[kChainBits];            // by bit position modulo kChainBits
+    uint8_t zpos[2][64][32];           // [batch][i][block]: twice (position of the block's i-th still-zero coefficient of the band, minus i);
+                                       // entry nz: Se + 1 - nz (as if position Se + 1 followed)
+    uint16_t ends[2][32];              // per block: how many still-zero positions there are (nz, at most 63) and, from bit 8
+                                       // on, the rank that ends the block (nz, or nz - 1 if the last of them is Se)
+    uint32_t start[2][32];             // per block: where it began (bit position; bit 31: inside an end-of-band run)
     uint32_t ring[kChainRing];
-    ChainLists lists[2];               // the batch being decoded and the one being prepared
-    ChainRecs recs[2];                 // the batch being decoded and the one being turned into side data
+    uint16_t quick[1 << kChainLutBits];         // q entries of the codes of at most kChainLutBits bits, 0: longer
+    uint16_t first[8], cnt[8], idx[8];          // the longer codes: first code, how many, index of the first value
     ChainMail mail[2];                 // by parity of the meeting point
     uint32_t job_gi, job_level;        // the pair's job (job_gi = 0xFFFFFFFF: none left)
-    uint32_t Ss, Se, total, rd0, lead, limit;   // of the job, for the decoder
+    uint32_t Ss, Se, total, lead, limit;        // of the job, for the decoder (bits counted from the interval's first word)
     volatile uint32_t phase_c, phase_h;         // meeting points each side has reached
 };
+static_assert(kChainPairs * sizeof(ChainShared) <= 227 * 1024, "one CTA per SM holds all its chains");
+
+// the n bits (1..32) at bit position p of the ring
+__device__ __forceinline__ uint32_t ring_bits(const uint32_t* ring, uint32_t p, uint32_t n) {
+    const uint32_t a = ring[(p >> 5) & (kChainRing - 1)], b = ring[((p >> 5) + 1u) & (kChainRing - 1)];
+    return __funnelshift_l(b, a, p & 31u) >> (32u - n);
+}
 
 // Polls *flag (another warp's progress word in global memory) until it reaches `need`; `seen` keeps
 // the last value read, so that a consumer that is behind anyway polls once per many batches.
@@ -813,18 +789,18 @@ __device__ __forceinline__ bool meet_helper(ChainShared& sh, uint32_t k, int lan
     if (lane == 0) { __threadfence_block(); sh.phase_h = k; }
     // (long sleeps: the helper is far ahead of the decoder, and its polls would take issue slots from the chains)
     bool ok = true;
-    if (lane == 0) ok = wait_at_least(&sh.phase_c, k, kSpinLimit, 512);
+    if (lane == 0) ok = wait_at_least(&sh.phase_c, k, kSpinLimit, 256);
     ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
     __threadfence_block();
     return ok;
 }
 
 // The decoding side of a chain: one thread.  It takes the pair's jobs (first the statically assigned
-// one, then tickets of its scheduler's queue), and per job follows the bit stream batch by batch:
-// the lists of still-zero positions of a batch come from the helper, the symbol records go back to it.
+// one, then tickets of its scheduler's queue), and per job follows the bit stream batch by batch.
 __device__ __forceinline__ void chain_decoder(const RefineList& fl, ChainShared& sh, const uint32_t* __restrict__ list, uint32_t n_groups,
                                               uint32_t* sync, uint32_t levels, uint32_t rounds, uint32_t q, uint32_t slot) {
     const uint32_t per_round = 4u * gridDim.x, statics = per_round * rounds;
+    const uint32_t a_q = (uint32_t)__cvta_generic_to_shared(sh.q), a_zpos = (uint32_t)__cvta_generic_to_shared(sh.zpos);
     uint32_t mk = 0;                                           // meeting points so far
     bool first_job = true;
     for (;;) {
@@ -848,78 +824,59 @@ __device__ __forceinline__ void chain_decoder(const RefineList& fl, ChainShared&
         if (!meet_decoder(sh, ++mk)) return;                   // tables, first lists and ring are ready
         if (sh.mail[mk & 1u].err_h) continue;                  // a scan whose bounds are off: the helper reports it
         uint32_t wr = sh.mail[mk & 1u].wr;
-        const uint32_t Ss = sh.Ss, Se = sh.Se, total = sh.total, limit = sh.limit;
-        ChainBits B;
-        B.init(sh.ring, sh.rd0, sh.lead);
+        const uint32_t Ss2 = 2u * sh.Ss, total = sh.total, limit = sh.limit;
+        uint32_t pos2 = 2u * sh.lead;                          // twice the bit position (the tables' entries are two bytes)
         uint32_t eobrun = 0, m = 0, p = 0;
         for (;;) {
             const uint32_t nblk = min(32u, total - m);
-            const ChainLists& L = sh.lists[p];
-            ChainRecs& R = sh.recs[p];
-            // positions inside a batch count from the word the batch starts in (fewer than 2^16 bits: 32
-            // blocks of kChainBlockWords words)
-            B.rebase();
-            const uint32_t base = (B.org - sh.rd0) * 32u;
-            R.base = base;
-            // a block is only begun while kChainBlockWords words lie ahead in the ring and the interval has
-            // not ended: one comparison for both, told apart behind the loop
-            const uint32_t avail = wr - B.org;
-            const uint32_t pause_bits = avail > kChainBlockWords + 2u ? (avail - (kChainBlockWords + 2u)) << 5 : 0u;
-            const uint32_t end_bits = limit >= base ? limit - base + 1u : 0u;      // first position that is past the end
-            const uint32_t stop_bits = min(pause_bits, end_bits);
-            uint32_t* recp = R.rec;
-            uint32_t* const rec_stop = R.rec + (kChainRecs - 64);
+            // a block is only begun while kChainBlockWords words lie ahead (q ends one word before the ring) and the
+            // interval has not ended: one comparison for both, told apart behind the loop
+            const uint32_t stop2 = 2u * min(32u * (wr - min(wr, kChainBlockWords + 3u)), limit + 1u);
+            const uint32_t zrow = a_zpos + 2048u * p;
             uint32_t nd = 0;
             int err = 0;
+            uint32_t next_ends = sh.ends[p][0];
             for (; nd < nblk; ++nd) {
-                if (B.bits >= stop_bits || recp > rec_stop) break;
-                R.first[nd] = (uint32_t)(recp - R.rec);
-                // zi: how many of the block's still-zero positions are passed; ep: the list entry of the last
-                // one reached (entry t = position - t, so that the difference of two entries is the number of
-                // non-zero positions between them: one correction bit each)
-                const uint32_t nz = L.nz[nd];
-                uint32_t zi = 0, ep = Ss;
-                bool band_done = false;
+                if (pos2 >= stop2) break;
+                const uint32_t nz = next_ends & 255u, tend = next_ends >> 8;
+                next_ends = sh.ends[p][(nd + 1u) & 31u];       // (the next block's, out of the way of its chain)
+                sh.start[p][nd] = (pos2 >> 1) | (eobrun ? 0x80000000u : 0u);
+                const uint32_t zb = zrow + nd;
+                // zi: how many of the block's still-zero positions are passed; ep2: twice the list entry of the last
+                // one reached (the difference of two entries is the number of non-zero positions between them: one
+                // correction bit each)
+                uint32_t ep2 = Ss2;
                 if (eobrun == 0) {
-                    for (;;) {
-                        const uint32_t win = B.win();
-                        uint32_t qe = sh.quick[win >> (32 - kChainLutBits)];
-                        if (qe == 0) {                         // not a plain (run, new coefficient) symbol
-                            const uint32_t e = chain_lookup(sh.tab, win);
-                            const uint32_t len = e >> 8, rs = e & 255u, newc = rs & 1u, r = rs >> 4;
-                            if (e == 0 || (rs & 14u)) { err = kErrCorrupt; break; }   // a refinement symbol has size 0 or 1
-                            if (!newc && r < 15u) {            // end of band for this block and eobrun - 1 more
-                                eobrun = 1u << r;
-                                if (r) eobrun += (win << len) >> (32u - r);
-                                B.skip(len + r);
-                                break;
-                            }
-                            qe = (len + newc) | (r << 5) | (newc << 15);   // a code longer than the table's index
+                    uint32_t zi = 0, t;
+                    bool band_done = false;
+#pragma unroll 1
+                    do {
+                        const uint32_t e = lds16(a_q + (pos2 & (2u * kChainBits - 1u)));
+                        if (e & kQSpecial) {
+                            if (e == kQSpecial) { err = kErrCorrupt; break; }
+                            const uint32_t x = (e >> 9) & 15u;              // the band ends for this block and eobrun - 1 more
+                            pos2 += e & 63u;
+                            eobrun = (1u << x) + ring_bits(sh.ring, (pos2 >> 1) - x, x);
+                            break;
                         }
                         // the target: the (r+1)-th still-zero position from here; a run past the last one ends
                         // at the list's closing entry (position Se + 1)
-                        const uint32_t t = min(zi + ((qe >> 5) & 127u), nz);
-                        const uint32_t e = L.zpos[t][nd];
-                        const uint32_t cnt = e - ep, pos = e + t, n1 = qe & 31u;
-                        *recp++ = ((B.bits + n1) << 16) | (pos << 8) | (qe & 0x8000u) | cnt;
-                        B.skip(n1 + cnt);                      // code, sign and correction bits in one step
+                        t = min(zi + (e >> 9), nz);
+                        const uint32_t e2 = lds8(zb + 32u * t);
+                        pos2 += (e & 63u) - ep2 + e2;          // code, sign and correction bits in one step
                         zi = t + 1u;
-                        ep = e;
-                        if (pos >= Se) { band_done = true; break; }
-                    }
+                        ep2 = e2;
+                        band_done = t >= tend;
+                    } while (!band_done);
+                    if (band_done) continue;
+                    if (err) break;
                 }
-                if (err) break;
-                if (!band_done) {                              // inside an end-of-band run: corrections for the rest of the band
-                    const uint32_t cnt = L.zpos[nz][nd] - ep;
-                    *recp++ = (B.bits << 16) | cnt;
-                    B.skip(cnt);
-                    --eobrun;
-                }
+                pos2 += lds8(zb + 32u * nz) - ep2;             // inside an end-of-band run: corrections for the rest of the band
+                --eobrun;
             }
-            R.first[nd] = (uint32_t)(recp - R.rec);
-            if (!err && B.bits >= end_bits) err = kErrCorrupt;     // read past the end of the interval
+            if (!err && (pos2 >> 1) > limit) err = kErrCorrupt;    // read past the end of the interval
             ++mk;
-            sh.mail[mk & 1u].nd = nd; sh.mail[mk & 1u].rd = B.word(); sh.mail[mk & 1u].err_c = (uint32_t)err;
+            sh.mail[mk & 1u].nd = nd; sh.mail[mk & 1u].rd = pos2 >> 6; sh.mail[mk & 1u].err_c = (uint32_t)err;
             if (!meet_decoder(sh, mk)) return;
             wr = sh.mail[mk & 1u].wr;
             if (err || sh.mail[mk & 1u].err_h) break;
@@ -938,9 +895,9 @@ __device__ __forceinline__ void chain_decoder(const RefineList& fl, ChainShared&
 }
 
 // The helper side of a chain: a whole warp.  Per job it builds the tables, then stays one batch ahead
-// of the decoder with the masks and lists of still-zero positions (waiting, with bounded polls, for
+// of the decoder with the lists of still-zero positions (waiting, with bounded polls, for
 // an earlier refinement of the same blocks when this launch decodes that too), keeps the ring of
-// bitstream words filled, and one batch behind it turns the symbol records into side data.
+// bitstream words and their symbols filled, and one batch behind it makes the side data.
 __device__ __forceinline__ void chain_helper(const Params& P, const RefineList& fl, ChainShared& sh, const uint32_t* __restrict__ list,
                                              uint32_t* progress_all, int lane) {
     const unsigned full = 0xffffffffu;
@@ -955,26 +912,47 @@ __device__ __forceinline__ void chain_helper(const Params& P, const RefineList& 
         uint32_t* progress = progress_all + 4ull * gi;
         volatile uint32_t* my_progress = progress + level;
         const int s = fl.scan[c][level];
-        const ScanDesc sd = P.scans[(uint32_t)s * (uint32_t)P.N + (uint32_t)img];
+        const ScanDesc& sd = P.scans[(uint32_t)s * (uint32_t)P.N + (uint32_t)img];
         const ScanScript sc = P.script[s];
         const Geometry g = make_geometry(P.imgs[img], P);
         const uint32_t Ss = (uint32_t)sc.Ss, Se = (uint32_t)sc.Se;
         const uint32_t mcu_w = g.ubw[c], total = g.ubw[c] * g.ubh[c], bw = g.bw[c];
-        build_hufftab(sh.tab, P.rec + sd.tab_off[0], lane);
-        for (int i = lane; i < (1 << kChainLutBits); i += 32) {
-            const uint32_t e = sh.tab.lut[i], len = e >> 8, rs = e & 255u, newc = rs & 1u, r = rs >> 4;
-            const bool plain = e != 0 && (rs & 14u) == 0 && (newc || r == 15u || r == 0u);   // run + new coefficient, sixteen zeros, end of band
-            sh.quick[i] = plain ? ((len + newc) | ((rs == 0u ? 64u : r) << 5) | (newc << 15)) : 0u;
+        // the code tables: q entries of the short codes, the canonical description of the longer ones
+        const uint8_t* dht = P.rec + sd.tab_off[0];
+        {
+            uint32_t* s_code = &sh.start[0][0];                // scratch (51 words): first code, first index, end of the codes
+            const uint32_t my = lane < 16 ? dht[lane] : 0u;
+            uint32_t code = 0, idx = 0;
+            for (int l = 1; l <= 16; ++l) {
+                const uint32_t n = __shfl_sync(full, my, l - 1);
+                if (lane == 0) {
+                    s_code[l] = code; s_code[17 + l] = idx;
+                    if (l <= kChainLutBits) s_code[34 + l] = (code + n) << (kChainLutBits - l);
+                    else { const int j = l - kChainLutBits - 1; sh.first[j] = (uint16_t)code; sh.cnt[j] = (uint16_t)n; sh.idx[j] = (uint16_t)idx; }
+                }
+                code = (code + n) << 1;
+                idx += n;
+            }
+            __syncwarp(full);
+            int l = 1;
+            for (int e = 0; e < (1 << kChainLutBits) / 32; ++e) {      // consecutive entries: the code length only grows
+                const uint32_t x = (uint32_t)lane * ((1u << kChainLutBits) / 32u) + (uint32_t)e;
+                while (l <= kChainLutBits && x >= s_code[34 + l]) ++l;
+                uint32_t v = 0;
+                if (l <= kChainLutBits) v = chain_entry((uint32_t)l, dht[16u + ((s_code[17 + l] + (x >> (kChainLutBits - l)) - s_code[l]) & 255u)]);
+                sh.quick[x] = (uint16_t)v;
+            }
+            __syncwarp(full);
         }
         const uint32_t* segtab = P.seg_start + sd.seg_base;
         const uint32_t bstart = segtab[0], bend = segtab[1] - 2u;
         const bool bad = bstart < sd.data_off || bend > sd.data_end || bend < bstart;
-        const uint32_t* words = reinterpret_cast<const uint32_t*>(P.ubuf);
         const uint32_t rd0 = bstart >> 2, lead = 8u * (bstart & 3u);
-        const uint32_t wlim = ((bend + 3u) >> 2) + 2u;         // words beyond are not read (zeros instead)
+        const uint32_t* words = reinterpret_cast<const uint32_t*>(P.ubuf) + rd0;
+        const uint32_t wlim = ((bend + 3u) >> 2) + 2u - rd0;   // words beyond are not read (zeros instead)
         if (lane == 0) {
-            sh.Ss = Ss; sh.Se = Se; sh.total = total; sh.rd0 = rd0; sh.lead = lead;
-            sh.limit = lead + 8u * (bend - bstart);            // first bit behind the interval, counted from word rd0
+            sh.Ss = Ss; sh.Se = Se; sh.total = total; sh.lead = lead;
+            sh.limit = lead + 8u * (bend - bstart);            // first bit behind the interval
         }
         // masks of the positions that are already non-zero: the union of up to four earlier scans; a
         // source that this launch decodes itself (an earlier level of the group) is waited for
@@ -998,11 +976,11 @@ __device__ __forceinline__ void chain_helper(const Params& P, const RefineList& 
         }
         uint64_t* outp = P.aux + ax.base + g.loff[c] * 4ull;
         uint32_t* ring = sh.ring;
-        uint32_t wr = rd0, seen0 = 0, seen1 = 0, seen2 = 0;
+        uint32_t wr = 0, seen0 = 0, seen1 = 0, seen2 = 0;
         int err = bad ? kErrCorrupt : 0;
         auto block_index = [&](uint32_t x) { const uint32_t row = x / mcu_w; return row * bw + (x - row * mcu_w); };
-        // the masks of blocks m0 .. m0 + 31 and their lists of still-zero positions
-        auto gather = [&](uint32_t m0, ChainLists& L) -> int {
+        // the masks of blocks m0 .. m0 + 31 (one per lane, returned in h) and their lists of still-zero positions
+        auto gather = [&](uint32_t m0, uint32_t b, uint64_t& h) -> int {
             const uint32_t nblk = min(32u, total - m0);
             if (prod0 && !wait_progress(prod0, m0 + nblk, seen0, kSpinLimit)) return kErrTimeout;
             if (prod1 && !wait_progress(prod1, m0 + nblk, seen1, kSpinLimit)) return kErrTimeout;
@@ -1015,59 +993,87 @@ __device__ __forceinline__ void chain_helper(const Params& P, const RefineList& 
                 if (src2) v |= __ldcg(src2 + (uint64_t)bi * st2);
                 if (src3) v |= __ldcg(src3 + (uint64_t)bi * st3);
                 v &= band;
-                L.h[lane] = v;
+                h = v;
                 // the positions of the band that are still zero, in order: the target of a run r is then one
-                // table look-up for the decoder (the (r+1)-th of those not yet passed).  (Listing the few non-zero
-                // positions instead and stepping over them measured 18 % slower: the steps sit on the chain.)
+                // table look-up for the decoder (the (r+1)-th of those not yet passed)
                 const uint64_t z = ~v & band;
+                uint8_t* dst = &sh.zpos[b][0][lane];
                 uint32_t n = 0;
 #pragma unroll
                 for (int half = 0; half < 2; ++half) {
                     uint32_t w = half ? (uint32_t)(z >> 32) : (uint32_t)z;
                     while (w) {
-                        L.zpos[n][lane] = (uint8_t)(32 * half + __ffs((int)w) - 1 - (int)n);
+                        dst[32u * n] = (uint8_t)(2u * (32u * half + (uint32_t)__ffs((int)w) - 1u - n));
                         ++n;
                         w &= w - 1u;
                     }
                 }
-                L.zpos[n][lane] = (uint8_t)(Se + 1u - n);      // closing entry: behind the band
-                L.nz[lane] = (uint8_t)n;
+                dst[32u * n] = (uint8_t)(2u * (Se + 1u - n));      // closing entry: behind the band
+                const uint32_t tend = (z >> Se) & 1u ? n - 1u : n; // the block also ends at a still-zero position Se
+                sh.ends[b][lane] = (uint16_t)(n | (tend << 8));
             }
             return 0;
         };
-        // the ring filled as far as it goes while word `oldest` is still needed
+        // The ring and q filled as far as they go while word `oldest` is still needed.  The symbol at a word's bits
+        // needs the word behind it, so q ends one word before the ring.
         auto top_up = [&](uint32_t oldest) {
-            while (wr - oldest + 32u <= (uint32_t)kChainRing) {
+            while (wr - oldest + 32u <= kChainRing) {
                 ring[(wr + lane) & (kChainRing - 1)] = wr + lane < wlim ? __ldg(words + wr + lane) : 0u;
+                __syncwarp(full);
+                for (uint32_t w = wr ? wr - 1u : 0u; w < wr + 31u; ++w) {
+                    const uint32_t win = __funnelshift_l(ring[(w + 1u) & (kChainRing - 1)], ring[w & (kChainRing - 1)], (uint32_t)lane);
+                    uint32_t e = sh.quick[win >> (32 - kChainLutBits)];
+                    if (e == 0) {                                  // a code longer than the table's index, or none
+                        e = kQSpecial;
+#pragma unroll 1
+                        for (uint32_t j = 0; j < 16u - kChainLutBits; ++j) {
+                            const uint32_t l = kChainLutBits + 1u + j, d = (win >> (32u - l)) - sh.first[j];
+                            if (d < sh.cnt[j]) { e = chain_entry(l, dht[16u + ((sh.idx[j] + d) & 255u)]); break; }
+                        }
+                    }
+                    sh.q[(32u * w + lane) & (kChainBits - 1u)] = (uint16_t)e;
+                }
                 wr += 32u;
+                __syncwarp(full);
             }
         };
-        // the records of blocks m0 .. m0 + nd - 1 -> side data, one block per lane; then the count
-        auto side_data = [&](uint32_t m0, uint32_t nd, const ChainRecs& R, const ChainLists& L) {
+        // the blocks m0 .. m0 + nd - 1 of batch buffer b once more, one per lane -> side data; then the count
+        auto side_data = [&](uint32_t m0, uint32_t nd, uint32_t b, uint64_t h) {
             bool over = false;
             if ((uint32_t)lane < nd) {
+                const uint32_t st = sh.start[b][lane], nz = sh.ends[b][lane] & 255u, tend = sh.ends[b][lane] >> 8;
+                const uint8_t* zp = &sh.zpos[b][0][lane];
+                uint32_t at = st & 0x7FFFFFFFu, zi = 0, ep = 2u * Ss, cn = 0;
+                bool open = true;                              // the band has not ended with a symbol
                 uint64_t cstr = 0, Nw = 0, NS = 0;
-                uint32_t cn = 0;
-                for (uint32_t i = R.first[lane]; i < R.first[lane + 1]; ++i) {
-                    const uint32_t rc = R.rec[i], at = R.base + (rc >> 16);
-                    uint32_t n = rc & 127u;
-                    if (rc & 0x8000u) {
-                        if (((rc >> 8) & 127u) > Se) { over = true; break; }   // a new coefficient behind the band
-                        const uint64_t bit = 1ull << ((rc >> 8) & 63u);
-                        Nw |= bit;
-                        if (ring_bits(ring, rd0, at - 1u, 1u)) NS |= bit;
-                    }
-                    if (cn + n > 64u) { over = true; break; }
+                auto corrections = [&](uint32_t n) {           // n bits at `at`
                     cn += n;
-                    uint32_t bp = at;
                     while (n) {
                         const uint32_t nn = min(n, 32u);
-                        cstr = (cstr << nn) | (uint64_t)ring_bits(ring, rd0, bp, nn);
-                        bp += nn; n -= nn;
+                        cstr = (cstr << nn) | (uint64_t)ring_bits(ring, at, nn);
+                        at += nn; n -= nn;
+                    }
+                };
+                if (!(st >> 31)) {
+                    for (int i = 0; i < 80; ++i) {             // (more symbols than a block can have)
+                        const uint32_t e = sh.q[at & (kChainBits - 1u)];
+                        at += (e & 63u) >> 1;
+                        if (e & kQSpecial) break;              // an end-of-band run begins
+                        const uint32_t t = min(zi + (e >> 9), nz), e2 = zp[32u * t], pos = (e2 >> 1) + t;
+                        if (e & kQNew) {
+                            if (pos > Se) { over = true; open = false; break; }    // a new coefficient behind the band
+                            Nw |= 1ull << pos;
+                            if (ring_bits(ring, at - 1u, 1u)) NS |= 1ull << pos;
+                        }
+                        corrections((e2 - ep) >> 1);
+                        ep = e2; zi = t + 1u;
+                        if (t >= tend) { open = false; break; }
                     }
                 }
+                if (open) corrections((zp[32u * nz] - ep) >> 1);
+                over = over || cn > 64u;
                 ulonglong2* o = reinterpret_cast<ulonglong2*>(outp + (uint64_t)block_index(m0 + lane) * 4);
-                o[0] = make_ulonglong2((L.h[lane] | Nw), cstr);
+                o[0] = make_ulonglong2(h | Nw, cstr);
                 o[1] = make_ulonglong2(Nw, NS);
             }
             if (__any_sync(full, over)) err = kErrCorrupt;
@@ -1075,19 +1081,20 @@ __device__ __forceinline__ void chain_helper(const Params& P, const RefineList& 
             __syncwarp(full);
             if (lane == 0) *my_progress = m0 + nd;
         };
+        uint64_t h_now = 0, h_next = 0, h_pend = 0;            // masks of the batch being decoded, the one after it, the one before it
         if (!bad) {
-            err = gather(0, sh.lists[0]);
-            top_up(rd0);
+            err = gather(0, 0, h_now);
+            top_up(0);
         }
         ++mk;
         if (lane == 0) { sh.mail[mk & 1u].wr = wr; sh.mail[mk & 1u].err_h = (uint32_t)err; }
         if (!meet_helper(sh, mk, lane)) return;
-        uint32_t m = 0, p = 0, rd_c = rd0, pend_m = 0, pend_n = 0, pend_p = 0;
+        uint32_t m = 0, p = 0, rd_c = 0, pend_m = 0, pend_n = 0, pend_p = 0;
         while (!err) {
             const uint32_t nblk = min(32u, total - m);
-            if (pend_n) { side_data(pend_m, pend_n, sh.recs[pend_p], sh.lists[pend_p]); pend_n = 0; }
+            if (pend_n) { side_data(pend_m, pend_n, pend_p, h_pend); pend_n = 0; }
             top_up(rd_c);
-            if (m + nblk < total) { const int e = gather(m + nblk, sh.lists[p ^ 1u]); if (!err) err = e; }
+            if (m + nblk < total) { const int e = gather(m + nblk, p ^ 1u, h_next); if (!err) err = e; }
             ++mk;
             if (lane == 0) { sh.mail[mk & 1u].wr = wr; sh.mail[mk & 1u].err_h = (uint32_t)err; }
             if (!meet_helper(sh, mk, lane)) return;
@@ -1096,15 +1103,16 @@ __device__ __forceinline__ void chain_helper(const Params& P, const RefineList& 
             rd_c = sh.mail[mk & 1u].rd;
             if (err || err_c) { if (!err) err = err_c; break; }
             if (nd == nblk) {
-                pend_m = m; pend_n = nd; pend_p = p;
+                pend_m = m; pend_n = nd; pend_p = p; h_pend = h_now;
+                h_now = h_next;
                 p ^= 1u;
                 m += nd;
-                if (m >= total) { side_data(pend_m, pend_n, sh.recs[pend_p], sh.lists[pend_p]); break; }
-            } else {                                           // the decoder stopped early: its records now, the lists from m again
-                if (nd) side_data(m, nd, sh.recs[p], sh.lists[p]);
+                if (m >= total) { side_data(pend_m, pend_n, pend_p, h_pend); break; }
+            } else {                                           // the decoder stopped early: its blocks now, the lists from m again
+                if (nd) side_data(m, nd, p, h_now);
                 m += nd;
                 top_up(rd_c);
-                { const int e = gather(m, sh.lists[p ^ 1u]); if (!err) err = e; }
+                { const int e = gather(m, p ^ 1u, h_now); if (!err) err = e; }
                 ++mk;
                 if (lane == 0) { sh.mail[mk & 1u].wr = wr; sh.mail[mk & 1u].err_h = (uint32_t)err; }
                 if (!meet_helper(sh, mk, lane)) return;
