@@ -665,7 +665,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
         const ScanScript& sc = r->script[s];
         const ScanDesc& sd = scans[(size_t)s * N + i];
         (void)sc;
-        return sd.nseg == 1 && sd.data_end - sd.data_off >= long_min;
+        return sd.nseg == 1 && sd.data_end - sd.data_off >= long_min && sd.data_end - sd.data_off < (1u << 27);   // (the chains count half bits)
     };
     // the AC refinements of one component of one image go together: all of them one interval each,
     // at least one of them long
@@ -677,7 +677,8 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
                 const ScanScript& sc = r->script[s];
                 if (sc.Ss == 0 || sc.Ah == 0 || sc.comp[0] != c) continue;
                 any = true;
-                one_interval = one_interval && scans[(size_t)s * N + i].nseg == 1;
+                const ScanDesc& sd = scans[(size_t)s * N + i];
+                one_interval = one_interval && sd.nseg == 1 && sd.data_end - sd.data_off < (1u << 27);
                 big = big || is_long((int)s, i);
             }
             grouped[(size_t)i * 3 + c] = any && one_interval && big;

@@ -695,7 +695,7 @@ __global__ void __launch_bounds__(32 * kSeqLongWarps) sequential_long_kernel(Par
 // A symbol is two dependent loads and a handful of additions (about 15 instructions; 35 with a bit reader and
 // symbol records).  Per block the thread leaves the bit position where it began; the helper warp decodes the
 // 32 blocks of a finished batch once more, one lane per block, to make the side data.
-// HAM-shaped record, 1024 images: the launch 3.4 -> @@ ms.
+// HAM-shaped record, 1024 images: the launch 3.4 -> 1.7 ms (about 100 cycles a symbol, 60 a block on the longest chain).
 //
 // A later refinement of the same component needs the masks the earlier one leaves, block by
 // block.  Both walk the same block grid in the same order, so the later chain runs behind the
@@ -722,16 +722,15 @@ __device__ __forceinline__ bool wait_at_least(const volatile uint32_t* flag, uin
     return false;
 }
 
-// Entry of q: twice the bits to skip (code, sign bit, run-length bits) in bits 0..5, 6 = a new coefficient, 7 = not a
-// plain step (an end-of-band run of more than this block: bits 9..12 its exponent; or no symbol: the rest is zero),
-// 9..15 = run of zeros (64: the rest of the band, the end of band of this block alone).
-constexpr uint32_t kQNew = 0x40u, kQSpecial = 0x80u;
+// Entry of q: twice the bits to skip (code, sign bit, run-length bits) in bits 0..5, 6 = a new coefficient, 7 = more than
+// a plain step (an end-of-band run that covers further blocks, or no symbol: the rest but bit 15 is zero),
+// 9..15 = run of zeros (from 64 on: the rest of the band; 64 + the exponent of an end-of-band run).
+constexpr uint32_t kQNew = 0x40u, kQSpecial = 0x80u, kQRest = 64u << 9, kQBad = kQSpecial | kQRest;
 __device__ __forceinline__ uint32_t chain_entry(uint32_t len, uint32_t rs) {
     const uint32_t r = rs >> 4, newc = rs & 1u;
-    if (len == 0 || (rs & 14u)) return kQSpecial;                       // a refinement symbol has size 0 or 1
+    if (rs & 14u) return kQBad;                                        // a refinement symbol has size 0 or 1
     if (newc || r == 15u) return (2u * (len + newc)) | (newc ? kQNew : 0u) | (r << 9);
-    if (r == 0u) return (2u * len) | (64u << 9);
-    return (2u * (len + r)) | kQSpecial | (r << 9);
+    return (2u * (len + r)) | (r ? kQSpecial : 0u) | kQRest | (r << 9);
 }
 
 struct ChainMail {                     // what the two warps of a chain tell each other at a meeting point
@@ -769,7 +768,7 @@ __device__ __forceinline__ bool wait_progress(const volatile uint32_t* flag, uin
     for (uint32_t i = 0; i < limit; ++i) {
         seen = *flag;
         if (seen >= need) return true;
-        __nanosleep(64);
+        __nanosleep(500);
     }
     return false;
 }
@@ -780,7 +779,7 @@ __device__ __forceinline__ bool wait_progress(const volatile uint32_t* flag, uin
 __device__ __forceinline__ bool meet_decoder(ChainShared& sh, uint32_t k) {          // one thread
     __threadfence_block();
     sh.phase_c = k;
-    const bool ok = wait_at_least(&sh.phase_h, k, kSpinLimit);
+    const bool ok = wait_at_least(&sh.phase_h, k, kSpinLimit, 300);
     __threadfence_block();
     return ok;
 }
@@ -789,7 +788,7 @@ __device__ __forceinline__ bool meet_helper(ChainShared& sh, uint32_t k, int lan
     if (lane == 0) { __threadfence_block(); sh.phase_h = k; }
     // (long sleeps: the helper is far ahead of the decoder, and its polls would take issue slots from the chains)
     bool ok = true;
-    if (lane == 0) ok = wait_at_least(&sh.phase_c, k, kSpinLimit, 256);
+    if (lane == 0) ok = wait_at_least(&sh.phase_c, k, kSpinLimit, 1000);
     ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
     __threadfence_block();
     return ok;
@@ -800,7 +799,9 @@ __device__ __forceinline__ bool meet_helper(ChainShared& sh, uint32_t k, int lan
 __device__ __forceinline__ void chain_decoder(const RefineList& fl, ChainShared& sh, const uint32_t* __restrict__ list, uint32_t n_groups,
                                               uint32_t* sync, uint32_t levels, uint32_t rounds, uint32_t q, uint32_t slot) {
     const uint32_t per_round = 4u * gridDim.x, statics = per_round * rounds;
-    const uint32_t a_q = (uint32_t)__cvta_generic_to_shared(sh.q), a_zpos = (uint32_t)__cvta_generic_to_shared(sh.zpos);
+    uint32_t a_q = (uint32_t)__cvta_generic_to_shared(sh.q), a_zpos = (uint32_t)__cvta_generic_to_shared(sh.zpos);
+    uint32_t a_ends = (uint32_t)__cvta_generic_to_shared(sh.ends), a_start = (uint32_t)__cvta_generic_to_shared(sh.start);
+    asm volatile("" : "+r"(a_q), "+r"(a_zpos), "+r"(a_ends), "+r"(a_start));   // (kept in registers)
     uint32_t mk = 0;                                           // meeting points so far
     bool first_job = true;
     for (;;) {
@@ -829,50 +830,57 @@ __device__ __forceinline__ void chain_decoder(const RefineList& fl, ChainShared&
         uint32_t eobrun = 0, m = 0, p = 0;
         for (;;) {
             const uint32_t nblk = min(32u, total - m);
-            // a block is only begun while kChainBlockWords words lie ahead (q ends one word before the ring) and the
-            // interval has not ended: one comparison for both, told apart behind the loop
-            const uint32_t stop2 = 2u * min(32u * (wr - min(wr, kChainBlockWords + 3u)), limit + 1u);
-            const uint32_t zrow = a_zpos + 2048u * p;
+            // A block is only begun while kChainBlockWords words lie ahead (q ends one word before the ring) and, the
+            // batch's first one, while the interval has not ended (reading on behind it is found below; zeros follow).
+            // Inside the loop the test is made a symbol early, with room for it: see below.
+            const uint32_t lead2 = 64u * (wr - min(wr, kChainBlockWords + 3u)), early2 = lead2 - min(lead2, 192u);
+            const uint32_t ends = a_ends + 64u * p, start = a_start + 128u * p;
+            uint32_t zb = a_zpos + 2048u * p;                  // of the block: its column of the lists
             uint32_t nd = 0;
             int err = 0;
-            uint32_t next_ends = sh.ends[p][0];
-            for (; nd < nblk; ++nd) {
-                if (pos2 >= stop2) break;
-                const uint32_t nz = next_ends & 255u, tend = next_ends >> 8;
-                next_ends = sh.ends[p][(nd + 1u) & 31u];       // (the next block's, out of the way of its chain)
-                sh.start[p][nd] = (pos2 >> 1) | (eobrun ? 0x80000000u : 0u);
-                const uint32_t zb = zrow + nd;
-                // zi: how many of the block's still-zero positions are passed; ep2: twice the list entry of the last
-                // one reached (the difference of two entries is the number of non-zero positions between them: one
-                // correction bit each)
-                uint32_t ep2 = Ss2;
+            uint32_t now = lds16(ends);
+            uint32_t nz = now & 255u, tend = now >> 8, next = lds16(ends + 2u);   // of the block, and of the next one
+            bool go = pos2 < lead2 && (pos2 >> 1) <= limit;
+            while (go) {
                 if (eobrun == 0) {
-                    uint32_t zi = 0, t;
-                    bool band_done = false;
+                    uint32_t e, before;
+                    for (;;) {
+                        sts32(start + 4u * nd, pos2 >> 1);
+                        // ep2: twice the list entry of the last still-zero position reached (the difference of two
+                        // entries is the number of non-zero positions between them: one correction bit each); zi:
+                        // how many are passed
+                        uint32_t zi = 0, ep2 = Ss2, t;
 #pragma unroll 1
-                    do {
-                        const uint32_t e = lds16(a_q + (pos2 & (2u * kChainBits - 1u)));
-                        if (e & kQSpecial) {
-                            if (e == kQSpecial) { err = kErrCorrupt; break; }
-                            const uint32_t x = (e >> 9) & 15u;              // the band ends for this block and eobrun - 1 more
-                            pos2 += e & 63u;
-                            eobrun = (1u << x) + ring_bits(sh.ring, (pos2 >> 1) - x, x);
-                            break;
-                        }
-                        // the target: the (r+1)-th still-zero position from here; a run past the last one ends
-                        // at the list's closing entry (position Se + 1)
-                        t = min(zi + (e >> 9), nz);
-                        const uint32_t e2 = lds8(zb + 32u * t);
-                        pos2 += (e & 63u) - ep2 + e2;          // code, sign and correction bits in one step
-                        zi = t + 1u;
-                        ep2 = e2;
-                        band_done = t >= tend;
-                    } while (!band_done);
-                    if (band_done) continue;
-                    if (err) break;
+                        do {
+                            before = pos2;
+                            e = lds16(a_q + (pos2 & (2u * kChainBits - 1u)));
+                            // the target: the (r+1)-th still-zero position from here; a run past the last one (an end
+                            // of band is one too) ends at the list's closing entry (position Se + 1)
+                            t = min(zi + (e >> 9), nz);
+                            const uint32_t e2 = lds8(zb + 32u * t);
+                            pos2 += (e & 63u) - ep2 + e2;      // code, sign and correction bits in one step
+                            zi = t + 1u;
+                            ep2 = e2;
+                        } while (t < tend);                    // (known before e2 is: the branch costs the chain nothing,
+                        ++nd; ++zb;                            // nor does what a new block takes)
+                        nz = next & 255u; tend = next >> 8;
+                        next = lds16(ends + 2u * ((nd + 1u) & 31u));
+                        if (nd == nblk || (e & kQSpecial) || before >= early2) break;
+                    }
+                    if (e & kQSpecial) {                       // the band also ends for the next eobrun blocks
+                        if (e == kQBad) { err = kErrCorrupt; --nd; break; }
+                        const uint32_t x = (e >> 9) & 15u;
+                        eobrun = (1u << x) + ring_bits(sh.ring, ((before + (e & 63u)) >> 1) - x, x) - 1u;
+                    }
+                } else {
+                    sts32(start + 4u * nd, (pos2 >> 1) | 0x80000000u);
+                    pos2 += lds8(zb + 32u * nz) - Ss2;         // inside an end-of-band run: corrections for the whole band
+                    --eobrun;
+                    ++nd; ++zb;
+                    nz = next & 255u; tend = next >> 8;
+                    next = lds16(ends + 2u * ((nd + 1u) & 31u));
                 }
-                pos2 += lds8(zb + 32u * nz) - ep2;             // inside an end-of-band run: corrections for the rest of the band
-                --eobrun;
+                go = nd < nblk && pos2 < lead2;
             }
             if (!err && (pos2 >> 1) > limit) err = kErrCorrupt;    // read past the end of the interval
             ++mk;
@@ -977,63 +985,94 @@ __device__ __forceinline__ void chain_helper(const Params& P, const RefineList& 
         uint64_t* outp = P.aux + ax.base + g.loff[c] * 4ull;
         uint32_t* ring = sh.ring;
         uint32_t wr = 0, seen0 = 0, seen1 = 0, seen2 = 0;
+        const bool watched = level + 1 < fl.n[c];              // a later level of the group reads the side data
         int err = bad ? kErrCorrupt : 0;
         auto block_index = [&](uint32_t x) { const uint32_t row = x / mcu_w; return row * bw + (x - row * mcu_w); };
-        // the masks of blocks m0 .. m0 + 31 (one per lane, returned in h) and their lists of still-zero positions
-        auto gather = [&](uint32_t m0, uint32_t b, uint64_t& h) -> int {
-            const uint32_t nblk = min(32u, total - m0);
-            if (prod0 && !wait_progress(prod0, m0 + nblk, seen0, kSpinLimit)) return kErrTimeout;
-            if (prod1 && !wait_progress(prod1, m0 + nblk, seen1, kSpinLimit)) return kErrTimeout;
-            if (prod2 && !wait_progress(prod2, m0 + nblk, seen2, kSpinLimit)) return kErrTimeout;
-            __threadfence();
+        // the masks of blocks m0 .. m0 + 31, one per lane (requested: nothing waits for the loads yet)
+        auto masks = [&](uint32_t m0, uint64_t& h) -> int {
+            const uint32_t nblk = min(32u, total - m0), need = m0 + nblk;
+            const bool polls = (prod0 && seen0 < need) || (prod1 && seen1 < need) || (prod2 && seen2 < need);
+            if (polls) {
+                if (prod0 && !wait_progress(prod0, need, seen0, kSpinLimit)) return kErrTimeout;
+                if (prod1 && !wait_progress(prod1, need, seen1, kSpinLimit)) return kErrTimeout;
+                if (prod2 && !wait_progress(prod2, need, seen2, kSpinLimit)) return kErrTimeout;
+                __threadfence();
+            }
+            h = 0;
             if ((uint32_t)lane < nblk) {
                 const uint32_t bi = block_index(m0 + lane);
                 uint64_t v = __ldcg(src0 + (uint64_t)bi * st0);    // not through L1: a line may hold blocks written later
                 if (src1) v |= __ldcg(src1 + (uint64_t)bi * st1);
                 if (src2) v |= __ldcg(src2 + (uint64_t)bi * st2);
                 if (src3) v |= __ldcg(src3 + (uint64_t)bi * st3);
-                v &= band;
                 h = v;
-                // the positions of the band that are still zero, in order: the target of a run r is then one
-                // table look-up for the decoder (the (r+1)-th of those not yet passed)
-                const uint64_t z = ~v & band;
-                uint8_t* dst = &sh.zpos[b][0][lane];
-                uint32_t n = 0;
-#pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    uint32_t w = half ? (uint32_t)(z >> 32) : (uint32_t)z;
-                    while (w) {
-                        dst[32u * n] = (uint8_t)(2u * (32u * half + (uint32_t)__ffs((int)w) - 1u - n));
-                        ++n;
-                        w &= w - 1u;
-                    }
-                }
-                dst[32u * n] = (uint8_t)(2u * (Se + 1u - n));      // closing entry: behind the band
-                const uint32_t tend = (z >> Se) & 1u ? n - 1u : n; // the block also ends at a still-zero position Se
-                sh.ends[b][lane] = (uint16_t)(n | (tend << 8));
             }
             return 0;
         };
+        // the blocks' lists of still-zero positions into batch buffer b
+        auto lists = [&](uint32_t m0, uint32_t b, uint64_t& h) {
+            const uint32_t nblk = min(32u, total - m0);
+            if ((uint32_t)lane < nblk) {
+                h &= band;
+                const uint64_t v = h;
+                // the positions of the band that are still zero, in order: the target of a run r is then one
+                // table look-up for the decoder (the (r+1)-th of those not yet passed)
+                const uint64_t z = ~v & band;
+                uint32_t dst = (uint32_t)__cvta_generic_to_shared(&sh.zpos[b][0][lane]);
+                const uint32_t dst0 = dst;
+                uint32_t v2 = 0;                                   // twice (position minus number of still-zero ones before it)
+                // (straight through all positions, lanes with different masks stay together; a position outside the band
+                // counts as non-zero)
+#pragma unroll
+                for (int pos = 0; pos < 64; ++pos) {
+                    const uint32_t zw = pos < 32 ? (uint32_t)z : (uint32_t)(z >> 32);
+                    if ((zw >> (pos & 31)) & 1u) {
+                        asm volatile("st.shared.u8 [%0], %1;" : : "r"(dst), "r"(v2) : "memory");
+                        dst += 32u;
+                    } else v2 += 2u;
+                }
+                const uint32_t n = (dst - dst0) >> 5;
+                asm volatile("st.shared.u8 [%0], %1;" : : "r"(dst), "r"(2u * (Se + 1u - n)) : "memory");      // closing entry: behind the band
+                const uint32_t tend = (z >> Se) & 1u ? n - 1u : n; // the block also ends at a still-zero position Se
+                sh.ends[b][lane] = (uint16_t)(n | (tend << 8));
+            }
+        };
         // The ring and q filled as far as they go while word `oldest` is still needed.  The symbol at a word's bits
-        // needs the word behind it, so q ends one word before the ring.
+        // needs the word behind it, so q ends one word before the ring.  The next words are requested ahead.
+        uint32_t ahead = 0;
+        auto request = [&]() { ahead = wr + lane < wlim ? __ldg(words + wr + lane) : 0u; };
         auto top_up = [&](uint32_t oldest) {
             while (wr - oldest + 32u <= kChainRing) {
-                ring[(wr + lane) & (kChainRing - 1)] = wr + lane < wlim ? __ldg(words + wr + lane) : 0u;
+                ring[(wr + lane) & (kChainRing - 1)] = ahead;
                 __syncwarp(full);
-                for (uint32_t w = wr ? wr - 1u : 0u; w < wr + 31u; ++w) {
-                    const uint32_t win = __funnelshift_l(ring[(w + 1u) & (kChainRing - 1)], ring[w & (kChainRing - 1)], (uint32_t)lane);
-                    uint32_t e = sh.quick[win >> (32 - kChainLutBits)];
-                    if (e == 0) {                                  // a code longer than the table's index, or none
-                        e = kQSpecial;
 #pragma unroll 1
-                        for (uint32_t j = 0; j < 16u - kChainLutBits; ++j) {
-                            const uint32_t l = kChainLutBits + 1u + j, d = (win >> (32u - l)) - sh.first[j];
-                            if (d < sh.cnt[j]) { e = chain_entry(l, dht[16u + ((sh.idx[j] + d) & 255u)]); break; }
+                for (uint32_t w = wr - 1u; w != wr + 31u; w += 8u) {   // (word -1 at first: never looked at)
+                    uint32_t x[9], e[8], none = 0;
+#pragma unroll
+                    for (uint32_t i = 0; i < 9; ++i) x[i] = ring[(w + i) & (kChainRing - 1)];
+#pragma unroll
+                    for (uint32_t i = 0; i < 8; ++i) {
+                        x[i] = __funnelshift_l(x[i + 1], x[i], (uint32_t)lane);
+                        e[i] = sh.quick[x[i] >> (32 - kChainLutBits)];
+                        none |= e[i] == 0 ? 1u << i : 0u;
+                    }
+                    if (none) {                                    // codes longer than the table's index, or none
+#pragma unroll
+                        for (uint32_t i = 0; i < 8; ++i) {
+                            if (!((none >> i) & 1u)) continue;
+                            e[i] = kQBad;
+#pragma unroll 1
+                            for (uint32_t j = 0; j < 16u - kChainLutBits; ++j) {
+                                const uint32_t l = kChainLutBits + 1u + j, d = (x[i] >> (32u - l)) - sh.first[j];
+                                if (d < sh.cnt[j]) { e[i] = chain_entry(l, dht[16u + ((sh.idx[j] + d) & 255u)]); break; }
+                            }
                         }
                     }
-                    sh.q[(32u * w + lane) & (kChainBits - 1u)] = (uint16_t)e;
+#pragma unroll
+                    for (uint32_t i = 0; i < 8; ++i) sh.q[(32u * (w + i) + lane) & (kChainBits - 1u)] = (uint16_t)e[i];
                 }
                 wr += 32u;
+                request();
                 __syncwarp(full);
             }
         };
@@ -1041,50 +1080,54 @@ __device__ __forceinline__ void chain_helper(const Params& P, const RefineList& 
         auto side_data = [&](uint32_t m0, uint32_t nd, uint32_t b, uint64_t h) {
             bool over = false;
             if ((uint32_t)lane < nd) {
-                const uint32_t st = sh.start[b][lane], nz = sh.ends[b][lane] & 255u, tend = sh.ends[b][lane] >> 8;
+                const uint32_t st = sh.start[b][lane], nz = sh.ends[b][lane] & 255u;
                 const uint8_t* zp = &sh.zpos[b][0][lane];
-                uint32_t at = st & 0x7FFFFFFFu, zi = 0, ep = 2u * Ss, cn = 0;
-                bool open = true;                              // the band has not ended with a symbol
-                uint64_t cstr = 0, Nw = 0, NS = 0;
-                auto corrections = [&](uint32_t n) {           // n bits at `at`
-                    cn += n;
-                    while (n) {
-                        const uint32_t nn = min(n, 32u);
-                        cstr = (cstr << nn) | (uint64_t)ring_bits(ring, at, nn);
-                        at += nn; n -= nn;
-                    }
-                };
-                if (!(st >> 31)) {
-                    for (int i = 0; i < 80; ++i) {             // (more symbols than a block can have)
-                        const uint32_t e = sh.q[at & (kChainBits - 1u)];
-                        at += (e & 63u) >> 1;
-                        if (e & kQSpecial) break;              // an end-of-band run begins
-                        const uint32_t t = min(zi + (e >> 9), nz), e2 = zp[32u * t], pos = (e2 >> 1) + t;
-                        if (e & kQNew) {
-                            if (pos > Se) { over = true; open = false; break; }    // a new coefficient behind the band
-                            Nw |= 1ull << pos;
-                            if (ring_bits(ring, at - 1u, 1u)) NS |= 1ull << pos;
+                uint32_t at = st & 0x7FFFFFFFu, zi = 0, ep = 2u * Ss, k = 0;
+                uint32_t s0 = 0, s1 = 0, N0 = 0, N1 = 0, G0 = 0, G1 = 0;
+                // a block inside an end-of-band run is one step over the rest of the band that takes no symbol
+                uint32_t e = st >> 31 ? kQRest : (uint32_t)sh.q[at & (kChainBits - 1u)];
+#pragma unroll 1
+                for (int i = 0; i < 80 && k < Se; ++i) {       // (bounded: more symbols than a block can have)
+                    const uint32_t skip = (e & 63u) >> 1, sign_at = at + skip - 1u;
+                    const uint32_t t = min(zi + (e >> 9), nz), e2 = zp[32u * t], n = (e2 - ep) >> 1;
+                    k = (e2 >> 1) + t;
+                    const uint32_t isnew = e & kQNew ? 1u : 0u;
+                    over = over || (isnew && k > Se);          // a new coefficient behind the band
+                    const uint32_t plus = isnew & (ring[(sign_at >> 5) & (kChainRing - 1)] >> (~sign_at & 31u));
+                    N0 |= shl0(isnew, k); N1 |= shl0(isnew, k - 32u);
+                    G0 |= shl0(plus, k); G1 |= shl0(plus, k - 32u);
+                    at += skip;
+                    if (n) {
+                        const uint32_t w = ring_bits(ring, at, 32u);
+                        if (n > 32u) {
+                            s1 = (w >> (64u - n)) | (s0 << (n - 32u));
+                            s0 = __funnelshift_l(ring_bits(ring, at + 32u, 32u), w, n - 32u);
+                        } else {
+                            s1 = __funnelshift_lc(s0, s1, n);
+                            s0 = shl0(s0, n) | (w >> (32u - n));
                         }
-                        corrections((e2 - ep) >> 1);
-                        ep = e2; zi = t + 1u;
-                        if (t >= tend) { open = false; break; }
+                        at += n;
                     }
+                    ep = e2; zi = t + 1u;
+                    e = sh.q[at & (kChainBits - 1u)];
                 }
-                if (open) corrections((zp[32u * nz] - ep) >> 1);
-                over = over || cn > 64u;
-                ulonglong2* o = reinterpret_cast<ulonglong2*>(outp + (uint64_t)block_index(m0 + lane) * 4);
-                o[0] = make_ulonglong2(h | Nw, cstr);
-                o[1] = make_ulonglong2(Nw, NS);
+                uint4* o = reinterpret_cast<uint4*>(outp + (uint64_t)block_index(m0 + lane) * 4);
+                o[0] = make_uint4((uint32_t)h | N0, (uint32_t)(h >> 32) | N1, s0, s1);
+                o[1] = make_uint4(N0, N1, G0, G1);
             }
             if (__any_sync(full, over)) err = kErrCorrupt;
-            __threadfence();                                   // the side data before the count
-            __syncwarp(full);
-            if (lane == 0) *my_progress = m0 + nd;
+            if (watched) {
+                __threadfence();                               // the side data before the count
+                __syncwarp(full);
+                if (lane == 0) *my_progress = m0 + nd;
+            }
         };
         uint64_t h_now = 0, h_next = 0, h_pend = 0;            // masks of the batch being decoded, the one after it, the one before it
         if (!bad) {
-            err = gather(0, 0, h_now);
+            err = masks(0, h_now);
+            request();
             top_up(0);
+            lists(0, 0, h_now);
         }
         ++mk;
         if (lane == 0) { sh.mail[mk & 1u].wr = wr; sh.mail[mk & 1u].err_h = (uint32_t)err; }
@@ -1092,9 +1135,11 @@ __device__ __forceinline__ void chain_helper(const Params& P, const RefineList& 
         uint32_t m = 0, p = 0, rd_c = 0, pend_m = 0, pend_n = 0, pend_p = 0;
         while (!err) {
             const uint32_t nblk = min(32u, total - m);
+            const bool more = m + nblk < total;
+            if (more) { const int e = masks(m + nblk, h_next); if (!err) err = e; }
             if (pend_n) { side_data(pend_m, pend_n, pend_p, h_pend); pend_n = 0; }
             top_up(rd_c);
-            if (m + nblk < total) { const int e = gather(m + nblk, p ^ 1u, h_next); if (!err) err = e; }
+            if (more) lists(m + nblk, p ^ 1u, h_next);
             ++mk;
             if (lane == 0) { sh.mail[mk & 1u].wr = wr; sh.mail[mk & 1u].err_h = (uint32_t)err; }
             if (!meet_helper(sh, mk, lane)) return;
@@ -1112,7 +1157,8 @@ __device__ __forceinline__ void chain_helper(const Params& P, const RefineList& 
                 if (nd) side_data(m, nd, p, h_now);
                 m += nd;
                 top_up(rd_c);
-                { const int e = gather(m, p ^ 1u, h_now); if (!err) err = e; }
+                { const int e = masks(m, h_now); if (!err) err = e; }
+                lists(m, p ^ 1u, h_now);
                 ++mk;
                 if (lane == 0) { sh.mail[mk & 1u].wr = wr; sh.mail[mk & 1u].err_h = (uint32_t)err; }
                 if (!meet_helper(sh, mk, lane)) return;
