@@ -14,6 +14,7 @@
 #include <algorithm>
 #include <atomic>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <thread>
@@ -74,6 +75,43 @@ void* dev_alloc(size_t n, int device) {
         if (cudaMalloc(&p, cls) != cudaSuccess) { cudaGetLastError(); return nullptr; }
     }
     return p;
+}
+
+// Page-locked host blocks in which pcr_open builds a record's tables: one asynchronous copy takes them to the
+// device, and a block that has been used before costs no page faults.  Kept for later opens up to kHostLimit bytes.
+struct HostCache {
+    std::mutex mu;
+    std::multimap<size_t, void*> free_;
+    size_t cached = 0;
+    static constexpr size_t kLimit = 256ull << 20;
+} g_host;
+
+void* host_alloc(size_t n) {
+    const size_t cls = size_class(n);
+    {
+        std::lock_guard<std::mutex> lk(g_host.mu);
+        auto it = g_host.free_.find(cls);
+        if (it != g_host.free_.end()) {
+            void* p = it->second;
+            g_host.free_.erase(it);
+            g_host.cached -= cls;
+            return p;
+        }
+    }
+    void* p = nullptr;
+    if (cudaHostAlloc(&p, cls, cudaHostAllocPortable) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    return p;
+}
+void host_release(void* p, size_t n) {
+    if (!p) return;
+    const size_t cls = size_class(n);
+    std::lock_guard<std::mutex> lk(g_host.mu);
+    if (g_host.cached + cls <= HostCache::kLimit) {
+        g_host.free_.insert({cls, p});
+        g_host.cached += cls;
+    } else {
+        cudaFreeHost(p);
+    }
 }
 
 // internal streams and (non-timing) events are pooled the same way
@@ -211,6 +249,7 @@ struct pcr_record {
     int* d_status = nullptr;
     std::vector<int> h_status;
     std::vector<std::pair<void*, size_t>> bufs;   // every device buffer of the record with its size
+    std::vector<std::pair<void*, size_t>> stages; // host blocks the tables were built in (their copies may be in flight)
     cudaStream_t up_stream = nullptr;             // pcr_open's uploads and memsets (never the default stream:
                                                   // that one would wait for every other record's decode)
     cudaEvent_t ev_ready = nullptr;               // the record's device state is set up
@@ -224,7 +263,7 @@ struct pcr_record {
     // optional stage timing
     bool profiling = false;
     std::vector<cudaEvent_t> events;
-    std::vector<pcr_stage_time> stages;   // names and launch counts of the last decode
+    std::vector<pcr_stage_time> profile;  // names and launch counts of the last decode
 };
 
 static const int kMaxStages = 16;
@@ -232,10 +271,14 @@ static const int kMaxStages = 16;
 static inline uint32_t rd32(const uint8_t* p) { return (uint32_t)p[0] | ((uint32_t)p[1] << 8) | ((uint32_t)p[2] << 16) | ((uint32_t)p[3] << 24); }
 static inline uint64_t rd64(const uint8_t* p) { return (uint64_t)rd32(p) | ((uint64_t)rd32(p + 4) << 32); }
 
-// Writes the list of pixel work units at set-up: block = position of the processing order.
+// Writes the list of pixel work units at set-up, and every (scan, image)'s place in the segment table into its
+// descriptor (the host has the places in an array of their own: the descriptors' cache lines belong to the threads that
+// made them): block = position of the processing order.
 __global__ void __launch_bounds__(128) units_kernel(const ImgDesc* __restrict__ imgs, const uint32_t* __restrict__ order,
-                                                    const uint32_t* __restrict__ prefix, Unit* __restrict__ units, uint32_t unit_mcus, uint32_t unit_rows) {
+                                                    const uint32_t* __restrict__ prefix, Unit* __restrict__ units, uint32_t unit_mcus, uint32_t unit_rows,
+                                                    ScanDesc* __restrict__ scans, const uint32_t* __restrict__ seg_base, uint32_t G) {
     const uint32_t img = order[blockIdx.x];
+    for (uint32_t g = threadIdx.x; g < G; g += 128) scans[(size_t)g * gridDim.x + img].seg_base = seg_base[(size_t)g * gridDim.x + img];
     const uint32_t per_row = (imgs[img].mx + unit_mcus - 1) / unit_mcus, n = per_row * ((imgs[img].my + unit_rows - 1) / unit_rows);
     Unit* dst = units + prefix[blockIdx.x];
     for (uint32_t j = threadIdx.x; j < n; j += 128) {
@@ -428,6 +471,8 @@ void free_device(pcr_record* r) {
     }
     for (auto& b : r->bufs) dev_release(b.first, b.second, r->device);
     r->bufs.clear();
+    for (auto& b : r->stages) host_release(b.first, b.second);
+    r->stages.clear();
 }
 
 template <class T>
@@ -438,14 +483,29 @@ int take(pcr_record* r, T** dst, size_t bytes) {
     return PCR_OK;
 }
 
-template <class T>
-int upload(pcr_record* r, T** dst, const std::vector<T>& v) {
-    size_t n = std::max<size_t>(v.size(), 1) * sizeof(T);
-    if (int rc = take(r, dst, n)) return rc;
-    // pageable source: the call returns once the bytes sit in the driver's staging memory
-    if (!v.empty() && cudaMemcpyAsync(*dst, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, r->up_stream) != cudaSuccess) return PCR_E_CUDA;
-    return PCR_OK;
-}
+// A run of tables laid out one behind the other, alike in a page-locked host block and on the device.
+struct Tables {
+    size_t bytes = 0;
+    uint8_t *host = nullptr, *dev = nullptr;
+    size_t add(size_t n) { const size_t at = bytes; bytes = (bytes + std::max<size_t>(n, 1) + 15) & ~(size_t)15; return at; }
+    template <class T> T* h(size_t at) const { return reinterpret_cast<T*>(host + at); }
+    template <class T> T* d(size_t at) const { return reinterpret_cast<T*>(dev + at); }
+    std::unique_ptr<uint8_t[]> pageable;              // (no device: the record is still validated)
+    int allocate(pcr_record* r, bool on_device = true) {
+        if (!on_device) {
+            pageable.reset(new uint8_t[bytes]);
+            host = pageable.get();
+            return PCR_OK;
+        }
+        host = static_cast<uint8_t*>(host_alloc(bytes));
+        if (!host) return PCR_E_NOMEM;
+        r->stages.push_back({host, bytes});
+        return take(r, &dev, bytes);
+    }
+    int copy(pcr_record* r, size_t n) const {
+        return !n || cudaMemcpyAsync(dev, host, n, cudaMemcpyHostToDevice, r->up_stream) == cudaSuccess ? PCR_OK : PCR_E_CUDA;
+    }
+};
 
 int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     if (len < 64 || len >= (1ull << 32)) return PCR_E_FORMAT;
@@ -465,17 +525,27 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
         if (r->group_end[g] < r->group_end[g - 1] || r->group_end[g] > len) return PCR_E_FORMAT;
     const uint8_t* chunk = rec + index_off + 8ull * (G + 1);
 
-    std::vector<ScanDesc> scans((size_t)G * N);
-    std::vector<ImgDesc> imgs(N);
-    std::vector<uint16_t> qtab((size_t)N * 192);
+    const bool on_device = cudaGetDevice(&r->device) == cudaSuccess;
+    if (on_device && !(r->up_stream = pool_stream_get(r->device))) return PCR_E_CUDA;
+    Tables T;
+    const size_t at_script = T.add(sizeof(ScanScript) * G), at_saux = T.add(sizeof(ScanAux) * G), at_scans = T.add(sizeof(ScanDesc) * G * N),
+                 at_imgs = T.add(sizeof(ImgDesc) * N), at_qtab = T.add(384ull * N), at_prefix = T.add(4ull * (N + 1)), at_order = T.add(4ull * N),
+                 at_base = T.add(4ull * G * N), at_group = T.add(12ull * N), at_long = T.add(4ull * G * N);
+    if (int rc = T.allocate(r, on_device)) return rc;
+    ScanDesc* const scans = T.h<ScanDesc>(at_scans);
+    ImgDesc* const imgs = T.h<ImgDesc>(at_imgs);
+    uint16_t* const qtab = T.h<uint16_t>(at_qtab);
     r->info.resize(N); r->blk_base.resize(N); r->nblk.resize(N);
     r->script.resize(G);
     // every image's chunks are walked independently (a few host threads for large records); the
     // running sums over images follow in one serial pass
-    std::vector<ScanScript> scripts((size_t)N * G);
-    std::vector<uint8_t> samplings(N, 0);
+    std::vector<uint32_t> nsegs((size_t)G * N), image_bytes(N);      // restart intervals by (scan, image); entropy-coded bytes
+    std::vector<uint8_t> one_interval(N, 0);                         // some scan of the image is one restart interval
+    uint8_t sampling0 = 0;
     auto parse_image = [&](uint32_t i) -> int {
         ImageParse im;
+        ScanScript script[64];
+        uint32_t sum = 0;
         const uint8_t* m = rec + meta_off + 16ull * i;
         for (uint32_t g = 0; g < G; ++g) {
             const uint8_t* c = chunk + 16ull * ((uint64_t)g * N + i);
@@ -487,7 +557,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
             ScanParse sp;
             int rc = parse_chunk(rec, off, clen, g == 0, im, sp);
             if (rc) return rc;
-            scripts[(size_t)i * G + g] = sp.sc;
+            script[g] = sp.sc;
             ScanDesc& sd = scans[(size_t)g * N + i];
             sd.data_off = sp.data_off; sd.data_end = sp.data_end; sd.ri = sp.ri;
             // up to two distinct tables per scan
@@ -513,14 +583,21 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
                 total_mcu = (uint64_t)((wc + 7) / 8) * ((hc + 7) / 8);
             }
             sd.nseg = sd.ri ? (uint32_t)((total_mcu + sd.ri - 1) / sd.ri) : 1u;
+            nsegs[(size_t)g * N + i] = sd.nseg;
+            if (sd.nseg == 1) one_interval[i] = 1;
+            sum += sd.data_end - sd.data_off;
         }
+        image_bytes[i] = sum;
         if (!im.have_frame) return PCR_E_FORMAT;
         if (rd32(m + 4) != im.W || rd32(m + 8) != im.H) return PCR_E_FORMAT;   // metadata and frame header agree
         for (int c = 0; c < im.nc; ++c) {
             if (!im.qdef[im.tq[c]]) return PCR_E_FORMAT;
             memcpy(&qtab[(size_t)i * 192 + 64 * c], im.q[im.tq[c]], 128);
         }
-        samplings[i] = (uint8_t)(im.hs | (im.vs << 2) | (im.nc << 4));
+        // one script and one sampling per record: the first image's
+        const uint8_t samp = (uint8_t)(im.hs | (im.vs << 2) | (im.nc << 4));
+        if (i == 0) { sampling0 = samp; std::copy(script, script + G, r->script.begin()); }
+        else if (samp != sampling0 || memcmp(script, r->script.data(), sizeof(ScanScript) * G) != 0) return PCR_E_FORMAT;
         pcr_image_info& inf = r->info[i];
         inf.width = im.W; inf.height = im.H; inf.label = (int32_t)rd32(m); inf.rsvd = 0;
         inf.out_bytes = 3ull * im.W * im.H;
@@ -530,14 +607,32 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     };
     {
         const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
-        const unsigned nthreads = N >= 256 ? std::min(4u, hw) : 1u;
+        const unsigned nthreads = std::min({8u, hw, N / 64 + 1u});
         std::vector<int> rcs(nthreads, PCR_OK);
-        auto work = [&](unsigned t) {
-            for (uint32_t i = t; i < N; i += nthreads) {
-                const int rc = parse_image(i);
-                if (rc != PCR_OK) { rcs[t] = rc; return; }
+        // The heads of an image's chunks lie all over the record: those of the next image are requested while
+        // one is walked (the walk waited for memory most of its time).
+        auto request = [&](uint32_t i) {
+            for (uint32_t g = 0; g < G; ++g) {
+                const uint64_t off = rd64(chunk + 16ull * ((uint64_t)g * N + i));
+                if (off >= len) continue;
+                const uint8_t* p = rec + off;
+                for (size_t b = 0; b < (g == 0 ? 384u : 128u) && off + b < len; b += 64) __builtin_prefetch(p + b);
             }
         };
+        std::atomic<uint32_t> next_image{1};
+        auto work = [&](unsigned t) {                    // (runs of images: the first threads work while the others start)
+            for (;;) {
+                const uint32_t i0 = next_image.fetch_add(16), i1 = std::min(N, i0 + 16);
+                if (i0 >= N) return;
+                request(i0);
+                for (uint32_t i = i0; i < i1; ++i) {
+                    if (i + 1 < i1) request(i + 1);
+                    const int rc = parse_image(i);
+                    if (rc != PCR_OK) { rcs[t] = rc; return; }
+                }
+            }
+        };
+        if (const int rc = parse_image(0)) return rc;
         std::vector<std::thread> pool;
         for (unsigned t = 1; t < nthreads; ++t) pool.emplace_back(work, t);
         work(0);
@@ -545,25 +640,26 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
         for (int rc : rcs) if (rc != PCR_OK) return rc;
     }
     uint64_t blocks = 0, out_off = 0, segs = 0;
-    r->hs = samplings[0] & 3; r->vs = (samplings[0] >> 2) & 3; r->nc = samplings[0] >> 4;
+    r->hs = sampling0 & 3; r->vs = (sampling0 >> 2) & 3; r->nc = sampling0 >> 4;
     const uint32_t bpm = (uint32_t)(r->hs * r->vs + (r->nc == 3 ? 2 : 0));      // blocks per MCU
     r->unit_mcus = kUnitMcus[sampling_code(r->hs, r->vs, r->nc)];
     r->unit_rows = kUnitRows[sampling_code(r->hs, r->vs, r->nc)];
-    for (uint32_t g = 0; g < G; ++g) r->script[g] = scripts[g];
+    uint64_t max_items = 1;
+    uint32_t* const seg_base = T.h<uint32_t>(at_base);
+    for (size_t j = 0; j < (size_t)G * N; ++j) {
+        seg_base[j] = (uint32_t)segs;
+        segs += (uint64_t)nsegs[j] + 1;               // one closing entry per (scan, image)
+        if (segs >= (1ull << 32)) return PCR_E_FORMAT;
+        max_items += nsegs[j] / kSegsPerItem + 1 + nsegs[j] / (kSegsPerItem / 2) + 1;     // (the pairs' items too)
+    }
+    bool single = false;                              // any scan of any image is one restart interval
     for (uint32_t i = 0; i < N; ++i) {
-        if (i && memcmp(&scripts[(size_t)i * G], &scripts[0], sizeof(ScanScript) * G) != 0) return PCR_E_FORMAT;   // one script per record
-        for (uint32_t g = 0; g < G; ++g) {
-            ScanDesc& sd = scans[(size_t)g * N + i];
-            sd.seg_base = (uint32_t)segs;
-            segs += sd.nseg + 1;                      // one closing entry per (scan, image)
-            if (segs >= (1ull << 32)) return PCR_E_FORMAT;
-        }
+        single = single || one_interval[i];
         pcr_image_info& inf = r->info[i];
         inf.out_offset = out_off;
         out_off += (inf.out_bytes + 127) & ~127ull;
         if (imgs[i].W & 15u) r->widths_mult16 = false;
         r->dc_refine_chunks = std::max(r->dc_refine_chunks, std::min(8u, (imgs[i].mx * imgs[i].my + 255u) / 256u));
-        if (samplings[i] != samplings[0]) return PCR_E_FORMAT;                                  // one sampling per record
         r->blk_base[i] = blocks; r->nblk[i] = (uint64_t)bpm * imgs[i].mx * imgs[i].my;
         imgs[i].blk_base = blocks; imgs[i].out_off = inf.out_offset;
         blocks += r->nblk[i];
@@ -571,6 +667,59 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     // 16 spare bytes behind the last image: the tensor epilogue reads pixels as aligned words and may
     // touch up to 8 bytes past a pixel pair
     r->total_blocks = blocks; r->out_bytes = out_off + 16; r->total_segs = segs;
+
+    // side data of the AC scans: one word per block for a first pass, four for a refinement
+    const uint64_t total_mcus = blocks / bpm;
+    uint64_t aux_words = 0;
+    r->saux.assign(G, ScanAux{});
+    int n_refine[3] = {0, 0, 0};
+    for (uint32_t s = 0; s < G; ++s)
+        if (r->script[s].Ss > 0 && r->script[s].Ah > 0 && ++n_refine[r->script[s].comp[0]] > 4) return PCR_E_FORMAT;
+    uint64_t n_tabs = 0;
+    for (uint32_t s = 0; s < G; ++s) {
+        const ScanScript& sc = r->script[s];
+        ScanAux& ax = r->saux[s];
+        ax.ntab = sc.Ss > 0 ? 1 : (sc.Se == 63 ? 4 : (sc.Ah == 0 ? 2 : 0));
+        ax.tab0 = (uint32_t)n_tabs;
+        n_tabs += (uint64_t)N * (uint64_t)ax.ntab;
+        if (sc.Ss == 0 && sc.Se != 63) continue;
+        ax.stride = sc.Ah ? 4u : (sc.Se >= 8 ? 2u : 1u);
+        ax.base = aux_words;
+        if (sc.Ss == 0) { aux_words += 2 * blocks; continue; }
+        aux_words += (sc.comp[0] == 0 ? (uint64_t)(r->hs * r->vs) : 1ull) * total_mcus * ax.stride;
+        aux_words = (aux_words + 1) & ~1ull;      // 16-byte alignment of every scan's area
+        if (sc.Ah) {
+            // positions already non-zero = union of the masks of earlier scans on this band; an
+            // earlier scan is covered by a later refinement whose band contains its own
+            std::vector<int> src;
+            for (uint32_t t = 0; t < s; ++t) {
+                const ScanScript& st = r->script[t];
+                if (st.Ss == 0 || st.comp[0] != sc.comp[0] || st.Ss > sc.Se || sc.Ss > st.Se) continue;
+                src.push_back((int)t);
+            }
+            std::vector<int> keep;
+            for (int t : src) {
+                bool covered = false;
+                for (int u : src)
+                    if (u > t && r->script[u].Ah && r->script[u].Ss <= r->script[t].Ss && r->script[u].Se >= r->script[t].Se) covered = true;
+                if (!covered) keep.push_back(t);
+            }
+            if (keep.empty() || keep.size() > 4) return PCR_E_FORMAT;
+            ax.nsrc = (int)keep.size();
+            for (size_t i = 0; i < keep.size(); ++i) ax.src[i] = keep[i];
+        }
+    }
+
+    // What has to be zero lies together; zeroing it (0.1 ms for 1024 ImageNet-shaped images) passes beside the rest of this call.
+    Tables Z;
+    const size_t at_aux = Z.add((size_t)aux_words * 8), at_ubuf = Z.add(len + 256), at_dc = Z.add((size_t)blocks * 2), at_head = Z.add((size_t)blocks * 16),
+                 at_seg = Z.add((size_t)(segs + 1) * 4), at_status = Z.add((size_t)N * 4), at_sync = Z.add((4 + 12 * (size_t)N) * 4);
+    if (on_device) {
+        if (int rc = take(r, &Z.dev, Z.bytes)) return rc;
+        r->d_aux = Z.d<uint64_t>(at_aux); r->d_ubuf = Z.d<uint8_t>(at_ubuf); r->d_dc = Z.d<int16_t>(at_dc); r->d_head = Z.d<int16_t>(at_head);
+        r->d_seg = Z.d<uint32_t>(at_seg); r->d_status = Z.d<int>(at_status); r->d_chain_sync = Z.d<uint32_t>(at_sync);
+        if (cudaMemsetAsync(Z.dev, 0, Z.bytes, r->up_stream) != cudaSuccess) return PCR_E_CUDA;
+    }
 
     // dependency waves of the script: a scan waits for every earlier scan that touches an
     // overlapping coefficient band of one of its components
@@ -643,25 +792,24 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     // entropy-coded bytes per MCU row, most first: the slice of the heaviest rows starts first, slices
     // of light images finish their waves early and their pixel stage overlaps the waves of the heavy
     // ones.  (By width alone, the first version of this order: 2 % slower on the ImageNet-shaped record.)
-    std::vector<uint32_t> order(N);
+    uint32_t* const order = T.h<uint32_t>(at_order);
     for (uint32_t i = 0; i < N; ++i) order[i] = i;
     if (r->n_slices > 1) {
         std::vector<double> key(N);
-        for (uint32_t i = 0; i < N; ++i) {
-            uint64_t b = 0;
-            for (uint32_t s2 = 0; s2 < G; ++s2) b += scans[(size_t)s2 * N + i].data_end - scans[(size_t)s2 * N + i].data_off;
-            key[i] = (double)b / (double)std::max<uint32_t>(1, imgs[i].my);
-        }
-        std::stable_sort(order.begin(), order.end(), [&](uint32_t a, uint32_t b) { return key[a] > key[b]; });
+        for (uint32_t i = 0; i < N; ++i) key[i] = (double)image_bytes[i] / (double)std::max<uint32_t>(1, imgs[i].my);
+        std::stable_sort(order, order + N, [&](uint32_t a, uint32_t b) { return key[a] > key[b]; });
     }
-    std::vector<Item> items;
-    items.reserve((size_t)(segs / 24 + (uint64_t)N * G));
+    Tables TI;
+    TI.add(sizeof(Item) * max_items);
+    if (int rc = TI.allocate(r, on_device)) return rc;
+    Item* const items = TI.h<Item>(0);
+    uint32_t n_items = 0;
     r->item_begin.assign((size_t)r->n_slices * G, 0); r->item_count.assign((size_t)r->n_slices * G, 0);
     // A scan that is one restart interval of at least this many bytes goes to the kernels for long
     // intervals; DC refinement scans have a kernel of their own and no items at all.
     uint32_t long_min = 64;
     if (const char* e = getenv("PCR_LONG_MIN_BYTES")) long_min = (uint32_t)std::max(0, atoi(e));
-    auto is_long = [&](int s, uint32_t i) {
+    auto ik0ng = [&](int s, uint32_t i) {
         const ScanScript& sc = r->script[s];
         const ScanDesc& sd = scans[(size_t)s * N + i];
         (void)sc;
@@ -670,7 +818,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     // the AC refinements of one component of one image go together: all of them one interval each,
     // at least one of them long
     std::vector<uint8_t> grouped((size_t)N * 3, 0);
-    for (uint32_t i = 0; i < N; ++i)
+    for (uint32_t i = 0; single && i < N; ++i)
         for (int c = 0; c < 3; ++c) {
             bool any = false, one_interval = true, big = false;
             for (uint32_t s = 0; s < G; ++s) {
@@ -679,31 +827,32 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
                 any = true;
                 const ScanDesc& sd = scans[(size_t)s * N + i];
                 one_interval = one_interval && sd.nseg == 1 && sd.data_end - sd.data_off < (1u << 27);
-                big = big || is_long((int)s, i);
+                big = big || ik0ng((int)s, i);
             }
             grouped[(size_t)i * 3 + c] = any && one_interval && big;
         }
-    auto takes_long_kernel = [&](int s, uint32_t i) {
+    auto takek0ng_kernel = [&](int s, uint32_t i) {
         const ScanScript& sc = r->script[s];
         if (sc.Ss > 0 && sc.Ah != 0) return grouped[(size_t)i * 3 + sc.comp[0]] != 0;
-        return is_long(s, i);
+        return ik0ng(s, i);
     };
-    std::vector<uint32_t> longs, groups;
+    uint32_t *const longs = T.h<uint32_t>(at_long), *const groups = T.h<uint32_t>(at_group);
+    uint32_t n_longs = 0, n_groups = 0;
     r->long_begin.assign((size_t)r->n_slices * G, 0); r->long_count.assign((size_t)r->n_slices * G, 0);
     for (int g = 0; g < r->n_slices; ++g) {
         for (int w = 0; w < r->n_waves; ++w)
             for (int s : r->wave_scans[w]) {
                 const ScanScript& sc = r->script[s];
                 if (sc.Ah != 0) continue;                      // first passes only
-                r->long_begin[(size_t)g * G + s] = (uint32_t)longs.size();
-                for (uint32_t pos = r->slice_img[g]; pos < r->slice_img[g + 1]; ++pos)
-                    if (is_long(s, order[pos])) longs.push_back((uint32_t)(s * N + order[pos]));
-                r->long_count[(size_t)g * G + s] = (uint32_t)longs.size() - r->long_begin[(size_t)g * G + s];
+                r->long_begin[(size_t)g * G + s] = n_longs;
+                for (uint32_t pos = r->slice_img[g]; single && pos < r->slice_img[g + 1]; ++pos)
+                    if (ik0ng(s, order[pos])) longs[n_longs++] = (uint32_t)(s * N + order[pos]);
+                r->long_count[(size_t)g * G + s] = n_longs - r->long_begin[(size_t)g * G + s];
             }
     }
     // one list for the whole record: luminance first (its chains are the longest), within a
     // component the images with the most refinement bytes first
-    for (int c = 0; c < 3; ++c) {
+    for (int c = 0; single && c < 3; ++c) {
         std::vector<std::pair<uint64_t, uint32_t>> byw;
         for (uint32_t i = 0; i < N; ++i) {
             if (!grouped[(size_t)i * 3 + c]) continue;
@@ -715,56 +864,58 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
             byw.push_back({bytes, i});
         }
         std::stable_sort(byw.begin(), byw.end(), [](const std::pair<uint64_t, uint32_t>& a, const std::pair<uint64_t, uint32_t>& b) { return a.first > b.first; });
-        for (auto& e : byw) groups.push_back(((uint32_t)c << 28) | e.second);
+        for (auto& e : byw) groups[n_groups++] = ((uint32_t)c << 28) | e.second;
     }
-    r->n_groups = (uint32_t)groups.size();
+    r->n_groups = n_groups;
     for (int g = 0; g < r->n_slices; ++g)
         for (int w = 0; w < r->n_waves; ++w)
             for (int s : r->wave_scans[w]) {
-                r->item_begin[(size_t)g * G + s] = (uint32_t)items.size();
+                const uint32_t begin = n_items;
+                const uint32_t* const ns = &nsegs[(size_t)s * N];
                 const bool ac = r->script[s].Ss > 0;
                 const bool dc_refine = r->script[s].Ss == 0 && r->script[s].Ah != 0;
+                Item* open = nullptr;                         // an unfilled last item that the next image may extend
                 for (uint32_t pos = r->slice_img[g]; pos < r->slice_img[g + 1] && !dc_refine; ++pos) {
                     const uint32_t i = order[pos];
-                    if (takes_long_kernel((int)s, i)) continue;
-                    const ScanDesc& sd = scans[(size_t)s * N + i];
+                    if (single && takek0ng_kernel((int)s, i)) continue;
+                    const uint32_t nseg = ns[i], si = (uint32_t)(s * N + i);
                     // full warps of 32 restart intervals; in AC scans the last warp of an image
                     // runs on into the first intervals of the next image (two tables per warp)
                     uint32_t j = 0;
-                    if (ac && !items.empty() && items.back().next == kItemOpen) {     // continued from the previous image
-                        Item& prev = items.back();
-                        const uint32_t take = std::min<uint32_t>(kSegsPerItem - prev.count, sd.nseg);
-                        prev.count += take; prev.next = (uint32_t)(s * N + i) + 1u;
-                        j = take;
+                    if (open) {                               // continued from the previous image
+                        j = std::min<uint32_t>(kSegsPerItem - open->count, nseg);
+                        open->count += j; open->next = si + 1u;
+                        open = nullptr;
                     }
-                    for (; j < sd.nseg; j += kSegsPerItem) {
-                        const uint32_t cnt = std::min<uint32_t>(kSegsPerItem, sd.nseg - j);
-                        // kItemOpen marks an unfilled last item that the next image may extend
-                        items.push_back(Item{(uint32_t)(s * N + i), j, cnt, (ac && cnt < (uint32_t)kSegsPerItem) ? kItemOpen : 0u, 0u});
+                    for (; j < nseg; j += kSegsPerItem) {
+                        const uint32_t cnt = std::min<uint32_t>(kSegsPerItem, nseg - j);
+                        items[n_items] = Item{si, j, cnt, 0u, 0u};
+                        open = ac && cnt < (uint32_t)kSegsPerItem ? &items[n_items] : nullptr;
+                        ++n_items;
                     }
                 }
-                if (!items.empty() && items.back().next == kItemOpen) items.back().next = 0;
-                r->item_count[(size_t)g * G + s] = (uint32_t)items.size() - r->item_begin[(size_t)g * G + s];
+                r->item_begin[(size_t)g * G + s] = begin;
+                r->item_count[(size_t)g * G + s] = n_items - begin;
             }
     // the pairs' items: sixteen intervals of one image
     r->pair_begin.assign((size_t)r->n_slices * G, 0); r->pair_count.assign((size_t)r->n_slices * G, 0);
     for (int g = 0; g < r->n_slices; ++g)
         for (uint32_t s = 0; s < G; ++s) {
-            r->pair_begin[(size_t)g * G + s] = (uint32_t)items.size();
+            const uint32_t begin = n_items;
             for (uint32_t pos = r->slice_img[g]; r->pair_of[s] >= 0 && pos < r->slice_img[g + 1]; ++pos) {
                 const uint32_t i = order[pos], a = (uint32_t)r->pair_of[s];
-                if (takes_long_kernel((int)s, i)) continue;
-                const uint32_t nseg = scans[(size_t)s * N + i].nseg;
+                if (single && takek0ng_kernel((int)s, i)) continue;
+                const uint32_t nseg = nsegs[(size_t)s * N + i];
                 for (uint32_t j = 0; j < nseg; j += kSegsPerItem / 2)
-                    items.push_back(Item{a * N + i, j, std::min<uint32_t>(kSegsPerItem / 2, nseg - j), 0u, (s - a) * N});
+                    items[n_items++] = Item{a * N + i, j, std::min<uint32_t>(kSegsPerItem / 2, nseg - j), 0u, (s - a) * N};
             }
-            r->pair_count[(size_t)g * G + s] = (uint32_t)items.size() - r->pair_begin[(size_t)g * G + s];
+            r->pair_begin[(size_t)g * G + s] = begin;
+            r->pair_count[(size_t)g * G + s] = n_items - begin;
         }
     // Pairs shorten the chain but leave the lanes of the shorter scan idle (about 1.4 times the warp instructions for the
     // ten-scan script), so they are for records whose waves fit the machine at once (18 warps an SM): 96 images of
     // 4:4:4 552 -> 434 us, 512 ImageNet-shaped images raised 2 -> 10 797 -> 768, 1024 of them at k = 10 991 -> 1022.
-    if (cudaGetDevice(&r->device) != cudaSuccess) return PCR_E_CUDA;
-    if (cudaDeviceGetAttribute(&r->n_sms, cudaDevAttrMultiProcessorCount, r->device) != cudaSuccess) return PCR_E_CUDA;
+    if (on_device && cudaDeviceGetAttribute(&r->n_sms, cudaDevAttrMultiProcessorCount, r->device) != cudaSuccess) return PCR_E_CUDA;
     for (const std::vector<int>& scans_of_wave : r->paired_waves) {
         std::vector<char> in_pair(G, 0);
         for (int s : scans_of_wave) if (r->pair_of[s] >= 0) in_pair[s] = in_pair[r->pair_of[s]] = 1;
@@ -779,7 +930,8 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     }
     // pixel work units (see Sampling in pcr_pixels.cuh), image by image in processing order, inside an image
     // MCU row by MCU row.  The host only counts them; a small kernel writes the list at set-up.
-    std::vector<uint32_t> unit_prefix(N + 1, 0);
+    uint32_t* const unit_prefix = T.h<uint32_t>(at_prefix);
+    unit_prefix[0] = 0;
     for (uint32_t pos = 0; pos < N; ++pos) {
         const ImgDesc& im = imgs[order[pos]];
         if (im.my > 65535 || im.mx > 65535) return PCR_E_FORMAT;
@@ -791,88 +943,23 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     for (int g = 0; g <= r->n_slices; ++g) r->slice_unit[g] = unit_prefix[r->slice_img[g]];
     r->n_units = unit_prefix[N];
 
-    // side data of the AC scans: one word per block for a first pass, four for a refinement
-    const uint64_t total_mcus = blocks / bpm;
-    uint64_t aux_words = 0;
-    r->saux.assign(G, ScanAux{});
-    int n_refine[3] = {0, 0, 0};
-    for (uint32_t s = 0; s < G; ++s)
-        if (r->script[s].Ss > 0 && r->script[s].Ah > 0 && ++n_refine[r->script[s].comp[0]] > 4) return PCR_E_FORMAT;
-    uint64_t n_tabs = 0;
-    for (uint32_t s = 0; s < G; ++s) {
-        const ScanScript& sc = r->script[s];
-        ScanAux& ax = r->saux[s];
-        ax.ntab = sc.Ss > 0 ? 1 : (sc.Se == 63 ? 4 : (sc.Ah == 0 ? 2 : 0));
-        ax.tab0 = (uint32_t)n_tabs;
-        n_tabs += (uint64_t)N * (uint64_t)ax.ntab;
-        if (sc.Ss == 0 && sc.Se != 63) continue;
-        ax.stride = sc.Ah ? 4u : (sc.Se >= 8 ? 2u : 1u);
-        ax.base = aux_words;
-        if (sc.Ss == 0) { aux_words += 2 * blocks; continue; }
-        aux_words += (sc.comp[0] == 0 ? (uint64_t)(r->hs * r->vs) : 1ull) * total_mcus * ax.stride;
-        aux_words = (aux_words + 1) & ~1ull;      // 16-byte alignment of every scan's area
-        if (sc.Ah) {
-            // positions already non-zero = union of the masks of earlier scans on this band; an
-            // earlier scan is covered by a later refinement whose band contains its own
-            std::vector<int> src;
-            for (uint32_t t = 0; t < s; ++t) {
-                const ScanScript& st = r->script[t];
-                if (st.Ss == 0 || st.comp[0] != sc.comp[0] || st.Ss > sc.Se || sc.Ss > st.Se) continue;
-                src.push_back((int)t);
-            }
-            std::vector<int> keep;
-            for (int t : src) {
-                bool covered = false;
-                for (int u : src)
-                    if (u > t && r->script[u].Ah && r->script[u].Ss <= r->script[t].Ss && r->script[u].Se >= r->script[t].Se) covered = true;
-                if (!covered) keep.push_back(t);
-            }
-            if (keep.empty() || keep.size() > 4) return PCR_E_FORMAT;
-            ax.nsrc = (int)keep.size();
-            for (size_t i = 0; i < keep.size(); ++i) ax.src[i] = keep[i];
-        }
-    }
-
-    // device state
-    if (!(r->up_stream = pool_stream_get(r->device))) return PCR_E_CUDA;
-    if (int rc = take(r, &r->d_aux, (size_t)(std::max<uint64_t>(aux_words, 2) * 8))) return rc;
-    // zeroing is enqueued after the table uploads: a copy from pageable memory first waits for
-    // everything already in its stream
-    std::vector<std::pair<void*, size_t>> zero;
-    zero.push_back({r->d_aux, (size_t)(std::max<uint64_t>(aux_words, 2) * 8)});
+    if (!on_device) return PCR_E_CUDA;
+    // the rest of the device state
+    std::copy(r->script.begin(), r->script.end(), T.h<ScanScript>(at_script));
+    std::copy(r->saux.begin(), r->saux.end(), T.h<ScanAux>(at_saux));
     if (int rc = take(r, &r->d_rec, (size_t)(len + 64))) return rc;
-    if (int rc = take(r, &r->d_ubuf, (size_t)(len + 256))) return rc;
-    zero.push_back({r->d_ubuf, len + 256});
     if (int rc = take(r, &r->d_tabs, (size_t)(std::max<uint64_t>(n_tabs, 1) * sizeof(ScanTab)))) return rc;
     if (int rc = take(r, &r->d_vals, (size_t)(8 * (len + 256)))) return rc;      // four values per byte, two bytes each
-    if (int rc = take(r, &r->d_dc, (size_t)(std::max<uint64_t>(blocks, 1) * 2))) return rc;
-    zero.push_back({r->d_dc, (size_t)(std::max<uint64_t>(blocks, 1) * 2)});
-    if (int rc = take(r, &r->d_head, (size_t)(std::max<uint64_t>(blocks, 1) * 16))) return rc;
-    zero.push_back({r->d_head, (size_t)(std::max<uint64_t>(blocks, 1) * 16)});
-    if (int rc = take(r, &r->d_seg, (size_t)((segs + 1) * 4))) return rc;
-    if (int rc = take(r, &r->d_status, (size_t)((size_t)N * 4))) return rc;
-    zero.push_back({r->d_seg, (size_t)((segs + 1) * 4)});
-    zero.push_back({r->d_status, (size_t)N * 4});
-    int rc;
-    if ((rc = upload(r, &r->d_script, r->script))) return rc;
-    if ((rc = upload(r, &r->d_saux, r->saux))) return rc;
-    if ((rc = upload(r, &r->d_scans, scans))) return rc;
-    if ((rc = upload(r, &r->d_imgs, imgs))) return rc;
-    if ((rc = upload(r, &r->d_items, items))) return rc;
-    if ((rc = upload(r, &r->d_long, longs))) return rc;
-    if ((rc = upload(r, &r->d_group, groups))) return rc;
-    if (r->n_groups) {
-        if ((rc = take(r, &r->d_chain_sync, (size_t)(4 + 4 * (size_t)r->n_groups) * 4))) return rc;
-        if (cudaFuncSetAttribute(ac_refine_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kChainPairs * sizeof(ChainShared))) != cudaSuccess) return PCR_E_CUDA;
-    }
-    if ((rc = upload(r, &r->d_qtab, qtab))) return rc;
-    if ((rc = upload(r, &r->d_unit_prefix, unit_prefix))) return rc;
-    if ((rc = take(r, &r->d_units, (size_t)std::max<uint32_t>(r->n_units, 1) * sizeof(Unit)))) return rc;
-    if ((rc = upload(r, &r->d_order, order))) return rc;
-    units_kernel<<<N, 128, 0, r->up_stream>>>(r->d_imgs, r->d_order, r->d_unit_prefix, r->d_units, r->unit_mcus, r->unit_rows);
+    if (int rc = take(r, &r->d_units, (size_t)std::max<uint32_t>(r->n_units, 1) * sizeof(Unit))) return rc;
+    r->d_script = T.d<ScanScript>(at_script); r->d_saux = T.d<ScanAux>(at_saux); r->d_scans = T.d<ScanDesc>(at_scans); r->d_imgs = T.d<ImgDesc>(at_imgs);
+    r->d_qtab = T.d<uint16_t>(at_qtab); r->d_unit_prefix = T.d<uint32_t>(at_prefix); r->d_order = T.d<uint32_t>(at_order);
+    r->d_group = T.d<uint32_t>(at_group); r->d_long = T.d<uint32_t>(at_long); r->d_items = TI.d<Item>(0);
+    if (int rc = T.copy(r, at_long + 4ull * n_longs)) return rc;
+    if (int rc = TI.copy(r, sizeof(Item) * (size_t)n_items)) return rc;
+    units_kernel<<<N, 128, 0, r->up_stream>>>(r->d_imgs, r->d_order, r->d_unit_prefix, r->d_units, r->unit_mcus, r->unit_rows,
+                                              r->d_scans, T.d<uint32_t>(at_base), G);
     ++g_launches;
-    for (auto& z : zero)
-        if (cudaMemsetAsync(z.first, 0, z.second, r->up_stream) != cudaSuccess) return PCR_E_CUDA;
+    if (n_groups && cudaFuncSetAttribute(ac_refine_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kChainPairs * sizeof(ChainShared))) != cudaSuccess) return PCR_E_CUDA;
     r->h_status.assign(N, 0);
     r->resident = 0;
     if (!(r->ev_done = pool_event_get(r->device))) return PCR_E_CUDA;
@@ -1062,8 +1149,8 @@ static void launch_pixels_sampled(const PixelPlan& pl, unsigned grid, cudaStream
 template <bool kRoi>
 static void launch_pixels_420(const PixelPlan& pl, unsigned grid, cudaStream_t q, const Params& Q, const CoefLists& cl, uint8_t* o8) {
     constexpr int T = unit_threads<kSamp420>();
-    if (pl.dc_only && pl.widths_mult16) dc_pixel_kernel<kRoi><<<grid, 128, 0, q>>>(Q, o8);
-    else if (pl.dc_only) dc_pixel_kernel<kRoi, false><<<grid, 128, 0, q>>>(Q, o8);
+    if (pl.dc_only && pl.widths_mult16) dc_pixel_kernel<kRoi><<<grid, 128, 0, q>>>(Q, make_uint3(cl.dc_mask[0], cl.dc_mask[1], cl.dc_mask[2]), o8);
+    else if (pl.dc_only) dc_pixel_kernel<kRoi, false><<<grid, 128, 0, q>>>(Q, make_uint3(cl.dc_mask[0], cl.dc_mask[1], cl.dc_mask[2]), o8);
     else if (pl.head_only) pixel_kernel<false, 3, kRoi><<<grid, T, 0, q>>>(Q, cl, o8);
     else if (pl.refine) pixel_kernel<true, 1, kRoi><<<grid, T, 0, q>>>(Q, cl, o8);
     else pixel_kernel<false, 1, kRoi><<<grid, T, 0, q>>>(Q, cl, o8);
@@ -1116,7 +1203,9 @@ static void coef_lists(const pcr_record* rec, int k, CoefLists* cl) {
     for (int s = 0; s < k; ++s) {
         const ScanScript& sc = rec->script[s];
         const ScanAux& ax = rec->saux[s];
-        if (sc.Ss == 0 && sc.Se != 63) continue;                   // DC scans: the DC plane
+        if (sc.Ss == 0)                                            // the DC plane
+            for (int q = 0; q < sc.ncomp; ++q) cl->dc_mask[sc.comp[q]] = 0xFFFFu & ~((1u << sc.Al) - 1u);
+        if (sc.Ss == 0 && sc.Se != 63) continue;
         for (int i = 0; i < sc.ncomp; ++i) {
             const int c = sc.comp[i];
             for (int p = std::max(1, sc.Ss); p <= std::min(7, sc.Se); ++p) mask[c][p] = 0xFFFFu;
@@ -1138,19 +1227,22 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const size_t need = (size_t)rec->group_end[k];
     const bool prof = rec->profiling;
-    rec->stages.clear();
+    rec->profile.clear();
     auto mark = [&](const char* name, int launches) {
-        if (!prof || rec->stages.size() + 1 >= rec->events.size()) return;
+        if (!prof || rec->profile.size() + 1 >= rec->events.size()) return;
         pcr_stage_time t;
         memset(&t, 0, sizeof t);
         strncpy(t.name, name, sizeof t.name - 1);
         t.launches = launches;
-        rec->stages.push_back(t);
-        cudaEventRecord(rec->events[rec->stages.size()], st);
+        rec->profile.push_back(t);
+        cudaEventRecord(rec->events[rec->profile.size()], st);
     };
+    const bool pipelined = rec->n_slices > 1 && !prof;
+    // (the copy of missing bytes, on a stream of its own, need not wait for pcr_open's uploads)
+    if (pipelined && rec->resident < need && (cudaEventRecord(rec->ev_fork, st) != cudaSuccess ||
+                                              cudaStreamWaitEvent(rec->copy_stream, rec->ev_fork, 0) != cudaSuccess)) return PCR_E_CUDA;
     if (cudaStreamWaitEvent(st, rec->ev_ready, 0) != cudaSuccess) return PCR_E_CUDA;      // pcr_open's uploads
     if (prof) cudaEventRecord(rec->events[0], st);
-    const bool pipelined = rec->n_slices > 1 && !prof;
     if (!pipelined && rec->resident < need) {
         size_t from = rec->resident & ~(size_t)15;
         if (cudaMemcpyAsync(rec->d_rec + from, rec->host + from, need - from, cudaMemcpyHostToDevice, st) != cudaSuccess) return PCR_E_CUDA;
@@ -1395,7 +1487,6 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
         if (cudaEventRecord(rec->ev_fork, st) != cudaSuccess) return PCR_E_CUDA;
         if (cudaStreamWaitEvent(rec->clear_stream, rec->ev_fork, 0) != cudaSuccess) return PCR_E_CUDA;
         if (rec->resident < need) {
-            if (cudaStreamWaitEvent(rec->copy_stream, rec->ev_fork, 0) != cudaSuccess) return PCR_E_CUDA;
             bool any = false;
             for (int w = 0; w < W; ++w) {
                 size_t upto = 0;
@@ -1475,6 +1566,10 @@ void pcr_release_cached_memory(void) {
     for (auto& kv : g_cache.free_) cudaFree(kv.second);
     g_cache.free_.clear();
     g_cache.cached = 0;
+    std::lock_guard<std::mutex> lh(g_host.mu);
+    for (auto& kv : g_host.free_) cudaFreeHost(kv.second);
+    g_host.free_.clear();
+    g_host.cached = 0;
 }
 
 int pcr_decode(pcr_record* rec, int k, void* out, void* stream) {
@@ -1554,7 +1649,12 @@ int pcr_msssim(pcr_record* rec, const void* rgb_a, const void* rgb_b, void* scra
     if (!rec->d_ms) {
         std::vector<MsDesc> table;
         msssim_layout(rec, &table);
-        if (int rc = upload(rec, &rec->d_ms, table)) return rc;
+        Tables T;
+        T.add(table.size() * sizeof(MsDesc));
+        if (int rc = T.allocate(rec)) return rc;
+        std::copy(table.begin(), table.end(), T.h<MsDesc>(0));
+        if (int rc = T.copy(rec, T.bytes)) return rc;
+        rec->d_ms = T.d<MsDesc>(0);
         if (cudaEventRecord(rec->ev_ready, rec->up_stream) != cudaSuccess) return PCR_E_CUDA;
     }
     if (cudaStreamWaitEvent(st, rec->ev_ready, 0) != cudaSuccess) return PCR_E_CUDA;
@@ -1664,8 +1764,8 @@ int pcr_set_profiling(pcr_record* rec, int enable) {
 int pcr_get_profile(pcr_record* rec, pcr_stage_time* out, int cap, int* n) {
     if (!rec || !out || !n || cap < 0) return PCR_E_ARG;
     *n = 0;
-    for (size_t i = 0; i < rec->stages.size() && (int)i < cap; ++i) {
-        out[i] = rec->stages[i];
+    for (size_t i = 0; i < rec->profile.size() && (int)i < cap; ++i) {
+        out[i] = rec->profile[i];
         if (cudaEventElapsedTime(&out[i].ms, rec->events[i], rec->events[i + 1]) != cudaSuccess) return PCR_E_CUDA;
         ++*n;
     }

@@ -104,7 +104,7 @@ __device__ __forceinline__ void expand_block(const Params& P, const CoefLists& c
     // all of the block's loads are requested before the first is used
     const uint4 zero4 = make_uint4(0, 0, 0, 0);
     uint4 head = __ldg(reinterpret_cast<const uint4*>(P.head + blk * 8));
-    const uint32_t dc = __ldg(reinterpret_cast<const uint16_t*>(P.dc) + blk);
+    const uint32_t dc = __ldg(reinterpret_cast<const uint16_t*>(P.dc) + blk) & cl.dc_mask[comp];
     uint4 rec = zero4;
     const uint64_t at_rec = cl.sequential ? blk : local;
     if (nfirst > 0) rec = __ldg(reinterpret_cast<const uint4*>(P.aux + cl.first[comp][0]) + at_rec);
@@ -265,7 +265,7 @@ pixel_kernel(Params P, CoefLists cl, uint8_t* __restrict__ out) {
         if (kMode == 3) {
             const uint4 hm = cl.head_mask[comp];
             head = __ldg(reinterpret_cast<const uint4*>(P.head + blk * 8));
-            head = make_uint4((head.x & hm.x) | __ldg(reinterpret_cast<const uint16_t*>(P.dc) + blk), head.y & hm.y, head.z & hm.z, head.w & hm.w);
+            head = make_uint4((head.x & hm.x) | (__ldg(reinterpret_cast<const uint16_t*>(P.dc) + blk) & cl.dc_mask[comp]), head.y & hm.y, head.z & hm.z, head.w & hm.w);
         }
         const uint4* dense = reinterpret_cast<const uint4*>(P.planes + blk * 64);
 #pragma unroll
@@ -460,7 +460,7 @@ pixel_kernel(Params P, CoefLists cl, uint8_t* __restrict__ out) {
 // words from the triples of the (at most two) pixels each word covers, and stores the chunk whole
 // when it lies inside the row, byte by byte at the row's two ends.
 template <bool kRoi, bool kAligned = true>
-__global__ void __launch_bounds__(128) dc_pixel_kernel(Params P, uint8_t* __restrict__ out) {
+__global__ void __launch_bounds__(128) dc_pixel_kernel(Params P, uint3 dc_mask, uint8_t* __restrict__ out) {
     constexpr int U = Sampling<kSamp420>::U, R = Sampling<kSamp420>::R;
     __shared__ uint32_t s_tri[2 * R][2 * U];           // [block row of the unit][block column]: R | G << 8 | B << 16
     const int tid = threadIdx.x;
@@ -480,7 +480,7 @@ __global__ void __launch_bounds__(128) dc_pixel_kernel(Params P, uint8_t* __rest
         if (brow >= 2 * r_lo && brow < 2 * r_hi && bcol < 2 * nm) {
             const uint16_t* q = P.qtab + (size_t)un.img * 192;
             auto sample = [&](uint64_t blk, int comp) {
-                const int F = (int)__ldg(P.dc + blk) * (int)q[64 * comp];
+                const int F = (int)(short)((uint32_t)__ldg(P.dc + blk) & (comp == 0 ? dc_mask.x : (comp == 1 ? dc_mask.y : dc_mask.z))) * (int)q[64 * comp];
                 const int T = (int)(K4 * (uint32_t)F + (1u << 11)) >> 12;
                 const int smp = ((int)(K4 * (uint32_t)T + (1u << 15)) >> 16) + 128;
                 return min(max(smp, 0), 255);

@@ -37,6 +37,8 @@ struct ScanAux {
 constexpr int kMaxFirst = 56;      // first passes of a component that reach beyond position 7: at most one per position
 struct CoefLists {
     uint4 head_mask[3];            // positions 1..7 that a decoded scan covers, as 16-bit lanes of the head plane's entries
+    uint32_t dc_mask[3];           // bits of the DC coefficient that a decoded scan covers (a refinement of an earlier
+                                   // decode may have left others in blocks that a damaged stream no longer reaches)
     int32_t n_first[3], n_refine[3];
     int32_t sequential;            // side data indexed by the block's number in the planes, not inside its component
     uint64_t first[3][kMaxFirst];  // first word of the scan's side data (two words per block)
@@ -91,7 +93,6 @@ struct ItemRuns {
     int32_t n;
     uint32_t first[kMaxRuns], end[kMaxRuns];   // first item of the run; items in this run and those before it
 };
-constexpr uint32_t kItemOpen = 0xFFFFFFFFu;   // host only, while the list is built: the item may still be extended
 
 // Crop rectangle of one image (pixels) and whether its columns are mirrored; the pixel kernel
 // skips work units that lie outside it when one is given.
