@@ -809,7 +809,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     // intervals; DC refinement scans have a kernel of their own and no items at all.
     uint32_t long_min = 64;
     if (const char* e = getenv("PCR_LONG_MIN_BYTES")) long_min = (uint32_t)std::max(0, atoi(e));
-    auto ik0ng = [&](int s, uint32_t i) {
+    auto is_long = [&](int s, uint32_t i) {
         const ScanScript& sc = r->script[s];
         const ScanDesc& sd = scans[(size_t)s * N + i];
         (void)sc;
@@ -827,14 +827,14 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
                 any = true;
                 const ScanDesc& sd = scans[(size_t)s * N + i];
                 one_interval = one_interval && sd.nseg == 1 && sd.data_end - sd.data_off < (1u << 27);
-                big = big || ik0ng((int)s, i);
+                big = big || is_long((int)s, i);
             }
             grouped[(size_t)i * 3 + c] = any && one_interval && big;
         }
-    auto takek0ng_kernel = [&](int s, uint32_t i) {
+    auto takes_long_kernel = [&](int s, uint32_t i) {
         const ScanScript& sc = r->script[s];
         if (sc.Ss > 0 && sc.Ah != 0) return grouped[(size_t)i * 3 + sc.comp[0]] != 0;
-        return ik0ng(s, i);
+        return is_long(s, i);
     };
     uint32_t *const longs = T.h<uint32_t>(at_long), *const groups = T.h<uint32_t>(at_group);
     uint32_t n_longs = 0, n_groups = 0;
@@ -846,7 +846,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
                 if (sc.Ah != 0) continue;                      // first passes only
                 r->long_begin[(size_t)g * G + s] = n_longs;
                 for (uint32_t pos = r->slice_img[g]; single && pos < r->slice_img[g + 1]; ++pos)
-                    if (ik0ng(s, order[pos])) longs[n_longs++] = (uint32_t)(s * N + order[pos]);
+                    if (is_long(s, order[pos])) longs[n_longs++] = (uint32_t)(s * N + order[pos]);
                 r->long_count[(size_t)g * G + s] = n_longs - r->long_begin[(size_t)g * G + s];
             }
     }
@@ -877,7 +877,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
                 Item* open = nullptr;                         // an unfilled last item that the next image may extend
                 for (uint32_t pos = r->slice_img[g]; pos < r->slice_img[g + 1] && !dc_refine; ++pos) {
                     const uint32_t i = order[pos];
-                    if (single && takek0ng_kernel((int)s, i)) continue;
+                    if (single && takes_long_kernel((int)s, i)) continue;
                     const uint32_t nseg = ns[i], si = (uint32_t)(s * N + i);
                     // full warps of 32 restart intervals; in AC scans the last warp of an image
                     // runs on into the first intervals of the next image (two tables per warp)
@@ -904,7 +904,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
             const uint32_t begin = n_items;
             for (uint32_t pos = r->slice_img[g]; r->pair_of[s] >= 0 && pos < r->slice_img[g + 1]; ++pos) {
                 const uint32_t i = order[pos], a = (uint32_t)r->pair_of[s];
-                if (single && takek0ng_kernel((int)s, i)) continue;
+                if (single && takes_long_kernel((int)s, i)) continue;
                 const uint32_t nseg = nsegs[(size_t)s * N + i];
                 for (uint32_t j = 0; j < nseg; j += kSegsPerItem / 2)
                     items[n_items++] = Item{a * N + i, j, std::min<uint32_t>(kSegsPerItem / 2, nseg - j), 0u, (s - a) * N};
