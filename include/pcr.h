@@ -280,7 +280,7 @@ int pcr_get_profile(pcr_record* rec, pcr_stage_time* out, int cap, int* n);
  *   host_qtab  : HOST, 3 x 64 uint16 quantisers (Y, Cb, Cr) in zigzag order; copied by value.
  *   dev_rgb    : DEVICE, caller-owned, 3*W*H bytes, 4-byte aligned start recommended.
  *   stream     : a cudaStream_t (NULL = default stream).  The call only enqueues work.
- * The kernel's small tables (image descriptor, work-unit list, quantisers: about 65 KB) live
+ * The kernel's small tables (image descriptor, work-unit list, quantisers: about 130 KB) live
  * in one fixed array inside the library's device image, which every GPU that loads the
  * library holds until the process exits.  All calls on a device share that array and each
  * call rewrites the part it uses, so two calls whose work overlaps on the GPU (different

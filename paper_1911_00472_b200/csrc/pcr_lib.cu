@@ -276,14 +276,17 @@ static inline uint64_t rd64(const uint8_t* p) { return (uint64_t)rd32(p) | ((uin
 // made them): block = position of the processing order.
 __global__ void __launch_bounds__(128) units_kernel(const ImgDesc* __restrict__ imgs, const uint32_t* __restrict__ order,
                                                     const uint32_t* __restrict__ prefix, Unit* __restrict__ units, uint32_t unit_mcus, uint32_t unit_rows,
-                                                    ScanDesc* __restrict__ scans, const uint32_t* __restrict__ seg_base, uint32_t G) {
+                                                    ScanDesc* __restrict__ scans, const uint32_t* __restrict__ seg_base, uint32_t G, uint32_t bpm) {
     const uint32_t img = order[blockIdx.x];
+    const ImgDesc im = imgs[img];
     for (uint32_t g = threadIdx.x; g < G; g += 128) scans[(size_t)g * gridDim.x + img].seg_base = seg_base[(size_t)g * gridDim.x + img];
-    const uint32_t per_row = (imgs[img].mx + unit_mcus - 1) / unit_mcus, n = per_row * ((imgs[img].my + unit_rows - 1) / unit_rows);
+    const uint32_t per_row = (im.mx + unit_mcus - 1) / unit_mcus, n = per_row * ((im.my + unit_rows - 1) / unit_rows);
     Unit* dst = units + prefix[blockIdx.x];
     for (uint32_t j = threadIdx.x; j < n; j += 128) {
         Unit un;
         un.img = img; un.mrow = (uint16_t)(j / per_row * unit_rows); un.mcol0 = (uint16_t)((j % per_row) * unit_mcus);
+        un.mx = (uint16_t)im.mx; un.my = (uint16_t)im.my; un.W = (uint16_t)im.W; un.H = (uint16_t)im.H;
+        un.mcus = im.blk_base / bpm; un.out_off = im.out_off;
         dst[j] = un;
     }
 }
@@ -957,7 +960,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     if (int rc = T.copy(r, at_long + 4ull * n_longs)) return rc;
     if (int rc = TI.copy(r, sizeof(Item) * (size_t)n_items)) return rc;
     units_kernel<<<N, 128, 0, r->up_stream>>>(r->d_imgs, r->d_order, r->d_unit_prefix, r->d_units, r->unit_mcus, r->unit_rows,
-                                              r->d_scans, T.d<uint32_t>(at_base), G);
+                                              r->d_scans, T.d<uint32_t>(at_base), G, bpm);
     ++g_launches;
     if (n_groups && cudaFuncSetAttribute(ac_refine_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kChainPairs * sizeof(ChainShared))) != cudaSuccess) return PCR_E_CUDA;
     r->h_status.assign(N, 0);
@@ -1137,12 +1140,13 @@ int pcr_evict(pcr_record* rec) {
 }  // extern "C"
 
 // The pixel kernels of one slice at one fidelity (see pcr_pixels.cuh for what the template arguments choose).
-struct PixelPlan { bool dc_only, head_only, refine, widths_mult16, triangle, roi; int samp; };
+struct PixelPlan { bool dc_only, head_only, refine, coarse, widths_mult16, triangle, roi; int samp; };
 
 template <int kSamp>
 static void launch_pixels_sampled(const PixelPlan& pl, unsigned grid, cudaStream_t q, const Params& Q, const CoefLists& cl, uint8_t* o8) {
     constexpr int T = unit_threads<kSamp>();
     if (pl.refine) pixel_kernel<true, 1, false, 0, kSamp><<<grid, T, 0, q>>>(Q, cl, o8);
+    else if (pl.coarse) pixel_kernel<false, 1, false, 0, kSamp, true><<<grid, T, 0, q>>>(Q, cl, o8);
     else pixel_kernel<false, 1, false, 0, kSamp><<<grid, T, 0, q>>>(Q, cl, o8);
 }
 
@@ -1151,8 +1155,9 @@ static void launch_pixels_420(const PixelPlan& pl, unsigned grid, cudaStream_t q
     constexpr int T = unit_threads<kSamp420>();
     if (pl.dc_only && pl.widths_mult16) dc_pixel_kernel<kRoi><<<grid, 128, 0, q>>>(Q, make_uint3(cl.dc_mask[0], cl.dc_mask[1], cl.dc_mask[2]), o8);
     else if (pl.dc_only) dc_pixel_kernel<kRoi, false><<<grid, 128, 0, q>>>(Q, make_uint3(cl.dc_mask[0], cl.dc_mask[1], cl.dc_mask[2]), o8);
-    else if (pl.head_only) pixel_kernel<false, 3, kRoi><<<grid, T, 0, q>>>(Q, cl, o8);
+    else if (pl.head_only) pixel_kernel<false, 3, kRoi, 0, kSamp420, true><<<grid, T, 0, q>>>(Q, cl, o8);
     else if (pl.refine) pixel_kernel<true, 1, kRoi><<<grid, T, 0, q>>>(Q, cl, o8);
+    else if (pl.coarse) pixel_kernel<false, 1, kRoi, 0, kSamp420, true><<<grid, T, 0, q>>>(Q, cl, o8);
     else pixel_kernel<false, 1, kRoi><<<grid, T, 0, q>>>(Q, cl, o8);
 }
 
@@ -1277,11 +1282,13 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
     const bool s420 = plan.samp == kSamp420;
     plan.dc_only = plan.head_only = s420;             // no AC scan at all / no scan beyond zigzag position 7, no refinement
     plan.refine = false;
+    plan.coarse = true;                               // every AC scan leaves low bits out (first passes ahead of refinements)
     for (int s = 0; s < k; ++s) {
         const ScanScript& sc = rec->script[s];
         if (sc.Ss > 0 || sc.Se > 0) plan.dc_only = false;
         if (sc.Se > 7 || (sc.Ss > 0 && sc.Ah > 0)) plan.head_only = false;
         if (sc.Ss > 0 && sc.Ah > 0) plan.refine = true;
+        if (sc.Se > 0 && sc.Al == 0) plan.coarse = false;
     }
     plan.widths_mult16 = rec->widths_mult16;
     plan.triangle = !targs && rec->upsampling == PCR_UPSAMPLE_TRIANGLE;
@@ -1816,7 +1823,6 @@ constexpr uint32_t kNoAllocMaxDim = 4096;                                       
 constexpr uint32_t kNoAllocMcus = kUnitMcus[kSamp420], kNoAllocRows = kUnitRows[kSamp420];
 constexpr uint32_t kNoAllocMaxUnits = (kNoAllocMaxDim / 16 / kNoAllocRows) * (kNoAllocMaxDim / 16 / kNoAllocMcus);
 struct NoAllocScratch {
-    ImgDesc img;
     uint16_t qtab[192];
     Unit units[kNoAllocMaxUnits];
 };
@@ -1829,14 +1835,11 @@ __global__ void noalloc_fill_kernel(uint32_t W, uint32_t H, QuantArg qa) {
     const uint32_t mx = (W + 15) / 16, my = (H + 15) / 16;
     const uint32_t per_row = (mx + kNoAllocMcus - 1) / kNoAllocMcus;
     const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
-    if (tid == 0) {
-        s->img.W = W; s->img.H = H; s->img.mx = mx; s->img.my = my;
-        s->img.blk_base = 0; s->img.out_off = 0;
-    }
     if (tid < 192) s->qtab[tid] = qa.q[tid];
     for (uint32_t u = tid; u < per_row * ((my + kNoAllocRows - 1) / kNoAllocRows); u += nth) {
         Unit un;
         un.img = 0; un.mrow = (uint16_t)(u / per_row * kNoAllocRows); un.mcol0 = (uint16_t)((u % per_row) * kNoAllocMcus);
+        un.mx = (uint16_t)mx; un.my = (uint16_t)my; un.W = (uint16_t)W; un.H = (uint16_t)H; un.mcus = 0; un.out_off = 0;
         s->units[u] = un;
     }
 }
@@ -1875,7 +1878,7 @@ int pcr_pixels_noalloc(const int16_t* dev_coeffs, uint32_t width, uint32_t heigh
     Params P;
     memset(&P, 0, sizeof P);
     P.planes = const_cast<int16_t*>(dev_coeffs);     // read only by the pixel kernel
-    P.imgs = &s->img; P.units = s->units; P.qtab = s->qtab; P.N = 1;
+    P.units = s->units; P.qtab = s->qtab; P.N = 1;
     CoefLists none;
     memset(&none, 0, sizeof none);
     pixel_kernel<false, 0><<<n_units, unit_threads<kSamp420>(), 0, st>>>(P, none, dev_rgb);

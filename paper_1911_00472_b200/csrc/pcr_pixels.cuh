@@ -59,23 +59,44 @@ struct ZigzagTable {
 };
 __device__ constexpr ZigzagTable kZigzag{};
 
-// One 8-point pass on the integer matrix M (see the header comment): out[n] = (sum_k M[n][k] x[k] + rnd) >> kShift
-template <int kShift>
-__device__ __forceinline__ void idct8(uint32_t& x0, uint32_t& x1, uint32_t& x2, uint32_t& x3, uint32_t& x4, uint32_t& x5,
-                                      uint32_t& x6, uint32_t& x7, uint32_t rnd) {
+// One 8-point pass on the integer matrix M (see the header comment) of a vector with x[N] .. x[7] = 0:
+// out[n] = (sum_k M[n][k] x[k] + rnd) >> kShift.  The compiler drops the terms of zeros.
+template <int kShift, int N>
+__device__ __forceinline__ void idct(const uint32_t (&x)[N], uint32_t rnd, uint32_t (&o)[8]) {
     constexpr uint32_t K1 = 8035, K2 = 7568, K3 = 6811, K4 = 5793, K5 = 4551, K6 = 3135, K7 = 1598;
-    const uint32_t a0 = K4 * (x0 + x4) + rnd, a1 = K4 * (x0 - x4) + rnd;
-    const uint32_t b0 = K2 * x2 + K6 * x6, b1 = K6 * x2 - K2 * x6;
+    const uint32_t x4 = N > 4 ? x[N > 4 ? 4 : 0] : 0u, x5 = N > 5 ? x[N > 5 ? 5 : 0] : 0u, x6 = N > 6 ? x[N > 6 ? 6 : 0] : 0u, x7 = N > 7 ? x[N > 7 ? 7 : 0] : 0u;
+    const uint32_t a0 = K4 * (x[0] + x4) + rnd, a1 = K4 * (x[0] - x4) + rnd;
+    const uint32_t b0 = K2 * x[2] + K6 * x6, b1 = K6 * x[2] - K2 * x6;
     const uint32_t e0 = a0 + b0, e3 = a0 - b0, e1 = a1 + b1, e2 = a1 - b1;
-    const uint32_t o0 = K1 * x1 + K3 * x3 + K5 * x5 + K7 * x7;
-    const uint32_t o1 = K3 * x1 - K7 * x3 - K1 * x5 - K5 * x7;
-    const uint32_t o2 = K5 * x1 - K1 * x3 + K7 * x5 + K3 * x7;
-    const uint32_t o3 = K7 * x1 - K5 * x3 + K3 * x5 - K1 * x7;
-    x0 = (uint32_t)((int)(e0 + o0) >> kShift); x7 = (uint32_t)((int)(e0 - o0) >> kShift);
-    x1 = (uint32_t)((int)(e1 + o1) >> kShift); x6 = (uint32_t)((int)(e1 - o1) >> kShift);
-    x2 = (uint32_t)((int)(e2 + o2) >> kShift); x5 = (uint32_t)((int)(e2 - o2) >> kShift);
-    x3 = (uint32_t)((int)(e3 + o3) >> kShift); x4 = (uint32_t)((int)(e3 - o3) >> kShift);
+    const uint32_t o0 = K1 * x[1] + K3 * x[3] + K5 * x5 + K7 * x7;
+    const uint32_t o1 = K3 * x[1] - K7 * x[3] - K1 * x5 - K5 * x7;
+    const uint32_t o2 = K5 * x[1] - K1 * x[3] + K7 * x5 + K3 * x7;
+    const uint32_t o3 = K7 * x[1] - K5 * x[3] + K3 * x5 - K1 * x7;
+    o[0] = (uint32_t)((int)(e0 + o0) >> kShift); o[7] = (uint32_t)((int)(e0 - o0) >> kShift);
+    o[1] = (uint32_t)((int)(e1 + o1) >> kShift); o[6] = (uint32_t)((int)(e1 - o1) >> kShift);
+    o[2] = (uint32_t)((int)(e2 + o2) >> kShift); o[5] = (uint32_t)((int)(e2 - o2) >> kShift);
+    o[3] = (uint32_t)((int)(e3 + o3) >> kShift); o[4] = (uint32_t)((int)(e3 - o3) >> kShift);
 }
+
+// Zigzag positions whose row and column are both below n, as a 64-bit mask, and the words of four positions that hold them.
+constexpr uint64_t corner_mask(int n) {
+    ZigzagTable z{};
+    uint64_t m = 0;
+    for (int k = 0; k < 64; ++k)
+        if ((z.nat[k] >> 3) < n && (z.nat[k] & 7) < n) m |= 1ull << k;
+    return m;
+}
+constexpr int corner_words(int n) {
+    int w = 0;
+    for (int k = 0; k < 64; ++k)
+        if ((corner_mask(n) >> k) & 1u) w = k / 4 + 1;
+    return w;
+}
+template <int N> struct Corner {
+    static constexpr int n = N, words = corner_words(N);
+    static constexpr uint64_t mask = corner_mask(N);
+};
+static_assert((corner_mask(4) & 0xFFu) == 0xFFu, "positions 0..7 lie in the smallest corner");
 
 // Two samples as a pair of 16-bit numbers, {clamp((a >> 16) + 128), clamp((b >> 16) + 128)} with clamp to 0..255: the
 // upper halves by one permutation, then two packed operations.  The upper end is cut before 128 is added, so
@@ -85,6 +106,9 @@ __device__ __forceinline__ uint32_t sample_pair(uint32_t a, uint32_t b) {
 }
 // bytes {lo(a), hi(a), lo(b), hi(b)} of two pairs
 __device__ __forceinline__ uint32_t pair_bytes(uint32_t a, uint32_t b) { return __byte_perm(a, b, 0x6420); }
+
+struct Image { uint32_t W, H, mx, my; uint64_t blk_base, out_off; };
+template <int kBpm> __device__ __forceinline__ Image image_of(const Unit& u) { return Image{u.W, u.H, u.mx, u.my, kBpm * u.mcus, u.out_off}; }
 
 // Where a decode's coefficients lie (built per call for the chosen k, see CoefLists in pcr_types.h): the
 // DC plane, the head plane (positions 1..7), and per first pass and component the masks and values of the rest.
@@ -96,39 +120,67 @@ __device__ __forceinline__ uint32_t pair_bytes(uint32_t a, uint32_t b) { return 
 // eight bytes: every thread keeps to its own banks, whatever position it addresses).
 // A correction moves a non-zero coefficient away from zero by 2^Al if its bit Al is still clear; a
 // new coefficient is +-2^Al.
-template <int kT, bool kRefine>
-__device__ __forceinline__ void expand_block(const Params& P, const CoefLists& cl, int comp, uint64_t blk, uint64_t local, uint8_t* line) {
+// Returns (for the whole warp, which calls it together) whether every coefficient lies in the low kCorner x kCorner
+// corner; then only the words of the line that hold the corner are written.  kCorner = 8: not asked for.
+template <int kT, bool kRefine, int kCorner>
+__device__ __forceinline__ bool expand_block(const Params& P, const CoefLists& cl, int comp, uint64_t blk, uint64_t local, uint8_t* line, bool valid) {
     constexpr int kPitch = 8 * kT;
     auto at = [&](int pos) { return reinterpret_cast<int16_t*>(line + (pos >> 2) * kPitch + 2 * (pos & 3)); };
     const int nfirst = cl.n_first[comp], nref = kRefine ? cl.n_refine[comp] : 0;
     // all of the block's loads are requested before the first is used
     const uint4 zero4 = make_uint4(0, 0, 0, 0);
-    uint4 head = __ldg(reinterpret_cast<const uint4*>(P.head + blk * 8));
-    const uint32_t dc = __ldg(reinterpret_cast<const uint16_t*>(P.dc) + blk) & cl.dc_mask[comp];
-    uint4 rec = zero4;
+    uint4 head = zero4, rec = zero4;
+    uint32_t dc = 0;
     const uint64_t at_rec = cl.sequential ? blk : local;
-    if (nfirst > 0) rec = __ldg(reinterpret_cast<const uint4*>(P.aux + cl.first[comp][0]) + at_rec);
     uint4 a0 = zero4, b0 = zero4, a1 = zero4, b1 = zero4;
-    if (kRefine) {
-        if (nref > 0) { const uint4* o = reinterpret_cast<const uint4*>(P.aux + cl.refine[comp][0]) + 2 * local; a0 = __ldg(o); b0 = __ldg(o + 1); }
-        if (nref > 1) { const uint4* o = reinterpret_cast<const uint4*>(P.aux + cl.refine[comp][1]) + 2 * local; a1 = __ldg(o); b1 = __ldg(o + 1); }
+    if (valid) {
+        head = __ldg(reinterpret_cast<const uint4*>(P.head + blk * 8));
+        dc = __ldg(reinterpret_cast<const uint16_t*>(P.dc) + blk) & cl.dc_mask[comp];
+        if (nfirst > 0) rec = __ldg(reinterpret_cast<const uint4*>(P.aux + cl.first[comp][0]) + at_rec);
+        if (kRefine) {
+            if (nref > 0) { const uint4* o = reinterpret_cast<const uint4*>(P.aux + cl.refine[comp][0]) + 2 * local; a0 = __ldg(o); b0 = __ldg(o + 1); }
+            if (nref > 1) { const uint4* o = reinterpret_cast<const uint4*>(P.aux + cl.refine[comp][1]) + 2 * local; a1 = __ldg(o); b1 = __ldg(o + 1); }
+        }
     }
+    bool small = false;
+    constexpr int kCornerWords = Corner<kCorner>::words;
+    if (kCorner < 8) {
+        // positions that are non-zero (a refinement's mask holds those before it too)
+        constexpr uint64_t kMask = Corner<kCorner>::mask;
+        uint32_t n0 = rec.x | a0.x | a1.x, n1 = rec.y | a0.y | a1.y;
+        if (valid) {
+            for (int i = 1; i < nfirst; ++i) { const uint2 r = __ldg(reinterpret_cast<const uint2*>(reinterpret_cast<const uint4*>(P.aux + cl.first[comp][i]) + at_rec)); n0 |= r.x; n1 |= r.y; }
+            if (kRefine)
+                for (int i = 2; i < nref; ++i) { const uint2 r = __ldg(reinterpret_cast<const uint2*>(reinterpret_cast<const uint4*>(P.aux + cl.refine[comp][i]) + 2 * local)); n0 |= r.x; n1 |= r.y; }
+        }
+        small = !__any_sync(0xffffffffu, ((n0 & ~(uint32_t)kMask) | (n1 & ~(uint32_t)(kMask >> 32))) != 0);
+    }
+    if (!valid) return small;
 #pragma unroll
-    for (int w = 2; w < 16; ++w) *reinterpret_cast<uint2*>(line + w * kPitch) = make_uint2(0, 0);
+    for (int w = 2; w < kCornerWords; ++w) *reinterpret_cast<uint2*>(line + w * kPitch) = make_uint2(0, 0);
+    if (!small) {
+#pragma unroll
+        for (int w = kCornerWords; w < 16; ++w) *reinterpret_cast<uint2*>(line + w * kPitch) = make_uint2(0, 0);
+    }
     const uint4 hm = cl.head_mask[comp];           // positions that no decoded scan covers may hold a later scan's values
     *reinterpret_cast<uint2*>(line) = make_uint2((head.x & hm.x) | dc, head.y & hm.y);
     *reinterpret_cast<uint2*>(line + kPitch) = make_uint2(head.z & hm.z, head.w & hm.w);
     for (int i = 0; i < nfirst; ++i) {
         if (i) rec = __ldg(reinterpret_cast<const uint4*>(P.aux + cl.first[comp][i]) + at_rec);
         const int16_t* v = reinterpret_cast<const int16_t*>(((uint64_t)rec.w << 32) | rec.z);
+        uint64_t m = ((uint64_t)rec.y << 32) | (rec.x & ~0xFFu);
+        while (m) {                                // four at a time, so that their loads are in flight together
+            int pos[4], x[4];
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            uint32_t m = half ? rec.y : rec.x & ~0xFFu;
-            while (m) {
-                const int pos = 32 * half + __ffs((int)m) - 1;
-                m &= m - 1u;
-                *at(pos) = __ldg(v++);
+            for (int e = 0; e < 4; ++e) {
+                pos[e] = m ? __ffsll((long long)m) - 1 : -1;
+                m &= m - 1ull;                     // (0 stays 0)
+                if (pos[e] >= 0) x[e] = __ldg(v + e);
             }
+            v += 4;
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (pos[e] >= 0) *at(pos[e]) = (int16_t)x[e];
         }
     }
     if (kRefine) {
@@ -168,6 +220,7 @@ __device__ __forceinline__ void expand_block(const Params& P, const CoefLists& c
             }
         }
     }
+    return small;
 }
 
 // kMode: 0 = all 64 coefficients sit in the block's 128-byte line (pcr_pixels_noalloc); 1 = coefficient lists
@@ -182,14 +235,18 @@ __device__ __forceinline__ void expand_block(const Params& P, const CoefLists& c
 // as in 0, chroma samples with a one-sample border read back from P.chroma, every pixel's chroma = (9 own +
 // 3 horizontally nearer + 3 vertically nearer + 1 diagonal + 8) >> 4, neighbours clamped to the MCU-padded
 // planes.  3 = no pixels: the expanded blocks are written to P.planes (pcr_coeffs).
+// kCoarse: every AC scan so far left low bits out (or kMode 3), so nearly all coefficients sit in the low 4x4 corner: warps
+// whose blocks have none outside it take a transform of that corner, which needs fewer registers, and the
+// kernel is compiled for more CTAs an SM (the full transform spills then).  1024 ImageNet-shaped images at
+// k = 5: 240 -> 166 us; for a record at full precision both would cost time (baseline 281 -> 418 us, k = 10 348 -> 478).
 // kSamp: the record's chroma sampling (see Sampling); the triangle filter (kStage 1, 2) exists for
 // 4:2:0 only.  A greyscale record has no chroma: every pixel is (Y, Y, Y).
 //
 // One thread per block through the whole transform; the chroma samples go through shared memory, the luminance
 // samples stay in the registers of the thread that made them and meet the chroma there, two pixels
 // per instruction (16-bit pairs).  Bound by instruction issue: see the table of kernels for the counts.
-template <bool kRefine, int kMode, bool kRoi = false, int kStage = 0, int kSamp = kSamp420>
-__global__ void __launch_bounds__(unit_threads<kSamp>(), 672 / unit_threads<kSamp>())
+template <bool kRefine, int kMode, bool kRoi = false, int kStage = 0, int kSamp = kSamp420, bool kCoarse = false>
+__global__ void __launch_bounds__(unit_threads<kSamp>(), (kCoarse ? 1152 : 672) / unit_threads<kSamp>())
 pixel_kernel(Params P, CoefLists cl, uint8_t* __restrict__ out) {
     using S = Sampling<kSamp>;
     constexpr int HS = S::HS, VS = S::VS, NC = S::NC, U = S::U, R = S::R, kT = unit_threads<kSamp>();
@@ -209,7 +266,7 @@ pixel_kernel(Params P, CoefLists cl, uint8_t* __restrict__ out) {
 
     const int tid = threadIdx.x;
     const Unit un = P.units[blockIdx.x];
-    const ImgDesc im = P.imgs[un.img];
+    const Image im = image_of<kBpm>(un);
     const int nm = min(U, (int)im.mx - (int)un.mcol0);                // MCUs across in this unit
     int r_lo = 0, r_hi = min(R, (int)im.my - (int)un.mrow);           // its MCU rows that are wanted
     if (kRoi) {
@@ -218,11 +275,13 @@ pixel_kernel(Params P, CoefLists cl, uint8_t* __restrict__ out) {
         r_lo = max(r_lo, y0); r_hi = min(r_hi, y1);
         if (r_lo >= r_hi || ux0 >= (int)(r.x0 + r.w) || ux0 + kPxW * nm <= (int)r.x0) return;      // whole CTA: nothing of this unit is wanted
     }
+    // (the quantisers are requested before the block's loads and stored behind them)
+    constexpr int kQLoads = (96 + kT - 1) / kT;
+    uint32_t q2[kQLoads];
     if (kStage != 3) {
-        for (int i = tid; i < 96; i += kT) {
-            const uint32_t q2 = __ldg(reinterpret_cast<const uint32_t*>(P.qtab + (size_t)un.img * 192) + i);
-            *reinterpret_cast<int2*>(&s_q[0][0] + 2 * i) = make_int2((int)(q2 & 0xFFFFu), (int)(q2 >> 16));
-        }
+#pragma unroll
+        for (int i = 0; i < kQLoads; ++i)
+            if (tid + i * kT < 96) q2[i] = __ldg(reinterpret_cast<const uint32_t*>(P.qtab + (size_t)un.img * 192) + tid + i * kT);
     }
     // ---- thread j owns block j: the unit's luminance block rows, then its Cb rows, then its Cr rows
     int comp = 0, yr, yc;                 // component, block row / column inside the unit
@@ -233,7 +292,7 @@ pixel_kernel(Params P, CoefLists cl, uint8_t* __restrict__ out) {
         valid = yc < HS * nm && yr >= VS * r_lo && yr < VS * r_hi && kStage != 1;
         local = (uint64_t)(VS * un.mrow + yr) * (HS * im.mx) + HS * un.mcol0 + yc;
         blk = im.blk_base + local;
-        local += (uint64_t)(HS * VS) * (im.blk_base / kBpm);
+        local += (uint64_t)(HS * VS) * (un.mcus);
     } else {
         const int i = tid - kYBlocks;
         comp = 1 + i / (U * R);
@@ -241,25 +300,30 @@ pixel_kernel(Params P, CoefLists cl, uint8_t* __restrict__ out) {
         valid = yc < nm && yr >= r_lo && yr < r_hi && kStage != 2;
         local = (uint64_t)(un.mrow + yr) * im.mx + un.mcol0 + yc;
         blk = im.blk_base + (uint64_t)(HS * VS + comp - 1) * im.mx * im.my + local;
-        local += im.blk_base / kBpm;
+        local += un.mcus;
     }
     uint8_t* const line = s_mem + 8 * tid;
-    if (kMode == 1 && valid) expand_block<kT, kRefine>(P, cl, comp, blk, local, line);
+    constexpr int kCorner = kCoarse ? 4 : 8;          // the corner that a shorter transform is made for
+    bool small = kMode == 3;              // every coefficient of the warp's blocks lies in it
+    if (kMode == 1) small = expand_block<kT, kRefine, kCorner>(P, cl, comp, blk, local, line, valid);
     if (kStage == 3) {
         if (valid) {
             uint4* dst = reinterpret_cast<uint4*>(P.planes + blk * 64);
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
-                const uint2 lo = *reinterpret_cast<const uint2*>(line + (2 * q) * 8 * kT), hi = *reinterpret_cast<const uint2*>(line + (2 * q + 1) * 8 * kT);
+                if (small && 2 * q >= Corner<kCorner>::words) { dst[q] = make_uint4(0, 0, 0, 0); continue; }
+                const uint2 lo = *reinterpret_cast<const uint2*>(line + (2 * q) * 8 * kT), hi = small && 2 * q + 1 >= Corner<kCorner>::words ? make_uint2(0, 0) : *reinterpret_cast<const uint2*>(line + (2 * q + 1) * 8 * kT);
                 dst[q] = make_uint4(lo.x, lo.y, hi.x, hi.y);
             }
         }
         return;
     }
+#pragma unroll
+    for (int i = 0; i < kQLoads; ++i)
+        if (tid + i * kT < 96) *reinterpret_cast<int2*>(&s_q[0][0] + 2 * (tid + i * kT)) = make_int2((int)(q2[i] & 0xFFFFu), (int)(q2[i] >> 16));
     __syncthreads();                  // the quantisers are there
     uint32_t yp[32];                      // a luminance block's samples, two per word (row y: words 4y .. 4y + 3)
     if (valid) {
-        uint32_t v[64];
         const int4* q4 = reinterpret_cast<const int4*>(&s_q[comp][0]);
         uint4 head = make_uint4(0, 0, 0, 0);
         if (kMode == 3) {
@@ -268,36 +332,57 @@ pixel_kernel(Params P, CoefLists cl, uint8_t* __restrict__ out) {
             head = make_uint4((head.x & hm.x) | (__ldg(reinterpret_cast<const uint16_t*>(P.dc) + blk) & cl.dc_mask[comp]), head.y & hm.y, head.z & hm.z, head.w & hm.w);
         }
         const uint4* dense = reinterpret_cast<const uint4*>(P.planes + blk * 64);
+        auto word = [&](int w) {                                      // zigzag positions 4w .. 4w + 3
+            if (kMode == 3) return w == 0 ? make_uint2(head.x, head.y) : (w == 1 ? make_uint2(head.z, head.w) : make_uint2(0, 0));
+            if (kMode == 0) return __ldg(reinterpret_cast<const uint2*>(dense) + w);
+            return *reinterpret_cast<const uint2*>(line + w * 8 * kT);
+        };
+        auto dequantise = [&](uint2 c2, const int4& q, uint32_t (&f)[4]) {
+            f[0] = (uint32_t)((int)(short)(c2.x & 0xFFFFu) * q.x); f[1] = (uint32_t)(((int)c2.x >> 16) * q.y);
+            f[2] = (uint32_t)((int)(short)(c2.y & 0xFFFFu) * q.z); f[3] = (uint32_t)(((int)c2.y >> 16) * q.w);
+        };
+        // Pass 1: columns (two fraction bits kept).  Pass 2: rows; the final shift by 16 takes the upper halves, the
+        // level shift is part of the clamping.  A warp whose blocks have nothing outside the low N x N corner takes N of the
+        // columns and N terms of each sum.
+        auto transform = [&](auto corner) {
+            constexpr int N = decltype(corner)::n, kWords = kMode == 3 ? 2 : Corner<N>::words;
+            constexpr uint64_t kIn = Corner<N>::mask;
+            uint32_t v[N][N];                                         // [column][row]
 #pragma unroll
-        for (int w = 0; w < 16; ++w) {                                // zigzag positions 4w .. 4w + 3
-            uint2 c2;
-            if (kMode == 3) c2 = w == 0 ? make_uint2(head.x, head.y) : (w == 1 ? make_uint2(head.z, head.w) : make_uint2(0, 0));
-            else if (kMode == 0) c2 = __ldg(reinterpret_cast<const uint2*>(dense) + w);
-            else c2 = *reinterpret_cast<const uint2*>(line + w * 8 * kT);
-            const int4 q = q4[w];
-            v[kZigzag.nat[4 * w]] = (uint32_t)((int)(short)(c2.x & 0xFFFFu) * q.x);
-            v[kZigzag.nat[4 * w + 1]] = (uint32_t)(((int)c2.x >> 16) * q.y);
-            v[kZigzag.nat[4 * w + 2]] = (uint32_t)((int)(short)(c2.y & 0xFFFFu) * q.z);
-            v[kZigzag.nat[4 * w + 3]] = (uint32_t)(((int)c2.y >> 16) * q.w);
-        }
-        // pass 1: columns (two fraction bits kept)
+            for (int k = 4 * kWords; k < 64; ++k)
+                if ((kIn >> k) & 1u) v[kZigzag.nat[k] & 7][kZigzag.nat[k] >> 3] = 0;
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
-            idct8<12>(v[u], v[8 + u], v[16 + u], v[24 + u], v[32 + u], v[40 + u], v[48 + u], v[56 + u], 1u << 11);
-        // pass 2: rows; the final shift by 16 takes the upper halves, the level shift is part of the clamping
+            for (int w = 0; w < kWords; ++w) {
+                uint32_t f[4];
+                dequantise(word(w), q4[w], f);
 #pragma unroll
-        for (int y = 0; y < 8; ++y) {
-            uint32_t* r = v + 8 * y;
-            idct8<0>(r[0], r[1], r[2], r[3], r[4], r[5], r[6], r[7], 1u << 15);
+                for (int e = 0; e < 4; ++e)
+                    if ((kIn >> (4 * w + e)) & 1u) v[kZigzag.nat[4 * w + e] & 7][kZigzag.nat[4 * w + e] >> 3] = f[e];
+            }
+            uint32_t t[8][N];
 #pragma unroll
-            for (int p = 0; p < 4; ++p) yp[4 * y + p] = sample_pair(r[2 * p], r[2 * p + 1]);
-        }
+            for (int u = 0; u < N; ++u) {
+                uint32_t o[8];
+                idct<12, N>(v[u], 1u << 11, o);
+#pragma unroll
+                for (int y = 0; y < 8; ++y) t[y][u] = o[y];
+            }
+#pragma unroll
+            for (int y = 0; y < 8; ++y) {
+                uint32_t r[8];
+                idct<0, N>(t[y], 1u << 15, r);
+#pragma unroll
+                for (int p = 0; p < 4; ++p) yp[4 * y + p] = sample_pair(r[2 * p], r[2 * p + 1]);
+            }
+        };
+        if (kMode == 3 || (kCorner < 8 && kMode == 1 && small)) transform(Corner<kCorner>{});
+        else if (kMode != 3) transform(Corner<8>{});
         if (NC == 3 && comp != 0) {
             uint8_t* dst;
             int pitch;
             if (kStage == 1) {
                 pitch = 8 * (int)im.mx;
-                dst = P.chroma + (im.blk_base / 6) * 128 + (comp == 2 ? 64ull * im.mx * im.my : 0ull) +
+                dst = P.chroma + (un.mcus) * 128 + (comp == 2 ? 64ull * im.mx * im.my : 0ull) +
                       (size_t)(8 * (un.mrow + yr)) * pitch + 8 * (un.mcol0 + yc);
             } else { dst = &s_c[comp - 1][8 * yr][8 * yc]; pitch = 8 * U; }
 #pragma unroll
@@ -309,7 +394,7 @@ pixel_kernel(Params P, CoefLists cl, uint8_t* __restrict__ out) {
     if (kStage == 2) {
         // chroma tile of the unit with a one-sample border, clamped to the padded planes
         const int cw = 8 * (int)im.mx, chh = 8 * (int)im.my, tw = 8 * nm + 2;
-        const uint8_t* cbase = P.chroma + (im.blk_base / 6) * 128;
+        const uint8_t* cbase = P.chroma + (un.mcus) * 128;
         for (int i = tid; i < 2 * (8 * R + 2) * tw; i += kT) {
             const int c = i / ((8 * R + 2) * tw), rem2 = i - c * (8 * R + 2) * tw, r = rem2 / tw, x = rem2 - r * tw;
             const int gy = min(max(8 * (int)un.mrow + r - 1, 0), chh - 1), gx2 = min(max(8 * (int)un.mcol0 + x - 1, 0), cw - 1);
@@ -465,7 +550,7 @@ __global__ void __launch_bounds__(128) dc_pixel_kernel(Params P, uint3 dc_mask, 
     __shared__ uint32_t s_tri[2 * R][2 * U];           // [block row of the unit][block column]: R | G << 8 | B << 16
     const int tid = threadIdx.x;
     const Unit un = P.units[blockIdx.x];
-    const ImgDesc im = P.imgs[un.img];
+    const Image im = image_of<6>(un);
     const int nm = min(U, (int)im.mx - (int)un.mcol0);
     int r_lo = 0, r_hi = min(R, (int)im.my - (int)un.mrow);
     if (kRoi) {

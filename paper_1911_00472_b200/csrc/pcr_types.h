@@ -101,9 +101,12 @@ struct CropRect {
 };
 
 // Pixel work unit: a run of MCUs in one MCU row of one image.
-struct Unit {
+// With what a CTA needs of its image, so that one load tells it everything.
+struct __align__(16) Unit {
     uint32_t img;
-    uint16_t mrow, mcol0;
+    uint16_t mrow, mcol0, mx, my, W, H;
+    uint64_t mcus;        // MCUs of the images before this one
+    uint64_t out_off;     // first byte of the image in the output buffer
 };
 
 struct ScanTab;             // lookup table of one Huffman table (pcr_entropy.cuh)
