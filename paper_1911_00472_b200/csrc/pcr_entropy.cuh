@@ -26,77 +26,12 @@ namespace pcr {
 
 constexpr int kErrCorrupt = -3;
 
-#ifndef PCR_LUT_BITS
-#define PCR_LUT_BITS 11
-#endif
 #ifndef PCR_ENTROPY_WARPS
 #define PCR_ENTROPY_WARPS 3
 #endif
-constexpr int kLutBits = PCR_LUT_BITS;
 constexpr int kEntropyWarps = PCR_ENTROPY_WARPS;
 
-// Decoder tables of one Huffman table: a direct lookup on the next kBits bits for short
-// codes, and the canonical first-code / count / index triple per length for the rest.
-template <int kBits>
-struct HuffTabT {
-    uint16_t lut[1 << kBits];  // (length << 8) | symbol, 0 = longer than kBits (or undefined)
-    uint32_t first[17];
-    uint16_t cnt[17];
-    uint16_t idx[17];
-    uint8_t vals[256];
-};
-using HuffTab = HuffTabT<kLutBits>;
-
-template <int kBits>
-__device__ __forceinline__ void build_hufftab(HuffTabT<kBits>& t, const uint8_t* __restrict__ dht, int lane) {
-    // dht: 16 length counts, then the symbol values in code order
-    uint32_t code = 0, p = 0;
-    for (int l = 1; l <= 16; ++l) {
-        uint32_t c = dht[l - 1];
-        if (lane == 0) { t.first[l] = code; t.cnt[l] = (uint16_t)c; t.idx[l] = (uint16_t)p; }
-        code = (code + c) << 1;
-        p += c;
-    }
-    const uint32_t nvals = min(p, 256u);
-    for (uint32_t j = lane; j < nvals; j += 32) t.vals[j] = dht[16 + j];
-    uint32_t* lw = reinterpret_cast<uint32_t*>(t.lut);
-    for (int e = lane; e < (1 << kBits) / 2; e += 32) lw[e] = 0;
-    __syncwarp();
-    // every symbol with a short code fills its 2^(kBits - length) entries, all lanes together
-    uint32_t j = 0;
-    for (int l = 1; l <= kBits; ++l) {
-        const uint32_t c = t.cnt[l], f = t.first[l], span = 1u << (kBits - l);
-        for (uint32_t i = 0; i < c && j < nvals; ++i, ++j) {
-            const uint32_t base = (f + i) << (kBits - l);
-            const uint16_t entry = (uint16_t)(((uint32_t)l << 8) | t.vals[j]);
-            if (base + span <= (1u << kBits))
-                for (uint32_t e = lane; e < span; e += 32) t.lut[base + e] = entry;
-        }
-    }
-    __syncwarp();
-}
-
 constexpr int kRingWords = 16;       // words of the bitstream a lane of the interval kernels holds in shared memory
-
-// Huffman symbol at the top of the 32-bit window; returns (length << 8) | symbol, 0 if undefined
-template <int kBits>
-__device__ __forceinline__ uint32_t huff_lookup(const HuffTabT<kBits>& t, uint32_t win) {
-    uint32_t e = t.lut[win >> (32 - kBits)];
-    if (e) return e;
-    const uint32_t w16 = win >> 16;
-    for (int l = kBits + 1; l <= 16; ++l) {
-        uint32_t d = (w16 >> (16 - l)) - t.first[l];
-        if (d < t.cnt[l]) return ((uint32_t)l << 8) | t.vals[(t.idx[l] + d) & 255u];   // (index masked: damaged tables stay in bounds)
-    }
-    return 0;
-}
-
-__device__ __forceinline__ int extend_bits(uint32_t v, int s) {
-    // value of an s-bit magnitude field: the top bit clear means negative
-    return s == 0 ? 0 : ((v >> (s - 1)) ? (int)v : (int)v - (1 << s) + 1);
-}
-// the top n bits of x (n in 0..32)
-__device__ __forceinline__ uint32_t top_bits(uint32_t x, int n) { return n ? x >> (32 - n) : 0u; }
 
 struct ScanList { int32_t n; int32_t s[64]; };      // the scans one launch covers
 
@@ -116,6 +51,7 @@ constexpr int kTabBits = 10;
 struct __align__(16) ScanTab {
     uint16_t lut[1 << kTabBits];
     uint16_t first[8], cnt[8], idx[8];      // codes of kTabBits + 1 + j bits: first code, how many, index of the first value
+                                            // (first[7]: the greatest 16 bits that begin with a code)
     uint8_t vals[256];
 };
 static_assert(sizeof(ScanTab) % 16 == 0, "tables are copied as 16-byte vectors");
@@ -153,6 +89,7 @@ __device__ __forceinline__ void build_scan_tab(ScanTab* __restrict__ t, const ui
         code = (code + c) << 1;
         p += c;
     }
+    if (lane == 0) t->first[7] = (uint16_t)((code >> 1) - 1u);
     const uint32_t nvals = min(p, 256u);
     for (uint32_t j = lane; j < 256u; j += 32) { const uint8_t v = j < nvals ? dht[16 + j] : 0; s_vals[j] = v; t->vals[j] = v; }
     __syncwarp();
@@ -474,6 +411,7 @@ __device__ __forceinline__ int magnitude(uint32_t win, uint32_t skip, uint32_t s
 // there is no such symbol.
 __device__ __forceinline__ uint32_t long_code(uint32_t t, uint32_t win, int kind) {
     const uint32_t w16 = win >> 16;
+    if (w16 > lds16(t + (uint32_t)offsetof(ScanTab, first) + 14u)) return 0;      // (the usual case of a reading from a wrong position)
 #pragma unroll 1
     for (uint32_t j = 0; j < 16 - kTabBits; ++j) {
         const uint32_t l = kTabBits + 1u + j, d = (w16 >> (16u - l)) - lds16(t + (uint32_t)offsetof(ScanTab, first) + 2u * j);

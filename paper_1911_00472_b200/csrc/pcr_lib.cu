@@ -1307,7 +1307,7 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
         const uint32_t pairs = (uint32_t)sl.n * (uint32_t)rec->N, nb = (pairs + 7) / 8;
         bool tables = false;
         for (int i = 0; i < sl.n; ++i)
-            for (int g = 0; g < rec->n_slices; ++g) tables = tables || rec->item_count[(size_t)g * rec->G + sl.s[i]] > 0;
+            for (int g = 0; g < rec->n_slices; ++g) tables = tables || rec->item_count[(size_t)g * rec->G + sl.s[i]] + rec->long_count[(size_t)g * rec->G + sl.s[i]] > 0;
         unstuff_index_kernel<<<nb + (tables ? (pairs + 1) / 2 : 0), 256, 0, q>>>(P, sl, 0, rec->N, nb);
         ++g_launches;
     };

@@ -82,253 +82,125 @@ __global__ void __launch_bounds__(256) dc_refine_kernel(Params P, int s, uint32_
 }
 
 // ---------------------------------------------------------------------------------------
-// Bit reader of one lane over the unstuffed big-endian words: a 64-bit window, the next word
-// already requested while the current bits are consumed.  Positions are bits counted from the
-// first bit of a base word.
+// First passes and sequential scans that are one restart interval.  The interval is cut into subsequences of equal bit
+// length, one per thread of a small CTA.  A position's state is the bit position and a number `st`: DC scans: the
+// block's place in its MCU; AC scans: the next zigzag position; sequential scans: 64 times the place plus the next
+// zigzag position (0: the block's DC symbol comes next).
+//
+// Search: every thread follows its subsequence from a guessed state; threads whose predecessor ended in another state than
+// they began with follow theirs again, until nothing changes.  A thread leaves its state behind at eight places of
+// its subsequence; a later reading that comes by in the same state has met the earlier one and stops there.  (Without
+// that every round cost a whole subsequence, and interleaved DC scans take 5 to 9 rounds.)  Count: once more, the blocks
+// finished and the DC differences summed; prefix sums give every thread its first block and predictors.  Write: once more.
+//
+// A step is a window (two loads that hit the L1 cache), a table entry that already holds what the step needs, and an
+// addition; bound by that chain, about 110 cycles a symbol (430 with a 64-bit buffer, a canonical table and selects).
 // ---------------------------------------------------------------------------------------
-struct WordReader {
-    const uint32_t* w;     // base word
-    uint32_t rd;           // index of the word held in `ahead`
-    uint64_t buf;          // left-aligned window
-    int nbits;
-    uint32_t ahead;
-    __device__ __forceinline__ void init(const uint32_t* base, uint32_t pos) {
-        w = base;
-        rd = pos >> 5;
-        const uint32_t first = __ldg(w + rd) << (pos & 31u);
-        buf = (uint64_t)first << 32;
-        nbits = 32 - (int)(pos & 31u);
-        ++rd;
-        ahead = __ldg(w + rd);
-    }
-    __device__ __forceinline__ void refill() {                 // afterwards at least 33 bits are held
-        if (nbits <= 32) {
-            buf |= (uint64_t)ahead << (32 - nbits);
-            nbits += 32;
-            ++rd;
-            ahead = __ldg(w + rd);
-        }
-    }
-    __device__ __forceinline__ uint32_t top32() const { return (uint32_t)(buf >> 32); }
-    __device__ __forceinline__ void skip(int n) { buf <<= n; nbits -= n; }
-    __device__ __forceinline__ uint32_t pos() const { return rd * 32u - (uint32_t)nbits; }
-};
-
-#ifndef PCR_LONG_WARPS
-#define PCR_LONG_WARPS 2
-#endif
-constexpr int kLongWarps = PCR_LONG_WARPS;   // warps per scan in first_pass_long_kernel: 32 subsequences each
-
-// ---------------------------------------------------------------------------------------
-// The search passes of first_pass_long_kernel (a thread decodes its subsequence only to learn in which
-// state it ends and how many blocks it finishes) are the serial part of that kernel: when a stream
-// does not re-synchronise (a stretch of equally long symbols, in which a shifted reading stays shifted)
-// the true state moves on by one subsequence per round.  So they are kept short: a lookup table that
-// already holds what the search needs of a symbol, and a reader of three words in registers.
-// ---------------------------------------------------------------------------------------
-struct GlobalBits {
-    const uint32_t* w;     // base word (global memory; the neighbouring threads share its cache lines)
-    uint32_t w0, w1, w2;   // the word the next bit lies in and the two after it
-    uint32_t bits;         // position of the next bit, counted from the first bit of the base word
-    __device__ __forceinline__ void init(const uint32_t* base, uint32_t pos) {
-        w = base;
-        bits = pos;
-        const uint32_t i = pos >> 5;
-        w0 = __ldg(w + i); w1 = __ldg(w + i + 1); w2 = __ldg(w + i + 2);
-    }
-    __device__ __forceinline__ uint32_t win() const { return __funnelshift_l(w1, w0, bits); }   // the next 32 bits (shift taken mod 32)
-    __device__ __forceinline__ void skip(uint32_t n) {        // n < 32: at most one word further
-        const uint32_t nb = bits + n;
-        if ((nb ^ bits) >> 5) { w0 = w1; w1 = w2; w2 = __ldg(w + (nb >> 5) + 2); }
-        bits = nb;
-    }
-};
-
-// What the search of an AC first pass needs of a symbol (a HuffTab entry (length << 8) | (run << 4 | size)):
-// bits 0..4 bits to skip (code and extra bits), 5..8 positions the symbol moves on minus one (run + 1 for
-// a coefficient, 16 for sixteen zeros), 9 end of band, 10..13 its run-length exponent.
-constexpr uint32_t kSearchEob = 0x200u;
-__device__ __forceinline__ uint32_t ac_search_entry(uint32_t t) {
-    if (t == 0) return 0;
-    const uint32_t len = t >> 8, r = (t >> 4) & 15u, sz = t & 15u;
-    if (sz) return (len + sz) | (r << 5);
-    if (r == 15u) return len | (15u << 5);
-    return (len + r) | kSearchEob | (r << 10);
+// w: the stream's words, in shared memory where they fit, else where they are (the loads are generic ones).
+__device__ __forceinline__ uint32_t long_window(const uint32_t* w, uint32_t pos) {
+    const uint32_t i = pos >> 5;
+    return __funnelshift_l(w[i + 1], w[i], pos);                           // (shift taken mod 32)
+}
+__device__ __forceinline__ uint32_t long_entry(uint32_t tab, uint32_t win, int kind) {
+    const uint32_t e = lds16(tab + ((win >> (32 - kTabBits)) << 1));
+    return e ? e : long_code(tab, win, kind);
+}
+// number of blocks that an end of band covers
+__device__ __forceinline__ uint32_t eob_blocks(uint32_t e, uint32_t win) {
+    const uint32_t r = (e >> 9) & 15u;
+    return (1u << r) + shr0(shl0(win, (e & 31u) - r), 32u - r);
 }
 
-// Search pass of an AC first pass: the symbols that START in [pos, pos_end), from zigzag position k.
-// An undefined code is skipped by one bit and a coefficient beyond the band ends the block (the thread
-// is then reading from a wrong entry point and only has to arrive somewhere).
-__device__ __forceinline__ void ac_search_span(const HuffTab& tab, const uint16_t* slut, const uint32_t* base, uint32_t pos, int k,
-                                               uint32_t pos_end, int Ss, int Se, uint32_t& pos_out, int& k_out, uint32_t& nblk) {
-    GlobalBits B;
-    B.init(base, pos);
-    uint32_t nb = 0;
-    while (B.bits < pos_end) {
-        const uint32_t win = B.win();
-        uint32_t e = slut[win >> (32 - kLutBits)];
-        if (e == 0) {                                          // a code longer than the table's index, or none
-            e = ac_search_entry(huff_lookup(tab, win));
-            if (e == 0) { B.skip(1); continue; }
-        }
-        if (e & kSearchEob) {
-            const uint32_t r = e >> 10;
-            nb += r ? (1u << r) + ((win << ((e & 31u) - r)) >> (32u - r)) : 1u;
-            k = Ss;
-        } else {
-            const int nk = k + (int)((e >> 5) & 15u) + 1;
-            if (nk > Se) { ++nb; k = Ss; } else k = nk;
-        }
-        B.skip(e & 31u);
+// What a symbol does to the state, and how many blocks it finishes.
+struct DcSteps {
+    uint32_t tabs, tbits, bpm;     // shared address of two tables; bit j: the table of the MCU's block j; blocks per MCU
+    __device__ __forceinline__ uint32_t entry(uint32_t win, uint32_t st) const {
+        return long_entry(tabs + ((tbits >> st) & 1u) * (uint32_t)sizeof(ScanTab), win, kTabDc);
     }
-    pos_out = B.bits;
-    k_out = k;
-    nblk = nb;
-}
-
-// Search pass of a DC first pass.  dlut: per table, (length << 4) | size of the codes of at most kLutBits
-// bits; tbits: bit j = the table of the j-th block of an MCU; cpack: two bits per j = its component.
-__device__ __forceinline__ void dc_search_span(const HuffTab* tabs2, const uint8_t* dlut, uint32_t tbits, uint32_t cpack, int bpm,
-                                               const uint32_t* base, uint32_t pos, int j, uint32_t pos_end, uint32_t& pos_out,
-                                               int& j_out, uint32_t& nblk, int& sum0, int& sum1, int& sum2) {
-    GlobalBits B;
-    B.init(base, pos);
-    uint32_t nb = 0;
-    int s0 = 0, s1 = 0, s2 = 0;
-    while (B.bits < pos_end) {
-        const uint32_t win = B.win();
-        const uint32_t tsel = (tbits >> j) & 1u;
-        const uint32_t e = dlut[(tsel << kLutBits) + (win >> (32 - kLutBits))];
-        int len = (int)(e >> 4), sz = (int)(e & 15u);
-        if (e == 0) {
-            const uint32_t t = huff_lookup(tabs2[tsel], win);
-            len = (int)(t >> 8); sz = (int)(t & 255u);
-            if (t == 0 || sz > 15) { B.skip(1); continue; }
-        }
-        const int d = extend_bits(top_bits(win << len, sz), sz);
-        const uint32_t c = (cpack >> (2 * j)) & 3u;
-        s0 += c == 0u ? d : 0; s1 += c == 1u ? d : 0; s2 += c == 2u ? d : 0;
-        B.skip((uint32_t)(len + sz));
-        ++nb;
-        if (++j == bpm) j = 0;
+    __device__ __forceinline__ uint32_t next(uint32_t, uint32_t, uint32_t& st) const { st = st + 1u == bpm ? 0u : st + 1u; return 1u; }
+};
+struct AcSteps {
+    uint32_t tab, Ss, Se;
+    __device__ __forceinline__ uint32_t entry(uint32_t win, uint32_t) const { return long_entry(tab, win, kTabAcFirst); }
+    __device__ __forceinline__ uint32_t next(uint32_t e, uint32_t win, uint32_t& st) const {
+        if (e & kEntEob) { st = Ss; return eob_blocks(e, win); }
+        st += ((e >> 9) & 15u) + 1u;                                       // (sixteen zeros: run 15 plus one)
+        if (st <= Se) return 0u;
+        st = Ss;
+        return 1u;
     }
-    pos_out = B.bits;
-    j_out = j;
-    nblk = nb;
-    sum0 = s0; sum1 = s1; sum2 = s2;
-}
-
-// What one lane needs to write the coefficients of an AC first pass.
-struct AcWrite {
-    int16_t* headp;        // the component's head entries
-    int16_t* vals;         // the value array from position 0 of the stream words on
-    uint64_t* auxp;        // the scan's side data of the image's component
-    bool lists;            // the band reaches beyond position 7: side data of two words, values in the array
-    uint32_t mcu_w, bw;    // blocks per row of the scan's (unpadded) grid / of the padded grid
-    uint32_t m, m1;        // the block the entry position lies in, one past the scan's last
-    int Al;
+};
+struct SeqSteps {
+    uint32_t tabs, tdc, tac, bpm;  // shared address of the tables DC 0, DC 1, AC 0, AC 1; bit j: which of them block j uses
+    __device__ __forceinline__ uint32_t entry(uint32_t win, uint32_t st) const {
+        const uint32_t j = st >> 6;
+        const bool dc = (st & 63u) == 0;
+        return long_entry(tabs + (dc ? (tdc >> j) & 1u : 2u + ((tac >> j) & 1u)) * (uint32_t)sizeof(ScanTab), win, dc ? kTabDc : kTabAcSeq);
+    }
+    __device__ __forceinline__ uint32_t next(uint32_t e, uint32_t, uint32_t& st) const {
+        const uint32_t k = (st & 63u) + ((e >> 9) & 15u) + 1u, j = st >> 6;
+        if (!(e & kEntEob) && k <= 63u) { st = (st & ~63u) + k; return 0u; }
+        st = (j + 1u == bpm ? 0u : j + 1u) << 6;
+        return 1u;
+    }
 };
 
-// Decodes and writes the blocks of an AC first pass that BEGIN in [pos, pos_end), the last one to its end; k =
-// the zigzag position at pos (a block that began before pos is passed over: the thread before writes it).  So
-// every block has one writer and its values one run in the value array.  The entry state is the true one:
-// an undefined code or a coefficient beyond the band means a corrupt stream.  Every step consumes at least
-// one bit, so the loop ends.
-__device__ __forceinline__ void ac_write_span(const HuffTab& tab, const uint32_t* base, uint32_t pos, int k, uint32_t pos_end,
-                                              uint32_t endbit, int Ss, int Se, AcWrite& W, bool& bad) {
-    WordReader br;
-    br.init(base, pos);
-    bool own = k == Ss;                                        // this block is this thread's to write
-    uint32_t M0 = 0, M1 = 0;
-    int16_t* vp = W.vals + ((pos + 1u) >> 1);
-    int16_t* vb = vp;
-    uint32_t bcol = W.m % W.mcu_w, bi = (W.m / W.mcu_w) * W.bw + bcol;
-    while (W.m < W.m1) {
-        const uint32_t at = br.pos();
-        if (at >= endbit || (k == Ss && at >= pos_end)) break;
-        if (!own && at >= pos_end) break;                      // the whole span lies inside a block of an earlier thread
-        br.refill();
-        const uint32_t win = br.top32();
-        uint32_t e = tab.lut[win >> (32 - kLutBits)];
-        if (e == 0) e = huff_lookup(tab, win);
-        if (e == 0) { bad = true; break; }
-        const int len = (int)(e >> 8), r = (int)(e >> 4) & 15, sz = (int)(e & 15u);
-        const bool is_coef = sz != 0, is_eob = sz == 0 && r < 15;
-        const int kk = k + r;
-        if (is_coef && kk > Se) { bad = true; break; }
-        const int extra = is_coef ? sz : (is_eob ? r : 0);
-        const uint32_t xb = top_bits(win << len, extra);
-        br.skip(len + extra);
-        if (is_coef && own) {
-            const int16_t val = (int16_t)(extend_bits(xb, sz) << W.Al);
-            if (kk < 8) W.headp[(uint64_t)bi * 8 + kk] = val;
-            else *vp++ = val;
-            if (kk < 32) M0 |= 1u << kk; else M1 |= 1u << (kk - 32);
-        }
-        k = is_coef ? kk + 1 : (is_eob ? k : k + 16);
-        if (is_eob || k > Se) {                                // the block ends, an end-of-band run skips more
-            if (M0 | M1) {
-                if (W.lists) *reinterpret_cast<uint4*>(W.auxp + (uint64_t)bi * 2) = value_record(M0, M1, vb);
-                else *reinterpret_cast<uint2*>(W.auxp + bi) = make_uint2(M0, M1);
+// The symbols that START in [pos, pos_end) from state st.  Every step consumes at least one bit, so the loop ends; an
+// undefined code is passed over by one bit (the thread is then reading from a wrong state and only has to arrive
+// somewhere).  marks: shared address of this thread's places, one every `every` bits from `begin` on (kPitch bytes apart).
+constexpr uint32_t kMarks = 8;
+template <class Steps, uint32_t kPitch>
+__device__ __forceinline__ void search_span(const Steps& S, const uint32_t* base, uint32_t begin, uint32_t every, uint32_t marks,
+                                            uint32_t pos, uint32_t st, uint32_t pos_end, uint32_t& pos_x, uint32_t& st_x) {
+    uint32_t mark_at = begin + every;      // (a symbol is at most 31 bits, `every` at least 32: a step passes one place at most)
+    bool met = false;
+    // (the whole warp goes round together: left to itself the loop lets lanes that have passed a place drift apart and
+    // runs them one after the other, seven times slower)
+    while (__any_sync(0xffffffffu, pos < pos_end)) {
+        if (pos < pos_end) {
+            const uint32_t win = long_window(base, pos);
+            const uint32_t e = S.entry(win, st);
+            if (e) S.next(e, win, st);
+            pos += e ? e & 31u : 1u;
+            if (pos >= mark_at) {                                          // (also behind the end: no place keeps an older reading's state)
+                const uint32_t key = (pos << 9) + st;                      // (equal keys are equal states: pos stays inside the subsequence)
+                met = lds32(marks) == key;                                 // met the reading before: it ends where that one did
+                sts32(marks, key);
+                marks += kPitch; mark_at += every;
+                if (met) pos = pos_end;
             }
-            const uint32_t adv = is_eob ? (1u << r) + xb : 1u;
-            k = Ss;
-            M0 = 0; M1 = 0;
-            if (!own) vp = W.vals + ((br.pos() + 1u) >> 1);     // this thread's values begin where its first block does
-            vb = vp;
-            own = true;
-            if (adv >= W.m1 - W.m) break;
-            W.m += adv;
-            bcol += adv; bi += adv;
-            if (bcol >= W.mcu_w) { bcol = W.m % W.mcu_w; bi = (W.m / W.mcu_w) * W.bw + bcol; }
         }
     }
+    if (!met) { pos_x = pos; st_x = st; }
 }
 
-// The same for a DC first pass: one symbol (size category, then that many difference bits) per block;
-// j = the block's place in its MCU (Y00 Y01 Y10 Y11 Cb Cr, or always 0 in a one-component scan).
-struct DcWrite {
-    int16_t* dc;
-    uint64_t coff[3];
-    uint32_t bw[3];
-    uint32_t mcu_w;
-    uint32_t hs, vs;       // luminance blocks per MCU
-    uint32_t n, n1;        // next block of the scan in scan order, one past its last
-    int pred[3];
-    int Al;
+// Where the interval of a long scan lies, and this thread's subsequence.
+struct LongSpan {
+    const uint32_t* base;          // the stream's words
+    const uint32_t* origin;        // where they lie in the unstuffed copy
+    uint32_t lead, endbit;         // its first bit and the one behind its last, counted from the first word
+    uint32_t begin, end, every;
+    bool ok;
+    // stage: shared memory for kStage words (the caller synchronises behind this)
+    template <uint32_t kThreads, uint32_t kStage>
+    __device__ __forceinline__ void init(const Params& P, const ScanDesc& sd, uint32_t tid, uint32_t* stage) {
+        const uint32_t* segtab = P.seg_start + sd.seg_base;
+        const uint32_t bstart = segtab[0], bend = segtab[1] - 2u;
+        ok = !(bstart < sd.data_off || bend > sd.data_end || bend < bstart);   // (the same for every thread)
+        base = origin = reinterpret_cast<const uint32_t*>(P.ubuf) + (bstart >> 2);
+        lead = 8u * (bstart & 3u); endbit = ok ? lead + 8u * (bend - bstart) : lead;
+        // whole words, at least eight of them: eight places at least 32 bits apart
+        const uint32_t words = max(8u, ((endbit + 31u) / 32u + kThreads - 1u) / kThreads);
+        const uint32_t len = 32u * words;
+        every = max(32u, len / kMarks);
+        begin = min(max(tid * len, lead), endbit); end = min((tid + 1u) * len, endbit);
+        const uint32_t need = endbit / 32u + 3u;               // (a symbol may begin in the last bit)
+        if (need <= kStage) {
+            for (uint32_t i = tid; i < need; i += kThreads) stage[i] = __ldg(origin + i);
+            base = stage;
+        }
+    }
 };
-
-__device__ __forceinline__ void dc_write_span(const HuffTab* tabs2, uint32_t slots, bool inter, int c0, const uint32_t* base,
-                                              uint32_t pos, int j, uint32_t pos_end, DcWrite& W, bool& bad) {
-    WordReader br;
-    br.init(base, pos);
-    const int ny = (int)(W.hs * W.vs), bpm = inter ? ny + 2 : 1;
-    const uint32_t m = W.n / (uint32_t)bpm;
-    uint32_t mrow = m / W.mcu_w, mcol = m - mrow * W.mcu_w;
-    while (W.n < W.n1 && br.pos() < pos_end) {
-        br.refill();
-        const uint32_t win = br.top32();
-        const int ci = inter ? (j < ny ? 0 : j - ny + 1) : 0;
-        const int c = inter ? ci : c0;
-        const HuffTab& tab = tabs2[(slots >> (2 * ci)) & 1u];
-        const uint32_t e = huff_lookup(tab, win);
-        const int len = (int)(e >> 8), sz = (int)(e & 255u);
-        if (e == 0 || sz > 15) { bad = true; break; }
-        const int d = extend_bits(top_bits(win << len, sz), sz);
-        br.skip(len + sz);
-        const int pv = (c == 0 ? W.pred[0] : (c == 1 ? W.pred[1] : W.pred[2])) + d;
-        if (c == 0) W.pred[0] = pv; else if (c == 1) W.pred[1] = pv; else W.pred[2] = pv;
-        uint64_t blk;
-        if (inter && c == 0) blk = W.coff[0] + (uint64_t)(W.vs * mrow + ((uint32_t)j >> (W.hs - 1u))) * W.bw[0] + W.hs * mcol + ((uint32_t)j & (W.hs - 1u));
-        else blk = W.coff[c] + (uint64_t)mrow * W.bw[c] + mcol;
-        W.dc[blk] = (int16_t)(pv << W.Al);
-        ++W.n;
-        if (++j == bpm) {
-            j = 0;
-            if (++mcol == W.mcu_w) { mcol = 0; ++mrow; }
-        }
-    }
-}
 
 // Exclusive prefix sum over the CTA's threads in thread order (warp scans, then the warps' totals
 // through shared memory); total = the sum over all threads.  Every thread of the CTA calls it.
@@ -350,332 +222,303 @@ __device__ __forceinline__ T cta_exclusive_sum(T v, T* s_tmp, int wid, int lane,
     return before + inc - v;
 }
 
-// One CTA of kLongWarps warps per listed (scan, image) whose scan is one restart interval; first
-// passes only.  The interval is cut into 32 * kLongWarps subsequences, one per thread.
+// Search of the whole CTA: the true state at the start of every thread's subsequence, in pos and st.
+template <class Steps, int kWarps>
+__device__ __forceinline__ void search_all(const Steps& S, const LongSpan& L, uint32_t* s_marks, uint32_t* s_pos, uint32_t* s_state, uint32_t st0,
+                                           uint32_t& pos, uint32_t& st) {
+    constexpr uint32_t kThreads = 32 * kWarps;
+    const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
+    const unsigned full = 0xffffffffu;
+#pragma unroll
+    for (uint32_t i = 0; i < kMarks; ++i) s_marks[i * kThreads + tid] = 0xFFFFFFFFu;
+    const uint32_t marks = (uint32_t)__cvta_generic_to_shared(s_marks + tid);
+    uint32_t pos_x = L.begin, st_x = st0;
+    pos = L.begin; st = st0;
+    bool again = true;
+    for (uint32_t round = 0; round <= kThreads; ++round) {
+        if (__any_sync(full, again)) {
+            uint32_t x = pos_x, y = st_x;
+            search_span<Steps, 4 * kThreads>(S, L.base, L.begin, L.every, marks, pos, st, again ? L.end : 0u, x, y);
+            if (again) { pos_x = x; st_x = y; }
+        }
+        // the state the previous thread ended in (a warp's last lane's through shared memory)
+        if (lane == 31) { s_pos[wid] = pos_x; s_state[wid] = st_x; }
+        __syncthreads();
+        uint32_t ppos = __shfl_up_sync(full, pos_x, 1), pst = __shfl_up_sync(full, st_x, 1);
+        if (lane == 0 && wid > 0) { ppos = s_pos[wid - 1]; pst = s_state[wid - 1]; }
+        ppos = min(ppos, L.endbit);
+        again = tid > 0 && (ppos != pos || pst != st);
+        if (again) { pos = ppos; st = pst; }
+        if (!__syncthreads_or(again)) break;
+    }
+}
+
+// ---------------------------------------------------------------------------------------
+// First passes: one CTA of kLongWarps warps per listed (scan, image) whose scan is one restart interval.
+// ---------------------------------------------------------------------------------------
+#ifndef PCR_LONG_WARPS
+#define PCR_LONG_WARPS 2
+#endif
+constexpr int kLongWarps = PCR_LONG_WARPS;
+constexpr uint32_t kLongStage = 2048;         // words of a scan that are staged: 8 KB, a 600x450 image's scans have up to 6
+
+// Copies n of the (scan, image)'s tables to shared memory; the CTA's threads together.
+__device__ __forceinline__ void load_tabs(uint32_t dst, const ScanTab* src, int n, int tid, int threads) {
+    const uint4* a = reinterpret_cast<const uint4*>(src);
+    for (int i = tid; i < n * (int)(sizeof(ScanTab) / 16); i += threads) sts128(dst + 16u * i, __ldg(a + i));
+}
+
 __global__ void __launch_bounds__(32 * kLongWarps) first_pass_long_kernel(Params P, const uint32_t* __restrict__ list, uint32_t count) {
-    __shared__ HuffTab tabs[2];
-    __shared__ uint32_t s_pos[kLongWarps];                     // end state of every warp's last lane, for the next warp's first
-    __shared__ int s_state[kLongWarps];
-    __shared__ uint32_t s_u[kLongWarps];
+    constexpr int kThreads = 32 * kLongWarps;
+    __shared__ __align__(16) uint8_t s_tabs[2 * sizeof(ScanTab)];
+    __shared__ uint32_t s_stage[kLongStage];
+    __shared__ uint32_t s_marks[kMarks * kThreads];
+    __shared__ uint32_t s_pos[kLongWarps], s_state[kLongWarps], s_u[kLongWarps];
     __shared__ int s_i[kLongWarps];
-    __shared__ __align__(4) uint16_t s_lut[1 << kLutBits];    // the search pass's table (AC), or two byte tables (DC)
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
+    const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
     const uint32_t it = blockIdx.x;
     if (it >= count) return;                                   // whole CTA
     const uint32_t si = list[it];
     const int s = (int)(si / (uint32_t)P.N), img = (int)(si % (uint32_t)P.N);
-    const ScanDesc sd = P.scans[si];
+    const ScanDesc& sd = P.scans[si];
     const ScanScript sc = P.script[s];
-    const ImgDesc im = P.imgs[img];
-    const Geometry g = make_geometry(im, P);
+    const ScanAux ax = P.saux[s];
+    const Geometry g = make_geometry(P.imgs[img], P);
     const bool dc = sc.Ss == 0, inter = sc.ncomp > 1;
-    const int c0 = sc.comp[0];
+    const uint32_t c0 = (uint32_t)sc.comp[0];
     const uint32_t mcu_w = inter ? g.mx : g.ubw[c0];
-    const uint32_t mcu_h = inter ? g.my : g.ubh[c0];
-    const uint32_t total = mcu_w * mcu_h;                      // MCUs of the scan (one interval)
-    const unsigned full = 0xffffffffu;
-    if (wid == 0) build_hufftab(tabs[0], P.rec + sd.tab_off[0], lane);
-    if (wid == (kLongWarps > 1 ? 1 : 0) && sd.tab_off[1]) build_hufftab(tabs[1], P.rec + sd.tab_off[1], lane);
+    const uint32_t total = mcu_w * (inter ? g.my : g.ubh[c0]);  // MCUs of the scan (one interval)
+    const uint32_t tabs = (uint32_t)__cvta_generic_to_shared(s_tabs);
+    load_tabs(tabs, P.tabs + ax.tab0 + (uint32_t)img * (uint32_t)ax.ntab, dc && sd.tab_off[1] ? 2 : 1, tid, kThreads);
+    LongSpan L;
+    L.init<kThreads, kLongStage>(P, sd, (uint32_t)tid, s_stage);
     __syncthreads();
-    if (dc) {
-        uint8_t* dl = reinterpret_cast<uint8_t*>(s_lut);
-        for (int i = tid; i < (2 << kLutBits); i += 32 * kLongWarps) {
-            const uint32_t t = ((i >> kLutBits) == 0 || sd.tab_off[1]) ? tabs[i >> kLutBits].lut[i & ((1 << kLutBits) - 1)] : 0u;
-            dl[i] = (uint8_t)((t != 0 && (t & 255u) <= 15u) ? ((t >> 8) << 4) | (t & 15u) : 0u);
-        }
-    } else {
-        for (int i = tid; i < (1 << kLutBits); i += 32 * kLongWarps) s_lut[i] = (uint16_t)ac_search_entry(tabs[0].lut[i]);
-    }
-    __syncthreads();
-    const uint32_t* segtab = P.seg_start + sd.seg_base;
-    const uint32_t bstart = segtab[0], bend = segtab[1] - 2u;
-    if (bstart < sd.data_off || bend > sd.data_end || bend < bstart) {   // (the same for every thread)
+    if (!L.ok) {
         if (tid == 0) atomicMin(&P.status[img], kErrCorrupt);
         return;
     }
-    const uint32_t* base = reinterpret_cast<const uint32_t*>(P.ubuf) + (bstart >> 2);
-    const uint32_t lead = 8u * (bstart & 3u), endbit = lead + 8u * (bend - bstart);
-    // subsequences of S bits (whole words, at least 8 of them)
-    constexpr uint32_t kSubs = 32u * kLongWarps;
-    const uint32_t nwords = (endbit + 31u) >> 5;
-    const uint32_t S = 32u * max(8u, (nwords + kSubs - 1u) / kSubs);
-    const uint32_t my_begin = min(max((uint32_t)tid * S, lead), endbit), my_end = min(((uint32_t)tid + 1u) * S, endbit);
     bool bad = false;
-    // the state the previous thread ended in (its last lane's through shared memory for a warp's first lane)
-    auto handed_on = [&](uint32_t pos_x, int st_x, uint32_t& ppos, int& pst) {
-        if (lane == 31) { s_pos[wid] = pos_x; s_state[wid] = st_x; }
-        __syncthreads();
-        ppos = __shfl_up_sync(full, pos_x, 1);
-        pst = __shfl_up_sync(full, st_x, 1);
-        if (lane == 0 && wid > 0) { ppos = s_pos[wid - 1]; pst = s_state[wid - 1]; }
-        ppos = min(ppos, endbit);
-    };
+    uint32_t pos, st, all, nb = 0;
     if (dc) {
-        DcWrite W;
-        W.dc = P.dc; W.mcu_w = mcu_w; W.Al = sc.Al; W.hs = (uint32_t)P.hs; W.vs = (uint32_t)P.vs;
-        const uint32_t bpm = inter ? (uint32_t)(P.hs * P.vs + 2) : 1u;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) { W.coff[c] = g.coff[c]; W.bw[c] = g.bw[c]; W.pred[c] = 0; }
-        W.n = 0; W.n1 = total * bpm;
-        // per block of the MCU: its table (one bit) and its component (two bits)
-        uint32_t tbits = 0, cpack = 0;
-        for (uint32_t jj = 0; jj < bpm; ++jj) {
-            const uint32_t ny = (uint32_t)(P.hs * P.vs), ci = inter ? (jj < ny ? 0u : jj - ny + 1u) : 0u;
-            tbits |= ((sd.slots >> (2u * ci)) & 1u) << jj;
-            cpack |= (inter ? ci : (uint32_t)c0) << (2u * jj);
+        const uint32_t ny = (uint32_t)(P.hs * P.vs), bpm = inter ? ny + 2u : 1u, hs = (uint32_t)P.hs;
+        DcSteps S;
+        S.tabs = tabs; S.bpm = bpm; S.tbits = 0;
+        for (uint32_t j = 0; j < bpm; ++j) S.tbits |= ((sd.slots >> (2u * (inter && j >= ny ? j - ny + 1u : 0u))) & 1u) << j;
+        search_all<DcSteps, kLongWarps>(S, L, s_marks, s_pos, s_state, 0u, pos, st);
+        int sum0 = 0, sum1 = 0, sum2 = 0;
+        const uint32_t j1 = inter ? ny : 6u, j2 = inter ? ny + 1u : 6u;          // the chroma blocks' places
+        for (uint32_t p = pos, j = st; p < L.end;) {
+            const uint32_t win = long_window(L.base, p), e = S.entry(win, j);
+            if (!e) { ++p; continue; }
+            const int d = magnitude(win, e & 31u, e >> 5);
+            sum0 += j < j1 ? d : 0; sum1 += j == j1 ? d : 0; sum2 += j == j2 ? d : 0;
+            nb += S.next(e, win, j);
+            p += e & 31u;
         }
-        uint32_t pos = my_begin, pos_x = my_begin, nb = 0;
-        int j = 0, j_x = 0, a0 = 0, a1 = 0, a2 = 0;
-        bool again = true;
-        for (int round = 0; round <= (int)kSubs; ++round) {
-            if (again) dc_search_span(tabs, reinterpret_cast<const uint8_t*>(s_lut), tbits, cpack, (int)bpm, base, pos, j, my_end, pos_x, j_x, nb, a0, a1, a2);
-            uint32_t ppos; int pj;
-            handed_on(pos_x, j_x, ppos, pj);
-            again = tid > 0 && (ppos != pos || pj != j);
-            if (again) { pos = ppos; j = pj; }
-            if (!__syncthreads_or(again)) break;
-        }
-        // first block and predictors of every thread: exclusive prefix sums
-        uint32_t all;
-        int t0, t1, t2;
-        W.n = min(cta_exclusive_sum(nb, s_u, wid, lane, kLongWarps, all), W.n1);
-        W.pred[0] = cta_exclusive_sum(a0, s_i, wid, lane, kLongWarps, t0);
-        W.pred[1] = cta_exclusive_sum(a1, s_i, wid, lane, kLongWarps, t1);
-        W.pred[2] = cta_exclusive_sum(a2, s_i, wid, lane, kLongWarps, t2);
+        int t;
+        uint32_t n = cta_exclusive_sum(nb, s_u, wid, lane, kLongWarps, all);
+        int pred0 = cta_exclusive_sum(sum0, s_i, wid, lane, kLongWarps, t);
+        int pred1 = cta_exclusive_sum(sum1, s_i, wid, lane, kLongWarps, t);
+        int pred2 = cta_exclusive_sum(sum2, s_i, wid, lane, kLongWarps, t);
+        const uint32_t n1 = total * bpm;
+        n = min(n, n1);
         // the place inside the MCU follows from the block number (equal to the handed-on state unless
         // the stream is damaged; taking it from the block number keeps every store inside the image)
-        if (nb && (uint32_t)j != W.n % bpm) bad = true;
-        j = (int)(W.n % bpm);
-        dc_write_span(tabs, sd.slots, inter, c0, base, pos, j, my_end, W, bad);
-        if (all < total * bpm) bad = true;                     // the stream ends before the last block
-    } else {
-        const int c = c0, Ss = sc.Ss, Se = sc.Se;
-        const ScanAux ax = P.saux[s];
-        AcWrite W;
-        W.headp = P.head + g.coff[c] * 8; W.vals = P.vals + 16ull * (bstart >> 2);
-        W.auxp = P.aux + ax.base + g.loff[c] * ax.stride; W.lists = ax.stride == 2u;
-        W.mcu_w = mcu_w; W.bw = g.bw[c]; W.m = 0; W.m1 = total; W.Al = sc.Al;
-        const HuffTab& tab = tabs[0];
-        uint32_t pos = my_begin, pos_x = my_begin, nb = 0;
-        int k = Ss, k_x = Ss;
-        bool again = true;
-        for (int round = 0; round <= (int)kSubs; ++round) {
-            if (again) ac_search_span(tab, s_lut, base, pos, k, my_end, Ss, Se, pos_x, k_x, nb);
-            uint32_t ppos; int pk;
-            handed_on(pos_x, k_x, ppos, pk);
-            again = tid > 0 && (ppos != pos || pk != k);
-            if (again) { pos = ppos; k = pk; }
-            if (!__syncthreads_or(again)) break;
+        if (nb && st != n % bpm) bad = true;
+        uint32_t j = n % bpm, m = n / bpm, mcol = m % mcu_w;
+        uint32_t yb = inter ? (uint32_t)P.vs * (m / mcu_w) * g.bw[0] + hs * mcol : (m / mcu_w) * g.bw[c0] + mcol;
+        int16_t* const yp = P.dc + g.coff[inter ? 0 : c0];
+        int16_t* const cp = P.dc + g.coff[1];
+        const uint32_t c_step = g.mx * g.my, step = inter ? hs : 1u;
+        const uint32_t wrap = (inter ? (uint32_t)P.vs * g.bw[0] : g.bw[c0]) - step * mcu_w;
+        for (uint32_t p = pos; p < L.end && n < n1; ++n) {
+            const uint32_t win = long_window(L.base, p), e = S.entry(win, j);
+            if (!e) { bad = true; break; }
+            const int d = magnitude(win, e & 31u, e >> 5);
+            p += e & 31u;
+            if (j < j1) {
+                pred0 += d;
+                yp[yb + (inter ? (j >> (hs - 1u)) * g.bw[0] + (j & (hs - 1u)) : 0u)] = (int16_t)(pred0 << sc.Al);
+            } else {
+                const bool first = j == j1;
+                const int v = d + (first ? pred1 : pred2);
+                if (first) pred1 = v; else pred2 = v;
+                cp[m + (first ? 0u : c_step)] = (int16_t)(v << sc.Al);
+            }
+            if (++j == bpm) {
+                j = 0; ++m;
+                yb += step;
+                if (++mcol == mcu_w) { mcol = 0; yb += wrap; }
+            }
         }
-        uint32_t all;
-        W.m = min(cta_exclusive_sum(nb, s_u, wid, lane, kLongWarps, all), total);
-        ac_write_span(tab, base, pos, k, my_end, endbit, Ss, Se, W, bad);
-        if (all < total) bad = true;                                         // the stream ends before the last block
+        if (all < n1) bad = true;                              // the stream ends before the last block
+    } else {
+        AcSteps S;
+        S.tab = tabs; S.Ss = (uint32_t)sc.Ss; S.Se = (uint32_t)sc.Se;
+        search_all<AcSteps, kLongWarps>(S, L, s_marks, s_pos, s_state, S.Ss, pos, st);
+        for (uint32_t p = pos, k = st; p < L.end;) {
+            const uint32_t win = long_window(L.base, p), e = S.entry(win, k);
+            if (!e) { ++p; continue; }
+            nb += S.next(e, win, k);
+            p += e & 31u;
+        }
+        uint32_t m = min(cta_exclusive_sum(nb, s_u, wid, lane, kLongWarps, all), total);
+        if (all < total) bad = true;                           // the stream ends before the last block
+        // The blocks that BEGIN in this subsequence, the last one to its end; a block that began before it is passed over
+        // (the thread before writes it).  So every block has one writer and its values one run in the value
+        // array.  What the state at `pos` says is true: an undefined code or a coefficient beyond the band means a
+        // corrupt stream.
+        const uint32_t Ss = S.Ss, Se = S.Se, bw = g.bw[c0];
+        int16_t* const headp = P.head + g.coff[c0] * 8;
+        int16_t* const vals = P.vals + 16ll * (L.origin - reinterpret_cast<const uint32_t*>(P.ubuf));
+        uint64_t* const auxp = P.aux + ax.base + g.loff[c0] * ax.stride;
+        const bool lists = ax.stride == 2u;                    // the band reaches beyond position 7
+        uint32_t k = st, M0 = 0, M1 = 0, lim = L.end;
+        bool own = k == Ss;
+        int16_t* vp = vals + ((pos + 1u) >> 1);
+        int16_t* vb = vp;
+        uint32_t bcol = m % mcu_w, bi = (m / mcu_w) * bw + bcol;
+        for (uint32_t p = pos; p < lim && m < total;) {
+            const uint32_t win = long_window(L.base, p), e = S.entry(win, k);
+            const uint32_t skip = e & 31u, sz = (e >> 5) & 15u;
+            p += skip;
+            k += (e >> 9) & 15u;                               // position of the coefficient
+            const bool eob = (e & kEntEob) != 0, coef = sz && own;
+            if (e == 0 || (sz && k > Se)) { bad = true; break; }
+            const int val = magnitude(win, skip, sz) << sc.Al;
+            if (coef && k < 8u) headp[8u * (uint64_t)bi + k] = (int16_t)val;
+            if (coef && k >= 8u) *vp = (int16_t)val;
+            vp += coef && k >= 8u ? 1 : 0;
+            M0 |= shl0(coef ? 1u : 0u, k); M1 |= shl0(coef ? 1u : 0u, k - 32u);
+            ++k;
+            if (own) lim = L.endbit;
+            if (eob || k > Se) {                               // the block ends, an end-of-band run skips more
+                if (M0 | M1) {
+                    if (lists) *reinterpret_cast<uint4*>(auxp + (uint64_t)bi * 2) = value_record(M0, M1, vb);
+                    else *reinterpret_cast<uint2*>(auxp + bi) = make_uint2(M0, M1);
+                }
+                k = Ss; M0 = 0; M1 = 0; lim = L.end;
+                if (!own) vp = vals + ((p + 1u) >> 1);         // this thread's values begin where its first block does
+                vb = vp;
+                own = true;
+                const uint32_t adv = eob ? eob_blocks(e, win) : 1u;
+                if (adv >= total - m) break;
+                m += adv; bcol += adv; bi += adv;
+                if (bcol >= mcu_w) { bcol = m % mcu_w; bi = (m / mcu_w) * bw + bcol; }
+            }
+        }
     }
     if (__syncthreads_or(bad) && tid == 0) atomicMin(&P.status[img], kErrCorrupt);
 }
 
 // ---------------------------------------------------------------------------------------
-// A sequential (baseline) scan that is one restart interval: the same scheme as the first passes.
-// The state a lane hands on is (bit position, block of the MCU, zigzag position inside the block;
-// 0 = the block's DC symbol comes next); every lane counts the blocks it finishes and sums the DC
-// differences it reads per component.
+// A sequential (baseline) scan that is one restart interval: one CTA of kSeqLongWarps warps per listed image.
 // ---------------------------------------------------------------------------------------
-struct SeqWrite {
-    int16_t* dc;
-    int16_t* head;
-    int16_t* vals;         // the value array from position 0 of the stream words on
-    uint64_t* auxp;        // the scan's side data
-    uint64_t coff[3];
-    uint32_t bw[3];
-    uint32_t mcu_w;
-    uint32_t hs, vs;
-    uint32_t n, n1;        // next block of the scan in scan order (the one being decoded), one past the last
-    int pred[3];
-};
-
-// a symbol of a sequential scan: false if there is none such (k, j: where the reader stands)
-struct SeqSymbol { int len, r, sz; bool is_coef, is_zrl, is_eob; };
-__device__ __forceinline__ bool seq_symbol(const HuffTab* tabs4, uint32_t slots, uint32_t slots_ac, int c, int k, uint32_t win, SeqSymbol& y) {
-    const bool is_dc = k == 0;
-    const int ti = is_dc ? (int)((slots >> (2 * c)) & 1u) : 2 + (int)((slots_ac >> (2 * c)) & 1u);
-    const uint32_t e = huff_lookup(tabs4[ti], win);
-    y.len = (int)(e >> 8); y.r = is_dc ? 0 : (int)(e >> 4) & 15; y.sz = is_dc ? (int)(e & 255u) : (int)(e & 15u);
-    y.is_coef = y.sz != 0; y.is_zrl = !is_dc && y.sz == 0 && y.r == 15; y.is_eob = !is_dc && y.sz == 0 && y.r == 0;
-    return !(e == 0 || y.sz > 15 || (!is_dc && !y.is_coef && !y.is_zrl && !y.is_eob) || (y.is_coef && k + y.r > 63));
-}
-
-// Search pass: from state (pos, j, k) to the end of the span (see the header comment); counts the blocks it
-// finishes and sums the DC differences it reads.
-__device__ __forceinline__ void seq_search_span(const HuffTab* tabs4, uint32_t slots, uint32_t slots_ac, int nc, uint32_t ny_, const uint32_t* base,
-                                                uint32_t pos, int j, int k, uint32_t pos_end, uint32_t& pos_out, int& j_out, int& k_out,
-                                                uint32_t& nblk, int& sum0, int& sum1, int& sum2) {
-    WordReader br;
-    br.init(base, pos);
-    const int ny = (int)ny_, bpm = nc == 3 ? ny + 2 : 1;
-    uint32_t nb = 0;
-    int s0 = 0, s1 = 0, s2 = 0;
-    while (br.pos() < pos_end) {
-        br.refill();
-        const uint32_t win = br.top32();
-        const int c = nc == 3 ? (j < ny ? 0 : j - ny + 1) : 0;
-        SeqSymbol y;
-        if (!seq_symbol(tabs4, slots, slots_ac, c, k, win, y)) { br.skip(1); continue; }
-        br.skip(y.len + y.sz);
-        if (k == 0) {
-            const int v = extend_bits(top_bits(win << y.len, y.sz), y.sz);
-            if (c == 0) s0 += v; else if (c == 1) s1 += v; else s2 += v;
-            k = 1;
-        } else if (y.is_coef) k += y.r + 1;
-        else if (y.is_zrl) k += 16;
-        if (y.is_eob || k > 63) {                             // block finished
-            k = 0;
-            ++nb;
-            if (++j == bpm) j = 0;
-        }
-    }
-    pos_out = br.pos();
-    j_out = j;
-    k_out = k;
-    nblk = nb;
-    sum0 = s0; sum1 = s1; sum2 = s2;
-}
-
-// Decodes and writes the blocks that BEGIN in [pos, pos_end), the last one to its end (see ac_write_span).
-__device__ __forceinline__ void seq_write_span(const HuffTab* tabs4, uint32_t slots, uint32_t slots_ac, int nc, const uint32_t* base,
-                                               uint32_t pos, int j, int k, uint32_t pos_end, uint32_t endbit, SeqWrite& W, bool& bad) {
-    WordReader br;
-    br.init(base, pos);
-    const int ny = (int)(W.hs * W.vs), bpm = nc == 3 ? ny + 2 : 1;
-    bool own = k == 0;
-    uint32_t M0 = 0, M1 = 0;
-    int16_t* vp = W.vals + ((pos + 1u) >> 1);
-    int16_t* vb = vp;
-    const uint32_t m = W.n / (uint32_t)bpm;
-    uint32_t mrow = m / W.mcu_w, mcol = m - mrow * W.mcu_w;
-    while (W.n < W.n1) {
-        const uint32_t at = br.pos();
-        if (at >= endbit || ((k == 0 || !own) && at >= pos_end)) break;
-        br.refill();
-        const uint32_t win = br.top32();
-        const int c = nc == 3 ? (j < ny ? 0 : j - ny + 1) : 0;
-        SeqSymbol y;
-        if (!seq_symbol(tabs4, slots, slots_ac, c, k, win, y)) { bad = true; break; }
-        const int v = extend_bits(top_bits(win << y.len, y.sz), y.sz), kk = k + y.r;
-        br.skip(y.len + y.sz);
-        const uint32_t local = (nc == 3 && c == 0) ? (W.vs * mrow + ((uint32_t)j >> (W.hs - 1u))) * W.bw[0] + W.hs * mcol + ((uint32_t)j & (W.hs - 1u))
-                                                   : mrow * W.bw[c] + mcol;
-        const uint64_t blk = W.coff[c] + local;
-        if (k == 0) {
-            const int pv = (c == 0 ? W.pred[0] : (c == 1 ? W.pred[1] : W.pred[2])) + v;
-            if (c == 0) W.pred[0] = pv; else if (c == 1) W.pred[1] = pv; else W.pred[2] = pv;
-            W.dc[blk] = (int16_t)pv;
-            k = 1;
-        } else if (y.is_coef) {
-            if (own) {
-                if (kk < 8) W.head[blk * 8 + kk] = (int16_t)v;
-                else {
-                    *vp++ = (int16_t)v;
-                    if (kk < 32) M0 |= 1u << kk; else M1 |= 1u << (kk - 32);
-                }
-            }
-            k = kk + 1;
-        } else if (y.is_zrl) {
-            k += 16;
-        }
-        if (y.is_eob || k > 63) {                             // block finished
-            if (M0 | M1) *reinterpret_cast<uint4*>(W.auxp + 2ull * blk) = value_record(M0, M1, vb);
-            k = 0; M0 = 0; M1 = 0;
-            if (!own) vp = W.vals + ((br.pos() + 1u) >> 1);
-            vb = vp;
-            own = true;
-            ++W.n;
-            if (++j == bpm) {
-                j = 0;
-                if (++mcol == W.mcu_w) { mcol = 0; ++mrow; }
-            }
-        }
-    }
-}
-
 #ifndef PCR_SEQ_LONG_WARPS
 #define PCR_SEQ_LONG_WARPS 4
 #endif
-constexpr int kSeqLongWarps = PCR_SEQ_LONG_WARPS;   // warps per image in sequential_long_kernel: 32 subsequences each
+constexpr int kSeqLongWarps = PCR_SEQ_LONG_WARPS;
+constexpr uint32_t kSeqLongStage = 6144;      // 24 KB
 
-// One CTA of kSeqLongWarps warps per listed image whose (one) sequential scan is one restart interval.
 __global__ void __launch_bounds__(32 * kSeqLongWarps) sequential_long_kernel(Params P, const uint32_t* __restrict__ list, uint32_t count) {
-    __shared__ HuffTab tabs[4];                                // DC 0, DC 1, AC 0, AC 1
-    __shared__ uint32_t s_pos[kSeqLongWarps];                  // end state of every warp's last lane, for the next warp's first
-    __shared__ int s_state[kSeqLongWarps];
-    __shared__ uint32_t s_u[kSeqLongWarps];
+    constexpr int kThreads = 32 * kSeqLongWarps;
+    __shared__ __align__(16) uint8_t s_tabs[4 * sizeof(ScanTab)];
+    __shared__ uint32_t s_stage[kSeqLongStage];
+    __shared__ uint32_t s_marks[kMarks * kThreads];
+    __shared__ uint32_t s_pos[kSeqLongWarps], s_state[kSeqLongWarps], s_u[kSeqLongWarps];
     __shared__ int s_i[kSeqLongWarps];
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
+    const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
     const uint32_t it = blockIdx.x;
     if (it >= count) return;                                   // whole CTA
     const uint32_t si = list[it];
     const int img = (int)(si % (uint32_t)P.N);
-    const ScanDesc sd = P.scans[si];
-    const ImgDesc im = P.imgs[img];
-    const Geometry g = make_geometry(im, P);
-    const uint32_t mcu_w = g.mx, total = g.mx * g.my;
-    const uint32_t bpm = P.nc == 3 ? (uint32_t)(P.hs * P.vs + 2) : 1u;
-    const unsigned full = 0xffffffffu;
-    // four tables, built by the warps in turn
-    for (int t = wid; t < 4; t += kSeqLongWarps) {
-        const uint32_t off = t == 0 ? sd.tab_off[0] : (t == 1 ? sd.tab_off[1] : (t == 2 ? sd.tab_ac[0] : sd.tab_ac[1]));
-        if (off) build_hufftab(tabs[t], P.rec + off, lane);
+    const ScanDesc& sd = P.scans[si];
+    const ScanAux ax = P.saux[si / (uint32_t)P.N];
+    const Geometry g = make_geometry(P.imgs[img], P);
+    const uint32_t mcu_w = g.mx, total = g.mx * g.my, ny = (uint32_t)(P.hs * P.vs), hs = (uint32_t)P.hs, vs = (uint32_t)P.vs;
+    const uint32_t bpm = P.nc == 3 ? ny + 2u : 1u;
+    SeqSteps S;
+    S.tabs = (uint32_t)__cvta_generic_to_shared(s_tabs); S.bpm = bpm; S.tdc = 0; S.tac = 0;
+    for (uint32_t j = 0; j < bpm; ++j) {
+        const uint32_t c = j < ny ? 0u : j - ny + 1u;
+        S.tdc |= ((sd.slots >> (2u * c)) & 1u) << j; S.tac |= ((sd.slots_ac >> (2u * c)) & 1u) << j;
     }
+    load_tabs(S.tabs, P.tabs + ax.tab0 + 4u * (uint32_t)img, 4, tid, kThreads);
+    LongSpan L;
+    L.init<kThreads, kSeqLongStage>(P, sd, (uint32_t)tid, s_stage);
     __syncthreads();
-    const uint32_t* segtab = P.seg_start + sd.seg_base;
-    const uint32_t bstart = segtab[0], bend = segtab[1] - 2u;
-    if (bstart < sd.data_off || bend > sd.data_end || bend < bstart) {   // (the same for every thread)
+    if (!L.ok) {
         if (tid == 0) atomicMin(&P.status[img], kErrCorrupt);
         return;
     }
-    const uint32_t* base = reinterpret_cast<const uint32_t*>(P.ubuf) + (bstart >> 2);
-    const uint32_t lead = 8u * (bstart & 3u), endbit = lead + 8u * (bend - bstart);
-    constexpr uint32_t kSubs = 32u * kSeqLongWarps;
-    const uint32_t nwords = (endbit + 31u) >> 5;
-    const uint32_t S = 32u * max(8u, (nwords + kSubs - 1u) / kSubs);
-    const uint32_t my_begin = min(max((uint32_t)tid * S, lead), endbit), my_end = min(((uint32_t)tid + 1u) * S, endbit);
     bool bad = false;
-    SeqWrite W;
-    const ScanAux ax = P.saux[si / (uint32_t)P.N];
-    W.dc = P.dc; W.head = P.head; W.vals = P.vals + 16ull * (bstart >> 2); W.mcu_w = mcu_w; W.hs = (uint32_t)P.hs; W.vs = (uint32_t)P.vs;
-    W.auxp = P.aux + ax.base;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) { W.coff[c] = g.coff[c]; W.bw[c] = g.bw[c]; W.pred[c] = 0; }
-    W.n = 0; W.n1 = total * bpm;
-    uint32_t pos = my_begin, pos_x = my_begin, nb = 0;
-    int j = 0, k = 0, j_x = 0, k_x = 0, a0 = 0, a1 = 0, a2 = 0;
-    bool again = true;
-    for (int round = 0; round <= (int)kSubs; ++round) {
-        if (again) seq_search_span(tabs, sd.slots, sd.slots_ac, P.nc, W.hs * W.vs, base, pos, j, k, my_end, pos_x, j_x, k_x, nb, a0, a1, a2);
-        // the state the previous thread ended in (block of the MCU and zigzag position in one word)
-        const int st_x = j_x * 64 + k_x;
-        if (lane == 31) { s_pos[wid] = pos_x; s_state[wid] = st_x; }
-        __syncthreads();
-        uint32_t ppos = __shfl_up_sync(full, pos_x, 1);
-        int pst = __shfl_up_sync(full, st_x, 1);
-        if (lane == 0 && wid > 0) { ppos = s_pos[wid - 1]; pst = s_state[wid - 1]; }
-        ppos = min(ppos, endbit);
-        again = tid > 0 && (ppos != pos || pst != j * 64 + k);
-        if (again) { pos = ppos; j = pst >> 6; k = pst & 63; }
-        if (!__syncthreads_or(again)) break;
+    uint32_t pos, st, all, nb = 0;
+    search_all<SeqSteps, kSeqLongWarps>(S, L, s_marks, s_pos, s_state, 0u, pos, st);
+    int sum0 = 0, sum1 = 0, sum2 = 0;
+    for (uint32_t p = pos, q = st; p < L.end;) {
+        const uint32_t win = long_window(L.base, p), e = S.entry(win, q), j = q >> 6;
+        if (!e) { ++p; continue; }
+        const int d = (q & 63u) == 0 ? magnitude(win, e & 31u, (e >> 5) & 15u) : 0;
+        sum0 += j < ny ? d : 0; sum1 += j == ny ? d : 0; sum2 += j > ny ? d : 0;
+        nb += S.next(e, win, q);
+        p += e & 31u;
     }
-    uint32_t all;
-    int t0, t1, t2;
-    W.n = min(cta_exclusive_sum(nb, s_u, wid, lane, kSeqLongWarps, all), W.n1);
-    W.pred[0] = cta_exclusive_sum(a0, s_i, wid, lane, kSeqLongWarps, t0);
-    W.pred[1] = cta_exclusive_sum(a1, s_i, wid, lane, kSeqLongWarps, t1);
-    W.pred[2] = cta_exclusive_sum(a2, s_i, wid, lane, kSeqLongWarps, t2);
-    // the place inside the MCU follows from the block number (equal to the handed-on state unless the
-    // stream is damaged; taking it from the block number keeps every store inside the image)
-    if ((nb || k) && (uint32_t)j != W.n % bpm) bad = true;
-    j = (int)(W.n % bpm);
-    seq_write_span(tabs, sd.slots, sd.slots_ac, P.nc, base, pos, j, k, my_end, endbit, W, bad);
-    if (all < total * bpm) bad = true;                         // the stream ends before the last block
+    int t;
+    uint32_t n = cta_exclusive_sum(nb, s_u, wid, lane, kSeqLongWarps, all);
+    int pred0 = cta_exclusive_sum(sum0, s_i, wid, lane, kSeqLongWarps, t);
+    int pred1 = cta_exclusive_sum(sum1, s_i, wid, lane, kSeqLongWarps, t);
+    int pred2 = cta_exclusive_sum(sum2, s_i, wid, lane, kSeqLongWarps, t);
+    const uint32_t n1 = total * bpm;
+    n = min(n, n1);
+    // (as for the DC scans above)
+    if ((nb || (st & 63u)) && (st >> 6) != n % bpm) bad = true;
+    if (all < n1) bad = true;                                  // the stream ends before the last block
+    // the blocks that BEGIN in this subsequence (see above); a DC symbol is written by the thread that has it
+    int16_t* const dcp = P.dc + g.coff[0];
+    int16_t* const headp = P.head + g.coff[0] * 8;
+    int16_t* const vals = P.vals + 16ll * (L.origin - reinterpret_cast<const uint32_t*>(P.ubuf));
+    uint64_t* const auxp = P.aux + ax.base + 2 * g.coff[0];
+    uint32_t j = n % bpm, k = st & 63u, m = n / bpm, mcol = m % mcu_w, M0 = 0, M1 = 0, lim = L.end;
+    uint32_t yb = vs * (m / mcu_w) * g.bw[0] + hs * mcol;
+    const uint32_t wrap = (vs - 1u) * g.bw[0];
+    bool own = k == 0;
+    int16_t* vp = vals + ((pos + 1u) >> 1);
+    int16_t* vb = vp;
+    for (uint32_t p = pos; p < lim && n < n1;) {
+        const uint32_t win = long_window(L.base, p), e = S.entry(win, (j << 6) + k);
+        const uint32_t skip = e & 31u, sz = (e >> 5) & 15u;
+        const uint32_t blk = j < ny ? yb + (j >> (hs - 1u)) * g.bw[0] + (j & (hs - 1u)) : (ny + j - ny) * total + m;
+        p += skip;
+        const bool is_dc = k == 0;
+        k += (e >> 9) & 15u;
+        if (e == 0 || (sz && k > 63u)) { bad = true; break; }
+        int v = magnitude(win, skip, sz);
+        if (is_dc) {
+            v += j < ny ? pred0 : (j == ny ? pred1 : pred2);
+            if (j < ny) pred0 = v; else if (j == ny) pred1 = v; else pred2 = v;
+            dcp[blk] = (int16_t)v;
+        }
+        const bool coef = sz && own && !is_dc;
+        if (coef && k < 8u) headp[8u * (uint64_t)blk + k] = (int16_t)v;
+        if (coef && k >= 8u) *vp = (int16_t)v;
+        vp += coef && k >= 8u ? 1 : 0;
+        M0 |= shl0(coef && k >= 8u ? 1u : 0u, k); M1 |= shl0(coef ? 1u : 0u, k - 32u);
+        ++k;
+        if (own) lim = L.endbit;
+        if ((e & kEntEob) || k > 63u) {                        // block finished
+            if (M0 | M1) *reinterpret_cast<uint4*>(auxp + 2ull * blk) = value_record(M0, M1, vb);
+            k = 0; M0 = 0; M1 = 0; lim = L.end;
+            if (!own) vp = vals + ((p + 1u) >> 1);
+            vb = vp;
+            own = true;
+            ++n;
+            if (++j == bpm) {
+                j = 0; ++m;
+                yb += hs;
+                if (++mcol == mcu_w) { mcol = 0; yb += wrap; }
+            }
+        }
+    }
     if (__syncthreads_or(bad) && tid == 0) atomicMin(&P.status[img], kErrCorrupt);
 }
 

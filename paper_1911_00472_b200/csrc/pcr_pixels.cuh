@@ -349,8 +349,8 @@ pixel_kernel(Params P, CoefLists cl, uint8_t* __restrict__ out) {
             constexpr uint64_t kIn = Corner<N>::mask;
             uint32_t v[N][N];                                         // [column][row]
 #pragma unroll
-            for (int k = 4 * kWords; k < 64; ++k)
-                if ((kIn >> k) & 1u) v[kZigzag.nat[k] & 7][kZigzag.nat[k] >> 3] = 0;
+            for (int k = 0; k < 64; ++k)
+                if (k >= 4 * kWords && ((kIn >> k) & 1u)) v[kZigzag.nat[k] & 7][kZigzag.nat[k] >> 3] = 0;
 #pragma unroll
             for (int w = 0; w < kWords; ++w) {
                 uint32_t f[4];
