@@ -111,37 +111,43 @@ __device__ __forceinline__ uint32_t eob_blocks(uint32_t e, uint32_t win) {
     return (1u << r) + shr0(shl0(win, (e & 31u) - r), 32u - r);
 }
 
-// What a symbol does to the state, and how many blocks it finishes.
+// The symbol at a position (its entry as in ScanTab, 0 = none), and what it does to the state: true if a block ends.
 struct DcSteps {
-    uint32_t tabs, tbits, bpm;     // shared address of two tables; bit j: the table of the MCU's block j; blocks per MCU
-    __device__ __forceinline__ uint32_t entry(uint32_t win, uint32_t st) const {
-        return long_entry(tabs + ((tbits >> st) & 1u) * (uint32_t)sizeof(ScanTab), win, kTabDc);
+    const uint32_t* base;
+    uint32_t tabs;                 // shared address of two tables
+    uint32_t tbits, bpm;           // bit j: the table of the MCU's block j; blocks per MCU
+    __device__ __forceinline__ uint32_t entry(uint32_t pos, uint32_t st) const {
+        const uint32_t t = (tbits >> st) & 1u;
+        return long_entry(tabs + t * (uint32_t)sizeof(ScanTab), long_window(base, pos), kTabDc);
     }
-    __device__ __forceinline__ uint32_t next(uint32_t, uint32_t, uint32_t& st) const { st = st + 1u == bpm ? 0u : st + 1u; return 1u; }
+    __device__ __forceinline__ bool advance(uint32_t, uint32_t& st) const { st = st + 1u == bpm ? 0u : st + 1u; return true; }
 };
 struct AcSteps {
-    uint32_t tab, Ss, Se;
-    __device__ __forceinline__ uint32_t entry(uint32_t win, uint32_t) const { return long_entry(tab, win, kTabAcFirst); }
-    __device__ __forceinline__ uint32_t next(uint32_t e, uint32_t win, uint32_t& st) const {
-        if (e & kEntEob) { st = Ss; return eob_blocks(e, win); }
+    const uint32_t* base;
+    uint32_t tabs, Ss, Se;
+    __device__ __forceinline__ uint32_t entry(uint32_t pos, uint32_t) const {
+        return long_entry(tabs, long_window(base, pos), kTabAcFirst);
+    }
+    __device__ __forceinline__ bool advance(uint32_t e, uint32_t& st) const {
         st += ((e >> 9) & 15u) + 1u;                                       // (sixteen zeros: run 15 plus one)
-        if (st <= Se) return 0u;
-        st = Ss;
-        return 1u;
+        const bool end = (e & kEntEob) || st > Se;
+        st = end ? Ss : st;
+        return end;
     }
 };
 struct SeqSteps {
+    const uint32_t* base;
     uint32_t tabs, tdc, tac, bpm;  // shared address of the tables DC 0, DC 1, AC 0, AC 1; bit j: which of them block j uses
-    __device__ __forceinline__ uint32_t entry(uint32_t win, uint32_t st) const {
+    __device__ __forceinline__ uint32_t entry(uint32_t pos, uint32_t st) const {
         const uint32_t j = st >> 6;
         const bool dc = (st & 63u) == 0;
-        return long_entry(tabs + (dc ? (tdc >> j) & 1u : 2u + ((tac >> j) & 1u)) * (uint32_t)sizeof(ScanTab), win, dc ? kTabDc : kTabAcSeq);
+        return long_entry(tabs + (dc ? (tdc >> j) & 1u : 2u + ((tac >> j) & 1u)) * (uint32_t)sizeof(ScanTab), long_window(base, pos), dc ? kTabDc : kTabAcSeq);
     }
-    __device__ __forceinline__ uint32_t next(uint32_t e, uint32_t, uint32_t& st) const {
+    __device__ __forceinline__ bool advance(uint32_t e, uint32_t& st) const {
         const uint32_t k = (st & 63u) + ((e >> 9) & 15u) + 1u, j = st >> 6;
-        if (!(e & kEntEob) && k <= 63u) { st = (st & ~63u) + k; return 0u; }
-        st = (j + 1u == bpm ? 0u : j + 1u) << 6;
-        return 1u;
+        const bool end = (e & kEntEob) || k > 63u;
+        st = end ? (j + 1u == bpm ? 0u : j + 1u) << 6 : (st & ~63u) + k;
+        return end;
     }
 };
 
@@ -150,28 +156,31 @@ struct SeqSteps {
 // somewhere).  marks: shared address of this thread's places, one every `every` bits from `begin` on (kPitch bytes apart).
 constexpr uint32_t kMarks = 8;
 template <class Steps, uint32_t kPitch>
-__device__ __forceinline__ void search_span(const Steps& S, const uint32_t* base, uint32_t begin, uint32_t every, uint32_t marks,
+__device__ __forceinline__ void search_span(const Steps& S, uint32_t begin, uint32_t every, uint32_t marks,
                                             uint32_t pos, uint32_t st, uint32_t pos_end, uint32_t& pos_x, uint32_t& st_x) {
-    uint32_t mark_at = begin + every;      // (a symbol is at most 31 bits, `every` at least 32: a step passes one place at most)
-    bool met = false;
-    // (the whole warp goes round together: left to itself the loop lets lanes that have passed a place drift apart and
-    // runs them one after the other, seven times slower)
-    while (__any_sync(0xffffffffu, pos < pos_end)) {
-        if (pos < pos_end) {
-            const uint32_t win = long_window(base, pos);
-            const uint32_t e = S.entry(win, st);
-            if (e) S.next(e, win, st);
+    // (from place to place: the lanes of the warp meet there; a loop over the whole subsequence with the comparison inside
+    // let them drift apart and ran them one after the other, seven times slower)
+    uint32_t stop = begin;
+    bool met = pos >= pos_end;             // nothing to read
+    const bool idle = met;
+#pragma unroll 1
+    for (uint32_t i = 0; i < kMarks; ++i) {
+        stop += every;                     // (a symbol is at most 31 bits, `every` at least 32: a step passes one place at most)
+        const uint32_t bound = met ? 0u : min(stop, pos_end);
+        while (pos < bound) {
+            const uint32_t e = S.entry(pos, st);
+            if (e) S.advance(e, st);
             pos += e ? e & 31u : 1u;
-            if (pos >= mark_at) {                                          // (also behind the end: no place keeps an older reading's state)
-                const uint32_t key = (pos << 9) + st;                      // (equal keys are equal states: pos stays inside the subsequence)
-                met = lds32(marks) == key;                                 // met the reading before: it ends where that one did
-                sts32(marks, key);
-                marks += kPitch; mark_at += every;
-                if (met) pos = pos_end;
-            }
         }
+        __syncwarp();
+        if (!met && pos >= stop) {         // (also behind the end: no place keeps an older reading's state)
+            const uint32_t key = (pos << 9) + st;                          // (equal keys are equal states: pos stays inside the subsequence)
+            met = lds32(marks + i * kPitch) == key;                        // met the reading before: it ends where that one did
+            sts32(marks + i * kPitch, key);
+        }
+        if (__all_sync(0xffffffffu, met || pos >= pos_end)) break;
     }
-    if (!met) { pos_x = pos; st_x = st; }
+    if (!met || idle) { pos_x = pos; st_x = st; }
 }
 
 // Where the interval of a long scan lies, and this thread's subsequence.
@@ -181,9 +190,9 @@ struct LongSpan {
     uint32_t lead, endbit;         // its first bit and the one behind its last, counted from the first word
     uint32_t begin, end, every;
     bool ok;
-    // stage: shared memory for kStage words (the caller synchronises behind this)
-    template <uint32_t kThreads, uint32_t kStage>
-    __device__ __forceinline__ void init(const Params& P, const ScanDesc& sd, uint32_t tid, uint32_t* stage) {
+    // stage: shared memory for `room` words (the caller synchronises behind this)
+    template <uint32_t kThreads>
+    __device__ __forceinline__ void init(const Params& P, const ScanDesc& sd, uint32_t tid, uint32_t* stage, uint32_t room) {
         const uint32_t* segtab = P.seg_start + sd.seg_base;
         const uint32_t bstart = segtab[0], bend = segtab[1] - 2u;
         ok = !(bstart < sd.data_off || bend > sd.data_end || bend < bstart);   // (the same for every thread)
@@ -192,10 +201,10 @@ struct LongSpan {
         // whole words, at least eight of them: eight places at least 32 bits apart
         const uint32_t words = max(8u, ((endbit + 31u) / 32u + kThreads - 1u) / kThreads);
         const uint32_t len = 32u * words;
-        every = max(32u, len / kMarks);
+        every = len / kMarks;
         begin = min(max(tid * len, lead), endbit); end = min((tid + 1u) * len, endbit);
         const uint32_t need = endbit / 32u + 3u;               // (a symbol may begin in the last bit)
-        if (need <= kStage) {
+        if (need <= room) {
             for (uint32_t i = tid; i < need; i += kThreads) stage[i] = __ldg(origin + i);
             base = stage;
         }
@@ -224,7 +233,7 @@ __device__ __forceinline__ T cta_exclusive_sum(T v, T* s_tmp, int wid, int lane,
 
 // Search of the whole CTA: the true state at the start of every thread's subsequence, in pos and st.
 template <class Steps, int kWarps>
-__device__ __forceinline__ void search_all(const Steps& S, const LongSpan& L, uint32_t* s_marks, uint32_t* s_pos, uint32_t* s_state, uint32_t st0,
+__device__ __forceinline__ void search_all(const Steps& S, const LongSpan& L, uint32_t* s_marks, uint32_t* s_pos, uint32_t* s_state, uint32_t st0, uint32_t warm,
                                            uint32_t& pos, uint32_t& st) {
     constexpr uint32_t kThreads = 32 * kWarps;
     const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
@@ -232,13 +241,21 @@ __device__ __forceinline__ void search_all(const Steps& S, const LongSpan& L, ui
 #pragma unroll
     for (uint32_t i = 0; i < kMarks; ++i) s_marks[i * kThreads + tid] = 0xFFFFFFFFu;
     const uint32_t marks = (uint32_t)__cvta_generic_to_shared(s_marks + tid);
-    uint32_t pos_x = L.begin, st_x = st0;
-    pos = L.begin; st = st0;
+    // a first guess from `warm` bits in front of the subsequence: most readings have fallen in with the true one by then
+    pos = max(L.lead, L.begin - min(L.begin, warm)); st = st0;
+    while (__any_sync(full, pos < L.begin)) {
+        if (pos < L.begin) {
+            const uint32_t e = S.entry(pos, st);
+            if (e) S.advance(e, st);
+            pos += e ? e & 31u : 1u;
+        }
+    }
+    uint32_t pos_x = pos, st_x = st;
     bool again = true;
     for (uint32_t round = 0; round <= kThreads; ++round) {
         if (__any_sync(full, again)) {
             uint32_t x = pos_x, y = st_x;
-            search_span<Steps, 4 * kThreads>(S, L.base, L.begin, L.every, marks, pos, st, again ? L.end : 0u, x, y);
+            search_span<Steps, 4 * kThreads>(S, L.begin, L.every, marks, pos, st, again ? L.end : 0u, x, y);
             if (again) { pos_x = x; st_x = y; }
         }
         // the state the previous thread ended in (a warp's last lane's through shared memory)
@@ -269,12 +286,12 @@ __device__ __forceinline__ void load_tabs(uint32_t dst, const ScanTab* src, int 
 }
 
 __global__ void __launch_bounds__(32 * kLongWarps) first_pass_long_kernel(Params P, const uint32_t* __restrict__ list, uint32_t count) {
-    constexpr int kThreads = 32 * kLongWarps;
+    constexpr int kWarps = kLongWarps, kThreads = 32 * kWarps;
     __shared__ __align__(16) uint8_t s_tabs[2 * sizeof(ScanTab)];
     __shared__ uint32_t s_stage[kLongStage];
     __shared__ uint32_t s_marks[kMarks * kThreads];
-    __shared__ uint32_t s_pos[kLongWarps], s_state[kLongWarps], s_u[kLongWarps];
-    __shared__ int s_i[kLongWarps];
+    __shared__ uint32_t s_pos[kWarps], s_state[kWarps], s_u[kWarps];
+    __shared__ int s_i[kWarps];
     const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
     const uint32_t it = blockIdx.x;
     if (it >= count) return;                                   // whole CTA
@@ -289,9 +306,10 @@ __global__ void __launch_bounds__(32 * kLongWarps) first_pass_long_kernel(Params
     const uint32_t mcu_w = inter ? g.mx : g.ubw[c0];
     const uint32_t total = mcu_w * (inter ? g.my : g.ubh[c0]);  // MCUs of the scan (one interval)
     const uint32_t tabs = (uint32_t)__cvta_generic_to_shared(s_tabs);
-    load_tabs(tabs, P.tabs + ax.tab0 + (uint32_t)img * (uint32_t)ax.ntab, dc && sd.tab_off[1] ? 2 : 1, tid, kThreads);
+    const bool second = dc && sd.tab_off[1];
     LongSpan L;
-    L.init<kThreads, kLongStage>(P, sd, (uint32_t)tid, s_stage);
+    L.init<kThreads>(P, sd, (uint32_t)tid, s_stage, kLongStage);
+    load_tabs(tabs, P.tabs + ax.tab0 + (uint32_t)img * (uint32_t)ax.ntab, second ? 2 : 1, tid, kThreads);
     __syncthreads();
     if (!L.ok) {
         if (tid == 0) atomicMin(&P.status[img], kErrCorrupt);
@@ -302,24 +320,24 @@ __global__ void __launch_bounds__(32 * kLongWarps) first_pass_long_kernel(Params
     if (dc) {
         const uint32_t ny = (uint32_t)(P.hs * P.vs), bpm = inter ? ny + 2u : 1u, hs = (uint32_t)P.hs;
         DcSteps S;
-        S.tabs = tabs; S.bpm = bpm; S.tbits = 0;
+        S.base = L.base; S.tabs = tabs; S.bpm = bpm; S.tbits = 0;
         for (uint32_t j = 0; j < bpm; ++j) S.tbits |= ((sd.slots >> (2u * (inter && j >= ny ? j - ny + 1u : 0u))) & 1u) << j;
-        search_all<DcSteps, kLongWarps>(S, L, s_marks, s_pos, s_state, 0u, pos, st);
+        search_all<DcSteps, kWarps>(S, L, s_marks, s_pos, s_state, 0u, 512u, pos, st);
         int sum0 = 0, sum1 = 0, sum2 = 0;
         const uint32_t j1 = inter ? ny : 6u, j2 = inter ? ny + 1u : 6u;          // the chroma blocks' places
         for (uint32_t p = pos, j = st; p < L.end;) {
-            const uint32_t win = long_window(L.base, p), e = S.entry(win, j);
-            if (!e) { ++p; continue; }
-            const int d = magnitude(win, e & 31u, e >> 5);
+            const uint32_t e = S.entry(p, j);
+            const int d = magnitude(long_window(L.base, p), e & 31u, e >> 5);          // (no symbol: 0)
             sum0 += j < j1 ? d : 0; sum1 += j == j1 ? d : 0; sum2 += j == j2 ? d : 0;
-            nb += S.next(e, win, j);
-            p += e & 31u;
+            nb += e ? 1u : 0u;
+            if (e) S.advance(e, j);
+            p += e ? e & 31u : 1u;
         }
         int t;
-        uint32_t n = cta_exclusive_sum(nb, s_u, wid, lane, kLongWarps, all);
-        int pred0 = cta_exclusive_sum(sum0, s_i, wid, lane, kLongWarps, t);
-        int pred1 = cta_exclusive_sum(sum1, s_i, wid, lane, kLongWarps, t);
-        int pred2 = cta_exclusive_sum(sum2, s_i, wid, lane, kLongWarps, t);
+        uint32_t n = cta_exclusive_sum(nb, s_u, wid, lane, kWarps, all);
+        int pred0 = cta_exclusive_sum(sum0, s_i, wid, lane, kWarps, t);
+        int pred1 = cta_exclusive_sum(sum1, s_i, wid, lane, kWarps, t);
+        int pred2 = cta_exclusive_sum(sum2, s_i, wid, lane, kWarps, t);
         const uint32_t n1 = total * bpm;
         n = min(n, n1);
         // the place inside the MCU follows from the block number (equal to the handed-on state unless
@@ -332,7 +350,7 @@ __global__ void __launch_bounds__(32 * kLongWarps) first_pass_long_kernel(Params
         const uint32_t c_step = g.mx * g.my, step = inter ? hs : 1u;
         const uint32_t wrap = (inter ? (uint32_t)P.vs * g.bw[0] : g.bw[c0]) - step * mcu_w;
         for (uint32_t p = pos; p < L.end && n < n1; ++n) {
-            const uint32_t win = long_window(L.base, p), e = S.entry(win, j);
+            const uint32_t win = long_window(L.base, p), e = S.entry(p, j);
             if (!e) { bad = true; break; }
             const int d = magnitude(win, e & 31u, e >> 5);
             p += e & 31u;
@@ -354,15 +372,15 @@ __global__ void __launch_bounds__(32 * kLongWarps) first_pass_long_kernel(Params
         if (all < n1) bad = true;                              // the stream ends before the last block
     } else {
         AcSteps S;
-        S.tab = tabs; S.Ss = (uint32_t)sc.Ss; S.Se = (uint32_t)sc.Se;
-        search_all<AcSteps, kLongWarps>(S, L, s_marks, s_pos, s_state, S.Ss, pos, st);
+        S.base = L.base; S.tabs = tabs; S.Ss = (uint32_t)sc.Ss; S.Se = (uint32_t)sc.Se;
+        search_all<AcSteps, kWarps>(S, L, s_marks, s_pos, s_state, S.Ss, 0u, pos, st);
         for (uint32_t p = pos, k = st; p < L.end;) {
-            const uint32_t win = long_window(L.base, p), e = S.entry(win, k);
-            if (!e) { ++p; continue; }
-            nb += S.next(e, win, k);
-            p += e & 31u;
+            const uint32_t e = S.entry(p, k);
+            const uint32_t n = e & kEntEob ? eob_blocks(e, long_window(L.base, p)) : 1u;
+            if (e) nb += S.advance(e, k) ? n : 0u;
+            p += e ? e & 31u : 1u;
         }
-        uint32_t m = min(cta_exclusive_sum(nb, s_u, wid, lane, kLongWarps, all), total);
+        uint32_t m = min(cta_exclusive_sum(nb, s_u, wid, lane, kWarps, all), total);
         if (all < total) bad = true;                           // the stream ends before the last block
         // The blocks that BEGIN in this subsequence, the last one to its end; a block that began before it is passed over
         // (the thread before writes it).  So every block has one writer and its values one run in the value
@@ -379,7 +397,7 @@ __global__ void __launch_bounds__(32 * kLongWarps) first_pass_long_kernel(Params
         int16_t* vb = vp;
         uint32_t bcol = m % mcu_w, bi = (m / mcu_w) * bw + bcol;
         for (uint32_t p = pos; p < lim && m < total;) {
-            const uint32_t win = long_window(L.base, p), e = S.entry(win, k);
+            const uint32_t win = long_window(L.base, p), e = S.entry(p, k);
             const uint32_t skip = e & 31u, sz = (e >> 5) & 15u;
             p += skip;
             k += (e >> 9) & 15u;                               // position of the coefficient
@@ -445,7 +463,8 @@ __global__ void __launch_bounds__(32 * kSeqLongWarps) sequential_long_kernel(Par
     }
     load_tabs(S.tabs, P.tabs + ax.tab0 + 4u * (uint32_t)img, 4, tid, kThreads);
     LongSpan L;
-    L.init<kThreads, kSeqLongStage>(P, sd, (uint32_t)tid, s_stage);
+    L.init<kThreads>(P, sd, (uint32_t)tid, s_stage, kSeqLongStage);
+    S.base = L.base;
     __syncthreads();
     if (!L.ok) {
         if (tid == 0) atomicMin(&P.status[img], kErrCorrupt);
@@ -453,15 +472,14 @@ __global__ void __launch_bounds__(32 * kSeqLongWarps) sequential_long_kernel(Par
     }
     bool bad = false;
     uint32_t pos, st, all, nb = 0;
-    search_all<SeqSteps, kSeqLongWarps>(S, L, s_marks, s_pos, s_state, 0u, pos, st);
+    search_all<SeqSteps, kSeqLongWarps>(S, L, s_marks, s_pos, s_state, 0u, 0u, pos, st);
     int sum0 = 0, sum1 = 0, sum2 = 0;
     for (uint32_t p = pos, q = st; p < L.end;) {
-        const uint32_t win = long_window(L.base, p), e = S.entry(win, q), j = q >> 6;
-        if (!e) { ++p; continue; }
-        const int d = (q & 63u) == 0 ? magnitude(win, e & 31u, (e >> 5) & 15u) : 0;
+        const uint32_t e = S.entry(p, q), j = q >> 6;
+        const int d = (q & 63u) == 0 ? magnitude(long_window(L.base, p), e & 31u, (e >> 5) & 15u) : 0;      // (no symbol: 0)
         sum0 += j < ny ? d : 0; sum1 += j == ny ? d : 0; sum2 += j > ny ? d : 0;
-        nb += S.next(e, win, q);
-        p += e & 31u;
+        if (e) nb += S.advance(e, q) ? 1u : 0u;
+        p += e ? e & 31u : 1u;
     }
     int t;
     uint32_t n = cta_exclusive_sum(nb, s_u, wid, lane, kSeqLongWarps, all);
@@ -485,7 +503,7 @@ __global__ void __launch_bounds__(32 * kSeqLongWarps) sequential_long_kernel(Par
     int16_t* vp = vals + ((pos + 1u) >> 1);
     int16_t* vb = vp;
     for (uint32_t p = pos; p < lim && n < n1;) {
-        const uint32_t win = long_window(L.base, p), e = S.entry(win, (j << 6) + k);
+        const uint32_t win = long_window(L.base, p), e = S.entry(p, (j << 6) + k);
         const uint32_t skip = e & 31u, sz = (e >> 5) & 15u;
         const uint32_t blk = j < ny ? yb + (j >> (hs - 1u)) * g.bw[0] + (j & (hs - 1u)) : (ny + j - ny) * total + m;
         p += skip;
