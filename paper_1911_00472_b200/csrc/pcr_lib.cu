@@ -1177,6 +1177,14 @@ static void launch_pixels(const PixelPlan& pl, unsigned grid, cudaStream_t q, co
     ++g_launches;
 }
 
+template <typename OutT>
+static void launch_tensor(dim3 grid, cudaStream_t q, const Params& P, const TensorArgs& T, const uint8_t* rgb, uint32_t pos0) {
+    // pairs of columns where a pair never straddles rows and its store is aligned
+    const bool pairs = T.size % 2 == 0 && (reinterpret_cast<uintptr_t>(T.out) & (2 * sizeof(OutT) - 1)) == 0;
+    if (pairs) tensor_kernel<OutT, 2><<<grid, 128, 0, q>>>(P, T, rgb, pos0);
+    else tensor_kernel<OutT, 1><<<grid, 256, 0, q>>>(P, T, rgb, pos0);
+}
+
 // The expanded blocks of the whole record into the canonical planes.
 static void launch_planes(int samp, unsigned grid, const Params& Q, const CoefLists& cl) {
     if (samp == kSamp422) pixel_kernel<true, 1, false, 3, kSamp422><<<grid, unit_threads<kSamp422>()>>>(Q, cl, nullptr);
@@ -1444,9 +1452,9 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
             // the grid's second dimension (one image each) holds at most 65535 entries
             for (uint32_t p0 = i0; targs && p0 < i1; p0 += 65535u) {
                 const dim3 tg((unsigned)((targs->size + kTensorRows - 1) / kTensorRows), std::min(i1 - p0, 65535u));
-                if (targs->f32 == 2) tensor_kernel<__nv_bfloat16><<<tg, 256, 0, q>>>(P, *targs, static_cast<const uint8_t*>(out), p0);
-                else if (targs->f32) tensor_kernel<float><<<tg, 256, 0, q>>>(P, *targs, static_cast<const uint8_t*>(out), p0);
-                else tensor_kernel<__half><<<tg, 256, 0, q>>>(P, *targs, static_cast<const uint8_t*>(out), p0);
+                if (targs->f32 == 2) launch_tensor<__nv_bfloat16>(tg, q, P, *targs, static_cast<const uint8_t*>(out), p0);
+                else if (targs->f32) launch_tensor<float>(tg, q, P, *targs, static_cast<const uint8_t*>(out), p0);
+                else launch_tensor<__half>(tg, q, P, *targs, static_cast<const uint8_t*>(out), p0);
                 ++g_launches;
             }
         }

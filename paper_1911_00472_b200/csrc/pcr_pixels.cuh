@@ -677,6 +677,9 @@ struct TensorArgs {
 __device__ __forceinline__ void tensor_store(float* p, float v) { *p = v; }
 __device__ __forceinline__ void tensor_store(__half* p, float v) { *p = __float2half_rn(v); }
 __device__ __forceinline__ void tensor_store(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
+__device__ __forceinline__ void tensor_store2(float* p, float v, float w) { *reinterpret_cast<float2*>(p) = make_float2(v, w); }
+__device__ __forceinline__ void tensor_store2(__half* p, float v, float w) { *reinterpret_cast<__half2*>(p) = __floats2half2_rn(v, w); }
+__device__ __forceinline__ void tensor_store2(__nv_bfloat16* p, float v, float w) { *reinterpret_cast<__nv_bfloat162*>(p) = __floats2bfloat162_rn(v, w); }
 
 // Two horizontally adjacent RGB pixels (six bytes at any alignment) as floats, read as aligned
 // words: the word holding the first byte, the next one, and a third only when the six bytes reach
@@ -701,13 +704,14 @@ __device__ __forceinline__ void load_rgb_pair(const uint8_t* p, bool same, float
 #endif
 constexpr int kTensorRows = PCR_TENSOR_ROWS;      // output rows per CTA
 
-// One CTA per band of kTensorRows output rows of one image, one output column per thread (the
-// column's horizontal taps and weights are computed once for the band).  The taps are read from
-// global memory through the read-only path: neighbouring threads and rows hit the same cache
-// lines (staging the band's source rows in shared memory first was 40 % slower: it costs the
-// L1 capacity that these reads live on).
-template <typename OutT>
-__global__ void __launch_bounds__(256) tensor_kernel(Params P, TensorArgs T, const uint8_t* __restrict__ rgb, uint32_t pos0) {
+// One CTA per band of kTensorRows output rows of one image, kCols neighbouring output columns per thread (their
+// horizontal taps and weights are computed once for the band).  Two for even sizes: pairs of values are stored
+// together.  The taps are read from global memory through the read-only path: neighbouring threads and rows hit the same
+// cache lines (staging the band's source rows in shared memory first was 40 % slower: it costs the
+// L1 capacity that these reads live on).  A source row that the previous output row used, as the lower or the upper one, is
+// not interpolated again: a usual crop is about as large as the output, so one new source row per output row.
+template <typename OutT, int kCols>
+__global__ void __launch_bounds__(256 / kCols) tensor_kernel(Params P, TensorArgs T, const uint8_t* __restrict__ rgb, uint32_t pos0) {
     __shared__ int s_off0[kTensorRows], s_off1[kTensorRows];       // byte offsets of a row's upper / lower source row in the crop
     __shared__ float s_ay[kTensorRows];
     const uint32_t img = P.order[pos0 + blockIdx.y];
@@ -731,26 +735,52 @@ __global__ void __launch_bounds__(256) tensor_kernel(Params P, TensorArgs T, con
     const float k255 = 1.f / 255.f;
     const float m0 = T.mean[0], m1 = T.mean[1], m2 = T.mean[2], i0 = T.inv_std[0], i1 = T.inv_std[1], i2 = T.inv_std[2];
     OutT* const obase = static_cast<OutT*>(T.out) + (size_t)img * 3 * plane + (size_t)oy0 * S;
-    for (int ox = threadIdx.x; ox < S; ox += 256) {
-        const int u = r.flip ? S - 1 - ox : ox;
-        float fx = ((float)u + 0.5f) * sx - 0.5f;
-        fx = fminf(fmaxf(fx, 0.f), (float)(r.w - 1));
-        const int ix = (int)floorf(fx);
-        const float ax = fx - (float)ix, bx = 1.f - ax;
-        const uint8_t* p0 = crop0 + 3 * ix;
-        const bool same = ix + 1 > (int)r.w - 1;            // the right tap is clamped onto the left one
+    for (int ox = kCols * (int)threadIdx.x; ox < S; ox += 256) {
+        const uint8_t* p0[kCols];
+        float ax[kCols], bx[kCols];
+        bool same[kCols];
+#pragma unroll
+        for (int c = 0; c < kCols; ++c) {
+            const int u = r.flip ? S - 1 - (ox + c) : ox + c;
+            float fx = ((float)u + 0.5f) * sx - 0.5f;
+            fx = fminf(fmaxf(fx, 0.f), (float)(r.w - 1));
+            const int ix = (int)floorf(fx);
+            ax[c] = fx - (float)ix; bx[c] = 1.f - ax[c];
+            p0[c] = crop0 + 3 * ix;
+            same[c] = ix + 1 > (int)r.w - 1;                // the right tap is clamped onto the left one
+        }
+        float t[kCols][3], h[kCols][3];                     // the upper / lower source row at these columns
+        auto source_row = [&](int q, float (&v)[kCols][3]) {
+#pragma unroll
+            for (int c = 0; c < kCols; ++c) {
+                float r0, g0, b0, r1, g1, b1;
+                load_rgb_pair(p0[c] + q, same[c], r0, g0, b0, r1, g1, b1);
+                v[c][0] = bx[c] * r0 + ax[c] * r1; v[c][1] = bx[c] * g0 + ax[c] * g1; v[c][2] = bx[c] * b0 + ax[c] * b1;
+            }
+        };
+        auto copy_row = [&](float (&a)[kCols][3], const float (&b)[kCols][3]) {
+#pragma unroll
+            for (int c = 0; c < kCols; ++c) { a[c][0] = b[c][0]; a[c][1] = b[c][1]; a[c][2] = b[c][2]; }
+        };
+        int tq = -1, hq = -1;                               // their offsets
         OutT* o = obase + ox;
         for (int dy = 0; dy < nrows; ++dy, o += S) {
             const int q0 = s_off0[dy], q1 = s_off1[dy];
             const float ay = s_ay[dy], by = 1.f - ay;
-            float r00, g00, b00, r01, g01, b01, r10, g10, b10, r11, g11, b11;
-            load_rgb_pair(p0 + q0, same, r00, g00, b00, r01, g01, b01);
-            load_rgb_pair(p0 + q1, same, r10, g10, b10, r11, g11, b11);
-            const float tr = bx * r00 + ax * r01, tg = bx * g00 + ax * g01, tb = bx * b00 + ax * b01;
-            const float hr = bx * r10 + ax * r11, hg = bx * g10 + ax * g11, hb = bx * b10 + ax * b11;
-            tensor_store(o, ((by * tr + ay * hr) * k255 - m0) * i0);
-            tensor_store(o + plane, ((by * tg + ay * hg) * k255 - m1) * i1);
-            tensor_store(o + 2 * plane, ((by * tb + ay * hb) * k255 - m2) * i2);
+            if (q0 != tq) { if (q0 == hq) copy_row(t, h); else source_row(q0, t); tq = q0; }
+            if (q1 != hq) { if (q1 == tq) copy_row(h, t); else source_row(q1, h); hq = q1; }
+            float v[3][kCols];
+#pragma unroll
+            for (int c = 0; c < kCols; ++c) {
+                v[0][c] = ((by * t[c][0] + ay * h[c][0]) * k255 - m0) * i0;
+                v[1][c] = ((by * t[c][1] + ay * h[c][1]) * k255 - m1) * i1;
+                v[2][c] = ((by * t[c][2] + ay * h[c][2]) * k255 - m2) * i2;
+            }
+#pragma unroll
+            for (int e = 0; e < 3; ++e) {
+                if (kCols == 2) tensor_store2(o + e * plane, v[e][0], v[e][kCols - 1]);
+                else tensor_store(o + e * plane, v[e][0]);
+            }
         }
     }
 }
