@@ -681,22 +681,21 @@ __device__ __forceinline__ void tensor_store2(float* p, float v, float w) { *rei
 __device__ __forceinline__ void tensor_store2(__half* p, float v, float w) { *reinterpret_cast<__half2*>(p) = __floats2half2_rn(v, w); }
 __device__ __forceinline__ void tensor_store2(__nv_bfloat16* p, float v, float w) { *reinterpret_cast<__nv_bfloat162*>(p) = __floats2bfloat162_rn(v, w); }
 
-// Two horizontally adjacent RGB pixels (six bytes at any alignment) as floats, read as aligned
+// Two horizontally adjacent RGB pixels (six bytes from byte `off` on, at any alignment) as floats, read as aligned
 // words: the word holding the first byte, the next one, and a third only when the six bytes reach
-// into it.  `same`: the right neighbour is the pixel itself (clamped at the crop's edge).
-__device__ __forceinline__ void load_rgb_pair(const uint8_t* p, bool same, float& r0, float& g0, float& b0,
+// into it.
+__device__ __forceinline__ void load_rgb_pair(const uint32_t* base, uint32_t off, float& r0, float& g0, float& b0,
                                               float& r1, float& g1, float& b1) {
-    const uint32_t a = (uint32_t)(reinterpret_cast<uintptr_t>(p) & 3u);
-    const uint32_t* w = reinterpret_cast<const uint32_t*>(p - a);
+    const uint32_t* w = base + (off >> 2);
     const uint32_t w0 = __ldg(w), w1 = __ldg(w + 1);
-    const uint32_t w2 = (a == 3u && !same) ? __ldg(w + 2) : 0u;
-    const uint32_t lo = __funnelshift_r(w0, w1, 8 * a), hi = __funnelshift_r(w1, w2, 8 * a);   // bytes 0..3, 4..7
+    const uint32_t w2 = (off & 3u) == 3u ? __ldg(w + 2) : 0u;
+    const uint32_t lo = __funnelshift_r(w0, w1, 8 * off), hi = __funnelshift_r(w1, w2, 8 * off);   // bytes 0..3, 4..7 (shifts taken mod 32)
     r0 = __uint_as_float(__byte_perm(lo, 0x4B000000u, 0x7540)) - 8388608.f;      // byte into the mantissa of 2^23
     g0 = __uint_as_float(__byte_perm(lo, 0x4B000000u, 0x7541)) - 8388608.f;
     b0 = __uint_as_float(__byte_perm(lo, 0x4B000000u, 0x7542)) - 8388608.f;
-    r1 = same ? r0 : __uint_as_float(__byte_perm(lo, 0x4B000000u, 0x7543)) - 8388608.f;
-    g1 = same ? g0 : __uint_as_float(__byte_perm(hi, 0x4B000000u, 0x7540)) - 8388608.f;
-    b1 = same ? b0 : __uint_as_float(__byte_perm(hi, 0x4B000000u, 0x7541)) - 8388608.f;
+    r1 = __uint_as_float(__byte_perm(lo, 0x4B000000u, 0x7543)) - 8388608.f;
+    g1 = __uint_as_float(__byte_perm(hi, 0x4B000000u, 0x7540)) - 8388608.f;
+    b1 = __uint_as_float(__byte_perm(hi, 0x4B000000u, 0x7541)) - 8388608.f;
 }
 
 #ifndef PCR_TENSOR_ROWS
@@ -722,7 +721,8 @@ __global__ void __launch_bounds__(256 / kCols) tensor_kernel(Params P, TensorArg
     const CropRect r = T.crops[img];
     const float sx = (float)r.w / (float)S, sy = (float)r.h / (float)S;
     const uint32_t pitch = im.W * 3u;
-    const uint8_t* crop0 = rgb + im.out_off + (size_t)r.y0 * pitch + (size_t)r.x0 * 3;   // first byte of the crop
+    const uint32_t* const image = reinterpret_cast<const uint32_t*>(rgb + im.out_off);   // (images start at multiples of 128)
+    const uint32_t crop0 = r.y0 * pitch + r.x0 * 3u;          // first byte of the crop
     if ((int)threadIdx.x < nrows) {
         float fy = ((float)(oy0 + (int)threadIdx.x) + 0.5f) * sy - 0.5f;
         fy = fminf(fmaxf(fy, 0.f), (float)(r.h - 1));
@@ -732,13 +732,12 @@ __global__ void __launch_bounds__(256 / kCols) tensor_kernel(Params P, TensorArg
     }
     __syncthreads();
     const uint32_t plane = (uint32_t)S * (uint32_t)S;
-    const float k255 = 1.f / 255.f;
-    const float m0 = T.mean[0], m1 = T.mean[1], m2 = T.mean[2], i0 = T.inv_std[0], i1 = T.inv_std[1], i2 = T.inv_std[2];
+    const float w0 = T.inv_std[0] / 255.f, w1 = T.inv_std[1] / 255.f, w2 = T.inv_std[2] / 255.f;
+    const float z0 = -T.mean[0] * T.inv_std[0], z1 = -T.mean[1] * T.inv_std[1], z2 = -T.mean[2] * T.inv_std[2];
     OutT* const obase = static_cast<OutT*>(T.out) + (size_t)img * 3 * plane + (size_t)oy0 * S;
     for (int ox = kCols * (int)threadIdx.x; ox < S; ox += 256) {
-        const uint8_t* p0[kCols];
+        uint32_t p0[kCols];                                 // byte of the left tap in the crop's first row, from the image's first byte
         float ax[kCols], bx[kCols];
-        bool same[kCols];
 #pragma unroll
         for (int c = 0; c < kCols; ++c) {
             const int u = r.flip ? S - 1 - (ox + c) : ox + c;
@@ -746,15 +745,15 @@ __global__ void __launch_bounds__(256 / kCols) tensor_kernel(Params P, TensorArg
             fx = fminf(fmaxf(fx, 0.f), (float)(r.w - 1));
             const int ix = (int)floorf(fx);
             ax[c] = fx - (float)ix; bx[c] = 1.f - ax[c];
-            p0[c] = crop0 + 3 * ix;
-            same[c] = ix + 1 > (int)r.w - 1;                // the right tap is clamped onto the left one
+            // (at the crop's right edge the right tap has weight 0: whatever byte lies there does not count)
+            p0[c] = crop0 + 3u * (uint32_t)ix;
         }
         float t[kCols][3], h[kCols][3];                     // the upper / lower source row at these columns
         auto source_row = [&](int q, float (&v)[kCols][3]) {
 #pragma unroll
             for (int c = 0; c < kCols; ++c) {
                 float r0, g0, b0, r1, g1, b1;
-                load_rgb_pair(p0[c] + q, same[c], r0, g0, b0, r1, g1, b1);
+                load_rgb_pair(image, p0[c] + (uint32_t)q, r0, g0, b0, r1, g1, b1);
                 v[c][0] = bx[c] * r0 + ax[c] * r1; v[c][1] = bx[c] * g0 + ax[c] * g1; v[c][2] = bx[c] * b0 + ax[c] * b1;
             }
         };
@@ -772,9 +771,10 @@ __global__ void __launch_bounds__(256 / kCols) tensor_kernel(Params P, TensorArg
             float v[3][kCols];
 #pragma unroll
             for (int c = 0; c < kCols; ++c) {
-                v[0][c] = ((by * t[c][0] + ay * h[c][0]) * k255 - m0) * i0;
-                v[1][c] = ((by * t[c][1] + ay * h[c][1]) * k255 - m1) * i1;
-                v[2][c] = ((by * t[c][2] + ay * h[c][2]) * k255 - m2) * i2;
+                // (v / 255 - mean) / std as one multiplication and one addition
+                v[0][c] = (by * t[c][0] + ay * h[c][0]) * w0 + z0;
+                v[1][c] = (by * t[c][1] + ay * h[c][1]) * w1 + z1;
+                v[2][c] = (by * t[c][2] + ay * h[c][2]) * w2 + z2;
             }
 #pragma unroll
             for (int e = 0; e < 3; ++e) {
