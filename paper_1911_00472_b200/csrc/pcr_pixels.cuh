@@ -168,19 +168,22 @@ __device__ __forceinline__ bool expand_block(const Params& P, const CoefLists& c
     for (int i = 0; i < nfirst; ++i) {
         if (i) rec = __ldg(reinterpret_cast<const uint4*>(P.aux + cl.first[comp][i]) + at_rec);
         const int16_t* v = reinterpret_cast<const int16_t*>(((uint64_t)rec.w << 32) | rec.z);
-        uint64_t m = ((uint64_t)rec.y << 32) | (rec.x & ~0xFFu);
-        while (m) {                                // four at a time, so that their loads are in flight together
-            int pos[4], x[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                pos[e] = m ? __ffsll((long long)m) - 1 : -1;
-                m &= m - 1ull;                     // (0 stays 0)
-                if (pos[e] >= 0) x[e] = __ldg(v + e);
+        for (int half = 0; half < 2; ++half) {
+            uint32_t m = half ? rec.y : rec.x & ~0xFFu;
+            uint8_t* const lh = line + half * 8 * kPitch;
+            while (m) {                            // four at a time, so that their loads are in flight together
+                int pos[4], x[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    pos[e] = m ? __ffs((int)m) - 1 : -1;
+                    m &= m - 1u;                   // (0 stays 0)
+                    if (pos[e] >= 0) x[e] = __ldg(v++);
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (pos[e] >= 0) *reinterpret_cast<int16_t*>(lh + (pos[e] >> 2) * kPitch + 2 * (pos[e] & 3)) = (int16_t)x[e];
             }
-            v += 4;
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-                if (pos[e] >= 0) *at(pos[e]) = (int16_t)x[e];
         }
     }
     if (kRefine) {
