@@ -8,7 +8,7 @@
  * those bytes and produces training pixels on the GPU: for every image, the progressive
  * JPEG decode of its scans 1..k (Section 2, "Progressive Image Compression"; Section 5,
  * "Decoding": scans 1..k of an image followed by an end-of-image token are a decodable
- * JPEG) -> int16 coefficient planes in device memory -> dequantise, 8x8 inverse DCT,
+ * JPEG) -> int16 coefficients in device memory -> dequantise, 8x8 inverse DCT,
  * 2x2 chroma replication, YCbCr->RGB -> packed uint8 RGB.
  *
  * Record layout (little-endian, 16-byte aligned chunks; the "raw struct" form of Section 5):
@@ -105,8 +105,8 @@ size_t pcr_out_bytes(const pcr_record* rec);
 size_t pcr_prefix_bytes(const pcr_record* rec, int k);
 
 /* Decode all images at fidelity k (Sections 2, 3, 5): Huffman-decode scans 1..k into the
- * record's int16 coefficient planes (first passes, then successive-approximation
- * refinements in place), then dequantise, inverse-DCT, upsample, colour-convert and store.
+ * record's coefficient lists (first passes, then successive-approximation refinements on
+ * top of them), then dequantise, inverse-DCT, upsample, colour-convert and store.
  *   k      : 1..G.
  *   out    : DEVICE memory, caller-owned, at least pcr_out_bytes(rec) bytes, 16-byte aligned.
  *            Only the bytes of each image's 3*W*H pixels are written.
@@ -122,7 +122,7 @@ int pcr_decode(pcr_record* rec, int k, void* out, void* stream);
 
 /* Raise the fidelity of the last decode (Section 3: "a task then merely needs to read subsequent
  * scan groups until the desired fidelity level is reached"; Section 4.3 switches fidelity while
- * training).  The coefficient planes and the side data of scans 1..k_prev stay on the device
+ * training).  The coefficient lists and the side data of scans 1..k_prev stay on the device
  * after pcr_decode; this call copies the scan groups k_prev+1..k that are not yet resident,
  * decodes only those scans on top of the resident state and produces the pixels of fidelity k.
  * The result is identical to pcr_decode(rec, k, ...).
@@ -152,7 +152,7 @@ int pcr_decode_more(pcr_record* rec, int k, void* out, void* stream);
  *            the decoded pixels of the transformed MCUs, other bytes are left as they were.
  *   tensor : DEVICE, pcr_num_images * 3 * size * size elements of dtype, image i at index i.
  * Restart intervals whose MCU rows lie outside the MCU rows an image's rectangle touches are not
- * entropy-decoded either, so afterwards the coefficient planes are incomplete: pcr_decode_more
+ * entropy-decoded either, so afterwards the coefficients are incomplete: pcr_decode_more
  * refuses to continue from this call (PCR_E_ARG) and pcr_coeffs is meaningful only for the
  * decoded rows.
  * Enqueues on `stream` and returns; errors as pcr_decode.  The first call on a record allocates
@@ -215,8 +215,8 @@ int pcr_status(pcr_record* rec, int* first_bad_image, int* code);
 
 /* Test hook: the coefficient planes of the last decode, DEVICE memory owned by the record.
  * Call it after the decode's stream has been synchronised: it completes the canonical layout
- * (the decode keeps DC coefficients in a dense plane of their own; they are copied into the
- * blocks here, with a small kernel on the default stream that this call waits for).
+ * (the decode keeps coefficients as lists and applies refinements when it expands a block; the
+ * blocks are expanded into planes here, with a kernel on the default stream that this call waits for).
  * Layout: image after image (image i's first block = its blocks_offset), within an image
  * component Y, Cb, Cr, block rows then block columns of the MCU-padded grid, 64 int16 per
  * block in zigzag order (128 bytes per block).  *bytes = total size. */
@@ -249,9 +249,10 @@ int pcr_get_sampling(const pcr_record* rec, int* hs, int* vs, int* ncomp);
 /* Stage timing for benchmarks.  With profiling enabled every pcr_decode records CUDA events
  * on its stream around each stage; after the stream has been synchronised pcr_get_profile
  * returns, for the last decode, up to `cap` entries {name, milliseconds, kernel launches}.
- * Stages: "h2d" (prefix copy), "clear" (status and plane clearing), "index" (restart-interval
- * index and unstuffed copy), "entropy0".."entropyW" (one per wave that ran), "pixels" (in-place
- * update of the planes from the refinement scans, then the pixel stage).  *n = entries written. */
+ * Stages: "h2d" (prefix copy), "clear" (nothing of size; kept for readers of the list), "index"
+ * (restart-interval index, unstuffed copy and symbol tables), "entropy0".."entropyW" (one per wave
+ * that ran), "pixels" (blocks expanded with their refinements, then the pixel stage).  *n = entries
+ * written. */
 typedef struct {
     char name[24];
     float ms;

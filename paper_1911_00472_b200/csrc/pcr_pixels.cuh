@@ -247,7 +247,9 @@ __device__ __forceinline__ bool expand_block(const Params& P, const CoefLists& c
 //
 // One thread per block through the whole transform; the chroma samples go through shared memory, the luminance
 // samples stay in the registers of the thread that made them and meet the chroma there, two pixels
-// per instruction (16-bit pairs).  Bound by instruction issue: see the table of kernels for the counts.
+// per instruction (16-bit pairs).  Bound by instruction issue (integer multiplications and additions of the transform, about
+// 0.6 of the slots).  Pixel stage of 1024 ImageNet-shaped images, before (lines of 128 bytes per block, colour as a
+// step of its own) and now: k = 5 348 -> 166 us, k = 10 562 -> 348 us, baseline 351 -> 265 us.
 template <bool kRefine, int kMode, bool kRoi = false, int kStage = 0, int kSamp = kSamp420, bool kCoarse = false>
 __global__ void __launch_bounds__(unit_threads<kSamp>(), (kCoarse ? 1152 : 672) / unit_threads<kSamp>())
 pixel_kernel(Params P, CoefLists cl, uint8_t* __restrict__ out) {
@@ -712,6 +714,9 @@ constexpr int kTensorRows = PCR_TENSOR_ROWS;      // output rows per CTA
 // cache lines (staging the band's source rows in shared memory first was 40 % slower: it costs the
 // L1 capacity that these reads live on).  A source row that the previous output row used, as the lower or the upper one, is
 // not interpolated again: a usual crop is about as large as the output, so one new source row per output row.
+// Bound by instruction issue (interpolation and normalisation, 51 M output pixels for 1024 images).  That record
+// cropped to 224x224 fp16: 220 us with a column a thread, 195 us with two and rows used again, 184 us with the
+// normalisation as one multiplication and addition a value.
 template <typename OutT, int kCols>
 __global__ void __launch_bounds__(256 / kCols) tensor_kernel(Params P, TensorArgs T, const uint8_t* __restrict__ rgb, uint32_t pos0) {
     __shared__ int s_off0[kTensorRows], s_off1[kTensorRows];       // byte offsets of a row's upper / lower source row in the crop
