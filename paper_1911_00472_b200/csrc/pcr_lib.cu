@@ -1358,10 +1358,21 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
             runs.n = 0;
             uint32_t count = 0;
             bool refine = false;                           // waves without AC refinements need no mask queues
-            auto launch_items = [&]() {
+            int dc_n = 0;                                  // the wave's DC refinements, at most one per component
+            for (int s : waves[w])
+                if (s >= k0 && s < k && rec->script[s].Ss == 0 && rec->script[s].Ah != 0 && dc_n < 3) runs.dc_s[dc_n++] = s;
+            bool dc_done = dc_n == 0;
+            auto launch_items = [&](bool last) {
                 if (!count) return;
-                const unsigned nb = (count + kEntropyWarps - 1) / kEntropyWarps;
+                unsigned nb = (count + kEntropyWarps - 1) / kEntropyWarps;
                 const uint32_t smem = kEntropyWarps * (refine ? warp_bytes<true>() : warp_bytes<false>());
+                runs.item_blocks = nb;
+                if (last && refine && !dc_done) {          // (waves without AC refinements are compiled without this)
+                    runs.dc_pos0 = i0; runs.dc_images = i1 - i0;
+                    runs.dc_chunks = (rec->dc_refine_chunks + 1) / 2;      // about five MCUs a thread
+                    nb += dc_n * runs.dc_images * runs.dc_chunks;
+                    dc_done = true;
+                }
                 if (roi && refine) entropy_kernel<true, true><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
                 else if (roi) entropy_kernel<true, false><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
                 else if (refine) entropy_kernel<false, true><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
@@ -1386,7 +1397,7 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
             }
             for (int s : waves[w]) {
                 if (s < k0 || s >= k || in_pair[s]) continue;
-                if (runs.n == kMaxRuns && !sequential) launch_items();
+                if (runs.n == kMaxRuns && !sequential) launch_items(false);
                 add_run(rec->item_begin[(size_t)g * G + s], rec->item_count[(size_t)g * G + s]);
             }
             const uint32_t begin = runs.n ? runs.first[0] : 0u;
@@ -1404,7 +1415,7 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
                 }
                 return true;
             }
-            launch_items();
+            launch_items(true);
             // scans that are one long restart interval: the first passes of the wave (a contiguous run
             // of the list) ...
             {
@@ -1422,11 +1433,9 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
                 }
             }
             // ... (their AC refinements follow in one launch for the whole record, once every slice
-            // has finished its waves) and the DC refinement scans of every record
-            for (int s : waves[w]) {
-                if (s >= k) break;
-                const ScanScript& sc = rec->script[s];
-                if (s < k0 || sc.Ss != 0 || sc.Ah == 0) continue;
+            // has finished its waves) and the DC refinement scans that the interval kernel did not take
+            for (int j = 0; j < dc_n && !dc_done; ++j) {
+                const int s = runs.dc_s[j];
                 for (uint32_t p0 = i0; p0 < i1; p0 += 65535u) {
                     dc_refine_kernel<<<dim3(rec->dc_refine_chunks, std::min(i1 - p0, 65535u)), 256, 0, q>>>(P, s, p0);
                     ++g_launches;

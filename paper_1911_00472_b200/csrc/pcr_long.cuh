@@ -4,7 +4,7 @@
 // A Huffman stream is a serial chain, so a whole scan on one lane takes tens of thousands of
 // dependent steps.  These kernels shorten or remove that chain:
 //
-//  * dc_refine_kernel: a DC refinement scan carries exactly one raw bit per block, so after
+//  * dc_refine_image / dc_refine_kernel: a DC refinement scan carries exactly one raw bit per block, so after
 //    unstuffing bit j of a restart interval is block j of the interval in scan order: one thread
 //    per MCU, no chain at all.  Used for every record.
 //  * first_pass_long_kernel: DC and AC first passes.  One small CTA per (scan, image); the segment is
@@ -36,50 +36,10 @@
 namespace pcr {
 
 // ---------------------------------------------------------------------------------------
-// DC refinement: thread per MCU of the scan.  grid = (chunks of MCUs, images of the run).
+// DC refinement where no launch of interval warps can carry it (see entropy_kernel).  grid = (chunks of MCUs, images of the run).
 // ---------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) dc_refine_kernel(Params P, int s, uint32_t pos0) {
-    const int img = (int)P.order[pos0 + blockIdx.y];
-    const ScanDesc sd = P.scans[(size_t)s * P.N + img];
-    const ScanScript sc = P.script[s];
-    const ImgDesc im = P.imgs[img];
-    const Geometry g = make_geometry(im, P);
-    const bool inter = sc.ncomp > 1;
-    const int c0 = sc.comp[0];
-    const uint32_t mcu_w = inter ? g.mx : g.ubw[c0];
-    const uint32_t mcu_h = inter ? g.my : g.ubh[c0];
-    const uint32_t total = mcu_w * mcu_h;
-    const uint32_t bpm = inter ? (uint32_t)(P.hs * P.vs + 2) : 1u;   // blocks (= bits) per MCU
-    const uint32_t* segtab = P.seg_start + sd.seg_base;
-    const uint32_t* words = reinterpret_cast<const uint32_t*>(P.ubuf);
-    const int p1 = 1 << sc.Al;
-    bool bad = false;
-    for (uint32_t m = blockIdx.x * 256u + threadIdx.x; m < total; m += gridDim.x * 256u) {
-        const uint32_t seg = sd.ri ? m / sd.ri : 0u;
-        if (seg >= sd.nseg) { bad = true; continue; }
-        const uint32_t m0 = seg * sd.ri;                       // 0 without restart markers
-        const uint32_t bstart = segtab[seg], bend = segtab[seg + 1] - 2u;
-        if (bstart < sd.data_off || bend > sd.data_end || bend < bstart) { bad = true; continue; }   // a missing marker left a hole
-        const uint32_t bit = bpm * (m - m0);
-        if (bit + bpm > 8u * (bend - bstart)) { bad = true; continue; }                             // the interval is too short
-        const uint32_t p = 8u * (bstart & 3u) + bit;           // from the first bit of word bstart >> 2
-        const uint32_t wi = (bstart >> 2) + (p >> 5);
-        const uint32_t w0 = __ldg(words + wi), w1 = __ldg(words + wi + 1);   // the copy has spare bytes behind its end
-        const uint32_t v = __funnelshift_l(w1, w0, p & 31u) >> (32u - bpm);  // the MCU's bits, first block in the top bit
-        const uint32_t mrow = m / mcu_w, mcol = m - mrow * mcu_w;
-#pragma unroll
-        for (uint32_t j = 0; j < 6; ++j) {
-            if (j >= bpm) break;
-            if (!((v >> (bpm - 1u - j)) & 1u)) continue;
-            uint64_t blk;
-            int comp;
-            if (!inter) blk = g.coff[c0] + (uint64_t)mrow * g.bw[c0] + mcol;
-            else blk = mcu_block(g, P, mrow, mcol, (int)j, &comp);
-            int16_t* dcv = P.dc + blk;                        // (no other scan of the wave writes it)
-            *dcv = (int16_t)(*dcv | p1);
-        }
-    }
-    if (bad) atomicMin(&P.status[img], kErrCorrupt);
+    dc_refine_image(P, s, (int)P.order[pos0 + blockIdx.y], blockIdx.x * 256u + threadIdx.x, gridDim.x * 256u);
 }
 
 // ---------------------------------------------------------------------------------------

@@ -92,6 +92,10 @@ constexpr int kMaxRuns = 24;
 struct ItemRuns {
     int32_t n;
     uint32_t first[kMaxRuns], end[kMaxRuns];   // first item of the run; items in this run and those before it
+    // DC refinement scans in blocks behind those of the items: of the images order[dc_pos0 ..], dc_chunks blocks an image
+    uint32_t item_blocks;
+    int32_t dc_s[3];
+    uint32_t dc_pos0, dc_images, dc_chunks;
 };
 
 // Crop rectangle of one image (pixels) and whether its columns are mirrored; the pixel kernel

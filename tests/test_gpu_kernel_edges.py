@@ -62,6 +62,23 @@ def test_fidelity_lowered_on_one_handle(restart_rows):
     _compare(rec, range(len(script), 0, -1))
 
 
+@pytest.mark.parametrize("largest", [(192, 128), (400, 390)])
+@pytest.mark.parametrize("single", [True, False])
+def test_dc_refinement_beside_ac_refinement(largest, single):
+    """DC refinements in the blocks behind a wave's restart intervals: images of 1, 95, 96, 97 and 625 MCUs (a block takes 96
+    at a time, one or two blocks an image), one interleaved scan or one for each component, and the last one alone in its
+    wave."""
+    dc = [((c,), 0, 0, 2, 1) for c in range(3)] if single else [((0, 1, 2), 0, 0, 2, 1)]
+    script = [((0, 1, 2), 0, 0, 0, 2), ((0,), 1, 63, 0, 1), ((1,), 1, 63, 0, 0), ((2,), 1, 63, 0, 0)] + dc + [
+        ((0,), 1, 63, 1, 0), ((0, 1, 2), 0, 0, 1, 0)]
+    rng = np.random.default_rng(5)
+    dims = [largest, (16, 16), (19 * 16, 75), (97 * 16, 9)]
+    coeffs = [_field(rng, pcr_synth.num_blocks(w, h), 0.1, 9) for w, h in dims]
+    with pcr_synth.scan_script(script):
+        rec = pcr_synth.record_from_coeffs(dims, coeffs)
+    _compare(rec, range(len(script) - len(dc) - 1, len(script) + 1))
+
+
 @pytest.mark.parametrize("outside", [None, (4, 0), (0, 4), (7, 7)])
 @pytest.mark.parametrize("samp", [(2, 2, 3), (1, 1, 3), (1, 1, 1)])
 def test_corner_transform(outside, samp):
