@@ -134,7 +134,10 @@ __device__ __forceinline__ void search_span(const Steps& S, uint32_t begin, uint
             pos += e ? e & 31u : 1u;
         }
         __syncwarp();
-        if (!met && pos >= stop) {         // (also behind the end: no place keeps an older reading's state)
+        // (Only places inside the subsequence: every reading passes those or meets an earlier one in front of them, so the keys
+        // they hold are the latest reading's throughout, and so is the end state.  A place behind the end of a truncated
+        // subsequence is passed by some readings only and would keep an older one's key.)
+        if (!met && pos >= stop && stop <= pos_end) {
             const uint32_t key = (pos << 9) + st;                          // (equal keys are equal states: pos stays inside the subsequence)
             met = lds32(marks + i * kPitch) == key;                        // met the reading before: it ends where that one did
             sts32(marks + i * kPitch, key);
