@@ -26,7 +26,8 @@
  * MCU in each direction and one block per chroma component (4:2:0, 4:2:2, 4:4:0, 4:4:4: the paper's
  * per-scan example for HAM10000 is a 4:4:4 file), or one component (greyscale: every output pixel
  * is (Y, Y, Y)); one sampling per record; progressive
- * (SOF2) with any scan script that is the same for all images of a record, or baseline
+ * (SOF2) with any scan script that is the same for all images of a record (an AC coefficient is
+ * sent by one first pass, before its refinements, as T.81 has it), or baseline
  * sequential (SOF0, one interleaved scan = one scan group: the conventional JPEG that the paper's
  * Table 2 compares against); any restart interval.
  *

@@ -678,6 +678,17 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     int n_refine[3] = {0, 0, 0};
     for (uint32_t s = 0; s < G; ++s)
         if (r->script[s].Ss > 0 && r->script[s].Ah > 0 && ++n_refine[r->script[s].comp[0]] > 4) return PCR_E_FORMAT;
+    // An AC position is sent by one first pass, before any refinement of it (T.81 B.2.3: only the first scan of a band has
+    // Ah = 0).  The lists rely on it: at most kMaxFirst first passes of a component reach beyond position 7, first
+    // passes are expanded before refinements, and no two scans write the same values.
+    uint64_t sent[3] = {0, 0, 0};
+    for (const ScanScript& sc : r->script) {
+        const uint64_t band = (sc.Se == 63 ? ~0ull : (1ull << (sc.Se + 1)) - 1ull) & ~((1ull << std::max(1, sc.Ss)) - 1ull);
+        for (int i = 0; i < sc.ncomp; ++i) {
+            if (sc.Ah == 0 && (sent[sc.comp[i]] & band)) return PCR_E_FORMAT;
+            sent[sc.comp[i]] |= band;
+        }
+    }
     uint64_t n_tabs = 0;
     for (uint32_t s = 0; s < G; ++s) {
         const ScanScript& sc = r->script[s];

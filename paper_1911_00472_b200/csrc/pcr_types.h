@@ -34,7 +34,8 @@ struct ScanAux {
 };
 
 // Where the coefficients of the decoded scans lie, per component (built per call for the chosen k).
-constexpr int kMaxFirst = 56;      // first passes of a component that reach beyond position 7: at most one per position
+constexpr int kMaxFirst = 56;      // first passes of a component that reach beyond position 7: at most one for each of 8..63
+                                   // (pcr_open refuses a position that is sent twice)
 struct CoefLists {
     uint4 head_mask[3];            // positions 1..7 that a decoded scan covers, as 16-bit lanes of the head plane's entries
     uint32_t dc_mask[3];           // bits of the DC coefficient that a decoded scan covers (a refinement of an earlier

@@ -183,3 +183,29 @@ def oracle_record_pixels(pool, workers, rec_bytes, tmpdir, offsets, out_bytes, k
     shards = [(rec_path, out_path, out_bytes, offsets, k, lo, min(lo + per, n)) for lo in range(0, n, per)]
     assert sum(pool.map(oracle_rgb_shard, shards)) == n
     return np.array(np.memmap(out_path, dtype=np.uint8, mode="r", shape=(out_bytes,)))
+
+
+def record_from_groups(groups) -> np.ndarray:
+    """A record whose scan groups are taken from other records of the same images: groups = [(record bytes, group index)].
+    Written from the record layout alone (header, metadata, index, chunks at multiples of 16 bytes)."""
+    first = groups[0][0]
+    N = struct.unpack_from("<I", first, 8)[0]
+    G = len(groups)
+    meta_off = struct.unpack_from("<Q", first, 24)[0]
+    index_off = 64 + 16 * N
+    pos = (index_off + 8 * (G + 1) + 16 * G * N + 15) // 16 * 16
+    ends, index, parts = [pos], [], []
+    for rec, g in groups:
+        src_G = struct.unpack_from("<I", rec, 12)[0]
+        at = struct.unpack_from("<Q", rec, 32)[0] + 8 * (src_G + 1) + 16 * g * N
+        for i in range(N):
+            off, length, _ = struct.unpack_from("<QII", rec, at + 16 * i)
+            index.append(struct.pack("<QII", pos, length, 0))
+            parts.append(bytes(rec[off:off + length]) + b"\0" * (-length % 16))
+            pos += len(parts[-1])
+        ends.append(pos)
+    head = bytearray(bytes(first[:64]))
+    struct.pack_into("<II", head, 8, N, G)
+    struct.pack_into("<QQQQ", head, 24, 64, index_off, ends[0], pos)
+    body = bytes(head) + bytes(first[meta_off:meta_off + 16 * N]) + struct.pack(f"<{G + 1}Q", *ends) + b"".join(index)
+    return np.frombuffer(body + b"\0" * (ends[0] - len(body)) + b"".join(parts), dtype=np.uint8).copy()

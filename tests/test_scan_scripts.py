@@ -8,7 +8,7 @@ import pytest
 import pcr_synth
 from oracle import pcr_oracle as O
 
-from helpers import mask_truth, mask_truth_script
+from helpers import mask_truth, mask_truth_script, record_from_groups
 
 SCRIPTS = {"spectral4": pcr_synth.SCRIPT_SPECTRAL_4, "mixed6": pcr_synth.SCRIPT_MIXED_6, "deep14": pcr_synth.SCRIPT_DEEP_14}
 TEN = [((0, 1, 2), 0, 0, 0, 1), ((0,), 1, 5, 0, 2), ((2,), 1, 63, 0, 1), ((1,), 1, 63, 0, 1), ((0,), 6, 63, 0, 2),
@@ -83,6 +83,85 @@ def test_gpu_other_scripts_every_k(name, restart_rows):
         torch.cuda.synchronize()
         for i in range(rec.n_images):
             assert torch.equal(dec.image(out, i), dec.image(full, i)), (name, i)
+    finally:
+        dec.close()
+
+
+# ---- what a script may and may not hold
+def _position_by_position():
+    """A record of 64 scan groups: DC, then every zigzag position of the luminance by itself."""
+    parts = []
+    for lo in range(1, 64, 15):
+        with pcr_synth.scan_script([((0, 1, 2), 0, 0, 0, 0)] + [((0,), p, p, 0, 0) for p in range(lo, min(lo + 15, 64))]):
+            parts.append(pcr_synth.make_record(0, n_images=4))
+    groups = [(parts[0].bytes, 0)]
+    for part in parts:
+        groups += [(part.bytes, g) for g in range(1, O.record_info(part.bytes)[1])]
+    return record_from_groups(groups)
+
+
+def _open(raw):
+    """pcr_open's status: without a device a valid record ends at the first allocation on it."""
+    import ctypes as C
+    from paper_1911_00472_b200 import binding, build
+    build.build()
+    h = C.c_void_p()
+    rc = binding.lib().pcr_open(raw.ctypes.data, raw.size, C.byref(h))
+    if h.value:
+        binding.lib().pcr_close(h)
+    return rc
+
+
+Y = (0,)
+DC = ((0, 1, 2), 0, 0, 0, 1)
+REPEATED = {"the band again": [DC, (Y, 1, 63, 0, 0), (Y, 1, 63, 0, 0)],
+            "one position again": [DC, (Y, 1, 9, 0, 0), (Y, 9, 63, 0, 0)],
+            "below position 8": [DC, (Y, 1, 5, 0, 1), (Y, 2, 2, 0, 0)],
+            "after its refinement": [DC, (Y, 1, 63, 0, 1), (Y, 1, 63, 1, 0), (Y, 1, 63, 0, 0)],
+            "first pass behind a refinement that covers it": [DC, (Y, 1, 5, 0, 1), (Y, 1, 63, 1, 0), (Y, 6, 63, 0, 0)]}
+ALLOWED = {"disjoint bands": [DC, (Y, 1, 9, 0, 0), (Y, 10, 63, 0, 0)],
+           "the same band of other components": [DC, (Y, 1, 63, 0, 0), ((1,), 1, 63, 0, 0), ((2,), 1, 63, 0, 0)],
+           "refinement over two bands": [DC, (Y, 1, 5, 0, 1), (Y, 6, 63, 0, 1), (Y, 1, 63, 1, 0)],
+           "DC sent twice": [DC, DC, (Y, 1, 63, 0, 0)]}
+
+
+@pytest.mark.parametrize("name", sorted(REPEATED) + sorted(ALLOWED))
+def test_an_ac_position_is_sent_once(name):
+    with pcr_synth.scan_script((REPEATED | ALLOWED)[name]):
+        rec = pcr_synth.make_record(0, n_images=2)
+    assert (_open(rec.bytes) == -2) == (name in REPEATED)
+
+
+def test_many_first_passes_of_a_component_are_refused():
+    """63 scans of positions 1..63 of the luminance: more than the table of coefficient lists has entries."""
+    with pcr_synth.scan_script([DC, (Y, 1, 63, 0, 0)]):
+        raw = pcr_synth.make_record(0, n_images=2).bytes
+    assert _open(raw) != -2
+    assert _open(record_from_groups([(raw, 0)] + [(raw, 1)] * 63)) == -2
+    with pcr_synth.scan_script(pcr_synth.SCRIPT_BASELINE):
+        raw = pcr_synth.make_record(0, n_images=2).bytes
+    assert _open(raw) != -2 and _open(record_from_groups([(raw, 0)])) != -2
+    assert _open(_position_by_position()) != -2
+
+
+@pytest.mark.gpu
+def test_gpu_64_scan_groups():
+    """As many coefficient lists as a component can have (one for each of the positions 8..63)."""
+    import torch
+    from paper_1911_00472_b200 import Decoder
+    raw = _position_by_position()
+    dec = Decoder(raw)
+    try:
+        assert dec.n_groups == 64
+        for k in (8, 9, 64, 40):
+            out = dec.decode(k)
+            torch.cuda.synchronize()
+            assert dec.status() == (-1, 0), k
+            coef = dec.coeffs().cpu().numpy()
+            want = [O.decode_image(raw, i, k) for i in range(dec.n_images)]
+            assert np.array_equal(coef, np.concatenate([c for c, _ in want])), k
+            for i, (_, rgb) in enumerate(want):
+                assert np.array_equal(dec.image(out, i).cpu().numpy(), rgb), (k, i)
     finally:
         dec.close()
 
