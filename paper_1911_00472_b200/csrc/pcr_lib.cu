@@ -17,6 +17,7 @@
 #include <memory>
 #include <mutex>
 #include <new>
+#include <system_error>
 #include <thread>
 #include <utility>
 #include <vector>
@@ -637,7 +638,10 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
         };
         if (const int rc = parse_image(0)) return rc;
         std::vector<std::thread> pool;
-        for (unsigned t = 1; t < nthreads; ++t) pool.emplace_back(work, t);
+        pool.reserve(nthreads);
+        try {
+            for (unsigned t = 1; t < nthreads; ++t) pool.emplace_back(work, t);
+        } catch (const std::system_error&) {}            // (no more threads to be had: those there are and this one do it)
         work(0);
         for (auto& th : pool) th.join();
         for (int rc : rcs) if (rc != PCR_OK) return rc;

@@ -54,6 +54,33 @@ def test_argument_errors_need_no_device(lib):
     assert lib.pcr_strerror(-3) == b"corrupt entropy-coded data"
 
 
+def test_open_without_threads_to_be_had(tmp_path, lib):
+    """pcr_open walks the images on a few threads; where none can be started it does the work itself, and nothing is thrown
+    through the C ABI.  (A preloaded pthread_create that always fails; no device, so a valid record ends with PCR_E_CUDA.)"""
+    import subprocess
+    import sys
+    import pcr_synth
+    rec = pcr_synth.make_record(0, n_images=200)
+    rec.bytes.tofile(tmp_path / "record")
+    damaged = rec.bytes.copy()
+    damaged[int.from_bytes(damaged[40:48].tobytes(), "little") + 4] ^= 0xFF       # the first image's first marker segment
+    damaged.tofile(tmp_path / "damaged")
+    (tmp_path / "shim.c").write_text("#include <errno.h>\nint pthread_create(void* a, const void* b, void* (*f)(void*), void* p) "
+                                     "{ (void)a; (void)b; (void)f; (void)p; return EAGAIN; }\n")
+    shim = tmp_path / "shim.so"
+    subprocess.check_call(["gcc", "-shared", "-fPIC", "-o", str(shim), str(tmp_path / "shim.c")])
+    code = ("import ctypes, sys\n"
+            "lib = ctypes.CDLL(sys.argv[1])\n"
+            "lib.pcr_open.argtypes = [ctypes.c_char_p, ctypes.c_size_t, ctypes.POINTER(ctypes.c_void_p)]\n"
+            "for name in sys.argv[2:]:\n"
+            "    raw, h = open(name, 'rb').read(), ctypes.c_void_p()\n"
+            "    print(lib.pcr_open(raw, len(raw), ctypes.byref(h)))\n")
+    env = dict(os.environ, LD_PRELOAD=str(shim), CUDA_VISIBLE_DEVICES="")
+    res = subprocess.run([sys.executable, "-c", code, lib._name, str(tmp_path / "record"), str(tmp_path / "damaged")], env=env,
+                         capture_output=True, text=True, timeout=120)
+    assert res.returncode == 0 and res.stdout.split() == ["-5", "-2"], res
+
+
 def test_product_path_does_not_touch_the_oracle():
     """Neither the package nor the generator imports or mentions the oracle."""
     for folder in ("paper_1911_00472_b200", "pcr_synth"):
