@@ -72,7 +72,12 @@ typedef struct {
 /* Section 3 (metadata + scan groups) and Section 5 "Decoding" (locate the offsets).
  * Parses and validates the header, the group table, every chunk's position and every
  * image's JPEG frame, table and scan headers; allocates the per-record device state
- * (record bytes, coefficient planes, tables) on the current CUDA device.
+ * (record bytes, coefficient lists, side data, tables) on the current CUDA device.
+ * Device memory: ten bytes per record byte (the record, its copy without stuffing, and eight for
+ * the values that those bits can hold, whatever k is asked for), 18 bytes per 8x8 block, and per
+ * block of the scan's component 8 or 16 bytes for every AC first pass and 32 for every AC
+ * refinement: 650 MB for an ImageNet-shaped record of 1024 images and 26 MB.  A record near the
+ * 4 GiB limit takes more than 40 GB.
  *   bytes : the whole record, HOST memory (pinned memory makes the copies asynchronous).
  *           BORROWED: it must stay valid and unchanged until pcr_close.
  *   len   : its length in bytes (< 4 GiB).
@@ -81,7 +86,8 @@ typedef struct {
  * decode of the record waits (on the device) for that set-up first.  Different records may be
  * opened and used from different host threads at the same time (a loader parses the next record
  * while the current one decodes); one record belongs to one thread at a time.  Device buffers of
- * closed records are kept for later opens (pcr_release_cached_memory returns them).
+ * closed records, and the page-locked host blocks in which the tables are built (up to 256 MiB),
+ * are kept for later opens (pcr_release_cached_memory returns them).
  * Errors: PCR_E_ARG, PCR_E_FORMAT, PCR_E_NOMEM, PCR_E_CUDA. */
 int pcr_open(const void* bytes, size_t len, pcr_record** rec);
 
@@ -250,10 +256,10 @@ int pcr_get_sampling(const pcr_record* rec, int* hs, int* vs, int* ncomp);
 /* Stage timing for benchmarks.  With profiling enabled every pcr_decode records CUDA events
  * on its stream around each stage; after the stream has been synchronised pcr_get_profile
  * returns, for the last decode, up to `cap` entries {name, milliseconds, kernel launches}.
- * Stages: "h2d" (prefix copy), "clear" (nothing of size; kept for readers of the list), "index"
+ * Stages: "h2d" (prefix copy), "clear" (the status words; kept for readers of the list), "index"
  * (restart-interval index, unstuffed copy and symbol tables), "entropy0".."entropyW" (one per wave
- * that ran), "pixels" (blocks expanded with their refinements, then the pixel stage).  *n = entries
- * written. */
+ * that ran), "chains" (the AC refinements of scans without restart markers, where there are any),
+ * "pixels" (blocks expanded with their refinements, then the pixel stage).  *n = entries written. */
 typedef struct {
     char name[24];
     float ms;
@@ -316,22 +322,24 @@ void pcr_close(pcr_record* rec);
 
 /* Cache of closed records (Section 5: a loader reads the same records epoch after epoch).  With a
  * limit above zero pcr_close parks the whole record (parse results, device tables and buffers:
- * about 1.5 GB for a 1024-image ImageNet-shaped record) instead of freeing it, and a later pcr_open
+ * about 650 MB for a 1024-image ImageNet-shaped record) instead of freeing it, and a later pcr_open
  * of the same record takes it back, which saves the host-side walk over every image's marker
- * segments and the table uploads (about 0.7 ms per 1024 images).  The handle it returns is fresh:
+ * segments and the table uploads (0.38 -> 0.15 ms for 1024 images).  The handle it returns is fresh:
  * nothing resident, nothing decoded, default settings.  A record is recognised by the address and
  * length of its bytes, the PCR_SLICES / PCR_LONG_MIN_BYTES settings, the current device, and a
  * hash of its header, sample metadata, index (position and length of every chunk) and the first
  * 256 bytes of every image's first chunk (frame header, quantisation and Huffman tables).  Bytes
  * that changed elsewhere under the same address are the caller's responsibility, exactly as for
- * an open handle.
+ * an open handle: a decode clears nothing, it writes what its bytes hold, so a block without
+ * coefficients in the new bytes shows those that the old bytes left.
  *   max_device_bytes : device memory the parked records may hold together; the least recently
  *                      closed ones are freed beyond it; 0 (the default) switches the cache off
  *                      and frees what it holds.
  * Errors: none (always PCR_OK). */
 int pcr_set_record_cache(size_t max_device_bytes);
 
-/* Returns the cached device buffers of closed records (and parked records) to the driver. */
+/* Returns the cached device buffers and page-locked host blocks of closed records (and parked
+ * records) to the driver. */
 void pcr_release_cached_memory(void);
 
 #ifdef __cplusplus

@@ -146,7 +146,7 @@ __device__ __forceinline__ void tables_warp(const Params& P, const ScanList& sl,
 // Tile by tile of 512 bytes, lanes take 16-byte slices.  Stuffed zeros and markers are found four bytes at
 // a time; one warp prefix sum places the slices; a lane writes the output words that begin in its slice,
 // taking up to three bytes of the last one from its neighbour, so nothing goes through shared memory.  (The
-// byte-by-byte form with a staging row took 680 warp instructions a tile, this one about 200; bound by the
+// byte-by-byte form with a staging row took 680 warp instructions a tile, this one about 300; bound by the
 // latency of one warp's tiles, up to 50 for a baseline JPEG of 25 KB.  1024 ImageNet-shaped images at k = 10 125 -> 68 us.)
 // Blocks from index_blocks on build the lookup tables of the same scans and images (one warp per table).
 // ---------------------------------------------------------------------------------------
@@ -552,7 +552,7 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, I
     const int s = (int)((item.si + (half ? item.pair : 0u)) / (uint32_t)P.N);
     const ScanScript sc = P.script[s];
     const ScanAux ax = P.saux[s];
-    const bool dc = sc.Ss == 0;              // a DC first pass (DC refinement scans go to dc_refine_kernel)
+    const bool dc = sc.Ss == 0;              // a DC first pass (DC refinement scans have no items)
     // tables: a DC scan may use two tables of one image; an AC item may span two images
     const bool two_images = item.next != 0;
     const uint32_t si1 = two_images ? item.next - 1u : item.si + item.pair;
@@ -884,7 +884,7 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, I
 // symbol goes through the same instructions as the others (its entry has no run, its value is the
 // difference), stores are predicated, and what changes from block to block comes from a small table
 // in shared memory.  Coefficients go where the progressive first passes put them.
-// Bound by the length of a lane's chain (a row of 31 MCUs has about 2200 symbols; 13 % of the issue slots are used).  1024
+// Bound by the length of a lane's chain (a row of 31 MCUs has about 2200 symbols; 28 % of the issue slots are used).  1024
 // ImageNet-shaped images: 1294 us with a branch per kind of symbol, 676 us now.
 // ---------------------------------------------------------------------------------------
 constexpr int kSeqWarps = 2;

@@ -204,8 +204,8 @@ struct pcr_record {
     cudaEvent_t ev_start = nullptr;                             // index of the first wave done
     cudaEvent_t ev_fork = nullptr;
     cudaStream_t copy_stream = nullptr;                         // host-to-device copies of later scan groups
-    cudaStream_t clear_stream = nullptr;                        // index of the later waves, beside the first entropy wave
-    cudaEvent_t ev_clear = nullptr;
+    cudaStream_t side_stream = nullptr;                         // index of the later waves, beside the first entropy wave
+    cudaEvent_t ev_side = nullptr;
     std::vector<cudaEvent_t> ev_copy;                           // [n_waves] bytes of wave w have arrived
     std::vector<cudaEvent_t> ev_join;
     std::vector<std::vector<int>> wave_scans;
@@ -213,7 +213,7 @@ struct pcr_record {
     // scan s follows, or -1.  Empty when the script has no such pair.
     std::vector<std::vector<int>> paired_waves;
     std::vector<int> pair_of;
-    bool pairs_fit = true;                                      // the waves with pairs fit the machine at once
+    bool pairs_fit = true;                                      // the waves with pairs fit the machine (see open_impl)
     std::vector<uint32_t> pair_begin, pair_count;               // [n_slices][G] items of the pair, by its later scan
     uint32_t n_units = 0;
     // device state
@@ -457,10 +457,10 @@ void free_device(pcr_record* r) {
     r->ev_fork = nullptr;
     if (r->copy_stream) pool_stream_put(r->copy_stream, r->device);
     r->copy_stream = nullptr;
-    if (r->clear_stream) pool_stream_put(r->clear_stream, r->device);
-    r->clear_stream = nullptr;
-    if (r->ev_clear) pool_event_put(r->ev_clear, r->device);
-    r->ev_clear = nullptr;
+    if (r->side_stream) pool_stream_put(r->side_stream, r->device);
+    r->side_stream = nullptr;
+    if (r->ev_side) pool_event_put(r->ev_side, r->device);
+    r->ev_side = nullptr;
     for (cudaEvent_t e : r->ev_copy) pool_event_put(e, r->device);
     r->ev_copy.clear();
     for (cudaEvent_t e : r->ev_join) pool_event_put(e, r->device);
@@ -824,13 +824,11 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     uint32_t n_items = 0;
     r->item_begin.assign((size_t)r->n_slices * G, 0); r->item_count.assign((size_t)r->n_slices * G, 0);
     // A scan that is one restart interval of at least this many bytes goes to the kernels for long
-    // intervals; DC refinement scans have a kernel of their own and no items at all.
+    // intervals; DC refinement scans have no items at all (see dc_refine_image).
     uint32_t long_min = 64;
     if (const char* e = getenv("PCR_LONG_MIN_BYTES")) long_min = (uint32_t)std::max(0, atoi(e));
     auto is_long = [&](int s, uint32_t i) {
-        const ScanScript& sc = r->script[s];
         const ScanDesc& sd = scans[(size_t)s * N + i];
-        (void)sc;
         return sd.nseg == 1 && sd.data_end - sd.data_off >= long_min && sd.data_end - sd.data_off < (1u << 27);   // (the chains count half bits)
     };
     // the AC refinements of one component of one image go together: all of them one interval each,
@@ -931,8 +929,11 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
             r->pair_count[(size_t)g * G + s] = n_items - begin;
         }
     // Pairs shorten the chain but leave the lanes of the shorter scan idle (about 1.4 times the warp instructions for the
-    // ten-scan script), so they are for records whose waves fit the machine at once (18 warps an SM): 96 images of
-    // 4:4:4 552 -> 434 us, 512 ImageNet-shaped images raised 2 -> 10 797 -> 768, 1024 of them at k = 10 991 -> 1022.
+    // ten-scan script), so they are for records whose waves fit the machine, or nearly: it holds 18 of these warps an SM (three
+    // warps and 36 KB of shared memory a CTA), and up to 20 an SM the few that wait cost less than the chain gains.  Without and
+    // with pairs, by warps an SM, decode at k = 10 in us: ImageNet-shaped images 17.2 656 and 639, 18.3 671 and 640, 19.1 679 and
+    // 669, 20.8 700 and 700, 20.9 707 and 728, 23.6 775 and 778, 34 957 and 997; CelebA-shaped 18.2 452 and 441; mixed
+    // sizes in 4:4:4 2.3 551 and 438.  Raised 2 -> 10: 17.2 642 and 555, 34 834 and 853.
     if (on_device && cudaDeviceGetAttribute(&r->n_sms, cudaDevAttrMultiProcessorCount, r->device) != cudaSuccess) return PCR_E_CUDA;
     for (const std::vector<int>& scans_of_wave : r->paired_waves) {
         std::vector<char> in_pair(G, 0);
@@ -987,8 +988,8 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     if (r->n_slices > 1) {
         if (!(r->ev_fork = pool_event_get(r->device))) return PCR_E_CUDA;
         if (!(r->copy_stream = pool_stream_get(r->device))) return PCR_E_CUDA;
-        if (!(r->clear_stream = pool_stream_get(r->device))) return PCR_E_CUDA;
-        if (!(r->ev_clear = pool_event_get(r->device))) return PCR_E_CUDA;
+        if (!(r->side_stream = pool_stream_get(r->device))) return PCR_E_CUDA;
+        if (!(r->ev_side = pool_event_get(r->device))) return PCR_E_CUDA;
         if (!(r->ev_start = pool_event_get(r->device))) return PCR_E_CUDA;
         if (!(r->ev_chain = pool_event_get(r->device))) return PCR_E_CUDA;
         for (int w = 0; w < r->n_waves; ++w) {
@@ -1004,7 +1005,6 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
             r->streams.push_back(q);
             if (!(e = pool_event_get(r->device))) return PCR_E_CUDA;
             r->ev_join.push_back(e);
-
         }
     }
     return PCR_OK;
@@ -1297,11 +1297,7 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
     bool paired = false;
     for (int s = 0; s < k && rec->pairs_fit; ++s) paired = paired || (rec->pair_of[s] >= k0);
     const std::vector<std::vector<int>>& waves = paired ? rec->paired_waves : rec->wave_scans;
-    int first_refine_wave = -1;                 // wave of the first AC refinement this call decodes
-    for (int s = k0; s < k; ++s)
-        if (rec->script[s].Ss > 0 && rec->script[s].Ah > 0 && (first_refine_wave < 0 || rec->wave_of_scan[s] < first_refine_wave))
-            first_refine_wave = rec->wave_of_scan[s];
-    const bool chains = first_refine_wave >= 0 && rec->n_groups > 0;
+    const bool chains = fl.n[0] + fl.n[1] + fl.n[2] > 0 && rec->n_groups > 0;
     const int chain_depth = kChainPairs / 4;    // chains per scheduler of the chain launch
     PixelPlan plan;
     plan.samp = sampling_code(rec->hs, rec->vs, rec->nc);
@@ -1324,7 +1320,8 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
     rec->decoded_k = rec->lists_k = k;
     const int G = rec->G;
     std::vector<char> copied(rec->n_waves, 0);      // wave w has to wait for its copy event
-    // the stages of one slice; stage numbers: 0 clear, 1 index, 2+w entropy wave w, 2+W unused, 3+W pixels
+    // the stages of one slice; stage numbers: 0 nothing (in the profile: the status words' memset), 1 index, 2+w entropy wave w,
+    // 2+W chains, 3+W pixels
     const int W = (int)waves.size();
     std::vector<char> indexed(rec->n_waves, 0);     // wave w of the current slice has an index launch to wait for
     // index (and lookup tables, where the interval kernels will want them) of the listed scans, all images
@@ -1349,7 +1346,7 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
     auto run_stage = [&](int stage, int g, cudaStream_t q) -> bool {
         const uint32_t i0 = rec->slice_img[g], i1 = rec->slice_img[g + 1];
         const uint32_t u0 = rec->slice_unit[g], nu = rec->slice_unit[g + 1] - u0;
-        if (stage == 0) return true;             // (nothing to clear: every decode writes the same values to the same places)
+        if (stage == 0) return true;             // (coefficients need no clearing: every decode writes the same values to the same places)
         if (stage == 1) {
             if (pipelined || g != 0) return true;   // done wave by wave, as the bytes arrive; one launch covers every slice
             ScanList sl;
@@ -1526,7 +1523,7 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
         // every slice is its own pipeline on its own stream, forked from and joined to the caller's;
         // missing record bytes arrive on a copy stream, the scan groups of each wave behind an event
         if (cudaEventRecord(rec->ev_fork, st) != cudaSuccess) return PCR_E_CUDA;
-        if (cudaStreamWaitEvent(rec->clear_stream, rec->ev_fork, 0) != cudaSuccess) return PCR_E_CUDA;
+        if (cudaStreamWaitEvent(rec->side_stream, rec->ev_fork, 0) != cudaSuccess) return PCR_E_CUDA;
         if (rec->resident < need) {
             bool any = false;
             for (int w = 0; w < W; ++w) {
@@ -1549,10 +1546,10 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
         if (launch_index(0, st) < 0) return PCR_E_CUDA;
         if (cudaEventRecord(rec->ev_start, st) != cudaSuccess) return PCR_E_CUDA;
         for (int w = 1; w < W; ++w) {
-            const int li = launch_index(w, rec->clear_stream);
+            const int li = launch_index(w, rec->side_stream);
             if (li < 0) return PCR_E_CUDA;
             indexed[w] = li > 0;
-            if (li > 0 && cudaEventRecord(rec->ev_index[w], rec->clear_stream) != cudaSuccess) return PCR_E_CUDA;
+            if (li > 0 && cudaEventRecord(rec->ev_index[w], rec->side_stream) != cudaSuccess) return PCR_E_CUDA;
         }
         // with a chain launch the slices meet once: it follows the entropy waves of all of them
         const int meet = chains ? 2 + W : n_stages;
@@ -1581,8 +1578,8 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
         }
         // the side and copy streams rejoin the caller's stream too (implied by the slices' waits
         // whenever they carried work; stated so that every fork is joined)
-        if (cudaEventRecord(rec->ev_clear, rec->clear_stream) != cudaSuccess) return PCR_E_CUDA;
-        if (cudaStreamWaitEvent(st, rec->ev_clear, 0) != cudaSuccess) return PCR_E_CUDA;
+        if (cudaEventRecord(rec->ev_side, rec->side_stream) != cudaSuccess) return PCR_E_CUDA;
+        if (cudaStreamWaitEvent(st, rec->ev_side, 0) != cudaSuccess) return PCR_E_CUDA;
         if (copied[W - 1] && cudaStreamWaitEvent(st, rec->ev_copy[W - 1], 0) != cudaSuccess) return PCR_E_CUDA;
     }
     if (cudaEventRecord(rec->ev_done, st) != cudaSuccess) return PCR_E_CUDA;

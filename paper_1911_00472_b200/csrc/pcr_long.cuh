@@ -1,12 +1,13 @@
 // Entropy stage for scans that are ONE long restart interval (records written without restart
-// markers: one entropy-coded segment per image and scan), and the DC refinement scans of any record.
+// markers: one entropy-coded segment per image and scan), and DC refinement scans in waves without AC refinements.
 //
 // A Huffman stream is a serial chain, so a whole scan on one lane takes tens of thousands of
 // dependent steps.  These kernels shorten or remove that chain:
 //
-//  * dc_refine_image / dc_refine_kernel: a DC refinement scan carries exactly one raw bit per block, so after
+//  * dc_refine_kernel: a DC refinement scan carries exactly one raw bit per block, so after
 //    unstuffing bit j of a restart interval is block j of the interval in scan order: one thread
-//    per MCU, no chain at all.  Used for every record.
+//    per MCU, no chain at all (dc_refine_image).  Where the wave has AC refinements in interval warps, extra blocks
+//    of their launch do it instead (see entropy_kernel).
 //  * first_pass_long_kernel: DC and AC first passes.  One small CTA per (scan, image); the segment is
 //    cut into one subsequence of equal bit length per thread.  A thread that starts in the middle of the
 //    stream does not know where a code begins nor which coefficient (or which block of the MCU) it is
@@ -525,7 +526,10 @@ __global__ void __launch_bounds__(32 * kSeqLongWarps) sequential_long_kernel(Par
 // A symbol is two dependent loads and a handful of additions (about 15 instructions; 35 with a bit reader and
 // symbol records).  Per block the thread leaves the bit position where it began; the helper warp decodes the
 // 32 blocks of a finished batch once more, one lane per block, to make the side data.
-// HAM-shaped record, 1024 images: the launch 3.4 -> 1.7 ms (about 100 cycles a symbol, 60 a block on the longest chain).
+// HAM-shaped record, 1024 images: the launch 3.4 -> 1.7 ms, which is the longest luminance chain's (24.2 k symbols in 4275
+// blocks; all luminance chains start at once, the last chroma chain ends at 1.1 ms).  That chain takes 1.40 ms with at
+// most one chain a scheduler (89 cycles a symbol, 139 a block with its share of the meetings), 1.71 among sixteen an SM
+// (102 and 204).
 //
 // A later refinement of the same component needs the masks the earlier one leaves, block by
 // block.  Both walk the same block grid in the same order, so the later chain runs behind the

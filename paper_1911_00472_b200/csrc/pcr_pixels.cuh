@@ -248,7 +248,7 @@ __device__ __forceinline__ bool expand_block(const Params& P, const CoefLists& c
 // One thread per block through the whole transform; the chroma samples go through shared memory, the luminance
 // samples stay in the registers of the thread that made them and meet the chroma there, two pixels
 // per instruction (16-bit pairs).  Bound by instruction issue (integer multiplications and additions of the transform, about
-// 0.6 of the slots).  Pixel stage of 1024 ImageNet-shaped images, before (lines of 128 bytes per block, colour as a
+// 0.65 of the slots, 0.73 with kCoarse).  Pixel stage of 1024 ImageNet-shaped images, before (lines of 128 bytes per block, colour as a
 // step of its own) and now: k = 5 348 -> 166 us, k = 10 562 -> 348 us, baseline 351 -> 265 us.
 template <bool kRefine, int kMode, bool kRoi = false, int kStage = 0, int kSamp = kSamp420, bool kCoarse = false>
 __global__ void __launch_bounds__(unit_threads<kSamp>(), (kCoarse ? 1152 : 672) / unit_threads<kSamp>())

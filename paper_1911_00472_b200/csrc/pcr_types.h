@@ -128,8 +128,10 @@ struct Params {
                                 //    positions are the masks of the scan's side data.  A coefficient takes at least two
                                 //    bits of the stream, so the values of whatever begins at byte b of the
                                 //    unstuffed copy begin at index 4 b and nothing overlaps.
-                                // Every decode of a record writes the same values to the same places, so none of this is
-                                // cleared between decodes
+                                //    (Eight bytes per record byte: more than planes would take from about 0.4 bytes a
+                                //    pixel on in 4:2:0.)
+                                // Every decode of a record's bytes writes the same values to the same places, so none of this
+                                // is cleared between decodes
     const ScanScript* script;   // [G]
     const ScanAux* saux;        // [G]
     uint64_t* aux;              // side data of the AC scans

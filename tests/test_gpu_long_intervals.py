@@ -1,7 +1,7 @@
 """Records written without restart markers: every scan of an image is one long entropy-coded
-segment (the HAM10000-shaped workload).  Such scans take kernels of their own: first passes are
-decoded from 32 speculative entry points that re-synchronise, AC refinements by one chain per warp,
-DC refinements bit-parallel.  Here those kernels are compared with the oracle bit for bit at every
+segment (the HAM10000-shaped workload).  Such scans take kernels of their own: first passes and
+sequential scans are decoded from 64 or 128 speculative entry points that re-synchronise, AC refinements
+by chains of a decoding thread and a helper warp, DC refinements bit-parallel.  Here those kernels are compared with the oracle bit for bit at every
 fidelity, also on inputs far smaller than the ones they are meant for (the size threshold that
 routes a scan to them is lowered through PCR_LONG_MIN_BYTES, read when a record is opened), so that
 empty subsequences, blocks shared by neighbouring lanes and images of a single block are covered."""
