@@ -3,8 +3,8 @@
 
 One step = one pcr_decode of one synthetic ImageNet-shaped record (1024 images, sizes
 256..496, quality 90, 4:2:0, ten scans, restart every MCU row) at fidelity k: restart-interval
-index, Huffman decode of scans 1..k into int16 coefficient planes, refinement in place,
-dequantise / inverse DCT / upsample / colour convert to packed RGB.  `value` is measured with the
+index, Huffman decode of scans 1..k into int16 coefficient lists and refinement side data, then blocks expanded and
+refined, dequantise / inverse DCT / upsample / colour convert to packed RGB.  `value` is measured with the
 record already resident in device memory; `e2e` copies the record prefix from pinned host
 memory inside every step and reads the status words back.
 
@@ -71,15 +71,14 @@ def whole_job_rate(images_this_rank: int, steps: int, ms_this_rank: float, world
 
 
 def algorithmic_bytes(scans, infos, k: int, chains: bool = False):
-    """Bytes the method has to move for one decode at fidelity k, per stage.
+    """Bytes of one decode at fidelity k through planes of whole blocks, per stage: a fixed measure of the work, reported as
+    `plane_model_bytes_per_step` and nowhere else (this implementation keeps lists and moves layout_bytes).
 
     scans: [(ncomp, comp0, Ss, Se, Ah, wave, group_bytes)], infos: [(W, H)].
       index    : bytes of scan groups <= k, read once
       entropyW : compressed bytes of the wave's scans + 2 bytes per coefficient of every
                  block the scan visits (written once by a first pass, read and written by a
-                 refinement).  The refinement's share is what the method has to move for that
-                 step; this implementation moves it in the pixel kernel, which folds the
-                 refinement side data into the planes before it transforms a block.
+                 refinement)
       chains   : (records without restart markers) the AC refinements' share of the above, when the
                  library runs them as one stage of their own
       clear    : 128 bytes per block
@@ -119,6 +118,51 @@ def algorithmic_bytes(scans, infos, k: int, chains: bool = False):
     return out
 
 
+def layout_bytes(scans, infos, k: int, chains: bool = False):
+    """Bytes the stages of one decode at fidelity k exchange with memory in the layout the library keeps (4:2:0), as far as
+    they follow from the shapes: the non-zero values and the records of non-empty blocks that AC first passes write
+    depend on the contents and are not counted, so this is a lower bound.  Arguments as for algorithmic_bytes.
+      index    : bytes of scan groups <= k read, the copy without stuffing written
+      entropyW : that copy read; a DC first pass writes 2 bytes per block, a DC refinement reads and writes them; an AC
+                 refinement reads 8 bytes per block and mask source and writes 32 per block
+      chains   : the AC refinements' share, when they ran as one stage of their own
+      pixels   : per block 2 bytes DC and 16 of positions 1..7 (no AC scan: DC alone), 16 per first pass that reaches
+                 beyond position 7, 32 per refinement; 3 bytes per pixel written
+    """
+    out = {"index": 0.0, "pixels": 0.0}
+    pad, unp, px = [0, 0, 0], [0, 0, 0], 0
+    for W, H in infos:
+        mcus = ((W + 15) // 16) * ((H + 15) // 16)
+        cw, ch = (W + 1) // 2, (H + 1) // 2
+        for c, (n, w, h) in enumerate(((4 * mcus, W, H), (mcus, cw, ch), (mcus, cw, ch))):
+            pad[c] += n
+            unp[c] += ((w + 7) // 8) * ((h + 7) // 8)
+        px += W * H
+    chain_bytes = 0.0
+    any_ac = any(Se > 0 for _, _, _, Se, _, _, _ in scans[:k])
+    out["pixels"] = 3.0 * px + (18.0 if any_ac else 2.0) * sum(pad)
+    for s, (ncomp, comp0, Ss, Se, Ah, wave, gbytes) in enumerate(scans[:k]):
+        out["index"] += 2.0 * gbytes
+        blocks = sum(pad) if ncomp > 1 else pad[comp0]
+        moved = float(gbytes)
+        if Ss == 0:
+            moved += (4.0 if Ah else 2.0) * blocks
+        elif Ah:
+            before = [t for t in range(s) if scans[t][2] > 0 and scans[t][1] == comp0 and scans[t][2] <= Se and Ss <= scans[t][3]]
+            sources = [t for t in before if not any(u > t and scans[u][4] and scans[u][2] <= scans[t][2] and scans[u][3] >= scans[t][3] for u in before)]
+            moved += (32.0 + 8.0 * len(sources)) * unp[comp0]
+        if Se >= 8 or Ah and Ss > 0:
+            out["pixels"] += (32.0 if Ah else 16.0) * blocks
+        if chains and Ah and Ss > 0:
+            chain_bytes += moved
+        else:
+            out[f"entropy{wave}"] = out.get(f"entropy{wave}", 0.0) + moved
+    if chains:
+        out["chains"] = chain_bytes
+    out["total"] = sum(out.values())
+    return out
+
+
 def source_hash() -> str:
     """Hash of the CUDA sources: ncu counters are only quoted for the kernels they were taken on."""
     import glob
@@ -152,8 +196,8 @@ def measured_traffic(stage: str, k: int, n_images: int):
 
 
 def measured_bytes_per_decode(k: int, n_images: int):
-    """All DRAM bytes one decode at fidelity k moves (kernels' ncu counters plus the sizes of the
-    memsets), from the committed capture, or None."""
+    """All DRAM bytes one decode at fidelity k moves (kernels' ncu counters plus the size of the
+    status words' memset), from the committed capture, or None."""
     t = _traffic_table()
     if t is None or n_images != 1024:
         return None
@@ -425,7 +469,7 @@ def streamed_sweep(dev, recs, ks, peak, pool=None, cores=0, tmpdir=None):
         h2d = 0
         for d in decs:
             scans = [sc + (binding.pcr_get_scan(d.handle, s).bytes,) for s, sc in enumerate(scans0)]
-            model += algorithmic_bytes(scans, [(i.width, i.height) for i in d.info], k)["total"]
+            model += layout_bytes(scans, [(i.width, i.height) for i in d.info], k)["total"]
             h2d += d.prefix_bytes(k)
         per_k[str(k)] = {"images_per_s": n_img / dt, "ms_per_record": 1000.0 * dt / R, "hbm_gbs_model": model / dt / 1e9,
                          "model_frac_of_peak": model / dt / 1e9 / peak, "h2d_bytes_per_record": h2d // R,
@@ -670,7 +714,7 @@ def main():
             torch.cuda.synchronize(dev)
             st = 5
             per_k[str(kk)] = n_img * st / (timed_steps(kk, st) / 1000.0)
-            hbm_by_k[str(kk)] = algorithmic_bytes(scans, infos, kk)["total"] * per_k[str(kk)] / n_img / 1e9
+            hbm_by_k[str(kk)] = layout_bytes(scans, infos, kk)["total"] * per_k[str(kk)] / n_img / 1e9
             mb = measured_bytes_per_decode(kk, n_img) if wl == WORKLOAD else None
             hbm_meas_by_k[str(kk)] = mb * per_k[str(kk)] / n_img / 1e9 if mb is not None else None
         # decode straight to a fixed-size training batch (random-resized crops, flip, 224 x 224, fp16)
@@ -780,7 +824,7 @@ def main():
             stage_ms[name] = stage_ms.get(name, 0.0) + t / reps
             stage_n[name] = nl
     binding.pcr_set_profiling(dec.handle, False)
-    model = algorithmic_bytes(scans, infos, k, chains=stage_n.get("chains", 0) > 0)
+    model = layout_bytes(scans, infos, k, chains=stage_n.get("chains", 0) > 0)
     kernels = {n: t for n, t in stage_ms.items() if stage_n.get(n, 0) > 0}
     dom = max(kernels, key=kernels.get)
     peak, peak_src = hbm_peak()
@@ -791,6 +835,7 @@ def main():
                 "traffic": traffic, "peak_source": peak_src, "kernel_ms": kernels[dom],
                 "algorithmic_bytes_per_launch": model[dom],
                 "whole_path": {"algorithmic_bytes_per_step": model["total"], "achieved": whole, "frac": whole / peak},
+                "plane_model_bytes_per_step": algorithmic_bytes(scans, infos, k)["total"],
                 "step_ms": {"pipelined": ms_max / args.steps, "stages_one_after_the_other": sum(stage_ms.values()),
                             "note": "value is timed in the pipelined layout (image slices on their own streams); the stage "
                                     "times below come from the profiling layout, one stage after the other"},
@@ -832,13 +877,12 @@ def main():
             "hbm_model_frac_of_peak_by_k": {kk: v / peak for kk, v in hbm_by_k.items()},
             "hbm_gbs_measured_by_k": hbm_meas_by_k,
             "hbm_measured_frac_of_peak_by_k": {kk: (v / peak if v is not None else None) for kk, v in hbm_meas_by_k.items()},
-            "hbm_by_k_note": "model: algorithmic bytes of the decode at k (compressed prefix, zeroed and written coefficient planes, "
-                             "planes read by the pixel stage, pixels written) / time: a rate of useful work, NOT an achieved "
-                             "bandwidth (below k = 5 the implementation moves far fewer bytes than the model: positions 0..7 of "
-                             "every block live in a dense plane, the 128-byte lines are neither zeroed nor read while no scan "
-                             "reaches position 8).  measured: DRAM bytes the kernels and memsets of one decode really move "
-                             "(ncu dram__bytes of every kernel, committed under profiles/) / the same time; null when the "
-                             "kernels changed since the capture", "raise_fidelity_ms_per_record": raise_ms,
+            "hbm_by_k_note": "model: bytes the stages of a decode at k exchange with memory in the library's layout, as far as they follow "
+                             "from the shapes (compressed prefix read and copied without stuffing, DC and head planes, block records, "
+                             "refinement side data, pixels; without the values of AC first passes) / time; part of it stays in L2.  "
+                             "measured: DRAM bytes the kernels and memsets of one decode really move (ncu dram__bytes of every kernel, "
+                             "committed under profiles/) / the same time; null when the kernels changed since the capture",
+            "raise_fidelity_ms_per_record": raise_ms,
             "training_tensor": training_tensor, "predicted_io_speedup_by_k": io_speedup, "fidelity": fidelity, "baseline_jpeg": baseline_jpeg, "triangle_upsampling": triangle,
         }))
     dec.close()

@@ -59,3 +59,25 @@ def test_algorithmic_bytes_model():
     assert m["entropy1"] == 70 + 2 * 63 * 16 * 2
     m2 = bench.algorithmic_bytes(scans, [(32, 32)], 1)
     assert "entropy1" not in m2 and m2["index"] == 100
+
+
+def test_layout_bytes_model():
+    sys.path.insert(0, ROOT)
+    import bench
+    # one 17x20 image: 2x2 MCUs, so 16 + 4 + 4 padded blocks; Y unpadded 3 x 3, chroma 2 x 2 each
+    scans = [(3, 0, 0, 0, 0, 0, 100), (1, 0, 1, 5, 0, 0, 50), (1, 0, 6, 63, 0, 0, 60), (1, 0, 1, 63, 2, 1, 70), (3, 0, 0, 0, 1, 1, 3),
+             (1, 0, 1, 63, 1, 2, 90)]
+    infos = [(17, 20)]
+    m = bench.layout_bytes(scans, infos, 6)
+    assert m["index"] == 2 * 373
+    assert m["entropy0"] == 210 + 2 * 24                      # DC values; what AC first passes write depends on the contents
+    assert m["entropy1"] == 70 + (32 + 2 * 8) * 9 + 3 + 4 * 24   # masks of two earlier scans, DC bits read and written
+    assert m["entropy2"] == 90 + (32 + 8) * 9                 # the earlier refinement's mask covers both
+    assert m["pixels"] == 3 * 340 + 18 * 24 + (16 + 32 + 32) * 16
+    assert m["total"] == sum(v for n, v in m.items() if n != "total")
+    c = bench.layout_bytes(scans, infos, 6, chains=True)
+    assert c["total"] == m["total"] and c["chains"] == m["entropy2"] + 70 + (32 + 2 * 8) * 9 and c["entropy1"] == 3 + 4 * 24
+    assert bench.layout_bytes(scans, infos, 1)["pixels"] == 3 * 340 + 2 * 24
+    assert bench.layout_bytes(scans, infos, 2)["pixels"] == 3 * 340 + 18 * 24
+    b = bench.layout_bytes([(3, 0, 0, 63, 0, 0, 400)], infos, 1)        # baseline
+    assert b["entropy0"] == 400 + 2 * 24 and b["pixels"] == 3 * 340 + (18 + 16) * 24
