@@ -518,9 +518,11 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     uint64_t meta_off = rd64(rec + 24), index_off = rd64(rec + 32), data_off = rd64(rec + 40), total = rd64(rec + 48);
     if (N == 0 || G == 0 || G > 64 || N > (1u << 24)) return PCR_E_FORMAT;
     if (total != len) return PCR_E_FORMAT;
-    if (meta_off < 64 || meta_off + 16ull * N > len) return PCR_E_FORMAT;
-    if (index_off < 64 || index_off + 8ull * (G + 1) + 16ull * G * N > len) return PCR_E_FORMAT;
-    if (data_off > len || data_off < index_off + 8ull * (G + 1) + 16ull * G * N) return PCR_E_FORMAT;
+    // (offsets are compared with what is left behind them: a sum with one near 2^64 would wrap)
+    const uint64_t index_len = 8ull * (G + 1) + 16ull * G * N;
+    if (meta_off < 64 || meta_off > len || 16ull * N > len - meta_off) return PCR_E_FORMAT;
+    if (index_off < 64 || index_off > len || index_len > len - index_off) return PCR_E_FORMAT;
+    if (data_off > len || data_off < index_off + index_len) return PCR_E_FORMAT;
     r->host = rec; r->len = len; r->N = (int)N; r->G = (int)G;
     r->group_end.resize(G + 1);
     for (uint32_t g = 0; g <= G; ++g) r->group_end[g] = rd64(rec + index_off + 8ull * g);
@@ -556,7 +558,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
             uint64_t off = rd64(c);
             uint32_t clen = rd32(c + 8);
             uint64_t padded = ((uint64_t)clen + 15) & ~15ull;
-            if ((off & 15) || off < r->group_end[g] || off + padded > r->group_end[g + 1]) return PCR_E_FORMAT;
+            if ((off & 15) || off < r->group_end[g] || off > r->group_end[g + 1] || padded > r->group_end[g + 1] - off) return PCR_E_FORMAT;
             if (clen >= (1u << 28)) return PCR_E_FORMAT;        // bit positions inside a scan are 32-bit
             ScanParse sp;
             int rc = parse_chunk(rec, off, clen, g == 0, im, sp);
@@ -1049,7 +1051,7 @@ uint64_t record_identity(const uint8_t* rec, size_t len) {
     const uint32_t N = rd32(rec + 8), G = rd32(rec + 12);
     const uint64_t index_off = rd64(rec + 32), data_off = rd64(rec + 40);
     if (N == 0 || G == 0 || G > 64 || N > (1u << 24) || data_off > len) return 0;
-    if (index_off < 64 || index_off + 8ull * (G + 1) + 16ull * G * N > data_off) return 0;
+    if (index_off < 64 || index_off > data_off || 8ull * (G + 1) + 16ull * G * N > data_off - index_off) return 0;
     uint64_t h = hash_bytes(len, rec, (size_t)data_off);        // header, sample metadata, index
     const uint8_t* chunk = rec + index_off + 8ull * (G + 1);
     for (uint64_t j = 0; j < (uint64_t)N; ++j) {              // the chunks of scan group 1: frame header and tables of every image

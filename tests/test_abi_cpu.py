@@ -54,6 +54,46 @@ def test_argument_errors_need_no_device(lib):
     assert lib.pcr_strerror(-3) == b"corrupt entropy-coded data"
 
 
+@pytest.mark.parametrize("cache", [0, 1 << 30])
+def test_offsets_near_the_end_of_the_64_bit_range(tmp_path, lib, cache):
+    """Offsets so large that adding a length to them wraps are refused like any other offset past the end; with the cache of
+    closed records on too, which looks at the record before it is opened.  (In a child, behind a page without access: a wrong
+    check reads in front of the record.)"""
+    import struct
+    import subprocess
+    import sys
+    import pcr_synth
+    rec = pcr_synth.make_record(0, n_images=3).bytes
+    index_off = struct.unpack_from("<Q", rec, 32)[0]
+    chunk = index_off + 8 * 11
+    names = []
+    for at in (24, 32, 40, index_off, index_off + 8 * 10, chunk, chunk + 16 * 7):      # meta, index, data, group ends, chunks
+        for value in ((1 << 64) - 16, (1 << 64) - 64, (1 << 63), (1 << 32) - 16):
+            bad = rec.copy()
+            struct.pack_into("<Q", bad, at, value)
+            names.append(str(tmp_path / f"{at}_{value}"))
+            bad.tofile(names[-1])
+    code = ("import ctypes, mmap, sys\n"
+            "lib = ctypes.CDLL(sys.argv[1])\n"
+            "lib.pcr_set_record_cache.argtypes = [ctypes.c_size_t]\n"
+            "lib.pcr_set_record_cache(int(sys.argv[2]))\n"
+            "lib.pcr_open.argtypes = [ctypes.c_void_p, ctypes.c_size_t, ctypes.POINTER(ctypes.c_void_p)]\n"
+            "page = mmap.PAGESIZE\n"
+            "libc = ctypes.CDLL(None, use_errno=True)\n"
+            "libc.mprotect.argtypes = [ctypes.c_void_p, ctypes.c_size_t, ctypes.c_int]\n"
+            "for name in sys.argv[3:]:\n"
+            "    raw, h = open(name, 'rb').read(), ctypes.c_void_p()\n"
+            "    m = mmap.mmap(-1, page + len(raw))\n"
+            "    m[page:] = raw\n"
+            "    at = ctypes.addressof(ctypes.c_char.from_buffer(m))\n"
+            "    assert libc.mprotect(at, page, 0) == 0\n"
+            "    print(lib.pcr_open(at + page, len(raw), ctypes.byref(h)), flush=True)\n"
+            "    libc.mprotect(at, page, 3)\n")
+    res = subprocess.run([sys.executable, "-c", code, lib._name, str(cache)] + names, env=dict(os.environ, CUDA_VISIBLE_DEVICES=""),
+                         capture_output=True, text=True, timeout=120)
+    assert res.returncode == 0 and res.stdout.split() == ["-2"] * len(names), res
+
+
 def test_open_without_threads_to_be_had(tmp_path, lib):
     """pcr_open walks the images on a few threads; where none can be started it does the work itself, and nothing is thrown
     through the C ABI.  (A preloaded pthread_create that always fails; no device, so a valid record ends with PCR_E_CUDA.)"""
