@@ -15,6 +15,7 @@
 // inside it; one correction bit per set bit of the mask passed over) and leaves {new mask, correction bits, new
 // positions, their signs} as side data, which the pixel kernel applies when it expands the block.
 //
+// (AC refinements of records that do not fill the machine: pcr_refine.cuh.)
 // Bound by the latency of a lane's chain: about 155 warp instructions a refinement step (276 with masks searched for
 // the r-th zero and a bit reader that carries its state), at the issue rate that the resident warps allow.
 // 1024 ImageNet-shaped images at k = 10: the three waves 217 + 332 + 511 us before, 200 + 220 + 245 us now.
@@ -335,7 +336,7 @@ __device__ __forceinline__ uint64_t low_mask(int p) { return p >= 64 ? ~0ull : (
 // ---------------------------------------------------------------------------------------
 // Bit reader of the interval kernels.  The position is one number: bits counted from the first bit of a
 // 16-byte group of the unstuffed copy.  The words around it lie in the lane's column of a ring in shared
-// memory (one row more than the ring: it repeats row 0), so the window of the next 32 bits is two shared
+// memory (one row more than the ring: it repeats row 0; kAgain rows), so the window of the next 32 bits is two shared
 // loads and a funnel shift, and skipping is an addition: no buffer, no refill branch.  All lanes top their
 // columns up together.  `stop` is the first position at which a step may not begin (the ring runs out, the
 // interval has ended, the lane has nothing to do): one comparison per step.
@@ -344,8 +345,13 @@ __device__ __forceinline__ uint64_t low_mask(int p) { return p >= 64 ? ~0ull : (
 __device__ __forceinline__ uint32_t lds32(uint32_t a) { uint32_t v; asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory"); return v; }
 __device__ __forceinline__ uint32_t lds16(uint32_t a) { uint32_t v; asm volatile("ld.shared.u16 %0, [%1];" : "=r"(v) : "r"(a) : "memory"); return v; }
 __device__ __forceinline__ uint32_t lds8(uint32_t a) { uint32_t v; asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a) : "memory"); return v; }
+// nothing where `on` is false, without a branch
+__device__ __forceinline__ void sts16_if(bool on, uint32_t a, uint32_t v) {
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %2, 0; @p st.shared.u16 [%0], %1; }" : : "r"(a), "h"((uint16_t)v), "r"((uint32_t)on) : "memory");
+}
 __device__ __forceinline__ uint4 lds128(uint32_t a) { uint4 v; asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory"); return v; }
 __device__ __forceinline__ void sts32(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" : : "r"(a), "r"(v) : "memory"); }
+__device__ __forceinline__ void sts16(uint32_t a, uint32_t v) { asm volatile("st.shared.u16 [%0], %1;" : : "r"(a), "h"((uint16_t)v) : "memory"); }
 __device__ __forceinline__ void sts128(uint32_t a, const uint4& v) { asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" : : "r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory"); }
 // shifts that give 0 for counts of 32 and more
 __device__ __forceinline__ uint32_t shl0(uint32_t x, uint32_t n) { uint32_t y; asm("shl.b32 %0, %1, %2;" : "=r"(y) : "r"(x), "r"(n)); return y; }
@@ -360,6 +366,7 @@ template <class T> __device__ __forceinline__ void pin(T*& p) {
     p = static_cast<T*>(__cvta_global_to_generic(a));
 }
 
+template <uint32_t kWords = (uint32_t)kRingWords, uint32_t kAgain = 1>
 struct LaneBits {
     uint32_t col;          // shared address of this lane's column: row r at col + 128 r
     const uint4* g4;       // the 16-byte group that position 0 lies in
@@ -375,9 +382,9 @@ struct LaneBits {
         request();
     }
     __device__ __forceinline__ void put(uint32_t w, const uint4& v) {
-        const uint32_t p = col + (w & (kRingWords - 1)) * 128u;
+        const uint32_t p = col + (w & (kWords - 1)) * 128u;
         sts32(p, v.x); sts32(p + 128u, v.y); sts32(p + 256u, v.z); sts32(p + 384u, v.w);
-        if ((w & (kRingWords - 1)) == 0) sts32(p + kRingWords * 128u, v.x);
+        if ((w & (kWords - 1)) == 0) { sts32(p + kWords * 128u, v.x); if (kAgain > 1) sts32(p + kWords * 128u + 128u, v.y); }
     }
     // Top-up (all lanes of the warp together): what the next one will store first is requested right after
     // the previous one, so that its latency passes beside the decode steps.
@@ -387,7 +394,14 @@ struct LaneBits {
         va = __ldg(g); vb = __ldg(g + 1);
     }
     __device__ __forceinline__ void topup(bool on) {
-        const uint32_t room = on ? (kRingWords - (wr - (pos >> 5))) >> 2 : 0u;
+        take(on, on ? (kWords - (wr - (pos >> 5))) >> 2 : 0u);
+    }
+    // ... where the words from bit `keep` on are still needed and the ring holds more than one top-up brings; nothing is
+    // read far beyond the interval
+    __device__ __forceinline__ void topup_from(bool on, uint32_t keep) {
+        take(on, on && wr < (limit >> 5) + 8u ? min((kWords - (wr - (keep >> 5))) >> 2, 4u) : 0u);
+    }
+    __device__ __forceinline__ void take(bool on, uint32_t room) {
         if (room > 0) put(wr, va);
         if (room > 1) put(wr + 4, vb);
         if (room > 2) put(wr + 8, __ldg(g4 + (wr >> 2) + 2));
@@ -398,7 +412,7 @@ struct LaneBits {
     // steps may begin below this position: `words` words from the one the position lies in are in the ring
     __device__ __forceinline__ uint32_t ring_stop(uint32_t words) const { return 32u * (wr - min(wr, words - 1u)); }
     __device__ __forceinline__ uint32_t window(uint32_t at) const {
-        const uint32_t p = col + ((at << 2) & ((kRingWords - 1) * 128u));
+        const uint32_t p = col + ((at << 2) & ((kWords - 1) * 128u));
         return __funnelshift_l(lds32(p + 128u), lds32(p), at);    // (shift taken mod 32)
     }
 };
@@ -607,7 +621,7 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, I
         bad = true; done = true;
     }
     if (done) { bstart = sd.data_off; bend = sd.data_off; }
-    LaneBits br;
+    LaneBits<> br;
     br.init(mem + kWarpRing + 4u * lane, P.ubuf, bstart, bend);
     const int Al = sc.Al;
     if (m0 >= m1) done = true;
@@ -943,7 +957,7 @@ __global__ void __launch_bounds__(32 * kSeqWarps) sequential_kernel(Params P, ui
     bool bad = false;
     if (!done && (bstart < sd.data_off || bend > sd.data_end || bend < bstart)) { bad = true; done = true; }
     if (done) { bstart = sd.data_off; bend = sd.data_off; }
-    LaneBits br;
+    LaneBits<> br;
     br.init(mem + kSeqRing + 4u * lane, P.ubuf, bstart, bend);
     if (m0 >= m1) done = true;
 

@@ -27,6 +27,7 @@
 #include "pcr_long.cuh"
 #include "pcr_msssim.cuh"
 #include "pcr_pixels.cuh"
+#include "pcr_refine.cuh"
 #include "pcr_types.h"
 
 using namespace pcr;
@@ -214,6 +215,7 @@ struct pcr_record {
     std::vector<std::vector<int>> paired_waves;
     std::vector<int> pair_of;
     bool pairs_fit = true;                                      // the waves with pairs fit the machine (see open_impl)
+    uint32_t refine_ctas = 8;                                   // see refine_in_ctas (PCR_REFINE_CTAS overrides)
     std::vector<uint32_t> pair_begin, pair_count;               // [n_slices][G] items of the pair, by its later scan
     uint32_t n_units = 0;
     // device state
@@ -797,6 +799,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
             for (uint32_t s = 0; s < G; ++s) r->paired_waves[wave[s]].push_back((int)s);
         } else r->pair_of.assign(G, -1);
     }
+    if (const char* e = getenv("PCR_REFINE_CTAS")) r->refine_ctas = (uint32_t)std::max(0, atoi(e));
     // slices: enough images each to fill the machine, few enough to keep launches cheap
     {
         // four at most: one record decodes as fast with four slices as with eight, and two records
@@ -980,6 +983,8 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     units_kernel<<<N, 128, 0, r->up_stream>>>(r->d_imgs, r->d_order, r->d_unit_prefix, r->d_units, r->unit_mcus, r->unit_rows,
                                               r->d_scans, T.d<uint32_t>(at_base), G, bpm);
     ++g_launches;
+    if (cudaFuncSetAttribute(refine_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRefineBytes) != cudaSuccess ||
+        cudaFuncSetAttribute(refine_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRefineBytes) != cudaSuccess) return PCR_E_CUDA;
     if (n_groups && cudaFuncSetAttribute(ac_refine_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kChainPairs * sizeof(ChainShared))) != cudaSuccess) return PCR_E_CUDA;
     r->h_status.assign(N, 0);
     r->resident = 0;
@@ -1042,8 +1047,8 @@ uint64_t hash_bytes(uint64_t h, const uint8_t* p, size_t n) {
     return h;
 }
 uint32_t env_key() {
-    const char* a = getenv("PCR_SLICES"); const char* b = getenv("PCR_LONG_MIN_BYTES");
-    return (uint32_t)((a ? atoi(a) + 1 : 0) * 1000003 + (b ? atoi(b) + 1 : 0));
+    const char* a = getenv("PCR_SLICES"); const char* b = getenv("PCR_LONG_MIN_BYTES"); const char* c = getenv("PCR_REFINE_CTAS");
+    return ((a ? (uint32_t)atoi(a) + 1u : 0u) * 1000003u + (b ? (uint32_t)atoi(b) + 1u : 0u)) * 1009u + (c ? (uint32_t)atoi(c) + 1u : 0u);
 }
 // 0 when the bytes do not even look like a record (pcr_open then reports the error)
 uint64_t record_identity(const uint8_t* rec, size_t len) {
@@ -1254,6 +1259,25 @@ static void coef_lists(const pcr_record* rec, int k, CoefLists* cl) {
     for (int c = 0; c < 3; ++c) memcpy(&cl->head_mask[c], mask[c], 16);
 }
 
+// Whether refine_kernel's CTAs take the AC refinements among scans k0 .. k-1 of a wave, or lane-per-interval warps of
+// entropy_kernel.  A CTA's chains are four times as fast (170 to 220 against 700 cycles a symbol), but three CTAs are all an SM
+// holds, 96 chains against 576, so a launch of many items is better off with the warps.  Decode at k = 10 in us,
+// warps and CTAs, by CTAs an SM: ImageNet-shaped images 2 352 and 237, 3.8 405 and 304, 5.8 427 and 390, 7.8 422 and 372, 9.7 476
+// and 489, 11.7 534 and 568; CelebA-shaped 2.5 211 and 180, 5 235 and 225, 10 301 and 342, 20 489 and 519; mixed sizes in
+// 4:4:4 2.3 423 and 281, 6.2 422 and 281.
+static bool refine_in_ctas(const pcr_record* rec, const std::vector<int>& wave, bool paired, int k0, int k) {
+    uint64_t ctas = 0;
+    std::vector<char> counted(rec->G, 0);                     // scans that a pair's items stand for
+    for (int s : wave)
+        if (paired && s < k && rec->pair_of[s] >= k0) counted[rec->pair_of[s]] = 1;
+    for (int s : wave) {
+        if (s < k0 || s >= k || rec->script[s].Ss == 0 || rec->script[s].Ah == 0 || counted[s]) continue;
+        const std::vector<uint32_t>& items = paired && rec->pair_of[s] >= k0 ? rec->pair_count : rec->item_count;
+        for (int g = 0; g < rec->n_slices; ++g) ctas += items[(size_t)g * rec->G + s];
+    }
+    return ctas <= (uint64_t)rec->refine_ctas * (uint64_t)rec->n_sms;
+}
+
 // Decode scans k0 .. k-1 on top of the state scans 0 .. k0-1 left behind (k0 = 0: from scratch),
 // then produce the pixels of fidelity k.
 static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream, const TensorArgs* targs = nullptr) {
@@ -1367,26 +1391,28 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
             }
             const ScanScript& first = rec->script[waves[w][0]];
             const bool sequential = first.Ss == 0 && first.Se == 63;   // a baseline record: its one scan is sequential
-            // the runs of items of the wave's scans, pairs (the longest chains) first
-            ItemRuns runs;
-            runs.n = 0;
-            uint32_t count = 0;
+            // The runs of items of the wave's scans, pairs (the longest chains) first: those of lane-per-interval warps, and
+            // those of refine_kernel's CTAs.
+            ItemRuns runs, refs;
+            runs.n = refs.n = 0;
+            uint32_t count = 0, ref_count = 0;
             bool refine = false;                           // waves without AC refinements need no mask queues
-            int dc_n = 0;                                  // the wave's DC refinements, at most one per component
+            int dc_n = 0, dc_s[3];                         // the wave's DC refinements, at most one per component
             for (int s : waves[w])
-                if (s >= k0 && s < k && rec->script[s].Ss == 0 && rec->script[s].Ah != 0 && dc_n < 3) runs.dc_s[dc_n++] = s;
+                if (s >= k0 && s < k && rec->script[s].Ss == 0 && rec->script[s].Ah != 0 && dc_n < 3) dc_s[dc_n++] = s;
             bool dc_done = dc_n == 0;
+            auto carry_dc = [&](ItemRuns& with, unsigned chunks) -> unsigned {      // the DC refinements in extra blocks of a launch
+                with.dc_pos0 = i0; with.dc_images = i1 - i0; with.dc_chunks = chunks;
+                for (int j = 0; j < dc_n; ++j) with.dc_s[j] = dc_s[j];
+                dc_done = true;
+                return dc_n * with.dc_images * chunks;
+            };
             auto launch_items = [&](bool last) {
                 if (!count) return;
                 unsigned nb = (count + kEntropyWarps - 1) / kEntropyWarps;
                 const uint32_t smem = kEntropyWarps * (refine ? warp_bytes<true>() : warp_bytes<false>());
                 runs.item_blocks = nb;
-                if (last && refine && !dc_done) {          // (waves without AC refinements are compiled without this)
-                    runs.dc_pos0 = i0; runs.dc_images = i1 - i0;
-                    runs.dc_chunks = (rec->dc_refine_chunks + 1) / 2;      // about five MCUs a thread
-                    nb += dc_n * runs.dc_images * runs.dc_chunks;
-                    dc_done = true;
-                }
+                if (last && refine && !dc_done) nb += carry_dc(runs, (rec->dc_refine_chunks + 1) / 2);      // about five MCUs a thread (waves without AC refinements are compiled without this)
                 if (roi && refine) entropy_kernel<true, true><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
                 else if (roi) entropy_kernel<true, false><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
                 else if (refine) entropy_kernel<false, true><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
@@ -1394,25 +1420,38 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
                 ++g_launches;
                 runs.n = 0; count = 0;
             };
-            auto add_run = [&](uint32_t first, uint32_t n) {
+            auto launch_refinements = [&](bool last) {
+                if (!ref_count) return;
+                unsigned nb = ref_count;
+                refs.item_blocks = nb;
+                if (last && !dc_done) nb += carry_dc(refs, (rec->dc_refine_chunks + 1) / 2);      // about two MCUs a thread
+                if (roi) refine_kernel<true><<<nb, 32 * kRefineWarps, kRefineBytes, q>>>(P, refs);
+                else refine_kernel<false><<<nb, 32 * kRefineWarps, kRefineBytes, q>>>(P, refs);
+                ++g_launches;
+                refs.n = 0; ref_count = 0;
+            };
+            const bool ctas = refine_in_ctas(rec, waves[w], paired, k0, k);
+            auto add_run = [&](bool to_ctas, uint32_t first, uint32_t n) {
                 if (!n) return;
-                count += n;
-                if (runs.n && runs.first[runs.n - 1] + (runs.end[runs.n - 1] - (runs.n > 1 ? runs.end[runs.n - 2] : 0u)) == first) { runs.end[runs.n - 1] = count; return; }
-                runs.first[runs.n] = first; runs.end[runs.n] = count;
-                ++runs.n;
+                ItemRuns& to = to_ctas ? refs : runs;
+                uint32_t& n_to = to_ctas ? ref_count : count;
+                if (to.n == kMaxRuns) { if (to_ctas) launch_refinements(false); else launch_items(false); }
+                n_to += n;
+                if (to.n && to.first[to.n - 1] + (to.end[to.n - 1] - (to.n > 1 ? to.end[to.n - 2] : 0u)) == first) { to.end[to.n - 1] = n_to; return; }
+                to.first[to.n] = first; to.end[to.n] = n_to;
+                ++to.n;
             };
             std::vector<char> in_pair(rec->G, 0);
             for (int s : waves[w]) {
                 if (s < k0 || s >= k) continue;
-                refine = refine || (rec->script[s].Ss > 0 && rec->script[s].Ah != 0);
+                refine = refine || (!ctas && rec->script[s].Ss > 0 && rec->script[s].Ah != 0);
                 if (!paired || rec->pair_of[s] < k0) continue;
                 in_pair[s] = in_pair[rec->pair_of[s]] = 1;
-                if (!sequential) add_run(rec->pair_begin[(size_t)g * G + s], rec->pair_count[(size_t)g * G + s]);
+                if (!sequential) add_run(ctas, rec->pair_begin[(size_t)g * G + s], rec->pair_count[(size_t)g * G + s]);
             }
             for (int s : waves[w]) {
                 if (s < k0 || s >= k || in_pair[s]) continue;
-                if (runs.n == kMaxRuns && !sequential) launch_items(false);
-                add_run(rec->item_begin[(size_t)g * G + s], rec->item_count[(size_t)g * G + s]);
+                add_run(ctas && rec->script[s].Ss > 0 && rec->script[s].Ah != 0, rec->item_begin[(size_t)g * G + s], rec->item_count[(size_t)g * G + s]);
             }
             const uint32_t begin = runs.n ? runs.first[0] : 0u;
             if (sequential) {
@@ -1429,6 +1468,7 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
                 }
                 return true;
             }
+            launch_refinements(true);
             launch_items(true);
             // scans that are one long restart interval: the first passes of the wave (a contiguous run
             // of the list) ...
@@ -1449,7 +1489,7 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
             // ... (their AC refinements follow in one launch for the whole record, once every slice
             // has finished its waves) and the DC refinement scans that the interval kernel did not take
             for (int j = 0; j < dc_n && !dc_done; ++j) {
-                const int s = runs.dc_s[j];
+                const int s = dc_s[j];
                 for (uint32_t p0 = i0; p0 < i1; p0 += 65535u) {
                     dc_refine_kernel<<<dim3(rec->dc_refine_chunks, std::min(i1 - p0, 65535u)), 256, 0, q>>>(P, s, p0);
                     ++g_launches;
