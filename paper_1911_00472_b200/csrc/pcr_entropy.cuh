@@ -1,5 +1,5 @@
 // Entropy stage of the PCR decoder: restart-interval index with the symbol tables, and the Huffman decode of
-// one wave of scans (progressive) or of the one scan of a baseline image.
+// one wave of scans.  (Baseline images: pcr_sequential.cuh.)
 //
 // Parallel decomposition: one LANE per restart interval.  A warp takes up to 32 consecutive
 // restart intervals of one (scan, image) pair, so its lanes share the scan's Huffman tables
@@ -47,8 +47,9 @@ struct ScanList { int32_t n; int32_t s[64]; };      // the scans one launch cove
 //   bits 0..4   bits to skip: the code plus its extra bits (magnitude, sign, or run length)
 //   AC refinement: bit 5 a new coefficient, bits 8..14 run of zeros, or 64 + run-length exponent for an end
 //               of band (as a run it passes over every position there can be)
+//   sequential scans: bits 5..8 magnitude size, bits 9..13 positions that the symbol moves on by (DC: 1), bit 15 end of block
 //   otherwise:  bits 5..8 magnitude size, bits 9..12 run of zeros (an end of band: its run-length exponent),
-//               bit 13 end of band
+//               bit 15 end of band (as a part of the run it goes beyond every position)
 // 0 = a code longer than kTabBits bits, or no valid symbol of this kind of scan.
 // ---------------------------------------------------------------------------------------
 constexpr int kTabBits = 10;
@@ -59,13 +60,18 @@ struct __align__(16) ScanTab {
     uint8_t vals[256];
 };
 static_assert(sizeof(ScanTab) % 16 == 0, "tables are copied as 16-byte vectors");
-enum { kTabDc = 0, kTabAcFirst = 1, kTabAcRefine = 2, kTabAcSeq = 3 };
-constexpr uint32_t kEntEob = 0x2000u;         // first passes and sequential scans
+enum { kTabDc = 0, kTabAcFirst = 1, kTabAcRefine = 2, kTabAcSeq = 3, kTabDcSeq = 4 };
+constexpr uint32_t kEntEob = 0x8000u;         // first passes and sequential scans
 constexpr uint32_t kEntEobRefine = 0x4000u;   // end of band of one block in a refinement
 
 __device__ __forceinline__ uint32_t sym_entry(int kind, uint32_t len, uint32_t sym) {
     const uint32_t r = (sym >> 4) & 15u, sz = sym & 15u;
     if (kind == kTabDc) return sym > 15u ? 0u : ((len + sz) | (sz << 5));
+    if (kind == kTabDcSeq) return sym > 15u ? 0u : ((len + sz) | (sz << 5) | (1u << 9));
+    if (kind == kTabAcSeq) {
+        if (!sz && r && r != 15u) return 0u;
+        return (len + sz) | (sz << 5) | ((r + 1u) << 9) | (sz || r ? 0u : kEntEob);
+    }
     if (kind == kTabAcRefine) {
         if (sz > 1u) return 0u;
         if (sz || r == 15u) return (len + sz) | (sz << 5) | (r << 8);
@@ -73,7 +79,6 @@ __device__ __forceinline__ uint32_t sym_entry(int kind, uint32_t len, uint32_t s
     }
     if (sz) return (len + sz) | (sz << 5) | (r << 9);
     if (r == 15u) return len | (15u << 9);
-    if (kind == kTabAcSeq && r) return 0u;
     return (len + r) | (r << 9) | kEntEob;
 }
 
@@ -133,7 +138,7 @@ __device__ __forceinline__ void tables_warp(const Params& P, const ScanList& sl,
     const bool seq = sc.Ss == 0 && sc.Se == 63;
     const uint32_t off = seq && slot >= 2 ? sd.tab_ac[slot - 2] : sd.tab_off[slot];
     if (!off) return;
-    const int kind = seq ? (slot < 2 ? kTabDc : kTabAcSeq) : (sc.Ss == 0 ? kTabDc : (sc.Ah == 0 ? kTabAcFirst : kTabAcRefine));
+    const int kind = seq ? (slot < 2 ? kTabDcSeq : kTabAcSeq) : (sc.Ss == 0 ? kTabDc : (sc.Ah == 0 ? kTabAcFirst : kTabAcRefine));
     build_scan_tab(P.tabs + ax.tab0 + (uint32_t)img * (uint32_t)ax.ntab + (uint32_t)slot, P.rec + off, kind, lane, s_code, s_vals);
 }
 
@@ -336,7 +341,7 @@ __device__ __forceinline__ uint64_t low_mask(int p) { return p >= 64 ? ~0ull : (
 // ---------------------------------------------------------------------------------------
 // Bit reader of the interval kernels.  The position is one number: bits counted from the first bit of a
 // 16-byte group of the unstuffed copy.  The words around it lie in the lane's column of a ring in shared
-// memory (one row more than the ring: it repeats row 0; kAgain rows), so the window of the next 32 bits is two shared
+// memory (one row more than the ring: it repeats row 0), so the window of the next 32 bits is two shared
 // loads and a funnel shift, and skipping is an addition: no buffer, no refill branch.  All lanes top their
 // columns up together.  `stop` is the first position at which a step may not begin (the ring runs out, the
 // interval has ended, the lane has nothing to do): one comparison per step.
@@ -349,6 +354,10 @@ __device__ __forceinline__ uint32_t lds8(uint32_t a) { uint32_t v; asm volatile(
 __device__ __forceinline__ void sts16_if(bool on, uint32_t a, uint32_t v) {
     asm volatile("{ .reg .pred p; setp.ne.u32 p, %2, 0; @p st.shared.u16 [%0], %1; }" : : "r"(a), "h"((uint16_t)v), "r"((uint32_t)on) : "memory");
 }
+__device__ __forceinline__ void sts32_if(bool on, uint32_t a, uint32_t v) {
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %2, 0; @p st.shared.u32 [%0], %1; }" : : "r"(a), "r"(v), "r"((uint32_t)on) : "memory");
+}
+__device__ __forceinline__ uint2 lds64(uint32_t a) { uint2 v; asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a) : "memory"); return v; }
 __device__ __forceinline__ uint4 lds128(uint32_t a) { uint4 v; asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory"); return v; }
 __device__ __forceinline__ void sts32(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" : : "r"(a), "r"(v) : "memory"); }
 __device__ __forceinline__ void sts16(uint32_t a, uint32_t v) { asm volatile("st.shared.u16 [%0], %1;" : : "r"(a), "h"((uint16_t)v) : "memory"); }
@@ -366,7 +375,6 @@ template <class T> __device__ __forceinline__ void pin(T*& p) {
     p = static_cast<T*>(__cvta_global_to_generic(a));
 }
 
-template <uint32_t kWords = (uint32_t)kRingWords, uint32_t kAgain = 1>
 struct LaneBits {
     uint32_t col;          // shared address of this lane's column: row r at col + 128 r
     const uint4* g4;       // the 16-byte group that position 0 lies in
@@ -382,9 +390,9 @@ struct LaneBits {
         request();
     }
     __device__ __forceinline__ void put(uint32_t w, const uint4& v) {
-        const uint32_t p = col + (w & (kWords - 1)) * 128u;
+        const uint32_t p = col + (w & (kRingWords - 1)) * 128u;
         sts32(p, v.x); sts32(p + 128u, v.y); sts32(p + 256u, v.z); sts32(p + 384u, v.w);
-        if ((w & (kWords - 1)) == 0) { sts32(p + kWords * 128u, v.x); if (kAgain > 1) sts32(p + kWords * 128u + 128u, v.y); }
+        if ((w & (kRingWords - 1)) == 0) sts32(p + kRingWords * 128u, v.x);
     }
     // Top-up (all lanes of the warp together): what the next one will store first is requested right after
     // the previous one, so that its latency passes beside the decode steps.
@@ -394,14 +402,7 @@ struct LaneBits {
         va = __ldg(g); vb = __ldg(g + 1);
     }
     __device__ __forceinline__ void topup(bool on) {
-        take(on, on ? (kWords - (wr - (pos >> 5))) >> 2 : 0u);
-    }
-    // ... where the words from bit `keep` on are still needed and the ring holds more than one top-up brings; nothing is
-    // read far beyond the interval
-    __device__ __forceinline__ void topup_from(bool on, uint32_t keep) {
-        take(on, on && wr < (limit >> 5) + 8u ? min((kWords - (wr - (keep >> 5))) >> 2, 4u) : 0u);
-    }
-    __device__ __forceinline__ void take(bool on, uint32_t room) {
+        const uint32_t room = on ? (kRingWords - (wr - (pos >> 5))) >> 2 : 0u;
         if (room > 0) put(wr, va);
         if (room > 1) put(wr + 4, vb);
         if (room > 2) put(wr + 8, __ldg(g4 + (wr >> 2) + 2));
@@ -412,10 +413,67 @@ struct LaneBits {
     // steps may begin below this position: `words` words from the one the position lies in are in the ring
     __device__ __forceinline__ uint32_t ring_stop(uint32_t words) const { return 32u * (wr - min(wr, words - 1u)); }
     __device__ __forceinline__ uint32_t window(uint32_t at) const {
-        const uint32_t p = col + ((at << 2) & ((kWords - 1) * 128u));
+        const uint32_t p = col + ((at << 2) & ((kRingWords - 1) * 128u));
         return __funnelshift_l(lds32(p + 128u), lds32(p), at);    // (shift taken mod 32)
     }
 };
+
+// The same for the kernels whose CTAs follow 32 intervals at a time (pcr_refine.cuh, pcr_sequential.cuh): one warp reads along
+// the columns while another fills them, for the round after; the ring is larger because the blocks of the round before
+// are still read.  Two rows more than the ring repeat rows 0 and 1.
+template <uint32_t kWords>
+struct LaneRing {
+    uint32_t col;          // shared address of this lane's column: row r at col + 128 r
+    const uint4* g4;       // the 16-byte group that position 0 lies in
+    uint32_t wr, last;     // next word to fetch (a multiple of 4); words from this one on are not needed
+    uint4 v[4];
+    uint32_t room;
+
+    __device__ __forceinline__ void init(uint32_t column, const uint8_t* ubuf, uint32_t bstart, uint32_t bend) {
+        col = column;
+        g4 = reinterpret_cast<const uint4*>(ubuf) + (bstart >> 4);
+        wr = 0;
+        // (a step that begins at the end of the interval looks at four words; nothing is read far beyond)
+        last = bend > bstart ? (8u * (bstart & 15u) + 8u * (bend - bstart)) / 32u + 8u : 0u;
+    }
+    // up to sixteen words are requested; those from bit `keep` on are still read
+    __device__ __forceinline__ void request(uint32_t keep) {
+        room = wr < last ? min((kWords - (wr - (keep >> 5))) >> 2, 4u) : 0u;
+#pragma unroll
+        for (uint32_t i = 0; i < 4; ++i)
+            if (i < room) v[i] = __ldg(g4 + (wr >> 2) + i);
+    }
+    __device__ __forceinline__ void put() {
+#pragma unroll
+        for (uint32_t i = 0; i < 4; ++i) {
+            if (i >= room) continue;
+            const uint32_t w = (wr + 4u * i) & (kWords - 1), p = col + w * 128u;
+            sts32(p, v[i].x); sts32(p + 128u, v[i].y); sts32(p + 256u, v[i].z); sts32(p + 384u, v[i].w);
+            if (w == 0) { sts32(p + kWords * 128u, v[i].x); sts32(p + kWords * 128u + 128u, v[i].y); }
+        }
+        wr += 4u * room;
+    }
+};
+// A position in such a column: the words it lies in and the one behind them, requested ahead of their use.
+template <uint32_t kWords>
+struct RingWords {
+    uint32_t col, wa, wb, wc;
+    __device__ __forceinline__ void load(uint32_t pos) {
+        const uint32_t p = col + ((pos << 2) & ((kWords - 1) * 128u));
+        wa = lds32(p); wb = lds32(p + 128u); wc = lds32(p + 256u);
+    }
+    __device__ __forceinline__ void load_behind(uint32_t pos) {
+        const uint32_t p = col + ((pos << 2) & ((kWords - 1) * 128u));
+        wb = lds32(p + 128u); wc = lds32(p + 256u);
+    }
+    __device__ __forceinline__ uint32_t window(uint32_t pos) const { return __funnelshift_l(wb, wa, pos); }     // its 32 bits (shifts taken mod 32)
+    __device__ __forceinline__ uint32_t behind(uint32_t pos) const { return __funnelshift_l(wc, wb, pos); }     // the 32 after them
+};
+// Where the roles of a CTA's warps meet, each in a loop of its own (one loop with branches keeps every role's registers
+// alive in all of them).
+__device__ __forceinline__ void meet() { __syncwarp(); asm volatile("bar.sync 0;" : : : "memory"); }
+// entry of a table for the code at the front of a window
+__device__ __forceinline__ uint32_t tab_entry(uint32_t tab, uint32_t win) { return lds16(tab + ((win >> (31 - kTabBits)) & ((2u << kTabBits) - 2u))); }
 
 // The signed value of the sz-bit magnitude field that ends bit `skip` of the window.
 __device__ __forceinline__ int magnitude(uint32_t win, uint32_t skip, uint32_t sz) {
@@ -621,7 +679,7 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, I
         bad = true; done = true;
     }
     if (done) { bstart = sd.data_off; bend = sd.data_off; }
-    LaneBits<> br;
+    LaneBits br;
     br.init(mem + kWarpRing + 4u * lane, P.ubuf, bstart, bend);
     const int Al = sc.Al;
     if (m0 >= m1) done = true;
@@ -886,147 +944,6 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, I
                 done = done || bad || m >= m1;
             }
         }
-    }
-    if (bad) atomicMin(&P.status[img], kErrCorrupt);
-}
-
-// ---------------------------------------------------------------------------------------
-// Sequential (baseline) scans: one interleaved scan carries, block after block, the DC difference
-// and then the AC coefficients up to an end-of-block symbol.  Same decomposition as above (one
-// lane per restart interval, one Huffman symbol per step), four tables per warp (DC and AC,
-// luminance and chrominance).  Lanes stand at different kinds of symbol in every step, so a block's first
-// symbol goes through the same instructions as the others (its entry has no run, its value is the
-// difference), stores are predicated, and what changes from block to block comes from a small table
-// in shared memory.  Coefficients go where the progressive first passes put them.
-// Bound by the length of a lane's chain (a row of 31 MCUs has about 2200 symbols; 28 % of the issue slots are used).  1024
-// ImageNet-shaped images: 1294 us with a branch per kind of symbol, 676 us now.
-// ---------------------------------------------------------------------------------------
-constexpr int kSeqWarps = 2;
-constexpr uint32_t kSeqRing = 4 * sizeof(ScanTab), kSeqPlaces = kSeqRing + (kRingWords + 1) * 128, kSeqPreds = kSeqPlaces + 8 * 16;
-constexpr uint32_t kSeqWarpBytes = kSeqPreds + 3 * 128;
-
-template <bool kRoi>
-__global__ void __launch_bounds__(32 * kSeqWarps) sequential_kernel(Params P, uint32_t item_begin, uint32_t item_count) {
-    __shared__ __align__(16) uint8_t s_seq[kSeqWarps * kSeqWarpBytes];
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t it = blockIdx.x * kSeqWarps + wid;
-    if (it >= item_count) return;                             // whole warp
-    const Item item = P.items[item_begin + it];
-    const ScanDesc sd = P.scans[item.si];
-    const int img = (int)(item.si % (uint32_t)P.N);
-    const ScanAux ax = P.saux[item.si / (uint32_t)P.N];
-    bool done = (uint32_t)lane >= item.count;
-    uint32_t seg = item.seg0 + lane;
-    if (seg >= sd.nseg) { done = true; seg = 0; }
-    const ImgDesc im = P.imgs[img];
-    const uint32_t mcu_w = im.mx, total = im.mx * im.my;
-    const uint32_t m0 = sd.ri ? seg * sd.ri : 0;
-    const uint32_t m1 = sd.ri ? min(m0 + sd.ri, total) : total;
-    const unsigned full = 0xffffffffu;
-    if (kRoi) {
-        if (!done && m1 > m0) {
-            const CropRect rc = P.roi[img];
-            const uint32_t mh = 8u * (uint32_t)P.vs;                       // pixel rows of an MCU row
-            const uint32_t lo = mh * (rc.y0 / mh), hi = mh * ((rc.y0 + rc.h + mh - 1u) / mh);
-            const uint32_t r0 = m0 / mcu_w, r1 = (m1 - 1u) / mcu_w;
-            if ((r1 + 1u) * mh <= lo || r0 * mh >= hi) done = true;
-        }
-        if (__all_sync(full, done)) return;
-    }
-    const uint32_t mem = (uint32_t)__cvta_generic_to_shared(s_seq) + (uint32_t)wid * kSeqWarpBytes;
-    const uint32_t hs = (uint32_t)P.hs, vs = (uint32_t)P.vs, bw0 = hs * mcu_w;
-    const uint32_t ny = hs * vs, bpm = P.nc == 3 ? ny + 2u : 1u;      // blocks per MCU (a lone component: one block, no padding)
-    {
-        const uint4* a = reinterpret_cast<const uint4*>(P.tabs + ax.tab0 + 4u * (uint32_t)img);
-        for (int i = lane; i < (int)(4 * sizeof(ScanTab) / 16); i += 32) sts128(mem + 16 * i, __ldg(a + i));
-        // per block of the MCU: its two tables (shared addresses), where its predictor lies, its block number
-        // relative to the MCU's first luminance block or to the MCU's chroma place (bit 31)
-        if ((uint32_t)lane < bpm) {
-            const uint32_t j = (uint32_t)lane, c = j < ny ? 0u : j - ny + 1u;
-            const uint32_t tdc = mem + ((sd.slots >> (2u * c)) & 1u) * (uint32_t)sizeof(ScanTab);
-            const uint32_t tac = mem + (2u + ((sd.slots_ac >> (2u * c)) & 1u)) * (uint32_t)sizeof(ScanTab);
-            const uint32_t off = c ? (ny * total + (c - 1u) * total) | 0x80000000u : (j >> (hs - 1u)) * bw0 + (j & (hs - 1u));
-            sts128(mem + kSeqPlaces + 16u * j, make_uint4(tdc, tac, mem + kSeqPreds + 128u * c, off));
-        }
-#pragma unroll
-        for (int c = 0; c < 3; ++c) sts32(mem + kSeqPreds + 128u * c + 4u * lane, 0u);
-    }
-    const uint32_t* segtab = P.seg_start + sd.seg_base;
-    uint32_t bstart = segtab[seg];
-    uint32_t bend = segtab[seg + 1] - 2;
-    bool bad = false;
-    if (!done && (bstart < sd.data_off || bend > sd.data_end || bend < bstart)) { bad = true; done = true; }
-    if (done) { bstart = sd.data_off; bend = sd.data_off; }
-    LaneBits<> br;
-    br.init(mem + kSeqRing + 4u * lane, P.ubuf, bstart, bend);
-    if (m0 >= m1) done = true;
-
-    uint32_t m = m0, wrap_m = (m0 / mcu_w + 1u) * mcu_w;       // MCU, the first one of the next row
-    uint32_t my = (m0 / mcu_w) * vs * bw0 + hs * (m0 % mcu_w); // block number of the MCU's first luminance block (its chroma place is m)
-    const uint32_t my_wrap = (vs - 1u) * bw0;                  // what a new row adds beside hs per MCU
-    uint32_t place = mem + kSeqPlaces;                         // of the current block in the table
-    const uint32_t place_end = place + 16u * bpm;
-    uint32_t k = 0, M0 = 0, M1 = 0;                            // position (0: the block's DC symbol comes next), mask
-    int16_t* vp = P.vals + 4ull * bstart;                      // next value
-    int16_t* vb = vp;                                          // the block's first one
-    int16_t* dcp = P.dc + im.blk_base;
-    int16_t* headp = P.head + im.blk_base * 8;
-    uint64_t* auxp = P.aux + ax.base + im.blk_base * 2;
-    pin(dcp); pin(headp); pin(auxp);
-    uint32_t tdc = 0, tac = 0, pred = 0, blk = 0;
-    auto take = [&]() {
-        const uint4 v = lds128(place);
-        tdc = v.x; tac = v.y; pred = v.z + 4u * lane;
-        blk = (v.w & 0x7FFFFFFFu) + ((v.w >> 31) ? m : my);
-    };
-    bool fresh = true;
-    for (;;) {
-        br.topup(!done);
-        __syncwarp(full);
-        if (__all_sync(full, done)) break;
-        if (fresh) { take(); fresh = false; }
-        uint32_t stop = done ? 0u : min(br.ring_stop(2), br.limit + 1u);
-#pragma unroll 1
-        for (int t = 0; t < kDecodeSteps; ++t) {
-            if (br.pos < stop) {
-                const uint32_t win = br.window(br.pos);
-                const bool is_dc = k == 0;
-                const uint32_t tab = is_dc ? tdc : tac;
-                uint32_t e = lds16(tab + ((win >> (32 - kTabBits)) << 1));
-                if (e == 0) {
-                    e = long_code(tab, win, is_dc ? kTabDc : kTabAcSeq);
-                    if (e == 0) { bad = true; stop = 0; }
-                }
-                const uint32_t skip = e & 31u, sz = (e >> 5) & 15u;
-                br.pos += skip;
-                k += (e >> 9) & 15u;
-                int v = magnitude(win, skip, sz);
-                if (is_dc) { v += (int)lds32(pred); sts32(pred, (uint32_t)v); }
-                const bool coef = sz && k <= 63u, far = coef && k >= 8u;
-                if (is_dc) dcp[blk] = (int16_t)v;                          // (stored even if there was no such symbol: the image is corrupt then)
-                if (coef && !far && !is_dc) headp[8u * (uint64_t)blk + k] = (int16_t)v;
-                if (far) *vp = (int16_t)v;
-                vp += far ? 1 : 0;
-                M0 |= shl0(far ? 1u : 0u, k); M1 |= shl0(far ? 1u : 0u, k - 32u);
-                if (sz && k > 63u) { bad = true; stop = 0; }
-                ++k;
-                if ((e & kEntEob) || k > 63u) {                            // block finished
-                    if (M0 | M1) *reinterpret_cast<uint4*>(auxp + 2ull * blk) = value_record(M0, M1, vb);
-                    k = 0; M0 = 0; M1 = 0; vb = vp;
-                    place += 16u;
-                    if (place == place_end) {
-                        place = mem + kSeqPlaces;
-                        ++m; my += hs;
-                        if (m == wrap_m) { wrap_m += mcu_w; my += my_wrap; }
-                        if (m >= m1) stop = 0;
-                    }
-                    take();
-                }
-            }
-        }
-        __syncwarp(full);
-        bad = bad || br.pos > br.limit;
-        done = done || bad || m >= m1;
     }
     if (bad) atomicMin(&P.status[img], kErrCorrupt);
 }

@@ -28,6 +28,7 @@
 #include "pcr_msssim.cuh"
 #include "pcr_pixels.cuh"
 #include "pcr_refine.cuh"
+#include "pcr_sequential.cuh"
 #include "pcr_types.h"
 
 using namespace pcr;
@@ -1456,8 +1457,8 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
             const uint32_t begin = runs.n ? runs.first[0] : 0u;
             if (sequential) {
                 if (count) {
-                    if (roi) sequential_kernel<true><<<(count + kSeqWarps - 1) / kSeqWarps, 32 * kSeqWarps, 0, q>>>(P, begin, count);
-                    else sequential_kernel<false><<<(count + kSeqWarps - 1) / kSeqWarps, 32 * kSeqWarps, 0, q>>>(P, begin, count);
+                    if (roi) sequential_kernel<true><<<count, 32 * kSeqWarps, 0, q>>>(P, begin);
+                    else sequential_kernel<false><<<count, 32 * kSeqWarps, 0, q>>>(P, begin);
                     ++g_launches;
                 }
                 const int s0 = waves[w][0];      // the record's one scan

@@ -103,10 +103,10 @@ struct SeqSteps {
     __device__ __forceinline__ uint32_t entry(uint32_t pos, uint32_t st) const {
         const uint32_t j = st >> 6;
         const bool dc = (st & 63u) == 0;
-        return long_entry(tabs + (dc ? (tdc >> j) & 1u : 2u + ((tac >> j) & 1u)) * (uint32_t)sizeof(ScanTab), long_window(base, pos), dc ? kTabDc : kTabAcSeq);
+        return long_entry(tabs + (dc ? (tdc >> j) & 1u : 2u + ((tac >> j) & 1u)) * (uint32_t)sizeof(ScanTab), long_window(base, pos), dc ? kTabDcSeq : kTabAcSeq);
     }
     __device__ __forceinline__ bool advance(uint32_t e, uint32_t& st) const {
-        const uint32_t k = (st & 63u) + ((e >> 9) & 15u) + 1u, j = st >> 6;
+        const uint32_t k = (st & 63u) + ((e >> 9) & 31u), j = st >> 6;
         const bool end = (e & kEntEob) || k > 63u;
         st = end ? (j + 1u == bpm ? 0u : j + 1u) << 6 : (st & ~63u) + k;
         return end;
@@ -478,7 +478,7 @@ __global__ void __launch_bounds__(32 * kSeqLongWarps) sequential_long_kernel(Par
         const uint32_t blk = j < ny ? yb + (j >> (hs - 1u)) * g.bw[0] + (j & (hs - 1u)) : (ny + j - ny) * total + m;
         p += skip;
         const bool is_dc = k == 0;
-        k += (e >> 9) & 15u;
+        k += ((e >> 9) & 31u) - 1u;
         if (e == 0 || (sz && k > 63u)) { bad = true; break; }
         int v = magnitude(win, skip, sz);
         if (is_dc) {

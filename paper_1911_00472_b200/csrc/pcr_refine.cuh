@@ -14,9 +14,10 @@
 //
 // Bound by the latency of warp 0's step, 166 cycles a symbol alone on an SM and 200 to 220 beside other CTAs (entropy_kernel's, which
 // does all of it in the lane: 700).  What it took: nothing but the chain in the step; one straight line instead of branches
-// for block ends and rare cases (350 -> 175); the next symbol's entry requested before anything else that is loaded (-> 166).
+// for block ends and rare cases (350 -> 175); the next symbol's entry requested before anything else that is loaded (-> 166);
+// the rings filled by a helper.
 // Rounds of 16, 32, 48 and 64 symbols: 233, 177, 157 and 164 k cycles for the busiest CTA of 4 ImageNet-shaped images, whose
-// refinement wave took 211 us and takes 85.  1024 such images are better off with entropy_kernel: see refine_in_ctas.
+// refinement wave took 211 us and takes 84.  1024 such images are better off with entropy_kernel: see refine_in_ctas.
 //
 // Side data of a block: {mask of the band's non-zero positions after the scan, correction bits in reading order (the last
 // one in bit 0), newly non-zero positions, the positive ones among them}; the pixel kernel applies them.
@@ -42,7 +43,7 @@ struct RefineShared {
     struct { ScanTab t; uint8_t pad[4096 - sizeof(ScanTab)]; } tabs[2];
     uint8_t zpos[64][kRefineLists][32];       // [i][slot][lane]: position of the block's i-th still-zero coefficient of the band, minus
                                               // i; entry nz: Se + 1 - nz (as if position Se + 1 followed)
-    uint32_t ring[(kRefineRing + 2) * 32];    // see LaneBits
+    uint32_t ring[(kRefineRing + 2) * 32];    // see LaneRing
     uint64_t mask[kRefineLists][32];          // positions of the band that are non-zero before the scan
     uint32_t ends[kRefineLists][32];          // 256 nz + 255, nz = how many still-zero positions there are (at most 63), and, from
                                               // bit 16 on, 256 times the rank that ends the block (nz, or nz - 1 if the last of them is Se)
@@ -51,9 +52,12 @@ struct RefineShared {
     // of the lane's interval: masks of up to four earlier scans (null: none) and their words a block, a byte each;
     // side data of the scan, the first block's row (as a block index) and column, blocks a row in the scan and in the planes
     uint64_t src[4][32], out[32];
+    uint32_t range[2][32];                    // ... its bytes
     uint32_t stride[32], row0[32], col0[32], width[32], pitch[32], tab[32];
-    // by parity of the round: the blocks whose side data, and those whose lists are to be made: first and number
+    // By parity of the round: the blocks whose side data, and those whose lists are to be made: first and number
     uint32_t side_first[2][32], side_count[2][32], list_first[2][32], list_count[2][32], more[2];
+    // ... the first bit that is still read, and how far the ring is filled
+    uint32_t keep[2][32], filled[2][32];
 };
 static_assert(offsetof(RefineShared, tabs) == 0 && offsetof(RefineShared, zpos) % 512 == 0 && offsetof(RefineShared, ring) % 16 == 0, "see kRefineAlign");
 static_assert(32 * kRefineRing <= kEntEobRefine, "positions modulo the ring fit below the flag");
@@ -107,19 +111,8 @@ __device__ __forceinline__ void refine_list(RefineShared& sh, uint32_t lane, uin
     sh.ends[slot][lane] = (256u * n + 255u) | ((256u * ((z >> Se) & 1u ? n - 1u : n)) << 16);
 }
 
-// A symbol's place in the chain: the window, the entry, the target's list entry.  Shared by the chains and by the side data.
-struct RefineWords {
-    uint32_t col;                                              // shared address of the lane's column of the ring
-    uint32_t win, wa, wb, wc;                                  // the 32 bits at the position; the words it lies in, and behind it
-    __device__ __forceinline__ void words(uint32_t pos) {
-        const uint32_t p = col + ((pos << 2) & ((kRefineRing - 1) * 128u));
-        wa = lds32(p); wb = lds32(p + 128u); wc = lds32(p + 256u);
-    }
-    __device__ __forceinline__ void init(uint32_t pos) { words(pos); win = __funnelshift_l(wb, wa, pos); }
-    // the 32 bits behind the window (shift taken mod 32); a window from scratch
-    __device__ __forceinline__ uint32_t behind(uint32_t pos) const { return __funnelshift_l(wc, wb, pos); }
-    __device__ __forceinline__ uint32_t fresh(uint32_t pos) const { return __funnelshift_l(wb, wa, pos); }
-};
+using RefineWords = RingWords<kRefineRing>;
+// (a table's place and an index are put together by an OR)
 __device__ __forceinline__ uint32_t refine_entry(uint32_t tab, uint32_t win) {
     return lds16(tab | ((win >> (31 - kTabBits)) & ((2u << kTabBits) - 2u)));
 }
@@ -135,32 +128,33 @@ __device__ __forceinline__ void refine_side(RefineShared& sh, uint32_t lane, uin
     W.col = (uint32_t)__cvta_generic_to_shared(sh.ring) + 4u * lane;
     uint32_t at = st & (kEntEobRefine - 1u), zi = 0, ep = Ss, t;
     uint32_t s0 = 0, s1 = 0, N0 = 0, N1 = 0, G0 = 0, G1 = 0;   // correction bits, new positions, positive ones
-    W.init(at);
+    W.load(at);
+    uint32_t win = W.window(at);
 #pragma unroll 1
     do {
-        uint32_t e = refine_entry(tab, W.win);
+        uint32_t e = refine_entry(tab, win);
         const uint32_t behind = W.behind(at);
         e = st & kEntEobRefine ? kEntEobRefine : e;            // the whole block lies inside an end-of-band run
-        if (e == 0) e = long_code(tab, W.win, kTabAcRefine);   // (there is one: the chain has passed it)
+        if (e == 0) e = long_code(tab, win, kTabAcRefine);   // (there is one: the chain has passed it)
         t = min(zi + (e & kEntRunSkip), nz);                   // 256 times the target's rank, and eight other bits
         const uint32_t e2 = lds8(zb + 2u * (t & 0x3F00u)), skip = e & 31u, n = e2 - ep, k = e2 + (t >> 8);
-        const uint32_t isnew = (t | 255u) < nz && (e & kEntNew) ? 1u : 0u, plus = isnew & shr0(W.win, 32u - skip);
+        const uint32_t isnew = (t | 255u) < nz && (e & kEntNew) ? 1u : 0u, plus = isnew & shr0(win, 32u - skip);
         N0 |= shl0(isnew, k); N1 |= shl0(isnew, k - 32u);
         G0 |= shl0(plus, k); G1 |= shl0(plus, k - 32u);
-        const uint32_t corr = __funnelshift_l(behind, W.win, skip);
+        const uint32_t corr = __funnelshift_l(behind, win, skip);
         at += skip + n;
-        W.words(at);
+        W.load(at);
         if (n > 32u) {
             RefineWords V;
             V.col = W.col;
-            V.init(at - n + 32u);
+            V.load(at - n + 32u);
             s1 = shl0(s0, n - 32u) | (corr >> (64u - n));
-            s0 = __funnelshift_l(V.win, corr, n - 32u);
+            s0 = __funnelshift_l(V.window(at - n + 32u), corr, n - 32u);
         } else {
             s1 = __funnelshift_lc(s0, s1, n);
             s0 = shl0(s0, n) | shr0(corr, 32u - n);
         }
-        W.win = skip + n > 31u ? W.fresh(at) : __funnelshift_l(behind, W.win, skip + n);
+        win = skip + n > 31u ? W.window(at) : __funnelshift_l(behind, win, skip + n);
         zi = (t | 255u) + 1u; ep = e2;
     } while (t < tend);
     const uint64_t h = sh.mask[slot][lane];
@@ -252,34 +246,31 @@ __global__ void __launch_bounds__(32 * kRefineWarps, 3) refine_kernel(Params P, 
         for (uint32_t i = tid - 32u; i < (two_images || item.pair ? 2u : 1u) * words; i += 32u * (kRefineWarps - 1))
             sts128(t0 + (i < words ? 16u * i : 4096u + 16u * (i - words)), __ldg(i < words ? a + i : b + (i - words)));
     }
-    // warp 0's lane: block it stands at, lists that are there, lists that have been asked for, blocks handed on
-    uint32_t m = 0, have = 0, asked = half ? 0u : min(n, kRefineLists), handed = 0;
-    bool done = n == 0;
-    LaneBits<kRefineRing, 2> br;
-    uint32_t tab = 0;
+    const uint32_t ring = (uint32_t)__cvta_generic_to_shared(sh.ring) + 4u * lane;
     if (wid == 0) {
+        // the lane's block it stands at, lists that are there, lists that have been asked for, blocks handed on
+        uint32_t m = 0, have = 0, asked = half ? 0u : min(n, kRefineLists), handed = 0;
+        bool done = n == 0;
+        uint32_t pos = 8u * (bstart & 15u);                   // next bit of the lane's chain; the first one behind its interval
+        const uint32_t limit = pos + 8u * (bend - bstart);
+        uint32_t keep = pos, first = pos;                     // first bit of what is handed on next, of block m
+        uint32_t eobrun = 0, zi = 0xFFFFFFFFu, ep = Ss;       // zi: 256 times the still-zero positions passed, minus one
+        bool fresh = true;                                    // block m has not been begun
+        uint32_t idle = 0, trace = 0;                         // rounds in which nothing moved on
         sh.list_first[0][lane] = 0; sh.list_count[0][lane] = asked; sh.side_first[0][lane] = 0; sh.side_count[0][lane] = 0;
+        sh.keep[0][lane] = pos;
+        sh.range[0][lane] = bstart; sh.range[1][lane] = bend;
         const bool any = __any_sync(full, n != 0);
         if (lane == 0) sh.more[0] = any;
-        tab = sh.tab[lane];
-        br.init((uint32_t)__cvta_generic_to_shared(sh.ring) + 4u * lane, P.ubuf, bstart, bend);
-            }
-    uint32_t keep = br.pos, next_keep = br.pos;               // first bit of the blocks handed on last, of what is handed on next
-    uint32_t idle = 0, trace = 0;                             // rounds in which nothing moved on
-    uint32_t eobrun = 0, zi = 0xFFFFFFFFu, ep = Ss;           // zi: 256 times the still-zero positions passed, minus one
-    uint32_t first = br.pos;                                  // first bit of block m
-    bool fresh = true;                                        // ... which has not been begun
-    __syncthreads();
-
-    for (uint32_t round = 0;; ++round) {
-        const uint32_t b = round & 1u, nb = b ^ 1u;
-        if (!sh.more[b]) break;                               // whole CTA
-        if (wid == 0) {
+        const uint32_t tab = sh.tab[lane];
+        meet();
+        for (uint32_t round = 0;; ++round) {
+            const uint32_t b = round & 1u, nb = b ^ 1u;
+            if (!sh.more[b]) break;                           // whole CTA
             // ---- the chains
-            br.topup_from(!done, keep);
-            __syncwarp(full);
             // a step reads the 64 bits from its start on, and a block's side data up to three words behind its last symbol's
-            uint32_t stop = done ? 0u : min(br.ring_stop(4), br.limit + 1u);
+            const uint32_t filled = round ? sh.filled[nb][lane] : 0u;
+            uint32_t stop = done ? 0u : min(32u * (filled - min(filled, 3u)), limit + 1u);
             // A block's slot as the number its list, its ends and its start are addressed by: 32 slot + lane, and the place of the lists
             // (a multiple of 512) above.  The next block's ends are loaded ahead.
             const uint32_t lists = (uint32_t)__cvta_generic_to_shared(sh.zpos), to_ends = (uint32_t)__cvta_generic_to_shared(sh.ends) - 4u * lists;
@@ -288,22 +279,23 @@ __global__ void __launch_bounds__(32 * kRefineWarps, 3) refine_kernel(Params P, 
             uint32_t here = lists + (refine_slot(m) << 5) + lane, next = slot_behind(here);
             uint32_t ends = lds32(to_ends + 4u * here), ends_next = lds32(to_ends + 4u * next);
             RefineWords W;
-            W.col = br.col;
+            W.col = ring;
             if (m >= have) stop = 0;
-            if (fresh && stop) sts16(to_start + 2u * here, (br.pos & (32u * kRefineRing - 1u)) | (eobrun ? kEntEobRefine : 0u));
-            W.init(br.pos);
+            if (fresh && stop) sts16(to_start + 2u * here, (pos & (32u * kRefineRing - 1u)) | (eobrun ? kEntEobRefine : 0u));
+            W.load(pos);
+            uint32_t win = W.window(pos);
             uint32_t only = eobrun ? 0u : kEntRunSkip, force = eobrun ? kEntEobRefine : 0u;   // inside an end-of-band run no symbol is read
             // A step is one straight line: every lane walks it, what does not count is thrown away.  (With block ends and
             // rare cases as branches a step took 340 cycles.)  What is rare (a code longer than the table's index, a step that passed
             // more than 31 bits) makes the lane wait for the end of eight steps.  The chain: win -> e -> t -> e2 -> win.
             bool rare = false;
-            uint32_t raw = refine_entry(tab, W.win);
+            uint32_t raw = refine_entry(tab, win);
 #pragma unroll 1
             for (int s = 0; s < kRefineSteps; s += 8) {
 #pragma unroll 4
                 for (int q = 0; q < 8; ++q) {
-                    const bool wanted = br.pos < stop && !rare;
-                    const uint32_t behind = W.behind(br.pos), e = (raw & only) | force;
+                    const bool wanted = pos < stop && !rare;
+                    const uint32_t behind = W.behind(pos), e = (raw & only) | force;
                     const bool act = wanted && e != 0;
                     rare = rare || (wanted && e == 0);
                     const uint32_t t = min(zi + e + 1u, ends & 0xFFFFu);           // 256 times the target's rank, and eight other bits
@@ -312,15 +304,15 @@ __global__ void __launch_bounds__(32 * kRefineWarps, 3) refine_kernel(Params P, 
                     // the symbol, and a correction bit for every non-zero position passed
                     const uint32_t skip = e & 31u, d = act ? skip - ep + e2 : 0u;
                     // blocks behind this one that an end of band covers, or that are left of a run of them
-                    const uint32_t x = (e >> 8) & 15u, run = __funnelshift_l(shl0(W.win, skip - x), 1u, x);   // (2^x + the x bits that end the symbol)
+                    const uint32_t x = (e >> 8) & 15u, run = __funnelshift_l(shl0(win, skip - x), 1u, x);   // (2^x + the x bits that end the symbol)
                     const uint32_t left = (eobrun ? eobrun : (e >= kEntEobRefine ? run : 1u)) - 1u;
                     eobrun = end ? left : eobrun;
                     only = eobrun ? 0u : kEntRunSkip; force = eobrun ? kEntEobRefine : 0u;
-                    W.win = __funnelshift_l(behind, W.win, d);
-                    raw = refine_entry(tab, W.win);
-                    br.pos += d;
+                    win = __funnelshift_l(behind, win, d);
+                    raw = refine_entry(tab, win);
+                    pos += d;
                     rare = rare || d > 31u;
-                    W.words(br.pos);
+                    W.load_behind(pos);
                     zi = end ? 0xFFFFFFFFu : (act ? t | 255u : zi);
                     ep = end ? Ss : (act ? e2 : ep);
                     m += end ? 1u : 0u;
@@ -329,23 +321,24 @@ __global__ void __launch_bounds__(32 * kRefineWarps, 3) refine_kernel(Params P, 
                     next = slot_behind(here);
                     ends_next = lds32(to_ends + 4u * next);
                     const bool more = m < have;
-                    sts16_if(end && more, to_start + 2u * here, (br.pos & (32u * kRefineRing - 1u)) | force);
+                    sts16_if(end && more, to_start + 2u * here, (pos & (32u * kRefineRing - 1u)) | force);
                     stop = more ? stop : 0u;                   // also at the interval's end: have is at most n
                 }
                 if (rare) {
                     rare = false;
-                    W.init(br.pos);
-                    raw = refine_entry(tab, W.win);
-                    if (raw == 0 && !eobrun && br.pos < stop) {
-                        raw = long_code(tab, W.win, kTabAcRefine);
+                    W.load(pos);
+                    win = W.window(pos);
+                    raw = refine_entry(tab, win);
+                    if (raw == 0 && !eobrun && pos < stop) {
+                        raw = long_code(tab, win, kTabAcRefine);
                         if (raw == 0) { bad = true; stop = 0; }        // no such symbol: the lane ends here
                     }
                 }
-                if (!__any_sync(full, br.pos < stop)) break;
+                if (!__any_sync(full, pos < stop)) break;
             }
             fresh = m >= have;
-            first = fresh ? br.pos : br.pos - ((br.pos - lds16(to_start + 2u * here)) & (32u * kRefineRing - 1u));
-            bad = bad || (!done && br.pos > br.limit);
+            first = fresh ? pos : pos - ((pos - lds16(to_start + 2u * here)) & (32u * kRefineRing - 1u));
+            bad = bad || (!done && pos > limit);
             // ---- what the round left: blocks handed .. m - 1 are finished.  At the meeting the lists asked for so far
             // are there, and the side data of the blocks handed on so far: their slots are free
             const uint32_t pm = __shfl_sync(full, m, (int)li), ph = __shfl_sync(full, handed, (int)li);
@@ -356,32 +349,44 @@ __global__ void __launch_bounds__(32 * kRefineWarps, 3) refine_kernel(Params P, 
             sh.side_first[nb][lane] = handed; sh.side_count[nb][lane] = m - handed;
             sh.list_first[nb][lane] = asked; sh.list_count[nb][lane] = want - asked;
             // (every round in which a lane has work left moves something on; should none do so for some rounds, the lanes give up)
-            const uint32_t moved = br.pos + br.wr + m + have + want + handed + keep + next_keep;
+            const uint32_t moved = pos + filled + m + have + want + handed + keep;
             idle = __any_sync(full, moved != trace) ? 0u : idle + 1u;
             trace = moved;
             if (idle == 8u && !done) bad = done = true;
             const bool more = __any_sync(full, !done || m != handed);
             if (lane == 0) sh.more[nb] = more;
             asked = want; handed = m;
-            keep = next_keep; next_keep = first;
-        } else {
-            // ---- the helpers: the lane's finished blocks one after the other from the first helper on, lists from the last one on
-            constexpr uint32_t helpers = kRefineWarps - 1;
-            const uint32_t h0 = wid - 1u, h1 = helpers - 1u - h0;
-            const uint32_t lists = sh.list_count[b][lane], list0 = sh.list_first[b][lane], sides = sh.side_count[b][lane], side0 = sh.side_first[b][lane];
-            uint64_t h = 0;                                    // (requested before the side data, used behind it)
-            if (h1 < lists) h = refine_masks(sh, lane, list0 + h1);
-#pragma unroll 1
-            for (uint32_t i = h0; i < sides; i += helpers) refine_side(sh, lane, side0 + i, Ss);
-#pragma unroll 1
-            for (uint32_t i = h1; i < lists; i += helpers) {
-                refine_list(sh, lane, refine_slot(list0 + i), h, band, Se);
-                if (i + helpers < lists) h = refine_masks(sh, lane, list0 + i + helpers);
-            }
+            sh.keep[nb][lane] = keep;
+            keep = first;
+            meet();
         }
-        __syncthreads();
+        if (bad) atomicMin(&P.status[img], kErrCorrupt);
+        return;
     }
-    if (wid == 0 && bad) atomicMin(&P.status[img], kErrCorrupt);
+    // the last of the helpers also fills the rings
+    constexpr uint32_t helpers = kRefineWarps - 1, filler = kRefineWarps - 1;
+    const uint32_t h0 = wid - 1u, h1 = helpers - 1u - h0;
+    LaneRing<kRefineRing> fill;
+    meet();
+    if (wid == filler) fill.init(ring, P.ubuf, sh.range[0][lane], sh.range[1][lane]);
+    for (uint32_t round = 0;; ++round) {
+        const uint32_t b = round & 1u;
+        if (!sh.more[b]) break;
+        // ---- the helpers: the lane's finished blocks one after the other from the first helper on, lists from the last one on
+        const uint32_t lists = sh.list_count[b][lane], list0 = sh.list_first[b][lane], sides = sh.side_count[b][lane], side0 = sh.side_first[b][lane];
+        uint64_t h = 0;                                    // (requested before the side data, used behind it)
+        if (wid == filler) fill.request(sh.keep[b][lane]);
+        if (h1 < lists) h = refine_masks(sh, lane, list0 + h1);
+#pragma unroll 1
+        for (uint32_t i = h0; i < sides; i += helpers) refine_side(sh, lane, side0 + i, Ss);
+#pragma unroll 1
+        for (uint32_t i = h1; i < lists; i += helpers) {
+            refine_list(sh, lane, refine_slot(list0 + i), h, band, Se);
+            if (i + helpers < lists) h = refine_masks(sh, lane, list0 + i + helpers);
+        }
+        if (wid == filler) { fill.put(); sh.filled[b][lane] = fill.wr; }
+        meet();
+    }
 }
 
 }  // namespace pcr

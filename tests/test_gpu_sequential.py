@@ -1,0 +1,64 @@
+"""Baseline records with restart intervals, whose CTAs follow 32 intervals' symbols while other warps write the blocks: intervals
+of one MCU to several rows, blocks as long as the format allows and of two symbols, every chroma sampling (the blocks of an
+MCU change tables in different places), an interval that is damaged."""
+from __future__ import annotations
+
+import struct
+
+import numpy as np
+import pytest
+
+import pcr_synth
+from oracle import pcr_oracle as O
+from test_gpu_kernel_edges import _compare, _field
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("samp", [(2, 2, 3), (2, 1, 3), (1, 1, 3), (1, 1, 1)])
+@pytest.mark.parametrize("fixed", [0, 1, 5, 60])
+@pytest.mark.parametrize("kind", ["dense", "usual", "empty"])
+def test_blocks_and_intervals(kind, fixed, samp):
+    """fixed: MCUs an interval (0: a row).  dense: blocks of up to 64 symbols of many bits; empty: two symbols a block, so that a
+    round ends most blocks there can be."""
+    rng = np.random.default_rng(fixed)
+    dims = [(330, 33), (8, 8), (90, 41)]
+    density, top = {"dense": (1.0, 1023), "usual": (0.15, 40), "empty": (0.0, 1)}[kind]
+    with pcr_synth.sampling(*samp), pcr_synth.scan_script(pcr_synth.SCRIPT_BASELINE):
+        coeffs = [_field(rng, pcr_synth.num_blocks(w, h), density, top) for w, h in dims]
+        rec = pcr_synth.record_from_coeffs(dims, coeffs, restart_rows=fixed == 0, restart_fixed=fixed)
+    _compare(rec, (1,))
+
+
+def test_damaged_interval():
+    """The second half of one restart interval of one image replaced by ones (no code is all ones): that image is reported,
+    the others' pixels are the oracle's."""
+    import torch
+    from paper_1911_00472_b200 import Decoder
+    rng = np.random.default_rng(1)
+    dims = [(120, 60), (90, 41), (33, 70)]
+    with pcr_synth.scan_script(pcr_synth.SCRIPT_BASELINE):
+        rec = pcr_synth.record_from_coeffs(dims, [_field(rng, pcr_synth.num_blocks(w, h), 0.3, 20) for w, h in dims])
+    bad = np.array(rec.bytes, copy=True)
+    n, groups = struct.unpack_from("<II", bad, 8)
+    index = struct.unpack_from("<Q", bad, 32)[0] + 8 * (groups + 1)
+    off, length = struct.unpack_from("<QI", bad, index + 16)
+    chunk = bad[off:off + length].tobytes()
+    head = chunk.index(b"\xff\xda")
+    data = head + 2 + struct.unpack_from(">H", chunk, head + 2)[0]
+    first, end = chunk.index(b"\xff\xd0", data) + 2, chunk.index(b"\xff\xd1", data)
+    begin = (first + end) // 2
+    begin += (end - begin) % 2
+    bad[off + begin:off + end] = np.tile(np.array([0xFF, 0], dtype=np.uint8), (end - begin) // 2)
+    dec = Decoder(bad)
+    try:
+        out = dec.decode(1)
+        torch.cuda.synchronize()
+        assert dec.status() == (1, -3)
+        pixels = out.cpu().numpy()
+        for i in (0, 2):
+            want = O.decode_image(rec.bytes, i, 1)[1]
+            inf = dec.info[i]
+            assert np.array_equal(pixels[inf.out_offset:inf.out_offset + inf.out_bytes].reshape(want.shape), want), i
+    finally:
+        dec.close()
