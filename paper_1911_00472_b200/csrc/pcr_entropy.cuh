@@ -18,7 +18,7 @@
 // (AC refinements of records that do not fill the machine: pcr_refine.cuh.)
 // Bound by the latency of a lane's chain: about 155 warp instructions a refinement step (276 with masks searched for
 // the r-th zero and a bit reader that carries its state), at the issue rate that the resident warps allow.
-// 1024 ImageNet-shaped images at k = 10: the three waves 217 + 332 + 511 us before, 200 + 220 + 245 us now.
+// 1024 ImageNet-shaped images at k = 10: the three waves 217 + 332 + 511 us before, 176 + 220 + 245 us now.
 #pragma once
 #include <cuda_runtime.h>
 #include <stddef.h>
@@ -37,6 +37,16 @@ constexpr int kEntropyWarps = PCR_ENTROPY_WARPS;
 
 constexpr int kRingWords = 16;       // words of the bitstream a lane of the interval kernels holds in shared memory
 
+// A table entry as 16-byte loads: what a warp needs of several tables is requested before the first of it is used (a kernel's
+// start is a chain of dependent loads).
+template <class T> __device__ __forceinline__ T load_entry(const T* p) {
+    static_assert(sizeof(T) % 16 == 0 && alignof(T) >= 16, "whole vectors");
+    union U { uint4 v[sizeof(T) / 16]; T t; __device__ U() {} } u;
+#pragma unroll
+    for (size_t i = 0; i < sizeof(T) / 16; ++i) u.v[i] = __ldg(reinterpret_cast<const uint4*>(p) + i);
+    return u.t;
+}
+
 struct ScanList { int32_t n; int32_t s[64]; };      // the scans one launch covers
 
 // ---------------------------------------------------------------------------------------
@@ -47,9 +57,8 @@ struct ScanList { int32_t n; int32_t s[64]; };      // the scans one launch cove
 //   bits 0..4   bits to skip: the code plus its extra bits (magnitude, sign, or run length)
 //   AC refinement: bit 5 a new coefficient, bits 8..14 run of zeros, or 64 + run-length exponent for an end
 //               of band (as a run it passes over every position there can be)
-//   sequential scans: bits 5..8 magnitude size, bits 9..13 positions that the symbol moves on by (DC: 1), bit 15 end of block
-//   otherwise:  bits 5..8 magnitude size, bits 9..12 run of zeros (an end of band: its run-length exponent),
-//               bit 15 end of band (as a part of the run it goes beyond every position)
+//   otherwise:  bits 5..8 magnitude size, bits 9..13 positions that the symbol moves on by (sequential DC: 1; an end of band of an
+//               AC first pass: its run-length exponent), bit 15 end of band or block (beyond every position)
 // 0 = a code longer than kTabBits bits, or no valid symbol of this kind of scan.
 // ---------------------------------------------------------------------------------------
 constexpr int kTabBits = 10;
@@ -68,17 +77,13 @@ __device__ __forceinline__ uint32_t sym_entry(int kind, uint32_t len, uint32_t s
     const uint32_t r = (sym >> 4) & 15u, sz = sym & 15u;
     if (kind == kTabDc) return sym > 15u ? 0u : ((len + sz) | (sz << 5));
     if (kind == kTabDcSeq) return sym > 15u ? 0u : ((len + sz) | (sz << 5) | (1u << 9));
-    if (kind == kTabAcSeq) {
-        if (!sz && r && r != 15u) return 0u;
-        return (len + sz) | (sz << 5) | ((r + 1u) << 9) | (sz || r ? 0u : kEntEob);
-    }
     if (kind == kTabAcRefine) {
         if (sz > 1u) return 0u;
         if (sz || r == 15u) return (len + sz) | (sz << 5) | (r << 8);
         return (len + r) | ((64u + r) << 8);
     }
-    if (sz) return (len + sz) | (sz << 5) | (r << 9);
-    if (r == 15u) return len | (15u << 9);
+    if (sz || r == 15u) return (len + sz) | (sz << 5) | ((r + 1u) << 9);
+    if (kind == kTabAcSeq) return r ? 0u : len | (1u << 9) | kEntEob;
     return (len + r) | (r << 9) | kEntEob;
 }
 
@@ -341,7 +346,7 @@ __device__ __forceinline__ uint64_t low_mask(int p) { return p >= 64 ? ~0ull : (
 // ---------------------------------------------------------------------------------------
 // Bit reader of the interval kernels.  The position is one number: bits counted from the first bit of a
 // 16-byte group of the unstuffed copy.  The words around it lie in the lane's column of a ring in shared
-// memory (one row more than the ring: it repeats row 0), so the window of the next 32 bits is two shared
+// memory (two rows more than the ring: they repeat rows 0 and 1), so the window of the next 32 bits is two shared
 // loads and a funnel shift, and skipping is an addition: no buffer, no refill branch.  All lanes top their
 // columns up together.  `stop` is the first position at which a step may not begin (the ring runs out, the
 // interval has ended, the lane has nothing to do): one comparison per step.
@@ -356,6 +361,21 @@ __device__ __forceinline__ void sts16_if(bool on, uint32_t a, uint32_t v) {
 }
 __device__ __forceinline__ void sts32_if(bool on, uint32_t a, uint32_t v) {
     asm volatile("{ .reg .pred p; setp.ne.u32 p, %2, 0; @p st.shared.u32 [%0], %1; }" : : "r"(a), "r"(v), "r"((uint32_t)on) : "memory");
+}
+__device__ __forceinline__ void sts128_if(bool on, uint32_t a, const uint4& v) {
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %5, 0; @p st.shared.v4.u32 [%0], {%1, %2, %3, %4}; }" : : "r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"((uint32_t)on) : "memory");
+}
+__device__ __forceinline__ void stg16_if(bool on, void* a, uint32_t v) {
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %2, 0; @p st.global.u16 [%0], %1; }" : : "l"(a), "h"((uint16_t)v), "r"((uint32_t)on) : "memory");
+}
+__device__ __forceinline__ void stg32_if(bool on, void* a, uint32_t v) {
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %2, 0; @p st.global.u32 [%0], %1; }" : : "l"(a), "r"(v), "r"((uint32_t)on) : "memory");
+}
+__device__ __forceinline__ void stg64_if(bool on, void* a, uint32_t x, uint32_t y) {
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %3, 0; @p st.global.v2.u32 [%0], {%1, %2}; }" : : "l"(a), "r"(x), "r"(y), "r"((uint32_t)on) : "memory");
+}
+__device__ __forceinline__ void stg128_if(bool on, void* a, const uint4& v) {
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %5, 0; @p st.global.v4.u32 [%0], {%1, %2, %3, %4}; }" : : "l"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"((uint32_t)on) : "memory");
 }
 __device__ __forceinline__ uint2 lds64(uint32_t a) { uint2 v; asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a) : "memory"); return v; }
 __device__ __forceinline__ uint4 lds128(uint32_t a) { uint4 v; asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory"); return v; }
@@ -392,7 +412,7 @@ struct LaneBits {
     __device__ __forceinline__ void put(uint32_t w, const uint4& v) {
         const uint32_t p = col + (w & (kRingWords - 1)) * 128u;
         sts32(p, v.x); sts32(p + 128u, v.y); sts32(p + 256u, v.z); sts32(p + 384u, v.w);
-        if ((w & (kRingWords - 1)) == 0) sts32(p + kRingWords * 128u, v.x);
+        if ((w & (kRingWords - 1)) == 0) { sts32(p + kRingWords * 128u, v.x); sts32(p + kRingWords * 128u + 128u, v.y); }
     }
     // Top-up (all lanes of the warp together): what the next one will store first is requested right after
     // the previous one, so that its latency passes beside the decode steps.
@@ -534,8 +554,8 @@ __device__ __forceinline__ uint4 value_record(uint32_t m0, uint32_t m1, const in
 constexpr int kDecodeSteps = 16;     // decode steps between two top-ups of the rings
 constexpr int kMaskQueue = 8;        // blocks whose masks a refinement lane holds ahead
 
-// Shared memory of one warp (dynamic): two tables, the ring, and for waves with AC refinements the mask queue.
-constexpr uint32_t kWarpRing = 2 * sizeof(ScanTab), kWarpQueue = kWarpRing + (kRingWords + 1) * 128;
+// Shared memory of one warp (dynamic): two tables, the ring, a block's positions 0..7 per lane, and for waves with AC refinements the mask queue.
+constexpr uint32_t kWarpRing = 2 * sizeof(ScanTab), kWarpHead = kWarpRing + (kRingWords + 2) * 128, kWarpQueue = kWarpHead + 512;
 template <bool kRefine> __host__ __device__ constexpr uint32_t warp_bytes() { return kWarpQueue + (kRefine ? kMaskQueue * 512 : 0); }
 
 // DC refinement scan s of one image: a bit per block, so bit j of a restart interval is block j in scan order and a thread
@@ -597,7 +617,13 @@ __device__ __forceinline__ void dc_refine_image(const Params& P, int s, int img,
 // Blocks from runs.item_blocks on (kRefine) do the wave's DC refinement scans, which touch nothing the others do, in the
 // shadow of the chains instead of in a launch behind them: 32 images of 32x32 at k = 10 72 -> 66 us, 96 mixed 4:4:4 images
 // 457 -> 437 us, 1024 CelebA-shaped 498 -> 491 us.
-template <bool kRoi, bool kRefine>
+//
+// First passes: a step is one straight line of predicated instructions (with branches for block ends and long codes 300
+// cycles an AC symbol alone on an SM, now 230), and what a warp needs of the tables is loaded at once (the start of a warp 6 to 10 k cycles,
+// now 3.5 k).  kPack: see below and pack_first_passes; without it the stores of 1024 ImageNet-shaped images at k = 5 took half of
+// the load/store units' time, 197 us against 172 (before: 206).  64 images 66 -> 44 us.  DC alone of 1024 images 55 -> 40 us (pairs
+// of luminance blocks stored together, MCUs without a branch inside).
+template <bool kRoi, bool kRefine, bool kPack>
 __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, ItemRuns runs) {
     extern __shared__ __align__(16) uint8_t s_entropy[];
     __shared__ __align__(16) uint8_t s_sel[kRefine ? sizeof(SelectTable) : 16];
@@ -620,23 +646,26 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, I
     const Item item = P.items[runs.first[run_no] + it - (run_no ? runs.end[run_no - 1] : 0u)];
     const bool half = kRefine && item.pair && lane >= 16;     // this lane decodes the later scan of the pair
     const uint32_t li = kRefine && item.pair ? (uint32_t)lane & 15u : (uint32_t)lane;
-    const ScanDesc sd0 = P.scans[item.si];
-    const int s = (int)((item.si + (half ? item.pair : 0u)) / (uint32_t)P.N);
-    const ScanScript sc = P.script[s];
-    const ScanAux ax = P.saux[s];
-    const bool dc = sc.Ss == 0;              // a DC first pass (DC refinement scans have no items)
     // tables: a DC scan may use two tables of one image; an AC item may span two images
     const bool two_images = item.next != 0;
     const uint32_t si1 = two_images ? item.next - 1u : item.si + item.pair;
+    const uint32_t N = (uint32_t)P.N, s0 = item.si / N, s1 = si1 / N;
+    const int s = (int)(half ? s1 : s0);
+    const ScanDesc sd0 = load_entry(P.scans + item.si), sd1 = load_entry(P.scans + si1);
+    const ScanAux ax0 = load_entry(P.saux + s0), ax1 = load_entry(P.saux + s1);
+    const ScanScript sc = load_entry(P.script + s);
+    const ImgDesc im0 = load_entry(P.imgs + item.si % N), im1 = load_entry(P.imgs + si1 % N);
+    const bool dc = sc.Ss == 0;              // a DC first pass (DC refinement scans have no items)
+    const ScanAux ax = half ? ax1 : ax0;
     // From here on no lane leaves before the warp does: lanes without work just stay `done`.
     bool done = li >= item.count;
     const uint32_t rem0 = sd0.nseg - item.seg0;               // restart intervals left in the first image
     const uint32_t which = half || (two_images && li >= rem0) ? 1u : 0u;
     uint32_t seg = two_images && li >= rem0 ? li - rem0 : item.seg0 + li;
-    const ScanDesc sd = which ? P.scans[si1] : sd0;
-    const int img = (int)((which ? si1 : item.si) % (uint32_t)P.N);
+    const ScanDesc sd = which ? sd1 : sd0;
+    const int img = (int)((which ? si1 : item.si) % N);
     if (seg >= sd.nseg) { done = true; seg = 0; }
-    const ImgDesc im = P.imgs[img];
+    const ImgDesc im = which ? im1 : im0;
     const Geometry g = make_geometry(im, P);
 
     const bool inter = sc.ncomp > 1;
@@ -659,21 +688,28 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, I
         if (__all_sync(full, done)) return;                               // nothing of this item is wanted
     }
     const uint32_t mem = (uint32_t)__cvta_generic_to_shared(s_entropy) + (uint32_t)wid * warp_bytes<kRefine>();
+    const uint32_t* segtab = P.seg_start + sd.seg_base;
+    uint32_t bstart = __ldg(segtab + seg);
+    uint32_t bend = __ldg(segtab + seg + 1) - 2;
     {
-        const ScanAux ax0 = P.saux[item.si / (uint32_t)P.N];
-        const uint32_t t0 = ax0.tab0 + (item.si % (uint32_t)P.N) * (uint32_t)ax0.ntab;
-        const ScanAux ax1 = P.saux[si1 / (uint32_t)P.N];
-        const uint32_t t1 = dc ? t0 + 1u : ax1.tab0 + (si1 % (uint32_t)P.N) * (uint32_t)ax1.ntab;
+        const uint32_t t0 = ax0.tab0 + (item.si % N) * (uint32_t)ax0.ntab;
+        const uint32_t t1 = dc ? t0 + 1u : ax1.tab0 + (si1 % N) * (uint32_t)ax1.ntab;
         const bool second = two_images || item.pair || (dc && sd0.tab_off[1]);
         const uint4* a = reinterpret_cast<const uint4*>(P.tabs + t0);
         const uint4* b = reinterpret_cast<const uint4*>(P.tabs + t1);
         constexpr int n = (int)(sizeof(ScanTab) / 16);
-        for (int i = lane; i < n; i += 32) sts128(mem + 16 * i, __ldg(a + i));
-        if (second) for (int i = lane; i < n; i += 32) sts128(mem + 16 * (n + i), __ldg(b + i));
+        uint4 v[(n + 31) / 32];
+#pragma unroll
+        for (int i = 0; i < (n + 31) / 32; ++i) if (lane + 32 * i < n) v[i] = __ldg(a + lane + 32 * i);
+#pragma unroll
+        for (int i = 0; i < (n + 31) / 32; ++i) if (lane + 32 * i < n) sts128(mem + 16 * (lane + 32 * i), v[i]);
+        if (second) {
+#pragma unroll
+            for (int i = 0; i < (n + 31) / 32; ++i) if (lane + 32 * i < n) v[i] = __ldg(b + lane + 32 * i);
+#pragma unroll
+            for (int i = 0; i < (n + 31) / 32; ++i) if (lane + 32 * i < n) sts128(mem + 16 * (n + lane + 32 * i), v[i]);
+        }
     }
-    const uint32_t* segtab = P.seg_start + sd.seg_base;
-    uint32_t bstart = segtab[seg];
-    uint32_t bend = segtab[seg + 1] - 2;
     bool bad = false;
     if (!done && (bstart < sd.data_off || bend > sd.data_end || bend < bstart)) {   // a missing marker left a hole
         bad = true; done = true;
@@ -683,6 +719,8 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, I
     br.init(mem + kWarpRing + 4u * lane, P.ubuf, bstart, bend);
     const int Al = sc.Al;
     if (m0 >= m1) done = true;
+    RingWords<kRingWords> W;
+    W.col = br.col;
 
     if (dc) {
         // ---- DC first pass: one MCU per step, its blocks unrolled
@@ -694,39 +732,57 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, I
         const uint32_t y_off = inter ? 0u : (uint32_t)(g.coff[c0] - im.blk_base), c_off = (uint32_t)(g.coff[1] - im.blk_base), c_step = g.mx * g.my;
         int16_t* dcp = P.dc + im.blk_base;
         pin(dcp);
+        const uint32_t t0 = mem + (sd.slots & 1u) * (uint32_t)sizeof(ScanTab), t1 = mem + ((sd.slots >> 2) & 1u) * (uint32_t)sizeof(ScanTab),
+                       t2 = mem + ((sd.slots >> 4) & 1u) * (uint32_t)sizeof(ScanTab);      // tables of the luminance (or the scan's own) and the chroma blocks
         for (;;) {
             br.topup(!done);
             __syncwarp(full);
             if (__all_sync(full, done)) break;
-            // an MCU's symbols need at most 6 * 31 bits: seven words and the window's second one
-            const uint32_t stop = done ? 0u : min(br.ring_stop(8), br.limit + 1u);
+            // an MCU's symbols need at most 6 * 31 bits: seven words and the windows' second and third one
+            const uint32_t stop = done ? 0u : min(br.ring_stop(9), br.limit + 1u);
+            // (The chain: entry -> next window -> next entry; everything else is requested or done beside it.)
+            W.load(br.pos);
+            uint32_t win = W.window(br.pos), e = tab_entry(t0, win);
 #pragma unroll 1
             for (int t = 0; t < kDecodeSteps / 4; ++t) {
                 if (br.pos >= stop || m >= m1 || bad) continue;
                 const uint32_t yb = y_off + (vs * mrow) * bw0 + hs * mcol, cb = c_off + mrow * g.mx + mcol;
-                uint32_t e = 1;
+                // Straight through the MCU; one that holds a code longer than the table's index is gone over again (long codes
+                // looked up), so that nothing branches inside.
+                const uint32_t pos0 = br.pos, win0 = win, e0 = e;
+                const int was0 = pred0, was1 = pred1, was2 = pred2;
+                bool again = false, longs = false;
+                do {
+                    if (again) {
+                        longs = true; again = false;
+                        br.pos = pos0; win = win0; e = e0; pred0 = was0; pred1 = was1; pred2 = was2;
+                        W.load_behind(br.pos);
+                    }
+                    int before = 0;
 #pragma unroll
-                for (int j = 0; j < 6; ++j) {
-                    if (j >= bpm) break;
-                    if (br.pos > br.limit) break;
-                    const int ci = j < ny ? 0 : j - ny + 1;
-                    const uint32_t tab = mem + ((sd.slots >> (2 * ci)) & 1u) * (uint32_t)sizeof(ScanTab);
-                    const uint32_t win = br.window(br.pos);
-                    e = lds16(tab + ((win >> (32 - kTabBits)) << 1));
-                    if (e == 0) { e = long_code(tab, win, kTabDc); if (e == 0) break; }
-                    const uint32_t skip = e & 31u;
-                    const int d = magnitude(win, skip, e >> 5);
-                    br.pos += skip;
-                    int pv;
-                    uint32_t blk;
-                    if (j < ny || !inter) { pv = (pred0 += d); blk = yb + ((uint32_t)j & (hs - 1u)) + ((uint32_t)j >> (hs - 1u)) * bw0; }
-                    else if (j == ny) { pv = (pred1 += d); blk = cb; }
-                    else { pv = (pred2 += d); blk = cb + c_step; }
-                    dcp[blk] = (int16_t)(pv << Al);
-                }
+                    for (int j = 0; j < 6; ++j) {
+                        if (j >= bpm) break;
+                        const bool luma = j < ny || !inter, cbl = !luma && j == ny;
+                        if (longs && e == 0) { e = long_code(luma ? t0 : (cbl ? t1 : t2), win, kTabDc); bad = bad || e == 0; }      // (then nothing moves on)
+                        again = again || e == 0;
+                        const uint32_t skip = e & 31u, sz = e >> 5, behind = W.behind(br.pos), after = j + 1 >= bpm || j + 1 < ny ? t0 : (j + 1 == ny ? t1 : t2);
+                        const uint32_t next = __funnelshift_l(behind, win, skip);
+                        e = tab_entry(after, next);
+                        br.pos += skip;
+                        W.load_behind(br.pos);
+                        const int d = magnitude(win, skip, sz);
+                        win = next;
+                        if (luma) {
+                            pred0 += d;
+                            if (hs == 1u) dcp[yb + (uint32_t)j * bw0] = (int16_t)(pred0 << Al);
+                            else if (j & 1) *reinterpret_cast<uint32_t*>(dcp + yb + (uint32_t)(j >> 1) * bw0) = __byte_perm((uint32_t)(before << Al), (uint32_t)(pred0 << Al), 0x5410);
+                            before = pred0;
+                        } else if (cbl) dcp[cb] = (int16_t)((pred1 += d) << Al);
+                        else dcp[cb + c_step] = (int16_t)((pred2 += d) << Al);
+                    }
+                } while (again && !longs);
                 ++m;
                 if (++mcol == mcu_w) { mcol = 0; ++mrow; }
-                bad = e == 0;
             }
             __syncwarp(full);
             bad = bad || br.pos > br.limit;
@@ -745,53 +801,87 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, I
             int16_t* headp = P.head + g.coff[c] * 8;
             pin(auxp); pin(headp);
             const bool lists = ax.stride == 2u;            // the band reaches beyond position 7
-            int16_t* vp = P.vals + 4ull * bstart;           // next value
-            int16_t* vb = vp;                               // the block's first one
+            // kPack: values leave four at a time (the list is one run per interval), a block's positions 1..7 in whole words where
+            // the band holds whole words of them: a lane's store is a sector of its own, and the stores of five scans are
+            // what a full machine waits for.
+            int16_t* const vlist = P.vals + 4ull * bstart;
+            uint32_t nv = 0, nv0 = 0, v01 = 0, v23 = 0;     // values so far, those before the block, the last four
+            const uint32_t hlo = max(Ss, 1u), hhi = min(Se, 7u);
+            // how the head leaves: 0 by coefficient, 1 all of it, 2 its first six positions, 3 its last two
+            const int heads = !kPack ? 0 : (hlo == 1u && hhi == 7u ? 1 : (hlo == 1u && hhi == 5u ? 2 : (hlo == 6u && hhi == 7u ? 3 : 0)));
+            const uint32_t slot = mem + kWarpHead + 16u * lane;
+            sts128(slot, make_uint4(0, 0, 0, 0));
             uint32_t wrap_m = m + mcu_w - bcol;             // the first block of the next block row
             uint32_t M0 = 0, M1 = 0, k = Ss;
             for (;;) {
                 br.topup(!done);
                 __syncwarp(full);
                 if (__all_sync(full, done)) break;
-                uint32_t stop = done ? 0u : min(br.ring_stop(2), br.limit + 1u);
+                uint32_t stop = done ? 0u : min(br.ring_stop(3), br.limit + 1u);
+                W.load(br.pos);
+                uint32_t win = W.window(br.pos), raw = tab_entry(tab, win);
+                // A step is one straight line but for block rows that end.  An entry of zero moves nothing on: lanes that have
+                // arrived somewhere, and those that stand at a code longer than the table's index, wait.
 #pragma unroll 1
-                for (int t = 0; t < kDecodeSteps; ++t) {
-                    if (br.pos < stop) {
-                        const uint32_t win = br.window(br.pos);
-                        uint32_t e = lds16(tab + ((win >> (32 - kTabBits)) << 1));
-                        if (e == 0) e = long_code(tab, win, kTabAcFirst);
-                        const uint32_t skip = e & 31u, sz = (e >> 5) & 15u, r = (e >> 9) & 15u;
+                for (int t = 0; t < kDecodeSteps; t += 8) {
+#pragma unroll 4
+                    for (int q = 0; q < 8; ++q) {
+                        const uint32_t e = br.pos < stop ? raw : 0u, behind = W.behind(br.pos);
+                        const uint32_t skip = e & 31u, sz = (e >> 5) & 15u, next = __funnelshift_l(behind, win, skip);
+                        raw = tab_entry(tab, next);
                         br.pos += skip;
-                        k += r;                                            // position of the coefficient
-                        const bool coef = sz && k <= Se, far = coef && k >= 8u;
+                        W.load_behind(br.pos);
+                        k += e >> 9;                           // behind the coefficient (an end of band: beyond every position)
+                        const uint32_t at = k - 1u;
+                        const bool coef = sz && k <= Se + 1u, far = coef && k > 8u;
                         const int val = magnitude(win, skip, sz) << Al;
-                        if (coef && !far) headp[8u * (uint64_t)bi + k] = (int16_t)val;
-                        if (far) *vp = (int16_t)val;
-                        vp += far ? 1 : 0;
-                        M0 |= shl0(coef ? 1u : 0u, k); M1 |= shl0(coef ? 1u : 0u, k - 32u);
-                        if (e == 0 || (sz && k > Se)) { bad = true; stop = 0; k = 0; }   // no such symbol, or a coefficient behind the band
-                        ++k;                                               // (sixteen zeros: run 15 plus one)
-                        const bool is_eob = (e & kEntEob) != 0;
-                        if (is_eob || k > Se) {
-                            if (M0 | M1) {
-                                if (lists) *reinterpret_cast<uint4*>(auxp + (uint64_t)bi * 2) = value_record(M0, M1, vb);
-                                else *reinterpret_cast<uint2*>(auxp + bi) = make_uint2(M0, M1);
-                            }
-                            k = Ss; M0 = 0; M1 = 0; vb = vp;
-                            // an end of band may leave the following blocks empty too
-                            const uint32_t adv = is_eob ? (1u << r) + shr0(shl0(win, skip - r), 32u - r) : 1u;
-                            m += adv; bi += adv;
-                            if (m >= wrap_m) {                             // (rows in between only where an interval holds several)
-                                if (m >= m1) stop = 0;
-                                else { const uint32_t row = m / mcu_w; bi = row * bw + (m - row * mcu_w); wrap_m = (row + 1u) * mcu_w; }
-                            }
-                            if (m >= m1) stop = 0;
+                        const bool end = k > Se;               // the block is finished (also where nothing of the band is left)
+                        int16_t* const h = headp + 8u * (uint64_t)bi;
+                        M0 |= shl0(coef ? 1u : 0u, at); M1 |= shl0(coef ? 1u : 0u, at - 32u);
+                        nv += far ? 1u : 0u;
+                        if (kPack) {
+                            v01 = far ? __byte_perm(v01, v23, 0x5432) : v01;
+                            v23 = far ? __byte_perm(v23, (uint32_t)val, 0x5432) : v23;
+                            stg64_if(far && (nv & 3u) == 0, vlist + nv - 4u, v01, v23);
+                        } else stg16_if(far, vlist + nv - 1u, (uint32_t)val);
+                        if (heads == 0) stg16_if(coef && !far, h + at, (uint32_t)val);
+                        else {
+                            sts16_if(coef && !far, slot + 2u * at, (uint32_t)val);
+                            const uint4 v = lds128(slot);
+                            if (heads == 1) stg128_if(end && (M0 & 0xFEu), h, v);
+                            else if (heads == 2) { stg64_if(end && (v.x | v.y), h, v.x, v.y); stg32_if(end && v.z, h + 4, v.z); }
+                            else stg32_if(end && v.w, h + 6, v.w);
+                            sts128_if(end, slot, make_uint4(0, 0, 0, 0));
                         }
+                        const bool some = end && (M0 | M1) != 0;
+                        if (lists) stg128_if(some, auxp + (uint64_t)bi * 2, value_record(M0, M1, vlist + nv0));
+                        else stg64_if(some, auxp + bi, M0, M1);
+                        if (sz && k > Se + 1u) { bad = true; stop = 0; }           // a coefficient behind the band
+                        // an end of band may leave the following blocks empty too
+                        const uint32_t r = (e >> 9) & 15u, adv = e & kEntEob ? __funnelshift_l(shl0(win, skip - r), 1u, r) : 1u;   // 2^r + the r bits that end the symbol
+                        m += end ? adv : 0u; bi += end ? adv : 0u;
+                        k = end ? Ss : k; nv0 = end ? nv : nv0;
+                        M0 = end ? 0u : M0; M1 = end ? 0u : M1;
+                        if (m >= wrap_m && m < m1) {           // (only where an interval holds several rows)
+                            const uint32_t row = m / mcu_w;
+                            bi = row * bw + (m - row * mcu_w); wrap_m = (row + 1u) * mcu_w;
+                        }
+                        stop = m >= m1 ? 0u : stop;
+                        win = next;
+                    }
+                    if (raw == 0 && br.pos < stop) {           // (taken by the next step)
+                        raw = long_code(tab, win, kTabAcFirst);
+                        if (raw == 0) { bad = true; stop = 0; }        // no such symbol: the lane ends here
                     }
                 }
                 __syncwarp(full);
                 bad = bad || br.pos > br.limit;
                 done = done || bad || m >= m1;
+            }
+            // the last values (what lies behind them up to the group of four belongs to this interval too)
+            if (kPack && (nv & 3u)) {
+                for (uint32_t p = nv & 3u; p < 4u; ++p) { v01 = __byte_perm(v01, v23, 0x5432); v23 >>= 16; }
+                *reinterpret_cast<uint2*>(vlist + (nv & ~3u)) = make_uint2(v01, v23);
             }
         } else {
             // ---- AC refinement: one Huffman symbol, or one block of an end-of-band run, per step.

@@ -217,6 +217,7 @@ struct pcr_record {
     std::vector<int> pair_of;
     bool pairs_fit = true;                                      // the waves with pairs fit the machine (see open_impl)
     uint32_t refine_ctas = 8;                                   // see refine_in_ctas (PCR_REFINE_CTAS overrides)
+    uint32_t pack_warps = 12;                                   // see pack_first_passes (PCR_PACK_WARPS overrides)
     std::vector<uint32_t> pair_begin, pair_count;               // [n_slices][G] items of the pair, by its later scan
     uint32_t n_units = 0;
     // device state
@@ -801,6 +802,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
         } else r->pair_of.assign(G, -1);
     }
     if (const char* e = getenv("PCR_REFINE_CTAS")) r->refine_ctas = (uint32_t)std::max(0, atoi(e));
+    if (const char* e = getenv("PCR_PACK_WARPS")) r->pack_warps = (uint32_t)std::max(0, atoi(e));
     // slices: enough images each to fill the machine, few enough to keep launches cheap
     {
         // four at most: one record decodes as fast with four slices as with eight, and two records
@@ -984,8 +986,6 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     units_kernel<<<N, 128, 0, r->up_stream>>>(r->d_imgs, r->d_order, r->d_unit_prefix, r->d_units, r->unit_mcus, r->unit_rows,
                                               r->d_scans, T.d<uint32_t>(at_base), G, bpm);
     ++g_launches;
-    if (cudaFuncSetAttribute(refine_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRefineBytes) != cudaSuccess ||
-        cudaFuncSetAttribute(refine_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRefineBytes) != cudaSuccess) return PCR_E_CUDA;
     if (n_groups && cudaFuncSetAttribute(ac_refine_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kChainPairs * sizeof(ChainShared))) != cudaSuccess) return PCR_E_CUDA;
     r->h_status.assign(N, 0);
     r->resident = 0;
@@ -1048,8 +1048,12 @@ uint64_t hash_bytes(uint64_t h, const uint8_t* p, size_t n) {
     return h;
 }
 uint32_t env_key() {
-    const char* a = getenv("PCR_SLICES"); const char* b = getenv("PCR_LONG_MIN_BYTES"); const char* c = getenv("PCR_REFINE_CTAS");
-    return ((a ? (uint32_t)atoi(a) + 1u : 0u) * 1000003u + (b ? (uint32_t)atoi(b) + 1u : 0u)) * 1009u + (c ? (uint32_t)atoi(c) + 1u : 0u);
+    uint32_t h = 0;
+    for (const char* name : {"PCR_SLICES", "PCR_LONG_MIN_BYTES", "PCR_REFINE_CTAS", "PCR_PACK_WARPS"}) {
+        const char* v = getenv(name);
+        h = h * 1000003u + (v ? (uint32_t)atoi(v) + 1u : 0u);
+    }
+    return h;
 }
 // 0 when the bytes do not even look like a record (pcr_open then reports the error)
 uint64_t record_identity(const uint8_t* rec, size_t len) {
@@ -1260,6 +1264,18 @@ static void coef_lists(const pcr_record* rec, int k, CoefLists* cl) {
     for (int c = 0; c < 3; ++c) memcpy(&cl->head_mask[c], mask[c], 16);
 }
 
+// refine_kernel's shared memory is beyond what a launch may take unasked; asked for once per device and kernel (asking loads the kernel,
+// which records without refinements have no use for).
+template <bool kRoi>
+static bool allow_refine_smem(int device) {
+    static std::atomic<uint64_t> asked{0};
+    const uint64_t bit = 1ull << (device & 63);
+    if (device < 64 && (asked.load(std::memory_order_acquire) & bit)) return true;
+    if (cudaFuncSetAttribute(refine_kernel<kRoi>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRefineBytes) != cudaSuccess) return false;
+    if (device < 64) asked.fetch_or(bit, std::memory_order_release);
+    return true;
+}
+
 // Whether refine_kernel's CTAs take the AC refinements among scans k0 .. k-1 of a wave, or lane-per-interval warps of
 // entropy_kernel.  A CTA's chains are four times as fast (170 to 220 against 700 cycles a symbol), but three CTAs are all an SM
 // holds, 96 chains against 576, so a launch of many items is better off with the warps.  Decode at k = 10 in us,
@@ -1277,6 +1293,18 @@ static bool refine_in_ctas(const pcr_record* rec, const std::vector<int>& wave, 
         for (int g = 0; g < rec->n_slices; ++g) ctas += items[(size_t)g * rec->G + s];
     }
     return ctas <= (uint64_t)rec->refine_ctas * (uint64_t)rec->n_sms;
+}
+
+// Whether the first passes among scans k0 .. k-1 of a wave pack their stores (kPack of entropy_kernel): where the
+// machine is full, because stores are what it waits for; elsewhere a step without the packing is the shorter chain.  First wave in
+// us without and with packing, by warps an SM: ImageNet-shaped images at k = 5 0.2 38 and 58, 2.3 44 and 69, 9 61 and 86, 36 197
+// and 172; CelebA-shaped 18 98 and 86.
+static bool pack_first_passes(const pcr_record* rec, const std::vector<int>& wave, int k0, int k) {
+    uint64_t warps = 0;
+    for (int s : wave)
+        if (s >= k0 && s < k && rec->script[s].Ah == 0)
+            for (int g = 0; g < rec->n_slices; ++g) warps += rec->item_count[(size_t)g * rec->G + s];
+    return warps > (uint64_t)rec->pack_warps * (uint64_t)rec->n_sms;
 }
 
 // Decode scans k0 .. k-1 on top of the state scans 0 .. k0-1 left behind (k0 = 0: from scratch),
@@ -1397,7 +1425,7 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
             ItemRuns runs, refs;
             runs.n = refs.n = 0;
             uint32_t count = 0, ref_count = 0;
-            bool refine = false;                           // waves without AC refinements need no mask queues
+            bool refine = false, failed = false;           // waves without AC refinements need no mask queues
             int dc_n = 0, dc_s[3];                         // the wave's DC refinements, at most one per component
             for (int s : waves[w])
                 if (s >= k0 && s < k && rec->script[s].Ss == 0 && rec->script[s].Ah != 0 && dc_n < 3) dc_s[dc_n++] = s;
@@ -1414,15 +1442,23 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
                 const uint32_t smem = kEntropyWarps * (refine ? warp_bytes<true>() : warp_bytes<false>());
                 runs.item_blocks = nb;
                 if (last && refine && !dc_done) nb += carry_dc(runs, (rec->dc_refine_chunks + 1) / 2);      // about five MCUs a thread (waves without AC refinements are compiled without this)
-                if (roi && refine) entropy_kernel<true, true><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
-                else if (roi) entropy_kernel<true, false><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
-                else if (refine) entropy_kernel<false, true><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
-                else entropy_kernel<false, false><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
+                const bool pack = pack_first_passes(rec, waves[w], k0, k);
+                if (refine) {
+                    if (roi) entropy_kernel<true, true, true><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
+                    else entropy_kernel<false, true, true><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
+                } else if (pack) {
+                    if (roi) entropy_kernel<true, false, true><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
+                    else entropy_kernel<false, false, true><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
+                } else {
+                    if (roi) entropy_kernel<true, false, false><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
+                    else entropy_kernel<false, false, false><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
+                }
                 ++g_launches;
                 runs.n = 0; count = 0;
             };
             auto launch_refinements = [&](bool last) {
                 if (!ref_count) return;
+                if (!(roi ? allow_refine_smem<true>(rec->device) : allow_refine_smem<false>(rec->device))) failed = true;
                 unsigned nb = ref_count;
                 refs.item_blocks = nb;
                 if (last && !dc_done) nb += carry_dc(refs, (rec->dc_refine_chunks + 1) / 2);      // about two MCUs a thread
@@ -1471,6 +1507,7 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
             }
             launch_refinements(true);
             launch_items(true);
+            if (failed) return false;
             // scans that are one long restart interval: the first passes of the wave (a contiguous run
             // of the list) ...
             {

@@ -91,8 +91,8 @@ struct AcSteps {
         return long_entry(tabs, long_window(base, pos), kTabAcFirst);
     }
     __device__ __forceinline__ bool advance(uint32_t e, uint32_t& st) const {
-        st += ((e >> 9) & 15u) + 1u;                                       // (sixteen zeros: run 15 plus one)
-        const bool end = (e & kEntEob) || st > Se;
+        st += e >> 9;                                                      // (an end of band: beyond every position)
+        const bool end = st > Se;
         st = end ? Ss : st;
         return end;
     }
@@ -369,7 +369,7 @@ __global__ void __launch_bounds__(32 * kLongWarps) first_pass_long_kernel(Params
             const uint32_t win = long_window(L.base, p), e = S.entry(p, k);
             const uint32_t skip = e & 31u, sz = (e >> 5) & 15u;
             p += skip;
-            k += (e >> 9) & 15u;                               // position of the coefficient
+            k += (e >> 9) - 1u;                                // position of the coefficient (of an end of band: beyond every one)
             const bool eob = (e & kEntEob) != 0, coef = sz && own;
             if (e == 0 || (sz && k > Se)) { bad = true; break; }
             const int val = magnitude(win, skip, sz) << sc.Al;

@@ -188,7 +188,8 @@ __global__ void __launch_bounds__(32 * kRefineWarps, 3) refine_kernel(Params P, 
     const Item item = P.items[runs.first[run_no] + blockIdx.x - (run_no ? runs.end[run_no - 1] : 0u)];
     const bool two_images = item.next != 0;                   // (never a pair's item)
     const uint32_t si1 = two_images ? item.next - 1u : item.si + item.pair;
-    const ScanScript sc = P.script[item.si / (uint32_t)P.N];  // (a pair's scans have the same component and band)
+    const uint32_t N = (uint32_t)P.N, s0 = item.si / N, s1 = si1 / N;
+    const ScanScript sc = load_entry(P.script + s0);          // (a pair's scans have the same component and band)
     const uint32_t Ss = (uint32_t)sc.Ss, Se = (uint32_t)sc.Se;
     const uint64_t band = low_mask((int)Se + 1) & ~low_mask((int)Ss);
 
@@ -199,14 +200,15 @@ __global__ void __launch_bounds__(32 * kRefineWarps, 3) refine_kernel(Params P, 
     int img = 0;
     bool bad = false;
     if (wid == 0) {
-        const ScanDesc sd0 = P.scans[item.si];
+        const ScanDesc sd0 = load_entry(P.scans + item.si), sd1 = load_entry(P.scans + si1);
+        const ImgDesc im0 = load_entry(P.imgs + item.si % N), im1 = load_entry(P.imgs + si1 % N);
+        const ScanAux ax = load_entry(P.saux + (half ? s1 : s0));
         const uint32_t rem0 = sd0.nseg - item.seg0;           // restart intervals left in the first image
         const uint32_t which = half || (two_images && li >= rem0) ? 1u : 0u, si = which ? si1 : item.si;
         uint32_t seg = two_images && li >= rem0 ? li - rem0 : item.seg0 + li;
-        const ScanDesc sd = which ? P.scans[si1] : sd0;
-        img = (int)(si % (uint32_t)P.N);
-        const ScanAux ax = P.saux[si / (uint32_t)P.N];
-        const ImgDesc im = P.imgs[img];
+        const ScanDesc sd = which ? sd1 : sd0;
+        img = (int)(si % N);
+        const ImgDesc im = which ? im1 : im0;
         const Geometry g = make_geometry(im, P);
         const int c = sc.comp[0];
         bool done = li >= item.count;
@@ -229,7 +231,7 @@ __global__ void __launch_bounds__(32 * kRefineWarps, 3) refine_kernel(Params P, 
         uint32_t strides = 0;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const ScanAux x = P.saux[ax.src[q < ax.nsrc ? q : 0]];
+            const ScanAux x = load_entry(P.saux + ax.src[q < ax.nsrc ? q : 0]);
             sh.src[q][lane] = q < ax.nsrc ? reinterpret_cast<uint64_t>(P.aux + x.base + g.loff[c] * x.stride) : 0ull;
             strides |= x.stride << (8 * q);
         }
@@ -238,9 +240,9 @@ __global__ void __launch_bounds__(32 * kRefineWarps, 3) refine_kernel(Params P, 
         sh.row0[lane] = m0 / mcu_w * g.bw[c]; sh.col0[lane] = m0 % mcu_w; sh.width[lane] = mcu_w; sh.pitch[lane] = g.bw[c];
         sh.tab[lane] = (uint32_t)__cvta_generic_to_shared(&sh.tabs[which].t);
     } else {
-        const ScanAux ax0 = P.saux[item.si / (uint32_t)P.N], ax1 = P.saux[si1 / (uint32_t)P.N];
-        const uint4* a = reinterpret_cast<const uint4*>(P.tabs + ax0.tab0 + item.si % (uint32_t)P.N);      // (an AC scan has one table)
-        const uint4* b = reinterpret_cast<const uint4*>(P.tabs + ax1.tab0 + si1 % (uint32_t)P.N);
+        const ScanAux ax0 = load_entry(P.saux + s0), ax1 = load_entry(P.saux + s1);
+        const uint4* a = reinterpret_cast<const uint4*>(P.tabs + ax0.tab0 + item.si % N);      // (an AC scan has one table)
+        const uint4* b = reinterpret_cast<const uint4*>(P.tabs + ax1.tab0 + si1 % N);
         constexpr uint32_t words = sizeof(ScanTab) / 16;
         const uint32_t t0 = (uint32_t)__cvta_generic_to_shared(sh.tabs);
         for (uint32_t i = tid - 32u; i < (two_images || item.pair ? 2u : 1u) * words; i += 32u * (kRefineWarps - 1))

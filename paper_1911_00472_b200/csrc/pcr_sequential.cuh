@@ -50,10 +50,10 @@ __global__ void __launch_bounds__(32 * kSeqWarps, 4) sequential_kernel(Params P,
     const uint32_t tid = threadIdx.x, wid = tid >> 5, lane = tid & 31u;
     const unsigned full = 0xffffffffu;
     const Item item = P.items[item_begin + blockIdx.x];
-    const ScanDesc sd = P.scans[item.si];
+    const ScanDesc sd = load_entry(P.scans + item.si);
     const int img = (int)(item.si % (uint32_t)P.N);
-    const ScanAux ax = P.saux[item.si / (uint32_t)P.N];
-    const ImgDesc im = P.imgs[img];
+    const ScanAux ax = load_entry(P.saux + item.si / (uint32_t)P.N);
+    const ImgDesc im = load_entry(P.imgs + img);
     const uint32_t mcu_w = im.mx, total = im.mx * im.my;
     const uint32_t hs = (uint32_t)P.hs, vs = (uint32_t)P.vs, bw0 = hs * mcu_w;
     const uint32_t ny = hs * vs, bpm = P.nc == 3 ? ny + 2u : 1u;      // blocks per MCU (a lone component: one block, no padding)

@@ -6,7 +6,7 @@
 namespace pcr {
 
 // One scan of the (record-wide) scan script: which components, which band, which bit.
-struct ScanScript {
+struct __align__(16) ScanScript {
     int32_t ncomp;
     int32_t comp[3];
     int32_t Ss, Se, Ah, Al;
@@ -24,7 +24,7 @@ struct ScanScript {
 //    block's number in the planes.
 // A refinement scan finds the positions that were non-zero before it by OR-ing the masks of up
 // to four earlier scans (src), each read with its own stride.
-struct ScanAux {
+struct __align__(16) ScanAux {
     uint64_t base;        // first word of this scan's side data
     uint32_t stride;      // words per block: 1 or 2 (first passes), 4 (refinements)
     int32_t nsrc;
@@ -54,7 +54,7 @@ struct RefineList {
 };
 
 // One (scan, image) pair: where its entropy-coded bytes and Huffman tables live.
-struct ScanDesc {
+struct __align__(16) ScanDesc {
     uint32_t data_off;    // first entropy-coded byte (offset in the record)
     uint32_t data_end;    // one past the last byte of the chunk
     uint32_t seg_base;    // first entry of this pair in the segment table
@@ -66,7 +66,7 @@ struct ScanDesc {
     uint32_t slots_ac;    // 2 bits per scan component: which of tab_ac it uses
 };
 
-struct ImgDesc {
+struct __align__(16) ImgDesc {
     uint32_t W, H, mx, my;
     uint64_t blk_base;    // first block of the image in the coefficient planes
     uint64_t out_off;     // first byte of the image in the output buffer
