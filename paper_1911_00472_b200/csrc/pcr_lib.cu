@@ -217,6 +217,7 @@ struct pcr_record {
     std::vector<int> pair_of;
     bool pairs_fit = true;                                      // the waves with pairs fit the machine (see open_impl)
     uint32_t refine_ctas = 8;                                   // see refine_in_ctas (PCR_REFINE_CTAS overrides)
+    uint32_t index_ctas = 8;                                    // see launch_index_kernel (PCR_INDEX_CTAS overrides)
     uint32_t pack_warps = 12;                                   // see pack_first_passes (PCR_PACK_WARPS overrides)
     std::vector<uint32_t> pair_begin, pair_count;               // [n_slices][G] items of the pair, by its later scan
     uint32_t n_units = 0;
@@ -802,6 +803,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
         } else r->pair_of.assign(G, -1);
     }
     if (const char* e = getenv("PCR_REFINE_CTAS")) r->refine_ctas = (uint32_t)std::max(0, atoi(e));
+    if (const char* e = getenv("PCR_INDEX_CTAS")) r->index_ctas = (uint32_t)std::max(0, atoi(e));
     if (const char* e = getenv("PCR_PACK_WARPS")) r->pack_warps = (uint32_t)std::max(0, atoi(e));
     // slices: enough images each to fill the machine, few enough to keep launches cheap
     {
@@ -1049,7 +1051,7 @@ uint64_t hash_bytes(uint64_t h, const uint8_t* p, size_t n) {
 }
 uint32_t env_key() {
     uint32_t h = 0;
-    for (const char* name : {"PCR_SLICES", "PCR_LONG_MIN_BYTES", "PCR_REFINE_CTAS", "PCR_PACK_WARPS"}) {
+    for (const char* name : {"PCR_SLICES", "PCR_LONG_MIN_BYTES", "PCR_REFINE_CTAS", "PCR_PACK_WARPS", "PCR_INDEX_CTAS"}) {
         const char* v = getenv(name);
         h = h * 1000003u + (v ? (uint32_t)atoi(v) + 1u : 0u);
     }
@@ -1381,11 +1383,16 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
     std::vector<char> indexed(rec->n_waves, 0);     // wave w of the current slice has an index launch to wait for
     // index (and lookup tables, where the interval kernels will want them) of the listed scans, all images
     auto launch_index_kernel = [&](const ScanList& sl, cudaStream_t q) {
-        const uint32_t pairs = (uint32_t)sl.n * (uint32_t)rec->N, nb = (pairs + 7) / 8;
+        const uint32_t pairs = (uint32_t)sl.n * (uint32_t)rec->N;
         bool tables = false;
         for (int i = 0; i < sl.n; ++i)
             for (int g = 0; g < rec->n_slices; ++g) tables = tables || rec->item_count[(size_t)g * rec->G + sl.s[i]] + rec->long_count[(size_t)g * rec->G + sl.s[i]] > 0;
-        unstuff_index_kernel<<<nb + (tables ? (pairs + 1) / 2 : 0), 256, 0, q>>>(P, sl, 0, rec->N, nb);
+        // eight CTAs of this size are what an SM holds; decode in us with a warp and with a CTA a pair, by pairs an SM: 64 ImageNet-shaped
+        // images at k = 10 4.3 214 and 195, 256 8.6 (two waves side by side) 425 and 459, 1024 baseline JPEGs 6.9 753 and 683
+        const bool split = pairs <= (uint32_t)rec->index_ctas * (uint32_t)rec->n_sms;
+        const uint32_t nb = split ? pairs : (pairs + kIndexWarps - 1) / kIndexWarps, nt = tables ? (4 * pairs + kIndexWarps - 1) / kIndexWarps : 0;
+        if (split) unstuff_index_kernel<true><<<nb + nt, 32 * kIndexWarps, 0, q>>>(P, sl, 0, rec->N, nb);
+        else unstuff_index_kernel<false><<<nb + nt, 32 * kIndexWarps, 0, q>>>(P, sl, 0, rec->N, nb);
         ++g_launches;
     };
     // restart-interval index of wave w of slice g on stream q: 1 launched, 0 nothing to do, -1 error
