@@ -217,6 +217,7 @@ struct pcr_record {
     std::vector<int> pair_of;
     bool pairs_fit = true;                                      // the waves with pairs fit the machine (see open_impl)
     uint32_t refine_ctas = 8;                                   // see refine_in_ctas (PCR_REFINE_CTAS overrides)
+    uint32_t long_ctas = 3;                                     // see wide_long_scans (PCR_LONG_CTAS overrides)
     uint32_t index_ctas = 8;                                    // see launch_index_kernel (PCR_INDEX_CTAS overrides)
     uint32_t pack_warps = 12;                                   // see pack_first_passes (PCR_PACK_WARPS overrides)
     std::vector<uint32_t> pair_begin, pair_count;               // [n_slices][G] items of the pair, by its later scan
@@ -804,6 +805,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     }
     if (const char* e = getenv("PCR_REFINE_CTAS")) r->refine_ctas = (uint32_t)std::max(0, atoi(e));
     if (const char* e = getenv("PCR_INDEX_CTAS")) r->index_ctas = (uint32_t)std::max(0, atoi(e));
+    if (const char* e = getenv("PCR_LONG_CTAS")) r->long_ctas = (uint32_t)std::max(0, atoi(e));
     if (const char* e = getenv("PCR_PACK_WARPS")) r->pack_warps = (uint32_t)std::max(0, atoi(e));
     // slices: enough images each to fill the machine, few enough to keep launches cheap
     {
@@ -1051,7 +1053,7 @@ uint64_t hash_bytes(uint64_t h, const uint8_t* p, size_t n) {
 }
 uint32_t env_key() {
     uint32_t h = 0;
-    for (const char* name : {"PCR_SLICES", "PCR_LONG_MIN_BYTES", "PCR_REFINE_CTAS", "PCR_PACK_WARPS", "PCR_INDEX_CTAS"}) {
+    for (const char* name : {"PCR_SLICES", "PCR_LONG_MIN_BYTES", "PCR_REFINE_CTAS", "PCR_PACK_WARPS", "PCR_INDEX_CTAS", "PCR_LONG_CTAS"}) {
         const char* v = getenv(name);
         h = h * 1000003u + (v ? (uint32_t)atoi(v) + 1u : 0u);
     }
@@ -1309,6 +1311,20 @@ static bool pack_first_passes(const pcr_record* rec, const std::vector<int>& wav
     return warps > (uint64_t)rec->pack_warps * (uint64_t)rec->n_sms;
 }
 
+// Whether the long scans of a wave that are first passes (or sequential) get CTAs of four times as many warps: while
+// most of the machine is idle; beyond, the narrow ones do less in all.  Decode at k = 5 in us, narrow and wide, by CTAs
+// an SM: HAM-shaped images 2 242 and 184, 4.4 between 265 and 300
+// (contents that fall in quickly) or 356 and 300, 18 696 and 788; ImageNet-shaped 2.2 234 and 158, 8.6 233 and 233, 35 487
+// and 616; CelebA-shaped 2.2 163 and 116, 17 248 and 266.  Baseline: ImageNet-shaped 0.4 639 and 575, 1.7 706 and 747, HAM-shaped 0.4
+// 526 and 447, CelebA-shaped 0.4 471 and 483.
+static bool wide_long_scans(const pcr_record* rec, const std::vector<int>& wave, bool sequential, int k0, int k) {
+    uint64_t ctas = 0;
+    for (int s : wave)
+        if (s >= k0 && s < k && rec->script[s].Ah == 0)
+            for (int g = 0; g < rec->n_slices; ++g) ctas += rec->long_count[(size_t)g * rec->G + s];
+    return ctas * (sequential ? 4u : 1u) <= (uint64_t)rec->long_ctas * (uint64_t)rec->n_sms;
+}
+
 // Decode scans k0 .. k-1 on top of the state scans 0 .. k0-1 left behind (k0 = 0: from scratch),
 // then produce the pixels of fidelity k.
 static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream, const TensorArgs* targs = nullptr) {
@@ -1507,7 +1523,9 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
                 const int s0 = waves[w][0];      // the record's one scan
                 const uint32_t lc = (s0 >= k0 && s0 < k) ? rec->long_count[(size_t)g * G + s0] : 0u;
                 if (lc) {                                  // images whose scan is one long restart interval
-                    sequential_long_kernel<<<lc, 32 * kSeqLongWarps, 0, q>>>(P, rec->d_long + rec->long_begin[(size_t)g * G + s0], lc);
+                    const uint32_t* list = rec->d_long + rec->long_begin[(size_t)g * G + s0];
+                    if (wide_long_scans(rec, waves[w], true, k0, k)) sequential_long_kernel<kSeqLongWideWarps><<<lc, 32 * kSeqLongWideWarps, 0, q>>>(P, list, lc);
+                    else sequential_long_kernel<kSeqLongWarps><<<lc, 32 * kSeqLongWarps, 0, q>>>(P, list, lc);
                     ++g_launches;
                 }
                 return true;
@@ -1527,7 +1545,8 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
                     lc += rec->long_count[(size_t)g * G + s];
                 }
                 if (lc) {
-                    first_pass_long_kernel<<<lc, 32 * kLongWarps, 0, q>>>(P, rec->d_long + lb, lc);
+                    if (wide_long_scans(rec, waves[w], false, k0, k)) first_pass_long_kernel<kLongWideWarps><<<lc, 32 * kLongWideWarps, 0, q>>>(P, rec->d_long + lb, lc);
+                    else first_pass_long_kernel<kLongWarps><<<lc, 32 * kLongWarps, 0, q>>>(P, rec->d_long + lb, lc);
                     ++g_launches;
                 }
             }

@@ -67,6 +67,15 @@ __device__ __forceinline__ uint32_t long_entry(uint32_t tab, uint32_t win, int k
     const uint32_t e = lds16(tab + ((win >> (32 - kTabBits)) << 1));
     return e ? e : long_code(tab, win, kind);
 }
+// A position that a writing pass walks along: its 32 bits and the words behind them, requested ahead of their use.
+struct LongWalk {
+    const uint32_t* base;
+    uint32_t p, win, w1, w2;
+    __device__ __forceinline__ void load() { const uint32_t* w = base + (p >> 5); w1 = w[1]; w2 = w[2]; }
+    __device__ __forceinline__ LongWalk(const uint32_t* b, uint32_t at) : base(b), p(at) { win = __funnelshift_l(b[(at >> 5) + 1], b[at >> 5], at); load(); }
+    __device__ __forceinline__ uint32_t behind(uint32_t skip) const { return __funnelshift_l(__funnelshift_l(w2, w1, p), win, skip); }    // the 32 bits `skip` bits on
+    __device__ __forceinline__ void go(uint32_t skip, uint32_t next) { win = next; p += skip; load(); }
+};
 // number of blocks that an end of band covers
 __device__ __forceinline__ uint32_t eob_blocks(uint32_t e, uint32_t win) {
     const uint32_t r = (e >> 9) & 15u;
@@ -156,7 +165,8 @@ struct LongSpan {
     uint32_t begin, end, every;
     bool ok;
     // stage: shared memory for `room` words (the caller synchronises behind this)
-    template <uint32_t kThreads>
+    // kNarrow, kWords: threads that shorter scans are cut for, and the subsequence's words above which more threads are used
+    template <uint32_t kThreads, uint32_t kNarrow, uint32_t kWords>
     __device__ __forceinline__ void init(const Params& P, const ScanDesc& sd, uint32_t tid, uint32_t* stage, uint32_t room) {
         const uint32_t* segtab = P.seg_start + sd.seg_base;
         const uint32_t bstart = segtab[0], bend = segtab[1] - 2u;
@@ -164,11 +174,12 @@ struct LongSpan {
         base = origin = reinterpret_cast<const uint32_t*>(P.ubuf) + (bstart >> 2);
         lead = 8u * (bstart & 3u); endbit = ok ? lead + 8u * (bend - bstart) : lead;
         // whole words, at least eight of them: eight places at least 32 bits apart
-        const uint32_t words = max(8u, ((endbit + 31u) / 32u + kThreads - 1u) / kThreads);
+        // (shorter subsequences mean more rounds: how far a reading takes to fall in does not depend on them)
+        const uint32_t all = (endbit + 31u) / 32u, words = max(min(max(8u, (all + kNarrow - 1u) / kNarrow), kWords), (all + kThreads - 1u) / kThreads);
         const uint32_t len = 32u * words;
         every = len / kMarks;
         begin = min(max(tid * len, lead), endbit); end = min((tid + 1u) * len, endbit);
-        const uint32_t need = endbit / 32u + 3u;               // (a symbol may begin in the last bit)
+        const uint32_t need = endbit / 32u + 5u;               // (a symbol may begin in the last bit, and the words behind it are looked at)
         if (need <= room) {
             for (uint32_t i = tid; i < need; i += kThreads) stage[i] = __ldg(origin + i);
             base = stage;
@@ -229,24 +240,123 @@ __device__ __forceinline__ void search_all(const Steps& S, const LongSpan& L, ui
         uint32_t ppos = __shfl_up_sync(full, pos_x, 1), pst = __shfl_up_sync(full, st_x, 1);
         if (lane == 0 && wid > 0) { ppos = s_pos[wid - 1]; pst = s_state[wid - 1]; }
         ppos = min(ppos, L.endbit);
-        again = tid > 0 && (ppos != pos || pst != st);
+        // (behind the interval's end there is nothing to read and nobody to hand a state to: it would wander on a thread a round)
+        again = tid > 0 && L.begin < L.end && (ppos != pos || pst != st);
         if (again) { pos = ppos; st = pst; }
         if (!__syncthreads_or(again)) break;
     }
 }
 
+// A reading of a DC scan from some state on: blocks and differences per component summed.  An undefined code is passed over by
+// one bit.
+struct DcReading {
+    const DcSteps& S;
+    LongWalk w;
+    uint32_t st, tab, raw, nb;
+    int sum0, sum1, sum2;
+    __device__ __forceinline__ uint32_t table(uint32_t place) const { return S.tabs + ((S.tbits >> place) & 1u) * (uint32_t)sizeof(ScanTab); }
+    __device__ __forceinline__ DcReading(const DcSteps& s, const uint32_t* base, uint32_t pos, uint32_t place)
+        : S(s), w(base, pos), st(place), nb(0), sum0(0), sum1(0), sum2(0) { tab = table(st); raw = tab_entry(tab, w.win); }
+    // the symbols that start in front of `end`; j1, j2: the chroma blocks' places
+    __device__ __forceinline__ void to(uint32_t end, uint32_t j1, uint32_t j2) {
+#pragma unroll 1
+        while (w.p < end) {
+            const uint32_t e = raw ? raw : long_code(tab, w.win, kTabDc), skip = e ? e & 31u : 1u, win = w.win, next = w.behind(skip);
+            const uint32_t at = st;
+            st = e ? (st + 1u == S.bpm ? 0u : st + 1u) : st;
+            tab = table(st);
+            raw = tab_entry(tab, next);
+            w.go(skip, next);
+            const int d = e ? magnitude(win, skip, e >> 5) : 0;
+            sum0 += at < j1 ? d : 0; sum1 += at == j1 ? d : 0; sum2 += at == j2 ? d : 0;
+            nb += e ? 1u : 0u;
+        }
+    }
+};
+
+// Interleaved DC scans, wide CTAs.  Bit positions fall in within a few symbols, but a reading can go on for long with the
+// wrong place in the MCU (up to 23 rounds of the search above).  So every subsequence is read once from EVERY place, 512 bits ahead of
+// it, and one warp follows the true state through the readings; where none of them began its subsequence in the true state,
+// that subsequence is read once more.  On return a thread has the start of its subsequence (L.begin, L.end changed to match), its
+// blocks, the number of blocks and the sums of differences in front of it.
+template <uint32_t kThreads>
+__device__ __forceinline__ void dc_hypotheses(const DcSteps& S, LongSpan& L, uint32_t* mem, uint32_t j1, uint32_t j2, uint32_t& pos, uint32_t& st,
+                                              uint32_t& nb, uint32_t& n, int& pred0, int& pred1, int& pred2, uint32_t& all) {
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, H = S.bpm, subs = kThreads / H;
+    const unsigned full = 0xffffffffu;
+    const uint32_t len = 32u * max(8u, ((L.endbit + 31u) / 32u + subs - 1u) / subs);
+    auto begin_of = [&](uint32_t i) { return min(max(i * len, L.lead), L.endbit); };
+    auto end_of = [&](uint32_t i) { return min((i + 1u) * len, L.endbit); };
+    // by hypothesis and subsequence: the state it begins in (one number: equal ones within a subsequence are equal states), the one
+    // it ends in, blocks and sums; in the end, by subsequence, what the caller asks for
+    uint32_t* const key = mem;
+    uint32_t* const x_pos = mem + kThreads;
+    uint32_t* const x_st = mem + 2 * kThreads;
+    uint32_t* const x_nb = mem + 3 * kThreads;
+    int* const x_sum = reinterpret_cast<int*>(mem + 4 * kThreads);                 // [3][kThreads]
+    {
+        const uint32_t h = tid / subs, i = tid - h * subs, b = begin_of(i), e = end_of(i);
+        uint32_t k = 0xFFFFFFFFu;
+        if (h < H && b < e && (i != 0 || h == 0)) {
+            const uint32_t from = i == 0 ? L.lead : max(L.lead, b - min(b, 512u));
+            DcReading R(S, L.base, from, from == L.lead ? 0u : h);
+            R.to(b, j1, j2);
+            k = (R.w.p << 3) + R.st;
+            R.nb = 0; R.sum0 = R.sum1 = R.sum2 = 0;
+            R.to(e, j1, j2);
+            x_pos[tid] = R.w.p; x_st[tid] = R.st; x_nb[tid] = R.nb;
+            x_sum[tid] = R.sum0; x_sum[kThreads + tid] = R.sum1; x_sum[2 * kThreads + tid] = R.sum2;
+        }
+        key[tid] = k;
+    }
+    __syncthreads();
+    if (tid < 32u) {
+        uint32_t p = L.lead, s = 0, blocks = 0;
+        int a0 = 0, a1 = 0, a2 = 0;
+        for (uint32_t i = 0; i < subs; ++i) {
+            const uint32_t e = end_of(i), at = lane * subs + i;
+            const bool live = begin_of(i) < e;
+            const unsigned who = __ballot_sync(full, live && lane < H && key[at] == (p << 3) + s);
+            uint32_t q = 0, t = 0, c = 0;
+            int d0 = 0, d1 = 0, d2 = 0;
+            if (who) {
+                if (lane == (uint32_t)__ffs((int)who) - 1u) { q = x_pos[at]; t = x_st[at]; c = x_nb[at]; d0 = x_sum[at]; d1 = x_sum[kThreads + at]; d2 = x_sum[2 * kThreads + at]; }
+            } else if (live && lane == 0) {
+                DcReading R(S, L.base, p, s);
+                R.to(e, j1, j2);
+                q = R.w.p; t = R.st; c = R.nb; d0 = R.sum0; d1 = R.sum1; d2 = R.sum2;
+            }
+            const int src = who ? __ffs((int)who) - 1 : 0;
+            q = __shfl_sync(full, q, src); t = __shfl_sync(full, t, src); c = __shfl_sync(full, c, src);
+            d0 = __shfl_sync(full, d0, src); d1 = __shfl_sync(full, d1, src); d2 = __shfl_sync(full, d2, src);
+            __syncwarp(full);
+            if (lane == 0) { key[i] = p; x_pos[i] = s; x_nb[i] = blocks; x_sum[i] = a0; x_sum[kThreads + i] = a1; x_sum[2 * kThreads + i] = a2; }
+            if (live) { p = q; s = t; blocks += c; a0 += d0; a1 += d1; a2 += d2; }
+        }
+        if (lane == 0) x_st[0] = blocks;
+    }
+    __syncthreads();
+    const bool mine = tid < subs;
+    L.begin = mine ? begin_of(tid) : L.endbit; L.end = mine ? end_of(tid) : 0u;
+    pos = mine ? key[tid] : L.endbit; st = mine ? x_pos[tid] : 0u; n = mine ? x_nb[tid] : 0u;
+    pred0 = mine ? x_sum[tid] : 0; pred1 = mine ? x_sum[kThreads + tid] : 0; pred2 = mine ? x_sum[2 * kThreads + tid] : 0;
+    all = x_st[0];
+    nb = mine ? (tid + 1u < subs ? x_nb[tid + 1u] : all) - n : 0u;
+}
+
 // ---------------------------------------------------------------------------------------
-// First passes: one CTA of kLongWarps warps per listed (scan, image) whose scan is one restart interval.
+// First passes: one CTA of kWarps warps per listed (scan, image) whose scan is one restart interval.
 // Bound by the chain of one subsequence times the rounds until the slowest scan of the record has fallen in: a launch
-// waits for that scan.  The stream and the tables are in shared memory because every step of the search depends on
-// them.  256 HAM-shaped images at k = 5, decode: 570 us on average over six records when every round read its whole
-// subsequence from global memory, 350 us now; two, three or four warps a scan are equal within the noise.
+// waits for that scan; then by the pass that writes.  The stream and the tables are in shared memory because every step of the
+// search depends on them.  256 HAM-shaped images at k = 5, decode: 570 us on average over six records when every round read its whole
+// subsequence from global memory, 350 us with marks, 325 us now: four times the warps where most of the machine is idle, interleaved DC
+// scans read from every place of the MCU at once (dc_hypotheses; the search took up to 23 rounds, most of the kernel's time),
+// writing passes of straight-line steps, no rounds that only hand a state on behind the interval's end (up to 56).  64
+// ImageNet-shaped images 234 -> 158 us, 64 CelebA-shaped 171 -> 116 us.
 // ---------------------------------------------------------------------------------------
-#ifndef PCR_LONG_WARPS
-#define PCR_LONG_WARPS 2
-#endif
-constexpr int kLongWarps = PCR_LONG_WARPS;
-constexpr uint32_t kLongStage = 2048;         // words of a scan that are staged: 8 KB, a 600x450 image's scans have up to 6
+constexpr int kLongWarps = 2, kLongWideWarps = 8;
+// words of a scan that are staged: 8 KB, a 600x450 image's scans have up to 6 (of the luminance 12); 24 KB of a wide CTA
+template <int kWarps> __host__ __device__ constexpr uint32_t long_stage() { return kWarps == kLongWarps ? 2048 : 6144; }
 
 // Copies n of the (scan, image)'s tables to shared memory; the CTA's threads together.
 __device__ __forceinline__ void load_tabs(uint32_t dst, const ScanTab* src, int n, int tid, int threads) {
@@ -254,8 +364,10 @@ __device__ __forceinline__ void load_tabs(uint32_t dst, const ScanTab* src, int 
     for (int i = tid; i < n * (int)(sizeof(ScanTab) / 16); i += threads) sts128(dst + 16u * i, __ldg(a + i));
 }
 
-__global__ void __launch_bounds__(32 * kLongWarps) first_pass_long_kernel(Params P, const uint32_t* __restrict__ list, uint32_t count) {
-    constexpr int kWarps = kLongWarps, kThreads = 32 * kWarps;
+template <int kWarps>
+__global__ void __launch_bounds__(32 * kWarps) first_pass_long_kernel(Params P, const uint32_t* __restrict__ list, uint32_t count) {
+    constexpr int kThreads = 32 * kWarps;
+    constexpr uint32_t kLongStage = long_stage<kWarps>();
     __shared__ __align__(16) uint8_t s_tabs[2 * sizeof(ScanTab)];
     __shared__ uint32_t s_stage[kLongStage];
     __shared__ uint32_t s_marks[kMarks * kThreads];
@@ -277,7 +389,7 @@ __global__ void __launch_bounds__(32 * kLongWarps) first_pass_long_kernel(Params
     const uint32_t tabs = (uint32_t)__cvta_generic_to_shared(s_tabs);
     const bool second = dc && sd.tab_off[1];
     LongSpan L;
-    L.init<kThreads>(P, sd, (uint32_t)tid, s_stage, kLongStage);
+    L.init<kThreads, 32 * kLongWarps, 16>(P, sd, (uint32_t)tid, s_stage, kLongStage);
     load_tabs(tabs, P.tabs + ax.tab0 + (uint32_t)img * (uint32_t)ax.ntab, second ? 2 : 1, tid, kThreads);
     __syncthreads();
     if (!L.ok) {
@@ -291,22 +403,22 @@ __global__ void __launch_bounds__(32 * kLongWarps) first_pass_long_kernel(Params
         DcSteps S;
         S.base = L.base; S.tabs = tabs; S.bpm = bpm; S.tbits = 0;
         for (uint32_t j = 0; j < bpm; ++j) S.tbits |= ((sd.slots >> (2u * (inter && j >= ny ? j - ny + 1u : 0u))) & 1u) << j;
-        search_all<DcSteps, kWarps>(S, L, s_marks, s_pos, s_state, 0u, 512u, pos, st);
-        int sum0 = 0, sum1 = 0, sum2 = 0;
         const uint32_t j1 = inter ? ny : 6u, j2 = inter ? ny + 1u : 6u;          // the chroma blocks' places
-        for (uint32_t p = pos, j = st; p < L.end;) {
-            const uint32_t e = S.entry(p, j);
-            const int d = magnitude(long_window(L.base, p), e & 31u, e >> 5);          // (no symbol: 0)
-            sum0 += j < j1 ? d : 0; sum1 += j == j1 ? d : 0; sum2 += j == j2 ? d : 0;
-            nb += e ? 1u : 0u;
-            if (e) S.advance(e, j);
-            p += e ? e & 31u : 1u;
+        uint32_t n;
+        int pred0, pred1, pred2;
+        if (kWarps != kLongWarps && bpm > 1u) {
+            dc_hypotheses<32 * kWarps>(S, L, s_marks, j1, j2, pos, st, nb, n, pred0, pred1, pred2, all);
+        } else {
+            search_all<DcSteps, kWarps>(S, L, s_marks, s_pos, s_state, 0u, 512u, pos, st);
+            int sum0 = 0, sum1 = 0, sum2 = 0, t;
+            DcReading R(S, L.base, pos, st);
+            R.to(L.end, j1, j2);
+            nb = R.nb; sum0 = R.sum0; sum1 = R.sum1; sum2 = R.sum2;
+            n = cta_exclusive_sum(nb, s_u, wid, lane, kWarps, all);
+            pred0 = cta_exclusive_sum(sum0, s_i, wid, lane, kWarps, t);
+            pred1 = cta_exclusive_sum(sum1, s_i, wid, lane, kWarps, t);
+            pred2 = cta_exclusive_sum(sum2, s_i, wid, lane, kWarps, t);
         }
-        int t;
-        uint32_t n = cta_exclusive_sum(nb, s_u, wid, lane, kWarps, all);
-        int pred0 = cta_exclusive_sum(sum0, s_i, wid, lane, kWarps, t);
-        int pred1 = cta_exclusive_sum(sum1, s_i, wid, lane, kWarps, t);
-        int pred2 = cta_exclusive_sum(sum2, s_i, wid, lane, kWarps, t);
         const uint32_t n1 = total * bpm;
         n = min(n, n1);
         // the place inside the MCU follows from the block number (equal to the handed-on state unless
@@ -360,38 +472,45 @@ __global__ void __launch_bounds__(32 * kLongWarps) first_pass_long_kernel(Params
         int16_t* const vals = P.vals + 16ll * (L.origin - reinterpret_cast<const uint32_t*>(P.ubuf));
         uint64_t* const auxp = P.aux + ax.base + g.loff[c0] * ax.stride;
         const bool lists = ax.stride == 2u;                    // the band reaches beyond position 7
-        uint32_t k = st, M0 = 0, M1 = 0, lim = L.end;
+        // (A step is one straight line that every lane of the warp walks, as in entropy_kernel: an entry of zero moves nothing on.)
+        uint32_t k = st, M0 = 0, M1 = 0, lim = m < total ? L.end : 0u;      // lim: the first bit at which no symbol is read
         bool own = k == Ss;
-        int16_t* vp = vals + ((pos + 1u) >> 1);
-        int16_t* vb = vp;
+        uint32_t nv = (pos + 1u) >> 1, nv0 = nv;               // next value, the block's first one
         uint32_t bcol = m % mcu_w, bi = (m / mcu_w) * bw + bcol;
-        for (uint32_t p = pos; p < lim && m < total;) {
-            const uint32_t win = long_window(L.base, p), e = S.entry(p, k);
-            const uint32_t skip = e & 31u, sz = (e >> 5) & 15u;
-            p += skip;
-            k += (e >> 9) - 1u;                                // position of the coefficient (of an end of band: beyond every one)
-            const bool eob = (e & kEntEob) != 0, coef = sz && own;
-            if (e == 0 || (sz && k > Se)) { bad = true; break; }
-            const int val = magnitude(win, skip, sz) << sc.Al;
-            if (coef && k < 8u) headp[8u * (uint64_t)bi + k] = (int16_t)val;
-            if (coef && k >= 8u) *vp = (int16_t)val;
-            vp += coef && k >= 8u ? 1 : 0;
-            M0 |= shl0(coef ? 1u : 0u, k); M1 |= shl0(coef ? 1u : 0u, k - 32u);
-            ++k;
-            if (own) lim = L.endbit;
-            if (eob || k > Se) {                               // the block ends, an end-of-band run skips more
-                if (M0 | M1) {
-                    if (lists) *reinterpret_cast<uint4*>(auxp + (uint64_t)bi * 2) = value_record(M0, M1, vb);
-                    else *reinterpret_cast<uint2*>(auxp + bi) = make_uint2(M0, M1);
-                }
-                k = Ss; M0 = 0; M1 = 0; lim = L.end;
-                if (!own) vp = vals + ((p + 1u) >> 1);         // this thread's values begin where its first block does
-                vb = vp;
-                own = true;
-                const uint32_t adv = eob ? eob_blocks(e, win) : 1u;
-                if (adv >= total - m) break;
+        LongWalk w(L.base, pos);
+        uint32_t raw = tab_entry(S.tabs, w.win);
+        while (__any_sync(0xffffffffu, w.p < lim)) {
+#pragma unroll 4
+            for (int q = 0; q < 8; ++q) {
+                const uint32_t e = w.p < lim ? raw : 0u, skip = e & 31u, sz = (e >> 5) & 15u, win = w.win, next = w.behind(skip);
+                raw = tab_entry(S.tabs, next);
+                w.go(skip, next);
+                k += e >> 9;                                   // behind the coefficient (an end of band: beyond every position)
+                const uint32_t at = k - 1u;
+                const bool over = sz && k > Se + 1u, coef = sz && own && !over, far = coef && k > 8u, end = k > Se;
+                const int val = magnitude(win, skip, sz) << sc.Al;
+                stg16_if(coef && !far, headp + 8u * (uint64_t)bi + at, (uint32_t)val);
+                stg16_if(far, vals + nv, (uint32_t)val);
+                nv += far ? 1u : 0u;
+                M0 |= shl0(coef ? 1u : 0u, at); M1 |= shl0(coef ? 1u : 0u, at - 32u);
+                const bool some = end && (M0 | M1) != 0;
+                if (lists) stg128_if(some, auxp + (uint64_t)bi * 2, value_record(M0, M1, vals + nv0));
+                else stg64_if(some, auxp + bi, M0, M1);
+                lim = own && e ? L.endbit : lim;
+                // the block ends, an end-of-band run skips more
+                const uint32_t r = (e >> 9) & 15u, adv = end ? (e & kEntEob ? __funnelshift_l(shl0(win, skip - r), 1u, r) : 1u) : 0u;   // 2^r + the r bits that end the symbol
+                lim = end ? (adv >= total - m ? 0u : L.end) : lim;
+                nv = end && !own ? (w.p + 1u) >> 1 : nv;       // this thread's values begin where its first block does
+                nv0 = end ? nv : nv0;
+                k = end ? Ss : k; own = own || end;
+                M0 = end ? 0u : M0; M1 = end ? 0u : M1;
+                if (over) { bad = true; lim = 0; }
                 m += adv; bcol += adv; bi += adv;
                 if (bcol >= mcu_w) { bcol = m % mcu_w; bi = (m / mcu_w) * bw + bcol; }
+            }
+            if (raw == 0 && w.p < lim) {                       // (taken by the next step)
+                raw = long_code(S.tabs, w.win, kTabAcFirst);
+                if (raw == 0) { bad = true; lim = 0; }
             }
         }
     }
@@ -402,19 +521,18 @@ __global__ void __launch_bounds__(32 * kLongWarps) first_pass_long_kernel(Params
 // A sequential (baseline) scan that is one restart interval: one CTA of kSeqLongWarps warps per listed image.  Bound like
 // the kernel above.
 // ---------------------------------------------------------------------------------------
-#ifndef PCR_SEQ_LONG_WARPS
-#define PCR_SEQ_LONG_WARPS 4
-#endif
-constexpr int kSeqLongWarps = PCR_SEQ_LONG_WARPS;
-constexpr uint32_t kSeqLongStage = 6144;      // 24 KB
+constexpr int kSeqLongWarps = 4, kSeqLongWideWarps = 16;
+template <int kWarps> __host__ __device__ constexpr uint32_t seq_long_stage() { return kWarps == kSeqLongWarps ? 6144 : 4096; }      // words
 
-__global__ void __launch_bounds__(32 * kSeqLongWarps) sequential_long_kernel(Params P, const uint32_t* __restrict__ list, uint32_t count) {
-    constexpr int kThreads = 32 * kSeqLongWarps;
+template <int kWarps>
+__global__ void __launch_bounds__(32 * kWarps) sequential_long_kernel(Params P, const uint32_t* __restrict__ list, uint32_t count) {
+    constexpr int kThreads = 32 * kWarps;
+    constexpr uint32_t kSeqLongStage = seq_long_stage<kWarps>();
     __shared__ __align__(16) uint8_t s_tabs[4 * sizeof(ScanTab)];
     __shared__ uint32_t s_stage[kSeqLongStage];
     __shared__ uint32_t s_marks[kMarks * kThreads];
-    __shared__ uint32_t s_pos[kSeqLongWarps], s_state[kSeqLongWarps], s_u[kSeqLongWarps];
-    __shared__ int s_i[kSeqLongWarps];
+    __shared__ uint32_t s_pos[kWarps], s_state[kWarps], s_u[kWarps];
+    __shared__ int s_i[kWarps];
     const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
     const uint32_t it = blockIdx.x;
     if (it >= count) return;                                   // whole CTA
@@ -433,7 +551,7 @@ __global__ void __launch_bounds__(32 * kSeqLongWarps) sequential_long_kernel(Par
     }
     load_tabs(S.tabs, P.tabs + ax.tab0 + 4u * (uint32_t)img, 4, tid, kThreads);
     LongSpan L;
-    L.init<kThreads>(P, sd, (uint32_t)tid, s_stage, kSeqLongStage);
+    L.init<kThreads, 32 * kSeqLongWarps, 32>(P, sd, (uint32_t)tid, s_stage, kSeqLongStage);
     S.base = L.base;
     __syncthreads();
     if (!L.ok) {
@@ -442,7 +560,7 @@ __global__ void __launch_bounds__(32 * kSeqLongWarps) sequential_long_kernel(Par
     }
     bool bad = false;
     uint32_t pos, st, all, nb = 0;
-    search_all<SeqSteps, kSeqLongWarps>(S, L, s_marks, s_pos, s_state, 0u, 0u, pos, st);
+    search_all<SeqSteps, kWarps>(S, L, s_marks, s_pos, s_state, 0u, 0u, pos, st);
     int sum0 = 0, sum1 = 0, sum2 = 0;
     for (uint32_t p = pos, q = st; p < L.end;) {
         const uint32_t e = S.entry(p, q), j = q >> 6;
@@ -452,10 +570,10 @@ __global__ void __launch_bounds__(32 * kSeqLongWarps) sequential_long_kernel(Par
         p += e ? e & 31u : 1u;
     }
     int t;
-    uint32_t n = cta_exclusive_sum(nb, s_u, wid, lane, kSeqLongWarps, all);
-    int pred0 = cta_exclusive_sum(sum0, s_i, wid, lane, kSeqLongWarps, t);
-    int pred1 = cta_exclusive_sum(sum1, s_i, wid, lane, kSeqLongWarps, t);
-    int pred2 = cta_exclusive_sum(sum2, s_i, wid, lane, kSeqLongWarps, t);
+    uint32_t n = cta_exclusive_sum(nb, s_u, wid, lane, kWarps, all);
+    int pred0 = cta_exclusive_sum(sum0, s_i, wid, lane, kWarps, t);
+    int pred1 = cta_exclusive_sum(sum1, s_i, wid, lane, kWarps, t);
+    int pred2 = cta_exclusive_sum(sum2, s_i, wid, lane, kWarps, t);
     const uint32_t n1 = total * bpm;
     n = min(n, n1);
     // (as for the DC scans above)
@@ -466,45 +584,52 @@ __global__ void __launch_bounds__(32 * kSeqLongWarps) sequential_long_kernel(Par
     int16_t* const headp = P.head + g.coff[0] * 8;
     int16_t* const vals = P.vals + 16ll * (L.origin - reinterpret_cast<const uint32_t*>(P.ubuf));
     uint64_t* const auxp = P.aux + ax.base + 2 * g.coff[0];
-    uint32_t j = n % bpm, k = st & 63u, m = n / bpm, mcol = m % mcu_w, M0 = 0, M1 = 0, lim = L.end;
+    uint32_t j = n % bpm, k = st & 63u, m = n / bpm, mcol = m % mcu_w, M0 = 0, M1 = 0, lim = n < n1 ? L.end : 0u;
     uint32_t yb = vs * (m / mcu_w) * g.bw[0] + hs * mcol;
     const uint32_t wrap = (vs - 1u) * g.bw[0];
     bool own = k == 0;
-    int16_t* vp = vals + ((pos + 1u) >> 1);
-    int16_t* vb = vp;
-    for (uint32_t p = pos; p < lim && n < n1;) {
-        const uint32_t win = long_window(L.base, p), e = S.entry(p, (j << 6) + k);
-        const uint32_t skip = e & 31u, sz = (e >> 5) & 15u;
-        const uint32_t blk = j < ny ? yb + (j >> (hs - 1u)) * g.bw[0] + (j & (hs - 1u)) : (ny + j - ny) * total + m;
-        p += skip;
-        const bool is_dc = k == 0;
-        k += ((e >> 9) & 31u) - 1u;
-        if (e == 0 || (sz && k > 63u)) { bad = true; break; }
-        int v = magnitude(win, skip, sz);
-        if (is_dc) {
-            v += j < ny ? pred0 : (j == ny ? pred1 : pred2);
-            if (j < ny) pred0 = v; else if (j == ny) pred1 = v; else pred2 = v;
-            dcp[blk] = (int16_t)v;
+    uint32_t nv = (pos + 1u) >> 1, nv0 = nv;                   // next value, the block's first one
+    LongWalk w(L.base, pos);
+    auto dc_tab = [&](uint32_t place) { return S.tabs + ((S.tdc >> place) & 1u) * (uint32_t)sizeof(ScanTab); };
+    auto ac_tab = [&](uint32_t place) { return S.tabs + (2u + ((S.tac >> place) & 1u)) * (uint32_t)sizeof(ScanTab); };
+    uint32_t raw = tab_entry(k ? ac_tab(j) : dc_tab(j), w.win);
+    while (__any_sync(0xffffffffu, w.p < lim)) {
+#pragma unroll 4
+        for (int q = 0; q < 8; ++q) {
+            const uint32_t e = w.p < lim ? raw : 0u, skip = e & 31u, sz = (e >> 5) & 15u, win = w.win, next = w.behind(skip);
+            const bool is_dc = k == 0;
+            const uint32_t kk = k + (e >> 9), after = j + 1u == bpm ? 0u : j + 1u;     // (an end of block goes beyond 63)
+            const bool over = sz && kk > 64u && !is_dc, end = kk > 63u;
+            raw = e ? tab_entry(end ? dc_tab(after) : ac_tab(j), next) : raw;
+            w.go(skip, next);
+            const uint32_t blk = j < ny ? yb + (j >> (hs - 1u)) * g.bw[0] + (j & (hs - 1u)) : j * total + m;
+            int v = magnitude(win, skip, sz);
+            v += is_dc ? (j < ny ? pred0 : (j == ny ? pred1 : pred2)) : 0;
+            const bool dc_now = is_dc && e;
+            pred0 = dc_now && j < ny ? v : pred0; pred1 = dc_now && j == ny ? v : pred1; pred2 = dc_now && j > ny ? v : pred2;
+            stg16_if(dc_now, dcp + blk, (uint32_t)v);
+            const bool coef = sz && own && !is_dc && !over, far = coef && kk > 8u;
+            stg16_if(coef && !far, headp + 8ull * blk + kk - 1u, (uint32_t)v);
+            stg16_if(far, vals + nv, (uint32_t)v);
+            nv += far ? 1u : 0u;
+            M0 |= shl0(far ? 1u : 0u, kk - 1u); M1 |= shl0(far ? 1u : 0u, kk - 33u);
+            stg128_if(end && (M0 | M1) != 0, auxp + 2ull * blk, value_record(M0, M1, vals + nv0));
+            lim = own && e ? L.endbit : lim;
+            n += end ? 1u : 0u;
+            lim = end ? (n < n1 ? L.end : 0u) : lim;
+            nv = end && !own ? (w.p + 1u) >> 1 : nv;
+            nv0 = end ? nv : nv0;
+            k = end ? 0u : kk; own = own || end;
+            M0 = end ? 0u : M0; M1 = end ? 0u : M1;
+            if (over) { bad = true; lim = 0; }
+            const bool mcu = end && after == 0;
+            j = end ? after : j;
+            m += mcu ? 1u : 0u; mcol += mcu ? 1u : 0u; yb += mcu ? hs : 0u;
+            if (mcol == mcu_w) { mcol = 0; yb += wrap; }
         }
-        const bool coef = sz && own && !is_dc;
-        if (coef && k < 8u) headp[8u * (uint64_t)blk + k] = (int16_t)v;
-        if (coef && k >= 8u) *vp = (int16_t)v;
-        vp += coef && k >= 8u ? 1 : 0;
-        M0 |= shl0(coef && k >= 8u ? 1u : 0u, k); M1 |= shl0(coef ? 1u : 0u, k - 32u);
-        ++k;
-        if (own) lim = L.endbit;
-        if ((e & kEntEob) || k > 63u) {                        // block finished
-            if (M0 | M1) *reinterpret_cast<uint4*>(auxp + 2ull * blk) = value_record(M0, M1, vb);
-            k = 0; M0 = 0; M1 = 0; lim = L.end;
-            if (!own) vp = vals + ((p + 1u) >> 1);
-            vb = vp;
-            own = true;
-            ++n;
-            if (++j == bpm) {
-                j = 0; ++m;
-                yb += hs;
-                if (++mcol == mcu_w) { mcol = 0; yb += wrap; }
-            }
+        if (raw == 0 && w.p < lim) {                           // (taken by the next step)
+            raw = long_code(k ? ac_tab(j) : dc_tab(j), w.win, k ? kTabAcSeq : kTabDcSeq);
+            if (raw == 0) { bad = true; lim = 0; }
         }
     }
     if (__syncthreads_or(bad) && tid == 0) atomicMin(&P.status[img], kErrCorrupt);
