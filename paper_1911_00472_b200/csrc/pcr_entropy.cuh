@@ -16,9 +16,11 @@
 // positions, their signs} as side data, which the pixel kernel applies when it expands the block.
 //
 // (AC refinements of records that do not fill the machine: pcr_refine.cuh.)
-// Bound by the latency of a lane's chain: about 155 warp instructions a refinement step (276 with masks searched for
-// the r-th zero and a bit reader that carries its state), at the issue rate that the resident warps allow.
-// 1024 ImageNet-shaped images at k = 10: the three waves 217 + 332 + 511 us before, 176 + 220 + 245 us now.
+// Bound by the latency of a lane's chain and, with the machine full, by the issue rate that the resident warps allow: a
+// refinement step is about 155 warp instructions (276 with masks searched for the r-th zero and a bit reader that carries its
+// state) in one straight line; with branches for block ends and rare cases the two refinement waves of 1024 ImageNet-shaped images
+// took 226 + 270 us, now 183 + 216.  (Registers held down to 112 for a sixth CTA an SM: 255 + 254.)  The three waves were 217 + 332 + 511
+// us with coefficient planes; now 165 + 183 + 216.
 #pragma once
 #include <cuda_runtime.h>
 #include <stddef.h>
@@ -419,6 +421,9 @@ __device__ __forceinline__ uint32_t lds8(uint32_t a) { uint32_t v; asm volatile(
 __device__ __forceinline__ void sts16_if(bool on, uint32_t a, uint32_t v) {
     asm volatile("{ .reg .pred p; setp.ne.u32 p, %2, 0; @p st.shared.u16 [%0], %1; }" : : "r"(a), "h"((uint16_t)v), "r"((uint32_t)on) : "memory");
 }
+__device__ __forceinline__ void lds128_if(bool on, uint32_t a, uint4& v) {
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %5, 0; @p ld.shared.v4.u32 {%0, %1, %2, %3}, [%4]; }" : "+r"(v.x), "+r"(v.y), "+r"(v.z), "+r"(v.w) : "r"(a), "r"((uint32_t)on) : "memory");
+}
 __device__ __forceinline__ void sts32_if(bool on, uint32_t a, uint32_t v) {
     asm volatile("{ .reg .pred p; setp.ne.u32 p, %2, 0; @p st.shared.u32 [%0], %1; }" : : "r"(a), "r"(v), "r"((uint32_t)on) : "memory");
 }
@@ -684,7 +689,7 @@ __device__ __forceinline__ void dc_refine_image(const Params& P, int s, int img,
 // the load/store units' time, 197 us against 172 (before: 206).  64 images 66 -> 44 us.  DC alone of 1024 images 55 -> 40 us (pairs
 // of luminance blocks stored together, MCUs without a branch inside).
 template <bool kRoi, bool kRefine, bool kPack>
-__global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, ItemRuns runs) {
+__global__ void __launch_bounds__(32 * kEntropyWarps, kRefine ? 4 : 1) entropy_kernel(Params P, ItemRuns runs) {
     extern __shared__ __align__(16) uint8_t s_entropy[];
     __shared__ __align__(16) uint8_t s_sel[kRefine ? sizeof(SelectTable) : 16];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1028,37 +1033,73 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, I
                 // a step reads the window at its start and, at most 31 bits on, two words (three for more than
                 // 32 correction bits)
                 uint32_t stop = done || m >= hm ? 0u : min(br.ring_stop(4), br.limit + 1u);
+                W.load(br.pos);
+                uint32_t win = W.window(br.pos), raw = tab_entry(tab, win);
+                bool late = false, rare = false;               // the step before passed more than 31 bits; a long code, or more than 32 correction bits
+                auto target = [&](uint32_t e, uint32_t nz, uint32_t& T, uint32_t& k, uint32_t& n) {
+                    T = min(zi + (e >> 8), nz);                // the rank of the target; nz = behind the band
+                    const uint32_t tt = T * 0x01010101u + 0x80808080u;
+                    const uint32_t j = (uint32_t)(__popc((tt - Z.z) & 0x80808080u) + __popc((tt - Z.w) & 0x80808080u));
+                    const uint32_t zb = __byte_perm(Z.x, Z.y, j) & 255u, cj = prmt(Z.z, Z.w, j - 1u) & 255u;   // (j = 0: no byte below, the selector's sign form gives 0)
+                    k = 8u * j + lds8(sel + 8u * zb + T - cj);
+                    k = T < nz ? k : Se + 1u;
+                    n = k - T - ep;                            // correction bits behind the symbol
+                };
+                // what a symbol does once it is known how many correction bits it has
+                auto apply = [&](bool act, uint32_t e, uint32_t nz, uint32_t T, uint32_t k, uint32_t n) {
+                    const uint32_t skip = e & 31u, d = act ? skip + n : 0u;
+                    const uint32_t isnew = act && T < nz ? (e >> 5) & 1u : 0u, plus = isnew & shr0(win, 32u - skip);
+                    N0 |= shl0(isnew, k); N1 |= shl0(isnew, k - 32u);
+                    G0 |= shl0(plus, k); G1 |= shl0(plus, k - 32u);
+                    const bool end = act && k >= Se;           // block finished
+                    const uint32_t x = (e >> 8) & 15u, run = __funnelshift_l(shl0(win, skip - x), 1u, x);   // of an end of band: blocks it covers (2^x + the x bits that end it)
+                    const uint32_t left = (eobrun ? eobrun : (e >= kEntEobRefine ? run : 1u)) - 1u;
+                    uint64_t* const o = outp + (uint64_t)bi * 4;
+                    stg128_if(end, o, make_uint4((~Z.x & band0) | N0, (~Z.y & band1) | N1, s0, s1));
+                    stg128_if(end, o + 2, make_uint4(N0, N1, G0, G1));
+                    eobrun = end ? left : eobrun;
+                    m += end ? 1u : 0u;
+                    const bool row = end && m == wrap_m;
+                    bi += row ? wrap : (end ? 1u : 0u); wrap_m += row ? mcu_w : 0u;
+                    zi = end ? 0u : (act ? T + 1u : zi); ep = end ? Ss : (act ? ep + n : ep);
+                    s0 = end ? 0u : s0; s1 = end ? 0u : s1; N0 = end ? 0u : N0; N1 = end ? 0u : N1; G0 = end ? 0u : G0; G1 = end ? 0u : G1;
+                    lds128_if(end, queue + ((m & (kMaskQueue - 1)) << 9), Z);      // (not read when the queue is empty)
+                    stop = m < hm ? stop : 0u;                 // also at the interval's end: hm is at most m1
+                    return d;
+                };
+                // A step is one straight line that every lane walks; what is rare waits for the end of eight.
 #pragma unroll 1
-                for (int t = 0; t < kDecodeSteps; ++t) {
-                    if (br.pos < stop) {
-                        const uint32_t win = br.window(br.pos), nz = Z.w >> 24;
-                        uint32_t e = lds16(tab + ((win >> (32 - kTabBits)) << 1));
-                        e = eobrun ? kEntEobRefine : e;                // this block lies inside an end-of-band run
+                for (int t = 0; t < kDecodeSteps; t += 8) {
+#pragma unroll 1
+                    for (int q = 0; q < 8; ++q) {
+                        const bool wanted = br.pos < stop && !late && !rare;
+                        const uint32_t nz = Z.w >> 24, e = eobrun ? kEntEobRefine : raw;    // (this block lies inside an end-of-band run)
+                        const uint32_t behind = W.behind(br.pos);
+                        if (late) win = W.window(br.pos);
                         uint32_t T, k, n;
-                        auto target = [&]() {                          // -> T, k, n; ep moves on
-                            T = min(zi + (e >> 8), nz);                // the rank of the target; nz = behind the band
-                            const uint32_t tt = T * 0x01010101u + 0x80808080u;
-                            const uint32_t j = (uint32_t)(__popc((tt - Z.z) & 0x80808080u) + __popc((tt - Z.w) & 0x80808080u));
-                            const uint32_t zb = __byte_perm(Z.x, Z.y, j) & 255u, cj = prmt(Z.z, Z.w, j - 1u) & 255u;   // (j = 0: no byte below, the selector's sign form gives 0)
-                            k = 8u * j + lds8(sel + 8u * zb + T - cj);
-                            k = T < nz ? k : Se + 1u;
-                            n = k - T - ep;                            // correction bits behind the symbol
-                            ep += n;
-                        };
-                        target();
-                        uint32_t skip = e & 31u;
-                        s1 = __funnelshift_lc(s0, s1, n);
-                        s0 = shl0(s0, n) | shr0(shl0(win, skip), 32u - n);
-                        if (e == 0 || skip + n > 32u) {                // rare: a long code, or bits beyond the window
-                            s0 = __funnelshift_rc(s0, s1, n);          // (taken back: n > 32 left the low word in s1)
-                            s1 = shr0(s1, n);
-                            if (e == 0) {
-                                ep -= n;
-                                e = long_code(tab, win, kTabAcRefine);
-                                target();
-                                skip = e & 31u;
-                            }
-                            const uint32_t at = br.pos + skip, cw = br.window(at);
+                        target(e, nz, T, k, n);
+                        const bool act = wanted && e != 0 && n <= 32u;
+                        rare = rare || (wanted && !act);
+                        const uint32_t bits = act ? n : 0u, corr = __funnelshift_l(behind, win, e & 31u);
+                        s1 = __funnelshift_lc(s0, s1, bits);
+                        s0 = shl0(s0, bits) | shr0(corr, 32u - bits);
+                        const uint32_t d = apply(act, e, nz, T, k, n);
+                        win = __funnelshift_l(behind, win, d);
+                        raw = tab_entry(tab, win);
+                        br.pos += d;
+                        late = d > 31u;
+                        W.load(br.pos);
+                    }
+                    if (late) { win = W.window(br.pos); raw = tab_entry(tab, win); late = false; }
+                    if (rare) {
+                        rare = false;
+                        const uint32_t nz = Z.w >> 24;
+                        uint32_t e = eobrun ? kEntEobRefine : raw, T, k, n;
+                        if (e == 0) e = long_code(tab, win, kTabAcRefine);
+                        target(e, nz, T, k, n);
+                        if (e == 0) { bad = true; stop = 0; }  // no such symbol: the lane ends here
+                        else {
+                            const uint32_t at = br.pos + (e & 31u), cw = br.window(at);
                             if (n > 32u) {
                                 s1 = (cw >> (64u - n)) | (s0 << (n - 32u));
                                 s0 = __funnelshift_l(br.window(at + 32u), cw, n - 32u);
@@ -1066,25 +1107,9 @@ __global__ void __launch_bounds__(32 * kEntropyWarps) entropy_kernel(Params P, I
                                 s1 = __funnelshift_lc(s0, s1, n);
                                 s0 = shl0(s0, n) | shr0(cw, 32u - n);
                             }
-                            if (e == 0) { bad = true; stop = 0; k = 0; }   // no such symbol: the lane ends here
-                        }
-                        br.pos += skip + n;
-                        zi = T + 1u;
-                        const uint32_t x = (e >> 8) & 15u;
-                        const uint32_t run = shl0(1u, x) + shr0(shl0(win, skip - x), 32u - x) - 1u;   // of an end of band: blocks behind this one
-                        eobrun = e > kEntEobRefine + 0xFFu ? run : eobrun - (eobrun ? 1u : 0u);
-                        const uint32_t isnew = T < nz ? (e >> 5) & 1u : 0u, plus = isnew & shr0(win, 32u - skip);
-                        N0 |= shl0(isnew, k); N1 |= shl0(isnew, k - 32u);
-                        G0 |= shl0(plus, k); G1 |= shl0(plus, k - 32u);
-                        if (k >= Se) {                                 // block finished
-                            uint4* o = reinterpret_cast<uint4*>(outp + (uint64_t)bi * 4);
-                            o[0] = make_uint4((~Z.x & band0) | N0, (~Z.y & band1) | N1, s0, s1);
-                            o[1] = make_uint4(N0, N1, G0, G1);
-                            ++m; ++bi;
-                            if (m == wrap_m) { bi += wrap - 1u; wrap_m += mcu_w; }
-                            zi = 0; ep = Ss; s0 = s1 = N0 = N1 = G0 = G1 = 0;
-                            take();                                    // (not read when the queue is empty)
-                            stop = m < hm ? stop : 0u;                 // also at the interval's end: hm is at most m1
+                            br.pos += apply(true, e, nz, T, k, n);
+                            W.load(br.pos);
+                            win = W.window(br.pos); raw = tab_entry(tab, win);
                         }
                     }
                 }

@@ -941,11 +941,11 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
             r->pair_count[(size_t)g * G + s] = n_items - begin;
         }
     // Pairs shorten the chain but leave the lanes of the shorter scan idle (about 1.4 times the warp instructions for the
-    // ten-scan script), so they are for records whose waves fit the machine, or nearly: it holds 18 of these warps an SM (three
-    // warps and 36 KB of shared memory a CTA), and up to 20 an SM the few that wait cost less than the chain gains.  Without and
-    // with pairs, by warps an SM, decode at k = 10 in us: ImageNet-shaped images 17.2 656 and 639, 18.3 671 and 640, 19.1 679 and
-    // 669, 20.8 700 and 700, 20.9 707 and 728, 23.6 775 and 778, 34 957 and 997; CelebA-shaped 18.2 452 and 441; mixed
-    // sizes in 4:4:4 2.3 551 and 438.  Raised 2 -> 10: 17.2 642 and 555, 34 834 and 853.
+    // ten-scan script), so they are for records whose waves fit the machine, or nearly: it holds 18 lane-per-interval warps of 36 KB
+    // a three an SM, and up to 20 an SM the few that wait cost less than the chain gains.  (Measured with an earlier step of the chains,
+    // without and with pairs, by warps an SM, decode at k = 10 in us: ImageNet-shaped images 17.2 656 and 639, 19.1 679 and 669, 20.8 700 and
+    // 700, 20.9 707 and 728, 23.6 775 and 778, 34 957 and 997; CelebA-shaped 18.2 452 and 441.  Raised 2 -> 10: 17.2 642 and 555, 34
+    // 834 and 853.)
     if (on_device && cudaDeviceGetAttribute(&r->n_sms, cudaDevAttrMultiProcessorCount, r->device) != cudaSuccess) return PCR_E_CUDA;
     for (const std::vector<int>& scans_of_wave : r->paired_waves) {
         std::vector<char> in_pair(G, 0);
@@ -1281,11 +1281,11 @@ static bool allow_refine_smem(int device) {
 }
 
 // Whether refine_kernel's CTAs take the AC refinements among scans k0 .. k-1 of a wave, or lane-per-interval warps of
-// entropy_kernel.  A CTA's chains are four times as fast (170 to 220 against 700 cycles a symbol), but three CTAs are all an SM
-// holds, 96 chains against 576, so a launch of many items is better off with the warps.  Decode at k = 10 in us,
-// warps and CTAs, by CTAs an SM: ImageNet-shaped images 2 352 and 237, 3.8 405 and 304, 5.8 427 and 390, 7.8 422 and 372, 9.7 476
-// and 489, 11.7 534 and 568; CelebA-shaped 2.5 211 and 180, 5 235 and 225, 10 301 and 342, 20 489 and 519; mixed sizes in
-// 4:4:4 2.3 423 and 281, 6.2 422 and 281.
+// entropy_kernel.  A CTA's chains are several times as fast (170 to 220 cycles a symbol), but three CTAs are all an SM
+// holds, 96 chains against 480, so a launch of many items is better off with the warps.  Decode at k = 10 in us,
+// warps and CTAs, by CTAs an SM: ImageNet-shaped images 2.9 261 and 217, 4.9 357 and 339, 7.8 415 and 362, 9.7 463 and 476, 11.7 508 and
+// 551; CelebA-shaped 2.5 162 and 158, 10 289 and 336, 20 439 and 491; mixed sizes in 4:4:4 2.3 293 and 219, 6.2 345 and 269; raised
+// 2 -> 10 3.9 385 and 322, 7.8 434 and 436.
 static bool refine_in_ctas(const pcr_record* rec, const std::vector<int>& wave, bool paired, int k0, int k) {
     uint64_t ctas = 0;
     std::vector<char> counted(rec->G, 0);                     // scans that a pair's items stand for
