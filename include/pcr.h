@@ -326,7 +326,7 @@ void pcr_close(pcr_record* rec);
  * of the same record takes it back, which saves the host-side walk over every image's marker
  * segments and the table uploads (0.38 -> 0.15 ms for 1024 images).  The handle it returns is fresh:
  * nothing resident, nothing decoded, default settings.  A record is recognised by the address and
- * length of its bytes, the PCR_SLICES / PCR_LONG_MIN_BYTES settings, the current device, and a
+ * length of its bytes, the PCR_* settings of the environment, the current device, and a
  * hash of its header, sample metadata, index (position and length of every chunk) and the first
  * 256 bytes of every image's first chunk (frame header, quantisation and Huffman tables).  Bytes
  * that changed elsewhere under the same address are the caller's responsibility, exactly as for
