@@ -26,9 +26,12 @@ namespace pcr {
 constexpr int kSeqWarps = 8;
 constexpr uint32_t kSeqRing = 128;            // words of the stream per lane.  A block takes at most 62 (64 symbols of at most 31
                                               // bits), and its first word is held until it has been written
-constexpr uint32_t kSeqSlots = 64;            // blocks of an interval whose beginnings are held: a round's and the round's before
+constexpr uint32_t kSeqSlots = 64;            // blocks of an interval whose beginnings are held
 constexpr int kSeqSteps = 64;                 // symbols a round (a block has two at least)
-static_assert(kSeqSteps <= (int)kSeqSlots, "");
+// Blocks a round finishes at most: while warp 0 stores where those behind block m begin, the others read where those of the round
+// before began, so the beginnings from m - kSeqRoundBlocks to m + kSeqRoundBlocks are in use at once.
+constexpr uint32_t kSeqRoundBlocks = 31;
+static_assert(2 * kSeqRoundBlocks + 1 <= kSeqSlots, "a slot is used again while it is read");
 
 struct SeqShared {
     ScanTab tabs[4];                          // DC, DC, AC, AC
@@ -115,7 +118,7 @@ __global__ void __launch_bounds__(32 * kSeqWarps, 4) sequential_kernel(Params P,
             // ---- the chains
             const uint32_t filled = round ? sh.filled[nb][lane] : 0u;
             uint32_t stop = done ? 0u : min(32u * (filled - min(filled, 3u)), limit + 1u);
-            const uint32_t start = (uint32_t)__cvta_generic_to_shared(sh.start) + 4u * lane, m_end = 32u * n;
+            const uint32_t start = (uint32_t)__cvta_generic_to_shared(sh.start) + 4u * lane, m_end = min(32u * n, 32u * (m + kSeqRoundBlocks));
             uint4 of = lds128(place);                          // see SeqShared::next
             W.load(pos);
             uint32_t tab = k ? of.x : of.w, win = W.window(pos), raw = tab_entry(tab, win), m32 = 32u * m;

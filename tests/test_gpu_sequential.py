@@ -15,7 +15,7 @@ from test_gpu_kernel_edges import _compare, _field
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("samp", [(2, 2, 3), (2, 1, 3), (1, 1, 3), (1, 1, 1)])
+@pytest.mark.parametrize("samp", [(2, 2, 3), (2, 1, 3), (1, 2, 3), (1, 1, 3), (1, 1, 1)])
 @pytest.mark.parametrize("fixed", [0, 1, 5, 60])
 @pytest.mark.parametrize("kind", ["dense", "usual", "empty"])
 def test_blocks_and_intervals(kind, fixed, samp):
@@ -27,6 +27,18 @@ def test_blocks_and_intervals(kind, fixed, samp):
     with pcr_synth.sampling(*samp), pcr_synth.scan_script(pcr_synth.SCRIPT_BASELINE):
         coeffs = [_field(rng, pcr_synth.num_blocks(w, h), density, top) for w, h in dims]
         rec = pcr_synth.record_from_coeffs(dims, coeffs, restart_rows=fixed == 0, restart_fixed=fixed)
+    _compare(rec, (1,))
+
+
+@pytest.mark.parametrize("samp", [(2, 2, 3), (1, 2, 3), (1, 1, 1)])
+def test_flat_rows(samp):
+    """Blocks of two symbols, hundreds of them an interval: round after round ends as many blocks as it can.  (The DC differences go
+    up and down, so a block read from another one's beginning shows.)"""
+    rng = np.random.default_rng(3)
+    dims = [(1600, 24), (800, 48), (130, 17)]
+    with pcr_synth.sampling(*samp), pcr_synth.scan_script(pcr_synth.SCRIPT_BASELINE):
+        coeffs = [_field(rng, pcr_synth.num_blocks(w, h), 0.0, 40) for w, h in dims]
+        rec = pcr_synth.record_from_coeffs(dims, coeffs, restart_rows=True)
     _compare(rec, (1,))
 
 
