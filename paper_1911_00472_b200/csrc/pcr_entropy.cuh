@@ -1063,7 +1063,9 @@ __global__ void __launch_bounds__(32 * kEntropyWarps, kRefine ? 4 : 1) entropy_k
                     bi += row ? wrap : (end ? 1u : 0u); wrap_m += row ? mcu_w : 0u;
                     zi = end ? 0u : (act ? T + 1u : zi); ep = end ? Ss : (act ? ep + n : ep);
                     s0 = end ? 0u : s0; s1 = end ? 0u : s1; N0 = end ? 0u : N0; N1 = end ? 0u : N1; G0 = end ? 0u : G0; G1 = end ? 0u : G1;
-                    lds128_if(end, queue + ((m & (kMaskQueue - 1)) << 9), Z);      // (not read when the queue is empty)
+                    // (only an entry that is there: waiting lanes look ranks up in their Z too, and a slot's old contents may lead
+                    // outside the table; the finished block's entry does not)
+                    lds128_if(end && m < hm, queue + ((m & (kMaskQueue - 1)) << 9), Z);
                     stop = m < hm ? stop : 0u;                 // also at the interval's end: hm is at most m1
                     return d;
                 };

@@ -53,3 +53,24 @@ def test_sequential_block_beginnings():
         assert m > handed
         rounds += 1
     assert rounds <= n // (steps // 2 - 1) + 1
+
+
+def test_refinement_mask_queue():
+    """Intervals of 1 to 40 blocks, any number of blocks finished between two top-ups: a lane loads its next block's entry only
+    if the queue holds that block's."""
+    text = _source("pcr_entropy.cuh")
+    size = _constants(text)["kMaskQueue"]
+    load = _one(r"lds128_if\(([^,]+), queue \+ \(\(m & \(kMaskQueue - 1\)\) << 9\), Z\)", text)
+    for blocks in range(1, 41):
+        for most in range(1, size + 1):
+            held, m, hm = [None] * size, 0, 0
+            while m < blocks:
+                while hm < blocks and hm - m < size:             # top-up
+                    held[hm % size] = hm
+                    hm += 1
+                for _ in range(most):
+                    if m >= hm:
+                        break
+                    m += 1
+                    if _value(load, {"end": True, "m": m, "hm": hm}):
+                        assert held[m % size] == m, (blocks, most, m, hm)
