@@ -276,9 +276,13 @@ struct DcReading {
 
 // Interleaved DC scans, wide CTAs.  Bit positions fall in within a few symbols, but a reading can go on for long with the
 // wrong place in the MCU (up to 23 rounds of the search above).  So every subsequence is read once from EVERY place, 512 bits ahead of
-// it, and one warp follows the true state through the readings; where none of them began its subsequence in the true state,
-// that subsequence is read once more.  On return a thread has the start of its subsequence (L.begin, L.end changed to match), its
-// blocks, the number of blocks and the sums of differences in front of it.
+// it, and one warp follows the true state through the readings.  Where none of them began its subsequence in the true state, that one
+// is read once more, and with the first such one the likely cases behind it, all at once: a lone lane took 14 us for each,
+// three in an image of 343x562 (DC alone of 16 images of mixed sizes 127 us, by rounds of the search 110, now 95).  On return a thread
+// has the start of its subsequence (L.begin, L.end changed to match), its blocks, the number of blocks and the sums of differences in
+// front of it.
+constexpr uint32_t kDcNone = 0xFFFFFFFFu;
+template <uint32_t kThreads> __host__ __device__ constexpr uint32_t dc_words() { return 14 * kThreads + 4; }     // of shared memory at mem
 template <uint32_t kThreads>
 __device__ __forceinline__ void dc_hypotheses(const DcSteps& S, LongSpan& L, uint32_t* mem, uint32_t j1, uint32_t j2, uint32_t& pos, uint32_t& st,
                                               uint32_t& nb, uint32_t& n, int& pred0, int& pred1, int& pred2, uint32_t& all) {
@@ -288,60 +292,87 @@ __device__ __forceinline__ void dc_hypotheses(const DcSteps& S, LongSpan& L, uin
     auto begin_of = [&](uint32_t i) { return min(max(i * len, L.lead), L.endbit); };
     auto end_of = [&](uint32_t i) { return min((i + 1u) * len, L.endbit); };
     // by hypothesis and subsequence: the state it begins in (one number: equal ones within a subsequence are equal states), the one
-    // it ends in, blocks and sums; in the end, by subsequence, what the caller asks for
-    uint32_t* const key = mem;
-    uint32_t* const x_pos = mem + kThreads;
-    uint32_t* const x_st = mem + 2 * kThreads;
-    uint32_t* const x_nb = mem + 3 * kThreads;
-    int* const x_sum = reinterpret_cast<int*>(mem + 4 * kThreads);                 // [3][kThreads]
+    // it ends in, blocks and sums; behind them the same once more for second readings; in the end, by subsequence, what the caller asks for
+    constexpr uint32_t kSet = 7 * kThreads;
+    auto store = [&](uint32_t at, const DcReading& R) {
+        mem[kThreads + at] = R.w.p; mem[2 * kThreads + at] = R.st; mem[3 * kThreads + at] = R.nb;
+        mem[4 * kThreads + at] = (uint32_t)R.sum0; mem[5 * kThreads + at] = (uint32_t)R.sum1; mem[6 * kThreads + at] = (uint32_t)R.sum2;
+    };
+    const uint32_t h = tid / subs, i = tid - h * subs, b = begin_of(i), e = end_of(i);
+    const bool some = h < H && b < e;
     {
-        const uint32_t h = tid / subs, i = tid - h * subs, b = begin_of(i), e = end_of(i);
-        uint32_t k = 0xFFFFFFFFu;
-        if (h < H && b < e && (i != 0 || h == 0)) {
+        uint32_t k = kDcNone;
+        if (some && (i != 0 || h == 0)) {
             const uint32_t from = i == 0 ? L.lead : max(L.lead, b - min(b, 512u));
             DcReading R(S, L.base, from, from == L.lead ? 0u : h);
             R.to(b, j1, j2);
             k = (R.w.p << 3) + R.st;
             R.nb = 0; R.sum0 = R.sum1 = R.sum2 = 0;
             R.to(e, j1, j2);
-            x_pos[tid] = R.w.p; x_st[tid] = R.st; x_nb[tid] = R.nb;
-            x_sum[tid] = R.sum0; x_sum[kThreads + tid] = R.sum1; x_sum[2 * kThreads + tid] = R.sum2;
+            store(tid, R);
         }
-        key[tid] = k;
+        mem[tid] = k;
+        mem[kSet + tid] = kDcNone;
     }
-    __syncthreads();
-    if (tid < 32u) {
-        uint32_t p = L.lead, s = 0, blocks = 0;
-        int a0 = 0, a1 = 0, a2 = 0;
-        for (uint32_t i = 0; i < subs; ++i) {
-            const uint32_t e = end_of(i), at = lane * subs + i;
-            const bool live = begin_of(i) < e;
-            const unsigned who = __ballot_sync(full, live && lane < H && key[at] == (p << 3) + s);
-            uint32_t q = 0, t = 0, c = 0;
-            int d0 = 0, d1 = 0, d2 = 0;
-            if (who) {
-                if (lane == (uint32_t)__ffs((int)who) - 1u) { q = x_pos[at]; t = x_st[at]; c = x_nb[at]; d0 = x_sum[at]; d1 = x_sum[kThreads + at]; d2 = x_sum[2 * kThreads + at]; }
-            } else if (live && lane == 0) {
-                DcReading R(S, L.base, p, s);
-                R.to(e, j1, j2);
-                q = R.w.p; t = R.st; c = R.nb; d0 = R.sum0; d1 = R.sum1; d2 = R.sum2;
+    // Warp 0 follows the true state from one subsequence to the next, lanes 0..15 looking for it among the first readings, 16..31 among
+    // the second ones.  Where it finds none, that subsequence is read once more, and beside it, once, every one behind it from each state that a
+    // reading of the one in front of it ended in and that none of its own began in.
+    uint32_t p = L.lead, s = 0, blocks = 0, next = 0;          // (warp 0)
+    int a0 = 0, a1 = 0, a2 = 0;
+    for (bool again = false;; again = true) {
+        __syncthreads();
+        if (tid < 32u) {
+            const uint32_t set = lane < 16u ? 0u : kSet, lh = lane & 15u;
+            for (; next < subs; ++next) {
+                const uint32_t at = set + lh * subs + next, end = end_of(next);
+                const bool live = begin_of(next) < end;
+                const unsigned who = __ballot_sync(full, live && lh < H && mem[at] == (p << 3) + s);
+                uint32_t q = 0, t = 0, c = 0;
+                int d0 = 0, d1 = 0, d2 = 0;
+                const uint32_t src = who ? (uint32_t)__ffs((int)who) - 1u : 0u;
+                if (who) {
+                    if (lane == src) { q = mem[kThreads + at]; t = mem[2 * kThreads + at]; c = mem[3 * kThreads + at]; d0 = (int)mem[4 * kThreads + at]; d1 = (int)mem[5 * kThreads + at]; d2 = (int)mem[6 * kThreads + at]; }
+                } else if (live) {
+                    if (!again) break;
+                    if (lane == 0) {
+                        DcReading R(S, L.base, p, s);
+                        R.to(end, j1, j2);
+                        q = R.w.p; t = R.st; c = R.nb; d0 = R.sum0; d1 = R.sum1; d2 = R.sum2;
+                    }
+                }
+                q = __shfl_sync(full, q, src); t = __shfl_sync(full, t, src); c = __shfl_sync(full, c, src);
+                d0 = __shfl_sync(full, d0, src); d1 = __shfl_sync(full, d1, src); d2 = __shfl_sync(full, d2, src);
+                __syncwarp(full);
+                if (lane == 0) {                               // (no reading of a subsequence passed is looked at again)
+                    mem[next] = p; mem[kThreads + next] = s; mem[2 * kThreads + next] = blocks;
+                    mem[3 * kThreads + next] = (uint32_t)a0; mem[4 * kThreads + next] = (uint32_t)a1; mem[5 * kThreads + next] = (uint32_t)a2;
+                }
+                if (live) { p = q; s = t; blocks += c; a0 += d0; a1 += d1; a2 += d2; }
             }
-            const int src = who ? __ffs((int)who) - 1 : 0;
-            q = __shfl_sync(full, q, src); t = __shfl_sync(full, t, src); c = __shfl_sync(full, c, src);
-            d0 = __shfl_sync(full, d0, src); d1 = __shfl_sync(full, d1, src); d2 = __shfl_sync(full, d2, src);
-            __syncwarp(full);
-            if (lane == 0) { key[i] = p; x_pos[i] = s; x_nb[i] = blocks; x_sum[i] = a0; x_sum[kThreads + i] = a1; x_sum[2 * kThreads + i] = a2; }
-            if (live) { p = q; s = t; blocks += c; a0 += d0; a1 += d1; a2 += d2; }
+            if (lane == 0) { mem[2 * kSet] = next; mem[2 * kSet + 1] = blocks; mem[2 * kSet + 2] = p; mem[2 * kSet + 3] = s; }
         }
-        if (lane == 0) x_st[0] = blocks;
+        __syncthreads();
+        const uint32_t stop = mem[2 * kSet];
+        if (again || stop >= subs) break;
+        if (some && (i == stop ? h == 0 : i > stop)) {
+            const uint32_t from = i == stop ? mem[2 * kSet + 2] : mem[kThreads + tid - 1u], place = i == stop ? mem[2 * kSet + 3] : mem[2 * kThreads + tid - 1u];
+            const uint32_t k = (from << 3) + place;
+            bool known = false;
+            for (uint32_t j = 0; j < H; ++j) known = known || mem[j * subs + i] == k;
+            if (!known) {
+                DcReading R(S, L.base, from, place);
+                R.to(e, j1, j2);
+                store(kSet + tid, R);
+                mem[kSet + tid] = k;
+            }
+        }
     }
-    __syncthreads();
     const bool mine = tid < subs;
     L.begin = mine ? begin_of(tid) : L.endbit; L.end = mine ? end_of(tid) : 0u;
-    pos = mine ? key[tid] : L.endbit; st = mine ? x_pos[tid] : 0u; n = mine ? x_nb[tid] : 0u;
-    pred0 = mine ? x_sum[tid] : 0; pred1 = mine ? x_sum[kThreads + tid] : 0; pred2 = mine ? x_sum[2 * kThreads + tid] : 0;
-    all = x_st[0];
-    nb = mine ? (tid + 1u < subs ? x_nb[tid + 1u] : all) - n : 0u;
+    pos = mine ? mem[tid] : L.endbit; st = mine ? mem[kThreads + tid] : 0u; n = mine ? mem[2 * kThreads + tid] : 0u;
+    pred0 = mine ? (int)mem[3 * kThreads + tid] : 0; pred1 = mine ? (int)mem[4 * kThreads + tid] : 0; pred2 = mine ? (int)mem[5 * kThreads + tid] : 0;
+    all = mem[2 * kSet + 1];
+    nb = mine ? (tid + 1u < subs ? mem[2 * kThreads + tid + 1u] : all) - n : 0u;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -370,7 +401,7 @@ __global__ void __launch_bounds__(32 * kWarps) first_pass_long_kernel(Params P, 
     constexpr uint32_t kLongStage = long_stage<kWarps>();
     __shared__ __align__(16) uint8_t s_tabs[2 * sizeof(ScanTab)];
     __shared__ uint32_t s_stage[kLongStage];
-    __shared__ uint32_t s_marks[kMarks * kThreads];
+    __shared__ uint32_t s_marks[kWarps == kLongWarps ? kMarks * kThreads : dc_words<kThreads>()];
     __shared__ uint32_t s_pos[kWarps], s_state[kWarps], s_u[kWarps];
     __shared__ int s_i[kWarps];
     const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;

@@ -32,3 +32,20 @@ def test_subsequences(script, samp, ctas, monkeypatch):
     monkeypatch.setenv("PCR_LONG_CTAS", str(ctas))
     last = {"ten": 6 if samp[2] == 1 else 10, "baseline": 1, "single": 6}[script]
     _compare(rec, sorted({1, min(5, last), last}))
+
+
+@pytest.mark.parametrize("ctas", [0, 1 << 20])
+@pytest.mark.parametrize("samp", [(2, 2, 3), (2, 1, 3), (1, 2, 3), (1, 1, 3)])
+@pytest.mark.parametrize("length", [350, 1000])
+def test_flat_stretches(length, samp, ctas, monkeypatch):
+    """DC scans with long stretches of one code: readings that begin inside one fall in late or not at all, so that some subsequences
+    have to be read once more, some behind others."""
+    rng = np.random.default_rng(length // 50)
+    dims = [(640, 400), (400, 640), (96, 1000)]
+    with pcr_synth.sampling(*samp):
+        coeffs = [_field(rng, pcr_synth.num_blocks(w, h), 0.0, 1) for w, h in dims]
+        for c in coeffs:
+            c[np.repeat(rng.random(len(c) // length + 1) < 0.6, length)[:len(c)], 0] = 7
+        rec = pcr_synth.record_from_coeffs(dims, coeffs, restart_rows=False)
+    monkeypatch.setenv("PCR_LONG_CTAS", str(ctas))
+    _compare(rec, (1,))
