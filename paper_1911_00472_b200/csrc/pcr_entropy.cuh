@@ -685,11 +685,18 @@ __device__ __forceinline__ void dc_refine_image(const Params& P, int s, int img,
 //
 // First passes: a step is one straight line of predicated instructions (with branches for block ends and long codes 300
 // cycles an AC symbol alone on an SM, now 230), and what a warp needs of the tables is loaded at once (the start of a warp 6 to 10 k cycles,
-// now 3.5 k).  kPack: see below and pack_first_passes; without it the stores of 1024 ImageNet-shaped images at k = 5 took half of
-// the load/store units' time, 197 us against 172 (before: 206).  64 images 66 -> 44 us.  DC alone of 1024 images 55 -> 40 us (pairs
-// of luminance blocks stored together, MCUs without a branch inside).
-template <bool kRoi, bool kRefine, bool kPack>
-__global__ void __launch_bounds__(32 * kEntropyWarps, kRefine ? 4 : 1) entropy_kernel(Params P, ItemRuns runs) {
+// now 3.5 k).  After eight steps a warp whose lanes have all arrived tops up at once: with short intervals (32x32 images) it stands
+// still for half of the steps otherwise.  DC alone of 1024 images 55 -> 40 us (pairs of luminance blocks stored together, MCUs
+// without a branch inside).
+// Three forms (which: first_pass_form).  kFirstFull packs the stores (see below): those of 1024 ImageNet-shaped images at k = 5 took
+// half of the load/store units' time, 197 us against 172 (before: 206); 64 images 44 us without packing, 66 with it.  kFirstShort is held
+// to registers for eight CTAs an SM instead of five: where intervals are short, what counts is how many warps start side by side.  Decode of
+// 32x32 images at k = 5, five and eight CTAs: 1024 73.4 and 71.5 us, 2048 110 and 104, 4096 178 and 167; of ImageNet-shaped images 64 80
+// and 80, 256 118 and 123, 1024 352 and 379.
+enum { kFirstFew = 0, kFirstFull = 1, kFirstShort = 2 };     // (see first_pass_form)
+template <bool kRoi, bool kRefine, int kForm>
+__global__ void __launch_bounds__(32 * kEntropyWarps, kRefine ? 4 : (kForm == kFirstShort ? 8 : 1)) entropy_kernel(Params P, ItemRuns runs) {
+    constexpr bool kPack = kForm == kFirstFull;
     extern __shared__ __align__(16) uint8_t s_entropy[];
     __shared__ __align__(16) uint8_t s_sel[kRefine ? sizeof(SelectTable) : 16];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -938,6 +945,7 @@ __global__ void __launch_bounds__(32 * kEntropyWarps, kRefine ? 4 : 1) entropy_k
                         raw = long_code(tab, win, kTabAcFirst);
                         if (raw == 0) { bad = true; stop = 0; }        // no such symbol: the lane ends here
                     }
+                    if (!__any_sync(full, br.pos < stop)) break;
                 }
                 __syncwarp(full);
                 bad = bad || br.pos > br.limit;

@@ -191,6 +191,7 @@ struct pcr_record {
     std::vector<uint32_t> slice_img;                            // [n_slices + 1] first image of each slice
     std::vector<uint32_t> slice_unit;                           // [n_slices + 1] first pixel unit of each slice
     std::vector<uint32_t> item_begin, item_count;               // [n_slices][G]
+    std::vector<uint64_t> first_bytes;                          // of AC first passes: entropy-coded bytes that items stand for
     // Scans that are one long restart interval take kernels of their own (pcr_long.cuh): first passes
     // as (scan, image) pairs sorted by (slice, wave, scan); AC refinements as (component, image)
     // groups sorted by slice (all refinement scans of the component that a call decodes, in one CTA)
@@ -219,7 +220,8 @@ struct pcr_record {
     uint32_t refine_ctas = 8;                                   // see refine_in_ctas (PCR_REFINE_CTAS overrides)
     uint32_t long_ctas = 3;                                     // see wide_long_scans (PCR_LONG_CTAS overrides)
     uint32_t index_ctas = 8;                                    // see launch_index_kernel (PCR_INDEX_CTAS overrides)
-    uint32_t pack_warps = 12;                                   // see pack_first_passes (PCR_PACK_WARPS overrides)
+    int64_t pack_warps = -1;                                    // see first_pass_form (PCR_PACK_WARPS: a line in warps an SM instead)
+    uint32_t short_warps = 20;                                  // see first_pass_form (PCR_SHORT_WARPS overrides)
     std::vector<uint32_t> pair_begin, pair_count;               // [n_slices][G] items of the pair, by its later scan
     uint32_t n_units = 0;
     // device state
@@ -806,7 +808,8 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     if (const char* e = getenv("PCR_REFINE_CTAS")) r->refine_ctas = (uint32_t)std::max(0, atoi(e));
     if (const char* e = getenv("PCR_INDEX_CTAS")) r->index_ctas = (uint32_t)std::max(0, atoi(e));
     if (const char* e = getenv("PCR_LONG_CTAS")) r->long_ctas = (uint32_t)std::max(0, atoi(e));
-    if (const char* e = getenv("PCR_PACK_WARPS")) r->pack_warps = (uint32_t)std::max(0, atoi(e));
+    if (const char* e = getenv("PCR_PACK_WARPS")) r->pack_warps = std::max(0, atoi(e));
+    if (const char* e = getenv("PCR_SHORT_WARPS")) r->short_warps = (uint32_t)std::max(0, atoi(e));
     // slices: enough images each to fill the machine, few enough to keep launches cheap
     {
         // four at most: one record decodes as fast with four slices as with eight, and two records
@@ -925,6 +928,12 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
                 r->item_begin[(size_t)g * G + s] = begin;
                 r->item_count[(size_t)g * G + s] = n_items - begin;
             }
+    r->first_bytes.assign(G, 0);
+    for (uint32_t s = 0; s < G; ++s)
+        for (uint32_t i = 0; r->script[s].Ss > 0 && r->script[s].Ah == 0 && i < N; ++i) {
+            const ScanDesc& sd = scans[(size_t)s * N + i];
+            if (!single || !takes_long_kernel((int)s, i)) r->first_bytes[s] += sd.data_end - sd.data_off;
+        }
     // the pairs' items: sixteen intervals of one image
     r->pair_begin.assign((size_t)r->n_slices * G, 0); r->pair_count.assign((size_t)r->n_slices * G, 0);
     for (int g = 0; g < r->n_slices; ++g)
@@ -1053,7 +1062,7 @@ uint64_t hash_bytes(uint64_t h, const uint8_t* p, size_t n) {
 }
 uint32_t env_key() {
     uint32_t h = 0;
-    for (const char* name : {"PCR_SLICES", "PCR_LONG_MIN_BYTES", "PCR_REFINE_CTAS", "PCR_PACK_WARPS", "PCR_INDEX_CTAS", "PCR_LONG_CTAS"}) {
+    for (const char* name : {"PCR_SLICES", "PCR_LONG_MIN_BYTES", "PCR_REFINE_CTAS", "PCR_PACK_WARPS", "PCR_SHORT_WARPS", "PCR_INDEX_CTAS", "PCR_LONG_CTAS"}) {
         const char* v = getenv(name);
         h = h * 1000003u + (v ? (uint32_t)atoi(v) + 1u : 0u);
     }
@@ -1299,16 +1308,23 @@ static bool refine_in_ctas(const pcr_record* rec, const std::vector<int>& wave, 
     return ctas <= (uint64_t)rec->refine_ctas * (uint64_t)rec->n_sms;
 }
 
-// Whether the first passes among scans k0 .. k-1 of a wave pack their stores (kPack of entropy_kernel): where the
-// machine is full, because stores are what it waits for; elsewhere a step without the packing is the shorter chain.  First wave in
-// us without and with packing, by warps an SM: ImageNet-shaped images at k = 5 0.2 38 and 58, 2.3 44 and 69, 9 61 and 86, 36 197
-// and 172; CelebA-shaped 18 98 and 86.
-static bool pack_first_passes(const pcr_record* rec, const std::vector<int>& wave, int k0, int k) {
-    uint64_t warps = 0;
+// Form of entropy_kernel for the first passes among scans k0 .. k-1 of a wave: kFirstFull where there is so much to store that stores are
+// what the machine waits for, which is a matter of how much data an SM has, not of how many warps it comes in; elsewhere a step
+// without the packing is the shorter chain.  Decode in us without and with packing, by entropy-coded kilobytes of AC scans an SM: k = 5
+// ImageNet-shaped images 5 102 and 134, 9 120 and 141, 13 157 and 165, 16 194 and 185, 18 213 and 209, 27 294 and 270, 34 357 and
+// 335; CelebA-shaped 9 120 and 126, 12 145 and 142, 18 185 and 180, 23 251 and 225; HAM-shaped 6 191 and 199, 9 266 and 270, 12 346 and
+// 324; 1024 of 96x96 5 85 and 93, 4096 of 32x32 4 167 and 188 (these two fill the machine with warps, 15 and 83 an SM).
+// kFirstShort for many warps of little data (see entropy_kernel).
+static int first_pass_form(const pcr_record* rec, const std::vector<int>& wave, int k0, int k) {
+    uint64_t warps = 0, bytes = 0;
     for (int s : wave)
-        if (s >= k0 && s < k && rec->script[s].Ah == 0)
+        if (s >= k0 && s < k && rec->script[s].Ah == 0) {
             for (int g = 0; g < rec->n_slices; ++g) warps += rec->item_count[(size_t)g * rec->G + s];
-    return warps > (uint64_t)rec->pack_warps * (uint64_t)rec->n_sms;
+            bytes += rec->first_bytes[s];
+        }
+    const uint64_t sms = (uint64_t)rec->n_sms;
+    if (rec->pack_warps >= 0 ? warps > (uint64_t)rec->pack_warps * sms : bytes > 11000ull * sms) return kFirstFull;
+    return warps > (uint64_t)rec->short_warps * sms ? kFirstShort : kFirstFew;
 }
 
 // Whether the long scans of a wave that are first passes (or sequential) get CTAs of four times as many warps: while
@@ -1465,16 +1481,19 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
                 const uint32_t smem = kEntropyWarps * (refine ? warp_bytes<true>() : warp_bytes<false>());
                 runs.item_blocks = nb;
                 if (last && refine && !dc_done) nb += carry_dc(runs, (rec->dc_refine_chunks + 1) / 2);      // about five MCUs a thread (waves without AC refinements are compiled without this)
-                const bool pack = pack_first_passes(rec, waves[w], k0, k);
+                const int form = first_pass_form(rec, waves[w], k0, k);
                 if (refine) {
-                    if (roi) entropy_kernel<true, true, true><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
-                    else entropy_kernel<false, true, true><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
-                } else if (pack) {
-                    if (roi) entropy_kernel<true, false, true><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
-                    else entropy_kernel<false, false, true><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
+                    if (roi) entropy_kernel<true, true, kFirstFull><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
+                    else entropy_kernel<false, true, kFirstFull><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
+                } else if (form == kFirstFull) {
+                    if (roi) entropy_kernel<true, false, kFirstFull><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
+                    else entropy_kernel<false, false, kFirstFull><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
+                } else if (form == kFirstShort) {
+                    if (roi) entropy_kernel<true, false, kFirstShort><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
+                    else entropy_kernel<false, false, kFirstShort><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
                 } else {
-                    if (roi) entropy_kernel<true, false, false><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
-                    else entropy_kernel<false, false, false><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
+                    if (roi) entropy_kernel<true, false, kFirstFew><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
+                    else entropy_kernel<false, false, kFirstFew><<<nb, 32 * kEntropyWarps, smem, q>>>(P, runs);
                 }
                 ++g_launches;
                 runs.n = 0; count = 0;

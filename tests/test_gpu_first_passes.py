@@ -1,6 +1,7 @@
-"""First passes in scans with restart intervals, with their stores packed (large launches) and one by one (PCR_PACK_WARPS, read when a
-record is opened, chooses): bands that hold whole words of a block's positions 1..7, parts of words or none, intervals of one
-block to several rows, lists of values that end anywhere in a group of four, codes longer than the tables' index."""
+"""First passes in scans with restart intervals, with their stores packed (much data) and one by one (PCR_PACK_WARPS, read when a
+record is opened, chooses), and in the form for many short intervals (PCR_SHORT_WARPS): bands that hold whole words of a block's
+positions 1..7, parts of words or none, intervals of one block to several rows, lists of values that end anywhere in a group
+of four, codes longer than the tables' index."""
 from __future__ import annotations
 
 import numpy as np
@@ -29,4 +30,17 @@ def test_bands_and_intervals(script, fixed, warps, monkeypatch):
         coeffs = [_field(rng, pcr_synth.num_blocks(w, h), d, t) for (w, h), d, t in zip(dims, (0.15, 1.0, 0.02), (60, 1023, 500))]
         rec = pcr_synth.record_from_coeffs(dims, coeffs, restart_rows=fixed == 0, restart_fixed=fixed)
     monkeypatch.setenv("PCR_PACK_WARPS", str(warps))
+    _compare(rec, (1, 5) if script == "ten" else range(1, len(SCRIPTS[script]) + 1))
+
+
+@pytest.mark.parametrize("fixed", [0, 1, 7])
+@pytest.mark.parametrize("script", list(SCRIPTS))
+def test_many_short_intervals(script, fixed, monkeypatch):
+    rng = np.random.default_rng(fixed)
+    dims = [(32, 32), (8, 8), (200, 33), (31, 33)]
+    with pcr_synth.scan_script(SCRIPTS[script]):
+        coeffs = [_field(rng, pcr_synth.num_blocks(w, h), d, t) for (w, h), d, t in zip(dims, (0.15, 1.0, 0.3, 0.02), (60, 1023, 100, 500))]
+        rec = pcr_synth.record_from_coeffs(dims, coeffs, restart_rows=fixed == 0, restart_fixed=fixed)
+    monkeypatch.setenv("PCR_PACK_WARPS", str(1 << 20))
+    monkeypatch.setenv("PCR_SHORT_WARPS", "0")
     _compare(rec, (1, 5) if script == "ten" else range(1, len(SCRIPTS[script]) + 1))
