@@ -1122,6 +1122,7 @@ __global__ void __launch_bounds__(32 * kEntropyWarps, kRefine ? 4 : (kForm == kF
                             win = W.window(br.pos); raw = tab_entry(tab, win);
                         }
                     }
+                    if (!__any_sync(full, br.pos < stop)) break;
                 }
                 __syncwarp(full);
                 fresh = m >= hm;
