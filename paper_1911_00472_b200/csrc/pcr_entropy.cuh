@@ -945,7 +945,7 @@ __global__ void __launch_bounds__(32 * kEntropyWarps, kRefine ? 4 : (kForm == kF
                         raw = long_code(tab, win, kTabAcFirst);
                         if (raw == 0) { bad = true; stop = 0; }        // no such symbol: the lane ends here
                     }
-                    if (!__any_sync(full, br.pos < stop)) break;
+                    if (!kRefine && !__any_sync(full, br.pos < stop)) break;      // (in the other form it costs registers that the refinements need)
                 }
                 __syncwarp(full);
                 bad = bad || br.pos > br.limit;
@@ -1122,7 +1122,7 @@ __global__ void __launch_bounds__(32 * kEntropyWarps, kRefine ? 4 : (kForm == kF
                             win = W.window(br.pos); raw = tab_entry(tab, win);
                         }
                     }
-                    if (!__any_sync(full, br.pos < stop)) break;
+                    if (t == 0 && __ballot_sync(full, br.pos < stop) == 0) break;
                 }
                 __syncwarp(full);
                 fresh = m >= hm;

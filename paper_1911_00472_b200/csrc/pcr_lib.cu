@@ -216,12 +216,15 @@ struct pcr_record {
     // scan s follows, or -1.  Empty when the script has no such pair.
     std::vector<std::vector<int>> paired_waves;
     std::vector<int> pair_of;
-    bool pairs_fit = true;                                      // the waves with pairs fit the machine (see open_impl)
-    uint32_t refine_ctas = 8;                                   // see refine_in_ctas (PCR_REFINE_CTAS overrides)
+    bool pairs_fit = true;                                      // lane-per-interval warps of the waves with pairs fit the machine
+    int pairs = -1;                                             // see pairs_pay (PCR_PAIRS overrides: 0 never, 1 always)
+    double refine_ctas = 4;                                     // see refine_load (PCR_REFINE_CTAS overrides)
     uint32_t long_ctas = 3;                                     // see wide_long_scans (PCR_LONG_CTAS overrides)
     uint32_t index_ctas = 8;                                    // see launch_index_kernel (PCR_INDEX_CTAS overrides)
     int64_t pack_warps = -1;                                    // see first_pass_form (PCR_PACK_WARPS: a line in warps an SM instead)
     uint32_t short_warps = 20;                                  // see first_pass_form (PCR_SHORT_WARPS overrides)
+    // Items of the AC refinements: the sum of their chains' bytes, an item counting with its longest.  By scan; by the pair's later scan
+    std::vector<uint64_t> chain_bytes, pair_chain_bytes;
     std::vector<uint32_t> pair_begin, pair_count;               // [n_slices][G] items of the pair, by its later scan
     uint32_t n_units = 0;
     // device state
@@ -554,6 +557,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     // every image's chunks are walked independently (a few host threads for large records); the
     // running sums over images follow in one serial pass
     std::vector<uint32_t> nsegs((size_t)G * N), image_bytes(N);      // restart intervals by (scan, image); entropy-coded bytes
+    std::vector<uint32_t> chains((size_t)G * N);                     // of AC refinements: bytes of an interval, on average
     std::vector<uint8_t> one_interval(N, 0);                         // some scan of the image is one restart interval
     uint8_t sampling0 = 0;
     auto parse_image = [&](uint32_t i) -> int {
@@ -598,6 +602,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
             }
             sd.nseg = sd.ri ? (uint32_t)((total_mcu + sd.ri - 1) / sd.ri) : 1u;
             nsegs[(size_t)g * N + i] = sd.nseg;
+            if (sp.sc.Ss > 0 && sp.sc.Ah != 0) chains[(size_t)g * N + i] = (sd.data_end - sd.data_off) / std::max(1u, sd.nseg);
             if (sd.nseg == 1) one_interval[i] = 1;
             sum += sd.data_end - sd.data_off;
         }
@@ -805,7 +810,8 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
             for (uint32_t s = 0; s < G; ++s) r->paired_waves[wave[s]].push_back((int)s);
         } else r->pair_of.assign(G, -1);
     }
-    if (const char* e = getenv("PCR_REFINE_CTAS")) r->refine_ctas = (uint32_t)std::max(0, atoi(e));
+    if (const char* e = getenv("PCR_REFINE_CTAS")) r->refine_ctas = atof(e);
+    if (const char* e = getenv("PCR_PAIRS")) r->pairs = atoi(e) != 0;
     if (const char* e = getenv("PCR_INDEX_CTAS")) r->index_ctas = (uint32_t)std::max(0, atoi(e));
     if (const char* e = getenv("PCR_LONG_CTAS")) r->long_ctas = (uint32_t)std::max(0, atoi(e));
     if (const char* e = getenv("PCR_PACK_WARPS")) r->pack_warps = std::max(0, atoi(e));
@@ -837,7 +843,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     if (int rc = TI.allocate(r, on_device)) return rc;
     Item* const items = TI.h<Item>(0);
     uint32_t n_items = 0;
-    r->item_begin.assign((size_t)r->n_slices * G, 0); r->item_count.assign((size_t)r->n_slices * G, 0);
+    r->chain_bytes.assign(G, 0); r->item_begin.assign((size_t)r->n_slices * G, 0); r->item_count.assign((size_t)r->n_slices * G, 0);
     // A scan that is one restart interval of at least this many bytes goes to the kernels for long
     // intervals; DC refinement scans have no items at all (see dc_refine_image).
     uint32_t long_min = 64;
@@ -906,6 +912,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
                 const bool ac = r->script[s].Ss > 0;
                 const bool dc_refine = r->script[s].Ss == 0 && r->script[s].Ah != 0;
                 Item* open = nullptr;                         // an unfilled last item that the next image may extend
+                uint32_t last = 0;                            // the longest chain of the last item
                 for (uint32_t pos = r->slice_img[g]; pos < r->slice_img[g + 1] && !dc_refine; ++pos) {
                     const uint32_t i = order[pos];
                     if (single && takes_long_kernel((int)s, i)) continue;
@@ -917,12 +924,14 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
                         j = std::min<uint32_t>(kSegsPerItem - open->count, nseg);
                         open->count += j; open->next = si + 1u;
                         open = nullptr;
+                        r->chain_bytes[s] += std::max(chains[si], last) - last;
                     }
                     for (; j < nseg; j += kSegsPerItem) {
                         const uint32_t cnt = std::min<uint32_t>(kSegsPerItem, nseg - j);
                         items[n_items] = Item{si, j, cnt, 0u, 0u};
                         open = ac && cnt < (uint32_t)kSegsPerItem ? &items[n_items] : nullptr;
                         ++n_items;
+                        r->chain_bytes[s] += last = chains[si];
                     }
                 }
                 r->item_begin[(size_t)g * G + s] = begin;
@@ -935,26 +944,22 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
             if (!single || !takes_long_kernel((int)s, i)) r->first_bytes[s] += sd.data_end - sd.data_off;
         }
     // the pairs' items: sixteen intervals of one image
-    r->pair_begin.assign((size_t)r->n_slices * G, 0); r->pair_count.assign((size_t)r->n_slices * G, 0);
+    r->pair_chain_bytes.assign(G, 0); r->pair_begin.assign((size_t)r->n_slices * G, 0); r->pair_count.assign((size_t)r->n_slices * G, 0);
     for (int g = 0; g < r->n_slices; ++g)
         for (uint32_t s = 0; s < G; ++s) {
             const uint32_t begin = n_items;
             for (uint32_t pos = r->slice_img[g]; r->pair_of[s] >= 0 && pos < r->slice_img[g + 1]; ++pos) {
                 const uint32_t i = order[pos], a = (uint32_t)r->pair_of[s];
                 if (single && takes_long_kernel((int)s, i)) continue;
-                const uint32_t nseg = nsegs[(size_t)s * N + i];
-                for (uint32_t j = 0; j < nseg; j += kSegsPerItem / 2)
+                const uint32_t nseg = nsegs[(size_t)s * N + i], longer = std::max(chains[(size_t)s * N + i], chains[(size_t)a * N + i]);
+                for (uint32_t j = 0; j < nseg; j += kSegsPerItem / 2) {
                     items[n_items++] = Item{a * N + i, j, std::min<uint32_t>(kSegsPerItem / 2, nseg - j), 0u, (s - a) * N};
+                    r->pair_chain_bytes[s] += longer;
+                }
             }
             r->pair_begin[(size_t)g * G + s] = begin;
             r->pair_count[(size_t)g * G + s] = n_items - begin;
         }
-    // Pairs shorten the chain but leave the lanes of the shorter scan idle (about 1.4 times the warp instructions for the
-    // ten-scan script), so they are for records whose waves fit the machine, or nearly: it holds 18 lane-per-interval warps of 36 KB
-    // a three an SM, and up to 20 an SM the few that wait cost less than the chain gains.  (Measured with an earlier step of the chains,
-    // without and with pairs, by warps an SM, decode at k = 10 in us: ImageNet-shaped images 17.2 656 and 639, 19.1 679 and 669, 20.8 700 and
-    // 700, 20.9 707 and 728, 23.6 775 and 778, 34 957 and 997; CelebA-shaped 18.2 452 and 441.  Raised 2 -> 10: 17.2 642 and 555, 34
-    // 834 and 853.)
     if (on_device && cudaDeviceGetAttribute(&r->n_sms, cudaDevAttrMultiProcessorCount, r->device) != cudaSuccess) return PCR_E_CUDA;
     for (const std::vector<int>& scans_of_wave : r->paired_waves) {
         std::vector<char> in_pair(G, 0);
@@ -966,7 +971,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
                 n += r->pair_count[(size_t)g * G + s] + (in_pair[s] ? 0u : r->item_count[(size_t)g * G + s]);
                 any = any || in_pair[s];
             }
-        if (any && n > 20ull * (uint64_t)r->n_sms) r->pairs_fit = false;
+        if (any && n > 20ull * (uint64_t)r->n_sms) r->pairs_fit = false;      // (see pairs_pay)
     }
     // pixel work units (see Sampling in pcr_pixels.cuh), image by image in processing order, inside an image
     // MCU row by MCU row.  The host only counts them; a small kernel writes the list at set-up.
@@ -1062,9 +1067,9 @@ uint64_t hash_bytes(uint64_t h, const uint8_t* p, size_t n) {
 }
 uint32_t env_key() {
     uint32_t h = 0;
-    for (const char* name : {"PCR_SLICES", "PCR_LONG_MIN_BYTES", "PCR_REFINE_CTAS", "PCR_PACK_WARPS", "PCR_SHORT_WARPS", "PCR_INDEX_CTAS", "PCR_LONG_CTAS"}) {
+    for (const char* name : {"PCR_SLICES", "PCR_LONG_MIN_BYTES", "PCR_PAIRS", "PCR_REFINE_CTAS", "PCR_PACK_WARPS", "PCR_SHORT_WARPS", "PCR_INDEX_CTAS", "PCR_LONG_CTAS"}) {
         const char* v = getenv(name);
-        h = h * 1000003u + (v ? (uint32_t)atoi(v) + 1u : 0u);
+        for (h = h * 1000003u + (v ? 1u : 0u); v && *v; ++v) h = h * 1000003u + (uint8_t)*v;
     }
     return h;
 }
@@ -1289,23 +1294,56 @@ static bool allow_refine_smem(int device) {
     return true;
 }
 
-// Whether refine_kernel's CTAs take the AC refinements among scans k0 .. k-1 of a wave, or lane-per-interval warps of
-// entropy_kernel.  A CTA's chains are several times as fast (170 to 220 cycles a symbol), but three CTAs are all an SM
-// holds, 96 chains against 480, so a launch of many items is better off with the warps.  Decode at k = 10 in us,
-// warps and CTAs, by CTAs an SM: ImageNet-shaped images 2.9 261 and 217, 4.9 357 and 339, 7.8 415 and 362, 9.7 463 and 476, 11.7 508 and
-// 551; CelebA-shaped 2.5 162 and 158, 10 289 and 336, 20 439 and 491; mixed sizes in 4:4:4 2.3 293 and 219, 6.2 345 and 269; raised
-// 2 -> 10 3.9 385 and 322, 7.8 434 and 436.
-static bool refine_in_ctas(const pcr_record* rec, const std::vector<int>& wave, bool paired, int k0, int k) {
-    uint64_t ctas = 0;
+// The AC refinements among scans k0 .. k-1 of a wave in items an SM, an item counting by how long its scan's chains are on average
+// (a chroma scan's are a third of luminance's).
+//
+// refine_kernel's CTAs take them up to four (rec->refine_ctas), lane-per-interval warps of entropy_kernel beyond.  A CTA's
+// chains are several times as fast (170 to 220 cycles a symbol), but three CTAs are all an SM holds, 96 chains against 480.  Decode in us,
+// CTAs and warps, by this number.  k = 9, one wave: ImageNet-shaped images 0.9 145 and 168, 2.6 213 and 226, 3.4 217 and 228, 4.0 262
+// and 281, 4.2 288 and 282, 5.3 330 and 302, 6.9 421 and 362; CelebA-shaped 3.2 170 and 180, 3.8 187 and 187, 4.3 206 and 196;
+// HAM-shaped 2.1 234 and 256, 3.1 304 and 312, 4.0 357 and 334.  k = 6, luminance alone: ImageNet-shaped 2.9 237 and 241, 3.9 291 and 283,
+// 4.4 314 and 299, 7.7 503 and 448; CelebA-shaped 3.0 187 and 191, 4.5 245 and 241; 32x32 3.5 85 and 85, 6.9 116 and 114.
+static double refine_load(const pcr_record* rec, const std::vector<int>& wave, bool paired, int k0, int k) {
+    double sum = 0, longest = 0;
     std::vector<char> counted(rec->G, 0);                     // scans that a pair's items stand for
     for (int s : wave)
         if (paired && s < k && rec->pair_of[s] >= k0) counted[rec->pair_of[s]] = 1;
     for (int s : wave) {
         if (s < k0 || s >= k || rec->script[s].Ss == 0 || rec->script[s].Ah == 0 || counted[s]) continue;
-        const std::vector<uint32_t>& items = paired && rec->pair_of[s] >= k0 ? rec->pair_count : rec->item_count;
-        for (int g = 0; g < rec->n_slices; ++g) ctas += items[(size_t)g * rec->G + s];
+        const bool pair = paired && rec->pair_of[s] >= k0;
+        uint64_t items = 0;
+        for (int g = 0; g < rec->n_slices; ++g) items += (pair ? rec->pair_count : rec->item_count)[(size_t)g * rec->G + s];
+        const double bytes = (double)std::max<uint64_t>(items, (pair ? rec->pair_chain_bytes : rec->chain_bytes)[s]);
+        sum += bytes;
+        if (items) longest = std::max(longest, bytes / (double)items);
     }
-    return ctas <= (uint64_t)rec->refine_ctas * (uint64_t)rec->n_sms;
+    return sum > 0 ? sum / longest / rec->n_sms : 0;
+}
+
+// Behind another wave of refinements the line lies further out: the slices of the record get there one after the other.  Decode at k = 10 in us
+// with the later wave (luminance alone) in CTAs and in warps: ImageNet-shaped 4.4 468 and 537, 5.1 554 and 613, 6.2 603 and 609, 7.7 733
+// and 710; CelebA-shaped 4.5 356 and 368, 6.1 455 and 446; greyscale 5.1 485 and 546; HAM-shaped 4.6 626 and 578.
+static double refine_line(const pcr_record* rec, bool paired, bool later) { return rec->refine_ctas * (paired ? 1.125 : (later ? 1.6 : 1.0)); }
+
+// Whether refinements that follow one another are decoded in pairs (see refine_kernel).  Pairs shorten the chain but leave the lanes
+// of the shorter scan idle.  In CTAs they pay while these are about four an SM; beyond, the two waves are faster one after the other as
+// long as the later one's CTAs are.  Where that one goes to the warps too, both ways differ little until the machine is full: it holds 18
+// lane-per-interval warps of 36 KB a three an SM, and up to 20 the few that wait cost less than the chain gains.  Decode at k = 10 in us by
+// CTAs an SM.  Pairs in CTAs and no pairs: ImageNet-shaped images 1.6 197 and 225, 3.1 277 and 307, 3.9 340 and 320, 4.7 367 and 330, 6.1
+// 366 and 339, 7.7 479 and 400; CelebA-shaped 1.9 163 and 163, 2.8 177 and 187, 3.8 213 and 196, 5.6 262 and 235; HAM-shaped 1.8 236 and
+// 258, 2.7 265 and 296, 3.6 372 and 342; greyscale 2.9 240 and 266, 4.4 327 and 285; 4:4:4 2.0 223 and 252, 3.9 371 and 405, 5.8 490 and 451;
+// mixed sizes 1.3 212 and 254, 4.4 256 and 280, 9.8 446 and 371.  Pairs in warps and no pairs: ImageNet-shaped 9.5 515 and 438, 10.7 531 and
+// 468, 12.5 584 and 554, 15 661 and 603, 19 764 and 710; CelebA-shaped 9.4 328 and 313, 11.2 360 and 356; HAM-shaped 7.2 447 and 458, 10.7 582
+// and 626.
+static bool pairs_pay(const pcr_record* rec, int k0, int k) {
+    auto holds = [&](const std::vector<int>& wave) {          // the later scan of a pair of this call
+        for (int s : wave) if (s < k && rec->pair_of[s] >= k0) return true;
+        return false;
+    };
+    bool ctas = true, warps = rec->pairs_fit;
+    for (const std::vector<int>& wave : rec->paired_waves) ctas = ctas && (!holds(wave) || refine_load(rec, wave, true, k0, k) <= refine_line(rec, true, false));
+    for (const std::vector<int>& wave : rec->wave_scans) warps = warps && (!holds(wave) || refine_load(rec, wave, false, k0, k) > refine_line(rec, false, true));
+    return ctas || warps;
 }
 
 // Form of entropy_kernel for the first passes among scans k0 .. k-1 of a wave: kFirstFull where there is so much to store that stores are
@@ -1384,7 +1422,8 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
     coef_lists(rec, k, &cl);
     // the waves of this call: with pairs of refinements when both scans of a pair are to be decoded
     bool paired = false;
-    for (int s = 0; s < k && rec->pairs_fit; ++s) paired = paired || (rec->pair_of[s] >= k0);
+    for (int s = 0; s < k; ++s) paired = paired || (rec->pair_of[s] >= k0);
+    if (paired) paired = rec->pairs < 0 ? pairs_pay(rec, k0, k) : rec->pairs != 0;
     const std::vector<std::vector<int>>& waves = paired ? rec->paired_waves : rec->wave_scans;
     const bool chains = fl.n[0] + fl.n[1] + fl.n[2] > 0 && rec->n_groups > 0;
     const int chain_depth = kChainPairs / 4;    // chains per scheduler of the chain launch
@@ -1509,7 +1548,10 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
                 ++g_launches;
                 refs.n = 0; ref_count = 0;
             };
-            const bool ctas = refine_in_ctas(rec, waves[w], paired, k0, k);
+            bool later = false;                            // a wave before this one holds refinements too
+            for (int v = 0; v < w; ++v)
+                for (int s : waves[v]) later = later || (s >= k0 && s < k && rec->script[s].Ss > 0 && rec->script[s].Ah != 0);
+            const bool ctas = refine_load(rec, waves[w], paired, k0, k) <= refine_line(rec, paired, later);
             auto add_run = [&](bool to_ctas, uint32_t first, uint32_t n) {
                 if (!n) return;
                 ItemRuns& to = to_ctas ? refs : runs;

@@ -1,6 +1,6 @@
 """AC refinements of scans with restart intervals, by the CTAs that take them in small launches and by the lane-per-interval
-warps of large ones (PCR_REFINE_CTAS, read when a record is opened, chooses): intervals of one block to several rows,
-runs of blocks that last a whole interval, blocks as long as the format allows, streams that are cut short."""
+warps of large ones (PCR_REFINE_CTAS, read when a record is opened, chooses), in pairs of scans and one after the other
+(PCR_PAIRS): intervals of one block to several rows, runs of blocks that last a whole interval, blocks as long as the format allows, streams that are cut short."""
 from __future__ import annotations
 
 import numpy as np
@@ -13,10 +13,11 @@ from test_gpu_kernel_edges import _compare, _field
 pytestmark = pytest.mark.gpu
 
 
+@pytest.mark.parametrize("pairs", [0, 1])
 @pytest.mark.parametrize("ctas", [0, 1 << 20])
 @pytest.mark.parametrize("fixed", [0, 1, 7, 150])
 @pytest.mark.parametrize("kind", ["dense", "wide", "sparse", "empty"])
-def test_blocks_and_intervals(kind, fixed, ctas, monkeypatch):
+def test_blocks_and_intervals(kind, fixed, ctas, pairs, monkeypatch):
     """fixed: MCUs an interval (0: a row).  dense: every block takes nearly as many bits as one can; wide: rows of 90 blocks,
     a few rounds of lists; sparse and empty: end-of-band runs over blocks, rows and whole intervals."""
     rng = np.random.default_rng(fixed)
@@ -25,6 +26,7 @@ def test_blocks_and_intervals(kind, fixed, ctas, monkeypatch):
     coeffs = [_field(rng, pcr_synth.num_blocks(w, h), density, 1023 if kind == "dense" else 20) for w, h in dims]
     rec = pcr_synth.record_from_coeffs(dims, coeffs, restart_rows=fixed == 0, restart_fixed=fixed)
     monkeypatch.setenv("PCR_REFINE_CTAS", str(ctas))
+    monkeypatch.setenv("PCR_PAIRS", str(pairs))
     _compare(rec, (6, 9, 10))
 
 
