@@ -191,6 +191,7 @@ struct pcr_record {
     std::vector<uint32_t> slice_img;                            // [n_slices + 1] first image of each slice
     std::vector<uint32_t> slice_unit;                           // [n_slices + 1] first pixel unit of each slice
     std::vector<uint32_t> item_begin, item_count;               // [n_slices][G]
+    std::vector<uint32_t> longest;                              // by scan: entropy-coded bytes of the image that has most
     std::vector<uint64_t> first_bytes;                          // of AC first passes: entropy-coded bytes that items stand for
     // Scans that are one long restart interval take kernels of their own (pcr_long.cuh): first passes
     // as (scan, image) pairs sorted by (slice, wave, scan); AC refinements as (component, image)
@@ -220,7 +221,7 @@ struct pcr_record {
     int pairs = -1;                                             // see pairs_pay (PCR_PAIRS overrides: 0 never, 1 always)
     double refine_ctas = 4;                                     // see refine_load (PCR_REFINE_CTAS overrides)
     uint32_t long_ctas = 3;                                     // see wide_long_scans (PCR_LONG_CTAS overrides)
-    uint32_t index_ctas = 8;                                    // see launch_index_kernel (PCR_INDEX_CTAS overrides)
+    int64_t index_ctas = -1;                                    // see launch_index_kernel (PCR_INDEX_CTAS: a line in pairs an SM instead)
     int64_t pack_warps = -1;                                    // see first_pass_form (PCR_PACK_WARPS: a line in warps an SM instead)
     uint32_t short_warps = 20;                                  // see first_pass_form (PCR_SHORT_WARPS overrides)
     // Items of the AC refinements: the sum of their chains' bytes, an item counting with its longest.  By scan; by the pair's later scan
@@ -556,7 +557,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     r->script.resize(G);
     // every image's chunks are walked independently (a few host threads for large records); the
     // running sums over images follow in one serial pass
-    std::vector<uint32_t> nsegs((size_t)G * N), image_bytes(N);      // restart intervals by (scan, image); entropy-coded bytes
+    std::vector<uint32_t> nsegs((size_t)G * N), lens((size_t)G * N), image_bytes(N);      // restart intervals and entropy-coded bytes by (scan, image)
     std::vector<uint32_t> chains((size_t)G * N);                     // of AC refinements: bytes of an interval, on average
     std::vector<uint8_t> one_interval(N, 0);                         // some scan of the image is one restart interval
     uint8_t sampling0 = 0;
@@ -601,7 +602,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
                 total_mcu = (uint64_t)((wc + 7) / 8) * ((hc + 7) / 8);
             }
             sd.nseg = sd.ri ? (uint32_t)((total_mcu + sd.ri - 1) / sd.ri) : 1u;
-            nsegs[(size_t)g * N + i] = sd.nseg;
+            nsegs[(size_t)g * N + i] = sd.nseg; lens[(size_t)g * N + i] = sd.data_end - sd.data_off;
             if (sp.sc.Ss > 0 && sp.sc.Ah != 0) chains[(size_t)g * N + i] = (sd.data_end - sd.data_off) / std::max(1u, sd.nseg);
             if (sd.nseg == 1) one_interval[i] = 1;
             sum += sd.data_end - sd.data_off;
@@ -812,7 +813,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     }
     if (const char* e = getenv("PCR_REFINE_CTAS")) r->refine_ctas = atof(e);
     if (const char* e = getenv("PCR_PAIRS")) r->pairs = atoi(e) != 0;
-    if (const char* e = getenv("PCR_INDEX_CTAS")) r->index_ctas = (uint32_t)std::max(0, atoi(e));
+    if (const char* e = getenv("PCR_INDEX_CTAS")) r->index_ctas = std::max(0, atoi(e));
     if (const char* e = getenv("PCR_LONG_CTAS")) r->long_ctas = (uint32_t)std::max(0, atoi(e));
     if (const char* e = getenv("PCR_PACK_WARPS")) r->pack_warps = std::max(0, atoi(e));
     if (const char* e = getenv("PCR_SHORT_WARPS")) r->short_warps = (uint32_t)std::max(0, atoi(e));
@@ -937,12 +938,15 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
                 r->item_begin[(size_t)g * G + s] = begin;
                 r->item_count[(size_t)g * G + s] = n_items - begin;
             }
-    r->first_bytes.assign(G, 0);
-    for (uint32_t s = 0; s < G; ++s)
-        for (uint32_t i = 0; r->script[s].Ss > 0 && r->script[s].Ah == 0 && i < N; ++i) {
-            const ScanDesc& sd = scans[(size_t)s * N + i];
-            if (!single || !takes_long_kernel((int)s, i)) r->first_bytes[s] += sd.data_end - sd.data_off;
+    r->first_bytes.assign(G, 0); r->longest.assign(G, 0);
+    for (uint32_t s = 0; s < G; ++s) {
+        const bool first = r->script[s].Ss > 0 && r->script[s].Ah == 0;
+        for (uint32_t i = 0; i < N; ++i) {
+            const uint32_t bytes = lens[(size_t)s * N + i];
+            r->longest[s] = std::max(r->longest[s], bytes);
+            if (first && !(single && takes_long_kernel((int)s, i))) r->first_bytes[s] += bytes;
         }
+    }
     // the pairs' items: sixteen intervals of one image
     r->pair_chain_bytes.assign(G, 0); r->pair_begin.assign((size_t)r->n_slices * G, 0); r->pair_count.assign((size_t)r->n_slices * G, 0);
     for (int g = 0; g < r->n_slices; ++g)
@@ -1458,9 +1462,16 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
         bool tables = false;
         for (int i = 0; i < sl.n; ++i)
             for (int g = 0; g < rec->n_slices; ++g) tables = tables || rec->item_count[(size_t)g * rec->G + sl.s[i]] + rec->long_count[(size_t)g * rec->G + sl.s[i]] > 0;
-        // eight CTAs of this size are what an SM holds; decode in us with a warp and with a CTA a pair, by pairs an SM: 64 ImageNet-shaped
-        // images at k = 10 4.3 214 and 195, 256 8.6 (two waves side by side) 425 and 459, 1024 baseline JPEGs 6.9 753 and 683
-        const bool split = pairs <= (uint32_t)rec->index_ctas * (uint32_t)rec->n_sms;
+        // A CTA a pair while an SM has few of them (it holds eight) and the longest scan of the launch is long enough for eight warps.  Decode in us
+        // with a warp and with a CTA a pair, by pairs an SM and bytes of the longest scan: 64 ImageNet-shaped images at k = 10 4.3 5 k 227 and
+        // 199, 256 (two waves side by side) 8.6 5 k 425 and 459, baseline 128 0.9 30 k 293 and 219, 1024 6.9 753 and 682, k = 1 768 5.2
+        // 4 k equal, 1024 (no markers) 6.9 226 and 228; CelebA-shaped k = 1 512 3.5 1.2 k 62 and 64, 1024 6.9 87 and 92, k = 5 (no
+        // markers) 128 4.3 2 k 180 and 182; 96 of mixed sizes (no markers) 3.2 8 k 180 and 162; 512 of 64x64 k = 1 3.5 0.3 k 36 and 39; 1024 of
+        // 32x32 6.9 0.3 k 38 and 41.
+        uint64_t bytes = 0;
+        for (int i = 0; i < sl.n; ++i) bytes = std::max<uint64_t>(bytes, rec->longest[sl.s[i]]);
+        const uint64_t sms = (uint64_t)rec->n_sms;
+        const bool split = rec->index_ctas >= 0 ? pairs <= (uint64_t)rec->index_ctas * sms : pairs <= 8 * sms && pairs <= bytes * sms / 700;
         const uint32_t nb = split ? pairs : (pairs + kIndexWarps - 1) / kIndexWarps, nt = tables ? (4 * pairs + kIndexWarps - 1) / kIndexWarps : 0;
         if (split) unstuff_index_kernel<true><<<nb + nt, 32 * kIndexWarps, 0, q>>>(P, sl, 0, rec->N, nb);
         else unstuff_index_kernel<false><<<nb + nt, 32 * kIndexWarps, 0, q>>>(P, sl, 0, rec->N, nb);
