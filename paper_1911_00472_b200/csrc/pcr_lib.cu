@@ -191,7 +191,8 @@ struct pcr_record {
     std::vector<uint32_t> slice_img;                            // [n_slices + 1] first image of each slice
     std::vector<uint32_t> slice_unit;                           // [n_slices + 1] first pixel unit of each slice
     std::vector<uint32_t> item_begin, item_count;               // [n_slices][G]
-    std::vector<uint32_t> longest;                              // by scan: entropy-coded bytes of the image that has most
+    std::vector<uint32_t> longest, longest_chain;               // by scan: entropy-coded bytes, and bytes of an interval, of the image that has most
+    std::vector<uint64_t> intervals;                            // by scan
     std::vector<uint64_t> first_bytes;                          // of AC first passes: entropy-coded bytes that items stand for
     // Scans that are one long restart interval take kernels of their own (pcr_long.cuh): first passes
     // as (scan, image) pairs sorted by (slice, wave, scan); AC refinements as (component, image)
@@ -221,10 +222,11 @@ struct pcr_record {
     int pairs = -1;                                             // see pairs_pay (PCR_PAIRS overrides: 0 never, 1 always)
     double refine_ctas = 4;                                     // see refine_load (PCR_REFINE_CTAS overrides)
     uint32_t long_ctas = 3;                                     // see wide_long_scans (PCR_LONG_CTAS overrides)
+    int64_t seq_ctas = -1;                                      // see sequential_in_ctas (PCR_SEQ_CTAS: a line in items an SM instead)
     int64_t index_ctas = -1;                                    // see launch_index_kernel (PCR_INDEX_CTAS: a line in pairs an SM instead)
     int64_t pack_warps = -1;                                    // see first_pass_form (PCR_PACK_WARPS: a line in warps an SM instead)
     uint32_t short_warps = 20;                                  // see first_pass_form (PCR_SHORT_WARPS overrides)
-    // Items of the AC refinements: the sum of their chains' bytes, an item counting with its longest.  By scan; by the pair's later scan
+    // Items of the AC refinements (and of a sequential scan): the sum of their chains' bytes, an item counting with its longest.  By scan; by the pair's later scan
     std::vector<uint64_t> chain_bytes, pair_chain_bytes;
     std::vector<uint32_t> pair_begin, pair_count;               // [n_slices][G] items of the pair, by its later scan
     uint32_t n_units = 0;
@@ -558,7 +560,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     // every image's chunks are walked independently (a few host threads for large records); the
     // running sums over images follow in one serial pass
     std::vector<uint32_t> nsegs((size_t)G * N), lens((size_t)G * N), image_bytes(N);      // restart intervals and entropy-coded bytes by (scan, image)
-    std::vector<uint32_t> chains((size_t)G * N);                     // of AC refinements: bytes of an interval, on average
+    std::vector<uint32_t> chains((size_t)G * N);                     // of AC refinements and sequential scans: bytes of an interval, on average
     std::vector<uint8_t> one_interval(N, 0);                         // some scan of the image is one restart interval
     uint8_t sampling0 = 0;
     auto parse_image = [&](uint32_t i) -> int {
@@ -603,7 +605,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
             }
             sd.nseg = sd.ri ? (uint32_t)((total_mcu + sd.ri - 1) / sd.ri) : 1u;
             nsegs[(size_t)g * N + i] = sd.nseg; lens[(size_t)g * N + i] = sd.data_end - sd.data_off;
-            if (sp.sc.Ss > 0 && sp.sc.Ah != 0) chains[(size_t)g * N + i] = (sd.data_end - sd.data_off) / std::max(1u, sd.nseg);
+            if (sp.sc.Ss > 0 ? sp.sc.Ah != 0 : sp.sc.Se == 63) chains[(size_t)g * N + i] = (sd.data_end - sd.data_off) / std::max(1u, sd.nseg);
             if (sd.nseg == 1) one_interval[i] = 1;
             sum += sd.data_end - sd.data_off;
         }
@@ -813,6 +815,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     }
     if (const char* e = getenv("PCR_REFINE_CTAS")) r->refine_ctas = atof(e);
     if (const char* e = getenv("PCR_PAIRS")) r->pairs = atoi(e) != 0;
+    if (const char* e = getenv("PCR_SEQ_CTAS")) r->seq_ctas = std::max(0, atoi(e));
     if (const char* e = getenv("PCR_INDEX_CTAS")) r->index_ctas = std::max(0, atoi(e));
     if (const char* e = getenv("PCR_LONG_CTAS")) r->long_ctas = (uint32_t)std::max(0, atoi(e));
     if (const char* e = getenv("PCR_PACK_WARPS")) r->pack_warps = std::max(0, atoi(e));
@@ -938,12 +941,14 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
                 r->item_begin[(size_t)g * G + s] = begin;
                 r->item_count[(size_t)g * G + s] = n_items - begin;
             }
-    r->first_bytes.assign(G, 0); r->longest.assign(G, 0);
+    r->first_bytes.assign(G, 0); r->longest.assign(G, 0); r->longest_chain.assign(G, 0); r->intervals.assign(G, 0);
     for (uint32_t s = 0; s < G; ++s) {
         const bool first = r->script[s].Ss > 0 && r->script[s].Ah == 0;
         for (uint32_t i = 0; i < N; ++i) {
             const uint32_t bytes = lens[(size_t)s * N + i];
             r->longest[s] = std::max(r->longest[s], bytes);
+            r->longest_chain[s] = std::max(r->longest_chain[s], chains[(size_t)s * N + i]);
+            r->intervals[s] += nsegs[(size_t)s * N + i];
             if (first && !(single && takes_long_kernel((int)s, i))) r->first_bytes[s] += bytes;
         }
     }
@@ -1071,7 +1076,7 @@ uint64_t hash_bytes(uint64_t h, const uint8_t* p, size_t n) {
 }
 uint32_t env_key() {
     uint32_t h = 0;
-    for (const char* name : {"PCR_SLICES", "PCR_LONG_MIN_BYTES", "PCR_PAIRS", "PCR_REFINE_CTAS", "PCR_PACK_WARPS", "PCR_SHORT_WARPS", "PCR_INDEX_CTAS", "PCR_LONG_CTAS"}) {
+    for (const char* name : {"PCR_SLICES", "PCR_LONG_MIN_BYTES", "PCR_PAIRS", "PCR_REFINE_CTAS", "PCR_PACK_WARPS", "PCR_SHORT_WARPS", "PCR_SEQ_CTAS", "PCR_INDEX_CTAS", "PCR_LONG_CTAS"}) {
         const char* v = getenv(name);
         for (h = h * 1000003u + (v ? 1u : 0u); v && *v; ++v) h = h * 1000003u + (uint8_t)*v;
     }
@@ -1369,6 +1374,20 @@ static int first_pass_form(const pcr_record* rec, const std::vector<int>& wave, 
     return warps > (uint64_t)rec->short_warps * sms ? kFirstShort : kFirstFew;
 }
 
+// Whether sequential_kernel's CTAs take the sequential scan's items or sequential_lane_kernel's warps.  A CTA's chains are five times as fast,
+// but an SM holds four CTAs and eighteen warps, and a CTA costs the same whether its lanes are in use or not: the warps are better where
+// images have few intervals and there are many images, by the items an SM in units of the longest chain.  Decode in us, CTAs and warps:
+// CelebA-shaped images (14 lanes in use) 3.8 350 and 467, 5.1 450 and 513, 7.0 596 and 612, 7.6 642 and 629, 10.1 833 and 741, 15 1224 and
+// 1049; 64x64 (4) 6.3 120 and 145, 9.5 172 and 169, 12.6 210 and 198; 96x96 (6) 9.6 226 and 227, 12.7 285 and 268; 32x32 (2) 5.6 88 and 102,
+// 10.5 135 and 133, 20.7 236 and 214; mixed sizes (12) 3.1 622 and 1114; HAM-shaped (29) 3.6 972 and 1080, 7.3 1931 and 2182; ImageNet-shaped (23)
+// 3.9 682 and 960, 8.0 1343 and 1417, 4:4:4 13.4 1853 and 1878.
+static bool sequential_in_ctas(const pcr_record* rec, int s) {
+    uint64_t items = 0;
+    for (int g = 0; g < rec->n_slices; ++g) items += rec->item_count[(size_t)g * rec->G + s];
+    if (rec->seq_ctas >= 0) return items <= (uint64_t)rec->seq_ctas * (uint64_t)rec->n_sms;
+    return rec->intervals[s] >= 20 * items || (double)rec->chain_bytes[s] <= 7.4 * rec->n_sms * rec->longest_chain[s];
+}
+
 // Whether the long scans of a wave that are first passes (or sequential) get CTAs of four times as many warps: while
 // most of the machine is idle; beyond, the narrow ones do less in all.  Decode at k = 5 in us, narrow and wide, by CTAs
 // an SM: HAM-shaped images 2 242 and 184, 4.4 between 265 and 300
@@ -1588,8 +1607,12 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
             const uint32_t begin = runs.n ? runs.first[0] : 0u;
             if (sequential) {
                 if (count) {
-                    if (roi) sequential_kernel<true><<<count, 32 * kSeqWarps, 0, q>>>(P, begin);
-                    else sequential_kernel<false><<<count, 32 * kSeqWarps, 0, q>>>(P, begin);
+                    const unsigned nl = (count + kSeqLaneWarps - 1) / kSeqLaneWarps;
+                    if (sequential_in_ctas(rec, waves[w][0])) {
+                        if (roi) sequential_kernel<true><<<count, 32 * kSeqWarps, 0, q>>>(P, begin);
+                        else sequential_kernel<false><<<count, 32 * kSeqWarps, 0, q>>>(P, begin);
+                    } else if (roi) sequential_lane_kernel<true><<<nl, 32 * kSeqLaneWarps, 0, q>>>(P, begin, count);
+                    else sequential_lane_kernel<false><<<nl, 32 * kSeqLaneWarps, 0, q>>>(P, begin, count);
                     ++g_launches;
                 }
                 const int s0 = waves[w][0];      // the record's one scan

@@ -11,7 +11,7 @@
 //
 // Bound by warp 0's step: a window, a table entry, and where both lead next, 125 cycles a symbol (a lane that did everything
 // itself took 600), then by the warps of four CTAs an SM sharing its schedulers.  1024 ImageNet-shaped images 742 -> 437 us, 64
-// such images 713 -> 177 us.  (A step with a predicate for every case 180 cycles; both possible tables looked up and one entry
+// such images 713 -> 177 us; launches of many images with few intervals keep a lane an interval (at the end of the file).  (A step with a predicate for every case 180 cycles; both possible tables looked up and one entry
 // chosen afterwards: 189 us; 6 or 12 warps a CTA: 183, 181 us and 467, 460; rounds of 48 symbols 184, of 96 equal.)
 #pragma once
 #include <cuda_runtime.h>
@@ -254,6 +254,142 @@ __global__ void __launch_bounds__(32 * kSeqWarps, 4) sequential_kernel(Params P,
             if (M0 | M1) *reinterpret_cast<uint4*>(auxp + 2ull * blk) = value_record(M0, M1, vb);
         }
         meet();
+    }
+    if (bad) atomicMin(&P.status[img], kErrCorrupt);
+}
+
+// ---------------------------------------------------------------------------------------
+// The same, one lane per restart interval, for launches of many items (see sequential_in_ctas): a warp an item instead of eight, 18
+// items an SM instead of four.  Lanes stand at different kinds of symbol in every step, so a block's first symbol goes through the same
+// instructions as the others (its value is the difference), stores are predicated, and what changes from block to block comes
+// from a small table in shared memory.  Bound by the length of a lane's chain, 600 cycles a symbol.
+// ---------------------------------------------------------------------------------------
+constexpr int kSeqLaneWarps = 2;
+constexpr uint32_t kSeqLaneRing = 4 * sizeof(ScanTab), kSeqLanePlaces = kSeqLaneRing + (kRingWords + 2) * 128, kSeqLanePreds = kSeqLanePlaces + 8 * 16;
+constexpr uint32_t kSeqLaneBytes = kSeqLanePreds + 3 * 128;
+
+template <bool kRoi>
+__global__ void __launch_bounds__(32 * kSeqLaneWarps) sequential_lane_kernel(Params P, uint32_t item_begin, uint32_t item_count) {
+    __shared__ __align__(16) uint8_t s_seq[kSeqLaneWarps * kSeqLaneBytes];
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t it = blockIdx.x * kSeqLaneWarps + wid;
+    if (it >= item_count) return;                             // whole warp
+    const Item item = P.items[item_begin + it];
+    const ScanDesc sd = load_entry(P.scans + item.si);
+    const int img = (int)(item.si % (uint32_t)P.N);
+    const ScanAux ax = load_entry(P.saux + item.si / (uint32_t)P.N);
+    bool done = (uint32_t)lane >= item.count;
+    uint32_t seg = item.seg0 + lane;
+    if (seg >= sd.nseg) { done = true; seg = 0; }
+    const ImgDesc im = load_entry(P.imgs + img);
+    const uint32_t mcu_w = im.mx, total = im.mx * im.my;
+    const uint32_t m0 = sd.ri ? seg * sd.ri : 0;
+    const uint32_t m1 = sd.ri ? min(m0 + sd.ri, total) : total;
+    const unsigned full = 0xffffffffu;
+    if (kRoi) {
+        if (!done && m1 > m0) {
+            const CropRect rc = P.roi[img];
+            const uint32_t mh = 8u * (uint32_t)P.vs;                       // pixel rows of an MCU row
+            const uint32_t lo = mh * (rc.y0 / mh), hi = mh * ((rc.y0 + rc.h + mh - 1u) / mh);
+            const uint32_t r0 = m0 / mcu_w, r1 = (m1 - 1u) / mcu_w;
+            if ((r1 + 1u) * mh <= lo || r0 * mh >= hi) done = true;
+        }
+        if (__all_sync(full, done)) return;
+    }
+    const uint32_t mem = (uint32_t)__cvta_generic_to_shared(s_seq) + (uint32_t)wid * kSeqLaneBytes;
+    const uint32_t hs = (uint32_t)P.hs, vs = (uint32_t)P.vs, bw0 = hs * mcu_w;
+    const uint32_t ny = hs * vs, bpm = P.nc == 3 ? ny + 2u : 1u;      // blocks per MCU (a lone component: one block, no padding)
+    {
+        const uint4* a = reinterpret_cast<const uint4*>(P.tabs + ax.tab0 + 4u * (uint32_t)img);
+        for (int i = lane; i < (int)(4 * sizeof(ScanTab) / 16); i += 32) sts128(mem + 16 * i, __ldg(a + i));
+        // per block of the MCU: its two tables (shared addresses), where its predictor lies, its block number
+        // relative to the MCU's first luminance block or to the MCU's chroma place (bit 31)
+        if ((uint32_t)lane < bpm) {
+            const uint32_t j = (uint32_t)lane, c = j < ny ? 0u : j - ny + 1u;
+            const uint32_t tdc = mem + ((sd.slots >> (2u * c)) & 1u) * (uint32_t)sizeof(ScanTab);
+            const uint32_t tac = mem + (2u + ((sd.slots_ac >> (2u * c)) & 1u)) * (uint32_t)sizeof(ScanTab);
+            const uint32_t off = c ? (ny * total + (c - 1u) * total) | 0x80000000u : (j >> (hs - 1u)) * bw0 + (j & (hs - 1u));
+            sts128(mem + kSeqLanePlaces + 16u * j, make_uint4(tdc, tac, mem + kSeqLanePreds + 128u * c, off));
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) sts32(mem + kSeqLanePreds + 128u * c + 4u * lane, 0u);
+    }
+    const uint32_t* segtab = P.seg_start + sd.seg_base;
+    uint32_t bstart = segtab[seg];
+    uint32_t bend = segtab[seg + 1] - 2;
+    bool bad = false;
+    if (!done && (bstart < sd.data_off || bend > sd.data_end || bend < bstart)) { bad = true; done = true; }
+    if (done) { bstart = sd.data_off; bend = sd.data_off; }
+    LaneBits br;
+    br.init(mem + kSeqLaneRing + 4u * lane, P.ubuf, bstart, bend);
+    if (m0 >= m1) done = true;
+
+    uint32_t m = m0, wrap_m = (m0 / mcu_w + 1u) * mcu_w;       // MCU, the first one of the next row
+    uint32_t my = (m0 / mcu_w) * vs * bw0 + hs * (m0 % mcu_w); // block number of the MCU's first luminance block (its chroma place is m)
+    const uint32_t my_wrap = (vs - 1u) * bw0;                  // what a new row adds beside hs per MCU
+    uint32_t place = mem + kSeqLanePlaces;                     // of the current block in the table
+    const uint32_t place_end = place + 16u * bpm;
+    uint32_t k = 0, M0 = 0, M1 = 0;                            // position (0: the block's DC symbol comes next), mask
+    int16_t* vp = P.vals + 4ull * bstart;                      // next value
+    int16_t* vb = vp;                                          // the block's first one
+    int16_t* dcp = P.dc + im.blk_base;
+    int16_t* headp = P.head + im.blk_base * 8;
+    uint64_t* auxp = P.aux + ax.base + im.blk_base * 2;
+    pin(dcp); pin(headp); pin(auxp);
+    uint32_t tdc = 0, tac = 0, pred = 0, blk = 0;
+    auto take = [&]() {
+        const uint4 v = lds128(place);
+        tdc = v.x; tac = v.y; pred = v.z + 4u * lane;
+        blk = (v.w & 0x7FFFFFFFu) + ((v.w >> 31) ? m : my);
+    };
+    bool fresh = true;
+    for (;;) {
+        br.topup(!done);
+        __syncwarp(full);
+        if (__all_sync(full, done)) break;
+        if (fresh) { take(); fresh = false; }
+        uint32_t stop = done ? 0u : min(br.ring_stop(2), br.limit + 1u);
+#pragma unroll 1
+        for (int t = 0; t < kDecodeSteps; ++t) {
+            if (br.pos < stop) {
+                const uint32_t win = br.window(br.pos);
+                const bool is_dc = k == 0;
+                const uint32_t tab = is_dc ? tdc : tac;
+                uint32_t e = tab_entry(tab, win);
+                if (e == 0) {
+                    e = long_code(tab, win, is_dc ? kTabDcSeq : kTabAcSeq);
+                    if (e == 0) { bad = true; stop = 0; }
+                }
+                const uint32_t skip = e & 31u, sz = (e >> 5) & 15u;
+                br.pos += skip;
+                k += (e >> 9) & 31u;                                       // behind the coefficient
+                const uint32_t at = k - 1u;
+                int v = magnitude(win, skip, sz);
+                if (is_dc) { v += (int)lds32(pred); sts32(pred, (uint32_t)v); }
+                const bool coef = sz && k <= 64u, far = coef && k > 8u;
+                if (is_dc) dcp[blk] = (int16_t)v;                          // (stored even if there was no such symbol: the image is corrupt then)
+                if (coef && !far && !is_dc) headp[8u * (uint64_t)blk + at] = (int16_t)v;
+                if (far) *vp = (int16_t)v;
+                vp += far ? 1 : 0;
+                M0 |= shl0(far ? 1u : 0u, at); M1 |= shl0(far ? 1u : 0u, at - 32u);
+                if (sz && k > 64u && !is_dc) { bad = true; stop = 0; }
+                if ((e & kEntEob) || k > 63u) {                            // block finished
+                    if (M0 | M1) *reinterpret_cast<uint4*>(auxp + 2ull * blk) = value_record(M0, M1, vb);
+                    k = 0; M0 = 0; M1 = 0; vb = vp;
+                    place += 16u;
+                    if (place == place_end) {
+                        place = mem + kSeqLanePlaces;
+                        ++m; my += hs;
+                        if (m == wrap_m) { wrap_m += mcu_w; my += my_wrap; }
+                        if (m >= m1) stop = 0;
+                    }
+                    take();
+                }
+            }
+        }
+        __syncwarp(full);
+        bad = bad || br.pos > br.limit;
+        done = done || bad || m >= m1;
     }
     if (bad) atomicMin(&P.status[img], kErrCorrupt);
 }

@@ -1,6 +1,7 @@
-"""Baseline records with restart intervals, whose CTAs follow 32 intervals' symbols while other warps write the blocks: intervals
-of one MCU to several rows, blocks as long as the format allows and of two symbols, every chroma sampling (the blocks of an
-MCU change tables in different places), an interval that is damaged."""
+"""Baseline records with restart intervals, by CTAs that follow 32 intervals' symbols while other warps write the blocks and by the
+lane-per-interval warps of large launches (PCR_SEQ_CTAS, read when a record is opened, chooses): intervals of one MCU to several
+rows, blocks as long as the format allows and of two symbols, every chroma sampling (the blocks of an MCU change tables in
+different places), an interval that is damaged."""
 from __future__ import annotations
 
 import struct
@@ -15,10 +16,11 @@ from test_gpu_kernel_edges import _compare, _field
 pytestmark = pytest.mark.gpu
 
 
+@pytest.mark.parametrize("ctas", [0, 1 << 20])
 @pytest.mark.parametrize("samp", [(2, 2, 3), (2, 1, 3), (1, 2, 3), (1, 1, 3), (1, 1, 1)])
 @pytest.mark.parametrize("fixed", [0, 1, 5, 60])
 @pytest.mark.parametrize("kind", ["dense", "usual", "empty"])
-def test_blocks_and_intervals(kind, fixed, samp):
+def test_blocks_and_intervals(kind, fixed, samp, ctas, monkeypatch):
     """fixed: MCUs an interval (0: a row).  dense: blocks of up to 64 symbols of many bits; empty: two symbols a block, so that a
     round ends most blocks there can be."""
     rng = np.random.default_rng(fixed)
@@ -27,6 +29,7 @@ def test_blocks_and_intervals(kind, fixed, samp):
     with pcr_synth.sampling(*samp), pcr_synth.scan_script(pcr_synth.SCRIPT_BASELINE):
         coeffs = [_field(rng, pcr_synth.num_blocks(w, h), density, top) for w, h in dims]
         rec = pcr_synth.record_from_coeffs(dims, coeffs, restart_rows=fixed == 0, restart_fixed=fixed)
+    monkeypatch.setenv("PCR_SEQ_CTAS", str(ctas))
     _compare(rec, (1,))
 
 
@@ -42,7 +45,8 @@ def test_flat_rows(samp):
     _compare(rec, (1,))
 
 
-def test_damaged_interval():
+@pytest.mark.parametrize("ctas", [0, 1 << 20])
+def test_damaged_interval(ctas, monkeypatch):
     """The second half of one restart interval of one image replaced by ones (no code is all ones): that image is reported,
     the others' pixels are the oracle's."""
     import torch
@@ -62,6 +66,7 @@ def test_damaged_interval():
     begin = (first + end) // 2
     begin += (end - begin) % 2
     bad[off + begin:off + end] = np.tile(np.array([0xFF, 0], dtype=np.uint8), (end - begin) // 2)
+    monkeypatch.setenv("PCR_SEQ_CTAS", str(ctas))
     dec = Decoder(bad)
     try:
         out = dec.decode(1)
