@@ -192,7 +192,7 @@ struct pcr_record {
     std::vector<uint32_t> slice_unit;                           // [n_slices + 1] first pixel unit of each slice
     std::vector<uint32_t> item_begin, item_count;               // [n_slices][G]
     std::vector<uint32_t> longest, longest_chain;               // by scan: entropy-coded bytes, and bytes of an interval, of the image that has most
-    std::vector<uint64_t> intervals;                            // by scan
+    std::vector<uint64_t> intervals, long_bytes;                // by scan: intervals; entropy-coded bytes that kernels for long intervals read
     std::vector<uint64_t> first_bytes;                          // of AC first passes: entropy-coded bytes that items stand for
     // Scans that are one long restart interval take kernels of their own (pcr_long.cuh): first passes
     // as (scan, image) pairs sorted by (slice, wave, scan); AC refinements as (component, image)
@@ -221,7 +221,7 @@ struct pcr_record {
     bool pairs_fit = true;                                      // lane-per-interval warps of the waves with pairs fit the machine
     int pairs = -1;                                             // see pairs_pay (PCR_PAIRS overrides: 0 never, 1 always)
     double refine_ctas = 4;                                     // see refine_load (PCR_REFINE_CTAS overrides)
-    uint32_t long_ctas = 3;                                     // see wide_long_scans (PCR_LONG_CTAS overrides)
+    int64_t long_ctas = -1;                                     // see wide_long_scans (PCR_LONG_CTAS: a line in CTAs an SM instead)
     int64_t seq_ctas = -1;                                      // see sequential_in_ctas (PCR_SEQ_CTAS: a line in items an SM instead)
     int64_t index_ctas = -1;                                    // see launch_index_kernel (PCR_INDEX_CTAS: a line in pairs an SM instead)
     int64_t pack_warps = -1;                                    // see first_pass_form (PCR_PACK_WARPS: a line in warps an SM instead)
@@ -817,7 +817,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     if (const char* e = getenv("PCR_PAIRS")) r->pairs = atoi(e) != 0;
     if (const char* e = getenv("PCR_SEQ_CTAS")) r->seq_ctas = std::max(0, atoi(e));
     if (const char* e = getenv("PCR_INDEX_CTAS")) r->index_ctas = std::max(0, atoi(e));
-    if (const char* e = getenv("PCR_LONG_CTAS")) r->long_ctas = (uint32_t)std::max(0, atoi(e));
+    if (const char* e = getenv("PCR_LONG_CTAS")) r->long_ctas = std::max(0, atoi(e));
     if (const char* e = getenv("PCR_PACK_WARPS")) r->pack_warps = std::max(0, atoi(e));
     if (const char* e = getenv("PCR_SHORT_WARPS")) r->short_warps = (uint32_t)std::max(0, atoi(e));
     // slices: enough images each to fill the machine, few enough to keep launches cheap
@@ -941,7 +941,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
                 r->item_begin[(size_t)g * G + s] = begin;
                 r->item_count[(size_t)g * G + s] = n_items - begin;
             }
-    r->first_bytes.assign(G, 0); r->longest.assign(G, 0); r->longest_chain.assign(G, 0); r->intervals.assign(G, 0);
+    r->first_bytes.assign(G, 0); r->longest.assign(G, 0); r->longest_chain.assign(G, 0); r->long_bytes.assign(G, 0); r->intervals.assign(G, 0);
     for (uint32_t s = 0; s < G; ++s) {
         const bool first = r->script[s].Ss > 0 && r->script[s].Ah == 0;
         for (uint32_t i = 0; i < N; ++i) {
@@ -950,6 +950,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
             r->longest_chain[s] = std::max(r->longest_chain[s], chains[(size_t)s * N + i]);
             r->intervals[s] += nsegs[(size_t)s * N + i];
             if (first && !(single && takes_long_kernel((int)s, i))) r->first_bytes[s] += bytes;
+            if (single && r->script[s].Ah == 0 && takes_long_kernel((int)s, i)) r->long_bytes[s] += bytes;
         }
     }
     // the pairs' items: sixteen intervals of one image
@@ -1388,18 +1389,29 @@ static bool sequential_in_ctas(const pcr_record* rec, int s) {
     return rec->intervals[s] >= 20 * items || (double)rec->chain_bytes[s] <= 7.4 * rec->n_sms * rec->longest_chain[s];
 }
 
-// Whether the long scans of a wave that are first passes (or sequential) get CTAs of four times as many warps: while
-// most of the machine is idle; beyond, the narrow ones do less in all.  Decode at k = 5 in us, narrow and wide, by CTAs
-// an SM: HAM-shaped images 2 242 and 184, 4.4 between 265 and 300
-// (contents that fall in quickly) or 356 and 300, 18 696 and 788; ImageNet-shaped 2.2 234 and 158, 8.6 233 and 233, 35 487
-// and 616; CelebA-shaped 2.2 163 and 116, 17 248 and 266.  Baseline: ImageNet-shaped 0.4 639 and 575, 1.7 706 and 747, HAM-shaped 0.4
-// 526 and 447, CelebA-shaped 0.4 471 and 483.
+// Whether the long scans of a wave that are first passes (or sequential) get CTAs of four times as many warps: while most of the
+// machine is idle, by the number of CTAs an SM or by what there is to read in units of the longest scan (an SM holds few wide CTAs, but those of
+// chroma scans are soon gone); beyond, the narrow ones do less in all.  Decode in us, narrow and wide, means over two or three contents.
+// k = 5, by longest scans an SM: ImageNet-shaped 0.3 232 and 155, 0.9 221 and 201, 1.4 253 and 236, 1.8 291 and 264, 2.5 330 and 381; CelebA-shaped
+// 1.0 163 and 112, 1.5 173 and 145, 2.3 196 and 182, 2.9 202 and 205; HAM-shaped 0.4 283 and 255, 1.6 366 and 345, 3 437 and 435; greyscale 1.2
+// 214 and 170, 2.4 212 and 238; mixed sizes 0.4 396 and 196.  k = 1, by CTAs an SM: ImageNet-shaped 0.4 178 and 105, 1.3 160 and 122, 2.6 171 and
+// 143, 4.3 181 and 176, 6.9 225 and 246; HAM-shaped 1.7 215 and 194, 3.0 255 and 263; 128x128 2.6 95 and 77.  Scans below a kilobyte gain only
+// side by side with few others: 128x128 k = 5 4.3 CTAs an SM 106 and 108, 6.5 110 and 120; 64x64 8.6 100 and 120.
+// Baseline, by CTAs an SM: ImageNet-shaped 0.4 654 and 615, 0.9 638 and 595, 1.1 676 and 758; HAM-shaped 0.4 465 and 448, 1.1 593 and 615; mixed
+// sizes 1.7 719 and 632; 1024x1024 0.4 2031 and 1126.  Scans that a narrow CTA's threads read in 32 words each gain nothing: CelebA-shaped
+// 0.4 436 and 448, 1.3 562 and 577, 32x32 142 and 148.
 static bool wide_long_scans(const pcr_record* rec, const std::vector<int>& wave, bool sequential, int k0, int k) {
-    uint64_t ctas = 0;
-    for (int s : wave)
-        if (s >= k0 && s < k && rec->script[s].Ah == 0)
-            for (int g = 0; g < rec->n_slices; ++g) ctas += rec->long_count[(size_t)g * rec->G + s];
-    return ctas * (sequential ? 4u : 1u) <= (uint64_t)rec->long_ctas * (uint64_t)rec->n_sms;
+    uint64_t ctas = 0, bytes = 0, longest = 0;
+    for (int s : wave) {
+        if (s < k0 || s >= k || rec->script[s].Ah != 0) continue;
+        for (int g = 0; g < rec->n_slices; ++g) ctas += rec->long_count[(size_t)g * rec->G + s];
+        bytes += rec->long_bytes[s];
+        longest = std::max<uint64_t>(longest, rec->longest[s]);
+    }
+    const uint64_t sms = (uint64_t)rec->n_sms;
+    if (rec->long_ctas >= 0) return ctas * (sequential ? 4u : 1u) <= (uint64_t)rec->long_ctas * sms;
+    if (sequential) return longest > 128u * kSeqLongWarps * 32u && (4u * ctas <= 3u * sms || (double)bytes <= 0.55 * sms * longest);
+    return ctas <= 3u * sms || (longest >= 1000u && (double)bytes <= 2.2 * sms * longest);
 }
 
 // Decode scans k0 .. k-1 on top of the state scans 0 .. k0-1 left behind (k0 = 0: from scratch),
