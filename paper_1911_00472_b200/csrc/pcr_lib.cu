@@ -559,8 +559,12 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     r->script.resize(G);
     // every image's chunks are walked independently (a few host threads for large records); the
     // running sums over images follow in one serial pass
-    std::vector<uint32_t> nsegs((size_t)G * N), lens((size_t)G * N), image_bytes(N);      // restart intervals and entropy-coded bytes by (scan, image)
-    std::vector<uint32_t> chains((size_t)G * N);                     // of AC refinements and sequential scans: bytes of an interval, on average
+    struct Counts {                                                  // of a (scan, image)
+        uint32_t nseg, bytes;                                        // restart intervals, entropy-coded bytes
+        uint32_t chain() const { return (uint32_t)((float)bytes / (float)nseg); }      // bytes of an interval, on average
+    };
+    std::vector<Counts> counts((size_t)G * N);
+    std::vector<uint32_t> image_bytes(N);                            // entropy-coded bytes
     std::vector<uint8_t> one_interval(N, 0);                         // some scan of the image is one restart interval
     uint8_t sampling0 = 0;
     auto parse_image = [&](uint32_t i) -> int {
@@ -604,8 +608,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
                 total_mcu = (uint64_t)((wc + 7) / 8) * ((hc + 7) / 8);
             }
             sd.nseg = sd.ri ? (uint32_t)((total_mcu + sd.ri - 1) / sd.ri) : 1u;
-            nsegs[(size_t)g * N + i] = sd.nseg; lens[(size_t)g * N + i] = sd.data_end - sd.data_off;
-            if (sp.sc.Ss > 0 ? sp.sc.Ah != 0 : sp.sc.Se == 63) chains[(size_t)g * N + i] = (sd.data_end - sd.data_off) / std::max(1u, sd.nseg);
+            counts[(size_t)g * N + i] = Counts{sd.nseg, sd.data_end - sd.data_off};
             if (sd.nseg == 1) one_interval[i] = 1;
             sum += sd.data_end - sd.data_off;
         }
@@ -673,9 +676,9 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     uint32_t* const seg_base = T.h<uint32_t>(at_base);
     for (size_t j = 0; j < (size_t)G * N; ++j) {
         seg_base[j] = (uint32_t)segs;
-        segs += (uint64_t)nsegs[j] + 1;               // one closing entry per (scan, image)
+        segs += (uint64_t)counts[j].nseg + 1;               // one closing entry per (scan, image)
         if (segs >= (1ull << 32)) return PCR_E_FORMAT;
-        max_items += nsegs[j] / kSegsPerItem + 1 + nsegs[j] / (kSegsPerItem / 2) + 1;     // (the pairs' items too)
+        max_items += counts[j].nseg / kSegsPerItem + 1 + counts[j].nseg / (kSegsPerItem / 2) + 1;     // (the pairs' items too)
     }
     bool single = false;                              // any scan of any image is one restart interval
     for (uint32_t i = 0; i < N; ++i) {
@@ -912,15 +915,16 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
         for (int w = 0; w < r->n_waves; ++w)
             for (int s : r->wave_scans[w]) {
                 const uint32_t begin = n_items;
-                const uint32_t* const ns = &nsegs[(size_t)s * N];
+                const Counts* const of = &counts[(size_t)s * N];
                 const bool ac = r->script[s].Ss > 0;
-                const bool dc_refine = r->script[s].Ss == 0 && r->script[s].Ah != 0;
+                const bool dc_refine = r->script[s].Ss == 0 && r->script[s].Ah != 0, chains = ac ? r->script[s].Ah != 0 : r->script[s].Se == 63;
                 Item* open = nullptr;                         // an unfilled last item that the next image may extend
                 uint32_t last = 0;                            // the longest chain of the last item
+                uint64_t load = 0;
                 for (uint32_t pos = r->slice_img[g]; pos < r->slice_img[g + 1] && !dc_refine; ++pos) {
                     const uint32_t i = order[pos];
                     if (single && takes_long_kernel((int)s, i)) continue;
-                    const uint32_t nseg = ns[i], si = (uint32_t)(s * N + i);
+                    const uint32_t nseg = of[i].nseg, si = (uint32_t)(s * N + i), chain = chains ? of[i].chain() : 0u;
                     // full warps of 32 restart intervals; in AC scans the last warp of an image
                     // runs on into the first intervals of the next image (two tables per warp)
                     uint32_t j = 0;
@@ -928,29 +932,34 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
                         j = std::min<uint32_t>(kSegsPerItem - open->count, nseg);
                         open->count += j; open->next = si + 1u;
                         open = nullptr;
-                        r->chain_bytes[s] += std::max(chains[si], last) - last;
+                        load += std::max(chain, last) - last;
                     }
                     for (; j < nseg; j += kSegsPerItem) {
                         const uint32_t cnt = std::min<uint32_t>(kSegsPerItem, nseg - j);
                         items[n_items] = Item{si, j, cnt, 0u, 0u};
                         open = ac && cnt < (uint32_t)kSegsPerItem ? &items[n_items] : nullptr;
                         ++n_items;
-                        r->chain_bytes[s] += last = chains[si];
+                        load += last = chain;
                     }
                 }
+                r->chain_bytes[s] += load;
                 r->item_begin[(size_t)g * G + s] = begin;
                 r->item_count[(size_t)g * G + s] = n_items - begin;
             }
     r->first_bytes.assign(G, 0); r->longest.assign(G, 0); r->longest_chain.assign(G, 0); r->long_bytes.assign(G, 0); r->intervals.assign(G, 0);
     for (uint32_t s = 0; s < G; ++s) {
-        const bool first = r->script[s].Ss > 0 && r->script[s].Ah == 0;
-        for (uint32_t i = 0; i < N; ++i) {
-            const uint32_t bytes = lens[(size_t)s * N + i];
-            r->longest[s] = std::max(r->longest[s], bytes);
-            r->longest_chain[s] = std::max(r->longest_chain[s], chains[(size_t)s * N + i]);
-            r->intervals[s] += nsegs[(size_t)s * N + i];
-            if (first && !(single && takes_long_kernel((int)s, i))) r->first_bytes[s] += bytes;
-            if (single && r->script[s].Ah == 0 && takes_long_kernel((int)s, i)) r->long_bytes[s] += bytes;
+        const Counts* const of = &counts[(size_t)s * N];
+        const bool first = r->script[s].Ah == 0, ac = r->script[s].Ss > 0;
+        uint32_t most = 0;
+        uint64_t sum = 0, long_sum = 0;
+        for (uint32_t i = 0; i < N; ++i) { most = std::max(most, of[i].bytes); sum += of[i].bytes; }
+        for (uint32_t i = 0; single && first && i < N; ++i) long_sum += takes_long_kernel((int)s, i) ? of[i].bytes : 0u;
+        r->longest[s] = most;
+        if (first) r->long_bytes[s] = long_sum;
+        if (first && ac) r->first_bytes[s] = sum - long_sum;
+        for (uint32_t i = 0; first && !ac && r->script[s].Se == 63 && i < N; ++i) {      // (sequential)
+            r->longest_chain[s] = std::max(r->longest_chain[s], of[i].chain());
+            r->intervals[s] += of[i].nseg;
         }
     }
     // the pairs' items: sixteen intervals of one image
@@ -958,15 +967,17 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     for (int g = 0; g < r->n_slices; ++g)
         for (uint32_t s = 0; s < G; ++s) {
             const uint32_t begin = n_items;
+            uint64_t load = 0;
             for (uint32_t pos = r->slice_img[g]; r->pair_of[s] >= 0 && pos < r->slice_img[g + 1]; ++pos) {
                 const uint32_t i = order[pos], a = (uint32_t)r->pair_of[s];
                 if (single && takes_long_kernel((int)s, i)) continue;
-                const uint32_t nseg = nsegs[(size_t)s * N + i], longer = std::max(chains[(size_t)s * N + i], chains[(size_t)a * N + i]);
+                const uint32_t nseg = counts[(size_t)s * N + i].nseg, longer = std::max(counts[(size_t)s * N + i].chain(), counts[(size_t)a * N + i].chain());
                 for (uint32_t j = 0; j < nseg; j += kSegsPerItem / 2) {
                     items[n_items++] = Item{a * N + i, j, std::min<uint32_t>(kSegsPerItem / 2, nseg - j), 0u, (s - a) * N};
-                    r->pair_chain_bytes[s] += longer;
+                    load += longer;
                 }
             }
+            r->pair_chain_bytes[s] += load;
             r->pair_begin[(size_t)g * G + s] = begin;
             r->pair_count[(size_t)g * G + s] = n_items - begin;
         }
