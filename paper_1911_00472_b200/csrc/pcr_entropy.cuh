@@ -211,7 +211,7 @@ __device__ __forceinline__ SliceMarks slice_marks(const uint4& v, uint32_t prev,
 // kSplit: a CTA takes a pair, its warps runs of the pair's tiles: they count what their run keeps and finds first, and meet; a word
 // that two runs share is written byte by byte.  For launches of few pairs, whose time is that of the longest scan: all scans
 // of 64 ImageNet-shaped images 38 -> 19 us, 1024 baseline JPEGs 124 -> 54 us.  The bytes are read twice, so launches that fill the
-// machine keep a warp a pair: 1024 ImageNet-shaped images at k = 10 72 us, split 95.
+// machine, and short scans, keep a warp a pair (see launch_index_kernel): 1024 ImageNet-shaped images at k = 10 72 us, split 95.
 constexpr int kIndexWarps = 8;
 template <bool kSplit>
 __global__ void __launch_bounds__(32 * kIndexWarps) unstuff_index_kernel(Params P, ScanList sl, int img0, int nimg, uint32_t index_blocks) {

@@ -226,7 +226,8 @@ struct pcr_record {
     int64_t index_ctas = -1;                                    // see launch_index_kernel (PCR_INDEX_CTAS: a line in pairs an SM instead)
     int64_t pack_warps = -1;                                    // see first_pass_form (PCR_PACK_WARPS: a line in warps an SM instead)
     uint32_t short_warps = 20;                                  // see first_pass_form (PCR_SHORT_WARPS overrides)
-    // Items of the AC refinements (and of a sequential scan): the sum of their chains' bytes, an item counting with its longest.  By scan; by the pair's later scan
+    // Items of the AC refinements (and of a sequential scan): the sum of their chains' bytes, an item counting with its longest.
+    // By scan; by the pair's later scan
     std::vector<uint64_t> chain_bytes, pair_chain_bytes;
     std::vector<uint32_t> pair_begin, pair_count;               // [n_slices][G] items of the pair, by its later scan
     uint32_t n_units = 0;

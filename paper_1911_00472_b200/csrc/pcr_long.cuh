@@ -380,10 +380,10 @@ __device__ __forceinline__ void dc_hypotheses(const DcSteps& S, LongSpan& L, uin
 // Bound by the chain of one subsequence times the rounds until the slowest scan of the record has fallen in: a launch
 // waits for that scan; then by the pass that writes.  The stream and the tables are in shared memory because every step of the
 // search depends on them.  256 HAM-shaped images at k = 5, decode: 570 us on average over six records when every round read its whole
-// subsequence from global memory, 350 us with marks, 325 us now: four times the warps where most of the machine is idle, interleaved DC
-// scans read from every place of the MCU at once (dc_hypotheses; the search took up to 23 rounds, most of the kernel's time),
-// writing passes of straight-line steps, no rounds that only hand a state on behind the interval's end (up to 56).  64
-// ImageNet-shaped images 234 -> 158 us, 64 CelebA-shaped 171 -> 116 us.
+// subsequence from global memory, 350 us with marks.  Writing passes of straight-line steps and no rounds that only hand a state on
+// behind the interval's end (up to 56): 399 and 366 us over three other records.  Four times the warps while most of the machine is
+// idle (wide_long_scans), interleaved DC scans then read from every place of the MCU at once (dc_hypotheses; the search took up to 23
+// rounds, most of the kernel's time): 345 us of those 366; 64 ImageNet-shaped images 267 -> 156 us, 64 CelebA-shaped 153 -> 100 us.
 // ---------------------------------------------------------------------------------------
 constexpr int kLongWarps = 2, kLongWideWarps = 8;
 // words of a scan that are staged: 8 KB, a 600x450 image's scans have up to 6 (of the luminance 12); 24 KB of a wide CTA

@@ -11,7 +11,8 @@
 //
 // Bound by warp 0's step: a window, a table entry, and where both lead next, 125 cycles a symbol (a lane that did everything
 // itself took 600), then by the warps of four CTAs an SM sharing its schedulers.  1024 ImageNet-shaped images 742 -> 437 us, 64
-// such images 713 -> 177 us; launches of many images with few intervals keep a lane an interval (at the end of the file).  (A step with a predicate for every case 180 cycles; both possible tables looked up and one entry
+// such images 713 -> 177 us; launches of many images with few intervals keep a lane an interval (at the end of the file).
+// (A step with a predicate for every case 180 cycles; both possible tables looked up and one entry
 // chosen afterwards: 189 us; 6 or 12 warps a CTA: 183, 181 us and 467, 460; rounds of 48 symbols 184, of 96 equal.)
 #pragma once
 #include <cuda_runtime.h>
@@ -262,7 +263,8 @@ __global__ void __launch_bounds__(32 * kSeqWarps, 4) sequential_kernel(Params P,
 // The same, one lane per restart interval, for launches of many items (see sequential_in_ctas): a warp an item instead of eight, 18
 // items an SM instead of four.  Lanes stand at different kinds of symbol in every step, so a block's first symbol goes through the same
 // instructions as the others (its value is the difference), stores are predicated, and what changes from block to block comes
-// from a small table in shared memory.  Bound by the length of a lane's chain, 600 cycles a symbol.
+// from a small table in shared memory.  Bound by the length of a lane's chain, 600 cycles a symbol: 3072 CelebA-shaped images 1049 us,
+// with the kernel above 1224; 1024 513 and 450.
 // ---------------------------------------------------------------------------------------
 constexpr int kSeqLaneWarps = 2;
 constexpr uint32_t kSeqLaneRing = 4 * sizeof(ScanTab), kSeqLanePlaces = kSeqLaneRing + (kRingWords + 2) * 128, kSeqLanePreds = kSeqLanePlaces + 8 * 16;
