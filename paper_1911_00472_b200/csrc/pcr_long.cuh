@@ -677,15 +677,20 @@ __global__ void __launch_bounds__(32 * kWarps) sequential_long_kernel(Params P, 
 // the chain, through two shared-memory tables that the chain's helper warp prepares:
 //   q[bit]       what the symbol that begins at this bit of the stream is (skip, run, flags): every bit position is
 //                decoded in advance, 32 at a time, so the thread neither assembles a window nor looks up a code;
-//   zpos[i][b]   position of the i-th still-zero coefficient of block b, minus i: the run's target, and by
-//                differences the number of correction bits passed.
-// A symbol is two dependent loads and a handful of additions (about 15 instructions; 35 with a bit reader and
-// symbol records).  Per block the thread leaves the bit position where it began; the helper warp decodes the
-// 32 blocks of a finished batch once more, one lane per block, to make the side data.
-// HAM-shaped record, 1024 images: the launch 3.4 -> 1.7 ms, which is the longest luminance chain's (24.2 k symbols in 4275
-// blocks; all luminance chains start at once, the last chroma chain ends at 1.1 ms).  That chain takes 1.40 ms with at
-// most one chain a scheduler (89 cycles a symbol, 139 a block with its share of the meetings), 1.71 among sixteen an SM
-// (102 and 204).
+//   zpos[b][i]   non-zero positions in front of the i-th still-zero coefficient of block b: by differences the number of
+//                correction bits passed; and whether the block ends there.
+// A symbol is two dependent loads and a handful of additions, and what a block that ends takes beyond that does not ask how many still-zero
+// positions there are: the list says where the block ends, and its entries beyond that are all closing ones.  Per block the thread leaves
+// the bit position where the next one begins; the helper warp decodes the 32 blocks of a finished batch once more, one lane per
+// block, to make the side data.
+// A lone thread takes about four cycles an instruction whatever it waits for, so the count of instructions decides.  The launch in us with 16
+// instructions a symbol and a block change that carried the next block's bounds along (370 cycles a block and 45 a symbol, clock64 in a copy), and now:
+// HAM-shaped, 1024 images 1728 -> 1565, 512 1468 -> 1285, 128 1412 -> 1230; mixed sizes, 200 3281 -> 2846; ImageNet-shaped, 1024 2843 -> 2483, 256
+// 2768 -> 2409; CelebA-shaped, 256 at k = 8 268 -> 237.  Not kept: block change by selects in the symbol's line (1785, 1349, 1279, 2890); a loop of one
+// load a symbol behind a block's last non-zero position (1599, 1335, 1273, 2786, ImageNet-shaped 2431); the entries behind the symbol's own bits requested
+// before the number of correction bits is known (2331, 1754, 1652, 3628); the loop unrolled (1869).
+// Codes longer than the quick table's index are looked up where the thread meets one; with the helper looking them up at every bit position,
+// filling q was 28 % of its time.
 //
 // A later refinement of the same component needs the masks the earlier one leaves, block by
 // block.  Both walk the same block grid in the same order, so the later chain runs behind the
@@ -714,8 +719,9 @@ __device__ __forceinline__ bool wait_at_least(const volatile uint32_t* flag, uin
 
 // Entry of q: twice the bits to skip (code, sign bit, run-length bits) in bits 0..5, 6 = a new coefficient, 7 = more than
 // a plain step (an end-of-band run that covers further blocks, or no symbol: the rest but bit 15 is zero),
-// 9..15 = run of zeros (from 64 on: the rest of the band; 64 + the exponent of an end-of-band run).
-constexpr uint32_t kQNew = 0x40u, kQSpecial = 0x80u, kQRest = 64u << 9, kQBad = kQSpecial | kQRest;
+// 9..15 = run of zeros (from 64 on: the rest of the band; 64 + the exponent of an end-of-band run).  kQLong: a code longer than the quick
+// table's index (an exponent that no run has); the decoding thread looks it up where it meets one, and leaves the entry there.
+constexpr uint32_t kQNew = 0x40u, kQSpecial = 0x80u, kQRest = 64u << 9, kQBad = kQSpecial | kQRest, kQLong = kQBad | (15u << 9);
 __device__ __forceinline__ uint32_t chain_entry(uint32_t len, uint32_t rs) {
     const uint32_t r = rs >> 4, newc = rs & 1u;
     if (rs & 14u) return kQBad;                                        // a refinement symbol has size 0 or 1
@@ -723,19 +729,21 @@ __device__ __forceinline__ uint32_t chain_entry(uint32_t len, uint32_t rs) {
     return (2u * (len + r)) | (r ? kQSpecial : 0u) | kQRest | (r << 9);
 }
 
+constexpr uint32_t kChainList = 68;          // bytes of a block's list (64 entries; blocks side by side fall on different banks)
+
 struct ChainMail {                     // what the two warps of a chain tell each other at a meeting point
     uint32_t nd, rd, err_c;            // decoder: blocks it decoded, the word it stands at, error
     uint32_t wr, err_h;                // helper: the ring is filled up to this word, error
 };
 struct ChainShared {
     uint16_t q[kChainBits];            // by bit position modulo kChainBits
-    uint8_t zpos[2][64][32];           // [batch][i][block]: twice (position of the block's i-th still-zero coefficient of the band, minus i);
-                                       // entry nz: Se + 1 - nz (as if position Se + 1 followed)
-    uint16_t ends[2][32];              // per block: how many still-zero positions there are (nz, at most 63) and, from bit 8
-                                       // on, the rank that ends the block (nz, or nz - 1 if the last of them is Se)
-    uint32_t start[2][32];             // per block: where it began (bit position; bit 31: inside an end-of-band run)
+    uint8_t zpos[2][32][kChainList];   // [batch][block][i]: twice the number of the band's non-zero positions in front of the block's i-th still-zero
+                                       // one; from the number of still-zero positions on, twice all of them.  Bit 7: the block ends there
+                                       // (those entries, and the one of a still-zero position Se)
+    uint32_t start[2][33];             // per block, and behind the last: where it began (bit position; bit 31: inside an end-of-band run)
     uint32_t ring[kChainRing];
-    uint16_t quick[1 << kChainLutBits];         // q entries of the codes of at most kChainLutBits bits, 0: longer
+    const uint8_t* dht;                         // the table's body: 16 length counts, then the values
+    uint16_t quick[1 << kChainLutBits];         // q entries of the codes of at most kChainLutBits bits, kQLong: longer
     uint16_t first[8], cnt[8], idx[8];          // the longer codes: first code, how many, index of the first value
     ChainMail mail[2];                 // by parity of the meeting point
     uint32_t job_gi, job_level;        // the pair's job (job_gi = 0xFFFFFFFF: none left)
@@ -748,6 +756,17 @@ static_assert(kChainPairs * sizeof(ChainShared) <= 227 * 1024, "one CTA per SM h
 __device__ __forceinline__ uint32_t ring_bits(const uint32_t* ring, uint32_t p, uint32_t n) {
     const uint32_t a = ring[(p >> 5) & (kChainRing - 1)], b = ring[((p >> 5) + 1u) & (kChainRing - 1)];
     return __funnelshift_l(b, a, p & 31u) >> (32u - n);
+}
+
+// The entry of the code longer than kChainLutBits bits that begins at bit p of the ring.
+__device__ __forceinline__ uint32_t chain_long(const ChainShared& sh, uint32_t p) {
+    const uint32_t x = ring_bits(sh.ring, p, 32u);
+#pragma unroll 1
+    for (uint32_t j = 0; j < 16u - kChainLutBits; ++j) {
+        const uint32_t l = kChainLutBits + 1u + j, d = (x >> (32u - l)) - sh.first[j];
+        if (d < sh.cnt[j]) return chain_entry(l, sh.dht[16u + ((sh.idx[j] + d) & 255u)]);
+    }
+    return kQBad;
 }
 
 // Polls *flag (another warp's progress word in global memory) until it reaches `need`; `seen` keeps
@@ -790,8 +809,8 @@ __device__ __forceinline__ void chain_decoder(const RefineList& fl, ChainShared&
                                               uint32_t* sync, uint32_t levels, uint32_t rounds, uint32_t q, uint32_t slot) {
     const uint32_t per_round = 4u * gridDim.x, statics = per_round * rounds;
     uint32_t a_q = (uint32_t)__cvta_generic_to_shared(sh.q), a_zpos = (uint32_t)__cvta_generic_to_shared(sh.zpos);
-    uint32_t a_ends = (uint32_t)__cvta_generic_to_shared(sh.ends), a_start = (uint32_t)__cvta_generic_to_shared(sh.start);
-    asm volatile("" : "+r"(a_q), "+r"(a_zpos), "+r"(a_ends), "+r"(a_start));   // (kept in registers)
+    uint32_t a_start = (uint32_t)__cvta_generic_to_shared(sh.start);
+    asm volatile("" : "+r"(a_q), "+r"(a_zpos), "+r"(a_start));   // (kept in registers)
     uint32_t mk = 0;                                           // meeting points so far
     bool first_job = true;
     for (;;) {
@@ -815,60 +834,68 @@ __device__ __forceinline__ void chain_decoder(const RefineList& fl, ChainShared&
         if (!meet_decoder(sh, ++mk)) return;                   // tables, first lists and ring are ready
         if (sh.mail[mk & 1u].err_h) continue;                  // a scan whose bounds are off: the helper reports it
         uint32_t wr = sh.mail[mk & 1u].wr;
-        const uint32_t Ss2 = 2u * sh.Ss, total = sh.total, limit = sh.limit;
+        const uint32_t total = sh.total, limit = sh.limit;
         uint32_t pos2 = 2u * sh.lead;                          // twice the bit position (the tables' entries are two bytes)
         uint32_t eobrun = 0, m = 0, p = 0;
         for (;;) {
             const uint32_t nblk = min(32u, total - m);
             // A block is only begun while kChainBlockWords words lie ahead (q ends one word before the ring) and, the
             // batch's first one, while the interval has not ended (reading on behind it is found below; zeros follow).
-            // Inside the loop the test is made a symbol early, with room for it: see below.
-            const uint32_t lead2 = 64u * (wr - min(wr, kChainBlockWords + 3u)), early2 = lead2 - min(lead2, 192u);
-            const uint32_t ends = a_ends + 64u * p, start = a_start + 128u * p;
-            uint32_t zb = a_zpos + 2048u * p;                  // of the block: its column of the lists
-            uint32_t nd = 0;
+            const uint32_t lead2 = 64u * (wr - min(wr, kChainBlockWords + 3u));
+            const uint32_t start = a_start + 132u * p;
+            // (addresses) the next entry of the block's list, and its last one
+            uint32_t r = a_zpos + 32u * kChainList * p, last = r + 63u;
+            uint32_t nd = 0, passed2 = 0;                      // blocks done; twice the non-zero positions passed in this one
             int err = 0;
-            uint32_t now = lds16(ends);
-            uint32_t nz = now & 255u, tend = now >> 8, next = lds16(ends + 2u);   // of the block, and of the next one
+            sts32(start, pos2 >> 1);
             bool go = pos2 < lead2 && (pos2 >> 1) <= limit;
             while (go) {
                 if (eobrun == 0) {
-                    uint32_t e, before;
-                    for (;;) {
-                        sts32(start + 4u * nd, pos2 >> 1);
-                        // ep2: twice the list entry of the last still-zero position reached (the difference of two
-                        // entries is the number of non-zero positions between them: one correction bit each); zi:
-                        // how many are passed
-                        uint32_t zi = 0, ep2 = Ss2, t;
+                    uint32_t e, raw = lds16(a_q + (pos2 & (2u * kChainBits - 1u))), corr2;     // (raw: the next symbol's entry)
+                    do {
+                        uint32_t entry;
 #pragma unroll 1
                         do {
-                            before = pos2;
-                            e = lds16(a_q + (pos2 & (2u * kChainBits - 1u)));
+                            e = raw;
                             // the target: the (r+1)-th still-zero position from here; a run past the last one (an end
-                            // of band is one too) ends at the list's closing entry (position Se + 1)
-                            t = min(zi + (e >> 9), nz);
-                            const uint32_t e2 = lds8(zb + 32u * t);
-                            pos2 += (e & 63u) - ep2 + e2;      // code, sign and correction bits in one step
-                            zi = t + 1u;
-                            ep2 = e2;
-                        } while (t < tend);                    // (known before e2 is: the branch costs the chain nothing,
-                        ++nd; ++zb;                            // nor does what a new block takes)
-                        nz = next & 255u; tend = next >> 8;
-                        next = lds16(ends + 2u * ((nd + 1u) & 31u));
-                        if (nd == nblk || (e & kQSpecial) || before >= early2) break;
-                    }
-                    if (e & kQSpecial) {                       // the band also ends for the next eobrun blocks
+                            // of band is one too) ends at a closing entry
+                            const uint32_t t = min(r + (e >> 9), last);
+                            entry = lds8(t);
+                            corr2 = (entry & 127u) - passed2;  // one correction bit for each non-zero position passed
+                            pos2 += (e & 63u) + corr2;         // code, sign and correction bits in one step
+                            raw = lds16(a_q + (pos2 & (2u * kChainBits - 1u)));
+                            r = t + 1u;
+                            passed2 = entry;
+                        } while (entry < 128u);
+                        r = last + (kChainList - 63u);
+                        last += kChainList;
+                        passed2 = 0;
+                        ++nd;
+                        sts32(start + 4u * nd, pos2 >> 1);
+                    } while (!(e & kQSpecial) && nd != nblk && pos2 < lead2);
+                    if (e & kQSpecial) {
+                        if (e == kQLong) {                     // its entry looked up, and the block once more from its beginning
+                            pos2 -= corr2;
+                            sts16(a_q + (pos2 & (2u * kChainBits - 1u)), chain_long(sh, pos2 >> 1));
+                            --nd; last -= kChainList;
+                            r = last - 63u; pos2 = 2u * lds32(start + 4u * nd);
+                            continue;
+                        }
                         if (e == kQBad) { err = kErrCorrupt; --nd; break; }
+                        // the band also ends for the next eobrun blocks
                         const uint32_t x = (e >> 9) & 15u;
-                        eobrun = (1u << x) + ring_bits(sh.ring, ((before + (e & 63u)) >> 1) - x, x) - 1u;
+                        eobrun = (1u << x) + ring_bits(sh.ring, ((pos2 - corr2) >> 1) - x, x) - 1u;
                     }
                 } else {
-                    sts32(start + 4u * nd, (pos2 >> 1) | 0x80000000u);
-                    pos2 += lds8(zb + 32u * nz) - Ss2;         // inside an end-of-band run: corrections for the whole band
-                    --eobrun;
-                    ++nd; ++zb;
-                    nz = next & 255u; tend = next >> 8;
-                    next = lds16(ends + 2u * ((nd + 1u) & 31u));
+#pragma unroll 1
+                    do {
+                        sts32(start + 4u * nd, (pos2 >> 1) | 0x80000000u);
+                        pos2 += lds8(last) & 127u;             // inside an end-of-band run: corrections for the whole band
+                        --eobrun;
+                        ++nd; last += kChainList;
+                    } while (eobrun && nd < nblk && pos2 < lead2);
+                    r = last - 63u;
+                    sts32(start + 4u * nd, pos2 >> 1);
                 }
                 go = nd < nblk && pos2 < lead2;
             }
@@ -936,7 +963,7 @@ __device__ __forceinline__ void chain_helper(const Params& P, const RefineList& 
             for (int e = 0; e < (1 << kChainLutBits) / 32; ++e) {      // consecutive entries: the code length only grows
                 const uint32_t x = (uint32_t)lane * ((1u << kChainLutBits) / 32u) + (uint32_t)e;
                 while (l <= kChainLutBits && x >= s_code[34 + l]) ++l;
-                uint32_t v = 0;
+                uint32_t v = kQLong;
                 if (l <= kChainLutBits) v = chain_entry((uint32_t)l, dht[16u + ((s_code[17 + l] + (x >> (kChainLutBits - l)) - s_code[l]) & 255u)]);
                 sh.quick[x] = (uint16_t)v;
             }
@@ -951,6 +978,7 @@ __device__ __forceinline__ void chain_helper(const Params& P, const RefineList& 
         if (lane == 0) {
             sh.Ss = Ss; sh.Se = Se; sh.total = total; sh.lead = lead;
             sh.limit = lead + 8u * (bend - bstart);            // first bit behind the interval
+            sh.dht = dht;
         }
         // masks of the positions that are already non-zero: the union of up to four earlier scans; a
         // source that this launch decodes itself (an earlier level of the group) is waited for
@@ -1008,9 +1036,11 @@ __device__ __forceinline__ void chain_helper(const Params& P, const RefineList& 
                 // the positions of the band that are still zero, in order: the target of a run r is then one
                 // table look-up for the decoder (the (r+1)-th of those not yet passed)
                 const uint64_t z = ~v & band;
-                uint32_t dst = (uint32_t)__cvta_generic_to_shared(&sh.zpos[b][0][lane]);
-                const uint32_t dst0 = dst;
-                uint32_t v2 = 0;                                   // twice (position minus number of still-zero ones before it)
+                const uint32_t n = (uint32_t)__popcll(z), row = (uint32_t)__cvta_generic_to_shared(&sh.zpos[b][lane][0]);
+                const uint32_t closing = (2u * (Se + 1u - Ss - n) | 128u) * 0x01010101u;
+#pragma unroll
+                for (uint32_t w = 0; w < kChainList; w += 4u) sts32(row + w, closing);
+                uint32_t dst = row, v2 = 0u - 2u * Ss;             // v2: twice the non-zero positions so far
                 // (straight through all positions, lanes with different masks stay together; a position outside the band
                 // counts as non-zero)
 #pragma unroll
@@ -1018,13 +1048,11 @@ __device__ __forceinline__ void chain_helper(const Params& P, const RefineList& 
                     const uint32_t zw = pos < 32 ? (uint32_t)z : (uint32_t)(z >> 32);
                     if ((zw >> (pos & 31)) & 1u) {
                         asm volatile("st.shared.u8 [%0], %1;" : : "r"(dst), "r"(v2) : "memory");
-                        dst += 32u;
+                        ++dst;
                     } else v2 += 2u;
                 }
-                const uint32_t n = (dst - dst0) >> 5;
-                asm volatile("st.shared.u8 [%0], %1;" : : "r"(dst), "r"(2u * (Se + 1u - n)) : "memory");      // closing entry: behind the band
-                const uint32_t tend = (z >> Se) & 1u ? n - 1u : n; // the block also ends at a still-zero position Se
-                sh.ends[b][lane] = (uint16_t)(n | (tend << 8));
+                if ((z >> Se) & 1u)                                // the block also ends at a still-zero position Se
+                    asm volatile("st.shared.u8 [%0], %1;" : : "r"(dst - 1u), "r"(closing) : "memory");
             }
         };
         // The ring and q filled as far as they go while word `oldest` is still needed.  The symbol at a word's bits
@@ -1037,27 +1065,11 @@ __device__ __forceinline__ void chain_helper(const Params& P, const RefineList& 
                 __syncwarp(full);
 #pragma unroll 1
                 for (uint32_t w = wr - 1u; w != wr + 31u; w += 8u) {   // (word -1 at first: never looked at)
-                    uint32_t x[9], e[8], none = 0;
+                    uint32_t x[9], e[8];
 #pragma unroll
                     for (uint32_t i = 0; i < 9; ++i) x[i] = ring[(w + i) & (kChainRing - 1)];
 #pragma unroll
-                    for (uint32_t i = 0; i < 8; ++i) {
-                        x[i] = __funnelshift_l(x[i + 1], x[i], (uint32_t)lane);
-                        e[i] = sh.quick[x[i] >> (32 - kChainLutBits)];
-                        none |= e[i] == 0 ? 1u << i : 0u;
-                    }
-                    if (none) {                                    // codes longer than the table's index, or none
-#pragma unroll
-                        for (uint32_t i = 0; i < 8; ++i) {
-                            if (!((none >> i) & 1u)) continue;
-                            e[i] = kQBad;
-#pragma unroll 1
-                            for (uint32_t j = 0; j < 16u - kChainLutBits; ++j) {
-                                const uint32_t l = kChainLutBits + 1u + j, d = (x[i] >> (32u - l)) - sh.first[j];
-                                if (d < sh.cnt[j]) { e[i] = chain_entry(l, dht[16u + ((sh.idx[j] + d) & 255u)]); break; }
-                            }
-                        }
-                    }
+                    for (uint32_t i = 0; i < 8; ++i) e[i] = sh.quick[__funnelshift_l(x[i + 1], x[i], (uint32_t)lane) >> (32 - kChainLutBits)];
 #pragma unroll
                     for (uint32_t i = 0; i < 8; ++i) sh.q[(32u * (w + i) + lane) & (kChainBits - 1u)] = (uint16_t)e[i];
                 }
@@ -1070,17 +1082,17 @@ __device__ __forceinline__ void chain_helper(const Params& P, const RefineList& 
         auto side_data = [&](uint32_t m0, uint32_t nd, uint32_t b, uint64_t h) {
             bool over = false;
             if ((uint32_t)lane < nd) {
-                const uint32_t st = sh.start[b][lane], nz = sh.ends[b][lane] & 255u;
-                const uint8_t* zp = &sh.zpos[b][0][lane];
-                uint32_t at = st & 0x7FFFFFFFu, zi = 0, ep = 2u * Ss, k = 0;
+                const uint32_t st = sh.start[b][lane], nz = Se + 1u - Ss - (uint32_t)__popcll(h);
+                const uint8_t* zp = &sh.zpos[b][lane][0];
+                uint32_t at = st & 0x7FFFFFFFu, zi = 0, ep = 0, k = 0;
                 uint32_t s0 = 0, s1 = 0, N0 = 0, N1 = 0, G0 = 0, G1 = 0;
                 // a block inside an end-of-band run is one step over the rest of the band that takes no symbol
                 uint32_t e = st >> 31 ? kQRest : (uint32_t)sh.q[at & (kChainBits - 1u)];
 #pragma unroll 1
                 for (int i = 0; i < 80 && k < Se; ++i) {       // (bounded: more symbols than a block can have)
                     const uint32_t skip = (e & 63u) >> 1, sign_at = at + skip - 1u;
-                    const uint32_t t = min(zi + (e >> 9), nz), e2 = zp[32u * t], n = (e2 - ep) >> 1;
-                    k = (e2 >> 1) + t;
+                    const uint32_t t = min(zi + (e >> 9), nz), e2 = zp[t] & 127u, n = (e2 - ep) >> 1;
+                    k = (e2 >> 1) + t + Ss;
                     const uint32_t isnew = e & kQNew ? 1u : 0u;
                     over = over || (isnew && k > Se);          // a new coefficient behind the band
                     const uint32_t plus = isnew & (ring[(sign_at >> 5) & (kChainRing - 1)] >> (~sign_at & 31u));

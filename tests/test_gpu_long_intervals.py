@@ -8,6 +8,7 @@ empty subsequences, blocks shared by neighbouring lanes and images of a single b
 import numpy as np
 import pytest
 
+import helpers
 import pcr_synth
 from oracle import pcr_oracle as O
 
@@ -56,6 +57,40 @@ def test_ham_shaped_small(rec3_small, min_bytes, monkeypatch):
 @pytest.mark.parametrize("config", [0, 1, 2])
 def test_other_shapes_without_restart_markers(config, monkeypatch):
     rec = pcr_synth.make_record(config, n_images=6, restart_rows=False)
+    _compare_every_k(rec, 0, monkeypatch)
+
+
+def _geometric_runs(rng, nb, more):
+    """AC fields whose runs of zeros are geometrically distributed: refinement alphabets with codes of up to sixteen bits."""
+    c = np.zeros((nb, 64), dtype=np.int16)
+    pos, live = np.zeros(nb, dtype=int), np.ones(nb, dtype=bool)
+    for _ in range(12):
+        pos = pos + np.minimum(rng.geometric(0.45, size=nb), 16)
+        live &= (pos < 64) & (rng.random(nb) < more)
+        at = np.nonzero(live)[0]
+        c[at, pos[at]] = rng.choice([-5, -2, -1, 1, 2, 5], p=[0.05, 0.05, 0.4, 0.4, 0.05, 0.05], size=at.size)
+    c[:, 0] = rng.integers(-100, 100, size=nb)
+    return c
+
+
+@pytest.mark.parametrize("more, last", [(0.9, 0), (0.97, 1), (0.5, 0)])
+def test_refinement_codes_longer_than_the_table(more, last, monkeypatch):
+    """Codes of more than nine bits are looked up by the chain's decoding thread, which then takes the block once more from its
+    beginning; with `last`, blocks that end at a still-zero position 63 and blocks without any still-zero position lie between."""
+    rng = np.random.default_rng(900 + int(100 * more))
+    dims = [(400, 300), (17, 9), (256, 8)]
+    coeffs = [_geometric_runs(rng, pcr_synth.num_blocks(w, h), more) for w, h in dims]
+    if last:
+        for c in coeffs:
+            c[rng.random(len(c)) < 0.2, 63] = 1
+            c[rng.random(len(c)) < 0.1, 1:] = 4
+    rec = pcr_synth.record_from_coeffs(dims, coeffs, restart_rows=False)
+    jpeg = bytes(O.reassemble(rec.bytes, 0, 10))
+    longest = 0
+    for marker, at, size, _ in helpers.jpeg_segments(jpeg):
+        if marker == 0xC4 and jpeg[at] >> 4 == 1:              # (the last AC tables belong to refinements)
+            longest = max(b + 1 for b in range(16) if jpeg[at + 1 + b])
+    assert longest > 9
     _compare_every_k(rec, 0, monkeypatch)
 
 
