@@ -684,11 +684,16 @@ __global__ void __launch_bounds__(32 * kWarps) sequential_long_kernel(Params P, 
 // the bit position where the next one begins; the helper warp decodes the 32 blocks of a finished batch once more, one lane per
 // block, to make the side data.
 // A lone thread takes about four cycles an instruction whatever it waits for, so the count of instructions decides.  The launch in us with 16
-// instructions a symbol and a block change that carried the next block's bounds along (370 cycles a block and 45 a symbol, clock64 in a copy), and now:
-// HAM-shaped, 1024 images 1728 -> 1565, 512 1468 -> 1285, 128 1412 -> 1230; mixed sizes, 200 3281 -> 2846; ImageNet-shaped, 1024 2843 -> 2483, 256
-// 2768 -> 2409; CelebA-shaped, 256 at k = 8 268 -> 237.  Not kept: block change by selects in the symbol's line (1785, 1349, 1279, 2890); a loop of one
-// load a symbol behind a block's last non-zero position (1599, 1335, 1273, 2786, ImageNet-shaped 2431); the entries behind the symbol's own bits requested
-// before the number of correction bits is known (2331, 1754, 1652, 3628); the loop unrolled (1869).
+// instructions a symbol and a block change that carried the next block's bounds along (370 cycles a block and 45 a symbol, clock64 in a copy); with
+// lists that say where a block ends; and now, with runs counted from the entry reached, the flag of the ending entry taken out once a block
+// instead of in every symbol, and the chain's place in shared memory in a uniform register:
+//   HAM-shaped, 1024 / 512 / 128 images   1728 -> 1565 -> 1420, 1468 -> 1285 -> 1182, 1412 -> 1230 -> 1127
+//   mixed sizes, 200                      3281 -> 2846 -> 2637
+//   ImageNet-shaped, 1024 / 256           2843 -> 2483 -> 2285, 2768 -> 2409 -> 2229
+//   CelebA-shaped, 256 at k = 8           268 -> 237 -> 219
+// Not kept (HAM-shaped 1024, 512, 128, mixed sizes; of the second form): block change by selects in the symbol's line (1785, 1349, 1279, 2890); a
+// loop of one load a symbol behind a block's last non-zero position (1599, 1335, 1273, 2786); the entries behind the symbol's own bits
+// requested before the number of correction bits is known (2331, 1754, 1652, 3628); the loop unrolled (1869).
 // Codes longer than the quick table's index are looked up where the thread meets one; with the helper looking them up at every bit position,
 // filling q was 28 % of its time.
 //
@@ -719,13 +724,13 @@ __device__ __forceinline__ bool wait_at_least(const volatile uint32_t* flag, uin
 
 // Entry of q: twice the bits to skip (code, sign bit, run-length bits) in bits 0..5, 6 = a new coefficient, 7 = more than
 // a plain step (an end-of-band run that covers further blocks, or no symbol: the rest but bit 15 is zero),
-// 9..15 = run of zeros (from 64 on: the rest of the band; 64 + the exponent of an end-of-band run).  kQLong: a code longer than the quick
+// 9..15 = run of zeros plus one (from 64 on: the rest of the band; 64 + the exponent of an end-of-band run).  kQLong: a code longer than the quick
 // table's index (an exponent that no run has); the decoding thread looks it up where it meets one, and leaves the entry there.
 constexpr uint32_t kQNew = 0x40u, kQSpecial = 0x80u, kQRest = 64u << 9, kQBad = kQSpecial | kQRest, kQLong = kQBad | (15u << 9);
 __device__ __forceinline__ uint32_t chain_entry(uint32_t len, uint32_t rs) {
     const uint32_t r = rs >> 4, newc = rs & 1u;
     if (rs & 14u) return kQBad;                                        // a refinement symbol has size 0 or 1
-    if (newc || r == 15u) return (2u * (len + newc)) | (newc ? kQNew : 0u) | (r << 9);
+    if (newc || r == 15u) return (2u * (len + newc)) | (newc ? kQNew : 0u) | ((r + 1u) << 9);
     return (2u * (len + r)) | (r ? kQSpecial : 0u) | kQRest | (r << 9);
 }
 
@@ -805,12 +810,11 @@ __device__ __forceinline__ bool meet_helper(ChainShared& sh, uint32_t k, int lan
 
 // The decoding side of a chain: one thread.  It takes the pair's jobs (first the statically assigned
 // one, then tickets of its scheduler's queue), and per job follows the bit stream batch by batch.
-__device__ __forceinline__ void chain_decoder(const RefineList& fl, ChainShared& sh, const uint32_t* __restrict__ list, uint32_t n_groups,
+// `base`: the shared address of sh, the same in the whole warp.
+__device__ __forceinline__ void chain_decoder(const RefineList& fl, ChainShared& sh, uint32_t base, const uint32_t* __restrict__ list, uint32_t n_groups,
                                               uint32_t* sync, uint32_t levels, uint32_t rounds, uint32_t q, uint32_t slot) {
     const uint32_t per_round = 4u * gridDim.x, statics = per_round * rounds;
-    uint32_t a_q = (uint32_t)__cvta_generic_to_shared(sh.q), a_zpos = (uint32_t)__cvta_generic_to_shared(sh.zpos);
-    uint32_t a_start = (uint32_t)__cvta_generic_to_shared(sh.start);
-    asm volatile("" : "+r"(a_q), "+r"(a_zpos), "+r"(a_start));   // (kept in registers)
+    const uint32_t a_q = base, a_zpos = base + (uint32_t)offsetof(ChainShared, zpos), a_start = base + (uint32_t)offsetof(ChainShared, start);
     uint32_t mk = 0;                                           // meeting points so far
     bool first_job = true;
     for (;;) {
@@ -843,8 +847,8 @@ __device__ __forceinline__ void chain_decoder(const RefineList& fl, ChainShared&
             // batch's first one, while the interval has not ended (reading on behind it is found below; zeros follow).
             const uint32_t lead2 = 64u * (wr - min(wr, kChainBlockWords + 3u));
             const uint32_t start = a_start + 132u * p;
-            // (addresses) the next entry of the block's list, and its last one
-            uint32_t r = a_zpos + 32u * kChainList * p, last = r + 63u;
+            // (addresses) the block's last entry, and the one its last symbol reached
+            uint32_t last = a_zpos + 32u * kChainList * p + 63u, r = last - 64u;
             uint32_t nd = 0, passed2 = 0;                      // blocks done; twice the non-zero positions passed in this one
             int err = 0;
             sts32(start, pos2 >> 1);
@@ -859,15 +863,18 @@ __device__ __forceinline__ void chain_decoder(const RefineList& fl, ChainShared&
                             e = raw;
                             // the target: the (r+1)-th still-zero position from here; a run past the last one (an end
                             // of band is one too) ends at a closing entry
-                            const uint32_t t = min(r + (e >> 9), last);
+                            const uint32_t t = __viaddmin_u32(r, e >> 9, last);
                             entry = lds8(t);
-                            corr2 = (entry & 127u) - passed2;  // one correction bit for each non-zero position passed
+                            corr2 = entry - passed2;           // one correction bit for each non-zero position passed
                             pos2 += (e & 63u) + corr2;         // code, sign and correction bits in one step
                             raw = lds16(a_q + (pos2 & (2u * kChainBits - 1u)));
-                            r = t + 1u;
+                            r = t;
                             passed2 = entry;
                         } while (entry < 128u);
-                        r = last + (kChainList - 63u);
+                        // (the flag of the ending entry, counted along until here)
+                        pos2 -= 128u; corr2 -= 128u;
+                        raw = lds16(a_q + (pos2 & (2u * kChainBits - 1u)));
+                        r = last + (kChainList - 64u);
                         last += kChainList;
                         passed2 = 0;
                         ++nd;
@@ -878,7 +885,7 @@ __device__ __forceinline__ void chain_decoder(const RefineList& fl, ChainShared&
                             pos2 -= corr2;
                             sts16(a_q + (pos2 & (2u * kChainBits - 1u)), chain_long(sh, pos2 >> 1));
                             --nd; last -= kChainList;
-                            r = last - 63u; pos2 = 2u * lds32(start + 4u * nd);
+                            r = last - 64u; pos2 = 2u * lds32(start + 4u * nd);
                             continue;
                         }
                         if (e == kQBad) { err = kErrCorrupt; --nd; break; }
@@ -894,7 +901,7 @@ __device__ __forceinline__ void chain_decoder(const RefineList& fl, ChainShared&
                         --eobrun;
                         ++nd; last += kChainList;
                     } while (eobrun && nd < nblk && pos2 < lead2);
-                    r = last - 63u;
+                    r = last - 64u;
                     sts32(start + 4u * nd, pos2 >> 1);
                 }
                 go = nd < nblk && pos2 < lead2;
@@ -1084,17 +1091,16 @@ __device__ __forceinline__ void chain_helper(const Params& P, const RefineList& 
             if ((uint32_t)lane < nd) {
                 const uint32_t st = sh.start[b][lane], nz = Se + 1u - Ss - (uint32_t)__popcll(h);
                 const uint8_t* zp = &sh.zpos[b][lane][0];
-                uint32_t at = st & 0x7FFFFFFFu, zi = 0, ep = 0, k = 0;
-                uint32_t s0 = 0, s1 = 0, N0 = 0, N1 = 0, G0 = 0, G1 = 0;
+                uint32_t at = st & 0x7FFFFFFFu, zi = 0xFFFFFFFFu, ep = 0, k = 0;     // zi: the entry reached
+                uint32_t s0 = 0, s1 = 0, N0 = 0, N1 = 0, G0 = 0, G1 = 0, isnew = 0;
                 // a block inside an end-of-band run is one step over the rest of the band that takes no symbol
                 uint32_t e = st >> 31 ? kQRest : (uint32_t)sh.q[at & (kChainBits - 1u)];
 #pragma unroll 1
                 for (int i = 0; i < 80 && k < Se; ++i) {       // (bounded: more symbols than a block can have)
                     const uint32_t skip = (e & 63u) >> 1, sign_at = at + skip - 1u;
-                    const uint32_t t = min(zi + (e >> 9), nz), e2 = zp[t] & 127u, n = (e2 - ep) >> 1;
+                    const uint32_t t = __viaddmin_u32(zi, e >> 9, nz), e2 = zp[t] & 127u, n = (e2 - ep) >> 1;
                     k = (e2 >> 1) + t + Ss;
-                    const uint32_t isnew = e & kQNew ? 1u : 0u;
-                    over = over || (isnew && k > Se);          // a new coefficient behind the band
+                    isnew = e & kQNew ? 1u : 0u;
                     const uint32_t plus = isnew & (ring[(sign_at >> 5) & (kChainRing - 1)] >> (~sign_at & 31u));
                     N0 |= shl0(isnew, k); N1 |= shl0(isnew, k - 32u);
                     G0 |= shl0(plus, k); G1 |= shl0(plus, k - 32u);
@@ -1110,9 +1116,10 @@ __device__ __forceinline__ void chain_helper(const Params& P, const RefineList& 
                         }
                         at += n;
                     }
-                    ep = e2; zi = t + 1u;
+                    ep = e2; zi = t;
                     e = sh.q[at & (kChainBits - 1u)];
                 }
+                over = isnew && k > Se;                        // a new coefficient behind the band
                 uint4* o = reinterpret_cast<uint4*>(outp + (uint64_t)block_index(m0 + lane) * 4);
                 o[0] = make_uint4((uint32_t)h | N0, (uint32_t)(h >> 32) | N1, s0, s1);
                 o[1] = make_uint4(N0, N1, G0, G1);
@@ -1195,7 +1202,9 @@ __global__ void __launch_bounds__(64 * kChainPairs, 1) ac_refine_group_kernel(Pa
     if ((int)threadIdx.x < pairs) { s_sh[threadIdx.x].phase_c = 0; s_sh[threadIdx.x].phase_h = 0; }
     __syncthreads();
     if (wid < pairs) {
-        if (lane == 0) chain_decoder(fl, s_sh[wid], list, n_groups, sync, (uint32_t)levels, (uint32_t)rounds, (uint32_t)wid & 3u, (uint32_t)wid >> 2);
+        // (a reduction leaves its result in a uniform register, which loads and stores add for nothing: 5 % of the launch)
+        const uint32_t base = __reduce_max_sync(0xffffffffu, (uint32_t)__cvta_generic_to_shared(&s_sh[wid]));
+        if (lane == 0) chain_decoder(fl, s_sh[wid], base, list, n_groups, sync, (uint32_t)levels, (uint32_t)rounds, (uint32_t)wid & 3u, (uint32_t)wid >> 2);
     } else {
         chain_helper(P, fl, s_sh[wid - pairs], list, sync + 4, lane);
     }
