@@ -11,7 +11,8 @@
 //
 // Bound by warp 0's step: a window, a table entry, and where both lead next, 125 cycles a symbol (a lane that did everything
 // itself took 600), then by the warps of four CTAs an SM sharing its schedulers.  1024 ImageNet-shaped images 742 -> 437 us, 64
-// such images 713 -> 177 us; launches of many images with few intervals keep a lane an interval (at the end of the file).
+// such images 713 -> 177 us.  The warps that write count for most of those schedulers' slots: with what a symbol needs only in damaged streams or at
+// block ends moved behind the block, decode of 1024 ImageNet-shaped images 688 -> 668 us, of 1024 CelebA-shaped 447 -> 414.  Launches of many images with few intervals keep a lane an interval (at the end of the file).
 // (A step with a predicate for every case 180 cycles; both possible tables looked up and one entry
 // chosen afterwards: 189 us; 6 or 12 warps a CTA: 183, 181 us and 467, 460; rounds of 48 symbols 184, of 96 equal.)
 #pragma once
@@ -228,7 +229,6 @@ __global__ void __launch_bounds__(32 * kSeqWarps, 4) sequential_kernel(Params P,
             if (x == 0) x = long_code(sh.next[place_i].w, w, kTabDcSeq);
             sts128(head, make_uint4(0, 0, 0, 0));
             uint32_t p = 1, M0 = 0, M1 = 0;                // position, mask of those from 8 on
-            bool some = false;                             // a coefficient among positions 1..7
             w = __funnelshift_l(W.behind(at), w, x & 31u);
             at += x & 31u;
             W.load(at);
@@ -239,19 +239,19 @@ __global__ void __launch_bounds__(32 * kSeqWarps, 4) sequential_kernel(Params P,
                 const uint32_t skip = x & 31u, sz = (x >> 5) & 15u, w1 = __funnelshift_l(W.behind(at), w, skip), x1 = tab_entry(t, w1);
                 at += skip;
                 W.load(at);
-                p += (x >> 9) & 31u;                           // (behind the coefficient)
+                p += x >> 9;                                   // (behind the coefficient; an end of block: beyond every position)
                 const int v = magnitude(w, skip, sz);
-                bad = bad || (sz && p > 64u);                  // a coefficient behind the block
-                const bool coef = sz && p <= 64u, far = coef && p > 8u, low = coef && p <= 8u;
-                sts16_if(low, head + 2u * p - 2u, (uint32_t)v);
-                some = some || low;
+                const bool far = sz && p > 8u;
+                sts16_if(sz && !far, head + 2u * p - 2u, (uint32_t)v);
+                // (a coefficient behind the block has bits of its own to be stored at, and no place in the masks)
                 if (far) *vp = (int16_t)v;
                 vp += far ? 1 : 0;
                 M0 |= shl0(far ? 1u : 0u, p - 1u); M1 |= shl0(far ? 1u : 0u, p - 33u);
-                if ((x & kEntEob) || p > 63u) break;
+                if (p > 63u) { bad = bad || (sz && p > 64u); break; }
                 w = w1; x = x1;
             }
-            if (some) *reinterpret_cast<uint4*>(headp + 8ull * blk) = lds128(head);
+            const uint4 low = lds128(head);                    // (a coefficient is never 0)
+            if (low.x | low.y | low.z | low.w) *reinterpret_cast<uint4*>(headp + 8ull * blk) = low;
             if (M0 | M1) *reinterpret_cast<uint4*>(auxp + 2ull * blk) = value_record(M0, M1, vb);
         }
         meet();
@@ -364,18 +364,18 @@ __global__ void __launch_bounds__(32 * kSeqLaneWarps) sequential_lane_kernel(Par
                 }
                 const uint32_t skip = e & 31u, sz = (e >> 5) & 15u;
                 br.pos += skip;
-                k += (e >> 9) & 31u;                                       // behind the coefficient
+                k += e >> 9;                                               // behind the coefficient (an end of block: beyond every position)
                 const uint32_t at = k - 1u;
                 int v = magnitude(win, skip, sz);
                 if (is_dc) { v += (int)lds32(pred); sts32(pred, (uint32_t)v); }
-                const bool coef = sz && k <= 64u, far = coef && k > 8u;
+                const bool far = sz && k > 8u;
                 if (is_dc) dcp[blk] = (int16_t)v;                          // (stored even if there was no such symbol: the image is corrupt then)
-                if (coef && !far && !is_dc) headp[8u * (uint64_t)blk + at] = (int16_t)v;
+                if (sz && !far && !is_dc) headp[8u * (uint64_t)blk + at] = (int16_t)v;
                 if (far) *vp = (int16_t)v;
                 vp += far ? 1 : 0;
                 M0 |= shl0(far ? 1u : 0u, at); M1 |= shl0(far ? 1u : 0u, at - 32u);
-                if (sz && k > 64u && !is_dc) { bad = true; stop = 0; }
-                if ((e & kEntEob) || k > 63u) {                            // block finished
+                if (k > 63u) {                                             // block finished
+                    if (sz && k > 64u) { bad = true; stop = 0; }           // (a coefficient behind the block: stored at bits of its own, not in the masks)
                     if (M0 | M1) *reinterpret_cast<uint4*>(auxp + 2ull * blk) = value_record(M0, M1, vb);
                     k = 0; M0 = 0; M1 = 0; vb = vp;
                     place += 16u;
