@@ -684,7 +684,8 @@ __global__ void __launch_bounds__(32 * kWarps) sequential_long_kernel(Params P, 
 // the bit position where the next one begins; the helper warp decodes the 32 blocks of a finished batch once more, one lane per
 // block, to make the side data.
 // A lone thread takes about four cycles an instruction whatever it waits for, so the count of instructions decides.  The launch in us with 16
-// instructions a symbol and a block change that carried the next block's bounds along (370 cycles a block and 45 a symbol, clock64 in a copy); with
+// instructions a symbol and a block change that carried the next block's bounds along (clock64 in a copy that took most symbols by one load: 45 cycles
+// a symbol and 370 a block); with
 // lists that say where a block ends; and now, with runs counted from the entry reached, the flag of the ending entry taken out once a block
 // instead of in every symbol, and the chain's place in shared memory in a uniform register:
 //   HAM-shaped, 1024 / 512 / 128 images   1728 -> 1565 -> 1420, 1468 -> 1285 -> 1182, 1412 -> 1230 -> 1127
