@@ -163,14 +163,20 @@ def layout_bytes(scans, infos, k: int, chains: bool = False):
     return out
 
 
+def source_code(text: str) -> str:
+    """C++ source without comments, runs of white space as one space: what a compiler makes kernels of, whatever is written about them."""
+    import re
+    return re.sub(r'"(?:\\.|[^"\\\n])*"|((?:\s|//[^\n]*|/\*.*?\*/)+)', lambda m: " " if m.group(1) else m.group(0), text, flags=re.S)
+
+
 def source_hash() -> str:
-    """Hash of the CUDA sources: ncu counters are only quoted for the kernels they were taken on."""
+    """Hash of the CUDA sources (their code, not their comments): ncu counters are only quoted for the kernels they were taken on."""
     import glob
     import hashlib
     h = hashlib.sha256()
     for f in sorted(glob.glob(os.path.join(ROOT, "paper_1911_00472_b200", "csrc", "*"))):
-        with open(f, "rb") as fh:
-            h.update(fh.read())
+        with open(f, encoding="utf-8") as fh:
+            h.update(source_code(fh.read()).encode())
     return h.hexdigest()[:16]
 
 

@@ -81,3 +81,14 @@ def test_layout_bytes_model():
     assert bench.layout_bytes(scans, infos, 2)["pixels"] == 3 * 340 + 18 * 24
     b = bench.layout_bytes([(3, 0, 0, 63, 0, 0, 400)], infos, 1)        # baseline
     assert b["entropy0"] == 400 + 2 * 24 and b["pixels"] == 3 * 340 + (18 + 16) * 24
+
+
+def test_counters_outlive_comments_and_nothing_else():
+    """The committed ncu counters are quoted while the kernels' code is what they were taken on: comments and line breaks may
+    change, code and string literals may not."""
+    sys.path.insert(0, ROOT)
+    import bench
+    a = bench.source_code('int f(int x) {  // twice\n    return 2 * x;\n}\nasm("add.u32 //x;");\n')
+    assert a == bench.source_code('/* doubles\n   x */int f(int x) {\n  return 2 * x;  /* not 3 */\n}\n// an addition\nasm("add.u32 //x;");\n').lstrip()
+    for other in ("int f(int x) {\n return 3 * x;\n}\nasm(\"add.u32 //x;\");\n", "int f(int x) {\n return 2 * x;\n}\nasm(\"add.u32 //y;\");\n"):
+        assert bench.source_code(other) != a
