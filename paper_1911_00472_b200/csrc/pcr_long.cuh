@@ -753,7 +753,7 @@ struct ChainShared {
     uint16_t first[8], cnt[8], idx[8];          // the longer codes: first code, how many, index of the first value
     ChainMail mail[2];                 // by parity of the meeting point
     uint32_t job_gi, job_level;        // the pair's job (job_gi = 0xFFFFFFFF: none left)
-    uint32_t Ss, Se, total, lead, limit;        // of the job, for the decoder (bits counted from the interval's first word)
+    uint32_t total, lead, limit;                // of the job, for the decoder (bits counted from the interval's first word)
     volatile uint32_t phase_c, phase_h;         // meeting points each side has reached
 };
 static_assert(kChainPairs * sizeof(ChainShared) <= 227 * 1024, "one CTA per SM holds all its chains");
@@ -984,7 +984,7 @@ __device__ __forceinline__ void chain_helper(const Params& P, const RefineList& 
         const uint32_t* words = reinterpret_cast<const uint32_t*>(P.ubuf) + rd0;
         const uint32_t wlim = ((bend + 3u) >> 2) + 2u - rd0;   // words beyond are not read (zeros instead)
         if (lane == 0) {
-            sh.Ss = Ss; sh.Se = Se; sh.total = total; sh.lead = lead;
+            sh.total = total; sh.lead = lead;
             sh.limit = lead + 8u * (bend - bstart);            // first bit behind the interval
             sh.dht = dht;
         }
