@@ -695,8 +695,12 @@ __global__ void __launch_bounds__(32 * kWarps) sequential_long_kernel(Params P, 
 // Not kept (HAM-shaped 1024, 512, 128, mixed sizes; of the second form): block change by selects in the symbol's line (1785, 1349, 1279, 2890); a
 // loop of one load a symbol behind a block's last non-zero position (1599, 1335, 1273, 2786); the entries behind the symbol's own bits
 // requested before the number of correction bits is known (2331, 1754, 1652, 3628); the loop unrolled (1869).
-// Codes longer than the quick table's index are looked up where the thread meets one; with the helper looking them up at every bit position,
-// filling q was 28 % of its time.
+// Codes longer than the quick table's index are looked up where the thread meets one, since few records have many of them; with the
+// helper looking them up at every bit position, filling q was 28 % of its time.  128 HAM-shaped images whose refinement tables have
+// longer codes than they need (us: looked up by the helper; by the thread, the block again for every one; and now): all 10 bits 9829,
+// 11333, 8344; all longer by the same number, the shortest 10 bits 14354, 13878, 10181; those of three bits and more by seven 6616,
+// 8105, 7314; those of five and more by six 3271, 3170, 3434.  (All of a block's long codes looked up from the first one on: 7224,
+// 8890, 5986, 3465, but 1 to 2 % on the mixed sizes and ImageNet-shaped records above.)
 //
 // A later refinement of the same component needs the masks the earlier one leaves, block by
 // block.  Both walk the same block grid in the same order, so the later chain runs behind the
@@ -754,6 +758,7 @@ struct ChainShared {
     ChainMail mail[2];                 // by parity of the meeting point
     uint32_t job_gi, job_level;        // the pair's job (job_gi = 0xFFFFFFFF: none left)
     uint32_t total, lead, limit;                // of the job, for the decoder (bits counted from the interval's first word)
+    uint32_t once;                              // where the block began whose long code was looked up last (a bit position)
     volatile uint32_t phase_c, phase_h;         // meeting points each side has reached
 };
 static_assert(kChainPairs * sizeof(ChainShared) <= 227 * 1024, "one CTA per SM holds all its chains");
@@ -764,15 +769,42 @@ __device__ __forceinline__ uint32_t ring_bits(const uint32_t* ring, uint32_t p, 
     return __funnelshift_l(b, a, p & 31u) >> (32u - n);
 }
 
-// The entry of the code longer than kChainLutBits bits that begins at bit p of the ring.
-__device__ __forceinline__ uint32_t chain_long(const ChainShared& sh, uint32_t p) {
-    const uint32_t x = ring_bits(sh.ring, p, 32u);
-#pragma unroll 1
+// The entry of the code longer than kChainLutBits bits at pos2 (twice its bit position), left in q too.
+template <int kUnroll>
+__device__ __forceinline__ uint32_t chain_long(uint32_t base, uint32_t pos2) {
+    constexpr uint32_t kRing = offsetof(ChainShared, ring), kFirst = offsetof(ChainShared, first), kCnt = offsetof(ChainShared, cnt), kIdx = offsetof(ChainShared, idx);
+    const uint32_t p = pos2 >> 1, w = base + kRing;
+    const uint32_t x = __funnelshift_l(lds32(w + 4u * (((p >> 5) + 1u) & (kChainRing - 1u))), lds32(w + 4u * ((p >> 5) & (kChainRing - 1u))), p & 31u);
+    uint32_t e = kQBad;
+#pragma unroll kUnroll
     for (uint32_t j = 0; j < 16u - kChainLutBits; ++j) {
-        const uint32_t l = kChainLutBits + 1u + j, d = (x >> (32u - l)) - sh.first[j];
-        if (d < sh.cnt[j]) return chain_entry(l, sh.dht[16u + ((sh.idx[j] + d) & 255u)]);
+        const uint32_t l = kChainLutBits + 1u + j, d = (x >> (32u - l)) - lds16(base + kFirst + 2u * j);
+        if (d < lds16(base + kCnt + 2u * j)) {
+            const uint2 a = lds64(base + (uint32_t)offsetof(ChainShared, dht));
+            e = chain_entry(l, reinterpret_cast<const uint8_t*>(((uint64_t)a.y << 32) | a.x)[16u + ((lds16(base + kIdx + 2u * j) + d) & 255u)]);
+            break;
+        }
     }
-    return kQBad;
+    sts16(base + (pos2 & (2u * kChainBits - 1u)), e);
+    return e;
+}
+
+// A block with several long codes, from its beginning (pos2: twice the bit position; last: its list's last entry): every one is looked up where it
+// stands.  -> where the decoder goes on, in front of the block's last symbol: r (or what leads to the same target), passed2 and pos2 there.
+// (Not inlined, and back into the decoder's own loop: with this loop, or another end of a block, beside it that one takes 2 to 5 % longer.)
+__device__ __noinline__ uint3 chain_long_codes(uint32_t base, uint32_t pos2, uint32_t last) {
+    uint32_t r = last - 64u, entry = 0, passed2, e, d2;
+#pragma unroll 1
+    do {
+        e = lds16(base + (pos2 & (2u * kChainBits - 1u)));
+        if (e == kQLong) e = chain_long<16 - kChainLutBits>(base, pos2);
+        r = __viaddmin_u32(r, e >> 9, last);
+        passed2 = entry;
+        entry = lds8(r);
+        d2 = (e & 63u) + entry - passed2;
+        pos2 += d2;
+    } while (entry < 128u);
+    return make_uint3(r - (e >> 9), passed2, pos2 - d2);
 }
 
 // Polls *flag (another warp's progress word in global memory) until it reaches `need`; `seen` keeps
@@ -840,6 +872,7 @@ __device__ __forceinline__ void chain_decoder(const RefineList& fl, ChainShared&
         if (sh.mail[mk & 1u].err_h) continue;                  // a scan whose bounds are off: the helper reports it
         uint32_t wr = sh.mail[mk & 1u].wr;
         const uint32_t total = sh.total, limit = sh.limit;
+        sh.once = 0xFFFFFFFFu;
         uint32_t pos2 = 2u * sh.lead;                          // twice the bit position (the tables' entries are two bytes)
         uint32_t eobrun = 0, m = 0, p = 0;
         for (;;) {
@@ -882,11 +915,19 @@ __device__ __forceinline__ void chain_decoder(const RefineList& fl, ChainShared&
                         sts32(start + 4u * nd, pos2 >> 1);
                     } while (!(e & kQSpecial) && nd != nblk && pos2 < lead2);
                     if (e & kQSpecial) {
-                        if (e == kQLong) {                     // its entry looked up, and the block once more from its beginning
-                            pos2 -= corr2;
-                            sts16(a_q + (pos2 & (2u * kChainBits - 1u)), chain_long(sh, pos2 >> 1));
+                        if (e == kQLong) {
+                            // A long code: its entry looked up, and the block once more from its beginning; where that happens a second
+                            // time, all of its long codes are, so that a block's symbols are walked three times at most.
                             --nd; last -= kChainList;
-                            r = last - 64u; pos2 = 2u * lds32(start + 4u * nd);
+                            const uint32_t from = lds32(start + 4u * nd);
+                            if (sh.once != from) {
+                                sh.once = from;
+                                chain_long<1>(base, pos2 - corr2);
+                                r = last - 64u; pos2 = 2u * from;
+                                continue;
+                            }
+                            const uint3 at = chain_long_codes(base, 2u * from, last);
+                            r = at.x; passed2 = at.y; pos2 = at.z;
                             continue;
                         }
                         if (e == kQBad) { err = kErrCorrupt; --nd; break; }

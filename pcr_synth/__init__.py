@@ -70,6 +70,7 @@ def _load():
             lib.synth_num_blocks.argtypes = [C.c_uint32, C.c_uint32]
             lib.synth_zigzag.argtypes = [C.c_void_p]
             lib.synth_set_script.argtypes = [C.c_void_p, C.c_int]
+            lib.synth_set_ac_code_length.argtypes = [C.c_int]
             lib.synth_set_sampling.argtypes = [C.c_int, C.c_int, C.c_int]
             lib.synth_rgb_to_coeffs.argtypes = [C.c_void_p, C.c_int, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p]
             _lib = lib
@@ -380,4 +381,21 @@ class scan_script:
 
     def __exit__(self, *exc):
         _load().synth_set_script(None, 0)
+        return False
+
+
+class ac_code_length:
+    """Context manager: records made inside have no AC code of fewer than `bits` bits (at most 16; a legal table that does not
+    fit its scan, as of an encoder with fixed tables).  Not thread safe (a process-wide setting)."""
+
+    def __init__(self, bits: int):
+        self.bits = bits
+
+    def __enter__(self):
+        if _load().synth_set_ac_code_length(self.bits) != 0:
+            raise ValueError("unsupported code length")
+        return self
+
+    def __exit__(self, *exc):
+        _load().synth_set_ac_code_length(0)
         return False

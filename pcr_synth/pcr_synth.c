@@ -487,7 +487,15 @@ static void enc_ac_refine(scan_enc* e, const int16_t* blk, int Ss, int Se, int A
 /* ------------------------------------------------------------------------- */
 typedef struct { uint8_t bits[17]; uint8_t vals[256]; int nvals; uint16_t code[256]; uint8_t len[256]; } hufftab;
 
-static void huff_build(const long freq_in[256], hufftab* h) {
+/* The shortest code an AC table may have (0: no bound); see synth_set_ac_code_length. */
+static int g_ac_code_length = 0;
+int synth_set_ac_code_length(int n) {
+    if (n < 0 || n > 16) return -1;
+    g_ac_code_length = n;
+    return 0;
+}
+
+static void huff_build(const long freq_in[256], hufftab* h, int shortest) {
     long freq[257]; int size[257], next[257];
     for (int i = 0; i < 256; ++i) freq[i] = freq_in[i];
     freq[256] = 1;                       /* placeholder that ends up with the all-ones code */
@@ -513,6 +521,7 @@ static void huff_build(const long freq_in[256], hufftab* h) {
         }
     int L = 16; while (count[L] == 0) --L;
     --count[L];                          /* drop the placeholder */
+    for (int l = 1; l < shortest; ++l) { count[shortest] += count[l]; count[l] = 0; }
     memset(h, 0, sizeof *h);
     for (int i = 1; i <= 16; ++i) h->bits[i] = (uint8_t)count[i];
     int n = 0;
@@ -606,7 +615,7 @@ static void encode_scan(enc_state* st, const geom_t* g, const int16_t* coef, con
      * (slots 0, 1) and AC tables 0, 1 (slots 2, 3) */
     for (int s = 0; s < 4; ++s)
         if (used[s]) {
-            huff_build(freq[s], &tab[s]);
+            huff_build(freq[s], &tab[s], is_dc && !(sequential && s >= 2) ? 0 : g_ac_code_length);
             if (sequential) write_dht(out, s >= 2 ? 1 : 0, s & 1, &tab[s]);
             else write_dht(out, is_dc ? 0 : 1, s, &tab[s]);
         }

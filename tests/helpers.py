@@ -209,3 +209,60 @@ def record_from_groups(groups) -> np.ndarray:
     struct.pack_into("<QQQQ", head, 24, 64, index_off, ends[0], pos)
     body = bytes(head) + bytes(first[meta_off:meta_off + 16 * N]) + struct.pack(f"<{G + 1}Q", *ends) + b"".join(index)
     return np.frombuffer(body + b"\0" * (ends[0] - len(body)) + b"".join(parts), dtype=np.uint8).copy()
+
+
+def entropy_data(rec: np.ndarray, image: int, group: int):
+    """(first byte, end) of the entropy-coded bytes of an image's scan in a record of one scan a group, and the scan's AC code
+    tables: {table id: {symbol: (code, bits)}}."""
+    N, G = struct.unpack_from("<II", rec, 8)
+    at = struct.unpack_from("<Q", rec, 32)[0] + 8 * (G + 1) + 16 * (group * N + image)
+    off, length = struct.unpack_from("<QI", rec, at)
+    chunk = bytes(rec[off:off + length])
+    tables, p = {}, 2 if chunk[:2] == b"\xff\xd8" else 0
+    while chunk[p + 1] != 0xDA:
+        size = struct.unpack_from(">H", chunk, p + 2)[0]
+        q = p + 4
+        while chunk[p + 1] == 0xC4 and q < p + 2 + size:
+            counts, codes, code, v = chunk[q + 1:q + 17], {}, 0, q + 17
+            for bits in range(1, 17):
+                for _ in range(counts[bits - 1]):
+                    codes[chunk[v]] = (code, bits)
+                    code, v = code + 1, v + 1
+                code <<= 1
+            if chunk[q] >> 4 == 1:
+                tables[chunk[q] & 15] = codes
+            q = v
+        p += 2 + size
+    return off + p + 2 + struct.unpack_from(">H", chunk, p + 2)[0], off + length, tables
+
+
+def overwrite_bits(rec: np.ndarray, begin: int, end: int, at: int, bits: str):
+    """Bits of the entropy-coded bytes begin .. end - 1 (which hold no markers) replaced in place from bit `at` on; what no longer
+    fits behind the zero bytes that follow each 0xFF is cut off."""
+    text = "".join(f"{b:08b}" for b in bytes(rec[begin:end]).replace(b"\xff\0", b"\xff"))
+    text = text[:at] + bits + text[at + len(bits):]
+    data = bytes(int(text[i:i + 8], 2) for i in range(0, len(text) // 8 * 8, 8)).replace(b"\xff", b"\xff\0")[:end - begin]
+    if data[-1] == 0xFF:
+        data = data[:-1] + b"\0"
+    rec[begin:begin + len(data)] = np.frombuffer(data, dtype=np.uint8)
+    rec[begin + len(data):end] = 0
+
+
+def decode_damaged(rec: np.ndarray, intact: np.ndarray, image: int, k: int):
+    """Decodes a record in which one image is damaged at fidelity k: that image is reported as corrupt, and the others' pixels are
+    the oracle's for the intact record."""
+    import torch
+    from oracle import pcr_oracle as O
+    from paper_1911_00472_b200 import Decoder
+    dec = Decoder(rec)
+    try:
+        out = dec.decode(k)
+        torch.cuda.synchronize()
+        assert dec.status() == (image, -3)
+        pixels = out.cpu().numpy()
+        for i, inf in enumerate(dec.info):
+            if i != image:
+                want = O.decode_image(intact, i, k)[1]
+                assert np.array_equal(pixels[inf.out_offset:inf.out_offset + inf.out_bytes].reshape(want.shape), want), i
+    finally:
+        dec.close()

@@ -94,6 +94,37 @@ def test_refinement_codes_longer_than_the_table(more, last, monkeypatch):
     _compare_every_k(rec, 0, monkeypatch)
 
 
+@pytest.mark.parametrize("bits", [10, 12, 16])
+def test_tables_of_long_codes_only(bits, monkeypatch):
+    """Every AC code is longer than the chains' quick table (from 12 bits on, than all kernels' tables): blocks full of codes that
+    are looked up one by one, runs of blocks among them."""
+    rng = np.random.default_rng(bits)
+    dims = [(150, 110), (17, 9), (300, 8)]
+    with pcr_synth.ac_code_length(bits):
+        rec = pcr_synth.record_from_coeffs(dims, [_geometric_runs(rng, pcr_synth.num_blocks(w, h), 0.9) for w, h in dims], restart_rows=False)
+        ham = pcr_synth.make_record(3, n_images=1, restart_rows=False)
+    _compare_every_k(rec, 0, monkeypatch)
+    _compare_every_k(ham, 0, monkeypatch)
+
+
+@pytest.mark.parametrize("block", [0, 31, 32])
+def test_undefined_refinement_code(block, monkeypatch):
+    """Ones from the beginning of a block of a refinement on (no code is all ones): the chain's thread looks the code up as a long
+    one, finds none, and the image is reported; the others are untouched.  31 and 32: last block of a batch, first of the next."""
+    dims = [(64, 40), (72, 40), (40, 64)]
+    coeffs = [np.zeros((pcr_synth.num_blocks(w, h), 64), dtype=np.int16) for w, h in dims]
+    for c in coeffs:
+        c[:, 63] = 1                                           # in the last scan: three runs of sixteen zeros, fourteen zeros and the one
+    with pcr_synth.ac_code_length(10):
+        rec = pcr_synth.record_from_coeffs(dims, coeffs, restart_rows=False)
+    bad = np.array(rec.bytes, copy=True)
+    begin, end, tables = helpers.entropy_data(bad, 1, 9)
+    size = 3 * tables[0][0xF0][1] + tables[0][0xE1][1] + 1     # of a block, in bits
+    helpers.overwrite_bits(bad, begin, end, block * size, "1" * (8 * (end - begin)))
+    monkeypatch.setenv("PCR_LONG_MIN_BYTES", "0")
+    helpers.decode_damaged(bad, rec.bytes, 1, 10)
+
+
 @pytest.mark.parametrize("seed", range(6))
 def test_random_coefficient_fields_without_restart_markers(seed, monkeypatch):
     rng = np.random.default_rng(300 + seed)
