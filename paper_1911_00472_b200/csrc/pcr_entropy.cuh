@@ -447,8 +447,9 @@ __device__ __forceinline__ uint4 lds128(uint32_t a) { uint4 v; asm volatile("ld.
 __device__ __forceinline__ void sts32(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" : : "r"(a), "r"(v) : "memory"); }
 __device__ __forceinline__ void sts16(uint32_t a, uint32_t v) { asm volatile("st.shared.u16 [%0], %1;" : : "r"(a), "h"((uint16_t)v) : "memory"); }
 __device__ __forceinline__ void sts128(uint32_t a, const uint4& v) { asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" : : "r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory"); }
-// shifts that give 0 for counts of 32 and more
+// shifts that give 0 for counts of as many bits as the word has, and more
 __device__ __forceinline__ uint32_t shl0(uint32_t x, uint32_t n) { uint32_t y; asm("shl.b32 %0, %1, %2;" : "=r"(y) : "r"(x), "r"(n)); return y; }
+__device__ __forceinline__ uint64_t shl0(uint64_t x, uint32_t n) { uint64_t y; asm("shl.b64 %0, %1, %2;" : "=l"(y) : "l"(x), "r"(n)); return y; }
 __device__ __forceinline__ uint32_t shr0(uint32_t x, uint32_t n) { uint32_t y; asm("shr.u32 %0, %1, %2;" : "=r"(y) : "r"(x), "r"(n)); return y; }
 // byte permutation with the selector's sign form (__byte_perm masks it out)
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t s) { uint32_t y; asm("prmt.b32 %0, %1, %2, %3;" : "=r"(y) : "r"(a), "r"(b), "r"(s)); return y; }

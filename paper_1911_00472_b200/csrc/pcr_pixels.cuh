@@ -196,9 +196,9 @@ __device__ __forceinline__ bool expand_block(const Params& P, const CoefLists& c
             // the walk through each half ends with its last set bit (no branch around a correction: 347 -> 334 us with the rest of this walk
             // in 32 bits, 1024 ImageNet-shaped images at k = 10)
             const uint32_t h0 = a.x & ~b.x, h1 = a.y & ~b.y;
-            uint64_t cc = ((uint64_t)a.w << 32) | a.z;
+            // (none of them: a shift by 64, which gives 0; the side data of a damaged image may have bits all the same)
             const int n0 = __popc(h0);
-            if (cc) cc <<= 64 - n0 - __popc(h1);
+            const uint64_t cc = shl0(((uint64_t)a.w << 32) | a.z, 64u - (uint32_t)(n0 + __popc(h1)));
 #pragma unroll
             for (int half = 0; half < 2; ++half) {
                 uint32_t h = half ? h1 : h0, c = half ? (uint32_t)((cc << n0) >> 32) : (uint32_t)(cc >> 32) & (n0 ? ~0u << (32 - n0) : 0u);

@@ -30,6 +30,30 @@ def test_blocks_and_intervals(kind, fixed, ctas, pairs, monkeypatch):
     _compare(rec, (6, 9, 10))
 
 
+@pytest.mark.parametrize("restart_rows", [True, False])
+def test_corrections_by_halves(restart_rows, monkeypatch):
+    """Correction bits of the pixel stage: blocks whose earlier coefficients fill one half of the positions, both or none, with the last
+    set bit in either half, at its end, or nowhere, and new coefficients among them."""
+    rng = np.random.default_rng(11)
+    dims = [(200, 120), (8, 8), (90, 41)]
+    coeffs = []
+    for w, h in dims:
+        nb = pcr_synth.num_blocks(w, h)
+        c = np.zeros((nb, 64), dtype=np.int16)
+        first, second = rng.choice([0.0, 0.1, 1.0], size=nb), rng.choice([0.0, 0.1, 1.0], size=nb)
+        for lo, hi, share in ((1, 32, first), (32, 64, second)):
+            # (4: earlier than every refinement; two low bits: none set, one, or any)
+            low = rng.integers(0, 4, size=(nb, hi - lo)) * (rng.random((nb, hi - lo)) < rng.choice([0.0, 0.03, 1.0], size=nb)[:, None])
+            low[rng.random(nb) < 0.1, -1] = 3
+            old = rng.random((nb, hi - lo)) < share[:, None]
+            new = ~old & (rng.random((nb, hi - lo)) < rng.choice([0.0, 0.05], size=nb)[:, None])
+            c[:, lo:hi] = (old * (4 + low) + new * rng.integers(1, 4, size=(nb, hi - lo))) * rng.choice([-1, 1], size=(nb, hi - lo))
+        c[:, 0] = rng.integers(-500, 501, nb)
+        coeffs.append(c)
+    monkeypatch.setenv("PCR_LONG_MIN_BYTES", "0")
+    _compare(pcr_synth.record_from_coeffs(dims, coeffs, restart_rows=restart_rows), (6, 9, 10))
+
+
 @pytest.mark.parametrize("scan", [5, 9])
 @pytest.mark.parametrize("ctas", [0, 1 << 20])
 def test_damaged_interval(ctas, scan, monkeypatch):
