@@ -9,6 +9,7 @@ import struct
 import numpy as np
 import pytest
 
+import helpers
 import pcr_synth
 from oracle import pcr_oracle as O
 from test_gpu_kernel_edges import _compare, _field
@@ -79,3 +80,33 @@ def test_damaged_interval(ctas, monkeypatch):
             assert np.array_equal(pixels[inf.out_offset:inf.out_offset + inf.out_bytes].reshape(want.shape), want), i
     finally:
         dec.close()
+
+
+@pytest.mark.parametrize("form", ["ctas", "lanes", "no markers"])
+@pytest.mark.parametrize("block", [0, 3])
+def test_coefficient_behind_the_block(block, form, monkeypatch):
+    """A run of fifteen zeros instead of fourteen puts a block's last coefficient at position 64: the image is reported, the blocks
+    behind it keep their places, and the other images are untouched."""
+    dims = [(64, 24), (72, 24), (24, 64)]
+    with pcr_synth.sampling(1, 1, 1), pcr_synth.scan_script(pcr_synth.SCRIPT_BASELINE), pcr_synth.ac_code_length(10):
+        coeffs = [np.zeros((pcr_synth.num_blocks(w, h), 64), dtype=np.int16) for w, h in dims]
+        for c in coeffs:
+            c[:, 63] = 1                                       # three runs of sixteen zeros, fourteen zeros and the one
+            c[-1, 16] = 1                                      # (gives the longer run a code)
+        rec = pcr_synth.record_from_coeffs(dims, coeffs, restart_rows=form != "no markers")
+    bad = np.array(rec.bytes, copy=True)
+    begin, end, tables = helpers.entropy_data(bad, 1, 0)
+    codes = tables[0]
+    (zeros, n), (short, m), (long, l) = codes[0xF0], codes[0xE1], codes[0xF1]
+    assert m == l
+    text = "".join(f"{b:08b}" for b in bytes(bad[begin:end]).replace(b"\xff\0", b"\xff"))
+    block_text = 3 * f"{zeros:0{n}b}" + f"{short:0{m}b}"
+    at = -1
+    for _ in range(block + 1):
+        at = text.index(block_text, at + 1)
+    if form != "no markers":
+        end = begin + bytes(bad[begin:end]).index(b"\xff\xd0")
+    helpers.overwrite_bits(bad, begin, end, at + 3 * n, f"{long:0{l}b}")
+    monkeypatch.setenv("PCR_SEQ_CTAS", "0" if form == "lanes" else str(1 << 20))
+    monkeypatch.setenv("PCR_LONG_MIN_BYTES", "0")
+    helpers.decode_damaged(bad, rec.bytes, 1, 1)
