@@ -1389,16 +1389,15 @@ static int first_pass_form(const pcr_record* rec, const std::vector<int>& wave, 
 
 // Whether sequential_kernel's CTAs take the sequential scan's items or sequential_lane_kernel's warps.  A CTA's chains are five times as fast,
 // but an SM holds four CTAs and eighteen warps, and a CTA costs the same whether its lanes are in use or not: the warps are better where
-// images have few intervals and there are many images, by the items an SM in units of the longest chain.  Decode in us, CTAs and warps:
-// CelebA-shaped images (14 lanes in use) 3.8 350 and 467, 5.1 450 and 513, 7.0 596 and 612, 7.6 642 and 629, 10.1 833 and 741, 15 1224 and
-// 1049; 64x64 (4) 6.3 120 and 145, 9.5 172 and 169, 12.6 210 and 198; 96x96 (6) 9.6 226 and 227, 12.7 285 and 268; 32x32 (2) 5.6 88 and 102,
-// 10.5 135 and 133, 20.7 236 and 214; mixed sizes (12) 3.1 622 and 1114; HAM-shaped (29) 3.6 972 and 1080, 7.3 1931 and 2182; ImageNet-shaped (23)
-// 3.9 682 and 960, 8.0 1343 and 1417, 4:4:4 13.4 1853 and 1878.
+// images have few intervals and there are many images, by the items an SM in units of the longest chain.  Decode in us, CTAs and warps, two
+// contents each: CelebA-shaped images (14 lanes in use) 5.1 411 and 481, 7.0 556 and 576, 7.7 597 and 595, 8.9 680 and 642, 10.2 766 and 694, 15 1118
+// and 980; 64x64 (4) 7.9 169 and 173, 10.1 200 and 193; 96x96 (6) 4.9 157 and 203, 7.4 217 and 230; mixed sizes (13) 1.7 305 and 750, 2.2 439 and
+// 870; HAM-shaped (29) 5.4 958 and 1048; ImageNet-shaped (23) 8.9 1268 and 1406.
 static bool sequential_in_ctas(const pcr_record* rec, int s) {
     uint64_t items = 0;
     for (int g = 0; g < rec->n_slices; ++g) items += rec->item_count[(size_t)g * rec->G + s];
     if (rec->seq_ctas >= 0) return items <= (uint64_t)rec->seq_ctas * (uint64_t)rec->n_sms;
-    return rec->intervals[s] >= 20 * items || (double)rec->chain_bytes[s] <= 7.4 * rec->n_sms * rec->longest_chain[s];
+    return rec->intervals[s] >= 20 * items || (double)rec->chain_bytes[s] <= 8.0 * rec->n_sms * rec->longest_chain[s];
 }
 
 // Whether the long scans of a wave that are first passes (or sequential) get CTAs of four times as many warps: while most of the
