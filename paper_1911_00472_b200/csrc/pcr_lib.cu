@@ -218,17 +218,17 @@ struct pcr_record {
     // scan s follows, or -1.  Empty when the script has no such pair.
     std::vector<std::vector<int>> paired_waves;
     std::vector<int> pair_of;
-    bool pairs_fit = true;                                      // lane-per-interval warps of the waves with pairs fit the machine
     int pairs = -1;                                             // see pairs_pay (PCR_PAIRS overrides: 0 never, 1 always)
-    double refine_ctas = 4;                                     // see refine_load (PCR_REFINE_CTAS overrides)
+    double refine_ctas = 3.4;                                   // see refine_load (PCR_REFINE_CTAS overrides)
     int64_t long_ctas = -1;                                     // see wide_long_scans (PCR_LONG_CTAS: a line in CTAs an SM instead)
     int64_t seq_ctas = -1;                                      // see sequential_in_ctas (PCR_SEQ_CTAS: a line in items an SM instead)
     int64_t index_ctas = -1;                                    // see launch_index_kernel (PCR_INDEX_CTAS: a line in pairs an SM instead)
     int64_t pack_warps = -1;                                    // see first_pass_form (PCR_PACK_WARPS: a line in warps an SM instead)
     uint32_t short_warps = 20;                                  // see first_pass_form (PCR_SHORT_WARPS overrides)
     // Items of the AC refinements (and of a sequential scan): the sum of their chains' bytes, an item counting with its longest.
-    // By scan; by the pair's later scan
+    // By scan; by the pair's later scan.  And the sum of their squares
     std::vector<uint64_t> chain_bytes, pair_chain_bytes;
+    std::vector<double> chain_squares, pair_chain_squares;
     std::vector<uint32_t> pair_begin, pair_count;               // [n_slices][G] items of the pair, by its later scan
     uint32_t n_units = 0;
     // device state
@@ -851,7 +851,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
     if (int rc = TI.allocate(r, on_device)) return rc;
     Item* const items = TI.h<Item>(0);
     uint32_t n_items = 0;
-    r->chain_bytes.assign(G, 0); r->item_begin.assign((size_t)r->n_slices * G, 0); r->item_count.assign((size_t)r->n_slices * G, 0);
+    r->chain_bytes.assign(G, 0); r->chain_squares.assign(G, 0); r->item_begin.assign((size_t)r->n_slices * G, 0); r->item_count.assign((size_t)r->n_slices * G, 0);
     // A scan that is one restart interval of at least this many bytes goes to the kernels for long
     // intervals; DC refinement scans have no items at all (see dc_refine_image).
     uint32_t long_min = 64;
@@ -922,6 +922,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
                 Item* open = nullptr;                         // an unfilled last item that the next image may extend
                 uint32_t last = 0;                            // the longest chain of the last item
                 uint64_t load = 0;
+                double squares = 0;
                 for (uint32_t pos = r->slice_img[g]; pos < r->slice_img[g + 1] && !dc_refine; ++pos) {
                     const uint32_t i = order[pos];
                     if (single && takes_long_kernel((int)s, i)) continue;
@@ -933,7 +934,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
                         j = std::min<uint32_t>(kSegsPerItem - open->count, nseg);
                         open->count += j; open->next = si + 1u;
                         open = nullptr;
-                        load += std::max(chain, last) - last;
+                        if (chain > last) { load += chain - last; squares += (double)chain * chain - (double)last * last; }
                     }
                     for (; j < nseg; j += kSegsPerItem) {
                         const uint32_t cnt = std::min<uint32_t>(kSegsPerItem, nseg - j);
@@ -941,9 +942,11 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
                         open = ac && cnt < (uint32_t)kSegsPerItem ? &items[n_items] : nullptr;
                         ++n_items;
                         load += last = chain;
+                        squares += (double)chain * chain;
                     }
                 }
                 r->chain_bytes[s] += load;
+                r->chain_squares[s] += squares;
                 r->item_begin[(size_t)g * G + s] = begin;
                 r->item_count[(size_t)g * G + s] = n_items - begin;
             }
@@ -964,7 +967,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
         }
     }
     // the pairs' items: sixteen intervals of one image
-    r->pair_chain_bytes.assign(G, 0); r->pair_begin.assign((size_t)r->n_slices * G, 0); r->pair_count.assign((size_t)r->n_slices * G, 0);
+    r->pair_chain_bytes.assign(G, 0); r->pair_chain_squares.assign(G, 0); r->pair_begin.assign((size_t)r->n_slices * G, 0); r->pair_count.assign((size_t)r->n_slices * G, 0);
     for (int g = 0; g < r->n_slices; ++g)
         for (uint32_t s = 0; s < G; ++s) {
             const uint32_t begin = n_items;
@@ -976,6 +979,7 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
                 for (uint32_t j = 0; j < nseg; j += kSegsPerItem / 2) {
                     items[n_items++] = Item{a * N + i, j, std::min<uint32_t>(kSegsPerItem / 2, nseg - j), 0u, (s - a) * N};
                     load += longer;
+                    r->pair_chain_squares[s] += (double)longer * longer;
                 }
             }
             r->pair_chain_bytes[s] += load;
@@ -983,18 +987,6 @@ int open_impl(const uint8_t* rec, size_t len, pcr_record* r) {
             r->pair_count[(size_t)g * G + s] = n_items - begin;
         }
     if (on_device && cudaDeviceGetAttribute(&r->n_sms, cudaDevAttrMultiProcessorCount, r->device) != cudaSuccess) return PCR_E_CUDA;
-    for (const std::vector<int>& scans_of_wave : r->paired_waves) {
-        std::vector<char> in_pair(G, 0);
-        for (int s : scans_of_wave) if (r->pair_of[s] >= 0) in_pair[s] = in_pair[r->pair_of[s]] = 1;
-        uint64_t n = 0;
-        bool any = false;
-        for (int s : scans_of_wave)
-            for (int g = 0; g < r->n_slices; ++g) {
-                n += r->pair_count[(size_t)g * G + s] + (in_pair[s] ? 0u : r->item_count[(size_t)g * G + s]);
-                any = any || in_pair[s];
-            }
-        if (any && n > 20ull * (uint64_t)r->n_sms) r->pairs_fit = false;      // (see pairs_pay)
-    }
     // pixel work units (see Sampling in pcr_pixels.cuh), image by image in processing order, inside an image
     // MCU row by MCU row.  The host only counts them; a small kernel writes the list at set-up.
     uint32_t* const unit_prefix = T.h<uint32_t>(at_prefix);
@@ -1316,16 +1308,10 @@ static bool allow_refine_smem(int device) {
     return true;
 }
 
-// The AC refinements among scans k0 .. k-1 of a wave in items an SM, an item counting by how long its scan's chains are on average
-// (a chroma scan's are a third of luminance's).
-//
-// refine_kernel's CTAs take them up to four (rec->refine_ctas), lane-per-interval warps of entropy_kernel beyond.  A CTA's
-// chains are several times as fast (170 to 220 cycles a symbol), but three CTAs are all an SM holds, 96 chains against 480.  Decode in us,
-// CTAs and warps, by this number.  k = 9, one wave: ImageNet-shaped images 0.9 145 and 168, 2.6 213 and 226, 3.4 217 and 228, 4.0 262
-// and 281, 4.2 288 and 282, 5.3 330 and 302, 6.9 421 and 362; CelebA-shaped 3.2 170 and 180, 3.8 187 and 187, 4.3 206 and 196;
-// HAM-shaped 2.1 234 and 256, 3.1 304 and 312, 4.0 357 and 334.  k = 6, luminance alone: ImageNet-shaped 2.9 237 and 241, 3.9 291 and 283,
-// 4.4 314 and 299, 7.7 503 and 448; CelebA-shaped 3.0 187 and 191, 4.5 245 and 241; 32x32 3.5 85 and 85, 6.9 116 and 114.
-static double refine_load(const pcr_record* rec, const std::vector<int>& wave, bool paired, int k0, int k) {
+// The AC refinements among scans k0 .. k-1 of a wave in items an SM, an item counting by its longest chain beside the chain that a byte of the
+// scan lies in on average (of the scan where that is longest; a chroma scan's are a third of luminance's).  Not the average item's chain: a
+// launch waits for the long ones, and with that unit records of mixed sizes changed sides at 1.4 times the number of others.
+static double refine_load(const pcr_record* rec, const std::vector<int>& wave, bool paired, int k0, int k, double* chain = nullptr) {
     double sum = 0, longest = 0;
     std::vector<char> counted(rec->G, 0);                     // scans that a pair's items stand for
     for (int s : wave)
@@ -1337,35 +1323,63 @@ static double refine_load(const pcr_record* rec, const std::vector<int>& wave, b
         for (int g = 0; g < rec->n_slices; ++g) items += (pair ? rec->pair_count : rec->item_count)[(size_t)g * rec->G + s];
         const double bytes = (double)std::max<uint64_t>(items, (pair ? rec->pair_chain_bytes : rec->chain_bytes)[s]);
         sum += bytes;
-        if (items) longest = std::max(longest, bytes / (double)items);
+        if (items) longest = std::max(longest, std::max(bytes, (pair ? rec->pair_chain_squares : rec->chain_squares)[s]) / bytes);
     }
+    if (chain) *chain = longest;
     return sum > 0 ? sum / longest / rec->n_sms : 0;
 }
 
-// Behind another wave of refinements the line lies further out: the slices of the record get there one after the other.  Decode at k = 10 in us
-// with the later wave (luminance alone) in CTAs and in warps: ImageNet-shaped 4.4 468 and 537, 5.1 554 and 613, 6.2 603 and 609, 7.7 733
-// and 710; CelebA-shaped 4.5 356 and 368, 6.1 455 and 446; greyscale 5.1 485 and 546; HAM-shaped 4.6 626 and 578.
-static double refine_line(const pcr_record* rec, bool paired, bool later) { return rec->refine_ctas * (paired ? 1.125 : (later ? 1.6 : 1.0)); }
+// refine_kernel's CTAs take a wave's refinements up to rec->refine_ctas by refine_load, lane-per-interval warps of entropy_kernel beyond.  A CTA's
+// chains are several times as fast (170 to 220 cycles a symbol), but three CTAs are all an SM holds, 96 chains against 480.
+// Decode in us, CTAs and warps, by refine_load, means over two or three contents.  k = 9, one wave: ImageNet-shaped images 3.0 242
+// and 248, 3.3 229 and 237, 3.8 262 and 259, 4.0 283 and 277; in 4:4:4 2.5 216 and 228, 3.0 255 and 236, 3.4 282 and 261; in 4:2:2 2.4 213 and 220,
+// 2.8 238 and 240, 3.4 276 and 265; CelebA-shaped 3.2 172 and 176, 3.4 183 and 182, 3.7 191 and 186, 4.2 223 and 214; HAM-shaped 2.5 242 and 243,
+// 3.0 280 and 267, 3.5 316 and 296; mixed sizes 2.7 228 and 246, 3.1 240 and 259, 3.7 247 and 247, 4.2 261 and 257; 128x128 2.3 107 and 110, 2.9 118
+// and 119.  k = 6, luminance alone: ImageNet-shaped 3.0 257 and 264, 3.7 292 and 281, 4.2 322 and 303; CelebA-shaped 3.0 198 and 201, 3.8 221
+// and 219, 4.5 249 and 243.  Short chains gain from fewer steps outside the loop: 32x32 at k = 9 3.7 106 and 110, 4.4 109 and 113, 5.0 114 and 117,
+// 6.3 111 and 99, at k = 6 2.7 87 and 96; 64x64 2.9 107 and 106, 3.5 118 and 120.
+//
+// Behind another wave of refinements the line lies further out: the slices of the record get there one after the other.  Decode at k = 10
+// with the later wave (luminance alone) in CTAs and in warps: ImageNet-shaped 5.0 552 and 556, 5.5 586 and 588, 5.9 601 and 600, 6.8 675 and 664,
+// 7.4 721 and 705; CelebA-shaped 4.5 359 and 359, 5.3 405 and 397, 6.0 442 and 429, 6.8 498 and 475; HAM-shaped 3.9 534 and 531, 4.6 602 and 585, 5.4
+// 677 and 644; greyscale 4.9 486 and 508, 5.4 508 and 530, 5.9 518 and 543; mixed sizes 3.4 438 and 503, 4.0 502 and 550.
+//
+// With pairs the line is where pairs cease to pay (see pairs_pay).
+static bool refine_in_ctas(const pcr_record* rec, const std::vector<int>& wave, bool paired, bool later, int k0, int k) {
+    double chain = 0, first = 0;                              // `first`: of the wave that would hold the pairs' earlier scans
+    const double load = refine_load(rec, wave, paired, k0, k, &chain);
+    bool pairs = false;
+    for (int s : wave) {
+        if (!paired || s >= k || rec->pair_of[s] < k0) continue;
+        pairs = true;
+        for (const std::vector<int>& w : rec->wave_scans)
+            if (std::find(w.begin(), w.end(), rec->pair_of[s]) != w.end()) first = std::max(first, refine_load(rec, w, false, k0, k));
+    }
+    double line = chain < 48.0 ? 1.32 : (pairs ? 0.91 + 0.22 * std::min(std::max(first - 1.85, 0.0), 1.45) : 1.0);
+    if (later && !pairs) line = 1.8;
+    return load <= rec->refine_ctas * line;
+}
 
 // Whether refinements that follow one another are decoded in pairs (see refine_kernel).  Pairs shorten the chain but leave the lanes
-// of the shorter scan idle.  In CTAs they pay while these are about four an SM; beyond, the two waves are faster one after the other as
-// long as the later one's CTAs are.  Where that one goes to the warps too, both ways differ little until the machine is full: it holds 18
-// lane-per-interval warps of 36 KB a three an SM, and up to 20 the few that wait cost less than the chain gains.  Decode at k = 10 in us by
-// CTAs an SM.  Pairs in CTAs and no pairs: ImageNet-shaped images 1.6 197 and 225, 3.1 277 and 307, 3.9 340 and 320, 4.7 367 and 330, 6.1
-// 366 and 339, 7.7 479 and 400; CelebA-shaped 1.9 163 and 163, 2.8 177 and 187, 3.8 213 and 196, 5.6 262 and 235; HAM-shaped 1.8 236 and
-// 258, 2.7 265 and 296, 3.6 372 and 342; greyscale 2.9 240 and 266, 4.4 327 and 285; 4:4:4 2.0 223 and 252, 3.9 371 and 405, 5.8 490 and 451;
-// mixed sizes 1.3 212 and 254, 4.4 256 and 280, 9.8 446 and 371.  Pairs in warps and no pairs: ImageNet-shaped 9.5 515 and 438, 10.7 531 and
-// 468, 12.5 584 and 554, 15 661 and 603, 19 764 and 710; CelebA-shaped 9.4 328 and 313, 11.2 360 and 356; HAM-shaped 7.2 447 and 458, 10.7 582
-// and 626.
+// of the shorter scan idle.  They pay in CTAs, while an SM's three hold them all at once; beyond, two waves take no longer than
+// the pairs' second round.  Decode at k = 10 in us by refine_load with pairs, pairs in CTAs and no pairs, means over two or three contents:
+// ImageNet-shaped images 2.2 232 and 255, 3.0 283 and 306, 3.3 314 and 306, 3.8 338 and 319; CelebA-shaped 2.8 185 and 193, 3.3 219 and 203, 3.8 225
+// and 203; HAM-shaped 2.7 252 and 285, 3.2 318 and 298, 3.6 356 and 321; greyscale 3.2 279 and 273, 3.6 298 and 270, 4.3 328 and 289; mixed sizes 2.7
+// 261 and 318, 3.4 300 and 314, 4.3 347 and 376; 128x128 1.6 112 and 117, 2.4 133 and 132, 2.8 140 and 136.
+// Chroma scans beside the earlier scan fill the first wave without pairs too (`first`), which then takes a second round itself: 4:2:2
+// ImageNet-shaped (first 1.9) 3.0 292 and 322, (2.1) 3.2 308 and 331, (2.4) 3.5 344 and 341, CelebA-shaped (2.1) 3.2 205 and 215, (2.4) 3.7 249 and
+// 231; 4:4:4 ImageNet-shaped (3.0) 3.3 314 and 353, (3.1) 3.5 351 and 387, (3.7) 4.1 390 and 416, (4.2) 4.7 432 and 406, CelebA-shaped (3.2) 3.6 223
+// and 238, (3.7) 4.2 257 and 262, HAM-shaped (3.2) 3.2 344 and 380, (3.7) 3.7 392 and 417, (4.3) 4.2 455 and 414, mixed sizes (3.5) 3.3 342 and 385.
+// Where chains are short, a wave less counts for more: 32x32 2.6 82 and 99, 3.7 109 and 121, 4.4 115 and 123, 5.2 121 and 140, 8.8 149 and 149;
+// 64x64 2.9 102 and 106, 3.5 115 and 128, 4.2 123 and 132, 5.9 148 and 141.
+// Pairs in warps and no pairs: ImageNet-shaped 10 526 and 484, 13 601 and 581, 18 747 and 697; CelebA-shaped 10 343 and 348, 13 399 and 402, 17 490
+// and 474; HAM-shaped 9 496 and 529, 11 565 and 586, 14 725 and 719, 18 877 and 847; greyscale 14 570 and 523, 17 670 and 602; mixed sizes 10 589 and 549:
+// never chosen, since what gains (HAM-shaped) gains less than the others lose.
 static bool pairs_pay(const pcr_record* rec, int k0, int k) {
-    auto holds = [&](const std::vector<int>& wave) {          // the later scan of a pair of this call
-        for (int s : wave) if (s < k && rec->pair_of[s] >= k0) return true;
-        return false;
-    };
-    bool ctas = true, warps = rec->pairs_fit;
-    for (const std::vector<int>& wave : rec->paired_waves) ctas = ctas && (!holds(wave) || refine_load(rec, wave, true, k0, k) <= refine_line(rec, true, false));
-    for (const std::vector<int>& wave : rec->wave_scans) warps = warps && (!holds(wave) || refine_load(rec, wave, false, k0, k) > refine_line(rec, false, true));
-    return ctas || warps;
+    for (const std::vector<int>& wave : rec->paired_waves)
+        for (int s : wave)
+            if (s < k && rec->pair_of[s] >= k0 && !refine_in_ctas(rec, wave, true, false, k0, k)) return false;
+    return true;
 }
 
 // Form of entropy_kernel for the first passes among scans k0 .. k-1 of a wave: kFirstFull where there is so much to store that stores are
@@ -1604,7 +1618,7 @@ static int decode_range(pcr_record* rec, int k0, int k, void* out, void* stream,
             bool later = false;                            // a wave before this one holds refinements too
             for (int v = 0; v < w; ++v)
                 for (int s : waves[v]) later = later || (s >= k0 && s < k && rec->script[s].Ss > 0 && rec->script[s].Ah != 0);
-            const bool ctas = refine_load(rec, waves[w], paired, k0, k) <= refine_line(rec, paired, later);
+            const bool ctas = refine_in_ctas(rec, waves[w], paired, later, k0, k);
             auto add_run = [&](bool to_ctas, uint32_t first, uint32_t n) {
                 if (!n) return;
                 ItemRuns& to = to_ctas ? refs : runs;
