@@ -219,7 +219,7 @@ struct pcr_record {
     std::vector<std::vector<int>> paired_waves;
     std::vector<int> pair_of;
     int pairs = -1;                                             // see pairs_pay (PCR_PAIRS overrides: 0 never, 1 always)
-    double refine_ctas = 3.4;                                   // see refine_load (PCR_REFINE_CTAS overrides)
+    double refine_ctas = 3.4;                                   // see refine_in_ctas (PCR_REFINE_CTAS overrides)
     int64_t long_ctas = -1;                                     // see wide_long_scans (PCR_LONG_CTAS: a line in CTAs an SM instead)
     int64_t seq_ctas = -1;                                      // see sequential_in_ctas (PCR_SEQ_CTAS: a line in items an SM instead)
     int64_t index_ctas = -1;                                    // see launch_index_kernel (PCR_INDEX_CTAS: a line in pairs an SM instead)

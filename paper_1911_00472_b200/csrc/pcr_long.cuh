@@ -679,22 +679,22 @@ __global__ void __launch_bounds__(32 * kWarps) sequential_long_kernel(Params P, 
 //                decoded in advance, 32 at a time, so the thread neither assembles a window nor looks up a code;
 //   zpos[b][i]   non-zero positions in front of the i-th still-zero coefficient of block b: by differences the number of
 //                correction bits passed; and whether the block ends there.
-// A symbol is two dependent loads and a handful of additions, and what a block that ends takes beyond that does not ask how many still-zero
-// positions there are: the list says where the block ends, and its entries beyond that are all closing ones.  Per block the thread leaves
-// the bit position where the next one begins; the helper warp decodes the 32 blocks of a finished batch once more, one lane per
-// block, to make the side data.
-// A lone thread takes about four cycles an instruction whatever it waits for, so the count of instructions decides.  The launch in us with 16
-// instructions a symbol and a block change that carried the next block's bounds along (clock64 in a copy that took most symbols by one load: 45 cycles
-// a symbol and 370 a block); with
-// lists that say where a block ends; and now, with runs counted from the entry reached, the flag of the ending entry taken out once a block
-// instead of in every symbol, and the chain's place in shared memory in a uniform register:
-//   HAM-shaped, 1024 / 512 / 128 images   1728 -> 1565 -> 1420, 1468 -> 1285 -> 1182, 1412 -> 1230 -> 1127
-//   mixed sizes, 200                      3281 -> 2846 -> 2637
-//   ImageNet-shaped, 1024 / 256           2843 -> 2483 -> 2285, 2768 -> 2409 -> 2229
-//   CelebA-shaped, 256 at k = 8           268 -> 237 -> 219
-// Not kept (HAM-shaped 1024, 512, 128, mixed sizes; of the second form): block change by selects in the symbol's line (1785, 1349, 1279, 2890); a
-// loop of one load a symbol behind a block's last non-zero position (1599, 1335, 1273, 2786); the entries behind the symbol's own bits
-// requested before the number of correction bits is known (2331, 1754, 1652, 3628); the loop unrolled (1869).
+// A symbol is two dependent loads and a handful of additions, and what a block that ends takes beyond that does not ask how many
+// still-zero positions there are: the list says where the block ends, and its entries beyond that are all closing ones.  Per block the
+// thread leaves the bit position where the next one begins; the helper warp decodes the 32 blocks of a finished batch once more, one
+// lane per block, to make the side data.
+// A lone thread takes about four cycles an instruction whatever it waits for, so the count of instructions decides.  The launch in us
+// with 16 instructions a symbol and a block change that carried the next block's bounds along (clock64 in a copy that took most symbols
+// by one load: 45 cycles a symbol and 370 a block); with lists that say where a block ends; and now, with runs counted from the entry
+// reached, the flag of the ending entry taken out once a block instead of in every symbol, and the chain's place in shared memory in a
+// uniform register:
+//   HAM-shaped, 1024 / 512 / 128 images   1728 -> 1565 -> 1414, 1468 -> 1285 -> 1181, 1412 -> 1230 -> 1127
+//   mixed sizes, 200                      3281 -> 2846 -> 2656
+//   ImageNet-shaped, 1024 / 256           2843 -> 2483 -> 2289, 2768 -> 2409 -> 2241
+//   CelebA-shaped, 256 at k = 8           268 -> 237 -> 221
+// Not kept (HAM-shaped 1024, 512, 128, mixed sizes; of the second form): block change by selects in the symbol's line (1785, 1349,
+// 1279, 2890); a loop of one load a symbol behind a block's last non-zero position (1599, 1335, 1273, 2786); the entries behind the
+// symbol's own bits requested before the number of correction bits is known (2331, 1754, 1652, 3628); the loop unrolled (1869).
 // Codes longer than the quick table's index are looked up where the thread meets one, since few records have many of them; with the
 // helper looking them up at every bit position, filling q was 28 % of its time.  128 HAM-shaped images whose refinement tables have
 // longer codes than they need (us: looked up by the helper; by the thread, the block again for every one; and now): all 10 bits 9829,

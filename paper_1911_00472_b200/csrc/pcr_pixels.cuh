@@ -193,8 +193,8 @@ __device__ __forceinline__ bool expand_block(const Params& P, const CoefLists& c
             if (i > 1) { const uint4* o = reinterpret_cast<const uint4*>(P.aux + cl.refine[comp][i]) + 2 * local; a = __ldg(o); b = __ldg(o + 1); }
             // corrections: the coefficients that were non-zero before the scan, in zigzag order, take the
             // correction bits in reading order (as many as there are such positions, the last one in bit 0);
-            // the walk through each half ends with its last set bit (no branch around a correction: 347 -> 334 us with the rest of this walk
-            // in 32 bits, 1024 ImageNet-shaped images at k = 10)
+            // the walk through each half ends with its last set bit (in 32 bits, and without a branch around a correction: 1024 ImageNet-shaped
+            // images at k = 10 347 -> 334 us)
             const uint32_t h0 = a.x & ~b.x, h1 = a.y & ~b.y;
             // (none of them: a shift by 64, which gives 0; the side data of a damaged image may have bits all the same)
             const int n0 = __popc(h0);
@@ -249,7 +249,7 @@ __device__ __forceinline__ bool expand_block(const Params& P, const CoefLists& c
 // samples stay in the registers of the thread that made them and meet the chroma there, two pixels
 // per instruction (16-bit pairs).  Bound by instruction issue (integer multiplications and additions of the transform, about
 // 0.65 of the slots, 0.73 with kCoarse).  Pixel stage of 1024 ImageNet-shaped images, before (lines of 128 bytes per block, colour as a
-// step of its own) and now: k = 5 348 -> 166 us, k = 10 562 -> 348 us, baseline 351 -> 265 us.
+// step of its own) and now: k = 5 348 -> 164 us, k = 10 562 -> 334 us, baseline 351 -> 272 us.
 template <bool kRefine, int kMode, bool kRoi = false, int kStage = 0, int kSamp = kSamp420, bool kCoarse = false>
 __global__ void __launch_bounds__(unit_threads<kSamp>(), (kCoarse ? 1152 : 672) / unit_threads<kSamp>())
 pixel_kernel(Params P, CoefLists cl, uint8_t* __restrict__ out) {

@@ -17,7 +17,7 @@
 // for block ends and rare cases (350 -> 175); the next symbol's entry requested before anything else that is loaded (-> 166);
 // the rings filled by a helper.
 // Rounds of 16, 32, 48 and 64 symbols: 233, 177, 157 and 164 k cycles for the busiest CTA of 4 ImageNet-shaped images, whose
-// refinement wave took 211 us and takes 84.  1024 such images are better off with entropy_kernel: see refine_load.
+// refinement wave took 211 us and takes 84.  1024 such images are better off with entropy_kernel: see refine_in_ctas.
 //
 // Side data of a block: {mask of the band's non-zero positions after the scan, correction bits in reading order (the last
 // one in bit 0), newly non-zero positions, the positive ones among them}; the pixel kernel applies them.

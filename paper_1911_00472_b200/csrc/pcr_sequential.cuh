@@ -10,11 +10,14 @@
 // collide.
 //
 // Bound by warp 0's step: a window, a table entry, and where both lead next, 125 cycles a symbol (a lane that did everything
-// itself took 600), then by the warps of four CTAs an SM sharing its schedulers.  1024 ImageNet-shaped images 742 -> 437 us, 64
-// such images 713 -> 177 us.  The warps that write count for most of those schedulers' slots: with what a symbol needs only in damaged streams or at
-// block ends moved behind the block, decode of 1024 ImageNet-shaped images 688 -> 668 us, of 1024 CelebA-shaped 447 -> 414.  Launches of many images with few intervals keep a lane an interval (at the end of the file).
-// (A step with a predicate for every case 180 cycles; both possible tables looked up and one entry
-// chosen afterwards: 189 us; 6 or 12 warps a CTA: 183, 181 us and 467, 460; rounds of 48 symbols 184, of 96 equal.)
+// itself took 600), then by the warps of four CTAs an SM sharing its schedulers.  1024 ImageNet-shaped images, one stage after the
+// other, 742 -> 391 us, 64 such images 713 -> 137 us.  The warps that write count for most of those schedulers' slots: with what a
+// symbol needs only in damaged streams or at block ends moved behind the block, and magnitudes by a funnel shift, decode of 1024
+// ImageNet-shaped images 688 -> 645 us, of 1024 CelebA-shaped 447 -> 407.  Launches of many images with few intervals keep a lane an
+// interval (at the end of the file).
+// (Before those two: a step with a predicate for every case 180 cycles; both possible tables looked up and one entry chosen
+// afterwards, 64 images 177 -> 189 us; 6 or 12 warps a CTA 183, 181 us, and 1024 images 437 -> 467, 460; rounds of 48 symbols 184,
+// of 96 equal.)
 #pragma once
 #include <cuda_runtime.h>
 #include <stddef.h>
@@ -263,8 +266,8 @@ __global__ void __launch_bounds__(32 * kSeqWarps, 4) sequential_kernel(Params P,
 // The same, one lane per restart interval, for launches of many items (see sequential_in_ctas): a warp an item instead of eight, 18
 // items an SM instead of four.  Lanes stand at different kinds of symbol in every step, so a block's first symbol goes through the same
 // instructions as the others (its value is the difference), stores are predicated, and what changes from block to block comes
-// from a small table in shared memory.  Bound by the length of a lane's chain, 600 cycles a symbol: 3072 CelebA-shaped images 1049 us,
-// with the kernel above 1224; 1024 513 and 450.
+// from a small table in shared memory.  Bound by the length of a lane's chain, 600 cycles a symbol: decode of 3072 CelebA-shaped images
+// 980 us, with the kernel above 1118; of 1024 480 and 411.
 // ---------------------------------------------------------------------------------------
 constexpr int kSeqLaneWarps = 2;
 constexpr uint32_t kSeqLaneRing = 4 * sizeof(ScanTab), kSeqLanePlaces = kSeqLaneRing + (kRingWords + 2) * 128, kSeqLanePreds = kSeqLanePlaces + 8 * 16;
